@@ -289,4 +289,45 @@ int tc_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, 
 int64_t tc_weight_grad_workspace(const rad_store* st, int64_t H);
 int sm_pairs();   // SM pairs the dW plans count on (see rad_sm_pairs)
 
+// ---- clusters of CTAs ----------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_nctas() {
+  uint32_t n;
+  asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n));
+  uint32_t m;
+  asm volatile("mov.u32 %0, %%cluster_nctaid.y;" : "=r"(m));
+  return n * m;
+}
+// every thread of every CTA of the cluster; shared-memory writes before it are seen by all after it
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the word that the cluster's CTA `rank` holds at this shared-memory address
+__device__ __forceinline__ float ld_cluster_f32(const float* smem, uint32_t rank) {
+  float v;
+  asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %1, %2;\n\tld.shared::cluster.f32 %0, [a];\n\t}"
+               : "=f"(v) : "r"((uint32_t)__cvta_generic_to_shared(smem)), "r"(rank) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_cluster_f32x4(const float* smem, uint32_t rank) {
+  float4 v;
+  asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %4, %5;\n\tld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [a];\n\t}"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"((uint32_t)__cvta_generic_to_shared(smem)), "r"(rank) : "memory");
+  return v;
+}
+template <typename K, typename... Args>
+int launch_with_cluster(K kernel, dim3 grid, int threads, size_t smem, dim3 cluster, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = cluster.x; attr.val.clusterDim.y = cluster.y; attr.val.clusterDim.z = cluster.z;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? RAD_OK : RAD_ECUDA;
+}
+
 }  // namespace rad

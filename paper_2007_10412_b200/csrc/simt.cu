@@ -325,88 +325,118 @@ __global__ void zero_rows_kernel(float* dW, int64_t ldw, int64_t D, int64_t H) {
     dW[(i / H) * ldw + (i % H)] = 0.0f;
 }
 
-// ---- column sums (bias gradient), two fixed-order stages ------------------------------------------
-constexpr int kColChunkRows = 128;
-template <typename T>
-__global__ void __launch_bounds__(256) colsum_partial_kernel(const T* dZ, int64_t ldz, int64_t B, int64_t H,
-                                                             float* partial) {
-  const int64_t h = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (h >= H) return;
-  const int64_t b0 = (int64_t)blockIdx.y * kColChunkRows, b1 = min(B, b0 + kColChunkRows);
-  float s = 0.0f;
-#pragma unroll 8
-  for (int64_t b = b0; b < b1; ++b) s += to_float(dZ[b * ldz + h]);
-  partial[(int64_t)blockIdx.y * H + h] = s;
-}
-// The same chunk sums with 16-byte loads: a thread owns eight neighbouring bf16 columns (two bytes per load and
-// lane leave most of the memory system idle); rows in the same order, so the sums are the same numbers.
-__global__ void __launch_bounds__(256) colsum_partial_vec8_kernel(const bf16* dZ, int64_t ldz, int64_t B, int64_t H,
-                                                                  float* partial) {
-  const int64_t h = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 8;
-  if (h >= H) return;
-  const int64_t b0 = (int64_t)blockIdx.y * kColChunkRows, b1 = min(B, b0 + kColChunkRows);
-  float s[8] = {};
-#pragma unroll 8
-  for (int64_t b = b0; b < b1; ++b) {
-    const uint4 v = *reinterpret_cast<const uint4*>(dZ + b * ldz + h);
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+// ---- column sums (bias gradient) -----------------------------------------------------------------
+// A CTA owns CL x V neighbouring columns (one 128-byte line where the matrix is wide) and a slab of rows: 256 / CL
+// row lanes, each with V columns in registers and 16-byte loads where the layout allows them.  The lanes of a
+// column are added by shuffles, the eight warps in shared memory, the CTAs of a cluster (its slabs of rows) by
+// distributed shared memory: every sum in a fixed order, one launch.
+// Bound by the latency of the loads in flight, so what matters is how many CTAs share the rows: with one CTA per
+// 128 rows x 2048 columns (the form before) a 4096 x 2048 bf16 matrix (16.8 MB) took 56 + 5 us on 32 CTAs whose
+// threads walked 128 rows each; here it is 256 CTAs of 16 rows per thread.
+constexpr int kColMaxCluster = 8;          // portable cluster size
+// From here on DRAM is what bounds the sum, and 512 bytes of a row per CTA read better than 128: 65536 x 8192 bf16
+// 186 us (5.8 TB/s) against 216 us with clusters on 128-byte columns and 200 us before; 16384 x 4096 (134 MB), which
+// L2 still helps, 33 against 30 us, so the line lies above it.
+constexpr int64_t kColBigBytes = 256ll << 20;
+template <typename T, int V>
+__device__ __forceinline__ void colsum_load(const T* p, float (&v)[V]) {
+  if constexpr (V == 1) {
+    v[0] = to_float(*p);
+  } else if constexpr (sizeof(T) == 4) {
+    const float4 x = *reinterpret_cast<const float4*>(p);
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+  } else {
+    const uint4 x = *reinterpret_cast<const uint4*>(p);
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      s[2 * i] += __uint_as_float(w[i] << 16);
-      s[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
+      v[2 * i] = __uint_as_float(w[i] << 16);
+      v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
     }
   }
-  float4* out = reinterpret_cast<float4*>(partial + (int64_t)blockIdx.y * H + h);
-  out[0] = make_float4(s[0], s[1], s[2], s[3]);
-  out[1] = make_float4(s[4], s[5], s[6], s[7]);
 }
-__global__ void __launch_bounds__(256) colsum_final_kernel(const float* partial, int64_t chunks, int64_t H,
-                                                           float* db) {
-  const int64_t h = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (h >= H) return;
-  float s = 0.0f;
+// grid (column blocks, CTAs along the rows); the latter is the cluster size where `out` is the result itself, and
+// the number of partial rows (cluster of one) where a second launch adds them
+template <typename T, int V>
+__global__ void __launch_bounds__(256) colsum_kernel(const T* dZ, int64_t ldz, int64_t B, int64_t H, int log_cl,
+                                                     int64_t rows_per_cta, float* out) {
+  __shared__ float s_warp[8][32 * V];
+  __shared__ float s_cta[32 * V];
+  const int CL = 1 << log_cl, RL = 256 >> log_cl, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int c = tid & (CL - 1), r = tid >> log_cl;
+  const int64_t h = ((int64_t)blockIdx.x * CL + c) * V;
+  const int64_t b0 = (int64_t)blockIdx.y * rows_per_cta, b1 = min(B, b0 + rows_per_cta);
+  float s[V] = {};
+  if (h < H) {
+    const T* p = dZ + h;
 #pragma unroll 8
-  for (int64_t c = 0; c < chunks; ++c) s += partial[c * H + h];      // loads in flight together, added in order
-  db[h] = s;
-}
-// First stage for a narrow matrix (at most 64 columns, e.g. the bias gradient of a convolution: B H W rows, 16
-// columns), where one thread per column would leave most of a CTA idle: the CTA's threads are R row lanes x HP
-// columns (HP the power of two that holds H); a lane sums every R-th row of the CTA's slab, then the column's
-// lanes are added in lane order.  Second stage as above.
-template <typename T>
-__global__ void __launch_bounds__(256) colsum_narrow_partial_kernel(const T* dZ, int64_t ldz, int64_t B, int H, int HP,
-                                                                    int64_t rows_per_block, float* partial) {
-  __shared__ float s[256];
-  const int c = threadIdx.x & (HP - 1), r = threadIdx.x / HP, R = 256 / HP;
-  const int64_t b0 = (int64_t)blockIdx.x * rows_per_block, b1 = min(B, b0 + rows_per_block);
-  float sum = 0.0f;
-  if (c < H)
-#pragma unroll 8
-    for (int64_t b = b0 + r; b < b1; b += R) sum += to_float(dZ[b * ldz + c]);
-  s[threadIdx.x] = sum;
+    for (int64_t b = b0 + r; b < b1; b += RL) {
+      float v[V];
+      colsum_load<T, V>(p + b * ldz, v);
+#pragma unroll
+      for (int i = 0; i < V; ++i) s[i] += v[i];
+    }
+  }
+  for (int o = CL; o < 32; o <<= 1) {
+#pragma unroll
+    for (int i = 0; i < V; ++i) s[i] += __shfl_xor_sync(0xffffffffu, s[i], o);
+  }
+  if (lane < CL) {
+#pragma unroll
+    for (int i = 0; i < V; ++i) s_warp[warp][lane * V + i] = s[i];
+  }
   __syncthreads();
-  if (r == 0 && c < H) {
+  const bool clustered = cluster_nctas() > 1;
+  const int64_t hc = (int64_t)blockIdx.x * CL * V + tid;       // the column this thread finishes
+  if (tid < CL * V) {
     float t = 0.0f;
-    for (int i = 0; i < R; ++i) t += s[i * HP + c];
-    partial[(int64_t)blockIdx.x * H + c] = t;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += s_warp[w][tid];
+    if (clustered) s_cta[tid] = t;
+    else if (hc < H) out[(int64_t)blockIdx.y * H + hc] = t;
   }
+  if (!clustered) return;
+  cluster_barrier();
+  if (blockIdx.y == 0 && tid < CL * V && hc < H) {
+    float t = 0.0f;
+    for (int q = 0; q < (int)gridDim.y; ++q) t += ld_cluster_f32(&s_cta[tid], (uint32_t)q);
+    out[hc] = t;
+  }
+  cluster_barrier();                       // no CTA leaves while another reads its sums
 }
-// Both stages in one launch for few rows (the small nets are bound by their launch count): the same chunk sums,
-// added in the same order, by the thread that owns the column.
-constexpr int kColSmallChunks = 2;
-template <typename T>
-__global__ void __launch_bounds__(256) colsum_small_kernel(const T* dZ, int64_t ldz, int64_t B, int64_t H, float* db) {
-  const int64_t h = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (h >= H) return;
-  float total = 0.0f;
-  for (int64_t b0 = 0; b0 < B; b0 += kColChunkRows) {
-    const int64_t b1 = min(B, b0 + kColChunkRows);
-    float s = 0.0f;
-#pragma unroll 8
-    for (int64_t b = b0; b < b1; ++b) s += to_float(dZ[b * ldz + h]);
-    total += s;
+
+template <typename T, int V>
+int launch_colsum(const T* dZ, int64_t ldz, int64_t B, int64_t H, int log_cl, int ny, bool clustered, float* out, cudaStream_t s) {
+  const int64_t colblocks = ceil_div(H, (int64_t)V << log_cl);
+  count_launch();
+  return launch_with_cluster(colsum_kernel<T, V>, dim3((unsigned)colblocks, (unsigned)ny), 256, 0, clustered ? dim3(1, (unsigned)ny) : dim3(1),
+                             s, dZ, ldz, B, H, log_cl, ceil_div(B, (int64_t)ny), out);
+}
+
+// Column lanes of a CTA: eight 16-byte vectors make a 128-byte line; a narrow matrix gets the power of two that
+// holds its columns, so that the other threads are row lanes.
+template <typename T, int V>
+int column_sums_of(const T* dZ, int64_t ldz, int64_t B, int64_t H, float* out, float* partial, int64_t max_slabs, cudaStream_t s) {
+  int log_cl = 0;
+  const int64_t vecs = ceil_div(H, (int64_t)V);
+  const bool big = V > 1 && vecs >= 32 && B * H * (int64_t)sizeof(T) >= kColBigBytes && max_slabs > kColMaxCluster;
+  while ((1 << log_cl) < vecs && log_cl < (V > 1 && !big ? 3 : 5)) ++log_cl;
+  const int64_t RL = 256 >> log_cl, colblocks = ceil_div(vecs, (int64_t)1 << log_cl);
+  // one launch: enough CTAs per column block that a thread adds about four rows, at most a cluster
+  int ny = 1;
+  while (ny < kColMaxCluster && B > 4 * RL * ny) ny *= 2;
+  // Two launches where a cluster per column block would leave most SMs idle and its threads with a long walk
+  // (a convolution's bias gradient: B H W rows of 16 to 64 channels; 4.2 M x 16 bf16 took 75 + 19 us, the second
+  // figure one CTA adding 296 partial rows one by one): first one partial row per slab, then the cluster form on those.
+  if (big || (ny == kColMaxCluster && colblocks * ny < 148 && B > 32 * RL * ny && max_slabs > kColMaxCluster)) {
+    const int64_t slabs = std::min<int64_t>(max_slabs, std::max<int64_t>(kColMaxCluster, (big ? 1184 : 592) / colblocks));
+    const int rc = launch_colsum<T, V>(dZ, ldz, B, H, log_cl, (int)slabs, false, partial, s);
+    if (rc != RAD_OK) return rc;
+    const bool vec = H % 4 == 0 && ((uintptr_t)partial & 15) == 0;
+    return vec ? column_sums_of<float, 4>(partial, H, slabs, H, out, nullptr, 0, s)
+               : column_sums_of<float, 1>(partial, H, slabs, H, out, nullptr, 0, s);
   }
-  db[h] = total;
+  return launch_colsum<T, V>(dZ, ldz, B, H, log_cl, ny, true, out, s);
 }
 
 }  // namespace
@@ -550,6 +580,7 @@ int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 
+constexpr int kColChunkRows = 128;         // rows of dZ per partial row of the workspace
 int64_t column_sums_workspace(int64_t B, int64_t H) {
   return round_up(ceil_div(B, kColChunkRows) * H * 4, 256);
 }
@@ -557,41 +588,17 @@ int64_t column_sums_workspace(int64_t B, int64_t H) {
 int column_sums(int dtype, int64_t B, int64_t H, const void* dZ, int64_t ldz, float* db, void* workspace,
                 int64_t workspace_bytes, cudaStream_t s) {
   if (workspace == nullptr || workspace_bytes < column_sums_workspace(B, H)) return RAD_EWORKSPACE;
-  const int64_t chunks = ceil_div(B, kColChunkRows);
-  if (chunks <= kColSmallChunks) {
-    count_launch();
-    if (dtype == RAD_BF16)
-      colsum_small_kernel<bf16><<<(unsigned)ceil_div(H, 256), 256, 0, s>>>(static_cast<const bf16*>(dZ), ldz, B, H, db);
-    else
-      colsum_small_kernel<float><<<(unsigned)ceil_div(H, 256), 256, 0, s>>>(static_cast<const float*>(dZ), ldz, B, H, db);
-    return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
-  }
   float* partial = static_cast<float*>(workspace);
-  count_launch(2);
-  if (H <= 64) {
-    // no more slabs than the chunk count the workspace was sized for
-    const int64_t slabs = std::min<int64_t>(chunks, 2 * 148);
-    const int64_t rows_per_block = ceil_div(B, slabs), nblocks = ceil_div(B, rows_per_block);
-    const int HP = H <= 16 ? 16 : H <= 32 ? 32 : 64;
-    if (dtype == RAD_BF16)
-      colsum_narrow_partial_kernel<bf16><<<(unsigned)nblocks, 256, 0, s>>>(static_cast<const bf16*>(dZ), ldz, B, (int)H, HP,
-                                                                          rows_per_block, partial);
-    else
-      colsum_narrow_partial_kernel<float><<<(unsigned)nblocks, 256, 0, s>>>(static_cast<const float*>(dZ), ldz, B, (int)H, HP,
-                                                                           rows_per_block, partial);
-    colsum_final_kernel<<<1, 256, 0, s>>>(partial, nblocks, H, db);
-    return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  const int64_t slabs = ceil_div(B, kColChunkRows);          // partial rows the workspace holds
+  const bool aligned = ((uintptr_t)dZ & 15) == 0;
+  if (dtype == RAD_BF16) {
+    const bf16* z = static_cast<const bf16*>(dZ);
+    return aligned && H % 8 == 0 && ldz % 8 == 0 ? column_sums_of<bf16, 8>(z, ldz, B, H, db, partial, slabs, s)
+                                                 : column_sums_of<bf16, 1>(z, ldz, B, H, db, partial, slabs, s);
   }
-  dim3 grid((unsigned)ceil_div(H, 256), (unsigned)chunks);
-  if (dtype == RAD_BF16 && H % 8 == 0 && ldz % 8 == 0 && ((uintptr_t)dZ & 15) == 0 && ((uintptr_t)partial & 15) == 0)
-    colsum_partial_vec8_kernel<<<dim3((unsigned)ceil_div(H, 2048), (unsigned)chunks), 256, 0, s>>>(static_cast<const bf16*>(dZ), ldz, B,
-                                                                                                   H, partial);
-  else if (dtype == RAD_BF16)
-    colsum_partial_kernel<bf16><<<grid, 256, 0, s>>>(static_cast<const bf16*>(dZ), ldz, B, H, partial);
-  else
-    colsum_partial_kernel<float><<<grid, 256, 0, s>>>(static_cast<const float*>(dZ), ldz, B, H, partial);
-  colsum_final_kernel<<<(unsigned)ceil_div(H, 256), 256, 0, s>>>(partial, chunks, H, db);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  const float* z = static_cast<const float*>(dZ);
+  return aligned && H % 4 == 0 && ldz % 4 == 0 ? column_sums_of<float, 4>(z, ldz, B, H, db, partial, slabs, s)
+                                               : column_sums_of<float, 1>(z, ldz, B, H, db, partial, slabs, s);
 }
 
 }  // namespace rad

@@ -149,3 +149,23 @@ def test_bias_gradient_alone_on_every_column_sum_route(B, H, dtype):
     want = dZ.astype(np.float64).sum(axis=0)
     bound = 2e-6 * np.abs(dZ.astype(np.float64)).sum(axis=0)
     assert (np.abs(to_host_f32(db).astype(np.float64) - want) <= bound).all()
+
+
+@pytest.mark.parametrize("B,H,ld,dtype", [(1, 1, 1, "f32"), (33, 8, 8, "bf16"), (1025, 24, 32, "bf16"), (257, 65, 65, "f32"),
+                                          (4097, 72, 72, "f32"), (300001, 8, 8, "bf16"), (300001, 7, 7, "f32"),
+                                          (140000, 20, 24, "bf16"), (70000, 132, 132, "f32")])
+def test_bias_gradient_over_clusters_and_slabs(B, H, ld, dtype):
+    """Column sums by one CTA, by a cluster of CTAs along the rows and by slabs of rows added in a second launch, with
+    vector and single-element loads (padded rows, odd widths), against float64 sums of the same numbers.  Every chain
+    of float32 additions is shorter than 4096 terms of a 2^-24 relative rounding each; the bound allows 33 in a row."""
+    import paper_2007_10412_b200 as rad
+    tdt = torch.float32 if dtype == "f32" else torch.bfloat16
+    g = torch.Generator(device="cuda").manual_seed(B + H)
+    wide = torch.randn(B, ld, generator=g, device="cuda").to(tdt)
+    dZ = wide[:, :H]
+    W = torch.zeros(8, ld, dtype=tdt, device="cuda")[:, :H]
+    db = torch.full((H,), float("nan"), dtype=torch.float32, device="cuda")
+    rad.rad_linear_input_grad(dZ, W, db=db)
+    torch.cuda.synchronize()
+    d64 = dZ.double()
+    assert ((db.double() - d64.sum(0)).abs() <= 2e-6 * d64.abs().sum(0)).all()
