@@ -315,6 +315,10 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(const float* smem, uint32_t r
                : "r"((uint32_t)__cvta_generic_to_shared(smem)), "r"(rank) : "memory");
   return v;
 }
+__device__ __forceinline__ void st_cluster_f32(float* smem, uint32_t rank, float v) {
+  asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, %1;\n\tst.shared::cluster.f32 [a], %2;\n\t}"
+               ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "r"(rank), "f"(v) : "memory");
+}
 template <typename K, typename... Args>
 int launch_with_cluster(K kernel, dim3 grid, int threads, size_t smem, dim3 cluster, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};

@@ -169,3 +169,32 @@ def test_bias_gradient_over_clusters_and_slabs(B, H, ld, dtype):
     torch.cuda.synchronize()
     d64 = dZ.double()
     assert ((db.double() - d64.sum(0)).abs() <= 2e-6 * d64.abs().sum(0)).all()
+
+
+@pytest.mark.parametrize("B,C,dtype", [(1, 1, "f32"), (33, 32, "bf16"), (257, 33, "f32"), (256, 257, "bf16"), (2048, 1024, "bf16"),
+                                       (2049, 1025, "f32"), (300, 2500, "f32")])
+def test_softmax_xent_over_clusters_and_row_lengths(B, C, dtype):
+    """The loss of one CTA, of a cluster of CTAs and of many rows, with rows that fit the registers of a warp (32, 256,
+    1024 logits) and longer ones, logits of -inf among them, against float64."""
+    import paper_2007_10412_b200 as rad
+    g = torch.Generator(device="cuda").manual_seed(B + C)
+    logits = torch.randn(B, C, generator=g, device="cuda") * 3
+    labels = torch.randint(0, C, (B,), generator=g, device="cuda", dtype=torch.int32)
+    if C > 2:
+        drop = torch.rand(B, C, generator=g, device="cuda") < 0.1
+        drop[torch.arange(B), labels.long()] = False
+        logits[drop] = float("-inf")
+    dz = torch.full((B, C), float("nan"), dtype=torch.float32 if dtype == "f32" else torch.bfloat16, device="cuda")
+    loss = torch.zeros(1, device="cuda")
+    rad.rad_softmax_xent(logits, labels, loss, dz)
+    torch.cuda.synchronize()
+    lp = torch.log_softmax(logits.double(), 1)
+    rows = torch.arange(B, device="cuda")
+    want = -lp[rows, labels.long()].mean().item()
+    ref = lp.exp()
+    ref[rows, labels.long()] -= 1
+    ref /= B
+    assert abs(loss.item() - want) <= 1e-5 * max(abs(want), 1e-3)
+    assert max(rel_err(to_host_f32(dz), ref.cpu().numpy())) <= (1e-5 if dtype == "f32" else 8e-3) or C == 1
+    if C == 1:
+        assert (dz == 0).all()
