@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/rad.h"
 
 #if defined(__CUDA_ARCH__) && (__CUDA_ARCH__ < 1000)
@@ -332,6 +334,18 @@ int launch_with_cluster(K kernel, dim3 grid, int threads, size_t smem, dim3 clus
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? RAD_OK : RAD_ECUDA;
+}
+
+// Lets `kernel` take `bytes` of dynamic shared memory on the current device, once per device (`ready`: its bits).
+template <typename K>
+bool allow_smem(K kernel, int bytes, std::atomic<uint64_t>& ready) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  const uint64_t bit = 1ull << (dev & 63);
+  if (dev < 64 && (ready.load(std::memory_order_acquire) & bit) != 0) return true;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+  if (dev < 64) ready.fetch_or(bit, std::memory_order_release);
+  return true;
 }
 
 }  // namespace rad

@@ -2,6 +2,7 @@
 // rounding, and bf16 problems whose shapes the TMA path cannot take.  These problems are small
 // and latency-bound; the kernels favour exact float32 accumulation in a fixed order over speed.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 
 #include "common.cuh"
@@ -9,12 +10,11 @@
 namespace rad {
 namespace {
 
-constexpr int kBM = 64, kBN = 64;      // the larger of the two tiles
-
 enum Epilogue { kEpiForward = 0, kEpiInputGrad = 1, kEpiScatterRows = 2 };
 
 struct GemmParams {
-  // C(m, n) = sum_k A(m, k) * Bm(k, n); element (m, k) of A at A[m * sam + k * sak], etc.
+  // C(m, n) = sum_k A(m, k) * Bm(k, n); element (m, k) of A at A[m * sam + k * sak], etc.  k is the contiguous index
+  // of A in the forward pass, of both operands in the input gradient and of neither in a scattered dW.
   const void* A; int64_t sam, sak;
   const void* Bm; int64_t sbk, sbn;
   int64_t M, N, K;
@@ -32,158 +32,366 @@ struct GemmParams {
   const uint32_t* row_idx;
   float* out_f32; int64_t ld_f32;
   float* db;                   // or NULL: column sums of Bm over k (the bias gradient), from the CTAs of tile row 0
-  int tile;                    // 64 or 32: rows and columns of C per CTA
+  // set by plan_gemm
+  int tile, splits;            // rows and columns of C per tile; CTAs (1, 2, 4 or 8) that share a tile's k
+  int vec_a, vec_b;            // 16-byte copies of the operand are aligned
+  int64_t k_per, gx, units;    // k per split, tiles per tile row, CTAs in all
 };
 
-// One TS x TS tile of C (TS = 64, or 32 where 64 would leave most SMs without a CTA) by one CTA of 256 threads,
-// TS/16 x TS/16 outputs per thread; (bx, by) = tile column and row.  The K loop is double
-// buffered: the next 16 rows of K travel from global memory to registers while the current ones are
-// multiplied out of shared memory, one barrier per step (these GEMMs serve the small nets, where a CTA's time
-// is the latency of its loads).  Every output is one chain of fused multiply-adds over k in ascending order.
-// K rows per step: the small tile takes four times as many, so that its steps, which are bound by the latency
-// of their loads, are a quarter as many.
-constexpr int gemm_bk(int ts) { return ts == 32 ? 64 : 16; }
-constexpr int kGemmSmemFloats = 4 * gemm_bk(32) * (32 + 4) > 4 * gemm_bk(64) * (64 + 4) ? 4 * gemm_bk(32) * (32 + 4)
-                                                                                         : 4 * gemm_bk(64) * (64 + 4);
-static_assert(kBM == kBN, "both operands share the staging layout");
+// Splitting a contraction over CTAs: the CTAs of a tile are neighbours in a cluster, each leaves its partial tile
+// in its own shared memory, and each then finishes (adds in split order, applies the epilogue to, writes) an equal
+// share of the tile's rows, reading the others' partial sums through distributed shared memory.
+__device__ __forceinline__ void share_barrier() {
+  if (cluster_nctas() > 1) cluster_barrier(); else __syncthreads();
+}
+__device__ __forceinline__ uint32_t cluster_rank_1d() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void copy_async16(float* dst, const float* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void copy_async4(float* dst, const float* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+
+constexpr int kGemmBK = 64;                          // k per block
+constexpr int kGemmStages = 3;                       // float32: K blocks in flight or being multiplied
+__host__ __device__ constexpr int gemm_operand_floats(int ts) { return ts * (kGemmBK + 4) > kGemmBK * (ts + 4) ? ts * (kGemmBK + 4) : kGemmBK * (ts + 4); }
+__host__ __device__ constexpr int gemm_smem_bytes(int ts) { return kGemmStages * 2 * gemm_operand_floats(ts) * 4; }
+constexpr int kGemmSmemBytes = gemm_smem_bytes(64);
+static_assert(gemm_smem_bytes(32) >= (4 * 32 * 32 + 32) * 4 && gemm_smem_bytes(64) >= (4 * 64 * 64 + 64) * 4,
+              "the partial tiles and column sums reuse the ring");
+
+// Two float32 multiply-adds per instruction (each rounded as fmaf rounds it): with one per instruction the FMA pipes
+// wait for the register file and the issue slots (4096 x 2048 x 2048: 31 TFLOP/s at 0.69 instructions per clock).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+  return v;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ void fma2(f32x2& acc, f32x2 a, f32x2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
+// Asynchronous copies of one operand's K blocks into the ring, in the layout it has in memory: TS rows of BK
+// contiguous k (kKM) or BK rows of TS contiguous columns, zeros outside the matrix and past the end of the split.
+// A thread keeps one running pointer; everything that does not change from block to block is found once.
+// kTurn: k is contiguous in memory, but the block lands as BK rows of TS columns (single elements).
+template <bool kKM, bool kTurn, int TS, int BK>
+struct BlockCopy {
+  static constexpr int kInner = kKM ? BK : TS, kLds = kTurn ? TS + 4 : kInner + 4;
+  static constexpr int kVec = TS * BK / 1024, kOne = TS * BK / 256;      // copies a thread makes per block
+  const float* src; const float* safe;
+  int64_t step, advance;
+  int o, i, fixed; uint32_t ok;
+  bool vec;
+  __device__ __forceinline__ void init(const float* X, int64_t ld, int64_t r0, int64_t rows, int64_t k0, bool vec16) {
+    vec = vec16 && !kTurn;
+    const int per_row = vec ? kInner / 4 : kInner, w = vec ? 4 : 1, ostep = 256 / per_row;
+    o = (int)threadIdx.x / per_row;
+    i = ((int)threadIdx.x % per_row) * w;
+    step = (int64_t)ostep * ld;
+    safe = X;
+    ok = 0;
+    if (kKM) {
+      for (int j = 0; j < kOne; ++j) ok |= (r0 + o + j * ostep < rows ? 1u : 0u) << j;
+      fixed = w * 4;
+      src = X + (r0 + o) * ld + k0 + i;
+      advance = BK;
+    } else {
+      const int64_t left = rows - (r0 + i);
+      fixed = left >= w ? w * 4 : left > 0 ? (int)left * 4 : 0;
+      src = X + (k0 + o) * ld + r0 + i;
+      advance = (int64_t)BK * ld;
+    }
+  }
+  template <bool kV>
+  __device__ __forceinline__ void copies(float* dst, int kleft) {
+    constexpr int per_row = kV ? kInner / 4 : kInner, ostep = 256 / per_row, w = kV ? 4 : 1;
+    float* d = kTurn ? dst + i * kLds + o : dst + o * kLds + i;
+#pragma unroll
+    for (int j = 0; j < (kV ? kVec : kOne); ++j) {
+      int bytes;
+      if (kKM) bytes = ((ok >> j) & 1u) != 0 ? min(max(kleft - i, 0), w) * 4 : 0;
+      else bytes = o + j * ostep < kleft ? fixed : 0;
+      const float* from = bytes != 0 ? src + j * step : safe;
+      if (kV) copy_async16(d + j * ostep * kLds, from, bytes); else copy_async4(d + j * ostep * (kTurn ? 1 : kLds), from, bytes);
+    }
+  }
+  __device__ __forceinline__ void issue(float* dst, int kleft) {         // kleft: k of the block inside the split, or more
+    if (!kTurn && vec) copies<true>(dst, kleft); else copies<false>(dst, kleft);
+    src += advance;
+  }
+};
+
+// One CTA's share of a TS x TS tile of C (256 threads).  Four groups of 64 threads take every fourth quartet of k of
+// a 64-deep K block; a thread of a group owns TS/8 x TS/8 outputs; the groups' tiles are added at the end.  float32
+// operands arrive through a three-deep ring of asynchronous copies (zero-filled outside the matrix), bf16 ones are
+// widened on the way through registers one block ahead.  B lies k-major in shared memory whichever way round it
+// is in memory: pairs of columns feed the paired multiply-adds without being assembled (the input gradient of
+// 4096 x 2048 x 2048: 1438 us with pairs assembled from rows, 865 with single-element copies that turn the block).
+// What bounds it: the FMA pipes and register file for layers that fill the chip (that input gradient: 1221 us
+// before; the forward pass 1175 -> 806 us, 43 TFLOP/s), else the latency of the chain load -> multiply -> add, so k
+// is split over the groups and up to eight CTAs (150 x 300 outputs, k = 784: 23.2 -> 9.3 us).  Sums over the groups and
+// splits are also several times shorter chains of roundings than one thread's walk along k.
 template <typename T, int EPI, int TS>
-__device__ __forceinline__ void gemm_body(const GemmParams& p, int64_t bx, int64_t by, float* smem) {
-  constexpr int kBM = TS, kBN = TS, TM = TS / 16, kBK = gemm_bk(TS), NF = TS * kBK / 256;
-  constexpr int kLdS = TS + 4;                       // floats per k row of a staged operand (16-byte multiples)
-  static_assert((kLdS * 4) % 16 == 0 && (TM == 4 || TM == 2), "vector reads of the staged operands");
+__device__ __forceinline__ void gemm_partial(const GemmParams& p, int64_t tile, int split, float* smem) {
+  constexpr bool kAK = EPI != kEpiScatterRows, kBK = EPI == kEpiInputGrad;      // k contiguous in memory?
+  constexpr int BK = kGemmBK, TM = TS / 8;
+  constexpr int kLdA = kAK ? BK + 4 : TS + 4, kLdB = TS + 4;                    // 16-byte multiples, conflict-free
+  constexpr int kGemmStageFloats = 2 * gemm_operand_floats(TS);
   int64_t M = p.M;
   if (p.M_dev != nullptr) M = min(M, *p.M_dev);
-  const int64_t m0 = by * kBM, n0 = bx * kBN;
-  const bool sums = EPI == kEpiScatterRows && p.db != nullptr && by == 0;
+  const int64_t m0 = (tile / p.gx) * TS, n0 = (tile % p.gx) * TS;
+  const bool sums = EPI == kEpiScatterRows && p.db != nullptr && m0 == 0;
   if (m0 >= M && !sums) return;
-  const int tid = threadIdx.x;
-  float colsum = 0.0f;
-  const int tm = (tid >> 4) * TM, tn = (tid & 15) * TM;
+  const int tid = threadIdx.x, group = tid >> 6, t = tid & 63, ty = t >> 3, tx = t & 7;
   const T* A = static_cast<const T*>(p.A);
   const T* Bm = static_cast<const T*>(p.Bm);
-  float acc[TM][TM] = {};
-  // TS x kBK elements of each operand per step; whichever index is contiguous in memory is made
-  // the fast thread index
-  float ra[NF], rb[NF];
-  auto fetch = [&](int64_t k0) {
-#pragma unroll
-    for (int j = 0; j < NF; ++j) {
-      const int i = tid + j * 256;
-      int mm, kk;
-      if (p.sak == 1) { kk = i % kBK; mm = i / kBK; } else { mm = i % kBM; kk = i / kBM; }
-      const int64_t m = m0 + mm, k = k0 + kk;
-      ra[j] = (m < M && k < p.K) ? to_float(A[m * p.sam + k * p.sak]) : 0.0f;
-      int nn;
-      if (p.sbk == 1) { kk = i % kBK; nn = i / kBK; } else { nn = i % kBN; kk = i / kBN; }
-      const int64_t n = n0 + nn, kb = k0 + kk;
-      rb[j] = (n < p.N && kb < p.K) ? to_float(Bm[kb * p.sbk + n * p.sbn]) : 0.0f;
+  const int64_t k0 = (int64_t)split * p.k_per, k1 = min(p.K, k0 + p.k_per);
+  const int nblk = k1 > k0 ? (int)((k1 - k0 + BK - 1) / BK) : 0;
+  f32x2 acc[TM][TM / 2] = {};                        // outputs in pairs of neighbouring columns j
+  float colsum = 0.0f;
+  BlockCopy<kAK, false, TS, BK> ca;
+  BlockCopy<kBK, kBK, TS, BK> cb;
+  if constexpr (sizeof(T) == 4) {
+    ca.init(reinterpret_cast<const float*>(A), kAK ? p.sam : p.sak, m0, M, k0, p.vec_a != 0);
+    cb.init(reinterpret_cast<const float*>(Bm), kBK ? p.sbn : p.sbk, n0, p.N, k0, p.vec_b != 0);
+  }
+  auto issue = [&](int kb) {
+    if constexpr (sizeof(T) == 4) {
+      if (kb < nblk) {
+        float* sA = smem + (kb % kGemmStages) * kGemmStageFloats;
+        const int kleft = (int)min((int64_t)BK, k1 - k0 - (int64_t)kb * BK);
+        ca.issue(sA, kleft);
+        cb.issue(sA + kGemmStageFloats / 2, kleft);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
     }
   };
-  auto stash = [&](int buf) {
-    float* sA = smem + buf * 2 * kBK * kLdS;
-    float* sB = sA + kBK * kLdS;
+  constexpr int NF = TS * BK / 256;
+  float ra[sizeof(T) == 2 ? NF : 1], rb[sizeof(T) == 2 ? NF : 1];
+  auto fetch = [&](int kb) {
+    if constexpr (sizeof(T) == 2) {
 #pragma unroll
-    for (int j = 0; j < NF; ++j) {
-      const int i = tid + j * 256;
-      if (p.sak == 1) sA[(i % kBK) * kLdS + i / kBK] = ra[j]; else sA[(i / kBM) * kLdS + i % kBM] = ra[j];
-      if (p.sbk == 1) sB[(i % kBK) * kLdS + i / kBK] = rb[j]; else sB[(i / kBN) * kLdS + i % kBN] = rb[j];
+      for (int j = 0; j < NF; ++j) {
+        const int c = tid + j * 256;
+        const int64_t ma = m0 + (kAK ? c / BK : c % TS), ka = k0 + (int64_t)kb * BK + (kAK ? c % BK : c / TS);
+        ra[j] = ma < M && ka < k1 ? to_float(A[ma * p.sam + ka * p.sak]) : 0.0f;
+        const int64_t nb = n0 + (kBK ? c / BK : c % TS), kk = k0 + (int64_t)kb * BK + (kBK ? c % BK : c / TS);
+        rb[j] = nb < p.N && kk < k1 ? to_float(Bm[kk * p.sbk + nb * p.sbn]) : 0.0f;
+      }
     }
   };
-  fetch(0);
-  stash(0);
+  auto stash = [&](int kb) {
+    if constexpr (sizeof(T) == 2) {
+      float* sA = smem + (kb % kGemmStages) * kGemmStageFloats;
+      float* sB = sA + kGemmStageFloats / 2;
+#pragma unroll
+      for (int j = 0; j < NF; ++j) {
+        const int c = tid + j * 256;
+        sA[(kAK ? c / BK : c / TS) * kLdA + (kAK ? c % BK : c % TS)] = ra[j];
+        sB[(kBK ? c % BK : c / TS) * kLdB + (kBK ? c / BK : c % TS)] = rb[j];
+      }
+    }
+  };
+  if constexpr (sizeof(T) == 4) {
+    for (int i = 0; i < kGemmStages - 1; ++i) issue(i);
+  } else if (nblk > 0) {
+    fetch(0);
+    stash(0);
+  }
+  for (int kb = 0; kb < nblk; ++kb) {
+    if constexpr (sizeof(T) == 4) asm volatile("cp.async.wait_group %0;" ::"n"(kGemmStages - 2) : "memory");
+    __syncthreads();                                 // block kb is in place, and everyone is done with block kb - 1
+    if constexpr (sizeof(T) == 4) issue(kb + kGemmStages - 1);
+    else if (kb + 1 < nblk) fetch(kb + 1);
+    const float* sA = smem + (kb % kGemmStages) * kGemmStageFloats;
+    const float* sB = sA + kGemmStageFloats / 2;
+    if (sums && tid < TS) {
+      // the block of Bm is in shared memory anyway: its column sums, row after row (rows past k1 hold zeros)
+#pragma unroll 8
+      for (int kk = 0; kk < BK; ++kk) colsum += sB[kk * kLdB + tid];
+    }
+    auto quartet = [&](int kc) {
+#pragma unroll
+      for (int h = 0; h < 4; h += 2) {               // two k at a time
+        float a[TM][2];
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          if (kAK) {
+            const float2 v = *reinterpret_cast<const float2*>(sA + (ty + 8 * i) * kLdA + kc + h);
+            a[i][0] = v.x; a[i][1] = v.y;
+          } else if (i % 4 == 0) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+              const float4 v = *reinterpret_cast<const float4*>(sA + (kc + h + k) * kLdA + ty * 4 + 8 * i);
+              a[i][k] = v.x; a[i + 1][k] = v.y; a[i + 2][k] = v.z; a[i + 3][k] = v.w;
+            }
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          f32x2 bb[TM / 2];
+#pragma unroll
+          for (int j = 0; j < TM / 2; j += 2) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(sB + (kc + h + k) * kLdB + tx * 4 + 16 * j);
+            bb[j] = v.x; bb[j + 1] = v.y;
+          }
+#pragma unroll
+          for (int i = 0; i < TM; ++i) {
+            const f32x2 aa = pack2(a[i][k], a[i][k]);
+#pragma unroll
+            for (int j = 0; j < TM / 2; ++j) fma2(acc[i][j], aa, bb[j]);
+          }
+        }
+      }
+    };
+    const int kvalid = (int)min((int64_t)BK, k1 - k0 - (int64_t)kb * BK);
+    if (kvalid == BK) {
+#pragma unroll
+      for (int kc = 0; kc < BK; kc += 16) quartet(kc + group * 4);
+    } else {
+#pragma unroll 1
+      for (int kc = group * 4; kc < kvalid; kc += 16) quartet(kc);
+    }
+    if constexpr (sizeof(T) == 2) {
+      if (kb + 1 < nblk) stash(kb + 1);
+    }
+  }
+  if constexpr (sizeof(T) == 4) asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  int buf = 0;
-  for (int64_t k0 = 0; k0 < p.K; k0 += kBK) {
-    const bool more = k0 + kBK < p.K;
-    if (more) fetch(k0 + kBK);
-    const float* sA = smem + buf * 2 * kBK * kLdS;
-    const float* sB = sA + kBK * kLdS;
-    if (sums && tid < kBN) {
-      // the block of Bm is in shared memory anyway: its column sums, row after row (rows past K hold zeros)
+  float* plane = smem + group * TS * TS;
 #pragma unroll
-      for (int kk = 0; kk < kBK; ++kk) colsum += sB[kk * kLdS + tid];
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TM; j += 2) {
+      const int m = kAK ? ty + 8 * i : ty * 4 + (i & 3) + 32 * (i >> 2);
+      const int n = tx * 4 + (j & 3) + 32 * (j >> 2);
+      unpack2(acc[i][j / 2], plane[m * TS + n], plane[m * TS + n + 1]);
     }
-#pragma unroll
-    for (int kk = 0; kk < kBK; ++kk) {
-      float a[TM], b[TM];
-      if (TM == 4) {
-        const float4 a4 = *reinterpret_cast<const float4*>(sA + kk * kLdS + tm);
-        const float4 b4 = *reinterpret_cast<const float4*>(sB + kk * kLdS + tn);
-        a[0] = a4.x; a[1] = a4.y; a[TM - 2] = a4.z; a[TM - 1] = a4.w;
-        b[0] = b4.x; b[1] = b4.y; b[TM - 2] = b4.z; b[TM - 1] = b4.w;
-      } else {
-        const float2 a2 = *reinterpret_cast<const float2*>(sA + kk * kLdS + tm);
-        const float2 b2 = *reinterpret_cast<const float2*>(sB + kk * kLdS + tn);
-        a[0] = a2.x; a[1] = a2.y;
-        b[0] = b2.x; b[1] = b2.y;
-      }
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TM; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    if (more) stash(buf ^ 1);
-    __syncthreads();
-    buf ^= 1;
+  if (sums && tid < TS) smem[4 * TS * TS + tid] = colsum;
+  __syncthreads();
+#pragma unroll 4
+  for (int e = tid; e < TS * TS; e += 256)
+    smem[e] = (smem[e] + smem[TS * TS + e]) + (smem[2 * TS * TS + e] + smem[3 * TS * TS + e]);
+}
+
+// The CTA's share of the tile's rows, from the partial tiles of all its splits.
+template <typename T, int EPI, int TS>
+__device__ __forceinline__ void gemm_finish(const GemmParams& p, int64_t tile, int split, const float* smem) {
+  int64_t M = p.M;
+  if (p.M_dev != nullptr) M = min(M, *p.M_dev);
+  const int64_t m0 = (tile / p.gx) * TS, n0 = (tile % p.gx) * TS;
+  const bool sums = EPI == kEpiScatterRows && p.db != nullptr && m0 == 0;
+  const int S = p.splits, rows = TS / S, tid = threadIdx.x;
+  const uint32_t rank0 = cluster_rank_1d() - (uint32_t)split;
+  if (sums && split == 0 && tid < TS && n0 + tid < p.N) {
+    float s = 0.0f;
+    for (int q = 0; q < S; ++q) s += S > 1 ? ld_cluster_f32(smem + 4 * TS * TS + tid, rank0 + q) : smem[4 * TS * TS + tid];
+    p.db[n0 + tid] = s;
   }
-  if (sums && tid < kBN && n0 + tid < p.N) p.db[n0 + tid] = colsum;
-#pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    const int64_t m = m0 + tm + i;
-    if (m >= M) continue;
-#pragma unroll
-    for (int j = 0; j < TM; ++j) {
-      const int64_t n = n0 + tn + j;
-      if (n >= p.N) continue;
-      float v = acc[i][j];
-      if (EPI == kEpiForward) {
-        if (p.bias != nullptr) v += p.bias[n];
-        if (p.out_z != nullptr) p.out_z[m * p.ld_z + n] = v;
-        if (p.out_zlow != nullptr) static_cast<T*>(p.out_zlow)[m * p.ld_zlow + n] = from_float<T>(v);
-        if (p.out_act != nullptr) {
-          const float a = p.act == RAD_ACT_RELU ? fmaxf(v, 0.0f) : p.act == RAD_ACT_GELU ? gelu_f(v) : v;
-          static_cast<T*>(p.out_act)[m * p.ld_act + n] = from_float<T>(a);
-        }
-      } else if (EPI == kEpiInputGrad) {
-        if (p.relubits != nullptr) {
-          if (((p.relubits[m * p.w32 + (n >> 5)] >> (n & 31)) & 1u) == 0) v = 0.0f;
-        } else if (p.z_prev != nullptr) {
-          v *= gelu_grad_f(to_float(static_cast<const T*>(p.z_prev)[m * p.ld_zprev + n]));
-        }
-        static_cast<T*>(p.out_low)[m * p.ld_low + n] = from_float<T>(v);
-      } else {
-        p.out_f32[(int64_t)p.row_idx[m] * p.ld_f32 + n] = v;
+  if (m0 >= M) return;
+#pragma unroll 4
+  for (int e0 = tid; e0 < rows * TS; e0 += 256) {
+    const int e = split * rows * TS + e0;
+    const int64_t m = m0 + e / TS, n = n0 + e % TS;
+    if (m >= M || n >= p.N) continue;
+    float v = 0.0f;
+    if (S > 1) {
+      for (int q = 0; q < S; ++q) v += ld_cluster_f32(smem + e, rank0 + q);
+    } else {
+      v = smem[e];
+    }
+    if (EPI == kEpiForward) {
+      if (p.bias != nullptr) v += p.bias[n];
+      if (p.out_z != nullptr) p.out_z[m * p.ld_z + n] = v;
+      if (p.out_zlow != nullptr) static_cast<T*>(p.out_zlow)[m * p.ld_zlow + n] = from_float<T>(v);
+      if (p.out_act != nullptr) {
+        const float a = p.act == RAD_ACT_RELU ? fmaxf(v, 0.0f) : p.act == RAD_ACT_GELU ? gelu_f(v) : v;
+        static_cast<T*>(p.out_act)[m * p.ld_act + n] = from_float<T>(a);
       }
+    } else if (EPI == kEpiInputGrad) {
+      if (p.relubits != nullptr) {
+        if (((p.relubits[m * p.w32 + (n >> 5)] >> (n & 31)) & 1u) == 0) v = 0.0f;
+      } else if (p.z_prev != nullptr) {
+        v *= gelu_grad_f(to_float(static_cast<const T*>(p.z_prev)[m * p.ld_zprev + n]));
+      }
+      static_cast<T*>(p.out_low)[m * p.ld_low + n] = from_float<T>(v);
+    } else {
+      p.out_f32[(int64_t)p.row_idx[m] * p.ld_f32 + n] = v;
     }
   }
 }
 
-// The tile a GEMM of M x N outputs runs with, and the body for it.
-inline int pick_tile(int64_t M, int64_t N) { return ceil_div(M, 64) * ceil_div(N, 64) < 64 ? 32 : 64; }
+// Tile and split of a contraction: the pair with the least estimated time, in clocks of the SM that gets the most
+// CTAs.  Two CTAs share an SM; per k of its share a pair takes 106 clocks with 64 x 64 tiles and 35 with 32 x 32
+// (0.60 and 0.46 of the FMA rate), a CTA alone 73 and 26; beginning and end of a CTA (first loads, the groups'
+// sums, epilogue) take 6000 and 3850, the launch 4000, the exchange inside a cluster 800.  Fitted to 32 timings
+// (both tiles, 1 to 8 splits); for 150 x 300 outputs it says 28 / 19 / 19 / 22 thousand clocks for 1 / 2 / 4 / 8 CTAs
+// per 32 x 32 tile at k = 784, measured 26 / 19 / 18 / 23; for 1500 x 777, k = 1001, 102 / 91 / 94 us for 1 / 2 / 4 CTAs
+// per 64 x 64 tile, measured 112 / 101 / 102.
+inline void plan_gemm(GemmParams& p, int64_t Mgrid, int es) {
+  double best = 1e300;
+  for (int ts = 32; ts <= 64; ts *= 2) {
+    const int64_t tiles = std::max<int64_t>(1, ceil_div(Mgrid, ts)) * ceil_div(p.N, ts);
+    const double pair = ts == 64 ? 106.0 : 35.0, alone = ts == 64 ? 73.0 : 26.0, ends = ts == 64 ? 6000.0 : 3850.0;
+    for (int s = 1; s <= 8; s *= 2) {
+      if (s > 1 && p.K / s < 16) break;
+      const int64_t per_sm = ceil_div(tiles * s, 148), k_per = round_up(ceil_div(p.K, s), 4);
+      const double clk = (double)k_per * ((double)(per_sm / 2) * pair + (double)(per_sm % 2) * alone) + (double)per_sm * ends + 4000.0 +
+                         (s > 1 ? 800.0 : 0.0);
+      if (clk < best) {
+        best = clk;
+        p.tile = ts; p.splits = s; p.k_per = k_per;
+        p.gx = ceil_div(p.N, ts); p.units = tiles * s;
+      }
+    }
+  }
+  const bool ak = p.sak == 1, bk = p.sbk == 1 && p.sbn != 1;
+  p.vec_a = es == 4 && ((uintptr_t)p.A & 15) == 0 && (ak ? p.sam : p.sak) % 4 == 0;
+  p.vec_b = es == 4 && ((uintptr_t)p.Bm & 15) == 0 && (bk ? p.sbn : p.sbk) % 4 == 0;
+}
 template <typename T, int EPI>
-__device__ __forceinline__ void gemm_tile(const GemmParams& p, int64_t bx, int64_t by, float* smem) {
-  if (p.tile == 32) gemm_body<T, EPI, 32>(p, bx, by, smem);
-  else gemm_body<T, EPI, 64>(p, bx, by, smem);
+__device__ __forceinline__ void gemm_unit_partial(const GemmParams& p, int64_t unit, float* smem) {
+  if (unit >= p.units) return;
+  if (p.tile == 32) gemm_partial<T, EPI, 32>(p, unit / p.splits, (int)(unit % p.splits), smem);
+  else gemm_partial<T, EPI, 64>(p, unit / p.splits, (int)(unit % p.splits), smem);
+}
+template <typename T, int EPI>
+__device__ __forceinline__ void gemm_unit_finish(const GemmParams& p, int64_t unit, const float* smem) {
+  if (unit >= p.units) return;
+  if (p.tile == 32) gemm_finish<T, EPI, 32>(p, unit / p.splits, (int)(unit % p.splits), smem);
+  else gemm_finish<T, EPI, 64>(p, unit / p.splits, (int)(unit % p.splits), smem);
 }
 
 template <typename T, int EPI>
-__global__ void __launch_bounds__(256) gemm_kernel(const GemmParams p) {
-  __shared__ __align__(16) float smem[kGemmSmemFloats];
-  gemm_tile<T, EPI>(p, blockIdx.x, blockIdx.y, smem);
+__global__ void __launch_bounds__(256, 2) gemm_kernel(const GemmParams p) {
+  extern __shared__ __align__(16) float smem[];
+  gemm_unit_partial<T, EPI>(p, blockIdx.x, smem);
+  share_barrier();
+  gemm_unit_finish<T, EPI>(p, blockIdx.x, smem);
+  if (cluster_nctas() > 1) cluster_barrier();        // no CTA leaves while another reads its partial tile
 }
 
 template <int EPI>
 int launch_gemm(int dtype, const GemmParams& p0, int64_t Mgrid, cudaStream_t s) {
   GemmParams p = p0;
-  p.tile = pick_tile(Mgrid, p.N);
-  dim3 grid((unsigned)ceil_div(p.N, p.tile), (unsigned)ceil_div(Mgrid, p.tile));
-  if (grid.x == 0 || grid.y == 0) return RAD_OK;
+  plan_gemm(p, Mgrid, dtype == RAD_BF16 ? 2 : 4);
+  if (p.units > 0x7fffffff) return RAD_EINVAL;
   count_launch();
-  if (dtype == RAD_BF16)
-    gemm_kernel<bf16, EPI><<<grid, 256, 0, s>>>(p);
-  else
-    gemm_kernel<float, EPI><<<grid, 256, 0, s>>>(p);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  if (dtype == RAD_BF16) {
+    static std::atomic<uint64_t> ready{0};
+    if (!allow_smem(gemm_kernel<bf16, EPI>, kGemmSmemBytes, ready)) return RAD_ECUDA;
+    return launch_with_cluster(gemm_kernel<bf16, EPI>, dim3((unsigned)p.units), 256, (size_t)gemm_smem_bytes(p.tile), dim3(p.splits), s, p);
+  }
+  static std::atomic<uint64_t> ready{0};
+  if (!allow_smem(gemm_kernel<float, EPI>, kGemmSmemBytes, ready)) return RAD_ECUDA;
+  return launch_with_cluster(gemm_kernel<float, EPI>, dim3((unsigned)p.units), 256, (size_t)gemm_smem_bytes(p.tile), dim3(p.splits), s, p);
 }
 
 // relubits[b, w] = bits of (X[b, 32w..] > 0)
@@ -214,6 +422,7 @@ struct SparseDwParams {
   const void* dZ; int64_t ldz;
   float* dW; int64_t ldw;
   float* db;                 // or NULL: column sums of dZ (the bias gradient), from the CTAs of column block 0
+  int32_t units;             // CTAs
 };
 
 template <typename T>
@@ -304,18 +513,23 @@ __global__ void __launch_bounds__(256) sparse_dw_kernel(const SparseDwParams p) 
 // input-gradient GEMM, each doing exactly what it does in a launch of its own (the nets that run on CUDA
 // cores are bound by their launch count).
 constexpr int kDwDxSmemA = kTileRows * (kTileCols + 1) * 4, kDwDxSmemZ = kTileRows * (kSparseBN + 1) * 4;
-static_assert(kDwDxSmemA + kDwDxSmemZ + 1024 >= kGemmSmemFloats * 4, "the GEMM's tiles fit the same buffer");
+static_assert(kDwDxSmemA + kDwDxSmemZ + 1024 <= kGemmSmemBytes, "the sparse tiles fit the GEMM's buffer");
 template <typename T>
-__global__ void __launch_bounds__(256) dw_dx_kernel(const SparseDwParams d, const GemmParams g, int dw_blocks, int gx) {
-  __shared__ __align__(16) unsigned char raw[kDwDxSmemA + kDwDxSmemZ + 1024];
-  if ((int)blockIdx.x < dw_blocks) {
-    sparse_dw_body<T>(d, (int)(blockIdx.x % d.ncb), blockIdx.x / d.ncb, reinterpret_cast<float(*)[kTileCols + 1]>(raw),
-                      reinterpret_cast<float(*)[kSparseBN + 1]>(raw + kDwDxSmemA),
-                      reinterpret_cast<uint32_t*>(raw + kDwDxSmemA + kDwDxSmemZ));
+__global__ void __launch_bounds__(256, 2) dw_dx_kernel(const SparseDwParams d, const GemmParams g, int dw_blocks) {
+  extern __shared__ __align__(16) float smem[];
+  unsigned char* raw = reinterpret_cast<unsigned char*>(smem);
+  const int b = (int)blockIdx.x, gu = b - dw_blocks;
+  if (b < dw_blocks) {
+    if (b < d.units)
+      sparse_dw_body<T>(d, b % d.ncb, b / d.ncb, reinterpret_cast<float(*)[kTileCols + 1]>(raw),
+                        reinterpret_cast<float(*)[kSparseBN + 1]>(raw + kDwDxSmemA),
+                        reinterpret_cast<uint32_t*>(raw + kDwDxSmemA + kDwDxSmemZ));
   } else {
-    const int b = (int)blockIdx.x - dw_blocks;
-    gemm_tile<T, kEpiInputGrad>(g, b % gx, b / gx, reinterpret_cast<float*>(raw));
+    gemm_unit_partial<T, kEpiInputGrad>(g, gu, smem);
   }
+  share_barrier();
+  if (b >= dw_blocks) gemm_unit_finish<T, kEpiInputGrad>(g, gu, smem);
+  if (cluster_nctas() > 1) cluster_barrier();
 }
 
 __global__ void zero_rows_kernel(float* dW, int64_t ldw, int64_t D, int64_t H) {
@@ -444,15 +658,16 @@ int column_sums_of(const T* dZ, int64_t ldz, int64_t B, int64_t H, float* out, f
 // The same for a same-sample store (Sec. 4.3): the first CTAs scatter A_c^T dZ into the kept rows of dW (and
 // leave the bias gradient), the next ones make the input gradient, the last ones write zeros to the rows of dW
 // whose column was not kept (bit d of keep_cols clear), which the scatter never touches.
+// The parts begin at multiples of the cluster size.
 template <typename T>
-__global__ void __launch_bounds__(256) same_dw_dx_kernel(const GemmParams w, const GemmParams g, int dw_blocks, int gxw,
-                                                         int dx_blocks, int gxg, const uint32_t* keep_cols, int64_t D, int64_t H) {
-  __shared__ __align__(16) float smem[kGemmSmemFloats];
+__global__ void __launch_bounds__(256, 2) same_dw_dx_kernel(const GemmParams w, const GemmParams g, int dw_blocks, int dx_blocks,
+                                                            const uint32_t* keep_cols, int64_t D, int64_t H) {
+  extern __shared__ __align__(16) float smem[];
   const int b = (int)blockIdx.x;
   if (b < dw_blocks) {
-    gemm_tile<T, kEpiScatterRows>(w, b % gxw, b / gxw, smem);
+    gemm_unit_partial<T, kEpiScatterRows>(w, b, smem);
   } else if (b < dw_blocks + dx_blocks) {
-    gemm_tile<T, kEpiInputGrad>(g, (b - dw_blocks) % gxg, (b - dw_blocks) / gxg, smem);
+    gemm_unit_partial<T, kEpiInputGrad>(g, b - dw_blocks, smem);
   } else {
     const int nz = (int)gridDim.x - dw_blocks - dx_blocks;
     for (int64_t d = b - dw_blocks - dx_blocks; d < D; d += nz) {
@@ -460,6 +675,10 @@ __global__ void __launch_bounds__(256) same_dw_dx_kernel(const GemmParams w, con
       for (int64_t h = threadIdx.x; h < H; h += 256) w.out_f32[d * w.ld_f32 + h] = 0.0f;
     }
   }
+  share_barrier();
+  if (b < dw_blocks) gemm_unit_finish<T, kEpiScatterRows>(w, b, smem);
+  else if (b < dw_blocks + dx_blocks) gemm_unit_finish<T, kEpiInputGrad>(g, b - dw_blocks, smem);
+  if (cluster_nctas() > 1) cluster_barrier();
 }
 
 int simt_forward(int dtype, int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t lda,
@@ -524,25 +743,28 @@ int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H
     p.row_idx = st->offsets; p.out_f32 = dW; p.ld_f32 = ldw;
     p.db = db;
     if (db_written != nullptr) *db_written = db != nullptr;
-    p.tile = pick_tile(p.M, p.N);
-    const int64_t gxw = ceil_div(p.N, p.tile), dw_blocks = gxw * std::max<int64_t>(1, ceil_div(p.M, p.tile));
+    const int es = st->dtype == RAD_BF16 ? 2 : 4;
+    plan_gemm(p, p.M, es);
     if (st->keepbits != nullptr) {
       // one launch: scatter, zeros for the rows not kept and, where asked for, the input gradient
       const bool with_dx = ig != nullptr && ig_done != nullptr;
       GemmParams g = with_dx ? input_grad_params(st->B, st->D, H, dZ, ldz, *ig) : GemmParams{};
-      g.tile = with_dx ? pick_tile(g.M, g.N) : 64;
-      const int64_t gxg = with_dx ? ceil_div(g.N, g.tile) : 1, dx_blocks = with_dx ? gxg * ceil_div(g.M, g.tile) : 0;
-      const int64_t nz = std::min<int64_t>(st->D, 148 * 4);
+      if (with_dx) plan_gemm(g, g.M, es);
+      const int64_t cluster = std::max(p.splits, with_dx ? g.splits : 1);
+      const int64_t dw_blocks = round_up(p.units, cluster), dx_blocks = with_dx ? round_up(g.units, cluster) : 0;
+      const int64_t nz = round_up(std::min<int64_t>(st->D, 148 * 2), cluster);
       if (dw_blocks + dx_blocks + nz <= 0x7fffffff) {
+        static std::atomic<uint64_t> ready_b{0}, ready_f{0};
+        const dim3 grid((unsigned)(dw_blocks + dx_blocks + nz)), cl((unsigned)cluster);
         count_launch();
-        if (st->dtype == RAD_BF16)
-          same_dw_dx_kernel<bf16><<<(unsigned)(dw_blocks + dx_blocks + nz), 256, 0, s>>>(p, g, (int)dw_blocks, (int)gxw, (int)dx_blocks,
-                                                                                          (int)gxg, st->keepbits, st->D, H);
-        else
-          same_dw_dx_kernel<float><<<(unsigned)(dw_blocks + dx_blocks + nz), 256, 0, s>>>(p, g, (int)dw_blocks, (int)gxw, (int)dx_blocks,
-                                                                                           (int)gxg, st->keepbits, st->D, H);
         if (with_dx) *ig_done = true;
-        return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+        if (st->dtype == RAD_BF16)
+          return !allow_smem(same_dw_dx_kernel<bf16>, kGemmSmemBytes, ready_b) ? RAD_ECUDA
+                 : launch_with_cluster(same_dw_dx_kernel<bf16>, grid, 256, kGemmSmemBytes, cl, s, p, g, (int)dw_blocks, (int)dx_blocks,
+                                       (const uint32_t*)st->keepbits, st->D, H);
+        return !allow_smem(same_dw_dx_kernel<float>, kGemmSmemBytes, ready_f) ? RAD_ECUDA
+               : launch_with_cluster(same_dw_dx_kernel<float>, grid, 256, kGemmSmemBytes, cl, s, p, g, (int)dw_blocks, (int)dx_blocks,
+                                     (const uint32_t*)st->keepbits, st->D, H);
       }
     }
     const int g = (int)std::min<int64_t>(ceil_div(st->D * H, 256), 148 * 16);
@@ -562,15 +784,18 @@ int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H
   count_launch();
   if (ig != nullptr && ig_done != nullptr) {
     GemmParams g = input_grad_params(st->B, st->D, H, dZ, ldz, *ig);
-    g.tile = pick_tile(g.M, g.N);
-    const int64_t gx = ceil_div(g.N, g.tile), gy = ceil_div(g.M, g.tile), dw_blocks = (int64_t)grid.x * grid.y;
-    if (dw_blocks + gx * gy <= 0x7fffffff) {
-      if (st->dtype == RAD_BF16)
-        dw_dx_kernel<bf16><<<(unsigned)(dw_blocks + gx * gy), 256, 0, s>>>(p, g, (int)dw_blocks, (int)gx);
-      else
-        dw_dx_kernel<float><<<(unsigned)(dw_blocks + gx * gy), 256, 0, s>>>(p, g, (int)dw_blocks, (int)gx);
+    plan_gemm(g, g.M, st->dtype == RAD_BF16 ? 2 : 4);
+    const int64_t units = (int64_t)grid.x * grid.y, dw_blocks = round_up(units, g.splits);
+    if (dw_blocks + g.units <= 0x7fffffff) {
+      static std::atomic<uint64_t> ready_b{0}, ready_f{0};
+      p.units = (int32_t)units;
       *ig_done = true;
-      return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+      const dim3 all((unsigned)(dw_blocks + g.units)), cl((unsigned)g.splits);
+      if (st->dtype == RAD_BF16)
+        return !allow_smem(dw_dx_kernel<bf16>, kGemmSmemBytes, ready_b) ? RAD_ECUDA
+               : launch_with_cluster(dw_dx_kernel<bf16>, all, 256, kGemmSmemBytes, cl, s, p, g, (int)dw_blocks);
+      return !allow_smem(dw_dx_kernel<float>, kGemmSmemBytes, ready_f) ? RAD_ECUDA
+             : launch_with_cluster(dw_dx_kernel<float>, all, 256, kGemmSmemBytes, cl, s, p, g, (int)dw_blocks);
     }
   }
   if (st->dtype == RAD_BF16)

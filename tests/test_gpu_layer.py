@@ -198,3 +198,33 @@ def test_softmax_xent_over_clusters_and_row_lengths(B, C, dtype):
     assert max(rel_err(to_host_f32(dz), ref.cpu().numpy())) <= (1e-5 if dtype == "f32" else 8e-3) or C == 1
     if C == 1:
         assert (dz == 0).all()
+
+
+@pytest.mark.parametrize("B,D,H,dtype", [(1, 1, 1, "f32"), (33, 130, 31, "f32"), (65, 1001, 33, "f32"), (150, 784, 300, "f32"),
+                                         (700, 257, 203, "f32"), (2000, 68, 1500, "f32"), (129, 3000, 70, "f32"),
+                                         (90, 100, 30, "bf16"), (700, 515, 333, "bf16")])
+def test_cuda_core_contractions_over_tiles_and_splits(B, D, H, dtype):
+    """Forward, input gradient and same-sample weight gradient on CUDA cores, from one CTA to clusters that share the
+    contraction index, 32 and 64 wide tiles with remainders, aligned and odd leading dimensions, against float64.
+    Bound per output: sqrt(K) + 16 roundings of 2^-24 of the sum of magnitudes, plus one bf16 rounding of the result."""
+    import paper_2007_10412_b200 as rad
+    tdt = torch.float32 if dtype == "f32" else torch.bfloat16
+    g = torch.Generator(device="cuda").manual_seed(B + D + H)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").to(tdt)
+    A, W, dZ = rnd(B, D), rnd(D, H), rnd(B, H)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = torch.full((B, H), float("nan"), dtype=torch.float32, device="cuda")
+    rad.rad_linear_forward(A, W, None, "none", out_z=out, dev_status=status)
+    dX = torch.full((B, D), float("nan"), dtype=tdt, device="cuda")
+    rad.rad_linear_input_grad(dZ, W, dZ_prev=dX, dev_status=status)
+    st = rad.Store("same", dtype, B, D, 1.0, relu_bits=False)
+    rad.rad_linear_forward_store(A, st, status)
+    dW = torch.full((D, H), float("nan"), dtype=torch.float32, device="cuda")
+    rad.rad_linear_weight_grad(st, dZ, dW, dev_status=status)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    A, W, dZ = A.double(), W.double(), dZ.double()
+    for got, x, y, low in ((out, A, W, False), (dX, dZ, W.T, dtype == "bf16"), (dW, A.T, dZ, False)):
+        ref, mag, K = x @ y, x.abs() @ y.abs(), x.shape[1]
+        bound = (K ** 0.5 + 16) * 2.0 ** -24 * mag + (2.0 ** -8 * ref.abs() if low else 0)
+        assert ((got.double() - ref).abs() <= bound + 1e-30).all()
