@@ -10,11 +10,11 @@
 namespace rad {
 namespace {
 
-enum Epilogue { kEpiForward = 0, kEpiInputGrad = 1, kEpiScatterRows = 2 };
+enum Epilogue { kEpiForward = 0, kEpiInputGrad = 1, kEpiScatterRows = 2, kEpiSparse = 3 };
 
 struct GemmParams {
   // C(m, n) = sum_k A(m, k) * Bm(k, n); element (m, k) of A at A[m * sam + k * sak], etc.  k is the contiguous index
-  // of A in the forward pass, of both operands in the input gradient and of neither in a scattered dW.
+  // of A in the forward pass, of both operands in the input gradient and of neither in a dW.
   const void* A; int64_t sam, sak;
   const void* Bm; int64_t sbk, sbn;
   int64_t M, N, K;
@@ -32,6 +32,8 @@ struct GemmParams {
   const uint32_t* row_idx;
   float* out_f32; int64_t ld_f32;
   float* db;                   // or NULL: column sums of Bm over k (the bias gradient), from the CTAs of tile row 0
+  // different-sample dW: A(m, k) = column m of row k of a compact store, whose packed values are `A`
+  const uint32_t* keepbits; const uint32_t* offsets; int64_t capacity; int32_t ncb;
   // set by plan_gemm
   int tile, splits;            // rows and columns of C per tile; CTAs (1, 2, 4 or 8) that share a tile's k
   int vec_a, vec_b;            // 16-byte copies of the operand are aligned
@@ -128,6 +130,50 @@ struct BlockCopy {
   }
 };
 
+// The A operand of a different-sample dW: K block = one slab of 64 rows of the store, TS of a store tile's 128 columns,
+// expanded on the way into the ring (every entry is a four-byte copy, of nothing where it was not kept).  A thread
+// takes every fourth column of one row, so that a warp's copies fall on all banks; a value's place is the row's
+// offset plus the kept entries before it.  The index words of the next slab are in registers before they are needed.
+// 1500 x 1001 x 777: 89 us at any keep probability, 172 (p = 0.1) to 385 us (p = 1) with a tile rebuilt by popcounts
+// between two barriers and four scalar shared-memory reads per operand; 4096 x 128 x 10 bf16: 356 -> 19 us (its 64 slabs
+// were one CTA's walk).  A walk over per-column lists of kept rows (no zeros multiplied) was slower from p = 0.1 up:
+// 95 / 274 / 554 us at p = 0.1 / 0.5 / 1 on the first shape.
+template <typename T, int TS>
+struct SparseCopy {
+  static constexpr int kN = TS / 4, kWords = TS / 32;
+  const uint32_t* tile; const uint32_t* offset; const T* values;
+  int64_t capacity, tile_step; int ncb, w0, r, q;
+  uint32_t word[kWords]; int64_t at[kWords];
+  __device__ __forceinline__ void init(const GemmParams& p, int64_t m0, int64_t k0) {
+    const int64_t t = k0 / kTileRows * p.ncb + m0 / kTileCols;
+    r = (int)threadIdx.x >> 2; q = (int)threadIdx.x & 3;
+    w0 = (int)(m0 % kTileCols) / 32;
+    tile = p.keepbits + t * kTileWords; offset = p.offsets + t;
+    ncb = p.ncb; tile_step = (int64_t)p.ncb * kTileWords;
+    values = static_cast<const T*>(p.A); capacity = p.capacity;
+  }
+  __device__ __forceinline__ void load_index() {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = tile[4 * r + i];
+    int64_t pos = (int64_t)*offset + ((tile[kBitWords + (r >> 1)] >> (16 * (r & 1))) & 0xffffu);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+#pragma unroll
+      for (int j = 0; j < kWords; ++j)
+        if (i == w0 + j) { word[j] = w[i]; at[j] = pos; }
+      pos += __popc(w[i]);
+    }
+    tile += tile_step; offset += ncb;
+  }
+  // place of element j (column q + 4 j of the TS), or -1 where it was not kept or lies past the store's capacity
+  __device__ __forceinline__ int64_t place(int j) const {
+    const uint32_t bit = 1u << (q + 4 * (j & 7));
+    const int64_t pos = at[j >> 3] + __popc(word[j >> 3] & (bit - 1));
+    return (word[j >> 3] & bit) != 0 && pos < capacity ? pos : -1;
+  }
+};
+
 // One CTA's share of a TS x TS tile of C (256 threads).  Four groups of 64 threads take every fourth quartet of k of
 // a 64-deep K block; a thread of a group owns TS/8 x TS/8 outputs; the groups' tiles are added at the end.  float32
 // operands arrive through a three-deep ring of asynchronous copies (zero-filled outside the matrix), bf16 ones are
@@ -140,14 +186,15 @@ struct BlockCopy {
 // splits are also several times shorter chains of roundings than one thread's walk along k.
 template <typename T, int EPI, int TS>
 __device__ __forceinline__ void gemm_partial(const GemmParams& p, int64_t tile, int split, float* smem) {
-  constexpr bool kAK = EPI != kEpiScatterRows, kBK = EPI == kEpiInputGrad;      // k contiguous in memory?
+  constexpr bool kSparse = EPI == kEpiSparse;
+  constexpr bool kAK = EPI == kEpiForward || EPI == kEpiInputGrad, kBK = EPI == kEpiInputGrad;      // k contiguous in memory?
   constexpr int BK = kGemmBK, TM = TS / 8;
   constexpr int kLdA = kAK ? BK + 4 : TS + 4, kLdB = TS + 4;                    // 16-byte multiples, conflict-free
   constexpr int kGemmStageFloats = 2 * gemm_operand_floats(TS);
   int64_t M = p.M;
   if (p.M_dev != nullptr) M = min(M, *p.M_dev);
   const int64_t m0 = (tile / p.gx) * TS, n0 = (tile % p.gx) * TS;
-  const bool sums = EPI == kEpiScatterRows && p.db != nullptr && m0 == 0;
+  const bool sums = (EPI == kEpiScatterRows || EPI == kEpiSparse) && p.db != nullptr && m0 == 0;
   if (m0 >= M && !sums) return;
   const int tid = threadIdx.x, group = tid >> 6, t = tid & 63, ty = t >> 3, tx = t & 7;
   const T* A = static_cast<const T*>(p.A);
@@ -158,8 +205,14 @@ __device__ __forceinline__ void gemm_partial(const GemmParams& p, int64_t tile, 
   float colsum = 0.0f;
   BlockCopy<kAK, false, TS, BK> ca;
   BlockCopy<kBK, kBK, TS, BK> cb;
+  SparseCopy<T, TS> cs;
+  static_assert(!kSparse || BK == kTileRows, "a K block of a different-sample dW is a slab of the store");
+  if constexpr (kSparse) {
+    cs.init(p, m0, k0);
+    if (nblk > 0) cs.load_index();
+  }
   if constexpr (sizeof(T) == 4) {
-    ca.init(reinterpret_cast<const float*>(A), kAK ? p.sam : p.sak, m0, M, k0, p.vec_a != 0);
+    if (!kSparse) ca.init(reinterpret_cast<const float*>(A), kAK ? p.sam : p.sak, m0, M, k0, p.vec_a != 0);
     cb.init(reinterpret_cast<const float*>(Bm), kBK ? p.sbn : p.sbk, n0, p.N, k0, p.vec_b != 0);
   }
   auto issue = [&](int kb) {
@@ -167,7 +220,16 @@ __device__ __forceinline__ void gemm_partial(const GemmParams& p, int64_t tile, 
       if (kb < nblk) {
         float* sA = smem + (kb % kGemmStages) * kGemmStageFloats;
         const int kleft = (int)min((int64_t)BK, k1 - k0 - (int64_t)kb * BK);
-        ca.issue(sA, kleft);
+        if constexpr (kSparse) {
+#pragma unroll
+          for (int j = 0; j < cs.kN; ++j) {
+            const int64_t at = cs.place(j);
+            copy_async4(sA + cs.r * kLdA + cs.q + 4 * j, reinterpret_cast<const float*>(cs.values) + (at >= 0 ? at : 0), at >= 0 ? 4 : 0);
+          }
+          if (kb + 1 < nblk) cs.load_index();
+        } else {
+          ca.issue(sA, kleft);
+        }
         cb.issue(sA + kGemmStageFloats / 2, kleft);
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
@@ -180,10 +242,18 @@ __device__ __forceinline__ void gemm_partial(const GemmParams& p, int64_t tile, 
 #pragma unroll
       for (int j = 0; j < NF; ++j) {
         const int c = tid + j * 256;
-        const int64_t ma = m0 + (kAK ? c / BK : c % TS), ka = k0 + (int64_t)kb * BK + (kAK ? c % BK : c / TS);
-        ra[j] = ma < M && ka < k1 ? to_float(A[ma * p.sam + ka * p.sak]) : 0.0f;
+        if constexpr (kSparse) {
+          const int64_t at = cs.place(j);
+          ra[j] = at >= 0 ? to_float(cs.values[at]) : 0.0f;
+        } else {
+          const int64_t ma = m0 + (kAK ? c / BK : c % TS), ka = k0 + (int64_t)kb * BK + (kAK ? c % BK : c / TS);
+          ra[j] = ma < M && ka < k1 ? to_float(A[ma * p.sam + ka * p.sak]) : 0.0f;
+        }
         const int64_t nb = n0 + (kBK ? c / BK : c % TS), kk = k0 + (int64_t)kb * BK + (kBK ? c % BK : c / TS);
         rb[j] = nb < p.N && kk < k1 ? to_float(Bm[kk * p.sbk + nb * p.sbn]) : 0.0f;
+      }
+      if constexpr (kSparse) {
+        if (kb + 1 < nblk) cs.load_index();
       }
     }
   };
@@ -194,7 +264,8 @@ __device__ __forceinline__ void gemm_partial(const GemmParams& p, int64_t tile, 
 #pragma unroll
       for (int j = 0; j < NF; ++j) {
         const int c = tid + j * 256;
-        sA[(kAK ? c / BK : c / TS) * kLdA + (kAK ? c % BK : c % TS)] = ra[j];
+        if (kSparse) sA[cs.r * kLdA + cs.q + 4 * j] = ra[j];
+        else sA[(kAK ? c / BK : c / TS) * kLdA + (kAK ? c % BK : c % TS)] = ra[j];
         sB[(kBK ? c % BK : c / TS) * kLdB + (kBK ? c / BK : c % TS)] = rb[j];
       }
     }
@@ -287,7 +358,7 @@ __device__ __forceinline__ void gemm_finish(const GemmParams& p, int64_t tile, i
   int64_t M = p.M;
   if (p.M_dev != nullptr) M = min(M, *p.M_dev);
   const int64_t m0 = (tile / p.gx) * TS, n0 = (tile % p.gx) * TS;
-  const bool sums = EPI == kEpiScatterRows && p.db != nullptr && m0 == 0;
+  const bool sums = (EPI == kEpiScatterRows || EPI == kEpiSparse) && p.db != nullptr && m0 == 0;
   const int S = p.splits, rows = TS / S, tid = threadIdx.x;
   const uint32_t rank0 = cluster_rank_1d() - (uint32_t)split;
   if (sums && split == 0 && tid < TS && n0 + tid < p.N) {
@@ -323,7 +394,7 @@ __device__ __forceinline__ void gemm_finish(const GemmParams& p, int64_t tile, i
       }
       static_cast<T*>(p.out_low)[m * p.ld_low + n] = from_float<T>(v);
     } else {
-      p.out_f32[(int64_t)p.row_idx[m] * p.ld_f32 + n] = v;
+      p.out_f32[(EPI == kEpiScatterRows ? (int64_t)p.row_idx[m] : m) * p.ld_f32 + n] = v;
     }
   }
 }
@@ -335,14 +406,14 @@ __device__ __forceinline__ void gemm_finish(const GemmParams& p, int64_t tile, i
 // (both tiles, 1 to 8 splits); for 150 x 300 outputs it says 28 / 19 / 19 / 22 thousand clocks for 1 / 2 / 4 / 8 CTAs
 // per 32 x 32 tile at k = 784, measured 26 / 19 / 18 / 23; for 1500 x 777, k = 1001, 102 / 91 / 94 us for 1 / 2 / 4 CTAs
 // per 64 x 64 tile, measured 112 / 101 / 102.
-inline void plan_gemm(GemmParams& p, int64_t Mgrid, int es) {
+inline void plan_gemm(GemmParams& p, int64_t Mgrid, int es, int64_t k_step = 4) {      // splits begin at multiples of k_step
   double best = 1e300;
   for (int ts = 32; ts <= 64; ts *= 2) {
     const int64_t tiles = std::max<int64_t>(1, ceil_div(Mgrid, ts)) * ceil_div(p.N, ts);
     const double pair = ts == 64 ? 106.0 : 35.0, alone = ts == 64 ? 73.0 : 26.0, ends = ts == 64 ? 6000.0 : 3850.0;
     for (int s = 1; s <= 8; s *= 2) {
-      if (s > 1 && p.K / s < 16) break;
-      const int64_t per_sm = ceil_div(tiles * s, 148), k_per = round_up(ceil_div(p.K, s), 4);
+      if (s > 1 && (p.K < 16 * s || p.K <= s / 2 * k_step)) break;
+      const int64_t per_sm = ceil_div(tiles * s, 148), k_per = round_up(ceil_div(p.K, s), k_step);
       const double clk = (double)k_per * ((double)(per_sm / 2) * pair + (double)(per_sm % 2) * alone) + (double)per_sm * ends + 4000.0 +
                          (s > 1 ? 800.0 : 0.0);
       if (clk < best) {
@@ -379,9 +450,7 @@ __global__ void __launch_bounds__(256, 2) gemm_kernel(const GemmParams p) {
 }
 
 template <int EPI>
-int launch_gemm(int dtype, const GemmParams& p0, int64_t Mgrid, cudaStream_t s) {
-  GemmParams p = p0;
-  plan_gemm(p, Mgrid, dtype == RAD_BF16 ? 2 : 4);
+int launch_planned(int dtype, const GemmParams& p, cudaStream_t s) {
   if (p.units > 0x7fffffff) return RAD_EINVAL;
   count_launch();
   if (dtype == RAD_BF16) {
@@ -392,6 +461,13 @@ int launch_gemm(int dtype, const GemmParams& p0, int64_t Mgrid, cudaStream_t s) 
   static std::atomic<uint64_t> ready{0};
   if (!allow_smem(gemm_kernel<float, EPI>, kGemmSmemBytes, ready)) return RAD_ECUDA;
   return launch_with_cluster(gemm_kernel<float, EPI>, dim3((unsigned)p.units), 256, (size_t)gemm_smem_bytes(p.tile), dim3(p.splits), s, p);
+}
+
+template <int EPI>
+int launch_gemm(int dtype, const GemmParams& p0, int64_t Mgrid, cudaStream_t s) {
+  GemmParams p = p0;
+  plan_gemm(p, Mgrid, dtype == RAD_BF16 ? 2 : 4);
+  return launch_planned<EPI>(dtype, p, s);
 }
 
 // relubits[b, w] = bits of (X[b, 32w..] > 0)
@@ -410,125 +486,19 @@ __global__ void __launch_bounds__(256) relu_bits_rows_kernel(const T* X, int64_t
   }
 }
 
-// ---- different-sample dW on CUDA cores ----------------------------------------------------------
-// One CTA owns 128 columns d of the layer input (one column block) and 32 outputs h.  Per row slab
-// it rebuilds the 64 x 128 tile of A_hat in shared memory from keep bits and packed values
-// (per-word popcount prefix), then accumulates A_hat^T dZ.
-constexpr int kSparseBN = 32;
-struct SparseDwParams {
-  const void* values; const uint32_t* keepbits; const uint32_t* offsets;
-  int64_t capacity;
-  int64_t B, D, H; int32_t ncb, nslabs;
-  const void* dZ; int64_t ldz;
-  float* dW; int64_t ldw;
-  float* db;                 // or NULL: column sums of dZ (the bias gradient), from the CTAs of column block 0
-  int32_t units;             // CTAs
-};
-
-template <typename T>
-__device__ __forceinline__ void sparse_dw_body(const SparseDwParams& p, int cb, int64_t by, float (*sAh)[kTileCols + 1],
-                                               float (*sZ)[kSparseBN + 1], uint32_t* s_scan) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t h0 = by * kSparseBN;
-  const T* vals = static_cast<const T*>(p.values);
-  const T* dZ = static_cast<const T*>(p.dZ);
-  // 128 x 32 outputs over 256 threads: 4 columns d x 4 outputs h each
-  const int td = (tid >> 3) * 4, th = (tid & 7) * 4;
-  float acc[4][4] = {};
-  float db_acc = 0.0f;
-  for (int slab = 0; slab < p.nslabs; ++slab) {
-    const int64_t tile = (int64_t)slab * p.ncb + cb;
-    const uint32_t word = p.keepbits[tile * kTileWords + tid];    // row tid/4, word tid%4
-    const uint32_t cnt = __popc(word);
-    // exclusive scan of the 256 per-word counts
-    uint32_t incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t n = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += n;
-    }
-    if (lane == 31) s_scan[warp] = incl;
-    __syncthreads();
-    uint32_t wbase = 0;
-    for (int w = 0; w < warp; ++w) wbase += s_scan[w];
-    const int64_t base = p.offsets[tile] + (wbase + incl - cnt);
-    const int r = tid >> 2, c0 = (tid & 3) * 32;
-    // every kept entry's place follows from the word alone, so the loads do not wait for one another
-#pragma unroll 16
-    for (int b = 0; b < 32; ++b) {
-      const int64_t at = base + __popc(word & ((1u << b) - 1u));
-      float v = 0.0f;
-      if (((word >> b) & 1u) != 0 && at < p.capacity) v = to_float(vals[at]);   // a store that overflowed is never read past
-      sAh[r][c0 + b] = v;
-    }
-    for (int i = tid; i < kTileRows * kSparseBN; i += 256) {
-      const int rr = i / kSparseBN, hh = i % kSparseBN;
-      const int64_t row = (int64_t)slab * kTileRows + rr, h = h0 + hh;
-      sZ[rr][hh] = (row < p.B && h < p.H) ? to_float(dZ[row * p.ldz + h]) : 0.0f;
-    }
-    __syncthreads();
-    if (p.db != nullptr && cb == 0 && tid < kSparseBN) {
-      // the dZ block is in shared memory anyway: its column sums, slab after slab in row order
-      float sum = 0.0f;
-      for (int rr = 0; rr < kTileRows; ++rr) sum += sZ[rr][tid];
-      db_acc += sum;
-    }
-#pragma unroll 4
-    for (int rr = 0; rr < kTileRows; ++rr) {
-      float a[4], z[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = sAh[rr][td + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) z[j] = sZ[rr][th + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], z[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-  if (p.db != nullptr && cb == 0 && tid < kSparseBN && h0 + tid < p.H) p.db[h0 + tid] = db_acc;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t d = (int64_t)cb * kTileCols + td + i;
-    if (d >= p.D) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t h = h0 + th + j;
-      if (h < p.H) p.dW[d * p.ldw + h] = acc[i][j];
-    }
-  }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) sparse_dw_kernel(const SparseDwParams p) {
-  __shared__ float sAh[kTileRows][kTileCols + 1];
-  __shared__ float sZ[kTileRows][kSparseBN + 1];
-  __shared__ uint32_t s_scan[256];
-  sparse_dw_body<T>(p, (int)blockIdx.x, blockIdx.y, sAh, sZ, s_scan);
-}
-
 // dW of a layer and the gradient of its input in one launch: both read the same dZ and neither reads the
-// other's result, so the first `dw_blocks` CTAs are those of sparse_dw_kernel and the rest those of the
-// input-gradient GEMM, each doing exactly what it does in a launch of its own (the nets that run on CUDA
-// cores are bound by their launch count).
-constexpr int kDwDxSmemA = kTileRows * (kTileCols + 1) * 4, kDwDxSmemZ = kTileRows * (kSparseBN + 1) * 4;
-static_assert(kDwDxSmemA + kDwDxSmemZ + 1024 <= kGemmSmemBytes, "the sparse tiles fit the GEMM's buffer");
+// other's result, so the first `dw_blocks` CTAs are those of the weight gradient in a launch of its own and the rest
+// those of the input gradient, each doing exactly what it does there (the nets that run on CUDA cores are bound by
+// their launch count).  `dw_blocks` is a multiple of the cluster size.
 template <typename T>
-__global__ void __launch_bounds__(256, 2) dw_dx_kernel(const SparseDwParams d, const GemmParams g, int dw_blocks) {
+__global__ void __launch_bounds__(256, 2) dw_dx_kernel(const GemmParams w, const GemmParams g, int dw_blocks) {
   extern __shared__ __align__(16) float smem[];
-  unsigned char* raw = reinterpret_cast<unsigned char*>(smem);
   const int b = (int)blockIdx.x, gu = b - dw_blocks;
-  if (b < dw_blocks) {
-    if (b < d.units)
-      sparse_dw_body<T>(d, b % d.ncb, b / d.ncb, reinterpret_cast<float(*)[kTileCols + 1]>(raw),
-                        reinterpret_cast<float(*)[kSparseBN + 1]>(raw + kDwDxSmemA),
-                        reinterpret_cast<uint32_t*>(raw + kDwDxSmemA + kDwDxSmemZ));
-  } else {
-    gemm_unit_partial<T, kEpiInputGrad>(g, gu, smem);
-  }
+  if (b < dw_blocks) gemm_unit_partial<T, kEpiSparse>(w, b, smem);
+  else gemm_unit_partial<T, kEpiInputGrad>(g, gu, smem);
   share_barrier();
-  if (b >= dw_blocks) gemm_unit_finish<T, kEpiInputGrad>(g, gu, smem);
+  if (b < dw_blocks) gemm_unit_finish<T, kEpiSparse>(w, b, smem);
+  else gemm_unit_finish<T, kEpiInputGrad>(g, gu, smem);
   if (cluster_nctas() > 1) cluster_barrier();
 }
 
@@ -772,37 +742,35 @@ int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H
     zero_rows_kernel<<<g, 256, 0, s>>>(dW, ldw, st->D, H);
     return launch_gemm<kEpiScatterRows>(st->dtype, p, std::max<int64_t>(p.M, 1), s);
   }
-  SparseDwParams p;
-  p.values = st->values; p.keepbits = st->keepbits; p.offsets = st->offsets;
-  p.capacity = st->values_capacity;
-  p.B = st->B; p.D = st->D; p.H = H;
-  p.ncb = (int32_t)ceil_div(st->D, kTileCols); p.nslabs = (int32_t)ceil_div(st->B, kTileRows);
-  p.dZ = dZ; p.ldz = ldz; p.dW = dW; p.ldw = ldw;
+  const bool low = st->dtype == RAD_BF16;
+  GemmParams p = {};
+  p.A = st->values; p.keepbits = st->keepbits; p.offsets = st->offsets; p.capacity = st->values_capacity;
+  p.ncb = (int32_t)ceil_div(st->D, kTileCols);
+  p.Bm = dZ; p.sbk = ldz; p.sbn = 1;
+  p.M = st->D; p.N = H; p.K = st->B;
+  p.out_f32 = dW; p.ld_f32 = ldw;
   p.db = db;
   if (db_written != nullptr) *db_written = db != nullptr;
-  dim3 grid((unsigned)p.ncb, (unsigned)ceil_div(H, kSparseBN));
-  count_launch();
+  plan_gemm(p, p.M, low ? 2 : 4, kTileRows);
   if (ig != nullptr && ig_done != nullptr) {
     GemmParams g = input_grad_params(st->B, st->D, H, dZ, ldz, *ig);
-    plan_gemm(g, g.M, st->dtype == RAD_BF16 ? 2 : 4);
-    const int64_t units = (int64_t)grid.x * grid.y, dw_blocks = round_up(units, g.splits);
-    if (dw_blocks + g.units <= 0x7fffffff) {
+    plan_gemm(g, g.M, low ? 2 : 4);
+    const int64_t cluster = std::max(p.splits, g.splits), dw_blocks = round_up(p.units, cluster);
+    const int64_t all = dw_blocks + round_up(g.units, cluster);
+    if (all <= 0x7fffffff) {
       static std::atomic<uint64_t> ready_b{0}, ready_f{0};
-      p.units = (int32_t)units;
+      const size_t smem = (size_t)std::max(gemm_smem_bytes(g.tile), gemm_smem_bytes(p.tile));
+      const dim3 grid((unsigned)all), cl((unsigned)cluster);
+      count_launch();
       *ig_done = true;
-      const dim3 all((unsigned)(dw_blocks + g.units)), cl((unsigned)g.splits);
-      if (st->dtype == RAD_BF16)
+      if (low)
         return !allow_smem(dw_dx_kernel<bf16>, kGemmSmemBytes, ready_b) ? RAD_ECUDA
-               : launch_with_cluster(dw_dx_kernel<bf16>, all, 256, kGemmSmemBytes, cl, s, p, g, (int)dw_blocks);
+               : launch_with_cluster(dw_dx_kernel<bf16>, grid, 256, smem, cl, s, p, g, (int)dw_blocks);
       return !allow_smem(dw_dx_kernel<float>, kGemmSmemBytes, ready_f) ? RAD_ECUDA
-             : launch_with_cluster(dw_dx_kernel<float>, all, 256, kGemmSmemBytes, cl, s, p, g, (int)dw_blocks);
+             : launch_with_cluster(dw_dx_kernel<float>, grid, 256, smem, cl, s, p, g, (int)dw_blocks);
     }
   }
-  if (st->dtype == RAD_BF16)
-    sparse_dw_kernel<bf16><<<grid, 256, 0, s>>>(p);
-  else
-    sparse_dw_kernel<float><<<grid, 256, 0, s>>>(p);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  return launch_planned<kEpiSparse>(st->dtype, p, s);
 }
 
 constexpr int kColChunkRows = 128;         // rows of dZ per partial row of the workspace

@@ -204,7 +204,7 @@ def test_softmax_xent_over_clusters_and_row_lengths(B, C, dtype):
                                          (700, 257, 203, "f32"), (2000, 68, 1500, "f32"), (129, 3000, 70, "f32"),
                                          (90, 100, 30, "bf16"), (700, 515, 333, "bf16")])
 def test_cuda_core_contractions_over_tiles_and_splits(B, D, H, dtype):
-    """Forward, input gradient and same-sample weight gradient on CUDA cores, from one CTA to clusters that share the
+    """Forward, input gradient and weight gradients (either mask) on CUDA cores, from one CTA to clusters that share the
     contraction index, 32 and 64 wide tiles with remainders, aligned and odd leading dimensions, against float64.
     Bound per output: sqrt(K) + 16 roundings of 2^-24 of the sum of magnitudes, plus one bf16 rounding of the result."""
     import paper_2007_10412_b200 as rad
@@ -221,10 +221,16 @@ def test_cuda_core_contractions_over_tiles_and_splits(B, D, H, dtype):
     rad.rad_linear_forward_store(A, st, status)
     dW = torch.full((D, H), float("nan"), dtype=torch.float32, device="cuda")
     rad.rad_linear_weight_grad(st, dZ, dW, dev_status=status)
+    sd = rad.Store("different", dtype, B, D, 0.3, seed=3, relu_bits=False)
+    rad.rad_linear_forward_store(A, sd, status)
+    dWd = torch.full((D, H), float("nan"), dtype=torch.float32, device="cuda")
+    rad.rad_linear_weight_grad(sd, dZ, dWd, dev_status=status)
     torch.cuda.synchronize()
     assert status.item() == 0
+    keep = torch.from_numpy(orc.keep_mask("different", B, D, 0.3, 3, 0, 0)).cuda()
+    Ah = torch.where(keep, (A.float() * float(orc.scale_factor(0.3))).to(tdt), torch.zeros((), dtype=tdt, device="cuda")).double()
     A, W, dZ = A.double(), W.double(), dZ.double()
-    for got, x, y, low in ((out, A, W, False), (dX, dZ, W.T, dtype == "bf16"), (dW, A.T, dZ, False)):
+    for got, x, y, low in ((out, A, W, False), (dX, dZ, W.T, dtype == "bf16"), (dW, A.T, dZ, False), (dWd, Ah.T, dZ, False)):
         ref, mag, K = x @ y, x.abs() @ y.abs(), x.shape[1]
         bound = (K ** 0.5 + 16) * 2.0 ** -24 * mag + (2.0 ** -8 * ref.abs() if low else 0)
         assert ((got.double() - ref).abs() <= bound + 1e-30).all()
