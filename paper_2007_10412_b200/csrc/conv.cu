@@ -7,8 +7,8 @@
 //
 // The whole net of this configuration is about 2 GFLOP per step, so these kernels are CUDA-core
 // kernels tuned for few launches and fixed summation order, not tensor-core kernels:
-//   conv_forward_pool   one thread per pooled output: four conv outputs, ReLU, 4 derivative bits
-//                       (a nibble; eight neighbouring channels make one word), rounded average
+//   conv_forward_pool   one thread per pooling window and eight channels: 32 conv outputs, ReLU, one word of
+//                       derivative bits (a nibble per channel), rounded averages
 //   conv_dz             dZ = 0.25 * dP * bit, the conv-output gradient in the working type
 //   conv_input_grad     direct transposed convolution, one thread per input entry
 //   conv_weight_grad    one CTA per minibatch row: the row's kept entries are listed in shared
@@ -16,6 +16,7 @@
 //                       (filter tap, output channel) walks the list in order
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include "common.cuh"
 
@@ -27,65 +28,97 @@ struct ConvShape {
   int32_t H, W, Cin, Cout;      // H, W: conv input = conv output size (padding 1)
 };
 
-// filters arrive as 3 x 3 x Cin x Cout in the working type; shared memory keeps them as float
-template <typename T>
-__device__ __forceinline__ void load_filters(const T* Wt, float* s_w, int n, int stride_in, int stride_out, int cout) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s_w[(i / cout) * stride_out + (i % cout)] = to_float(Wt[i]);
-  (void)stride_in;
-}
-
-template <typename T>
+// One thread per pooling window and eight neighbouring output channels (which share one word of derivative bits and,
+// in bf16, one 16-byte store).  The filters lie in shared memory as floats, so a tap costs two broadcast 16-byte
+// reads for its 32 multiply-adds (four outputs x eight channels, in pairs); with kCin > 0 the window's 4 x 4 x Cin input patch
+// is loaded once into registers, else its entries are read tap by tap.  Every output is one chain of fused
+// multiply-adds over (tap, channel) in ascending order, whichever way its entries are read.
+// Bound by the FMA pipes (first convolution of the CNN, 32 x 32 x 3 -> 16: batch 4096 1405 -> 136 us, with one thread
+// per output channel, four shared-memory reads per four multiply-adds and a bounds test per input entry before).
+constexpr int kConvCo = 8;
+template <typename T, int kCin>
 __global__ void __launch_bounds__(256) conv_forward_pool_kernel(const ConvShape s, const T* X, const T* Wt,
                                                                 const float* bias, T* P, uint32_t* relubits) {
-  extern __shared__ float s_w[];                     // 9 * Cin x Cout
-  load_filters(Wt, s_w, 9 * s.Cin * s.Cout, 0, s.Cout, s.Cout);
+  extern __shared__ __align__(16) float s_w[];       // 9 * Cin x Cout
+  const int Cin = kCin > 0 ? kCin : s.Cin, nw = 9 * Cin * s.Cout;
+  for (int i = threadIdx.x; i < nw; i += 256) s_w[i] = to_float(Wt[i]);
   __syncthreads();
-  const int Hp = s.H / 2, Wp = s.W / 2;
-  const int64_t total = s.B * Hp * Wp * s.Cout;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t nib = 0;
-  if (i < total) {
-    const int co = (int)(i % s.Cout);
-    const int64_t pix = i / s.Cout;
-    const int xp = (int)(pix % Wp), yp = (int)((pix / Wp) % Hp);
-    const int64_t b = pix / ((int64_t)Wp * Hp);
-    const T* Xb = X + b * s.H * s.W * s.Cin;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    // the 4 x 4 input patch around the 2 x 2 outputs
-    for (int py = 0; py < 4; ++py) {
-      const int yi = 2 * yp - 1 + py;
-      if (yi < 0 || yi >= s.H) continue;
-      for (int px = 0; px < 4; ++px) {
-        const int xi = 2 * xp - 1 + px;
-        if (xi < 0 || xi >= s.W) continue;
-        const T* xin = Xb + ((int64_t)yi * s.W + xi) * s.Cin;
-        for (int ci = 0; ci < s.Cin; ++ci) {
-          const float v = to_float(xin[ci]);
+  const int Hp = s.H / 2, Wp = s.W / 2, groups = s.Cout / kConvCo;
+  const int64_t total = s.B * Hp * Wp * groups;
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= total) return;
+  const int64_t win = i / groups;
+  const int co0 = (int)(i - win * groups) * kConvCo;
+  const int64_t line = win / Wp;
+  const int xp = (int)(win - line * Wp), yp = (int)(line % Hp);
+  const T* Xb = X + (line / Hp) * s.H * s.W * Cin;
+  // entry (py, px, ci) of the 4 x 4 input patch around the 2 x 2 outputs
+  auto entry = [&](int py, int px, int ci) {
+    const int yi = 2 * yp - 1 + py, xi = 2 * xp - 1 + px;
+    return yi >= 0 && yi < s.H && xi >= 0 && xi < s.W ? to_float(Xb[((int64_t)yi * s.W + xi) * Cin + ci]) : 0.0f;
+  };
+  float patch[kCin > 0 ? 16 * kCin : 1];
+  if (kCin > 0) {
 #pragma unroll
-          for (int o = 0; o < 4; ++o) {
-            const int ky = py - (o >> 1), kx = px - (o & 1);       // tap that maps this input to output o
-            if (ky >= 0 && ky < 3 && kx >= 0 && kx < 3)
-              acc[o] = fmaf(v, s_w[((ky * 3 + kx) * s.Cin + ci) * s.Cout + co], acc[o]);
-          }
-        }
+    for (int q = 0; q < 16; ++q)
+#pragma unroll
+      for (int ci = 0; ci < kCin; ++ci) patch[q * kCin + ci] = entry(q >> 2, q & 3, ci);
+  }
+  f32x2 acc[4][kConvCo / 2] = {};
+  auto tap = [&](int ky, int kx, int ci, const float (&v)[4]) {
+    const ulonglong2* w = reinterpret_cast<const ulonglong2*>(s_w + ((ky * 3 + kx) * Cin + ci) * s.Cout + co0);
+    const ulonglong2 w0 = w[0], w1 = w[1];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      const f32x2 vv = pack2(v[o], v[o]);
+      fma2(acc[o][0], vv, w0.x); fma2(acc[o][1], vv, w0.y); fma2(acc[o][2], vv, w1.x); fma2(acc[o][3], vv, w1.y);
+    }
+  };
+  if (kCin > 0) {
+#pragma unroll
+    for (int t = 0; t < 9; ++t)
+#pragma unroll
+      for (int ci = 0; ci < kCin; ++ci) {
+        const int q = (t / 3) * 4 + t % 3;
+        const float v[4] = {patch[q * kCin + ci], patch[(q + 1) * kCin + ci], patch[(q + 4) * kCin + ci], patch[(q + 5) * kCin + ci]};
+        tap(t / 3, t % 3, ci, v);
+      }
+  } else {
+    for (int t = 0; t < 9; ++t) {
+      const int ky = t / 3, kx = t - 3 * ky;
+#pragma unroll 2
+      for (int ci = 0; ci < Cin; ++ci) {
+        const float v[4] = {entry(ky, kx, ci), entry(ky, kx + 1, ci), entry(ky + 1, kx, ci), entry(ky + 1, kx + 1, ci)};
+        tap(ky, kx, ci, v);
       }
     }
-    const float bco = bias != nullptr ? bias[co] : 0.0f;
+  }
+  uint32_t word = 0;                                 // nibble k = channel co0 + k, bit o = output o of the window
+  T* out = P + win * s.Cout + co0;
+  T pooled[kConvCo];
+#pragma unroll
+  for (int c = 0; c < kConvCo; ++c) {
+    const float bco = bias != nullptr ? bias[co0 + c] : 0.0f;
     float sum = 0.0f;
 #pragma unroll
     for (int o = 0; o < 4; ++o) {
-      const float r = to_float(from_float<T>(fmaxf(acc[o] + bco, 0.0f)));     // the activation as the device would hold it
-      nib |= (r > 0.0f ? 1u : 0u) << o;
+      float lo, hi;
+      unpack2(acc[o][c / 2], lo, hi);
+      const float r = to_float(from_float<T>(fmaxf((c % 2 ? hi : lo) + bco, 0.0f)));     // the activation as the device would hold it
+      word |= (r > 0.0f ? 1u : 0u) << (4 * c + o);
       sum += r;
     }
-    P[i] = from_float<T>(0.25f * sum);
+    pooled[c] = from_float<T>(0.25f * sum);
   }
-  // eight neighbouring channels share one word of derivative bits: nibble k = channel co0 + k
-  uint32_t word = nib << (4 * (threadIdx.x & 7));
-  word |= __shfl_xor_sync(0xffffffffu, word, 1);
-  word |= __shfl_xor_sync(0xffffffffu, word, 2);
-  word |= __shfl_xor_sync(0xffffffffu, word, 4);
-  if ((threadIdx.x & 7) == 0 && i < total) relubits[i >> 3] = word;
+  if constexpr (sizeof(T) == 2) {
+    uint4 v;
+    memcpy(&v, pooled, 16);
+    *reinterpret_cast<uint4*>(out) = v;
+  } else {
+#pragma unroll
+    for (int c = 0; c < kConvCo; c += 4) *reinterpret_cast<float4*>(out + c) = make_float4(pooled[c], pooled[c + 1], pooled[c + 2], pooled[c + 3]);
+  }
+  relubits[i] = word;
 }
 
 template <typename T>
@@ -255,24 +288,29 @@ __global__ void __launch_bounds__(256) conv_sum_rows_kernel(const float* part, i
 
 }  // namespace
 
+namespace {
+template <typename T, int kCin>
+int launch_forward_pool(const ConvShape& s, int64_t total, const void* X, const void* Wt, const float* bias, void* P, uint32_t* relubits,
+                        cudaStream_t st) {
+  const size_t smem = (size_t)9 * s.Cin * s.Cout * 4;
+  count_launch();
+  RAD_CUDA_TRY(cudaFuncSetAttribute(conv_forward_pool_kernel<T, kCin>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  conv_forward_pool_kernel<T, kCin><<<(unsigned)ceil_div(total, 256), 256, smem, st>>>(s, static_cast<const T*>(X), static_cast<const T*>(Wt),
+                                                                                       bias, static_cast<T*>(P), relubits);
+  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+}
+}  // namespace
+
 // ---- launchers used by the whole-net step ---------------------------------------------------------------
 int conv_forward_pool(int dtype, int64_t B, int H, int W, int Cin, int Cout, const void* X, const void* Wt,
                       const float* bias, void* P, uint32_t* relubits, cudaStream_t st) {
-  ConvShape s = {B, H, W, Cin, Cout};
-  const int64_t total = B * (H / 2) * (W / 2) * Cout;
-  const size_t smem = (size_t)9 * Cin * Cout * 4;
-  const unsigned grid = (unsigned)ceil_div(total, 256);
-  count_launch();
-  if (dtype == RAD_BF16) {
-    RAD_CUDA_TRY(cudaFuncSetAttribute(conv_forward_pool_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    conv_forward_pool_kernel<bf16><<<grid, 256, smem, st>>>(s, static_cast<const bf16*>(X), static_cast<const bf16*>(Wt), bias,
-                                                           static_cast<bf16*>(P), relubits);
-  } else {
-    RAD_CUDA_TRY(cudaFuncSetAttribute(conv_forward_pool_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    conv_forward_pool_kernel<float><<<grid, 256, smem, st>>>(s, static_cast<const float*>(X), static_cast<const float*>(Wt), bias,
-                                                            static_cast<float*>(P), relubits);
-  }
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  const ConvShape s = {B, H, W, Cin, Cout};
+  const int64_t total = B * (H / 2) * (W / 2) * (Cout / kConvCo);
+  if (dtype == RAD_BF16)
+    return Cin == 3 ? launch_forward_pool<bf16, 3>(s, total, X, Wt, bias, P, relubits, st)
+                    : launch_forward_pool<bf16, 0>(s, total, X, Wt, bias, P, relubits, st);
+  return Cin == 3 ? launch_forward_pool<float, 3>(s, total, X, Wt, bias, P, relubits, st)
+                  : launch_forward_pool<float, 0>(s, total, X, Wt, bias, P, relubits, st);
 }
 
 int conv_dz(int dtype, int64_t B, int H, int W, int Cout, const void* dP, const uint32_t* relubits, void* dZ,

@@ -66,19 +66,6 @@ constexpr int kGemmSmemBytes = gemm_smem_bytes(64);
 static_assert(gemm_smem_bytes(32) >= (4 * 32 * 32 + 32) * 4 && gemm_smem_bytes(64) >= (4 * 64 * 64 + 64) * 4,
               "the partial tiles and column sums reuse the ring");
 
-// Two float32 multiply-adds per instruction (each rounded as fmaf rounds it): with one per instruction the FMA pipes
-// wait for the register file and the issue slots (4096 x 2048 x 2048: 31 TFLOP/s at 0.69 instructions per clock).
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-  f32x2 v;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
-  return v;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ void fma2(f32x2& acc, f32x2 a, f32x2 b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
-}
-
 // Asynchronous copies of one operand's K blocks into the ring, in the layout it has in memory: TS rows of BK
 // contiguous k (kKM) or BK rows of TS contiguous columns, zeros outside the matrix and past the end of the split.
 // A thread keeps one running pointer; everything that does not change from block to block is found once.
