@@ -205,6 +205,9 @@ extern "C" int rad_cnn_step(const rad_cnn_desc* d, const void* X, const int32_t*
   // ---- backward: conv blocks (g = gradient of the pooled output of block l) ----
   void* dz = ws + pl.dz;
   for (int l = pl.nc - 1; l >= 0; --l) {
+    if (l == 0 && conv_first_backward_ok(d->dtype, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], g))
+      return conv_first_backward(&st[l], pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], g, reinterpret_cast<const uint32_t*>(ws + pl.relubits[l]),
+                                 dconv_W[l], dconv_b[l], ws + pl.scratch, pl.scratch_bytes, s);
     rc = conv_dz(d->dtype, B, pl.H[l], pl.W[l], pl.Cout[l], g, reinterpret_cast<const uint32_t*>(ws + pl.relubits[l]), dz, s);
     if (rc != RAD_OK) return rc;
     if (conv_tc_ok(d->dtype, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], dz, conv_W[l]))

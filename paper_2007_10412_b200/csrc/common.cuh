@@ -249,6 +249,10 @@ int conv_dz(int dtype, int64_t B, int H, int W, int Cout, const void* dP, const 
 int conv_input_grad(int dtype, int64_t B, int H, int W, int Cin, int Cout, const void* dZ, const void* Wt, void* dX,
                     cudaStream_t st);
 int64_t conv_weight_grad_workspace(int64_t B, int Cin, int Cout);
+// filter and bias gradient of a first convolution straight from the gradient of its pooled output
+bool conv_first_backward_ok(int dtype, int H, int W, int Cin, int Cout, const void* dP);
+int conv_first_backward(const rad_store* store, int H, int W, int Cin, int Cout, const void* dP, const uint32_t* relubits, float* dW,
+                        float* db, void* workspace, int64_t workspace_bytes, cudaStream_t st);
 int conv_weight_grad(const rad_store* store, int H, int W, int Cin, int Cout, const void* dZ, float* dW, void* workspace,
                      int64_t workspace_bytes, cudaStream_t st);
 

@@ -67,3 +67,23 @@ def test_cnn_stored_bytes():
     assert s.full_backprop_bytes == 128 * per_sample_inputs * 2 + 128 * 10 * 4
     assert s.relu_bytes == 128 * (32 * 32 * 16 + 16 * 16 * 32 + 8 * 8 * 64) // 8 + 128 * 4 * 4
     assert s.value_bytes < 0.16 * 128 * per_sample_inputs * 2
+
+
+@pytest.mark.parametrize("B,hw,cin,channels,fc,dtype", [(1, 4, 1, (8,), (3,), "f32"), (800, 4, 2, (16,), (5,), "f32"),
+                                                        (66, 16, 4, (64,), (6,), "bf16"), (65, 12, 3, (24,), (4,), "f32"),
+                                                        (9, 16, 5, (8,), (3,), "f32")])
+@pytest.mark.parametrize("variant", ["different", "same"])
+def test_first_convolution_backward_over_channels_and_rows(B, hw, cin, channels, fc, dtype, variant):
+    """The one-launch backward of the first convolution at one to four input channels, at channel counts that leave one
+    to eight parts of the list of kept entries, with more rows than CTAs, and beside it the route of five channels."""
+    import paper_2007_10412_b200 as rad
+    X, y, cW, cb, fW, fb = cnn_inputs(B, hw, cin, channels, fc, dtype, seed=B + hw, bias_zero=False)
+    ref = orc.cnn_step(X, y, cW, cb, fW, fb, dtype=dtype, variant=variant, p=0.3, seed=4, step=1)
+    ctx = rad.CNNStep(B, hw, cin, channels, fc, dtype, variant, 0.3)
+    ctx(to_dev(X, dtype), torch.from_numpy(y).cuda(), [to_dev(w, dtype) for w in cW], [to_dev(b, "f32") for b in cb],
+        [to_dev(w, dtype) for w in fW], [to_dev(b, "f32") for b in fb], seed=4, step=1)
+    torch.cuda.synchronize()
+    assert ctx.dev_status.item() == 0
+    for got, want in zip(ctx.dconv_W + ctx.dconv_b, ref.dW_conv + ref.db_conv):
+        fro, mx = rel_err(got.double().cpu().numpy(), want)
+        assert fro <= TOL[dtype] and mx <= TOL[dtype] * (1 if dtype == "f32" else 2)
