@@ -119,17 +119,23 @@ struct CvCtl {
   int abort_flag;
 };
 
-// 16 bytes of a dense NHWC tensor at pixel (b, y, x), channel c0 .. c0 + 7, zero outside the image
-__device__ __forceinline__ uint4 cv_load_pixel(const bf16* T, int64_t b, int y, int x, int H, int W, int C, int c0) {
-  if (y < 0 || y >= H || x < 0 || x >= W) return make_uint4(0u, 0u, 0u, 0u);
-  return __ldg(reinterpret_cast<const uint4*>(T + ((b * H + y) * W + x) * C + c0));
+// 16 bytes of a dense NHWC tensor at pixel (y, x) of the image that starts at T, channel c0 .. c0 + 7, zero outside
+__device__ __forceinline__ uint4 cv_load_pixel(const bf16* T, bool in, int y, int x, int H, int W, int C, int c0) {
+  if (!in || y < 0 || y >= H || x < 0 || x >= W) return make_uint4(0u, 0u, 0u, 0u);
+  return __ldg(reinterpret_cast<const uint4*>(T + ((int64_t)y * W + x) * C + c0));
 }
 
 // kCvFwd: forward tile `blockIdx.x` (128 output pixels); kCvDw: filter-gradient unit (m tile, split) = blockIdx;
-// kCvDx: input-gradient tile `blockIdx.x` (128 input pixels in raster order)
+// kCvDx: input-gradient tile `blockIdx.x` (128 input pixels in raster order).
+// What bounds these kernels is the chain of a K block: gather (L2 latency), store to shared memory, fence, MMA.  So the
+// gather of the next block is in registers before this block's stage is waited for, a block costs one barrier, and all
+// of a thread's index arithmetic that does not change from block to block (its pixels in the forward and input
+// gradient, its tap and channels in the filter gradient) is done once.  CNN at batch 4096, second / third
+// convolution: forward 279 -> 164 / 123 -> 58 us, filter gradient (also 444 instead of 192 CTAs) 855 -> 138 /
+// 210 -> 58, input gradient 339 -> 175 / 165 -> 78.
 enum { kCvFwd = 0, kCvDw = 1, kCvDx = 2 };
 template <int kMode>
-__global__ void __launch_bounds__(kCvThreads) conv_tc_kernel(const ConvTcParams p) {
+__global__ void __launch_bounds__(kCvThreads, 3) conv_tc_kernel(const ConvTcParams p) {
   constexpr bool kDw = kMode == kCvDw, kDx = kMode == kCvDx;
   extern __shared__ uint8_t cv_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(cv_raw) + 1023) & ~(uintptr_t)1023);
@@ -149,16 +155,95 @@ __global__ void __launch_bounds__(kCvThreads) conv_tc_kernel(const ConvTcParams 
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(cv_smem(&ctl->tmem_base)), "r"(64u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = ctl->tmem_base;
 
   // what this CTA contracts over
   const int mtile = kDw ? (int)blockIdx.x : 0, split = kDw ? (int)blockIdx.y : 0;
   const int64_t tile = kDw ? 0 : blockIdx.x;
   const int nkb = kDw ? p.kblocks_per_split : ((kDx ? 9 * Cout : ktaps) + kCvK - 1) / kCvK;
   const int64_t kb0 = kDw ? (int64_t)split * p.kblocks_per_split : 0;
+
+  // Patch operand A.  Forward, input gradient: thread = 16-byte chunk cc (k = 8 cc ..) of rows m0 + 32 j, whose pixels
+  // stay; K-major.  Filter gradient: thread = chunk cc (eight (tap, ci) indices, which stay) of the pixels k0 + 16 j,
+  // which move on by 64 a block; MN-major.
+  constexpr int kRowShift = kDw ? 4 : 3;
+  const int cc = tid & ((1 << kRowShift) - 1), row0 = tid >> kRowShift;
+  const bf16* img[4];                                 // image of the pixel
+  int py[4], px[4];
+  bool in[4];
+  const int C = kDx ? Cout : Cin;                     // channels of the gathered tensor
+  const bf16* src = kDx ? p.dZ : p.X;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (kDw) {
+      const int64_t pix = kb0 * kCvK + row0 + 16 * j, line = pix / W;
+      px[j] = (int)(pix - line * W); py[j] = (int)(line % H);
+      img[j] = src + (line / H) * H * W * C;
+      in[j] = pix < npix;
+    } else if (kDx) {
+      const int64_t pix = tile * kCvM + row0 + 32 * j, line = pix / W;
+      px[j] = (int)(pix - line * W); py[j] = (int)(line % H);
+      img[j] = src + (line / H) * H * W * C;
+      in[j] = pix < npix;
+    } else {
+      // row m = window (tile * 32 + m / 4), pixel m % 4 of it
+      const int m = row0 + 32 * j, Wp = W >> 1, Hp = H >> 1;
+      const int64_t q = tile * 32 + (m >> 2), line = q / Wp;
+      px[j] = 2 * (int)(q - line * Wp) + (m & 1); py[j] = 2 * (int)(line % Hp) + ((m >> 1) & 1);
+      img[j] = src + (line / Hp) * H * W * C;
+      in[j] = q < npix / 4;
+    }
+  }
+  // the filter gradient's (tap, channels) and its step of 64 pixels
+  const int dw_m0 = mtile * kCvM + cc * 8, dw_tap = kDw ? dw_m0 / Cin : 0, dw_c0 = dw_m0 - dw_tap * Cin;
+  const int step_x = kCvK % W, step_l = kCvK / W, step_y = step_l % H;
+  const int64_t step_img = (int64_t)(step_l / H) * H * W * C, one_img = (int64_t)H * W * C;
+  uint4 va[4], vb[2];
+  int64_t left = kDw ? npix - kb0 * kCvK - row0 : 0;  // pixels from this thread's first one to the end
+  auto gather = [&](int kb) {
+    if (kDw) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        va[j] = cv_load_pixel(img[j], left > 16 * j && dw_tap < 9, py[j] + dw_tap / 3 - 1, px[j] + dw_tap % 3 - 1, H, W, C, dw_c0);
+        px[j] += step_x; py[j] += step_y; img[j] += step_img;
+        if (px[j] >= W) { px[j] -= W; ++py[j]; }
+        if (py[j] >= H) { py[j] -= H; img[j] += one_img; }
+      }
+      left -= kCvK;
+      // B: dZ of the pixel, 8 chunks of 8 channels per row
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int k = (tid >> 3) + 32 * j, c = (tid & 7) * 8;
+        const int64_t pix = (kb0 + kb) * kCvK + k;
+        vb[j] = pix < npix && c < Cout ? __ldg(reinterpret_cast<const uint4*>(p.dZ + pix * Cout + c)) : make_uint4(0u, 0u, 0u, 0u);
+      }
+    } else {
+      const int k0 = kb * kCvK + cc * 8, tap = k0 / C, c0 = k0 - tap * C, ty = tap / 3, tx = tap - 3 * ty;
+      // forward: the tap reads pixel (y + ty - 1, x + tx - 1); input gradient: the output pixel that reached this input
+      // pixel through the tap lies at (y - ty + 1, x - tx + 1)
+      const int dy = kDx ? 1 - ty : ty - 1, dx = kDx ? 1 - tx : tx - 1;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) va[j] = cv_load_pixel(img[j], in[j] && tap < 9, py[j] + dy, px[j] + dx, H, W, C, c0);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int r = (tid >> 3) + 32 * j;
+        vb[j] = make_uint4(0u, 0u, 0u, 0u);
+        if (kDx) {
+          // B: K-major, row n = input channel, k = (tap, co): W[tap, n, co0 .. co0 + 7] is contiguous
+          if (tap < 9 && r < Cin) vb[j] = __ldg(reinterpret_cast<const uint4*>(p.Wt + ((int64_t)tap * Cin + r) * Cout + c0));
+        } else {
+          // B: filter rows k (MN-major: Cout contiguous), 8 chunks of 8 channels per row
+          const int kg = kb * kCvK + r;
+          if (kg < ktaps && cc * 8 < Cout) vb[j] = __ldg(reinterpret_cast<const uint4*>(p.Wt + (int64_t)kg * Cout + cc * 8));
+        }
+      }
+    }
+  };
+  if (nkb > 0) gather(0);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = ctl->tmem_base;
+
   bool ok = true;
   for (int kb = 0; kb < nkb; ++kb) {
     const int s = kb & 1;
@@ -166,78 +251,21 @@ __global__ void __launch_bounds__(kCvThreads) conv_tc_kernel(const ConvTcParams 
     uint8_t* sB = sA + kCvABytes;
     // the MMAs of two K blocks ago have read this stage
     if (kb >= 2) ok = cv_wait(cv_smem(&ctl->done[s]), ((kb >> 1) - 1) & 1, abort_flag, p.wait_limit_ns);
-    if (!__syncthreads_and(ok ? 1 : 0)) { ok = false; break; }
-    if (kDx) {
-      // A: K-major patch tile of dZ, row m = input pixel tile * 128 + m, k = (tap, co): the output pixel that
-      // reached this input pixel through tap (ty, tx) lies at (y - ty + 1, x - tx + 1)
-      for (int c = tid; c < kCvM * 8; c += kCvThreads) {
-        const int m = c >> 3, cc = c & 7;
-        const int k0 = kb * kCvK + cc * 8, tap = k0 / Cout, co0 = k0 - tap * Cout;
-        const int64_t pix = tile * kCvM + m;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (tap < 9 && pix < npix) {
-          const int x = (int)(pix % W), y = (int)((pix / W) % H);
-          const int64_t b = pix / ((int64_t)W * H);
-          v = cv_load_pixel(p.dZ, b, y - tap / 3 + 1, x - tap % 3 + 1, H, W, Cout, co0);
-        }
-        *reinterpret_cast<uint4*>(sA + m * 128 + ((cc ^ (m & 7)) << 4)) = v;
+    if (ok) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int r = row0 + (kDw ? 16 : 32) * j;
+        if (kDw) *reinterpret_cast<uint4*>(sA + (cc >> 3) * 8192 + r * 128 + (((cc & 7) ^ (r & 7)) << 4)) = va[j];
+        else *reinterpret_cast<uint4*>(sA + r * 128 + ((cc ^ (r & 7)) << 4)) = va[j];
       }
-      // B: K-major, row n = input channel, k = (tap, co): W[tap, n, co0 .. co0 + 7] is contiguous
-      for (int c = tid; c < kCvN * 8; c += kCvThreads) {
-        const int n = c >> 3, cc = c & 7;
-        const int k0 = kb * kCvK + cc * 8, tap = k0 / Cout, co0 = k0 - tap * Cout;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (tap < 9 && n < Cin) v = __ldg(reinterpret_cast<const uint4*>(p.Wt + ((int64_t)tap * Cin + n) * Cout + co0));
-        *reinterpret_cast<uint4*>(sB + n * 128 + ((cc ^ (n & 7)) << 4)) = v;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int r = (tid >> 3) + 32 * j, c = tid & 7;
+        *reinterpret_cast<uint4*>(sB + r * 128 + ((c ^ (r & 7)) << 4)) = vb[j];
       }
-    } else if (!kDw) {
-      // A: K-major patch tile, row m = window (tile * 32 + m / 4), pixel m % 4 of it; 8 chunks of 8 k per row
-      for (int c = tid; c < kCvM * 8; c += kCvThreads) {
-        const int m = c >> 3, cc = c & 7;
-        const int k0 = kb * kCvK + cc * 8, tap = k0 / Cin, ci0 = k0 - tap * Cin;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        const int64_t q = tile * 32 + (m >> 2);
-        if (tap < 9 && q < npix / 4) {
-          const int Wp = W >> 1, Hp = H >> 1;
-          const int xp = (int)(q % Wp), yp = (int)((q / Wp) % Hp);
-          const int64_t b = q / ((int64_t)Wp * Hp);
-          const int y = 2 * yp + ((m >> 1) & 1), x = 2 * xp + (m & 1);
-          v = cv_load_pixel(p.X, b, y + tap / 3 - 1, x + tap % 3 - 1, H, W, Cin, ci0);
-        }
-        *reinterpret_cast<uint4*>(sA + m * 128 + ((cc ^ (m & 7)) << 4)) = v;
-      }
-      // B: filter rows k (MN-major: Cout contiguous), 8 chunks of 8 channels per row
-      for (int c = tid; c < kCvK * 8; c += kCvThreads) {
-        const int k = c >> 3, cc = c & 7;
-        const int kg = kb * kCvK + k;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (kg < ktaps && cc * 8 < Cout) v = __ldg(reinterpret_cast<const uint4*>(p.Wt + (int64_t)kg * Cout + cc * 8));
-        *reinterpret_cast<uint4*>(sB + k * 128 + ((cc ^ (k & 7)) << 4)) = v;
-      }
-    } else {
-      // A: MN-major, row k = pixel, 16 chunks of 8 (tap, ci) indices in two blocks of 64; B: dZ of the pixel
-      for (int c = tid; c < kCvK * 16; c += kCvThreads) {
-        const int k = c >> 4, cc = c & 15;
-        const int m0 = mtile * kCvM + cc * 8, tap = m0 / Cin, ci0 = m0 - tap * Cin;
-        const int64_t pix = (kb0 + kb) * kCvK + k;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (tap < 9 && pix < npix) {
-          const int x = (int)(pix % W), y = (int)((pix / W) % H);
-          const int64_t b = pix / ((int64_t)W * H);
-          v = cv_load_pixel(p.X, b, y + tap / 3 - 1, x + tap % 3 - 1, H, W, Cin, ci0);
-        }
-        *reinterpret_cast<uint4*>(sA + (cc >> 3) * 8192 + k * 128 + (((cc & 7) ^ (k & 7)) << 4)) = v;
-      }
-      for (int c = tid; c < kCvK * 8; c += kCvThreads) {
-        const int k = c >> 3, cc = c & 7;
-        const int64_t pix = (kb0 + kb) * kCvK + k;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (pix < npix && cc * 8 < Cout) v = __ldg(reinterpret_cast<const uint4*>(p.dZ + pix * Cout + cc * 8));
-        *reinterpret_cast<uint4*>(sB + k * 128 + ((cc ^ (k & 7)) << 4)) = v;
-      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
+    if (!__syncthreads_and(ok ? 1 : 0)) { ok = false; break; }
     if (tid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       constexpr uint32_t idesc = cv_idesc(kDw, !kDx);
@@ -250,6 +278,7 @@ __global__ void __launch_bounds__(kCvThreads) conv_tc_kernel(const ConvTcParams 
       }
       cv_commit(cv_smem(&ctl->done[s]));
     }
+    if (kb + 1 < nkb) gather(kb + 1);
   }
   // the last commit covers every MMA before it
   if (ok && nkb > 0) ok = cv_wait(cv_smem(&ctl->done[(nkb - 1) & 1]), ((nkb - 1) >> 1) & 1, abort_flag, p.wait_limit_ns);
@@ -279,28 +308,45 @@ __global__ void __launch_bounds__(kCvThreads) conv_tc_kernel(const ConvTcParams 
         }
       }
     } else if (!kDw) {
-      // rows 4 w .. 4 w + 3 are the 2 x 2 window w: bias, ReLU, derivative bits, rounded average
+      // rows 4 w .. 4 w + 3 are the 2 x 2 window w.  Each lane adds the bias, applies ReLU and rounds for its own pixel;
+      // then the four lanes of a window exchange (two rounds of shuffles), so that lane q holds all four pixels of channels
+      // 8 q .. 8 q + 7 of the chunk: one word of derivative bits and one 16-byte store of rounded averages.
       const int64_t win = tile * 32 + (m >> 2);
-      const bool win_ok = win < npix / 4;
-      const int quad = lane & ~3;
-      uint32_t word = 0;
+      const int q4 = lane & 3, co0 = chunk * 32 + q4 * 8;
+      float a[32];
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
         const int co = chunk * 32 + j;
-        float a = 0.0f;
-        if (co < Cout) {
-          const float z = __uint_as_float(r[j]) + (p.bias != nullptr ? __ldg(p.bias + co) : 0.0f);
-          a = __bfloat162float(__float2bfloat16_rn(fmaxf(z, 0.0f)));       // the activation as the device would hold it
+        const float z = __uint_as_float(r[j]) + (p.bias != nullptr && co < Cout ? __ldg(p.bias + co) : 0.0f);
+        a[j] = __bfloat162float(__float2bfloat16_rn(fmaxf(z, 0.0f)));       // the activation as the device would hold it
+      }
+      // round 1, partner lane ^ 1: keep channel blocks q & 1 and 2 + (q & 1) of eight
+      float mine[2][8], theirs[2][8];
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float lo = a[16 * h + c], hi = a[16 * h + 8 + c];
+          mine[h][c] = (q4 & 1) ? hi : lo;
+          theirs[h][c] = __shfl_xor_sync(0xffffffffu, (q4 & 1) ? lo : hi, 1);
         }
-        const uint32_t pos = __ballot_sync(0xffffffffu, a > 0.0f);
-        const float a0 = __shfl_sync(0xffffffffu, a, quad), a1 = __shfl_sync(0xffffffffu, a, quad + 1);
-        const float a2 = __shfl_sync(0xffffffffu, a, quad + 2), a3 = __shfl_sync(0xffffffffu, a, quad + 3);
-        word |= ((pos >> quad) & 0xfu) << (4 * (j & 7));
-        if ((lane & 3) == 0 && win_ok && co < Cout) {
-          p.P[win * Cout + co] = __float2bfloat16_rn(0.25f * (((a0 + a1) + a2) + a3));
-          if ((j & 7) == 7) p.relubits[(win * Cout + co) >> 3] = word;      // eight channels make one word
-        }
-        if ((j & 7) == 7) word = 0;
+      // round 2, partner lane ^ 2: keep half q >> 1; then the pixels in order 0 .. 3
+      uint32_t word = 0;
+      __align__(16) bf16 pooled[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const bool up = (q4 & 2) != 0, odd = (q4 & 1) != 0;
+        const float s0 = up ? mine[1][c] : mine[0][c], s1 = up ? theirs[1][c] : theirs[0][c];
+        const float t0 = __shfl_xor_sync(0xffffffffu, up ? mine[0][c] : mine[1][c], 2);
+        const float t1 = __shfl_xor_sync(0xffffffffu, up ? theirs[0][c] : theirs[1][c], 2);
+        const float se = odd ? s1 : s0, so = odd ? s0 : s1, te = odd ? t1 : t0, to = odd ? t0 : t1;     // even, odd pixel of either pair
+        const float a0 = up ? te : se, a1 = up ? to : so, a2 = up ? se : te, a3 = up ? so : to;
+        word |= ((a0 > 0.0f ? 1u : 0u) | (a1 > 0.0f ? 2u : 0u) | (a2 > 0.0f ? 4u : 0u) | (a3 > 0.0f ? 8u : 0u)) << (4 * c);
+        pooled[c] = __float2bfloat16_rn(0.25f * (((a0 + a1) + a2) + a3));
+      }
+      if (win < npix / 4 && co0 < Cout) {
+        *reinterpret_cast<uint4*>(p.P + win * Cout + co0) = *reinterpret_cast<const uint4*>(pooled);
+        p.relubits[(win * Cout + co0) >> 3] = word;
       }
     } else {
       const int mg = mtile * kCvM + m;
@@ -321,15 +367,6 @@ __global__ void __launch_bounds__(kCvThreads) conv_tc_kernel(const ConvTcParams 
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(64u) : "memory");
   }
-}
-
-// dW[i] = sum over splits of partial[s][i], in split order
-__global__ void __launch_bounds__(256) conv_tc_reduce_kernel(const float* partial, int splits, int64_t n, float* out) {
-  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (i >= n) return;
-  float acc = 0.0f;
-  for (int s = 0; s < splits; ++s) acc += partial[(int64_t)s * n + i];
-  out[i] = acc;
 }
 
 // A_hat (B x D, zero where dropped) from a compact store: the buffer is cleared first, then the kept values
@@ -411,18 +448,20 @@ int conv_tc_input_grad(int64_t B, int H, int W, int Cin, int Cout, const void* d
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 
-// K blocks of 64 pixels per CTA of the filter-gradient kernel, and the splits that follow from it
-static int conv_tc_splits(int64_t npix, int* kblocks_per_split) {
-  const int64_t kblocks = ceil_div(npix, kCvK);
-  int64_t per = std::max<int64_t>(4, ceil_div(kblocks, 96));      // about one wave of CTAs per M tile pair
+// K blocks of 64 pixels per CTA of the filter-gradient kernel, and the splits that follow from it: enough for three
+// CTAs on every SM (a K block is a chain of latencies, so CTAs side by side are what hides them), at least four each.
+static int conv_tc_splits(int64_t npix, int Cin, int* kblocks_per_split) {
+  const int64_t kblocks = ceil_div(npix, kCvK), want = std::max<int64_t>(1, 3 * 148 / ceil_div(9 * Cin, kCvM));
+  const int64_t per = std::max<int64_t>(4, ceil_div(kblocks, want));
   *kblocks_per_split = (int)per;
   return (int)ceil_div(kblocks, per);
 }
 
 int64_t conv_tc_weight_grad_workspace(int64_t B, int H, int W, int Cin, int Cout) {
   int per = 0;
-  const int splits = conv_tc_splits(B * H * W, &per);
-  return round_up(B * H * W * Cin * 2, 256) + round_up((int64_t)splits * 9 * Cin * Cout * 4, 256);
+  const int splits = conv_tc_splits(B * H * W, Cin, &per);
+  return round_up(B * H * W * Cin * 2, 256) + round_up((int64_t)splits * 9 * Cin * Cout * 4, 256) +
+         column_sums_workspace(splits, 9 * Cin * Cout);
 }
 
 int conv_tc_weight_grad(const rad_store* store, int H, int W, int Cin, int Cout, const void* dZ, float* dW, void* workspace,
@@ -446,13 +485,14 @@ int conv_tc_weight_grad(const rad_store* store, int H, int W, int Cin, int Cout,
   p.B = B; p.H = H; p.W = W; p.Cin = Cin; p.Cout = Cout;
   p.X = dense; p.dZ = static_cast<const bf16*>(dZ); p.partial = partial; p.dev_status = dev_status;
   p.wait_limit_ns = wait_limit_ns();
-  const int splits = conv_tc_splits(B * H * W, &p.kblocks_per_split);
+  const int splits = conv_tc_splits(B * H * W, Cin, &p.kblocks_per_split);
   RAD_CUDA_TRY(cudaFuncSetAttribute(conv_tc_kernel<kCvDw>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCvSmem));
-  count_launch(2);
+  count_launch();
   conv_tc_kernel<kCvDw><<<dim3((unsigned)ceil_div(9 * Cin, kCvM), (unsigned)splits), kCvThreads, kCvSmem, st>>>(p);
-  const int64_t n = (int64_t)9 * Cin * Cout;
-  conv_tc_reduce_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(partial, splits, n, dW);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_CUDA_TRY(cudaGetLastError());
+  // the splits' partial sums: column sums of a splits x (9 Cin Cout) matrix, in a fixed order
+  const int64_t n = (int64_t)9 * Cin * Cout, held = round_up((int64_t)splits * n * 4, 256);
+  return column_sums(RAD_F32, splits, n, partial, n, dW, reinterpret_cast<char*>(partial) + held, column_sums_workspace(splits, n), st);
 }
 
 }  // namespace rad
