@@ -43,6 +43,7 @@ struct TcParams {
   int64_t M, N, K;
   const int64_t* N_dev;      // same-sample dW: N = number of kept columns, read on the device
   const uint32_t* keep_cols; // same-sample dW: bit d set = column d of the layer input was kept
+  int32_t bn;                // dense forward and input gradient: columns of an output tile (64, 128 or 256)
   int32_t splits;            // K splits (1: epilogue writes final results)
   int32_t num_stages;
   int32_t comp_depth;        // sparse A: depth of the ring of compressed (index + values) buffers
@@ -158,11 +159,25 @@ struct Schedule {
   }
 };
 
+// Where a row's activations go in the next layer's store: the part of its index (in place before the launch) that
+// belongs to one row and one tile of 128 columns.  It needs no accumulator, so it is fetched while the MMAs run.
+struct StoreRow {
+  uint4 bits;                // the row's four keep-bit words of the tile
+  uint32_t first, off;       // tile offset, row offset
+  __device__ __forceinline__ void load(const TcParams& p, int64_t m, int64_t n) {
+    const int64_t tile = (m >> 6) * p.st_ncb + (n >> 7);
+    const uint32_t* tw = p.st_keepbits + tile * kTileWords;
+    bits = __ldg(reinterpret_cast<const uint4*>(tw + (int)(m & 63) * 4));
+    first = __ldg(p.st_offsets + tile);
+    off = __ldg(reinterpret_cast<const unsigned short*>(tw + kBitWords) + (int)(m & 63));
+  }
+};
+
 // ---- epilogue of one 32-column chunk of one accumulator row ------------------------------------------
 // r: the 32 float32 accumulators of row m, columns n .. n+31 (as bit patterns).
 template <int EPI>
 __device__ __forceinline__ void epilogue_chunk(const TcParams& p, uint32_t (&r)[32], int64_t m, int64_t n, bool row_ok,
-                                               int32_t split) {
+                                               int32_t split, const StoreRow& sr) {
   const int nvalid = (int)min((int64_t)32, p.N - n);      // multiple of 8
   if (EPI == kFwd) {
     float v[32];
@@ -227,10 +242,10 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, uint32_t (&r)[
           const int64_t tile = (m >> 6) * p.st_ncb + (n >> 7);
           const int rr = (int)(m & 63), wq = (int)((n >> 5) & 3);
           const uint32_t* tw = p.st_keepbits + tile * kTileWords;
-          const uint4 rowbits = __ldg(reinterpret_cast<const uint4*>(tw + rr * 4));
+          const uint4 rowbits = sr.bits;
           const uint32_t word = wq == 0 ? rowbits.x : wq == 1 ? rowbits.y : wq == 2 ? rowbits.z : rowbits.w;
-          const uint32_t first = __ldg(p.st_offsets + tile);
-          uint64_t pos = (uint64_t)first + __ldg(reinterpret_cast<const unsigned short*>(tw + kBitWords) + rr);
+          const uint32_t first = sr.first;
+          uint64_t pos = (uint64_t)first + sr.off;
           if (wq > 0) pos += __popc(rowbits.x);
           if (wq > 1) pos += __popc(rowbits.y);
           if (wq > 2) pos += __popc(rowbits.z);
@@ -419,8 +434,12 @@ __device__ __forceinline__ void expand_word(uint8_t* sA, const uint8_t* sC, int 
 // both CTAs), tmem_empty[b] (even CTA; every epilogue warp of the pair arrives).
 constexpr int kStage2Bytes = 2 * 128 * BK * 2;   // 16 KB of A + 16 KB of B per CTA and stage
 constexpr int kStages2 = 6;
-constexpr int kEpiWarps2 = 8;
-constexpr int kThreads2 = 32 * (2 + kEpiWarps2);
+// Epilogue warps.  Sixteen for a forward pass of up to kWideEpilogueK inputs: its epilogue, which also places the next
+// layer's store, hides its loads and scattered stores behind them (4096 x 1024 x 1024 with ReLU: 25.7 us with eight, 22.2
+// with sixteen).  Eight where the MMAs of a tile outlast the epilogue of the one before anyway (8192 x 4096 x 4096: 224
+// against 234 us) and for the others (input gradient of 4096 x 1024 x 1024: 14.2 against 15.4 us).
+constexpr int64_t kWideEpilogueK = 2048;
+constexpr int threads2(int epi_warps) { return 32 * (2 + epi_warps); }
 
 struct SmemCtl2 {
   uint64_t full[kStages2], empty[kStages2], tmem_full[2], tmem_empty[2];
@@ -494,8 +513,8 @@ __host__ __device__ constexpr uint32_t make_idesc_pair(bool a_mn, bool b_mn, uin
          ((n >> 3) << 17) | ((256u >> 4) << 24);
 }
 
-template <int AK, int BKIND, int EPI>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads2, 1)
+template <int AK, int BKIND, int EPI, int kEpiWarps2>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kEpiWarps2), 1)
 tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -510,7 +529,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
   // columns are cut into the fewest tiles of at most 256 and the tile width bn is what one of them needs,
   // rounded up to the MMA's granule of 16: 105 kept columns cost one tile of 112, not one of 256.
   int64_t n_cols = p.N;
-  int bn = BN;
+  int bn = p.bn;
   if (EPI == kDwT) {
     int64_t nd;
     asm volatile("ld.global.cg.s64 %0, [%1];" : "=l"(nd) : "l"(p.N_dev) : "memory");
@@ -519,8 +538,8 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
     bn = max(16, (int)(((n_cols + nt - 1) / nt + 15) / 16 * 16));
   }
   const Schedule sched(p.M, n_cols, p.K, p.splits, BM, bn);
-  const int boxes_b = (EPI == kDwT) ? (bn / 2 + 63) / 64 : 2;     // 64-column boxes of B this CTA stages per K block
-  const uint32_t stage_tx = 2u * (uint32_t)(kStage2Bytes / 2 + boxes_b * 8192);
+  const int boxes_b = (bn / 2 + 63) / 64;             // 64-column boxes of an MN-major B this CTA stages per K block
+  const uint32_t stage_tx = 2u * (uint32_t)(kStage2Bytes / 2 + (BKIND == kBK_ ? bn / 2 * 128 : boxes_b * 8192));
   const int64_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   if (tid == 0) {
     for (int s = 0; s < kStages2; ++s) {
@@ -631,10 +650,11 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
   } else {
     // ===== epilogue: thread = one accumulator row of this CTA, 128 columns per warp =====
     const int q = warp & 3;
-    // the two warps of a lane quarter split the tile's 32-column chunks between them
-    const int chunks = (bn + 31) / 32, half_chunks = (chunks + 1) / 2;
-    const int c_first = ((warp - 2) >> 2) * half_chunks * 32;
-    const int c_last = min(c_first + half_chunks * 32, chunks * 32);
+    // the warps of a lane quarter split the tile's 32-column chunks between them
+    constexpr int kPerQuarter = kEpiWarps2 / 4;
+    const int chunks = (bn + 31) / 32, own_chunks = (chunks + kPerQuarter - 1) / kPerQuarter;
+    const int c_first = ((warp - 2) >> 2) * own_chunks * 32;
+    const int c_last = min(c_first + own_chunks * 32, chunks * 32);
     const uint32_t empty_bar = map_to_cta(smem_u32(&ctl->tmem_empty[0]), 0u);     // [b] is 8 bytes further
     int buf = 0;
     uint32_t buf_phases = 0;
@@ -643,7 +663,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       // Rows of dW whose column was not kept are zero (Sec. 4.3: only the sampled part of the weight matrix
       // gets a gradient).  The epilogue warps have nothing to do until the first tile's MMAs retire, so they
       // write those rows now: row d belongs to CTA d mod grid, a thread writes 16 bytes at a time.
-      const int et = tid - 64;                       // 0 .. 255
+      const int et = tid - 64;                       // 0 .. 32 kEpiWarps2 - 1
       const int64_t h4 = p.M / 4;
       for (int64_t d = blockIdx.x; d < p.dw_rows; d += gridDim.x) {
         if ((__ldg(p.keep_cols + (d >> 5)) >> (d & 31)) & 1u) continue;
@@ -653,12 +673,19 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
     }
     for (int64_t u = pair; u < sched.units && ok; u += npairs) {
       const Unit w = sched.unit(u);
+      const int64_t m = w.m0 + 128 * (int64_t)rank + q * 32 + lane;
+      const bool row_ok = m < sched.M;
+      // what the epilogue reads besides the accumulators comes while the MMAs run (a warp's columns lie in one store tile)
+      StoreRow sr = {};
+      if (EPI == kFwd && w.n0 + c_first < n_cols) {
+        if (p.st_values != nullptr && row_ok) sr.load(p, m, w.n0 + c_first);
+        if (p.bias != nullptr && lane < own_chunks && w.n0 + c_first + 32 * lane < n_cols)
+          asm volatile("prefetch.global.L1 [%0];" ::"l"(p.bias + w.n0 + c_first + 32 * lane));
+      }
       if (lane == 0) ok = mbar_wait2(smem_u32(&ctl->tmem_full[0]) + 8u * buf, (buf_phases >> buf) & 1u, wc, 200u);
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       if (!ok) break;
       tc_fence_after();
-      const int64_t m = w.m0 + 128 * (int64_t)rank + q * 32 + lane;
-      const bool row_ok = m < sched.M;
 #pragma unroll 1
       for (int c0 = c_first; c0 < c_last; c0 += 32) {
         const int64_t n = w.n0 + c0;
@@ -668,7 +695,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
         tmem_ld_wait();
         // a chunk may reach past the tile's width (bn is a multiple of 16) and past the last kept column
         if (EPI == kDwT) epilogue_chunk_dwt(p, r, m, n, (int)min((int64_t)min(32, bn - c0), n_cols - n), row_ok, w.split);
-        else epilogue_chunk<(EPI == kDwT ? kDw : EPI)>(p, r, m, n, row_ok, w.split);
+        else epilogue_chunk<(EPI == kDwT ? kDw : EPI)>(p, r, m, n, row_ok, w.split, sr);
       }
       tc_fence_before();
       __syncwarp();
@@ -847,7 +874,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
         uint32_t r[32];
         tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
         tmem_ld_wait();
-        epilogue_chunk<kDw>(p, r, m, n, row_ok, w.split);
+        epilogue_chunk<kDw>(p, r, m, n, row_ok, w.split, StoreRow{});
       }
       tc_fence_before();
       __syncwarp();
@@ -1136,11 +1163,11 @@ DwPlan plan_dw(const rad_store* st, int64_t H) {
   }
 }
 
-template <int AK, int BKIND, int EPI>
+template <int AK, int BKIND, int EPI, int kEpiWarps2 = 8>
 int launch_pair(const TcParams& p, const CUtensorMap& ta, const CUtensorMap& tb, int64_t max_units, cudaStream_t s) {
   constexpr size_t smem = (size_t)kStages2 * kStage2Bytes + sizeof(SmemCtl2) + 1024;
   static_assert(smem <= 227 * 1024, "stage ring too deep");
-  auto kernel = tc_gemm_pair_kernel<AK, BKIND, EPI>;
+  auto kernel = tc_gemm_pair_kernel<AK, BKIND, EPI, kEpiWarps2>;
   // The kernel is persistent: the grid must not exceed the clusters that can be resident at once
   // (SM pairs that can host a cluster; fewer than half the SM count on some parts).
   static int resident_pairs = 0;
@@ -1148,7 +1175,7 @@ int launch_pair(const TcParams& p, const CUtensorMap& ta, const CUtensorMap& tb,
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return RAD_ECUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (num_sms() / 2));
-    cfg.blockDim = dim3(kThreads2);
+    cfg.blockDim = dim3(threads2(kEpiWarps2));
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -1164,7 +1191,7 @@ int launch_pair(const TcParams& p, const CUtensorMap& ta, const CUtensorMap& tb,
   }
   const int pairs = (int)std::max<int64_t>(1, std::min<int64_t>(max_units, resident_pairs));
   count_launch();
-  kernel<<<2 * pairs, kThreads2, smem, s>>>(p, ta, tb);
+  kernel<<<2 * pairs, threads2(kEpiWarps2), smem, s>>>(p, ta, tb);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 
@@ -1182,6 +1209,17 @@ int launch_sparse_pair(const TcParams& p, const CUtensorMap& tb, int64_t max_uni
   count_launch();
   tc_sparse_pair_kernel<<<2 * pairs, kSpThreads, smem, s>>>(p, tb);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+}
+
+// Columns of an output tile of the forward pass and the input gradient: the narrowest of 64, 128 and 256 with which
+// the tiles are still one wave of SM pairs, else 256.  An MMA takes the same time at every width, so within a wave a
+// narrower tile only spreads loads and epilogues over more SMs (2048 x 1024 x 1024 forward with store: 21.8 / 16.9 /
+// 22.0 us at 256 / 128 / 64, which are 32 / 64 / 128 tiles on 74 pairs; 328 x 640 x 520: 18.1 / 16.3 / 12.8), and a
+// second wave costs the whole contraction again (4096 x 1024 x 1024: 22.2 / 25.0 / 36.1).
+int dense_tile_width(int64_t M, int64_t N) {
+  for (int bn = 64; bn < BN; bn *= 2)
+    if (ceil_div(M, BM) * ceil_div(N, bn) <= planning_pairs()) return bn;
+  return BN;
 }
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
@@ -1211,7 +1249,7 @@ int tc_forward(int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t 
   rc = make_map(&tb, W, H, D, ldw, 64);               // MN-major B: box 64 (N) x 64 K rows
   if (rc != RAD_OK) return rc;
   TcParams p = {};
-  p.M = B; p.N = H; p.K = D; p.splits = 1; p.num_stages = 3;
+  p.M = B; p.N = H; p.K = D; p.splits = 1; p.num_stages = 3; p.bn = dense_tile_width(B, H);
   p.bias = bias; p.act = act;
   p.out_act = static_cast<bf16*>(out_act); p.ld_act = ld_act; p.out_z = out_z; p.ld_z = ld_z;
   p.out_zlow = static_cast<bf16*>(out_zlow); p.ld_zlow = ld_zlow; p.relubits = relubits; p.w32 = ceil_div(H, 32);
@@ -1226,7 +1264,8 @@ int tc_forward(int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t 
     p.st_scale = next->law == RAD_LAW_FIXED ? (float)H / (float)draws_per_row_host(next->p, H)
                                             : (float)kLaneRange / (float)keep_threshold_host(next->p);
   }
-  return launch_pair<kAK, kBMN, kFwd>(p, ta, tb, ceil_div(B, BM) * ceil_div(H, BN), s);
+  const int64_t units = ceil_div(B, BM) * ceil_div(H, p.bn);
+  return D <= kWideEpilogueK ? launch_pair<kAK, kBMN, kFwd, 16>(p, ta, tb, units, s) : launch_pair<kAK, kBMN, kFwd, 8>(p, ta, tb, units, s);
 }
 
 int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, const void* W, int64_t ldw,
@@ -1235,15 +1274,16 @@ int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, 
   CUtensorMap ta, tb;
   int rc = make_map(&ta, dZ, H, B, ldz, 128);         // K-major A (K = H)
   if (rc != RAD_OK) return rc;
-  rc = make_map(&tb, W, H, D, ldw, 128);              // K-major B: rows d (N), K = H contiguous
+  const int bn = dense_tile_width(B, D);
+  rc = make_map(&tb, W, H, D, ldw, bn / 2);           // K-major B: rows d (N), K = H contiguous
   if (rc != RAD_OK) return rc;
   TcParams p = {};
-  p.M = B; p.N = D; p.K = H; p.splits = 1; p.num_stages = 3;
+  p.M = B; p.N = D; p.K = H; p.splits = 1; p.num_stages = 3; p.bn = bn;
   p.relubits_prev = relubits_prev; p.z_prev = static_cast<const bf16*>(z_prev); p.ld_zprev = ld_zprev;
   p.out_dx = static_cast<bf16*>(dZ_prev); p.ld_dx = ldp;
   p.dev_status = dev_status;
   p.wait_limit_ns = wait_limit_ns();
-  return launch_pair<kAK, kBK_, kDx>(p, ta, tb, ceil_div(B, BM) * ceil_div(D, BN), s);
+  return launch_pair<kAK, kBK_, kDx>(p, ta, tb, ceil_div(B, BM) * ceil_div(D, bn), s);
 }
 
 int sm_pairs() { return planning_pairs(); }

@@ -234,3 +234,42 @@ def test_cuda_core_contractions_over_tiles_and_splits(B, D, H, dtype):
         ref, mag, K = x @ y, x.abs() @ y.abs(), x.shape[1]
         bound = (K ** 0.5 + 16) * 2.0 ** -24 * mag + (2.0 ** -8 * ref.abs() if low else 0)
         assert ((got.double() - ref).abs() <= bound + 1e-30).all()
+
+
+@pytest.mark.parametrize("B,D,H", [(64, 64, 64), (300, 72, 200), (257, 2048, 136), (1024, 640, 1000), (2500, 2056, 1032),
+                                   (5000, 128, 1096)])
+@pytest.mark.parametrize("act", ["relu", "gelu"])
+def test_dense_tile_widths(B, D, H, act):
+    """Forward with the next layer's store and input gradient on the tensor cores at tiles of 64, 128 and 256 columns with
+    remainders, and with either number of epilogue warps: the forward's store is the store of its own output bit for
+    bit, values against float64 within one bf16 rounding and the float32 sums' error."""
+    import paper_2007_10412_b200 as rad
+    bf = torch.bfloat16
+    g = torch.Generator(device="cuda").manual_seed(B + D + H)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").to(bf)
+    A, W, dZ, zp, b = rnd(B, D), rnd(D, H), rnd(B, H), rnd(B, D), rnd(H).float()
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    fill = rad.Store("different", "bf16", B, H, 0.2, seed=9, layer=2, step=3, relu_bits=True)
+    own = rad.Store("different", "bf16", B, H, 0.2, seed=9, layer=2, step=3, relu_bits=True)
+    for st in (fill, own):
+        st.values.zero_()
+    out, zl = torch.empty(B, H, dtype=bf, device="cuda"), torch.empty(B, H, dtype=bf, device="cuda")
+    rad.rad_linear_forward_fill(A, W, b, act, out, fill, out_zlow=zl, relubits=fill.relubits, dev_status=status)
+    rad.rad_linear_forward_store(out, own, status)
+    dX = torch.empty(B, D, dtype=bf, device="cuda")
+    rad.rad_linear_input_grad(dZ, W, z_prev=zp if act == "gelu" else None, dZ_prev=dX, dev_status=status)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    for x, y in ((fill.values, own.values), (fill.keepbits, own.keepbits), (fill.offsets, own.offsets), (fill.nnz, own.nnz),
+                 (fill.relubits, own.relubits)):
+        assert torch.equal(x, y)
+    z = A.double() @ W.double() + b.double()
+    tol = (max(D, H) ** 0.5 + 16) * 2.0 ** -24
+    mag = A.double().abs() @ W.double().abs() + b.abs()
+    assert ((zl.double() - z).abs() <= tol * mag + 2.0 ** -8 * z.abs()).all()
+    dx, mx = dZ.double() @ W.double().T, dZ.double().abs() @ W.double().abs().T
+    if act == "gelu":
+        x = zp.double()
+        d = 0.5 * (1 + torch.erf(x / 2 ** 0.5)) + x * torch.exp(-0.5 * x * x) / (2 * np.pi) ** 0.5
+        dx, mx = dx * d, mx * (d.abs() + 1e-3)
+    assert ((dX.double() - dx).abs() <= 8 * tol * mx + 2.0 ** -8 * dx.abs()).all()
