@@ -3,27 +3,33 @@
 // the cell is kept at the sampling fraction, the scalar input whole, ReLU derivatives at 1 bit).
 //
 // The recurrence of one minibatch row never looks at another row, so one CTA owns one row for all
-// T steps and no CTA ever waits for another.  Four warps carry the hidden units (one per thread,
-// the unit's column of W_hh in registers, the state broadcast from shared memory); a fifth warp
-// draws the step's Philox mask, compacts the kept entries of h_{t-1} and writes keep bits and
-// offsets.  Backward through time mirrors it: the fifth warp prefetches a step's kept entries into
-// shared memory while the others form dz_t, dh_{t-1} = dz_t W_hh^T and the row's share of dW_hh;
-// per-row partial gradients are summed over rows in row order by a last kernel.
+// T steps and no CTA ever waits for another.  What bounds both kernels is the chain of one step
+// (state out of shared memory, multiply-adds, sum, state back, barrier), so a step does nothing else on that chain:
+// four threads share a hidden unit (a quarter of its column, or row, of W_hh in registers, paired multiply-adds, two
+// shuffles), and everything that only needs a step's state (masks, compaction, derivative bits forward; lists of kept
+// entries backward) runs in other warps that meet the unit warps once every eight or four steps and stay a group
+// behind or ahead, half a warp per step.  A second CTA fits on an SM, which a batch of 150 on 148 SMs needs (and which
+// then sets the time: two CTAs share its issue slots).  Batch 150, T = 784, 100 hidden units, against one thread
+// per unit with the side work beside every step: forward 565 -> 279 us, backward 732 -> 470; the same with the updates
+// of dW_hh and the sums in four warps of their own, a column per thread: backward 511.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "common.cuh"
 
 namespace rad {
 namespace {
 
-constexpr int kHdMax = 128;          // hidden units per CTA row (one thread each)
-constexpr int kRnnThreads = 160;     // backward: 4 unit warps + 1 helper warp
-constexpr int kRnnFwdThreads = 192;  // forward: 4 unit warps, the store warp, the warp that draws the masks
+constexpr int kHdMax = 128;          // hidden units per row
+constexpr int kFwdGroup = 8;         // forward: steps between meetings of all warps, half a store warp each
+constexpr int kStoreWarps = kFwdGroup / 2;
+constexpr int kBwdGroup = 4;         // backward: the same, half a list warp each
+constexpr int kListWarps = kBwdGroup / 2;
 
 struct RnnParams {
   int64_t B, T;
-  int32_t Hd, w32, ngroups;
+  int32_t Hd, w32;
   int32_t same;                      // same-sample: the mask does not depend on the row
   KeepThreshold keepT;               // keep threshold
   float scale;
@@ -38,266 +44,371 @@ struct RnnParams {
   int64_t* nnz_rows;                 // B: kept entries of the row over all steps
   // backward
   const float* dh_last;              // B x Hd
-  float* part_whh;                   // B x Hd x Hd
-  float* part_vec;                   // B x 2 x Hd: dW_ih, db
+  float* part;                       // B x (Hd x Hd + 2 Hd): the row's shares of dW_hh, dW_ih, db
   int32_t* dev_status;
 };
 
-__global__ void __launch_bounds__(kRnnFwdThreads) irnn_forward_kernel(const RnnParams p, const PhiloxKeys ks) {
+// Barrier 1: the unit warps alone.
+__device__ __forceinline__ void unit_barrier(int threads) { asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory"); }
+
+// Unit j = 8 warp + lane % 8, part q = lane / 8 of its contraction: k = 16 i + 4 q .. + 3 for i < KP / 4 (Hd <= 4 KP).
+template <int KP>
+struct UnitDot {
+  f32x2 w[KP / 2];
+  // weight(k) = element k of the unit's column or row, zero outside
+  template <typename F>
+  __device__ __forceinline__ void init(int q, F weight) {
+#pragma unroll
+    for (int i = 0; i < KP / 4; ++i) {
+      const int k = 16 * i + 4 * q;
+      w[2 * i] = pack2(weight(k), weight(k + 1));
+      w[2 * i + 1] = pack2(weight(k + 2), weight(k + 3));
+    }
+  }
+  // multiply-adds of state entries 16 i + 4 q .. for i in [I0, I1) onto the part's four running sums
+  template <int I0, int I1>
+  __device__ __forceinline__ void add(const float* state, int q, f32x2& a0, f32x2& a1) const {
+#pragma unroll
+    for (int i = I0; i < I1; ++i) {
+      const ulonglong2 s = *reinterpret_cast<const ulonglong2*>(state + 16 * i + 4 * q);
+      fma2(a0, w[2 * i], s.x);
+      fma2(a1, w[2 * i + 1], s.y);
+    }
+  }
+  // the sums of all parts; all four lanes get it
+  static __device__ __forceinline__ float reduce(f32x2 a0, f32x2 a1) {
+    float b0, b1, b2, b3;
+    unpack2(a0, b0, b1);
+    unpack2(a1, b2, b3);
+    float z = (b0 + b1) + (b2 + b3);
+    z += __shfl_xor_sync(0xffffffffu, z, 8);
+    z += __shfl_xor_sync(0xffffffffu, z, 16);
+    return z;
+  }
+};
+
+template <int KP>
+__global__ void __launch_bounds__(32 * (KP / 2 + kStoreWarps), 2) irnn_forward_kernel(const RnnParams p, const PhiloxKeys ks, int unit_warps) {
   extern __shared__ float sm[];
   float* s_x = sm;                                   // T inputs of this row
-  __shared__ __align__(16) float s_h[2][kHdMax];
+  constexpr int kGroup = kFwdGroup, kRing = 4 * kGroup;                  // states: two groups of steps and what the store warps still read
+  __shared__ __align__(16) float s_h[kRing][kHdMax];
+  __shared__ __align__(16) uint32_t s_mask[2][kGroup][4];
+  __shared__ uint32_t s_cnt[2][kGroup];             // kept entries of a step
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t b = blockIdx.x;
   const int Hd = p.Hd;
-  for (int64_t t = tid; t < p.T; t += kRnnFwdThreads) s_x[t] = p.x[b * p.T + t];
-  if (tid < kHdMax) { s_h[0][tid] = 0.0f; s_h[1][tid] = 0.0f; }
-  // unit j keeps column j of W_hh in registers (zero beyond Hd)
-  float wcol[kHdMax];
-  float bias = 0.0f, wih = 0.0f;
-  const int j = tid;
-  if (warp < 4) {
-#pragma unroll
-    for (int k = 0; k < kHdMax; ++k) wcol[k] = (k < Hd && j < Hd) ? p.W_hh[(int64_t)k * Hd + j] : 0.0f;
-    if (j < Hd) { bias = p.b_ih[j] + p.b_hh[j]; wih = p.W_ih[j]; }
-  }
-  // The keep decisions need no data: the sixth warp draws the words of step t + 2 while step t runs (one
-  // keep-bit word decides 32 units; four lanes make it together, one generator output each).
-  __shared__ uint32_t s_mask[4][8];
-  const uint32_t mask_row = p.same ? 0u : (uint32_t)b;
-  auto draw = [&](int64_t t) {
-    const uint32_t m = philox_keep32_quad((uint32_t)(lane >> 2), mask_row, p.c2, p.step0 + (uint32_t)t, ks, p.keepT, lane);
-    if ((lane & 3) == 0) s_mask[t & 3][lane >> 2] = m;
-  };
-  if (warp == 5) {
-    draw(1);
-    if (p.T >= 2) draw(2);
-  }
+  for (int64_t t = tid; t < p.T; t += blockDim.x) s_x[t] = p.x[b * p.T + t];
+  for (int i = tid; i < kRing * kHdMax; i += blockDim.x) (&s_h[0][0])[i] = 0.0f;
+  const int64_t groups = (p.T + kGroup - 1) / kGroup;
   __syncthreads();
-  uint32_t off = 0;                                  // store warp: values of this row so far
-  for (int64_t t = 1; t <= p.T; ++t) {
-    const float* hc = s_h[(t - 1) & 1];
-    if (warp == 5) {
-      if (t + 2 <= p.T) draw(t + 2);
-    } else if (warp == 4) {
-      // store of h_{t-1}: keep bits of the step, kept entries scaled and appended to the row's values
-      // four lanes share a keep-bit word and place eight of its units each
-      const int wi = lane >> 2, q = lane & 3;
-      uint32_t m = s_mask[t & 3][wi];
-      const bool word_ok = wi * 32 < Hd;
-      m = word_ok ? m & (0xffffffffu >> (32 - min(32, Hd - wi * 32))) : 0u;
-      // the word's count enters the scan once (first lane of the four); every lane then places a quarter of it
-      const uint32_t c = q == 0 ? __popc(m) : 0u;
-      uint32_t incl = c;
+  if (warp < unit_warps) {
+    const int j = warp * 8 + (lane & 7), q = lane >> 3;
+    UnitDot<KP> dot;
+    dot.init(q, [&](int k) { return k < Hd && j < Hd ? p.W_hh[(int64_t)k * Hd + j] : 0.0f; });
+    float bias = 0.0f, wih = 0.0f;
+    if (j < Hd && q == 0) { bias = p.b_ih[j] + p.b_hh[j]; wih = p.W_ih[j]; }
+    const bool writer = lane < 8 && j < Hd;
+    const float* x = s_x;
+    int left = (int)p.T;
+    for (int g = 0; left > 0; ++g, left -= kGroup, x += kGroup) {
+      float* h = s_h[(g * kGroup) % kRing];          // the group's first state; the next group's first may be the ring's first
+      float* h_next = s_h[(g * kGroup + kGroup) % kRing];
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t n = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += n;
+      for (int s = 0; s < kGroup; ++s) {
+        if (s < left) {
+          // z_j = x_t W_ih[j] + b_ih[j] + b_hh[j] + sum_k h_{t-1}[k] W_hh[k][j]
+          f32x2 a0 = pack2(fmaf(x[s], wih, bias), 0.0f), a1 = 0;
+          dot.template add<0, KP / 4>(h + s * kHdMax, q, a0, a1);
+          const float z = dot.reduce(a0, a1);
+          if (writer) (s + 1 < kGroup ? h + (s + 1) * kHdMax : h_next)[j] = fmaxf(z, 0.0f);
+          if (s + 1 < kGroup && s + 1 < left) unit_barrier(32 * unit_warps);
+        }
       }
-      const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-      const uint32_t word_pos = __shfl_sync(0xffffffffu, off + incl - c, lane & ~3);
+      __syncthreads();
+    }
+    if (writer) p.h_last[b * Hd + j] = s_h[p.T % kRing][j];
+    return;
+  }
+  // ---- store warps: half a warp per step; masks of group g and the store of group g - 1 while the units run group g ----
+  const int half = lane >> 4, l = lane & 15, s = 2 * (warp - unit_warps) + half, wi = l >> 2, q = l & 3;
+  const uint32_t mask_row = p.same ? 0u : (uint32_t)b;
+  const uint32_t word_ok = wi * 32 < Hd ? 0xffffffffu >> (32 - min(32, Hd - wi * 32)) : 0u;
+  uint32_t base = 0;                                 // values of this row before the group that is being stored
+  // derivative bits of state h (every lane of the half passes its step's): word w in lanes w of the half
+  auto relu_words = [&](const float* h) {
+    uint32_t mine = 0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const uint32_t bal = __ballot_sync(0xffffffffu, h[16 * r + l] > 0.0f);
+      if (l == r >> 1) mine |= ((bal >> (16 * half)) & 0xffffu) << (16 * (r & 1));
+    }
+    return mine;
+  };
+  auto store_group = [&](int64_t g) {
+    const int64_t t = g * kGroup + 1 + s;
+    const bool in = t <= p.T;
+    const float* h = s_h[(t - 1) % kRing];
+    const uint4 mw = *reinterpret_cast<const uint4*>(s_mask[g & 1][s]);
+    uint32_t before = 0, all = 0;                    // kept entries of the group's earlier steps, of the group
+#pragma unroll
+    for (int i = 0; i < kGroup; ++i) {
+      const uint32_t c = s_cnt[g & 1][i];
+      before += i < s ? c : 0u;
+      all += c;
+    }
+    const uint32_t relu = relu_words(h);
+    if (in && t > 1 && l < p.w32) p.relubits[((t - 2) * p.B + b) * p.w32 + l] = relu;
+    const uint32_t m = wi == 0 ? mw.x : wi == 1 ? mw.y : wi == 2 ? mw.z : mw.w;
+    const uint32_t total = s_cnt[g & 1][s];
+    const uint32_t off = base + before;
+    if (in) {
       if ((int64_t)off + total <= p.cap_row) {
-        // units 8 q .. 8 q + 7 of the word: loaded whether kept or not (two 16-byte loads instead of up to
-        // eight dependent ones), stored where kept
+        // units 8 q .. 8 q + 7 of the word: loaded whether kept or not, stored where kept
         const uint32_t sub = (m >> (8 * q)) & 0xffu;
         if (sub != 0) {
-          const float4 lo = *reinterpret_cast<const float4*>(hc + wi * 32 + 8 * q);
-          const float4 hi = *reinterpret_cast<const float4*>(hc + wi * 32 + 8 * q + 4);
+          const float4 lo = *reinterpret_cast<const float4*>(h + wi * 32 + 8 * q);
+          const float4 hi = *reinterpret_cast<const float4*>(h + wi * 32 + 8 * q + 4);
           const float v[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-          float* out = p.values + b * p.cap_row + word_pos + __popc(m & ((1u << (8 * q)) - 1u));
+          const uint32_t earlier = (wi > 0 ? __popc(mw.x) : 0) + (wi > 1 ? __popc(mw.y) : 0) + (wi > 2 ? __popc(mw.z) : 0);
+          float* out = p.values + b * p.cap_row + off + earlier + __popc(m & ((1u << (8 * q)) - 1u));
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             if ((sub >> i) & 1u) *out++ = v[i] * p.scale;
         }
-      } else if (lane == 0) {
+      } else if (l == 0) {
         raise_status(p.dev_status, RAD_DEV_ECAPACITY);
       }
       const int64_t sb = (t - 1) * p.B + b;
       if (q == 0 && wi < p.w32) p.keepbits[sb * p.w32 + wi] = m;
-      if (lane == 0) p.offsets[sb] = off;
-      off += total;
-    } else {
-      // z_j = x_t W_ih[j] + b_ih[j] + b_hh[j] + sum_k h_{t-1}[k] W_hh[k][j]
-      // four partial sums keep the FMA pipe busy; they are combined in a fixed order
-      float z0 = fmaf(s_x[t - 1], wih, bias), z1 = 0.0f, z2 = 0.0f, z3 = 0.0f;
-#pragma unroll
-      for (int k = 0; k < kHdMax; k += 4) {
-        const float4 h4 = *reinterpret_cast<const float4*>(hc + k);
-        z0 = fmaf(h4.x, wcol[k], z0); z1 = fmaf(h4.y, wcol[k + 1], z1);
-        z2 = fmaf(h4.z, wcol[k + 2], z2); z3 = fmaf(h4.w, wcol[k + 3], z3);
-      }
-      const float z = (z0 + z1) + (z2 + z3);
-      const float hn = (j < Hd) ? fmaxf(z, 0.0f) : 0.0f;
-      s_h[t & 1][j] = hn;
-      const uint32_t bits = __ballot_sync(0xffffffffu, hn > 0.0f);
-      if (lane == 0 && warp < p.w32) p.relubits[((t - 1) * p.B + b) * p.w32 + warp] = bits;
+      if (l == 0) p.offsets[sb] = off;
     }
+    base += all;
+  };
+  for (int64_t g = 0; g < groups; ++g) {
+    const int64_t t = g * kGroup + 1 + s;
+    const uint32_t m = philox_keep32_quad((uint32_t)wi, mask_row, p.c2, p.step0 + (uint32_t)t, ks, p.keepT, lane) &
+                       (t <= p.T ? word_ok : 0u);
+    uint32_t c = __popc(m);
+    c += __shfl_xor_sync(0xffffffffu, c, 4);
+    c += __shfl_xor_sync(0xffffffffu, c, 8);
+    if (q == 0) s_mask[g & 1][s][wi] = m;
+    if (l == 0) s_cnt[g & 1][s] = c;
+    if (g > 0) store_group(g - 1);
     __syncthreads();
   }
-  if (warp < 4 && j < Hd) p.h_last[b * Hd + j] = s_h[p.T & 1][j];
-  if (warp == 4 && lane == 0) p.nnz_rows[b] = off;
+  store_group(groups - 1);
+  const uint32_t relu = relu_words(s_h[p.T % kRing]);
+  if (s == 0 && l < p.w32) p.relubits[((p.T - 1) * p.B + b) * p.w32 + l] = relu;
+  if (s == 0 && l == 0) p.nnz_rows[b] = base;
 }
 
-constexpr int kRing = 8;             // steps of kept entries in flight in the backward kernel
-
-__global__ void __launch_bounds__(kRnnThreads) irnn_backward_kernel(const RnnParams p) {
-  extern __shared__ float sm[];
+template <int KP>
+__global__ void __launch_bounds__(32 * (KP / 2 + kListWarps), 2) irnn_backward_kernel(const RnnParams p, int unit_warps) {
+  extern __shared__ __align__(16) float sm[];
+  constexpr int kGroup = kBwdGroup;
   const int Hd = p.Hd;
-  const int S = Hd + 1;                               // odd stride: conflict-free rows and columns
+  const int S = (Hd + 3) & ~3;                        // floats per row of the row's share of dW_hh
   const int64_t Tp = (p.T + 3) & ~(int64_t)3;
   float* s_x = sm;                                    // T
-  float* s_dw = s_x + Tp;                             // Hd x S: this row's share of dW_hh
-  uint32_t* s_keep = reinterpret_cast<uint32_t*>(s_dw + ((Hd * S + 3) & ~3));   // T x w32 keep bits of the row
+  float* s_dw = s_x + Tp;                             // Hd x S
+  uint32_t* s_keep = reinterpret_cast<uint32_t*>(s_dw + Hd * S);                // T x w32 keep bits of the row
   uint32_t* s_rl = s_keep + p.T * p.w32;              // T x w32 ReLU bits
   uint32_t* s_off = s_rl + p.T * p.w32;               // T value offsets
-  __shared__ __align__(16) float s_dz[2][kHdMax];
-  __shared__ __align__(16) uint32_t s_kidx[kRing][kHdMax];
-  __shared__ __align__(16) float s_kval[kRing][kHdMax];
-  __shared__ uint32_t s_kcnt[kRing];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ __align__(16) float s_dz[4][kHdMax];
+  __shared__ uint32_t s_kidx[2 * kGroup][kHdMax];     // kept units of a step of this group or the next: offset of their row of s_dw
+  __shared__ float s_kval[2 * kGroup][kHdMax];
+  __shared__ uint32_t s_kcnt[2 * kGroup];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, threads = blockDim.x;
   const int64_t b = blockIdx.x;
-  for (int64_t t = tid; t < p.T; t += kRnnThreads) {
+  for (int64_t t = tid; t < p.T; t += threads) {
     s_x[t] = p.x[b * p.T + t];
     s_off[t] = p.offsets[t * p.B + b];
   }
-  for (int64_t i = tid; i < p.T * p.w32; i += kRnnThreads) {
+  for (int64_t i = tid; i < p.T * p.w32; i += threads) {
     const int64_t at = ((i / p.w32) * p.B + b) * p.w32 + (i % p.w32);
     s_keep[i] = p.keepbits[at];
     s_rl[i] = p.relubits[at];
   }
-  for (int i = tid; i < Hd * S; i += kRnnThreads) s_dw[i] = 0.0f;
-  if (tid < kHdMax) { s_dz[0][tid] = 0.0f; s_dz[1][tid] = 0.0f; }
-  const int k = tid;                                  // unit k: row k of W_hh in registers
-  float wrow[kHdMax];
-  float dh = 0.0f, dwih = 0.0f, dbs = 0.0f, dwih_c = 0.0f, dbs_c = 0.0f;
-  if (warp < 4) {
-#pragma unroll
-    for (int jj = 0; jj < kHdMax; ++jj) wrow[jj] = (k < Hd && jj < Hd) ? p.W_hh[(int64_t)k * Hd + jj] : 0.0f;
-    if (k < Hd) dh = p.dh_last[b * Hd + k];
-  }
+  for (int i = tid; i < Hd * S; i += threads) s_dw[i] = 0.0f;
+  for (int i = tid; i < 4 * kHdMax; i += threads) (&s_dz[0][0])[i] = 0.0f;
+  const int64_t groups = (p.T + kGroup - 1) / kGroup;
   __syncthreads();
-  // helper warp: list of the kept units of step t and an asynchronous copy of their values into
-  // ring slot t % kRing; one commit group per call, so groups can be counted
-  auto prefetch = [&](int64_t t) {
-    if (t >= 1) {
-      const int slot = (int)(t % kRing);
+  const int64_t n_part = (int64_t)Hd * Hd + 2 * Hd;
+  if (warp >= unit_warps) {
+    // ---- list warps: half a warp per step; the kept entries of group g + 1 while the units run group g ----
+    const int half = lane >> 4, l = lane & 15, s = 2 * (warp - unit_warps) + half;
+    auto list_group = [&](int64_t g) {
+      const int64_t t = p.T - g * kGroup - s;         // descending
+      const int slot = (int)(g & 1) * kGroup + s;
       uint32_t m = 0;
-      if (lane < p.ngroups) m = (s_keep[(t - 1) * p.w32 + (lane >> 2)] >> (8 * (lane & 3))) & 0xffu;
+      if (t >= 1 && (l >> 2) < p.w32) m = (s_keep[(t - 1) * p.w32 + (l >> 2)] >> (8 * (l & 3))) & 0xffu;
       const uint32_t c = __popc(m);
       uint32_t incl = c;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t n = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += n;
+      for (int o = 1; o < 16; o <<= 1) {
+        const uint32_t n = __shfl_up_sync(0xffffffffu, incl, o, 16);
+        if (l >= o) incl += n;
       }
-      const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-      const uint32_t off = s_off[t - 1];
-      uint32_t pos = incl - c;
+      const uint32_t total = __shfl_sync(0xffffffffu, incl, 15, 16);
+      if (t >= 1) {
+        const uint32_t off = s_off[t - 1];
+        uint32_t pos = incl - c;
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if ((m >> i) & 1u) s_kidx[slot][pos++] = (uint32_t)(lane * 8 + i);
-      const bool fits = (int64_t)off + total <= p.cap_row;
-      for (uint32_t i = lane; i < total; i += 32) {
-        if (fits) {
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(&s_kval[slot][i])),
-                       "l"(p.values + b * p.cap_row + off + i) : "memory");
-        } else {
-          s_kval[slot][i] = 0.0f;
+        for (int i = 0; i < 8; ++i)
+          if ((m >> i) & 1u) s_kidx[slot][pos++] = (uint32_t)((l * 8 + i) * S);
+        const bool fits = (int64_t)off + total <= p.cap_row;
+        for (uint32_t i = l; i < total; i += 16) {
+          if (fits)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(&s_kval[slot][i])),
+                         "l"(p.values + b * p.cap_row + off + i) : "memory");
+          else
+            s_kval[slot][i] = 0.0f;
         }
+        if (l == 0) s_kcnt[slot] = total;
       }
-      if (lane == 0) s_kcnt[slot] = total;
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  if (warp == 4) {
-    for (int d = 0; d < kRing - 1; ++d) prefetch(p.T - d);
-    asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 2) : "memory");      // step T has landed
-  }
-  // dz_t = dh_t * relu'(h_t) and the exact gradients of the input weights and biases, by the thread of unit k;
-  // the two buffers of dz alternate, so a step needs one barrier: the dz of step t - 1 is written at the end of
-  // step t while the other threads may still read the dz of step t
-  auto make_dz = [&](int64_t t) {
-    const uint32_t rbits = warp < p.w32 ? s_rl[(t - 1) * p.w32 + warp] : 0u;
-    const float dz = ((rbits >> lane) & 1u) ? dh : 0.0f;
-    s_dz[t & 1][k] = dz;
-    // compensated sums: T terms of one sign would otherwise drift past the float32 tolerance
-    const float yi = fmaf(s_x[t - 1], dz, -dwih_c), ti = dwih + yi;
-    dwih_c = (ti - dwih) - yi; dwih = ti;
-    const float yb = dz - dbs_c, tb = dbs + yb;
-    dbs_c = (tb - dbs) - yb; dbs = tb;
-  };
-  if (warp < 4) make_dz(p.T);
-  __syncthreads();
-  for (int64_t t = p.T; t >= 1; --t) {
-    const int slot = (int)(t % kRing);
-    if (warp < 4) {
-      const float* dzv = s_dz[t & 1];
-      // dh_{t-1}[k] = sum_j dz[j] W_hh[k][j]
-      float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
-#pragma unroll
-      for (int jj = 0; jj < kHdMax; jj += 4) {
-        const float4 d4 = *reinterpret_cast<const float4*>(dzv + jj);
-        a0 = fmaf(d4.x, wrow[jj], a0); a1 = fmaf(d4.y, wrow[jj + 1], a1);
-        a2 = fmaf(d4.z, wrow[jj + 2], a2); a3 = fmaf(d4.w, wrow[jj + 3], a3);
-      }
-      dh = (a0 + a1) + (a2 + a3);
-      // dW_hh[kept unit d, j] += h_hat_{t-1}[d] * dz[j]: thread j owns column j of every row
-      if (k < Hd) {
-        const float dzj = dzv[k];
-        const uint32_t cnt = s_kcnt[slot];
-        uint32_t n = 0;
-        // four kept units at a time: their rows of dW_hh are different, so the four updates do not wait
-        // for one another
-        for (; n + 4 <= cnt; n += 4) {
-          const uint4 id = *reinterpret_cast<const uint4*>(&s_kidx[slot][n]);
-          const float4 hv = *reinterpret_cast<const float4*>(&s_kval[slot][n]);
-          float* c0 = s_dw + id.x * S + k; float* c1 = s_dw + id.y * S + k;
-          float* c2 = s_dw + id.z * S + k; float* c3 = s_dw + id.w * S + k;
-          const float x0 = *c0, x1 = *c1, x2 = *c2, x3 = *c3;
-          *c0 = fmaf(hv.x, dzj, x0); *c1 = fmaf(hv.y, dzj, x1);
-          *c2 = fmaf(hv.z, dzj, x2); *c3 = fmaf(hv.w, dzj, x3);
-        }
-        for (; n < cnt; ++n) {
-          float* cell = s_dw + s_kidx[slot][n] * S + k;
-          *cell = fmaf(s_kval[slot][n], dzj, *cell);
-        }
-      }
-      if (t > 1) make_dz(t - 1);
-    } else {
-      // beside the unit warps: the list of a later step (its ring slot was read a step ago)
-      prefetch(t - (kRing - 1));
-      asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 2) : "memory");    // step t - 1 has landed
-    }
+      asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    };
+    list_group(0);
     __syncthreads();
+    for (int64_t g = 0; g < groups; ++g) {
+      if (g + 1 < groups) list_group(g + 1);
+      __syncthreads();
+    }
+  } else {
+    const int k = warp * 8 + (lane & 7), q = lane >> 3;                  // unit k: row k of W_hh
+    UnitDot<KP> dot;
+    dot.init(q, [&](int jj) { return k < Hd && jj < Hd ? p.W_hh[(int64_t)k * Hd + jj] : 0.0f; });
+    const int quads = S / 4, n0 = tid / quads, jq = tid - n0 * quads, nstep = 32 * unit_warps / quads;   // dW_hh: (kept entry, four columns)
+    float sum = 0.0f, comp = 0.0f;                    // part 0: dW_ih of the unit, part 1: its bias gradient
+    const bool real = k < Hd;
+    const uint32_t my_bit = real ? 1u << (k & 31) : 0u;
+    const uint32_t* rl = s_rl + (p.T - 1) * p.w32 + (warp >> 2);          // derivative bits of the step whose dz is made next
+    const float* x = s_x + (p.T - 1);
+    // dz_t = dh_t * relu'(h_t) into place, and the exact gradients of the input weight and bias: compensated sums,
+    // T terms of one sign would otherwise drift past the float32 tolerance
+    auto make_dz = [&](float* place, float dh) {
+      const float dz = (*rl & my_bit) != 0 ? dh : 0.0f;
+      if (lane < 8) place[k] = dz;
+      const float y = fmaf(q == 0 ? *x : 1.0f, dz, -comp), v = sum + y;
+      comp = (v - sum) - y; sum = v;
+      rl -= p.w32; --x;
+    };
+    // dW_hh[kept unit d, j] += h_hat_{t-1}[d] * dz_t[j]: a thread takes four neighbouring columns of every nstep-th kept
+    // unit.  Off the chain: a step's update runs beside the next step's multiply-adds (the group's last one at its end).
+    const bool updater = n0 < nstep;
+    const int my_n = min(n0, kHdMax - 1);
+    struct Update { float4 z; float* cell; float v; uint32_t cnt; };
+    auto fetch = [&](const float* dz, int slot) {
+      Update u;
+      u.cnt = updater ? s_kcnt[slot] : 0u;
+      u.cell = s_dw + s_kidx[slot][my_n] + 4 * jq;
+      u.v = s_kval[slot][my_n];
+      u.z = *reinterpret_cast<const float4*>(dz + 4 * jq);
+      return u;
+    };
+    auto apply = [&](float4* cell, float v, const float4& z) {
+      float4 c = *cell;
+      c.x = fmaf(v, z.x, c.x); c.y = fmaf(v, z.y, c.y); c.z = fmaf(v, z.z, c.z); c.w = fmaf(v, z.w, c.w);
+      *cell = c;
+    };
+    auto add_dw = [&](const Update& u, int slot) {
+      if ((uint32_t)n0 < u.cnt) {
+        apply(reinterpret_cast<float4*>(u.cell), u.v, u.z);
+        for (uint32_t n = n0 + nstep; n < u.cnt; n += nstep)
+          apply(reinterpret_cast<float4*>(s_dw + s_kidx[slot][n] + 4 * jq), s_kval[slot][n], u.z);
+      }
+    };
+    make_dz(s_dz[0], real ? p.dh_last[b * Hd + k] : 0.0f);
+    __syncthreads();
+    int left = (int)p.T;
+    for (int g = 0; left > 0; ++g, left -= kGroup) {
+      const int slot0 = (g & 1) * kGroup;
+      Update u;
+#pragma unroll
+      for (int s = 0; s < kGroup; ++s) {
+        if (s < left) {
+          // dh_{t-1}[k] = sum_j dz_t[j] W_hh[k][j]; dz_t lies at place s of the ring
+          if (s > 0) u = fetch(s_dz[s - 1], slot0 + s - 1);
+          f32x2 a0 = 0, a1 = 0;
+          dot.template add<0, KP / 4>(s_dz[s], q, a0, a1);
+          const float dh = dot.reduce(a0, a1);
+          if (s + 1 < left) make_dz(s_dz[(s + 1) % kGroup], dh);
+          if (s > 0) add_dw(u, slot0 + s - 1);
+          if (s + 1 < kGroup && s + 1 < left) unit_barrier(32 * unit_warps);
+        }
+      }
+      const int last = min(kGroup, left) - 1;
+      u = fetch(s_dz[last], slot0 + last);
+      if (last > 0) unit_barrier(32 * unit_warps);    // the update before the last one is in place
+      add_dw(u, slot0 + last);
+      __syncthreads();
+    }
+    if (real && q < 2) p.part[b * n_part + (int64_t)Hd * Hd + q * Hd + k] = sum;
   }
-  for (int i = tid; i < Hd * Hd; i += kRnnThreads) p.part_whh[b * Hd * Hd + i] = s_dw[(i / Hd) * S + (i % Hd)];
-  if (warp < 4 && k < Hd) {
-    p.part_vec[(b * 2 + 0) * Hd + k] = dwih;
-    p.part_vec[(b * 2 + 1) * Hd + k] = dbs;
+  for (int i = tid; i < Hd * Hd; i += threads) p.part[b * n_part + i] = s_dw[(i / Hd) * S + (i % Hd)];
+}
+
+// Sums over the rows' shares: dW_hh (n1 numbers), dW_ih and db (Hd each): 32 columns and 32 row lanes per CTA, the lanes'
+// sums added in order; the first CTA also adds the rows' counts.  One launch; with one thread per column it was
+// four of 7 to 15 us.
+__global__ void __launch_bounds__(1024) irnn_sum_rows_kernel(const float* part, int64_t B, int64_t n1, int64_t Hd, float* dW_hh, float* dW_ih,
+                                                             float* db, const int64_t* nnz_rows, const int64_t* nnz_last, int64_t* nnz_out) {
+  __shared__ float s[32][33];
+  const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
+  const int64_t i = (int64_t)blockIdx.x * 32 + lane, n = n1 + 2 * Hd;
+  float acc = 0.0f;
+  if (i < n)
+#pragma unroll 8
+    for (int64_t b = r; b < B; b += 32) acc += part[b * n + i];
+  s[r][lane] = acc;
+  __syncthreads();
+  if (r == 0 && i < n) {
+    float t = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 32; ++q) t += s[q][lane];
+    (i < n1 ? dW_hh[i] : i < n1 + Hd ? dW_ih[i - n1] : db[i - n1 - Hd]) = t;
+  }
+  if (r == 1 && blockIdx.x == 0 && nnz_out != nullptr) {
+    int64_t c = 0;
+    for (int64_t b = lane; b < B; b += 32) c += nnz_rows[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (lane == 0) { nnz_out[0] = c; nnz_out[1] = nnz_last[0]; }
   }
 }
 
-// out[i] = sum over rows of part[b][i], in row order
-__global__ void __launch_bounds__(256) sum_rows_kernel(const float* part, int64_t B, int64_t n, int64_t stride,
-                                                       int64_t offset, float* out) {
-  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (i >= n) return;
-  float s = 0.0f;
-  for (int64_t b = 0; b < B; ++b) s += part[b * stride + offset + i];
-  out[i] = s;
+// The kernels for a hidden size: KP = entries of a unit's contraction per thread, 4 KP >= Hd.
+template <int KP>
+int launch_irnn_forward(const RnnParams& p, const PhiloxKeys& ks, size_t smem, cudaStream_t s) {
+  const int uw = (int)ceil_div(p.Hd, 8);
+  RAD_CUDA_TRY(cudaFuncSetAttribute(irnn_forward_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem, 1024)));
+  count_launch();
+  irnn_forward_kernel<KP><<<(unsigned)p.B, 32 * (uw + kStoreWarps), smem, s>>>(p, ks, uw);
+  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
-
-__global__ void sum_nnz_kernel(const int64_t* rows, int64_t B, int64_t* out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    int64_t s = 0;
-    for (int64_t b = 0; b < B; ++b) s += rows[b];
-    out[0] = s;
-  }
+template <int KP>
+int launch_irnn_backward(const RnnParams& p, size_t smem, cudaStream_t s) {
+  const int uw = (int)ceil_div(p.Hd, 8);
+  RAD_CUDA_TRY(cudaFuncSetAttribute(irnn_backward_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  count_launch();
+  irnn_backward_kernel<KP><<<(unsigned)p.B, 32 * (uw + kListWarps), smem, s>>>(p, uw);
+  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+}
+// f(std::integral_constant<KP>) for the smallest KP in 8, 16, 20, 24, 28, 32 that holds Hd units
+template <typename F>
+int with_parts(int Hd, F f) {
+  if (Hd <= 32) return f(std::integral_constant<int, 8>());
+  if (Hd <= 64) return f(std::integral_constant<int, 16>());
+  if (Hd <= 80) return f(std::integral_constant<int, 20>());
+  if (Hd <= 96) return f(std::integral_constant<int, 24>());
+  if (Hd <= 112) return f(std::integral_constant<int, 28>());
+  return f(std::integral_constant<int, 32>());
 }
 
 struct RnnPlan {
-  int64_t cap_row, values, offsets, keepbits, relubits, nnz_rows, h_last, dh_last, logits, dlogits, part_whh,
-      part_vec, out_values, out_keepbits, out_offsets, out_nnz, scratch, scratch_bytes, total;
+  int64_t cap_row, values, offsets, keepbits, relubits, nnz_rows, h_last, dh_last, logits, dlogits, part,
+      out_values, out_keepbits, out_offsets, out_nnz, scratch, scratch_bytes, total;
   rad_store_sizes out_sizes;
 };
 
@@ -322,8 +433,7 @@ int make_rnn_plan(const rad_irnn_desc* d, RnnPlan* pl) {
   pl->dh_last = take(d->B * d->Hd * 4);
   pl->logits = take(d->B * d->C * 4);
   pl->dlogits = take(d->B * d->C * 4);
-  pl->part_whh = take(d->B * d->Hd * d->Hd * 4);
-  pl->part_vec = take(d->B * 2 * d->Hd * 4);
+  pl->part = take(d->B * (d->Hd * d->Hd + 2 * d->Hd) * 4);
   int rc = rad_store_size_query(d->variant, RAD_F32, d->B, d->Hd, d->p, &pl->out_sizes);
   if (rc != RAD_OK) return rc;
   const rad_store_sizes& sz = pl->out_sizes;
@@ -381,7 +491,7 @@ extern "C" int rad_irnn_step(const rad_irnn_desc* d, const float* x, const int32
   char* ws = static_cast<char*>(workspace);
   const uint32_t Tk = keep_threshold_host(d->p);
   RnnParams p = {};
-  p.B = d->B; p.T = d->T; p.Hd = (int32_t)d->Hd; p.w32 = (int32_t)ceil_div(d->Hd, 32); p.ngroups = (int32_t)ceil_div(d->Hd, 8);
+  p.B = d->B; p.T = d->T; p.Hd = (int32_t)d->Hd; p.w32 = (int32_t)ceil_div(d->Hd, 32);
   p.same = d->variant == RAD_SAME_SAMPLE ? 1 : 0;
   p.keepT = make_keep_threshold(Tk); p.scale = (float)kLaneRange / (float)Tk;
   p.c2 = counter_word2(0, d->variant); p.step0 = d->step0;
@@ -393,20 +503,16 @@ extern "C" int rad_irnn_step(const rad_irnn_desc* d, const float* x, const int32
   p.relubits = reinterpret_cast<uint32_t*>(ws + pl.relubits);
   p.nnz_rows = reinterpret_cast<int64_t*>(ws + pl.nnz_rows);
   p.dh_last = reinterpret_cast<float*>(ws + pl.dh_last);
-  p.part_whh = reinterpret_cast<float*>(ws + pl.part_whh);
-  p.part_vec = reinterpret_cast<float*>(ws + pl.part_vec);
+  p.part = reinterpret_cast<float*>(ws + pl.part);
   p.dev_status = dev_status;
   const PhiloxKeys ks = philox_expand_key(d->seed);
   const size_t smem_f = (size_t)d->T * 4;
   const int64_t w32s = ceil_div(d->Hd, 32);
-  const size_t smem_b = (size_t)((d->T + 3) & ~(int64_t)3) * 4 + (size_t)((d->Hd * (d->Hd + 1) + 3) & ~3) * 4 +
+  const size_t smem_b = (size_t)((d->T + 3) & ~(int64_t)3) * 4 + (size_t)d->Hd * (size_t)((d->Hd + 3) & ~(int64_t)3) * 4 +
                         (size_t)d->T * (2 * w32s + 1) * 4;
   if (smem_f > 200 * 1024 || smem_b > 200 * 1024) return RAD_ELIMIT;
-  RAD_CUDA_TRY(cudaFuncSetAttribute(irnn_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem_f, 1024)));
-  RAD_CUDA_TRY(cudaFuncSetAttribute(irnn_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b));
-  count_launch();
-  irnn_forward_kernel<<<(unsigned)d->B, kRnnFwdThreads, smem_f, s>>>(p, ks);
-  RAD_CUDA_TRY(cudaGetLastError());
+  rc = with_parts(p.Hd, [&](auto kp) { return launch_irnn_forward<decltype(kp)::value>(p, ks, smem_f, s); });
+  if (rc != RAD_OK) return rc;
 
   // output layer on the last hidden state: sampled like any other layer input (layer index 1)
   rad_store st = {};
@@ -435,16 +541,11 @@ extern "C" int rad_irnn_step(const rad_irnn_desc* d, const float* x, const int32
                              ws + pl.dh_last, d->Hd, db_out, ws + pl.scratch, pl.scratch_bytes, dev_status, stream);
   if (rc != RAD_OK) return rc;
 
-  count_launch(5);
-  irnn_backward_kernel<<<(unsigned)d->B, kRnnThreads, smem_b, s>>>(p);
+  rc = with_parts(p.Hd, [&](auto kp) { return launch_irnn_backward<decltype(kp)::value>(p, smem_b, s); });
+  if (rc != RAD_OK) return rc;
   const int64_t hh = d->Hd * d->Hd;
-  sum_rows_kernel<<<(unsigned)ceil_div(hh, 256), 256, 0, s>>>(p.part_whh, d->B, hh, hh, 0, dW_hh);
-  sum_rows_kernel<<<(unsigned)ceil_div(d->Hd, 256), 256, 0, s>>>(p.part_vec, d->B, d->Hd, 2 * d->Hd, 0, dW_ih);
-  sum_rows_kernel<<<(unsigned)ceil_div(d->Hd, 256), 256, 0, s>>>(p.part_vec, d->B, d->Hd, 2 * d->Hd, d->Hd, db);
-  if (nnz_out != nullptr) {
-    sum_nnz_kernel<<<1, 32, 0, s>>>(p.nnz_rows, d->B, nnz_out);
-    RAD_CUDA_TRY(cudaMemcpyAsync(nnz_out + 1, st.nnz, 8, cudaMemcpyDeviceToDevice, s));
-  }
+  count_launch();
+  irnn_sum_rows_kernel<<<(unsigned)ceil_div(hh + 2 * d->Hd, 32), 1024, 0, s>>>(p.part, d->B, hh, d->Hd, dW_hh, dW_ih, db, p.nnz_rows, st.nnz, nnz_out);
   RAD_CUDA_TRY(cudaGetLastError());
   return RAD_OK;
 }

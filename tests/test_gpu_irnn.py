@@ -52,3 +52,26 @@ def test_irnn_stored_bytes():
     assert 4.5 < s.full_backprop_bytes / held < 8.0
     # without the keep bits and offsets, which the paper's count leaves out, the saving is near its 7.15x
     assert 6.0 < s.full_backprop_bytes / (held - s.index_bytes) < 7.2
+
+
+@pytest.mark.parametrize("B,T,Hd,C", [(1, 1, 1, 2), (3, 4, 8, 3), (2, 5, 33, 4), (151, 9, 63, 3), (2, 17, 81, 10), (3, 8, 97, 2),
+                                      (2, 33, 113, 5), (2, 12, 128, 3)])
+@pytest.mark.parametrize("p", [0.05, 0.6])
+def test_irnn_step_over_hidden_sizes_and_groups_of_steps(B, T, Hd, C, p):
+    """Hidden sizes on either side of every instantiation of the kernels, and numbers of steps that leave whole and partial
+    groups (of eight steps forward, four backward), against the oracle."""
+    import paper_2007_10412_b200 as rad
+    args = irnn_inputs(B, T, Hd, C, seed=B + T + Hd, identity=False)
+    ref = orc.irnn_step(*args, variant="different", p=p, seed=6, step0=77)
+    ctx = rad.IRNNStep(B, T, Hd, C, "different", p)
+    dev = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in args]
+    ctx(*dev, seed=6, step0=77)
+    torch.cuda.synchronize()
+    assert ctx.dev_status.item() == 0
+    nnz = ctx.nnz.cpu().numpy()
+    assert nnz[0] == ref.nnz_steps.sum() and nnz[1] == ref.nnz_out
+    assert abs(ctx.loss.item() - ref.loss) <= 1e-5 * abs(ref.loss)
+    for name, got, want in (("dW_hh", ctx.dW_hh, ref.dW_hh), ("dW_out", ctx.dW_out, ref.dW_out),
+                            ("dW_ih", ctx.dW_ih, ref.dW_ih), ("db", ctx.db, ref.db), ("db_out", ctx.db_out, ref.db_out)):
+        want = np.asarray(want)
+        assert np.abs(got.double().cpu().numpy() - want).max() <= 1e-5 * max(np.abs(want).max(), 1e-30), name
