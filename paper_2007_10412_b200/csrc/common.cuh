@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <utility>
 
 #include "../../include/rad.h"
 
@@ -339,19 +340,35 @@ __device__ __forceinline__ void st_cluster_f32(float* smem, uint32_t rank, float
   asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, %1;\n\tst.shared::cluster.f32 [a], %2;\n\t}"
                ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "r"(rank), "f"(v) : "memory");
 }
-template <typename K, typename... Args>
-int launch_with_cluster(K kernel, dim3 grid, int threads, size_t smem, dim3 cluster, cudaStream_t s, Args... args) {
+// ---- launches ------------------------------------------------------------------------------------
+// Every kernel may be launched while the one before it in the stream still runs (programmatic stream serialization): its
+// CTAs come up as SMs fall free and wait here until that one has ended and its writes are visible, so what is
+// saved is the gap between two launches (MNIST-shaped step of ten launches: see DESIGN).  Nothing that another kernel could
+// have written, or could still read, is touched before; the next launch is let in after the wait, one ahead at most.
+__device__ __forceinline__ void begin_after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... Args>
+int launch_with_cluster(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, dim3 cluster, cudaStream_t s, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3((unsigned)threads);
+  cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = cluster.x; attr.val.clusterDim.y = cluster.y; attr.val.clusterDim.z = cluster.z;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster.x; attr[1].val.clusterDim.y = cluster.y; attr[1].val.clusterDim.z = cluster.z;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster.x == 0 ? 1 : 2;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...) == cudaSuccess ? RAD_OK : RAD_ECUDA;
+}
+// without a cluster, or with the one the kernel is compiled for
+template <typename... P, typename... Args>
+int launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
+  return launch_with_cluster(kernel, grid, block, smem, dim3(0, 1, 1), s, std::forward<Args>(args)...);
 }
 
 // Lets `kernel` take `bytes` of dynamic shared memory on the current device, once per device (`ready`: its bits).

@@ -40,6 +40,7 @@ constexpr int kConvCo = 8;
 template <typename T, int kCin>
 __global__ void __launch_bounds__(256) conv_forward_pool_kernel(const ConvShape s, const T* X, const T* Wt,
                                                                 const float* bias, T* P, uint32_t* relubits) {
+  begin_after_previous();
   extern __shared__ __align__(16) float s_w[];       // 9 * Cin x Cout
   const int Cin = kCin > 0 ? kCin : s.Cin, nw = 9 * Cin * s.Cout;
   for (int i = threadIdx.x; i < nw; i += 256) s_w[i] = to_float(Wt[i]);
@@ -126,6 +127,7 @@ __global__ void __launch_bounds__(256) conv_forward_pool_kernel(const ConvShape 
 // pixels of 16-byte writes.  Bound by memory: 4096 x 16 x 16 x 32 bf16 16 us, 69 with one channel per thread.
 template <typename T>
 __global__ void __launch_bounds__(256) conv_dz_kernel(const ConvShape s, const T* dP, const uint32_t* relubits, T* dZ) {
+  begin_after_previous();
   const int Hp = s.H / 2, Wp = s.W / 2, groups = s.Cout / 8;
   const int64_t total = s.B * Hp * Wp * groups;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -159,6 +161,7 @@ __global__ void __launch_bounds__(256) conv_dz_kernel(const ConvShape s, const T
 
 template <typename T>
 __global__ void __launch_bounds__(256) conv_input_grad_kernel(const ConvShape s, const T* dZ, const T* Wt, T* dX) {
+  begin_after_previous();
   extern __shared__ float s_w[];                     // 9 * Cin rows of Cout + 1 floats (odd stride)
   const int stride = s.Cout + 1;
   for (int i = threadIdx.x; i < 9 * s.Cin * s.Cout; i += blockDim.x)
@@ -200,6 +203,7 @@ struct ConvDwParams {
 // One CTA per minibatch row b; blockDim = 9 * Cout threads (tap, co).
 template <typename T>
 __global__ void conv_weight_grad_kernel(const ConvDwParams p) {
+  begin_after_previous();
   extern __shared__ float sm[];
   const ConvShape& s = p.s;
   const int ncell = 9 * s.Cin * s.Cout;
@@ -318,6 +322,7 @@ inline size_t conv_first_smem(int H, int W, int Cout, int es, int64_t D) {
 
 template <typename T, int kCin>
 __global__ void __launch_bounds__(kFirstThreads) conv_first_backward_kernel(const ConvFirstParams p) {
+  begin_after_previous();
   extern __shared__ __align__(16) uint8_t cf_raw[];
   const ConvShape& s = p.s;
   const int Wq = s.W + 2, Cout = s.Cout, image = (s.H + 2) * Wq * Cout;
@@ -487,6 +492,7 @@ __global__ void __launch_bounds__(kFirstThreads) conv_first_backward_kernel(cons
 // out1[i] (i < n1) and out2[i - n1] (i < n) = sum over rows of part[row][i]: 32 columns and 32 row lanes per CTA, the
 // lanes' sums added in order (one thread per column took 293 us for 4096 rows of 432)
 __global__ void __launch_bounds__(1024) conv_sum_rows_kernel(const float* part, int64_t rows, int64_t n, int64_t n1, float* out1, float* out2) {
+  begin_after_previous();
   __shared__ float s[32][33];
   const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
   const int64_t i = (int64_t)blockIdx.x * 32 + lane;
@@ -513,7 +519,7 @@ int launch_forward_pool(const ConvShape& s, int64_t total, const void* X, const 
   const size_t smem = (size_t)9 * s.Cin * s.Cout * 4;
   count_launch();
   RAD_CUDA_TRY(cudaFuncSetAttribute(conv_forward_pool_kernel<T, kCin>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  conv_forward_pool_kernel<T, kCin><<<(unsigned)ceil_div(total, 256), 256, smem, st>>>(s, static_cast<const T*>(X), static_cast<const T*>(Wt),
+  launch_kernel(conv_forward_pool_kernel<T, kCin>, (unsigned)ceil_div(total, 256), 256, smem, st, s, static_cast<const T*>(X), static_cast<const T*>(Wt),
                                                                                        bias, static_cast<T*>(P), relubits);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
@@ -537,9 +543,9 @@ int conv_dz(int dtype, int64_t B, int H, int W, int Cout, const void* dP, const 
   const unsigned grid = (unsigned)ceil_div(B * (H / 2) * (W / 2) * (Cout / 8), 256);
   count_launch();
   if (dtype == RAD_BF16)
-    conv_dz_kernel<bf16><<<grid, 256, 0, st>>>(s, static_cast<const bf16*>(dP), relubits, static_cast<bf16*>(dZ));
+    launch_kernel(conv_dz_kernel<bf16>, grid, 256, 0, st, s, static_cast<const bf16*>(dP), relubits, static_cast<bf16*>(dZ));
   else
-    conv_dz_kernel<float><<<grid, 256, 0, st>>>(s, static_cast<const float*>(dP), relubits, static_cast<float*>(dZ));
+    launch_kernel(conv_dz_kernel<float>, grid, 256, 0, st, s, static_cast<const float*>(dP), relubits, static_cast<float*>(dZ));
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 
@@ -551,11 +557,11 @@ int conv_input_grad(int dtype, int64_t B, int H, int W, int Cin, int Cout, const
   count_launch();
   if (dtype == RAD_BF16) {
     RAD_CUDA_TRY(cudaFuncSetAttribute(conv_input_grad_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    conv_input_grad_kernel<bf16><<<grid, 256, smem, st>>>(s, static_cast<const bf16*>(dZ), static_cast<const bf16*>(Wt),
+    launch_kernel(conv_input_grad_kernel<bf16>, grid, 256, smem, st, s, static_cast<const bf16*>(dZ), static_cast<const bf16*>(Wt),
                                                          static_cast<bf16*>(dX));
   } else {
     RAD_CUDA_TRY(cudaFuncSetAttribute(conv_input_grad_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    conv_input_grad_kernel<float><<<grid, 256, smem, st>>>(s, static_cast<const float*>(dZ), static_cast<const float*>(Wt),
+    launch_kernel(conv_input_grad_kernel<float>, grid, 256, smem, st, s, static_cast<const float*>(dZ), static_cast<const float*>(Wt),
                                                           static_cast<float*>(dX));
   }
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
@@ -577,7 +583,7 @@ int launch_first_backward(const ConvFirstParams& p, unsigned grid, size_t smem, 
   static std::atomic<uint64_t> ready[5];
   auto launch = [&](auto kernel, std::atomic<uint64_t>& r) {
     if (!allow_smem(kernel, 160 * 1024, r)) return (int)RAD_ECUDA;
-    kernel<<<grid, kFirstThreads, smem, st>>>(p);
+    launch_kernel(kernel, grid, kFirstThreads, smem, st, p);
     return cudaGetLastError() == cudaSuccess ? (int)RAD_OK : (int)RAD_ECUDA;
   };
   switch (p.s.Cin) {
@@ -612,7 +618,7 @@ int conv_first_backward(const rad_store* store, int H, int W, int Cin, int Cout,
   const int rc = store->dtype == RAD_BF16 ? launch_first_backward<bf16>(p, (unsigned)grid, smem, st)
                                           : launch_first_backward<float>(p, (unsigned)grid, smem, st);
   if (rc != RAD_OK) return rc;
-  conv_sum_rows_kernel<<<(unsigned)ceil_div(ncell + Cout, 32), 1024, 0, st>>>(p.partial, grid, ncell + Cout, ncell, dW, db);
+  launch_kernel(conv_sum_rows_kernel, (unsigned)ceil_div(ncell + Cout, 32), 1024, 0, st, p.partial, grid, ncell + Cout, ncell, dW, db);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 
@@ -635,12 +641,12 @@ int conv_weight_grad(const rad_store* store, int H, int W, int Cin, int Cout, co
   count_launch(2);
   if (store->dtype == RAD_BF16) {
     RAD_CUDA_TRY(cudaFuncSetAttribute(conv_weight_grad_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    conv_weight_grad_kernel<bf16><<<(unsigned)store->B, threads, smem, st>>>(p);
+    launch_kernel(conv_weight_grad_kernel<bf16>, (unsigned)store->B, threads, smem, st, p);
   } else {
     RAD_CUDA_TRY(cudaFuncSetAttribute(conv_weight_grad_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    conv_weight_grad_kernel<float><<<(unsigned)store->B, threads, smem, st>>>(p);
+    launch_kernel(conv_weight_grad_kernel<float>, (unsigned)store->B, threads, smem, st, p);
   }
-  conv_sum_rows_kernel<<<(unsigned)ceil_div(ncell, 32), 1024, 0, st>>>(p.partial, store->B, ncell, ncell, dW, nullptr);
+  launch_kernel(conv_sum_rows_kernel, (unsigned)ceil_div(ncell, 32), 1024, 0, st, p.partial, store->B, ncell, ncell, dW, nullptr);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 

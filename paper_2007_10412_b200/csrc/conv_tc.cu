@@ -136,6 +136,7 @@ __device__ __forceinline__ uint4 cv_load_pixel(const bf16* T, bool in, int y, in
 enum { kCvFwd = 0, kCvDw = 1, kCvDx = 2 };
 template <int kMode>
 __global__ void __launch_bounds__(kCvThreads, 3) conv_tc_kernel(const ConvTcParams p) {
+  begin_after_previous();
   constexpr bool kDw = kMode == kCvDw, kDx = kMode == kCvDx;
   extern __shared__ uint8_t cv_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(cv_raw) + 1023) & ~(uintptr_t)1023);
@@ -373,6 +374,7 @@ __global__ void __launch_bounds__(kCvThreads, 3) conv_tc_kernel(const ConvTcPara
 // are dropped in place.  different-sample: a thread per keep-bit word; same-sample: a thread per kept entry.
 __global__ void __launch_bounds__(256) densify_different_kernel(const bf16* values, const uint32_t* keepbits, const uint32_t* offsets,
                                                                 int64_t B, int64_t D, int32_t ncb, int64_t capacity, bf16* out) {
+  begin_after_previous();
   const int64_t nwords = ((B + kTileRows - 1) / kTileRows) * ncb * kBitWords;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nwords; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t tile = i / kBitWords;
@@ -393,6 +395,7 @@ __global__ void __launch_bounds__(256) densify_different_kernel(const bf16* valu
 }
 __global__ void __launch_bounds__(256) densify_same_kernel(const bf16* values, const uint32_t* idx, const int64_t* nnz, int64_t B,
                                                            int64_t D, int64_t ld, bf16* out) {
+  begin_after_previous();
   const int64_t k = min(nnz[0], ld);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < B * k; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t b = i / k, j = i - b * k;
@@ -423,7 +426,7 @@ int conv_tc_forward_pool(int64_t B, int H, int W, int Cin, int Cout, const void*
   RAD_CUDA_TRY(cudaFuncSetAttribute(conv_tc_kernel<kCvFwd>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCvSmem));
   const int64_t windows = B * (H / 2) * (W / 2);
   count_launch();
-  conv_tc_kernel<kCvFwd><<<(unsigned)ceil_div(windows, 32), kCvThreads, kCvSmem, st>>>(p);
+  launch_kernel(conv_tc_kernel<kCvFwd>, (unsigned)ceil_div(windows, 32), kCvThreads, kCvSmem, st, p);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 
@@ -444,7 +447,7 @@ int conv_tc_input_grad(int64_t B, int H, int W, int Cin, int Cout, const void* d
   p.dev_status = dev_status; p.wait_limit_ns = wait_limit_ns();
   RAD_CUDA_TRY(cudaFuncSetAttribute(conv_tc_kernel<kCvDx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCvSmem));
   count_launch();
-  conv_tc_kernel<kCvDx><<<(unsigned)ceil_div(B * H * W, kCvM), kCvThreads, kCvSmem, st>>>(p);
+  launch_kernel(conv_tc_kernel<kCvDx>, (unsigned)ceil_div(B * H * W, kCvM), kCvThreads, kCvSmem, st, p);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 
@@ -473,13 +476,11 @@ int conv_tc_weight_grad(const rad_store* store, int H, int W, int Cin, int Cout,
   RAD_CUDA_TRY(cudaMemsetAsync(dense, 0, (size_t)(B * D * 2), st));
   count_launch();
   if (store->variant == RAD_SAME_SAMPLE) {
-    densify_same_kernel<<<(unsigned)std::min<int64_t>(ceil_div(B * store->values_ld, 256), 148 * 16), 256, 0, st>>>(
-        static_cast<const bf16*>(store->values), store->offsets, store->nnz, B, D, store->values_ld, dense);
+    launch_kernel(densify_same_kernel, (unsigned)std::min<int64_t>(ceil_div(B * store->values_ld, 256), 148 * 16), 256, 0, st, static_cast<const bf16*>(store->values), store->offsets, store->nnz, B, D, store->values_ld, dense);
   } else {
     const int32_t ncb = (int32_t)ceil_div(D, kTileCols);
     const int64_t nwords = ceil_div(B, kTileRows) * ncb * kBitWords;
-    densify_different_kernel<<<(unsigned)std::min<int64_t>(ceil_div(nwords, 256), 148 * 16), 256, 0, st>>>(
-        static_cast<const bf16*>(store->values), store->keepbits, store->offsets, B, D, ncb, store->values_capacity, dense);
+    launch_kernel(densify_different_kernel, (unsigned)std::min<int64_t>(ceil_div(nwords, 256), 148 * 16), 256, 0, st, static_cast<const bf16*>(store->values), store->keepbits, store->offsets, B, D, ncb, store->values_capacity, dense);
   }
   ConvTcParams p = {};
   p.B = B; p.H = H; p.W = W; p.Cin = Cin; p.Cout = Cout;
@@ -488,7 +489,7 @@ int conv_tc_weight_grad(const rad_store* store, int H, int W, int Cin, int Cout,
   const int splits = conv_tc_splits(B * H * W, Cin, &p.kblocks_per_split);
   RAD_CUDA_TRY(cudaFuncSetAttribute(conv_tc_kernel<kCvDw>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCvSmem));
   count_launch();
-  conv_tc_kernel<kCvDw><<<dim3((unsigned)ceil_div(9 * Cin, kCvM), (unsigned)splits), kCvThreads, kCvSmem, st>>>(p);
+  launch_kernel(conv_tc_kernel<kCvDw>, dim3((unsigned)ceil_div(9 * Cin, kCvM), (unsigned)splits), kCvThreads, kCvSmem, st, p);
   RAD_CUDA_TRY(cudaGetLastError());
   // the splits' partial sums: column sums of a splits x (9 Cin Cout) matrix, in a fixed order
   const int64_t n = (int64_t)9 * Cin * Cout, held = round_up((int64_t)splits * n * 4, 256);

@@ -89,6 +89,7 @@ struct UnitDot {
 
 template <int KP>
 __global__ void __launch_bounds__(32 * (KP / 2 + kStoreWarps), 2) irnn_forward_kernel(const RnnParams p, const PhiloxKeys ks, int unit_warps) {
+  begin_after_previous();
   extern __shared__ float sm[];
   float* s_x = sm;                                   // T inputs of this row
   constexpr int kGroup = kFwdGroup, kRing = 4 * kGroup;                  // states: two groups of steps and what the store warps still read
@@ -205,6 +206,7 @@ __global__ void __launch_bounds__(32 * (KP / 2 + kStoreWarps), 2) irnn_forward_k
 
 template <int KP>
 __global__ void __launch_bounds__(32 * (KP / 2 + kListWarps), 2) irnn_backward_kernel(const RnnParams p, int unit_warps) {
+  begin_after_previous();
   extern __shared__ __align__(16) float sm[];
   constexpr int kGroup = kBwdGroup;
   const int Hd = p.Hd;
@@ -354,6 +356,7 @@ __global__ void __launch_bounds__(32 * (KP / 2 + kListWarps), 2) irnn_backward_k
 // four of 7 to 15 us.
 __global__ void __launch_bounds__(1024) irnn_sum_rows_kernel(const float* part, int64_t B, int64_t n1, int64_t Hd, float* dW_hh, float* dW_ih,
                                                              float* db, const int64_t* nnz_rows, const int64_t* nnz_last, int64_t* nnz_out) {
+  begin_after_previous();
   __shared__ float s[32][33];
   const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
   const int64_t i = (int64_t)blockIdx.x * 32 + lane, n = n1 + 2 * Hd;
@@ -384,7 +387,7 @@ int launch_irnn_forward(const RnnParams& p, const PhiloxKeys& ks, size_t smem, c
   const int uw = (int)ceil_div(p.Hd, 8);
   RAD_CUDA_TRY(cudaFuncSetAttribute(irnn_forward_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem, 1024)));
   count_launch();
-  irnn_forward_kernel<KP><<<(unsigned)p.B, 32 * (uw + kStoreWarps), smem, s>>>(p, ks, uw);
+  launch_kernel(irnn_forward_kernel<KP>, (unsigned)p.B, 32 * (uw + kStoreWarps), smem, s, p, ks, uw);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 template <int KP>
@@ -392,7 +395,7 @@ int launch_irnn_backward(const RnnParams& p, size_t smem, cudaStream_t s) {
   const int uw = (int)ceil_div(p.Hd, 8);
   RAD_CUDA_TRY(cudaFuncSetAttribute(irnn_backward_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   count_launch();
-  irnn_backward_kernel<KP><<<(unsigned)p.B, 32 * (uw + kListWarps), smem, s>>>(p, uw);
+  launch_kernel(irnn_backward_kernel<KP>, (unsigned)p.B, 32 * (uw + kListWarps), smem, s, p, uw);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 // f(std::integral_constant<KP>) for the smallest KP in 8, 16, 20, 24, 28, 32 that holds Hd units
@@ -545,7 +548,7 @@ extern "C" int rad_irnn_step(const rad_irnn_desc* d, const float* x, const int32
   if (rc != RAD_OK) return rc;
   const int64_t hh = d->Hd * d->Hd;
   count_launch();
-  irnn_sum_rows_kernel<<<(unsigned)ceil_div(hh + 2 * d->Hd, 32), 1024, 0, s>>>(p.part, d->B, hh, d->Hd, dW_hh, dW_ih, db, p.nnz_rows, st.nnz, nnz_out);
+  launch_kernel(irnn_sum_rows_kernel, (unsigned)ceil_div(hh + 2 * d->Hd, 32), 1024, 0, s, p.part, d->B, hh, d->Hd, dW_hh, dW_ih, db, p.nnz_rows, st.nnz, nnz_out);
   RAD_CUDA_TRY(cudaGetLastError());
   return RAD_OK;
 }

@@ -55,6 +55,7 @@ template <typename T, int NV>
 __global__ void __launch_bounds__(256) xent_rows_kernel(const float* logits, int64_t ldl, const int32_t* labels,
                                                         int64_t B, int64_t C, T* dZ, int64_t ldz,
                                                         float* row_loss) {
+  begin_after_previous();
   const int lane = threadIdx.x & 31;
   const int64_t b = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (b >= B) return;
@@ -72,6 +73,7 @@ constexpr int kXentCluster = 8;            // portable cluster size
 template <typename T, int NV>
 __global__ void __launch_bounds__(1024) xent_small_kernel(const float* logits, int64_t ldl, const int32_t* labels, int64_t B,
                                                           int64_t C, T* dZ, int64_t ldz, float* loss) {
+  begin_after_previous();
   __shared__ float s_row[kXentSmallRows];
   __shared__ float s[1024];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -100,6 +102,7 @@ __global__ void __launch_bounds__(1024) xent_small_kernel(const float* logits, i
 
 // Fixed-order mean of the per-row losses (one CTA).
 __global__ void __launch_bounds__(1024) mean_kernel(const float* row_loss, int64_t B, float* loss) {
+  begin_after_previous();
   __shared__ float s[1024];
   float acc = 0.0f;
   for (int64_t i = threadIdx.x; i < B; i += 1024) acc += row_loss[i];
@@ -121,8 +124,8 @@ int launch_xent(const float* logits, int64_t ldl, const int32_t* labels, int64_t
     return launch_with_cluster(xent_small_kernel<T, NV>, dim3(ctas), 1024, 0, dim3(ctas), s, logits, ldl, labels, B, C, dZ, ldz, loss);
   }
   count_launch(2);
-  xent_rows_kernel<T, NV><<<(unsigned)ceil_div(B, 8), 256, 0, s>>>(logits, ldl, labels, B, C, dZ, ldz, rows);
-  mean_kernel<<<1, 1024, 0, s>>>(rows, B, loss);
+  launch_kernel(xent_rows_kernel<T, NV>, (unsigned)ceil_div(B, 8), 256, 0, s, logits, ldl, labels, B, C, dZ, ldz, rows);
+  launch_kernel(mean_kernel, 1, 1024, 0, s, rows, B, loss);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 template <typename T>

@@ -23,6 +23,7 @@ struct SignParams {
 // output for counter (j / 128, d, c2, c3); set means -1.  Columns k .. ld-1 are zero.
 template <typename T>
 __global__ void __launch_bounds__(256) rademacher_kernel(const SignParams p, const PhiloxKeys ks) {
+  begin_after_previous();
   const int64_t groups = p.ld / 32 + (p.ld % 32 != 0 ? 1 : 0);
   const int64_t n = p.D * groups;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -41,12 +42,14 @@ __global__ void __launch_bounds__(256) rademacher_kernel(const SignParams p, con
 
 template <typename T>
 __global__ void __launch_bounds__(256) scale_convert_kernel(const float* in, T* out, int64_t n, float scale) {
+  begin_after_previous();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     out[i] = from_float<T>(__fmul_rn(in[i], scale));
 }
 
 // idx: the identity list of ld columns; bits: bit j set for j < k (the columns of S that hold data)
 __global__ void project_meta_kernel(uint32_t* idx, uint32_t* bits, int64_t ld, int64_t* nnz, int64_t k, int64_t B) {
+  begin_after_previous();
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < ld; j += (int64_t)gridDim.x * blockDim.x) {
     if (idx != nullptr) idx[j] = (uint32_t)j;
     if (bits != nullptr && (j & 31) == 0) {
@@ -69,9 +72,9 @@ int draw_signs(int dtype, void* out, int64_t D, int64_t k, int64_t ld, uint64_t 
   const int grid = (int)std::min<int64_t>(ceil_div(n, 256), 148 * 16);
   count_launch();
   if (dtype == RAD_BF16)
-    rademacher_kernel<bf16><<<grid, 256, 0, s>>>(p, ks);
+    launch_kernel(rademacher_kernel<bf16>, grid, 256, 0, s, p, ks);
   else
-    rademacher_kernel<float><<<grid, 256, 0, s>>>(p, ks);
+    launch_kernel(rademacher_kernel<float>, grid, 256, 0, s, p, ks);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 
@@ -112,7 +115,7 @@ int project_forward_store(const void* A, int64_t lda, const rad_store* st, void*
   int rc = draw_signs(st->dtype, workspace, st->D, k, ld, st->seed, st->layer, st->step, s);
   if (rc != RAD_OK) return rc;
   count_launch();
-  project_meta_kernel<<<1, 32, 0, s>>>(nullptr, nullptr, 0, st->nnz, k, st->B);
+  launch_kernel(project_meta_kernel, 1, 32, 0, s, nullptr, nullptr, 0, st->nnz, k, st->B);
   // S = A R': B x D times D x ld, stored in the working type
   rc = rad_linear_forward(st->dtype, RAD_ACT_NONE, st->B, st->D, ld, A, lda, workspace, ld, nullptr, st->values, ld,
                           nullptr, 0, nullptr, 0, nullptr, dev_status, stream);
@@ -137,7 +140,7 @@ int project_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_
   int rc = draw_signs(st->dtype, R, st->D, k, ld, st->seed, st->layer, st->step, s);
   if (rc != RAD_OK) return rc;
   count_launch();
-  project_meta_kernel<<<(unsigned)std::min<int64_t>(ceil_div(ld, 256), 1024), 256, 0, s>>>(idx, bits, ld, nullptr, k, 0);
+  launch_kernel(project_meta_kernel, (unsigned)std::min<int64_t>(ceil_div(ld, 256), 1024), 256, 0, s, idx, bits, ld, nullptr, k, 0);
   // G32 = S^T dZ (ld x H): the dense block of S goes through the same-sample contraction with every column kept
   const rad_store t = as_dense_block(st, idx, bits);
   rc = rad_linear_weight_grad(&t, dZ, ldz, H, G32, H, ws, inner, dev_status, stream);
@@ -147,9 +150,9 @@ int project_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_
   const int grid = (int)std::min<int64_t>(ceil_div(n, 256), 148 * 16);
   count_launch();
   if (st->dtype == RAD_BF16)
-    scale_convert_kernel<bf16><<<grid, 256, 0, s>>>(G32, static_cast<bf16*>(G), n, 1.0f / (float)k);
+    launch_kernel(scale_convert_kernel<bf16>, grid, 256, 0, s, G32, static_cast<bf16*>(G), n, 1.0f / (float)k);
   else
-    scale_convert_kernel<float><<<grid, 256, 0, s>>>(G32, static_cast<float*>(G), n, 1.0f / (float)k);
+    launch_kernel(scale_convert_kernel<float>, grid, 256, 0, s, G32, static_cast<float*>(G), n, 1.0f / (float)k);
   if (cudaGetLastError() != cudaSuccess) return RAD_ECUDA;
   // dW_hat = R' G: D x ld times ld x H, float32 out
   return rad_linear_forward(st->dtype, RAD_ACT_NONE, st->D, ld, H, R, ld, G, H, nullptr, nullptr, 0, dW, ldw, nullptr, 0,

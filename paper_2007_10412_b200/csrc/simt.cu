@@ -429,6 +429,7 @@ __device__ __forceinline__ void gemm_unit_finish(const GemmParams& p, int64_t un
 
 template <typename T, int EPI>
 __global__ void __launch_bounds__(256, 2) gemm_kernel(const GemmParams p) {
+  begin_after_previous();
   extern __shared__ __align__(16) float smem[];
   gemm_unit_partial<T, EPI>(p, blockIdx.x, smem);
   share_barrier();
@@ -461,6 +462,7 @@ int launch_gemm(int dtype, const GemmParams& p0, int64_t Mgrid, cudaStream_t s) 
 template <typename T>
 __global__ void __launch_bounds__(256) relu_bits_rows_kernel(const T* X, int64_t ld, int64_t B, int64_t H,
                                                              int64_t w32, uint32_t* out) {
+  begin_after_previous();
   const int64_t n = B * w32;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -479,6 +481,7 @@ __global__ void __launch_bounds__(256) relu_bits_rows_kernel(const T* X, int64_t
 // their launch count).  `dw_blocks` is a multiple of the cluster size.
 template <typename T>
 __global__ void __launch_bounds__(256, 2) dw_dx_kernel(const GemmParams w, const GemmParams g, int dw_blocks) {
+  begin_after_previous();
   extern __shared__ __align__(16) float smem[];
   const int b = (int)blockIdx.x, gu = b - dw_blocks;
   if (b < dw_blocks) gemm_unit_partial<T, kEpiSparse>(w, b, smem);
@@ -490,6 +493,7 @@ __global__ void __launch_bounds__(256, 2) dw_dx_kernel(const GemmParams w, const
 }
 
 __global__ void zero_rows_kernel(float* dW, int64_t ldw, int64_t D, int64_t H) {
+  begin_after_previous();
   const int64_t n = D * H;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
@@ -531,6 +535,7 @@ __device__ __forceinline__ void colsum_load(const T* p, float (&v)[V]) {
 template <typename T, int V>
 __global__ void __launch_bounds__(256) colsum_kernel(const T* dZ, int64_t ldz, int64_t B, int64_t H, int log_cl,
                                                      int64_t rows_per_cta, float* out) {
+  begin_after_previous();
   __shared__ float s_warp[8][32 * V];
   __shared__ float s_cta[32 * V];
   const int CL = 1 << log_cl, RL = 256 >> log_cl, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -619,6 +624,7 @@ int column_sums_of(const T* dZ, int64_t ldz, int64_t B, int64_t H, float* out, f
 template <typename T>
 __global__ void __launch_bounds__(256, 2) same_dw_dx_kernel(const GemmParams w, const GemmParams g, int dw_blocks, int dx_blocks,
                                                             const uint32_t* keep_cols, int64_t D, int64_t H) {
+  begin_after_previous();
   extern __shared__ __align__(16) float smem[];
   const int b = (int)blockIdx.x;
   if (b < dw_blocks) {
@@ -657,9 +663,9 @@ int simt_forward(int dtype, int act, int64_t B, int64_t D, int64_t H, const void
     const int g = (int)std::min<int64_t>(ceil_div(n, 256), 148 * 16);
     count_launch();
     if (dtype == RAD_BF16)
-      relu_bits_rows_kernel<bf16><<<g, 256, 0, s>>>(static_cast<const bf16*>(out_act), ld_act, B, H, w32, relubits);
+      launch_kernel(relu_bits_rows_kernel<bf16>, g, 256, 0, s, static_cast<const bf16*>(out_act), ld_act, B, H, w32, relubits);
     else
-      relu_bits_rows_kernel<float><<<g, 256, 0, s>>>(static_cast<const float*>(out_act), ld_act, B, H, w32, relubits);
+      launch_kernel(relu_bits_rows_kernel<float>, g, 256, 0, s, static_cast<const float*>(out_act), ld_act, B, H, w32, relubits);
     if (cudaGetLastError() != cudaSuccess) return RAD_ECUDA;
   }
   return RAD_OK;
@@ -726,7 +732,7 @@ int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H
     }
     const int g = (int)std::min<int64_t>(ceil_div(st->D * H, 256), 148 * 16);
     count_launch();
-    zero_rows_kernel<<<g, 256, 0, s>>>(dW, ldw, st->D, H);
+    launch_kernel(zero_rows_kernel, g, 256, 0, s, dW, ldw, st->D, H);
     return launch_gemm<kEpiScatterRows>(st->dtype, p, std::max<int64_t>(p.M, 1), s);
   }
   const bool low = st->dtype == RAD_BF16;

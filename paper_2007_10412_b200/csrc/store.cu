@@ -110,6 +110,7 @@ __device__ __forceinline__ uint32_t transpose4x4_bytes(uint32_t v, int k) {
 enum MaskSource { kMaskDraw = 0, kMaskCounts = 1, kMaskIndex = 2 };
 template <typename T, int kMask>
 __global__ void __launch_bounds__(256) store_different_kernel(const StoreParams p, const PhiloxKeys ks) {
+  begin_after_previous();
   constexpr bool kReplace = kMask == kMaskCounts;
   __shared__ uint32_t s_rowcnt[kTileRows];
   __shared__ uint32_t s_rowoff[kTileRows];
@@ -321,6 +322,7 @@ struct SameParams {
 
 // One CTA draws the D column decisions and writes the ascending kept-column list.
 __global__ void __launch_bounds__(1024) same_mask_kernel(const SameParams p, const PhiloxKeys ks) {
+  begin_after_previous();
   __shared__ uint32_t s_warp[32];
   __shared__ uint32_t s_running;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -373,6 +375,7 @@ __global__ void __launch_bounds__(1024) same_mask_kernel(const SameParams p, con
 // values[b, j] = A[b, idx[j]] * scale for j < k', zero up to ld.  One warp per row at a time.
 template <typename T>
 __global__ void __launch_bounds__(256) same_gather_kernel(const SameParams p, const float* colscale) {
+  begin_after_previous();
   const int64_t k = min(p.nnz[0], p.ld);
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -401,6 +404,7 @@ __global__ void __launch_bounds__(256) same_gather_kernel(const SameParams p, co
 // columns sit in shared memory as 16-bit numbers (D <= 65536).
 template <typename T>
 __global__ void __launch_bounds__(256) same_gather_rows_kernel(const SameParams p, uint32_t* relubits, int64_t w32, int warps) {
+  begin_after_previous();
   extern __shared__ __align__(16) unsigned char s_dyn[];
   constexpr int kPer = 16 / (int)sizeof(T);
   const int64_t k = min(p.nnz[0], p.ld);
@@ -453,6 +457,7 @@ __global__ void __launch_bounds__(256) same_gather_rows_kernel(const SameParams 
 template <typename T>
 __global__ void __launch_bounds__(256) relu_bits_kernel(const T* A, int64_t lda, int64_t B, int64_t D,
                                                         int64_t w32, uint32_t* out) {
+  begin_after_previous();
   const int64_t n = B * w32;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -477,6 +482,7 @@ struct ReplaceParams {
 // One CTA per row: the k draws of the row land in a shared-memory histogram (a byte per column, four to
 // a word), which is then written out as the row of the multiplicity matrix.
 __global__ void __launch_bounds__(128) replace_counts_kernel(const ReplaceParams p, const PhiloxKeys ks) {
+  begin_after_previous();
   extern __shared__ uint32_t s_hist[];
   const int64_t row = blockIdx.x;
   const int words = (int)(p.ldc / 4);
@@ -506,6 +512,7 @@ __global__ void __launch_bounds__(128) replace_counts_kernel(const ReplaceParams
 constexpr int kFixedRows = 64;
 __global__ void __launch_bounds__(128) fixed_counts_kernel(const ReplaceParams p, const PhiloxKeys ks, int rows_per_cta,
                                                            int words) {
+  begin_after_previous();
   extern __shared__ uint32_t s_bits[];            // rows_per_cta x words
   const int tid = threadIdx.x;
   for (int i = tid; i < rows_per_cta * words; i += 128) s_bits[i] = 0;
@@ -553,6 +560,7 @@ struct SameReplaceParams {
 // ascending list of the columns that were hit, their weights and the keep-bit words.
 __global__ void __launch_bounds__(1024) same_replace_mask_kernel(const SameParams p, const SameReplaceParams r,
                                                                  const PhiloxKeys ks) {
+  begin_after_previous();
   __shared__ uint32_t s_warp[32];
   __shared__ uint32_t s_running;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -652,9 +660,9 @@ int launch_store_fill(const StoreParams& p, const PhiloxKeys& ks, int dtype, dou
   }
   count_launch();
   if (dtype == RAD_BF16)
-    store_different_kernel<bf16, kMaskIndex><<<p.ntiles, 256, 0, s>>>(p, ks);
+    launch_kernel(store_different_kernel<bf16, kMaskIndex>, p.ntiles, 256, 0, s, p, ks);
   else
-    store_different_kernel<float, kMaskIndex><<<p.ntiles, 256, 0, s>>>(p, ks);
+    launch_kernel(store_different_kernel<float, kMaskIndex>, p.ntiles, 256, 0, s, p, ks);
   RAD_CUDA_TRY(cudaGetLastError());
   return RAD_OK;
 }
@@ -672,13 +680,13 @@ int launch_store_different(const StoreParams& p, const PhiloxKeys& ks, int dtype
   count_launch();
   if (p.counts != nullptr) {
     if (dtype == RAD_BF16)
-      store_different_kernel<bf16, kMaskCounts><<<p.ntiles, 256, 0, s>>>(p, ks);
+      launch_kernel(store_different_kernel<bf16, kMaskCounts>, p.ntiles, 256, 0, s, p, ks);
     else
-      store_different_kernel<float, kMaskCounts><<<p.ntiles, 256, 0, s>>>(p, ks);
+      launch_kernel(store_different_kernel<float, kMaskCounts>, p.ntiles, 256, 0, s, p, ks);
   } else if (dtype == RAD_BF16) {
-    store_different_kernel<bf16, kMaskDraw><<<p.ntiles, 256, 0, s>>>(p, ks);
+    launch_kernel(store_different_kernel<bf16, kMaskDraw>, p.ntiles, 256, 0, s, p, ks);
   } else {
-    store_different_kernel<float, kMaskDraw><<<p.ntiles, 256, 0, s>>>(p, ks);
+    launch_kernel(store_different_kernel<float, kMaskDraw>, p.ntiles, 256, 0, s, p, ks);
   }
   RAD_CUDA_TRY(cudaGetLastError());
   return RAD_OK;
@@ -713,9 +721,9 @@ int launch_relu_bits(int dtype, const void* A, int64_t lda, int64_t B, int64_t D
   const int g2 = (int)std::min<int64_t>(ceil_div(n, 256), 148 * 16);
   count_launch();
   if (dtype == RAD_BF16)
-    relu_bits_kernel<bf16><<<g2, 256, 0, s>>>(static_cast<const bf16*>(A), lda, B, D, w32, relubits);
+    launch_kernel(relu_bits_kernel<bf16>, g2, 256, 0, s, static_cast<const bf16*>(A), lda, B, D, w32, relubits);
   else
-    relu_bits_kernel<float><<<g2, 256, 0, s>>>(static_cast<const float*>(A), lda, B, D, w32, relubits);
+    launch_kernel(relu_bits_kernel<float>, g2, 256, 0, s, static_cast<const float*>(A), lda, B, D, w32, relubits);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 }  // namespace rad
@@ -932,12 +940,12 @@ extern "C" int rad_linear_forward_store(const void* A, int64_t lda, const rad_st
         if (smem > 48 * 1024)
           RAD_CUDA_TRY(cudaFuncSetAttribute(fixed_counts_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)kMaxCountsRowBytes));
-        fixed_counts_kernel<<<(unsigned)ceil_div(st->B, rows), 128, smem, s>>>(rp, ks, rows, words);
+        launch_kernel(fixed_counts_kernel, (unsigned)ceil_div(st->B, rows), 128, smem, s, rp, ks, rows, words);
       } else {
         if (rp.ldc > 48 * 1024)
           RAD_CUDA_TRY(cudaFuncSetAttribute(replace_counts_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)kMaxCountsRowBytes));
-        replace_counts_kernel<<<(unsigned)st->B, 128, (size_t)rp.ldc, s>>>(rp, ks);
+        launch_kernel(replace_counts_kernel, (unsigned)st->B, 128, (size_t)rp.ldc, s, rp, ks);
       }
       RAD_CUDA_TRY(cudaGetLastError());
       p.counts = rp.counts; p.ldc = rp.ldc;
@@ -963,9 +971,9 @@ extern "C" int rad_linear_forward_store(const void* A, int64_t lda, const rad_st
     r.hist = reinterpret_cast<uint32_t*>(static_cast<char*>(workspace) + 256);
     r.colscale = reinterpret_cast<float*>(static_cast<char*>(workspace) + 256 + 4 * st->D);
     colscale = r.colscale;
-    same_replace_mask_kernel<<<1, 1024, 0, s>>>(p, r, ks);
+    launch_kernel(same_replace_mask_kernel, 1, 1024, 0, s, p, r, ks);
   } else {
-    same_mask_kernel<<<1, 1024, 0, s>>>(p, ks);
+    launch_kernel(same_mask_kernel, 1, 1024, 0, s, p, ks);
   }
   // Dense masks (most 32-byte sectors of a row hold a kept column) and calls that also want the ReLU bits take
   // the row-staging kernel; sparse masks without ReLU bits keep the gather that skips the sectors it does not need.
@@ -987,10 +995,10 @@ extern "C" int rad_linear_forward_store(const void* A, int64_t lda, const rad_st
       const int grid_r = (int)std::min<int64_t>(ceil_div(st->B, warps), sms);
       if (st->dtype == RAD_BF16) {
         RAD_CUDA_TRY(cudaFuncSetAttribute(same_gather_rows_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_budget));
-        same_gather_rows_kernel<bf16><<<grid_r, 256, smem, s>>>(p, st->relubits, w32, warps);
+        launch_kernel(same_gather_rows_kernel<bf16>, grid_r, 256, smem, s, p, st->relubits, w32, warps);
       } else {
         RAD_CUDA_TRY(cudaFuncSetAttribute(same_gather_rows_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_budget));
-        same_gather_rows_kernel<float><<<grid_r, 256, smem, s>>>(p, st->relubits, w32, warps);
+        launch_kernel(same_gather_rows_kernel<float>, grid_r, 256, smem, s, p, st->relubits, w32, warps);
       }
       RAD_CUDA_TRY(cudaGetLastError());
       return RAD_OK;
@@ -998,17 +1006,17 @@ extern "C" int rad_linear_forward_store(const void* A, int64_t lda, const rad_st
   }
   const int grid = (int)std::min<int64_t>(ceil_div(st->B, 8), 148 * 8);
   if (st->dtype == RAD_BF16)
-    same_gather_kernel<bf16><<<grid, 256, 0, s>>>(p, colscale);
+    launch_kernel(same_gather_kernel<bf16>, grid, 256, 0, s, p, colscale);
   else
-    same_gather_kernel<float><<<grid, 256, 0, s>>>(p, colscale);
+    launch_kernel(same_gather_kernel<float>, grid, 256, 0, s, p, colscale);
   if (st->relubits != nullptr) {
     const int64_t n = st->B * w32;
     const int g2 = (int)std::min<int64_t>(ceil_div(n, 256), 148 * 16);
     count_launch();
     if (st->dtype == RAD_BF16)
-      relu_bits_kernel<bf16><<<g2, 256, 0, s>>>(static_cast<const bf16*>(A), lda, st->B, st->D, w32, st->relubits);
+      launch_kernel(relu_bits_kernel<bf16>, g2, 256, 0, s, static_cast<const bf16*>(A), lda, st->B, st->D, w32, st->relubits);
     else
-      relu_bits_kernel<float><<<g2, 256, 0, s>>>(static_cast<const float*>(A), lda, st->B, st->D, w32, st->relubits);
+      launch_kernel(relu_bits_kernel<float>, g2, 256, 0, s, static_cast<const float*>(A), lda, st->B, st->D, w32, st->relubits);
   }
   RAD_CUDA_TRY(cudaGetLastError());
   return RAD_OK;

@@ -34,6 +34,7 @@ struct IndexParams {
 // the eight turns, gives every row its offset in (row, column) order.
 constexpr int kIndexWarps = 4;
 __global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const IndexParams p, const PhiloxKeys ks) {
+  begin_after_previous();
   const int lane = threadIdx.x & 31;
   const uint32_t warp0 = blockIdx.x * kIndexWarps + (threadIdx.x >> 5), nwarps = gridDim.x * kIndexWarps;
   const uint32_t nrows = (uint32_t)p.B, ncols = (uint32_t)p.D, ncb = (uint32_t)p.ncb;
@@ -74,6 +75,7 @@ __global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const Ind
 // 16-byte aligned), adds them up locally, and one warp scan plus one pass over the warp sums places them.
 constexpr int kScanPer = 16;
 __global__ void __launch_bounds__(1024) offsets_scan_kernel(const IndexParams p, int vec) {
+  begin_after_previous();
   __shared__ uint64_t s_warp[32];                   // padded sum in the high half, exact sum in the low half
   __shared__ uint64_t s_carry;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -152,7 +154,7 @@ int launch_offsets_scan(uint32_t* offsets, int64_t ntiles, int64_t* nnz, int64_t
   IndexParams p = {};
   p.ntiles = (int32_t)ntiles; p.offsets = offsets; p.nnz = nnz; p.capacity = capacity; p.dev_status = dev_status;
   count_launch();
-  offsets_scan_kernel<<<1, 1024, 0, s>>>(p, ((uintptr_t)offsets & 15) == 0 ? 1 : 0);
+  launch_kernel(offsets_scan_kernel, 1, 1024, 0, s, p, ((uintptr_t)offsets & 15) == 0 ? 1 : 0);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 
@@ -172,7 +174,7 @@ int launch_store_index(const rad_store* st, bool check_capacity, int32_t* dev_st
   const int grid = (int)std::min<int64_t>(ceil_div(p.ntiles, kIndexWarps), 148 * 12);
   if (st->law == RAD_LAW_FIXED) return launch_fixed_index(st, check_capacity, dev_status, s);
   count_launch();
-  store_index_kernel<<<grid, 32 * kIndexWarps, 0, s>>>(p, ks);
+  launch_kernel(store_index_kernel, grid, 32 * kIndexWarps, 0, s, p, ks);
   if (cudaGetLastError() != cudaSuccess) return RAD_ECUDA;
   return launch_offsets_scan(p.offsets, p.ntiles, p.nnz, p.capacity, dev_status, s);
 }

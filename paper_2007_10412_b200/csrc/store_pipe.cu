@@ -182,6 +182,7 @@ __device__ __forceinline__ void copy_scaled(const T* wb, T* out, uint32_t first,
 template <typename T, int S, bool kFill>
 __global__ void __launch_bounds__(kPipeThreads, 2) store_pipelined_kernel(const StoreParams p, const PhiloxKeys ks,
                                                                       const __grid_constant__ CUtensorMap tmA) {
+  begin_after_previous();
   // A stage of the ring must always serve the same half of the compute warps: a waiter tells the phases of
   // a barrier apart by one parity bit, which only works if it has itself waited for the phase before.
   static_assert(S % kTilesPerStep == 0, "stages and tiles worked on side by side");
@@ -599,7 +600,7 @@ int launch_typed(const StoreParams& p, const PhiloxKeys& ks, const CUtensorMap& 
   const int64_t nchunks = ceil_div(p.ntiles, kChunk);
   const int grid = (int)std::min<int64_t>(nchunks, grid_cap[dev]);
   count_launch();
-  kernel<<<grid, kPipeThreads, smem, s>>>(p, ks, map);
+  launch_kernel(kernel, grid, kPipeThreads, smem, s, p, ks, map);
   RAD_CUDA_TRY(cudaGetLastError());
   return RAD_OK;
 }

@@ -109,6 +109,7 @@ constexpr int kRowsWarps = 8;
 
 template <typename T, bool kRowsOut>
 __global__ void __launch_bounds__(32 * kRowsWarps) rows_fixed_kernel(const RowsParams p, const PhiloxKeys ks) {
+  begin_after_previous();
   extern __shared__ __align__(16) uint32_t s_dyn[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // per warp: bitmap (words), draws (draws_stride), column list (k 16-bit numbers, kRowsOut only)
@@ -205,6 +206,7 @@ __global__ void __launch_bounds__(256) rows_to_tiles_kernel(const T* values, con
                                                             int64_t ld, int32_t ncb, const uint32_t* keepbits,
                                                             const uint32_t* offsets, T* out, int64_t capacity,
                                                             int32_t* dev_status) {
+  begin_after_previous();
   const int lane = threadIdx.x & 31;
   for (int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); row < B; row += (int64_t)gridDim.x * 8) {
     const int64_t slab = row >> 6;
@@ -242,6 +244,7 @@ __global__ void __launch_bounds__(256) rows_to_tiles_kernel(const T* values, con
 template <typename T>
 __global__ void __launch_bounds__(256) tile_padding_kernel(const uint32_t* keepbits, const uint32_t* offsets, int64_t ntiles,
                                                            T* out, int64_t capacity) {
+  begin_after_previous();
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t* tw = keepbits + t * kTileWords;
     const uint4 q = *reinterpret_cast<const uint4*>(tw + 63 * 4);
@@ -257,6 +260,7 @@ __global__ void __launch_bounds__(256) tile_padding_kernel(const uint32_t* keepb
 // extras: `extras_ld` words per row: word 0 = entries that follow, each (column | count << 16), count >= 2.
 __global__ void __launch_bounds__(32 * kRowsWarps) replace_index_kernel(const RowsParams p, const PhiloxKeys ks, uint32_t* extras,
                                                                         int32_t extras_ld) {
+  begin_after_previous();
   extern __shared__ __align__(16) uint32_t s_dyn[];
   __shared__ uint32_t s_nrep[kRowsWarps], s_nex[kRowsWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -337,6 +341,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) replace_extras_kernel(const T* A, int64_t lda, int64_t B, int32_t ncb, const uint32_t* extras,
                                                              int32_t extras_ld, const uint32_t* keepbits, const uint32_t* offsets,
                                                              T* values, int64_t capacity, float scale) {
+  begin_after_previous();
   const int lane = threadIdx.x & 31;
   for (int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); row < B; row += (int64_t)gridDim.x * 8) {
     const uint32_t* ex = extras + row * extras_ld;
@@ -388,10 +393,10 @@ int launch_rows_fixed(const RowsParams& p, int dtype, uint64_t seed, int64_t sme
   count_launch();
   if (dtype == RAD_BF16) {
     RAD_CUDA_TRY(cudaFuncSetAttribute(rows_fixed_kernel<bf16, kRowsOut>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmemBudget));
-    rows_fixed_kernel<bf16, kRowsOut><<<grid, 32 * kRowsWarps, (size_t)smem, s>>>(p, ks);
+    launch_kernel(rows_fixed_kernel<bf16, kRowsOut>, grid, 32 * kRowsWarps, (size_t)smem, s, p, ks);
   } else {
     RAD_CUDA_TRY(cudaFuncSetAttribute(rows_fixed_kernel<float, kRowsOut>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmemBudget));
-    rows_fixed_kernel<float, kRowsOut><<<grid, 32 * kRowsWarps, (size_t)smem, s>>>(p, ks);
+    launch_kernel(rows_fixed_kernel<float, kRowsOut>, grid, 32 * kRowsWarps, (size_t)smem, s, p, ks);
   }
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
@@ -460,7 +465,7 @@ int launch_replace_index(const rad_store* st, uint32_t* extras, bool check_capac
   const PhiloxKeys ks = philox_expand_key(st->seed);
   count_launch();
   RAD_CUDA_TRY(cudaFuncSetAttribute(replace_index_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmemBudget));
-  replace_index_kernel<<<(int)std::min<int64_t>(slabs, 148 * 8), 32 * kRowsWarps, (size_t)smem, s>>>(p, ks, extras, (int32_t)ld);
+  launch_kernel(replace_index_kernel, (int)std::min<int64_t>(slabs, 148 * 8), 32 * kRowsWarps, (size_t)smem, s, p, ks, extras, (int32_t)ld);
   if (cudaGetLastError() != cudaSuccess) return RAD_ECUDA;
   return launch_offsets_scan(st->offsets, slabs * p.ncb, st->nnz, check_capacity ? st->values_capacity : -1, dev_status, s);
 }
@@ -475,10 +480,10 @@ int launch_replace_extras(const void* A, int64_t lda, const rad_store* st, const
   const int grid = (int)std::min<int64_t>(ceil_div(st->B, 8), 148 * 64);   // short dependent chains: many warps in flight
   count_launch();
   if (st->dtype == RAD_BF16)
-    replace_extras_kernel<bf16><<<grid, 256, 0, s>>>(static_cast<const bf16*>(A), lda, st->B, ncb, extras, (int32_t)ld, st->keepbits,
+    launch_kernel(replace_extras_kernel<bf16>, grid, 256, 0, s, static_cast<const bf16*>(A), lda, st->B, ncb, extras, (int32_t)ld, st->keepbits,
                                                      st->offsets, static_cast<bf16*>(st->values), st->values_capacity, scale);
   else
-    replace_extras_kernel<float><<<grid, 256, 0, s>>>(static_cast<const float*>(A), lda, st->B, ncb, extras, (int32_t)ld, st->keepbits,
+    launch_kernel(replace_extras_kernel<float>, grid, 256, 0, s, static_cast<const float*>(A), lda, st->B, ncb, extras, (int32_t)ld, st->keepbits,
                                                       st->offsets, static_cast<float*>(st->values), st->values_capacity, scale);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
@@ -492,16 +497,16 @@ int rows_to_tiles(const rad_store* rows, const rad_store* tiles, int32_t* dev_st
   const int grid_t = (int)std::min<int64_t>(ceil_div(ntiles, 256), 148 * 8);
   count_launch(2);
   if (rows->dtype == RAD_BF16) {
-    rows_to_tiles_kernel<bf16><<<grid, 256, 0, s>>>(static_cast<const bf16*>(rows->values), reinterpret_cast<const uint16_t*>(rows->keepbits),
+    launch_kernel(rows_to_tiles_kernel<bf16>, grid, 256, 0, s, static_cast<const bf16*>(rows->values), reinterpret_cast<const uint16_t*>(rows->keepbits),
                                                     rows->B, k, rows->values_ld, ncb, tiles->keepbits, tiles->offsets,
                                                     static_cast<bf16*>(tiles->values), tiles->values_capacity, dev_status);
-    tile_padding_kernel<bf16><<<grid_t, 256, 0, s>>>(tiles->keepbits, tiles->offsets, ntiles, static_cast<bf16*>(tiles->values),
+    launch_kernel(tile_padding_kernel<bf16>, grid_t, 256, 0, s, tiles->keepbits, tiles->offsets, ntiles, static_cast<bf16*>(tiles->values),
                                                      tiles->values_capacity);
   } else {
-    rows_to_tiles_kernel<float><<<grid, 256, 0, s>>>(static_cast<const float*>(rows->values), reinterpret_cast<const uint16_t*>(rows->keepbits),
+    launch_kernel(rows_to_tiles_kernel<float>, grid, 256, 0, s, static_cast<const float*>(rows->values), reinterpret_cast<const uint16_t*>(rows->keepbits),
                                                      rows->B, k, rows->values_ld, ncb, tiles->keepbits, tiles->offsets,
                                                      static_cast<float*>(tiles->values), tiles->values_capacity, dev_status);
-    tile_padding_kernel<float><<<grid_t, 256, 0, s>>>(tiles->keepbits, tiles->offsets, ntiles, static_cast<float*>(tiles->values),
+    launch_kernel(tile_padding_kernel<float>, grid_t, 256, 0, s, tiles->keepbits, tiles->offsets, ntiles, static_cast<float*>(tiles->values),
                                                       tiles->values_capacity);
   }
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;

@@ -516,6 +516,7 @@ __host__ __device__ constexpr uint32_t make_idesc_pair(bool a_mn, bool b_mn, uin
 template <int AK, int BKIND, int EPI, int kEpiWarps2>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kEpiWarps2), 1)
 tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB) {
+  begin_after_previous();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   SmemCtl2* ctl = reinterpret_cast<SmemCtl2*>(smem + (size_t)kStages2 * kStage2Bytes);
@@ -742,6 +743,7 @@ struct SmemCtlSp {
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSpThreads, 1)
 tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB) {
+  begin_after_previous();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int stages = p.num_stages;
@@ -1005,6 +1007,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64, 1) wait_probe_pa
 __global__ void __launch_bounds__(256) dw_reduce_kernel(const float* partial, int64_t partial_rows, int splits,
                                                         int64_t M, const int64_t* M_dev, int64_t N,
                                                         const uint32_t* row_idx, float* out, int64_t ldw) {
+  begin_after_previous();
   if (M_dev != nullptr) M = min(M, *M_dev);
   const int64_t n4 = N / 4, total = M * n4;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
@@ -1191,7 +1194,7 @@ int launch_pair(const TcParams& p, const CUtensorMap& ta, const CUtensorMap& tb,
   }
   const int pairs = (int)std::max<int64_t>(1, std::min<int64_t>(max_units, resident_pairs));
   count_launch();
-  kernel<<<2 * pairs, threads2(kEpiWarps2), smem, s>>>(p, ta, tb);
+  launch_kernel(kernel, 2 * pairs, threads2(kEpiWarps2), smem, s, p, ta, tb);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 
@@ -1207,7 +1210,7 @@ int launch_sparse_pair(const TcParams& p, const CUtensorMap& tb, int64_t max_uni
   }
   const int pairs = (int)std::max<int64_t>(1, std::min<int64_t>(max_units, resident_pairs));
   count_launch();
-  tc_sparse_pair_kernel<<<2 * pairs, kSpThreads, smem, s>>>(p, tb);
+  launch_kernel(tc_sparse_pair_kernel, 2 * pairs, kSpThreads, smem, s, p, tb);
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
 
@@ -1329,7 +1332,7 @@ int tc_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, 
     const int64_t work = rows * (H / 4);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(work, 256), 148 * 16));
     count_launch();
-    dw_reduce_kernel<<<grid, 256, 0, s>>>(p.partial, d.partial_rows, d.splits, rows, p.N_dev, H, p.row_idx, dW, ldw);
+    launch_kernel(dw_reduce_kernel, grid, 256, 0, s, p.partial, d.partial_rows, d.splits, rows, p.N_dev, H, p.row_idx, dW, ldw);
   }
   return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
 }
