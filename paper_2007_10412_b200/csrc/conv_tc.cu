@@ -136,7 +136,7 @@ __device__ __forceinline__ uint4 cv_load_pixel(const bf16* T, bool in, int y, in
 enum { kCvFwd = 0, kCvDw = 1, kCvDx = 2 };
 template <int kMode>
 __global__ void __launch_bounds__(kCvThreads, 3) conv_tc_kernel(const ConvTcParams p) {
-  begin_after_previous();
+  wait_for_previous();
   constexpr bool kDw = kMode == kCvDw, kDx = kMode == kCvDx;
   extern __shared__ uint8_t cv_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(cv_raw) + 1023) & ~(uintptr_t)1023);
@@ -244,6 +244,7 @@ __global__ void __launch_bounds__(kCvThreads, 3) conv_tc_kernel(const ConvTcPara
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = ctl->tmem_base;
+  let_next_start();
 
   bool ok = true;
   for (int kb = 0; kb < nkb; ++kb) {

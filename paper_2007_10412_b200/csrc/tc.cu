@@ -67,6 +67,7 @@ struct TcParams {
 // ---- PTX wrappers ---------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) { asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory"); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -516,7 +517,6 @@ __host__ __device__ constexpr uint32_t make_idesc_pair(bool a_mn, bool b_mn, uin
 template <int AK, int BKIND, int EPI, int kEpiWarps2>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kEpiWarps2), 1)
 tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB) {
-  begin_after_previous();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   SmemCtl2* ctl = reinterpret_cast<SmemCtl2*>(smem + (size_t)kStages2 * kStage2Bytes);
@@ -526,23 +526,10 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
   const uint32_t rank = cluster_ctarank();         // 0: issues the MMAs; both stage operands and run epilogues
   const uint32_t peer_abort = map_to_cta(smem_u32(&ctl->abort_flag), rank ^ 1u);
   const PairWait wc = {abort_flag, peer_abort, p.wait_limit_ns};
-  // Same-sample dW (kDwT): the tile is dW^T, M = H, N = kept columns (known on the device only).  The kept
-  // columns are cut into the fewest tiles of at most 256 and the tile width bn is what one of them needs,
-  // rounded up to the MMA's granule of 16: 105 kept columns cost one tile of 112, not one of 256.
-  int64_t n_cols = p.N;
-  int bn = p.bn;
-  if (EPI == kDwT) {
-    int64_t nd;
-    asm volatile("ld.global.cg.s64 %0, [%1];" : "=l"(nd) : "l"(p.N_dev) : "memory");
-    n_cols = nd < n_cols ? nd : n_cols;
-    const int64_t nt = max((int64_t)1, (n_cols + BN - 1) / BN);
-    bn = max(16, (int)(((n_cols + nt - 1) / nt + 15) / 16 * 16));
-  }
-  const Schedule sched(p.M, n_cols, p.K, p.splits, BM, bn);
-  const int boxes_b = (bn / 2 + 63) / 64;             // 64-column boxes of an MN-major B this CTA stages per K block
-  const uint32_t stage_tx = 2u * (uint32_t)(kStage2Bytes / 2 + (BKIND == kBK_ ? bn / 2 * 128 : boxes_b * 8192));
   const int64_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   if (tid == 0) {
+    prefetch_map(&tmA);
+    prefetch_map(&tmB);
     for (int s = 0; s < kStages2; ++s) {
       mbar_init(smem_u32(&ctl->full[s]), 1);
       mbar_init(smem_u32(&ctl->empty[s]), 1);
@@ -564,6 +551,23 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
   const uint32_t smem_base = smem_u32(smem);
+  // so far nothing of another kernel was touched: the above runs under the tail of the kernel before
+  begin_after_previous();
+  // Same-sample dW (kDwT): the tile is dW^T, M = H, N = kept columns (known on the device only).  The kept
+  // columns are cut into the fewest tiles of at most 256 and the tile width bn is what one of them needs,
+  // rounded up to the MMA's granule of 16: 105 kept columns cost one tile of 112, not one of 256.
+  int64_t n_cols = p.N;
+  int bn = p.bn;
+  if (EPI == kDwT) {
+    int64_t nd;
+    asm volatile("ld.global.cg.s64 %0, [%1];" : "=l"(nd) : "l"(p.N_dev) : "memory");
+    n_cols = nd < n_cols ? nd : n_cols;
+    const int64_t nt = max((int64_t)1, (n_cols + BN - 1) / BN);
+    bn = max(16, (int)(((n_cols + nt - 1) / nt + 15) / 16 * 16));
+  }
+  const Schedule sched(p.M, n_cols, p.K, p.splits, BM, bn);
+  const int boxes_b = (bn / 2 + 63) / 64;             // 64-column boxes of an MN-major B this CTA stages per K block
+  const uint32_t stage_tx = 2u * (uint32_t)(kStage2Bytes / 2 + (BKIND == kBK_ ? bn / 2 * 128 : boxes_b * 8192));
 
   if (warp == 0) {
     // ===== TMA producer: this CTA's 128 rows of A and 128 rows (N) of B, completing on the even CTA's barrier =====
@@ -743,7 +747,6 @@ struct SmemCtlSp {
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSpThreads, 1)
 tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB) {
-  begin_after_previous();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int stages = p.num_stages;
@@ -759,6 +762,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
   const Schedule sched(p.M, p.N, p.K, p.splits, kSpBM, kSpBN);
   const int64_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   if (tid == 0) {
+    prefetch_map(&tmB);
     for (int s = 0; s < stages; ++s) {
       mbar_init(smem_u32(&ctl->full[s]), 1 + 2 * kSpExpanderWarps);
       mbar_init(smem_u32(&ctl->empty[s]), 1);
@@ -782,6 +786,8 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
   const uint32_t smem_base = smem_u32(smem);
+  // so far nothing of another kernel was touched: the above runs under the tail of the kernel before
+  begin_after_previous();
   // this CTA's store tile column (128 columns of the layer input) of a unit, and whether it exists
   auto tile_col_of = [&](const Unit& w) -> int64_t { return (w.m0 + 128 * (int64_t)rank) / kTileCols; };
 
