@@ -37,7 +37,7 @@ constexpr int kRasterGroup = 16;               // m-tiles per raster group (16 x
 
 enum AKind { kAK = 0, kAMN = 1, kASparse = 2 };
 enum BKind { kBK_ = 0, kBMN = 1 };
-enum EpiKind { kFwd = 0, kDx = 1, kDw = 2, kDwT = 3 };
+enum EpiKind { kFwd = 0, kDx = 1, kDwT = 2 };
 
 struct TcParams {
   int64_t M, N, K;
@@ -108,6 +108,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
         "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
         "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr) : "memory");
+}
+// 16 lanes x 32 columns: register 4 i + e holds lane (thread / 4) + 8 (e / 2), column 8 i + 2 (thread % 4) + e % 2.
+__device__ __forceinline__ void tmem_ld16x32(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -270,7 +279,7 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, uint32_t (&r)[
         }
       }
     }
-  } else if (EPI == kDx) {
+  } else {
     if (row_ok) {
       uint32_t bits = 0xffffffffu;
       if (p.relubits_prev != nullptr) bits = __ldg(p.relubits_prev + m * ((p.N + 31) / 32) + (n >> 5));
@@ -300,22 +309,34 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, uint32_t (&r)[
         }
       }
     }
-  } else {
-    if (row_ok) {
-      float* dst;
-      if (p.splits > 1) {
-        dst = p.partial + ((int64_t)split * p.partial_rows + m) * p.N + n;
-      } else {
-        const int64_t row = (p.row_idx != nullptr) ? (int64_t)__ldg(p.row_idx + m) : m;
-        if (row >= p.dw_rows) { raise_status(p.dev_status, RAD_DEV_EINTERNAL); return; }
-        dst = p.out_dw + row * p.ld_dw + n;
-      }
-      float4* d4 = reinterpret_cast<float4*>(dst);
+  }
+}
+
+// Different-sample dW: 32 accumulator rows (from row `m0`, tensor-memory address `taddr`) x 32 columns by one warp.
+// With a row per thread every 16-byte store of a warp touches 32 lines, one look-up each: 8 us for a CTA's 128 x 512
+// tile, whatever the number of warps.  Here the accumulators come in the layout of matrix fragments and neighbouring
+// threads exchange column pairs, so that a store covers 64 bytes of eight rows.
+__device__ __forceinline__ void epilogue_dw(const TcParams& p, uint32_t taddr, int64_t m0, int64_t n, int32_t split, int lane) {
+  const int nvalid = (int)min((int64_t)32, p.N - n);      // multiple of 8
+  uint32_t r[2][16];
+  tmem_ld16x32(taddr, r[0]);
+  tmem_ld16x32(taddr + (16u << 16), r[1]);
+  tmem_ld_wait();
+  const bool odd = (lane & 1) != 0;
 #pragma unroll
-      for (int j = 0; j < 32; j += 4)
-        if (j < nvalid)
-          d4[j >> 2] = make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
-                                   __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+  for (int h = 0; h < 4; ++h) {                            // rows 8 h + lane / 4
+    const int64_t m = m0 + 8 * h + (lane >> 2);
+    float* dst = p.splits > 1 ? p.partial + ((int64_t)split * p.partial_rows + m) * p.N + n : p.out_dw + m * p.ld_dw + n;
+#pragma unroll
+    for (int i = 0; i < 4; i += 2) {                       // column blocks i (even threads keep it) and i + 1 (odd threads)
+      const uint32_t* a = &r[h >> 1][4 * i + 2 * (h & 1)];
+      const uint32_t* b = a + 4;
+      const uint32_t t0 = __shfl_xor_sync(0xffffffffu, odd ? a[0] : b[0], 1);
+      const uint32_t t1 = __shfl_xor_sync(0xffffffffu, odd ? a[1] : b[1], 1);
+      const float4 v = odd ? make_float4(__uint_as_float(t0), __uint_as_float(t1), __uint_as_float(b[0]), __uint_as_float(b[1]))
+                           : make_float4(__uint_as_float(a[0]), __uint_as_float(a[1]), __uint_as_float(t0), __uint_as_float(t1));
+      const int col = 8 * (i + (lane & 1)) + 4 * ((lane >> 1) & 1);
+      if (m < p.M && col < nvalid) *reinterpret_cast<float4*>(dst + col) = v;
     }
   }
 }
@@ -700,7 +721,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
         tmem_ld_wait();
         // a chunk may reach past the tile's width (bn is a multiple of 16) and past the last kept column
         if (EPI == kDwT) epilogue_chunk_dwt(p, r, m, n, (int)min((int64_t)min(32, bn - c0), n_cols - n), row_ok, w.split);
-        else epilogue_chunk<(EPI == kDwT ? kDw : EPI)>(p, r, m, n, row_ok, w.split, sr);
+        else epilogue_chunk<(EPI == kDwT ? kDx : EPI)>(p, r, m, n, row_ok, w.split, sr);
       }
       tc_fence_before();
       __syncwarp();
@@ -862,27 +883,23 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
       }
     }
   } else if (warp < 6) {
-    // ===== epilogue: thread = one accumulator row (512 columns) =====
+    // ===== epilogue: a warp = 32 accumulator rows (512 columns) =====
     const int q = warp & 3;
     const uint32_t empty_bar = map_to_cta(smem_u32(&ctl->tmem_empty), 0u);
     uint32_t unit_phase = 0;
     bool ok = true;
     for (int64_t u = pair; u < sched.units && ok; u += npairs) {
       const Unit w = sched.unit(u);
-      if (lane == 0) ok = mbar_wait2(smem_u32(&ctl->tmem_full), unit_phase, wc, 1000u);
+      if (lane == 0) ok = mbar_wait2(smem_u32(&ctl->tmem_full), unit_phase, wc, 200u);
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       if (!ok) break;
       tc_fence_after();
-      const int64_t m = w.m0 + 128 * (int64_t)rank + q * 32 + lane;
-      const bool row_ok = m < sched.M;
+      const int64_t m0 = w.m0 + 128 * (int64_t)rank + q * 32;
 #pragma unroll 1
       for (int c0 = 0; c0 < kSpBN; c0 += 32) {
         const int64_t n = w.n0 + c0;
         if (n >= p.N) break;                  // warp-uniform
-        uint32_t r[32];
-        tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
-        tmem_ld_wait();
-        epilogue_chunk<kDw>(p, r, m, n, row_ok, w.split, StoreRow{});
+        epilogue_dw(p, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, m0, n, w.split, lane);
       }
       tc_fence_before();
       __syncwarp();
