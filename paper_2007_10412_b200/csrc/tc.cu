@@ -758,6 +758,7 @@ constexpr int kSpStageBytes = kSpAStageBytes + kSpBStageBytes;
 constexpr int kSpMaxStages = 4;
 constexpr int kSpExpanderWarps = 8;                    // per K block: one thread per keep-bit word of the store tile
 constexpr int kSpExpanderGroups = 2;                   // groups of eight warps take alternate K blocks
+constexpr int kSpEpiShare = 1 + kSpExpanderWarps * kSpExpanderGroups / 4;   // warps of a lane quarter that share the epilogue
 constexpr int kSpThreads = 32 * (kFirstExpanderWarp + kSpExpanderGroups * kSpExpanderWarps);
 
 struct SmemCtlSp {
@@ -793,7 +794,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
       mbar_init(smem_u32(&ctl->comp_empty[c]), kSpExpanderWarps);
     }
     mbar_init(smem_u32(&ctl->tmem_full), 1);
-    mbar_init(smem_u32(&ctl->tmem_empty), 8);          // four epilogue warps in each CTA
+    mbar_init(smem_u32(&ctl->tmem_empty), 2 * 4 * kSpEpiShare);      // epilogue and expander warps of both CTAs
     ctl->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -811,6 +812,26 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
   begin_after_previous();
   // this CTA's store tile column (128 columns of the layer input) of a unit, and whether it exists
   auto tile_col_of = [&](const Unit& w) -> int64_t { return (w.m0 + 128 * (int64_t)rank) / kTileCols; };
+  // A warp's part of a unit's epilogue: 32-column chunks `first`, first + kSpEpiShare, ... of its lane quarter's rows
+  auto unit_epilogue = [&](const Unit& w, int first, uint32_t parity) -> bool {
+    const int q = warp & 3;
+    bool ready = true;
+    if (lane == 0) ready = mbar_wait2(smem_u32(&ctl->tmem_full), parity, wc, 100u);
+    ready = __shfl_sync(0xffffffffu, ready ? 1 : 0, 0) != 0;
+    if (!ready) return false;
+    tc_fence_after();
+    const int64_t m0 = w.m0 + 128 * (int64_t)rank + q * 32;
+#pragma unroll 1
+    for (int c0 = first * 32; c0 < kSpBN; c0 += kSpEpiShare * 32) {
+      const int64_t n = w.n0 + c0;
+      if (n >= p.N) break;                  // warp-uniform
+      epilogue_dw(p, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, m0, n, w.split, lane);
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive_remote(map_to_cta(smem_u32(&ctl->tmem_empty), 0u));
+    return true;
+  };
 
   if (warp == 0) {
     // ===== dZ producer: this CTA's 128 columns of each 256-column half of the dZ tile =====
@@ -883,27 +904,11 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
       }
     }
   } else if (warp < 6) {
-    // ===== epilogue: a warp = 32 accumulator rows (512 columns) =====
-    const int q = warp & 3;
-    const uint32_t empty_bar = map_to_cta(smem_u32(&ctl->tmem_empty), 0u);
+    // ===== epilogue: a warp = 32 accumulator rows, every kSpEpiShare-th 32-column chunk (the expanders take the others) =====
     uint32_t unit_phase = 0;
     bool ok = true;
     for (int64_t u = pair; u < sched.units && ok; u += npairs) {
-      const Unit w = sched.unit(u);
-      if (lane == 0) ok = mbar_wait2(smem_u32(&ctl->tmem_full), unit_phase, wc, 200u);
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      if (!ok) break;
-      tc_fence_after();
-      const int64_t m0 = w.m0 + 128 * (int64_t)rank + q * 32;
-#pragma unroll 1
-      for (int c0 = 0; c0 < kSpBN; c0 += 32) {
-        const int64_t n = w.n0 + c0;
-        if (n >= p.N) break;                  // warp-uniform
-        epilogue_dw(p, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, m0, n, w.split, lane);
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_remote(empty_bar);
+      ok = unit_epilogue(sched.unit(u), 0, unit_phase);
       unit_phase ^= 1u;
     }
   } else if (warp == 6) {
@@ -966,7 +971,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
     const int wi = et & 255;
     const int r = (wi & 7) + ((wi >> 5) << 3), wq = (wi >> 3) & 3;
     int stage = 0, slot = 0;
-    uint32_t phase = 0, cphase = 0, turn = 0;
+    uint32_t phase = 0, cphase = 0, turn = 0, unit_phase = 0;
     bool ok = true;
     for (int64_t u = pair; u < sched.units && ok; u += npairs) {
       const Unit w = sched.unit(u);
@@ -993,6 +998,9 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
         if (++stage == stages) { stage = 0; phase ^= 1u; }
         if (++slot == p.comp_depth) { slot = 0; cphase ^= 1u; }
       }
+      // the next unit's MMAs wait for this unit's accumulators to be read, so the expanders have nothing better to do
+      if (ok) ok = unit_epilogue(w, 1 + (warp - kFirstExpanderWarp) / 4, unit_phase);
+      unit_phase ^= 1u;
     }
   }
 
