@@ -36,6 +36,7 @@ struct GemmParams {
   const uint32_t* keepbits; const uint32_t* offsets; int64_t capacity; int32_t ncb;
   // set by plan_gemm
   int tile, splits;            // rows and columns of C per tile; CTAs (1, 2, 4 or 8) that share a tile's k
+  int walk;                    // one CTA walks all of k (splits is 1)
   int vec_a, vec_b;            // 16-byte copies of the operand are aligned
   int64_t k_per, gx, units;    // k per split, tiles per tile row, CTAs in all
 };
@@ -63,6 +64,7 @@ constexpr int kGemmStages = 3;                       // float32: K blocks in fli
 __host__ __device__ constexpr int gemm_operand_floats(int ts) { return ts * (kGemmBK + 4) > kGemmBK * (ts + 4) ? ts * (kGemmBK + 4) : kGemmBK * (ts + 4); }
 __host__ __device__ constexpr int gemm_smem_bytes(int ts) { return kGemmStages * 2 * gemm_operand_floats(ts) * 4; }
 constexpr int kGemmSmemBytes = gemm_smem_bytes(64);
+static_assert(gemm_smem_bytes(32) >= 4 * 64 * (32 + 4) * 4, "the walking form fits the same buffer");
 static_assert(gemm_smem_bytes(32) >= (4 * 32 * 32 + 32) * 4 && gemm_smem_bytes(64) >= (4 * 64 * 64 + 64) * 4,
               "the partial tiles and column sums reuse the ring");
 
@@ -339,6 +341,29 @@ __device__ __forceinline__ void gemm_partial(const GemmParams& p, int64_t tile, 
     smem[e] = (smem[e] + smem[TS * TS + e]) + (smem[2 * TS * TS + e] + smem[3 * TS * TS + e]);
 }
 
+// Epilogue of one output.
+template <typename T, int EPI>
+__device__ __forceinline__ void gemm_store(const GemmParams& p, int64_t m, int64_t n, float v) {
+  if (EPI == kEpiForward) {
+    if (p.bias != nullptr) v += p.bias[n];
+    if (p.out_z != nullptr) p.out_z[m * p.ld_z + n] = v;
+    if (p.out_zlow != nullptr) static_cast<T*>(p.out_zlow)[m * p.ld_zlow + n] = from_float<T>(v);
+    if (p.out_act != nullptr) {
+      const float a = p.act == RAD_ACT_RELU ? fmaxf(v, 0.0f) : p.act == RAD_ACT_GELU ? gelu_f(v) : v;
+      static_cast<T*>(p.out_act)[m * p.ld_act + n] = from_float<T>(a);
+    }
+  } else if (EPI == kEpiInputGrad) {
+    if (p.relubits != nullptr) {
+      if (((p.relubits[m * p.w32 + (n >> 5)] >> (n & 31)) & 1u) == 0) v = 0.0f;
+    } else if (p.z_prev != nullptr) {
+      v *= gelu_grad_f(to_float(static_cast<const T*>(p.z_prev)[m * p.ld_zprev + n]));
+    }
+    static_cast<T*>(p.out_low)[m * p.ld_low + n] = from_float<T>(v);
+  } else {
+    p.out_f32[(EPI == kEpiScatterRows ? (int64_t)p.row_idx[m] : m) * p.ld_f32 + n] = v;
+  }
+}
+
 // The CTA's share of the tile's rows, from the partial tiles of all its splits.
 template <typename T, int EPI, int TS>
 __device__ __forceinline__ void gemm_finish(const GemmParams& p, int64_t tile, int split, const float* smem) {
@@ -365,23 +390,107 @@ __device__ __forceinline__ void gemm_finish(const GemmParams& p, int64_t tile, i
     } else {
       v = smem[e];
     }
-    if (EPI == kEpiForward) {
-      if (p.bias != nullptr) v += p.bias[n];
-      if (p.out_z != nullptr) p.out_z[m * p.ld_z + n] = v;
-      if (p.out_zlow != nullptr) static_cast<T*>(p.out_zlow)[m * p.ld_zlow + n] = from_float<T>(v);
-      if (p.out_act != nullptr) {
-        const float a = p.act == RAD_ACT_RELU ? fmaxf(v, 0.0f) : p.act == RAD_ACT_GELU ? gelu_f(v) : v;
-        static_cast<T*>(p.out_act)[m * p.ld_act + n] = from_float<T>(a);
+    gemm_store<T, EPI>(p, m, n, v);
+  }
+}
+
+// The other form, for short contractions and most bf16 shapes (see plan_gemm): one TS x TS tile of C by one CTA of 256
+// threads that walks all of k, TS/16 x TS/16 outputs per thread, the next step's rows of K in registers while the
+// current ones are multiplied out of shared memory; nothing to add at the end.  Every output is one chain of fused
+// multiply-adds over k in ascending order.  K rows per step: the small tile takes four times as many, so that its
+// steps, which are bound by the latency of their loads, are a quarter as many.
+constexpr int walk_bk(int ts) { return ts == 32 ? 64 : 16; }
+constexpr int walk_smem_bytes(int ts) { return 4 * walk_bk(ts) * (ts + 4) * 4; }
+template <typename T, int EPI, int TS>
+__device__ __forceinline__ void gemm_walk(const GemmParams& p, int64_t tile, float* smem) {
+  constexpr int kBM = TS, kBN = TS, TM = TS / 16, kBK = walk_bk(TS), NF = TS * kBK / 256;
+  constexpr int kLdS = TS + 4;                       // floats per k row of a staged operand (16-byte multiples)
+  static_assert((kLdS * 4) % 16 == 0 && (TM == 4 || TM == 2), "vector reads of the staged operands");
+  int64_t M = p.M;
+  if (p.M_dev != nullptr) M = min(M, *p.M_dev);
+  const int64_t m0 = tile / p.gx * kBM, n0 = tile % p.gx * kBN;
+  const bool sums = EPI == kEpiScatterRows && p.db != nullptr && m0 == 0;
+  if (m0 >= M && !sums) return;
+  const int tid = threadIdx.x;
+  float colsum = 0.0f;
+  const int tm = (tid >> 4) * TM, tn = (tid & 15) * TM;
+  const T* A = static_cast<const T*>(p.A);
+  const T* Bm = static_cast<const T*>(p.Bm);
+  float acc[TM][TM] = {};
+  // TS x kBK elements of each operand per step; whichever index is contiguous in memory is made
+  // the fast thread index
+  float ra[NF], rb[NF];
+  auto fetch = [&](int64_t k0) {
+#pragma unroll
+    for (int j = 0; j < NF; ++j) {
+      const int i = tid + j * 256;
+      int mm, kk;
+      if (p.sak == 1) { kk = i % kBK; mm = i / kBK; } else { mm = i % kBM; kk = i / kBM; }
+      const int64_t m = m0 + mm, k = k0 + kk;
+      ra[j] = (m < M && k < p.K) ? to_float(A[m * p.sam + k * p.sak]) : 0.0f;
+      int nn;
+      if (p.sbk == 1) { kk = i % kBK; nn = i / kBK; } else { nn = i % kBN; kk = i / kBN; }
+      const int64_t n = n0 + nn, kb = k0 + kk;
+      rb[j] = (n < p.N && kb < p.K) ? to_float(Bm[kb * p.sbk + n * p.sbn]) : 0.0f;
+    }
+  };
+  auto stash = [&](int buf) {
+    float* sA = smem + buf * 2 * kBK * kLdS;
+    float* sB = sA + kBK * kLdS;
+#pragma unroll
+    for (int j = 0; j < NF; ++j) {
+      const int i = tid + j * 256;
+      if (p.sak == 1) sA[(i % kBK) * kLdS + i / kBK] = ra[j]; else sA[(i / kBM) * kLdS + i % kBM] = ra[j];
+      if (p.sbk == 1) sB[(i % kBK) * kLdS + i / kBK] = rb[j]; else sB[(i / kBN) * kLdS + i % kBN] = rb[j];
+    }
+  };
+  fetch(0);
+  stash(0);
+  __syncthreads();
+  int buf = 0;
+  for (int64_t k0 = 0; k0 < p.K; k0 += kBK) {
+    const bool more = k0 + kBK < p.K;
+    if (more) fetch(k0 + kBK);
+    const float* sA = smem + buf * 2 * kBK * kLdS;
+    const float* sB = sA + kBK * kLdS;
+    if (sums && tid < kBN) {
+      // the block of Bm is in shared memory anyway: its column sums, row after row (rows past K hold zeros)
+#pragma unroll
+      for (int kk = 0; kk < kBK; ++kk) colsum += sB[kk * kLdS + tid];
+    }
+#pragma unroll
+    for (int kk = 0; kk < kBK; ++kk) {
+      float a[TM], b[TM];
+      if (TM == 4) {
+        const float4 a4 = *reinterpret_cast<const float4*>(sA + kk * kLdS + tm);
+        const float4 b4 = *reinterpret_cast<const float4*>(sB + kk * kLdS + tn);
+        a[0] = a4.x; a[1] = a4.y; a[TM - 2] = a4.z; a[TM - 1] = a4.w;
+        b[0] = b4.x; b[1] = b4.y; b[TM - 2] = b4.z; b[TM - 1] = b4.w;
+      } else {
+        const float2 a2 = *reinterpret_cast<const float2*>(sA + kk * kLdS + tm);
+        const float2 b2 = *reinterpret_cast<const float2*>(sB + kk * kLdS + tn);
+        a[0] = a2.x; a[1] = a2.y;
+        b[0] = b2.x; b[1] = b2.y;
       }
-    } else if (EPI == kEpiInputGrad) {
-      if (p.relubits != nullptr) {
-        if (((p.relubits[m * p.w32 + (n >> 5)] >> (n & 31)) & 1u) == 0) v = 0.0f;
-      } else if (p.z_prev != nullptr) {
-        v *= gelu_grad_f(to_float(static_cast<const T*>(p.z_prev)[m * p.ld_zprev + n]));
-      }
-      static_cast<T*>(p.out_low)[m * p.ld_low + n] = from_float<T>(v);
-    } else {
-      p.out_f32[(EPI == kEpiScatterRows ? (int64_t)p.row_idx[m] : m) * p.ld_f32 + n] = v;
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TM; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    }
+    if (more) stash(buf ^ 1);
+    __syncthreads();
+    buf ^= 1;
+  }
+  if (sums && tid < kBN && n0 + tid < p.N) p.db[n0 + tid] = colsum;
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    const int64_t m = m0 + tm + i;
+    if (m >= M) continue;
+#pragma unroll
+    for (int j = 0; j < TM; ++j) {
+      const int64_t n = n0 + tn + j;
+      if (n >= p.N) continue;
+      gemm_store<T, EPI>(p, m, n, acc[i][j]);
     }
   }
 }
@@ -389,24 +498,36 @@ __device__ __forceinline__ void gemm_finish(const GemmParams& p, int64_t tile, i
 // Tile and split of a contraction: the pair with the least estimated time, in clocks of the SM that gets the most
 // CTAs.  Two CTAs share an SM; per k of its share a pair takes 106 clocks with 64 x 64 tiles and 35 with 32 x 32
 // (0.60 and 0.46 of the FMA rate), a CTA alone 73 and 26; beginning and end of a CTA (first loads, the groups'
-// sums, epilogue) take 6000 and 3850, the launch 4000, the exchange inside a cluster 800.  Fitted to 32 timings
+// sums, epilogue) take 7500 and 3850, the launch 4000, the exchange inside a cluster 800.  Fitted to 32 timings
 // (both tiles, 1 to 8 splits); for 150 x 300 outputs it says 28 / 19 / 19 / 22 thousand clocks for 1 / 2 / 4 / 8 CTAs
 // per 32 x 32 tile at k = 784, measured 26 / 19 / 18 / 23; for 1500 x 777, k = 1001, 102 / 91 / 94 us for 1 / 2 / 4 CTAs
 // per 64 x 64 tile, measured 112 / 101 / 102.
-inline void plan_gemm(GemmParams& p, int64_t Mgrid, int es, int64_t k_step = 4) {      // splits begin at multiples of k_step
+// The walking form (no split, no sums at the end) is weighed with figures of its own, and bf16 operands, which both forms
+// widen on the way through registers, with others again (the split form's depend on whether k is contiguous: more
+// address arithmetic and spilled registers then).  So the walking form takes short contractions (4096 x 1001 f32, k =
+// 10: 16 us against 30; the lines cross near k = 200 where the chip is full and near k = 80 where it is not) and bf16
+// shapes that fill the chip (1024 x 1023 x 1021 forward: 92 against 137 us).
+struct GemmCost { double pair, alone, ends; };
+inline void plan_gemm(GemmParams& p, int64_t Mgrid, int es, int64_t k_step = 4, bool may_walk = true) {   // splits begin at multiples of k_step
+  static const GemmCost split_cost[3][2] = {{{35, 26, 3850}, {106, 73, 7500}},      // f32, at 32 x 32 and 64 x 64
+                                            {{72, 45, 4500}, {258, 150, 11000}},    // bf16, k contiguous
+                                            {{72, 45, 4500}, {150, 90, 7500}}};     // bf16, dW
+  static const GemmCost walk_cost[2][2] = {{{80, 46, 2000}, {158, 100, 3500}}, {{110, 72, 2000}, {168, 110, 3800}}};
+  const int kind = es == 4 ? 0 : p.sak == 1 ? 1 : 2;
   double best = 1e300;
   for (int ts = 32; ts <= 64; ts *= 2) {
     const int64_t tiles = std::max<int64_t>(1, ceil_div(Mgrid, ts)) * ceil_div(p.N, ts);
-    const double pair = ts == 64 ? 106.0 : 35.0, alone = ts == 64 ? 73.0 : 26.0, ends = ts == 64 ? 6000.0 : 3850.0;
-    for (int s = 1; s <= 8; s *= 2) {
+    for (int s = may_walk ? 0 : 1; s <= 8; s = s == 0 ? 1 : 2 * s) {               // 0: the walking form
       if (s > 1 && (p.K < 16 * s || p.K <= s / 2 * k_step)) break;
-      const int64_t per_sm = ceil_div(tiles * s, 148), k_per = round_up(ceil_div(p.K, s), k_step);
-      const double clk = (double)k_per * ((double)(per_sm / 2) * pair + (double)(per_sm % 2) * alone) + (double)per_sm * ends + 4000.0 +
-                         (s > 1 ? 800.0 : 0.0);
+      const int n = std::max(s, 1);
+      const GemmCost& c = (s == 0 ? walk_cost[es == 2] : split_cost[kind])[ts == 64];
+      const int64_t per_sm = ceil_div(tiles * n, 148), k_per = round_up(ceil_div(p.K, n), k_step);
+      const double clk = (double)k_per * ((double)(per_sm / 2) * c.pair + (double)(per_sm % 2) * c.alone) + (double)per_sm * c.ends + 4000.0 +
+                         (n > 1 ? 800.0 : 0.0);
       if (clk < best) {
         best = clk;
-        p.tile = ts; p.splits = s; p.k_per = k_per;
-        p.gx = ceil_div(p.N, ts); p.units = tiles * s;
+        p.tile = ts; p.splits = n; p.k_per = k_per; p.walk = s == 0 ? 1 : 0;
+        p.gx = ceil_div(p.N, ts); p.units = tiles * n;
       }
     }
   }
@@ -417,12 +538,18 @@ inline void plan_gemm(GemmParams& p, int64_t Mgrid, int es, int64_t k_step = 4) 
 template <typename T, int EPI>
 __device__ __forceinline__ void gemm_unit_partial(const GemmParams& p, int64_t unit, float* smem) {
   if (unit >= p.units) return;
+  if constexpr (EPI != kEpiSparse) {
+    if (p.walk) {
+      if (p.tile == 32) gemm_walk<T, EPI, 32>(p, unit, smem); else gemm_walk<T, EPI, 64>(p, unit, smem);
+      return;
+    }
+  }
   if (p.tile == 32) gemm_partial<T, EPI, 32>(p, unit / p.splits, (int)(unit % p.splits), smem);
   else gemm_partial<T, EPI, 64>(p, unit / p.splits, (int)(unit % p.splits), smem);
 }
 template <typename T, int EPI>
 __device__ __forceinline__ void gemm_unit_finish(const GemmParams& p, int64_t unit, const float* smem) {
-  if (unit >= p.units) return;
+  if (unit >= p.units || p.walk) return;
   if (p.tile == 32) gemm_finish<T, EPI, 32>(p, unit / p.splits, (int)(unit % p.splits), smem);
   else gemm_finish<T, EPI, 64>(p, unit / p.splits, (int)(unit % p.splits), smem);
 }
@@ -437,10 +564,25 @@ __global__ void __launch_bounds__(256, 2) gemm_kernel(const GemmParams p) {
   if (cluster_nctas() > 1) cluster_barrier();        // no CTA leaves while another reads its partial tile
 }
 
+template <typename T, int EPI>
+__global__ void __launch_bounds__(256) gemm_walk_kernel(const GemmParams p) {
+  begin_after_previous();
+  extern __shared__ __align__(16) float smem[];
+  if (p.tile == 32) gemm_walk<T, EPI, 32>(p, blockIdx.x, smem); else gemm_walk<T, EPI, 64>(p, blockIdx.x, smem);
+}
+
 template <int EPI>
 int launch_planned(int dtype, const GemmParams& p, cudaStream_t s) {
   if (p.units > 0x7fffffff) return RAD_EINVAL;
   count_launch();
+  if constexpr (EPI != kEpiSparse) {
+    if (p.walk) {
+      const dim3 grid((unsigned)p.units);
+      const size_t smem = (size_t)walk_smem_bytes(p.tile);
+      return dtype == RAD_BF16 ? launch_kernel(gemm_walk_kernel<bf16, EPI>, grid, 256, smem, s, p)
+                               : launch_kernel(gemm_walk_kernel<float, EPI>, grid, 256, smem, s, p);
+    }
+  }
   if (dtype == RAD_BF16) {
     static std::atomic<uint64_t> ready{0};
     if (!allow_smem(gemm_kernel<bf16, EPI>, kGemmSmemBytes, ready)) return RAD_ECUDA;
@@ -744,7 +886,7 @@ int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H
   p.out_f32 = dW; p.ld_f32 = ldw;
   p.db = db;
   if (db_written != nullptr) *db_written = db != nullptr;
-  plan_gemm(p, p.M, low ? 2 : 4, kTileRows);
+  plan_gemm(p, p.M, low ? 2 : 4, kTileRows, false);
   if (ig != nullptr && ig_done != nullptr) {
     GemmParams g = input_grad_params(st->B, st->D, H, dZ, ldz, *ig);
     plan_gemm(g, g.M, low ? 2 : 4);
