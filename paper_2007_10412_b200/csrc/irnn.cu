@@ -96,11 +96,13 @@ __global__ void __launch_bounds__(32 * (KP / 2 + kStoreWarps), 2) irnn_forward_k
   __shared__ __align__(16) float s_h[kRing][kHdMax];
   __shared__ __align__(16) uint32_t s_mask[2][kGroup][4];
   __shared__ uint32_t s_cnt[2][kGroup];             // kept entries of a step
+  __shared__ float s_none[kGroup];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t b = blockIdx.x;
   const int Hd = p.Hd;
   for (int64_t t = tid; t < p.T; t += blockDim.x) s_x[t] = p.x[b * p.T + t];
   for (int i = tid; i < kRing * kHdMax; i += blockDim.x) (&s_h[0][0])[i] = 0.0f;
+  if (tid < kGroup) s_none[tid] = 0.0f;
   const int64_t groups = (p.T + kGroup - 1) / kGroup;
   __syncthreads();
   if (warp < unit_warps) {
@@ -110,9 +112,11 @@ __global__ void __launch_bounds__(32 * (KP / 2 + kStoreWarps), 2) irnn_forward_k
     float bias = 0.0f, wih = 0.0f;
     if (j < Hd && q == 0) { bias = p.b_ih[j] + p.b_hh[j]; wih = p.W_ih[j]; }
     const bool writer = lane < 8 && j < Hd;
-    const float* x = s_x;
+    // the input enters through the first part; the others read zeros (an infinite input times their zero weight is a NaN)
+    const float* x = q == 0 ? s_x : s_none;
+    const int x_step = q == 0 ? kGroup : 0;
     int left = (int)p.T;
-    for (int g = 0; left > 0; ++g, left -= kGroup, x += kGroup) {
+    for (int g = 0; left > 0; ++g, left -= kGroup, x += x_step) {
       float* h = s_h[(g * kGroup) % kRing];          // the group's first state; the next group's first may be the ring's first
       float* h_next = s_h[(g * kGroup + kGroup) % kRing];
 #pragma unroll

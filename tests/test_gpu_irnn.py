@@ -75,3 +75,23 @@ def test_irnn_step_over_hidden_sizes_and_groups_of_steps(B, T, Hd, C, p):
                             ("dW_ih", ctx.dW_ih, ref.dW_ih), ("db", ctx.db, ref.db), ("db_out", ctx.db_out, ref.db_out)):
         want = np.asarray(want)
         assert np.abs(got.double().cpu().numpy() - want).max() <= 1e-5 * max(np.abs(want).max(), 1e-30), name
+
+
+def test_an_infinite_input_is_not_lost():
+    """x_T = +inf in one row: the hidden units with a positive input weight are +inf, so the loss is not finite; the other
+    row's share of dW_ih and the counts are untouched (their sum is not finite either, as in the oracle)."""
+    import paper_2007_10412_b200 as rad
+    B, T, Hd, C = 2, 5, 40, 4
+    args = list(irnn_inputs(B, T, Hd, C, seed=12, identity=False))
+    args[0] = args[0].copy()
+    args[0][1, T - 1] = np.inf
+    assert (args[2] > 0).any() and (args[2] < 0).any()
+    with np.errstate(all="ignore"):
+        ref = orc.irnn_step(*args, variant="different", p=0.5, seed=6, step0=77)
+    ctx = rad.IRNNStep(B, T, Hd, C, "different", 0.5)
+    ctx(*[torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in args], seed=6, step0=77)
+    torch.cuda.synchronize()
+    assert not np.isfinite(ref.loss) and not np.isfinite(ctx.loss.item())
+    assert ctx.nnz.cpu().numpy()[0] == ref.nnz_steps.sum()
+    # kept units of the last state: those that are infinite make their row of dW_out so
+    assert (np.isfinite(ctx.dW_out.cpu().numpy()) == np.isfinite(ref.dW_out)).all()
