@@ -192,10 +192,19 @@ inline int64_t redrawn_index_bytes(int64_t B, int64_t D) {
   return round_up(ceil_div(B, kTileRows) * ceil_div(D, kTileCols) * kTileWords * 4, 256);
 }
 
+// A CUDA call that fails is reported by the call of this library that made it, and by that one alone: the runtime's last
+// error is taken away with it, or a later check, the caller's own included, would find it again.
 #define RAD_CUDA_TRY(expr)                          \
   do {                                              \
-    cudaError_t e__ = (expr);                       \
-    if (e__ != cudaSuccess) return RAD_ECUDA;       \
+    if ((expr) != cudaSuccess) {                    \
+      (void)cudaGetLastError();                     \
+      return RAD_ECUDA;                             \
+    }                                               \
+  } while (0)
+#define RAD_TRY(expr)                               \
+  do {                                              \
+    const int rc__ = (expr);                        \
+    if (rc__ != RAD_OK) return rc__;                \
   } while (0)
 
 // internal launchers shared across translation units --------------------------------------------
@@ -353,6 +362,7 @@ __device__ __forceinline__ void begin_after_previous() {
   wait_for_previous();
   let_next_start();
 }
+// Every caller passes the code on.
 template <typename... P, typename... Args>
 int launch_with_cluster(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, dim3 cluster, cudaStream_t s, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -367,7 +377,8 @@ int launch_with_cluster(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem
   attr[1].val.clusterDim.x = cluster.x; attr[1].val.clusterDim.y = cluster.y; attr[1].val.clusterDim.z = cluster.z;
   cfg.attrs = attr;
   cfg.numAttrs = cluster.x == 0 ? 1 : 2;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...) == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...));
+  return RAD_OK;
 }
 // without a cluster, or with the one the kernel is compiled for
 template <typename... P, typename... Args>
@@ -382,7 +393,10 @@ bool allow_smem(K kernel, int bytes, std::atomic<uint64_t>& ready) {
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   const uint64_t bit = 1ull << (dev & 63);
   if (dev < 64 && (ready.load(std::memory_order_acquire) & bit) != 0) return true;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
   if (dev < 64) ready.fetch_or(bit, std::memory_order_release);
   return true;
 }

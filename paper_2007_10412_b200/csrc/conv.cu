@@ -519,9 +519,9 @@ int launch_forward_pool(const ConvShape& s, int64_t total, const void* X, const 
   const size_t smem = (size_t)9 * s.Cin * s.Cout * 4;
   count_launch();
   RAD_CUDA_TRY(cudaFuncSetAttribute(conv_forward_pool_kernel<T, kCin>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  launch_kernel(conv_forward_pool_kernel<T, kCin>, (unsigned)ceil_div(total, 256), 256, smem, st, s, static_cast<const T*>(X), static_cast<const T*>(Wt),
-                                                                                       bias, static_cast<T*>(P), relubits);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_TRY(launch_kernel(conv_forward_pool_kernel<T, kCin>, (unsigned)ceil_div(total, 256), 256, smem, st, s, static_cast<const T*>(X), static_cast<const T*>(Wt),
+                                                                                       bias, static_cast<T*>(P), relubits));
+  return RAD_OK;
 }
 }  // namespace
 
@@ -543,10 +543,10 @@ int conv_dz(int dtype, int64_t B, int H, int W, int Cout, const void* dP, const 
   const unsigned grid = (unsigned)ceil_div(B * (H / 2) * (W / 2) * (Cout / 8), 256);
   count_launch();
   if (dtype == RAD_BF16)
-    launch_kernel(conv_dz_kernel<bf16>, grid, 256, 0, st, s, static_cast<const bf16*>(dP), relubits, static_cast<bf16*>(dZ));
+    RAD_TRY(launch_kernel(conv_dz_kernel<bf16>, grid, 256, 0, st, s, static_cast<const bf16*>(dP), relubits, static_cast<bf16*>(dZ)));
   else
-    launch_kernel(conv_dz_kernel<float>, grid, 256, 0, st, s, static_cast<const float*>(dP), relubits, static_cast<float*>(dZ));
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+    RAD_TRY(launch_kernel(conv_dz_kernel<float>, grid, 256, 0, st, s, static_cast<const float*>(dP), relubits, static_cast<float*>(dZ)));
+  return RAD_OK;
 }
 
 int conv_input_grad(int dtype, int64_t B, int H, int W, int Cin, int Cout, const void* dZ, const void* Wt, void* dX,
@@ -557,14 +557,14 @@ int conv_input_grad(int dtype, int64_t B, int H, int W, int Cin, int Cout, const
   count_launch();
   if (dtype == RAD_BF16) {
     RAD_CUDA_TRY(cudaFuncSetAttribute(conv_input_grad_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    launch_kernel(conv_input_grad_kernel<bf16>, grid, 256, smem, st, s, static_cast<const bf16*>(dZ), static_cast<const bf16*>(Wt),
-                                                         static_cast<bf16*>(dX));
+    RAD_TRY(launch_kernel(conv_input_grad_kernel<bf16>, grid, 256, smem, st, s, static_cast<const bf16*>(dZ), static_cast<const bf16*>(Wt),
+                                                         static_cast<bf16*>(dX)));
   } else {
     RAD_CUDA_TRY(cudaFuncSetAttribute(conv_input_grad_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    launch_kernel(conv_input_grad_kernel<float>, grid, 256, smem, st, s, static_cast<const float*>(dZ), static_cast<const float*>(Wt),
-                                                          static_cast<float*>(dX));
+    RAD_TRY(launch_kernel(conv_input_grad_kernel<float>, grid, 256, smem, st, s, static_cast<const float*>(dZ), static_cast<const float*>(Wt),
+                                                          static_cast<float*>(dX)));
   }
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  return RAD_OK;
 }
 
 int64_t conv_weight_grad_workspace(int64_t B, int Cin, int Cout) { return round_up(B * (9 * Cin + 1) * Cout * 4, 256); }
@@ -583,8 +583,8 @@ int launch_first_backward(const ConvFirstParams& p, unsigned grid, size_t smem, 
   static std::atomic<uint64_t> ready[5];
   auto launch = [&](auto kernel, std::atomic<uint64_t>& r) {
     if (!allow_smem(kernel, 160 * 1024, r)) return (int)RAD_ECUDA;
-    launch_kernel(kernel, grid, kFirstThreads, smem, st, p);
-    return cudaGetLastError() == cudaSuccess ? (int)RAD_OK : (int)RAD_ECUDA;
+    RAD_TRY(launch_kernel(kernel, grid, kFirstThreads, smem, st, p));
+    return (int)RAD_OK;
   };
   switch (p.s.Cin) {
     case 1: return launch(conv_first_backward_kernel<T, 1>, ready[1]);
@@ -618,8 +618,8 @@ int conv_first_backward(const rad_store* store, int H, int W, int Cin, int Cout,
   const int rc = store->dtype == RAD_BF16 ? launch_first_backward<bf16>(p, (unsigned)grid, smem, st)
                                           : launch_first_backward<float>(p, (unsigned)grid, smem, st);
   if (rc != RAD_OK) return rc;
-  launch_kernel(conv_sum_rows_kernel, (unsigned)ceil_div(ncell + Cout, 32), 1024, 0, st, p.partial, grid, ncell + Cout, ncell, dW, db);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_TRY(launch_kernel(conv_sum_rows_kernel, (unsigned)ceil_div(ncell + Cout, 32), 1024, 0, st, p.partial, grid, ncell + Cout, ncell, dW, db));
+  return RAD_OK;
 }
 
 int conv_weight_grad(const rad_store* store, int H, int W, int Cin, int Cout, const void* dZ, float* dW, void* workspace,
@@ -641,13 +641,13 @@ int conv_weight_grad(const rad_store* store, int H, int W, int Cin, int Cout, co
   count_launch(2);
   if (store->dtype == RAD_BF16) {
     RAD_CUDA_TRY(cudaFuncSetAttribute(conv_weight_grad_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    launch_kernel(conv_weight_grad_kernel<bf16>, (unsigned)store->B, threads, smem, st, p);
+    RAD_TRY(launch_kernel(conv_weight_grad_kernel<bf16>, (unsigned)store->B, threads, smem, st, p));
   } else {
     RAD_CUDA_TRY(cudaFuncSetAttribute(conv_weight_grad_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    launch_kernel(conv_weight_grad_kernel<float>, (unsigned)store->B, threads, smem, st, p);
+    RAD_TRY(launch_kernel(conv_weight_grad_kernel<float>, (unsigned)store->B, threads, smem, st, p));
   }
-  launch_kernel(conv_sum_rows_kernel, (unsigned)ceil_div(ncell, 32), 1024, 0, st, p.partial, store->B, ncell, ncell, dW, nullptr);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_TRY(launch_kernel(conv_sum_rows_kernel, (unsigned)ceil_div(ncell, 32), 1024, 0, st, p.partial, store->B, ncell, ncell, dW, nullptr));
+  return RAD_OK;
 }
 
 }  // namespace rad

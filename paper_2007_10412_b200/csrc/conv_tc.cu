@@ -427,8 +427,8 @@ int conv_tc_forward_pool(int64_t B, int H, int W, int Cin, int Cout, const void*
   RAD_CUDA_TRY(cudaFuncSetAttribute(conv_tc_kernel<kCvFwd>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCvSmem));
   const int64_t windows = B * (H / 2) * (W / 2);
   count_launch();
-  launch_kernel(conv_tc_kernel<kCvFwd>, (unsigned)ceil_div(windows, 32), kCvThreads, kCvSmem, st, p);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_TRY(launch_kernel(conv_tc_kernel<kCvFwd>, (unsigned)ceil_div(windows, 32), kCvThreads, kCvSmem, st, p));
+  return RAD_OK;
 }
 
 // Shapes the input-gradient kernel takes: as above with the channel counts in each other's roles (K runs over
@@ -448,8 +448,8 @@ int conv_tc_input_grad(int64_t B, int H, int W, int Cin, int Cout, const void* d
   p.dev_status = dev_status; p.wait_limit_ns = wait_limit_ns();
   RAD_CUDA_TRY(cudaFuncSetAttribute(conv_tc_kernel<kCvDx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCvSmem));
   count_launch();
-  launch_kernel(conv_tc_kernel<kCvDx>, (unsigned)ceil_div(B * H * W, kCvM), kCvThreads, kCvSmem, st, p);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_TRY(launch_kernel(conv_tc_kernel<kCvDx>, (unsigned)ceil_div(B * H * W, kCvM), kCvThreads, kCvSmem, st, p));
+  return RAD_OK;
 }
 
 // K blocks of 64 pixels per CTA of the filter-gradient kernel, and the splits that follow from it: enough for three
@@ -477,11 +477,11 @@ int conv_tc_weight_grad(const rad_store* store, int H, int W, int Cin, int Cout,
   RAD_CUDA_TRY(cudaMemsetAsync(dense, 0, (size_t)(B * D * 2), st));
   count_launch();
   if (store->variant == RAD_SAME_SAMPLE) {
-    launch_kernel(densify_same_kernel, (unsigned)std::min<int64_t>(ceil_div(B * store->values_ld, 256), 148 * 16), 256, 0, st, static_cast<const bf16*>(store->values), store->offsets, store->nnz, B, D, store->values_ld, dense);
+    RAD_TRY(launch_kernel(densify_same_kernel, (unsigned)std::min<int64_t>(ceil_div(B * store->values_ld, 256), 148 * 16), 256, 0, st, static_cast<const bf16*>(store->values), store->offsets, store->nnz, B, D, store->values_ld, dense));
   } else {
     const int32_t ncb = (int32_t)ceil_div(D, kTileCols);
     const int64_t nwords = ceil_div(B, kTileRows) * ncb * kBitWords;
-    launch_kernel(densify_different_kernel, (unsigned)std::min<int64_t>(ceil_div(nwords, 256), 148 * 16), 256, 0, st, static_cast<const bf16*>(store->values), store->keepbits, store->offsets, B, D, ncb, store->values_capacity, dense);
+    RAD_TRY(launch_kernel(densify_different_kernel, (unsigned)std::min<int64_t>(ceil_div(nwords, 256), 148 * 16), 256, 0, st, static_cast<const bf16*>(store->values), store->keepbits, store->offsets, B, D, ncb, store->values_capacity, dense));
   }
   ConvTcParams p = {};
   p.B = B; p.H = H; p.W = W; p.Cin = Cin; p.Cout = Cout;
@@ -490,8 +490,7 @@ int conv_tc_weight_grad(const rad_store* store, int H, int W, int Cin, int Cout,
   const int splits = conv_tc_splits(B * H * W, Cin, &p.kblocks_per_split);
   RAD_CUDA_TRY(cudaFuncSetAttribute(conv_tc_kernel<kCvDw>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCvSmem));
   count_launch();
-  launch_kernel(conv_tc_kernel<kCvDw>, dim3((unsigned)ceil_div(9 * Cin, kCvM), (unsigned)splits), kCvThreads, kCvSmem, st, p);
-  RAD_CUDA_TRY(cudaGetLastError());
+  RAD_TRY(launch_kernel(conv_tc_kernel<kCvDw>, dim3((unsigned)ceil_div(9 * Cin, kCvM), (unsigned)splits), kCvThreads, kCvSmem, st, p));
   // the splits' partial sums: column sums of a splits x (9 Cin Cout) matrix, in a fixed order
   const int64_t n = (int64_t)9 * Cin * Cout, held = round_up((int64_t)splits * n * 4, 256);
   return column_sums(RAD_F32, splits, n, partial, n, dW, reinterpret_cast<char*>(partial) + held, column_sums_workspace(splits, n), st);

@@ -391,16 +391,16 @@ int launch_irnn_forward(const RnnParams& p, const PhiloxKeys& ks, size_t smem, c
   const int uw = (int)ceil_div(p.Hd, 8);
   RAD_CUDA_TRY(cudaFuncSetAttribute(irnn_forward_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem, 1024)));
   count_launch();
-  launch_kernel(irnn_forward_kernel<KP>, (unsigned)p.B, 32 * (uw + kStoreWarps), smem, s, p, ks, uw);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_TRY(launch_kernel(irnn_forward_kernel<KP>, (unsigned)p.B, 32 * (uw + kStoreWarps), smem, s, p, ks, uw));
+  return RAD_OK;
 }
 template <int KP>
 int launch_irnn_backward(const RnnParams& p, size_t smem, cudaStream_t s) {
   const int uw = (int)ceil_div(p.Hd, 8);
   RAD_CUDA_TRY(cudaFuncSetAttribute(irnn_backward_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   count_launch();
-  launch_kernel(irnn_backward_kernel<KP>, (unsigned)p.B, 32 * (uw + kListWarps), smem, s, p, uw);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_TRY(launch_kernel(irnn_backward_kernel<KP>, (unsigned)p.B, 32 * (uw + kListWarps), smem, s, p, uw));
+  return RAD_OK;
 }
 // f(std::integral_constant<KP>) for the smallest KP in 8, 16, 20, 24, 28, 32 that holds Hd units
 template <typename F>
@@ -552,7 +552,6 @@ extern "C" int rad_irnn_step(const rad_irnn_desc* d, const float* x, const int32
   if (rc != RAD_OK) return rc;
   const int64_t hh = d->Hd * d->Hd;
   count_launch();
-  launch_kernel(irnn_sum_rows_kernel, (unsigned)ceil_div(hh + 2 * d->Hd, 32), 1024, 0, s, p.part, d->B, hh, d->Hd, dW_hh, dW_ih, db, p.nnz_rows, st.nnz, nnz_out);
-  RAD_CUDA_TRY(cudaGetLastError());
+  RAD_TRY(launch_kernel(irnn_sum_rows_kernel, (unsigned)ceil_div(hh + 2 * d->Hd, 32), 1024, 0, s, p.part, d->B, hh, d->Hd, dW_hh, dW_ih, db, p.nnz_rows, st.nnz, nnz_out));
   return RAD_OK;
 }

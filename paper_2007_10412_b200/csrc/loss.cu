@@ -124,9 +124,9 @@ int launch_xent(const float* logits, int64_t ldl, const int32_t* labels, int64_t
     return launch_with_cluster(xent_small_kernel<T, NV>, dim3(ctas), 1024, 0, dim3(ctas), s, logits, ldl, labels, B, C, dZ, ldz, loss);
   }
   count_launch(2);
-  launch_kernel(xent_rows_kernel<T, NV>, (unsigned)ceil_div(B, 8), 256, 0, s, logits, ldl, labels, B, C, dZ, ldz, rows);
-  launch_kernel(mean_kernel, 1, 1024, 0, s, rows, B, loss);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_TRY(launch_kernel(xent_rows_kernel<T, NV>, (unsigned)ceil_div(B, 8), 256, 0, s, logits, ldl, labels, B, C, dZ, ldz, rows));
+  RAD_TRY(launch_kernel(mean_kernel, 1, 1024, 0, s, rows, B, loss));
+  return RAD_OK;
 }
 template <typename T>
 int launch_xent_of(const float* logits, int64_t ldl, const int32_t* labels, int64_t B, int64_t C, T* dZ, int64_t ldz, float* loss,

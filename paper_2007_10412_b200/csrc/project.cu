@@ -72,10 +72,10 @@ int draw_signs(int dtype, void* out, int64_t D, int64_t k, int64_t ld, uint64_t 
   const int grid = (int)std::min<int64_t>(ceil_div(n, 256), 148 * 16);
   count_launch();
   if (dtype == RAD_BF16)
-    launch_kernel(rademacher_kernel<bf16>, grid, 256, 0, s, p, ks);
+    RAD_TRY(launch_kernel(rademacher_kernel<bf16>, grid, 256, 0, s, p, ks));
   else
-    launch_kernel(rademacher_kernel<float>, grid, 256, 0, s, p, ks);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+    RAD_TRY(launch_kernel(rademacher_kernel<float>, grid, 256, 0, s, p, ks));
+  return RAD_OK;
 }
 
 // the stand-in the same-sample weight-gradient path takes: a B x ld block with all of its columns kept
@@ -115,7 +115,7 @@ int project_forward_store(const void* A, int64_t lda, const rad_store* st, void*
   int rc = draw_signs(st->dtype, workspace, st->D, k, ld, st->seed, st->layer, st->step, s);
   if (rc != RAD_OK) return rc;
   count_launch();
-  launch_kernel(project_meta_kernel, 1, 32, 0, s, nullptr, nullptr, 0, st->nnz, k, st->B);
+  RAD_TRY(launch_kernel(project_meta_kernel, 1, 32, 0, s, nullptr, nullptr, 0, st->nnz, k, st->B));
   // S = A R': B x D times D x ld, stored in the working type
   rc = rad_linear_forward(st->dtype, RAD_ACT_NONE, st->B, st->D, ld, A, lda, workspace, ld, nullptr, st->values, ld,
                           nullptr, 0, nullptr, 0, nullptr, dev_status, stream);
@@ -140,7 +140,7 @@ int project_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_
   int rc = draw_signs(st->dtype, R, st->D, k, ld, st->seed, st->layer, st->step, s);
   if (rc != RAD_OK) return rc;
   count_launch();
-  launch_kernel(project_meta_kernel, (unsigned)std::min<int64_t>(ceil_div(ld, 256), 1024), 256, 0, s, idx, bits, ld, nullptr, k, 0);
+  RAD_TRY(launch_kernel(project_meta_kernel, (unsigned)std::min<int64_t>(ceil_div(ld, 256), 1024), 256, 0, s, idx, bits, ld, nullptr, k, 0));
   // G32 = S^T dZ (ld x H): the dense block of S goes through the same-sample contraction with every column kept
   const rad_store t = as_dense_block(st, idx, bits);
   rc = rad_linear_weight_grad(&t, dZ, ldz, H, G32, H, ws, inner, dev_status, stream);
@@ -150,10 +150,9 @@ int project_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_
   const int grid = (int)std::min<int64_t>(ceil_div(n, 256), 148 * 16);
   count_launch();
   if (st->dtype == RAD_BF16)
-    launch_kernel(scale_convert_kernel<bf16>, grid, 256, 0, s, G32, static_cast<bf16*>(G), n, 1.0f / (float)k);
+    RAD_TRY(launch_kernel(scale_convert_kernel<bf16>, grid, 256, 0, s, G32, static_cast<bf16*>(G), n, 1.0f / (float)k));
   else
-    launch_kernel(scale_convert_kernel<float>, grid, 256, 0, s, G32, static_cast<float*>(G), n, 1.0f / (float)k);
-  if (cudaGetLastError() != cudaSuccess) return RAD_ECUDA;
+    RAD_TRY(launch_kernel(scale_convert_kernel<float>, grid, 256, 0, s, G32, static_cast<float*>(G), n, 1.0f / (float)k));
   // dW_hat = R' G: D x ld times ld x H, float32 out
   return rad_linear_forward(st->dtype, RAD_ACT_NONE, st->D, ld, H, R, ld, G, H, nullptr, nullptr, 0, dW, ldw, nullptr, 0,
                             nullptr, dev_status, stream);

@@ -805,10 +805,9 @@ int simt_forward(int dtype, int act, int64_t B, int64_t D, int64_t H, const void
     const int g = (int)std::min<int64_t>(ceil_div(n, 256), 148 * 16);
     count_launch();
     if (dtype == RAD_BF16)
-      launch_kernel(relu_bits_rows_kernel<bf16>, g, 256, 0, s, static_cast<const bf16*>(out_act), ld_act, B, H, w32, relubits);
+      RAD_TRY(launch_kernel(relu_bits_rows_kernel<bf16>, g, 256, 0, s, static_cast<const bf16*>(out_act), ld_act, B, H, w32, relubits));
     else
-      launch_kernel(relu_bits_rows_kernel<float>, g, 256, 0, s, static_cast<const float*>(out_act), ld_act, B, H, w32, relubits);
-    if (cudaGetLastError() != cudaSuccess) return RAD_ECUDA;
+      RAD_TRY(launch_kernel(relu_bits_rows_kernel<float>, g, 256, 0, s, static_cast<const float*>(out_act), ld_act, B, H, w32, relubits));
   }
   return RAD_OK;
 }

@@ -660,10 +660,9 @@ int launch_store_fill(const StoreParams& p, const PhiloxKeys& ks, int dtype, dou
   }
   count_launch();
   if (dtype == RAD_BF16)
-    launch_kernel(store_different_kernel<bf16, kMaskIndex>, p.ntiles, 256, 0, s, p, ks);
+    RAD_TRY(launch_kernel(store_different_kernel<bf16, kMaskIndex>, p.ntiles, 256, 0, s, p, ks));
   else
-    launch_kernel(store_different_kernel<float, kMaskIndex>, p.ntiles, 256, 0, s, p, ks);
-  RAD_CUDA_TRY(cudaGetLastError());
+    RAD_TRY(launch_kernel(store_different_kernel<float, kMaskIndex>, p.ntiles, 256, 0, s, p, ks));
   return RAD_OK;
 }
 
@@ -680,15 +679,14 @@ int launch_store_different(const StoreParams& p, const PhiloxKeys& ks, int dtype
   count_launch();
   if (p.counts != nullptr) {
     if (dtype == RAD_BF16)
-      launch_kernel(store_different_kernel<bf16, kMaskCounts>, p.ntiles, 256, 0, s, p, ks);
+      RAD_TRY(launch_kernel(store_different_kernel<bf16, kMaskCounts>, p.ntiles, 256, 0, s, p, ks));
     else
-      launch_kernel(store_different_kernel<float, kMaskCounts>, p.ntiles, 256, 0, s, p, ks);
+      RAD_TRY(launch_kernel(store_different_kernel<float, kMaskCounts>, p.ntiles, 256, 0, s, p, ks));
   } else if (dtype == RAD_BF16) {
-    launch_kernel(store_different_kernel<bf16, kMaskDraw>, p.ntiles, 256, 0, s, p, ks);
+    RAD_TRY(launch_kernel(store_different_kernel<bf16, kMaskDraw>, p.ntiles, 256, 0, s, p, ks));
   } else {
-    launch_kernel(store_different_kernel<float, kMaskDraw>, p.ntiles, 256, 0, s, p, ks);
+    RAD_TRY(launch_kernel(store_different_kernel<float, kMaskDraw>, p.ntiles, 256, 0, s, p, ks));
   }
-  RAD_CUDA_TRY(cudaGetLastError());
   return RAD_OK;
 }
 
@@ -721,10 +719,10 @@ int launch_relu_bits(int dtype, const void* A, int64_t lda, int64_t B, int64_t D
   const int g2 = (int)std::min<int64_t>(ceil_div(n, 256), 148 * 16);
   count_launch();
   if (dtype == RAD_BF16)
-    launch_kernel(relu_bits_kernel<bf16>, g2, 256, 0, s, static_cast<const bf16*>(A), lda, B, D, w32, relubits);
+    RAD_TRY(launch_kernel(relu_bits_kernel<bf16>, g2, 256, 0, s, static_cast<const bf16*>(A), lda, B, D, w32, relubits));
   else
-    launch_kernel(relu_bits_kernel<float>, g2, 256, 0, s, static_cast<const float*>(A), lda, B, D, w32, relubits);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+    RAD_TRY(launch_kernel(relu_bits_kernel<float>, g2, 256, 0, s, static_cast<const float*>(A), lda, B, D, w32, relubits));
+  return RAD_OK;
 }
 }  // namespace rad
 
@@ -940,14 +938,13 @@ extern "C" int rad_linear_forward_store(const void* A, int64_t lda, const rad_st
         if (smem > 48 * 1024)
           RAD_CUDA_TRY(cudaFuncSetAttribute(fixed_counts_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)kMaxCountsRowBytes));
-        launch_kernel(fixed_counts_kernel, (unsigned)ceil_div(st->B, rows), 128, smem, s, rp, ks, rows, words);
+        RAD_TRY(launch_kernel(fixed_counts_kernel, (unsigned)ceil_div(st->B, rows), 128, smem, s, rp, ks, rows, words));
       } else {
         if (rp.ldc > 48 * 1024)
           RAD_CUDA_TRY(cudaFuncSetAttribute(replace_counts_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)kMaxCountsRowBytes));
-        launch_kernel(replace_counts_kernel, (unsigned)st->B, 128, (size_t)rp.ldc, s, rp, ks);
+        RAD_TRY(launch_kernel(replace_counts_kernel, (unsigned)st->B, 128, (size_t)rp.ldc, s, rp, ks));
       }
-      RAD_CUDA_TRY(cudaGetLastError());
       p.counts = rp.counts; p.ldc = rp.ldc;
     }
     return launch_store_different(p, ks, st->dtype, T, s);
@@ -971,9 +968,9 @@ extern "C" int rad_linear_forward_store(const void* A, int64_t lda, const rad_st
     r.hist = reinterpret_cast<uint32_t*>(static_cast<char*>(workspace) + 256);
     r.colscale = reinterpret_cast<float*>(static_cast<char*>(workspace) + 256 + 4 * st->D);
     colscale = r.colscale;
-    launch_kernel(same_replace_mask_kernel, 1, 1024, 0, s, p, r, ks);
+    RAD_TRY(launch_kernel(same_replace_mask_kernel, 1, 1024, 0, s, p, r, ks));
   } else {
-    launch_kernel(same_mask_kernel, 1, 1024, 0, s, p, ks);
+    RAD_TRY(launch_kernel(same_mask_kernel, 1, 1024, 0, s, p, ks));
   }
   // Dense masks (most 32-byte sectors of a row hold a kept column) and calls that also want the ReLU bits take
   // the row-staging kernel; sparse masks without ReLU bits keep the gather that skips the sectors it does not need.
@@ -995,30 +992,28 @@ extern "C" int rad_linear_forward_store(const void* A, int64_t lda, const rad_st
       const int grid_r = (int)std::min<int64_t>(ceil_div(st->B, warps), sms);
       if (st->dtype == RAD_BF16) {
         RAD_CUDA_TRY(cudaFuncSetAttribute(same_gather_rows_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_budget));
-        launch_kernel(same_gather_rows_kernel<bf16>, grid_r, 256, smem, s, p, st->relubits, w32, warps);
+        RAD_TRY(launch_kernel(same_gather_rows_kernel<bf16>, grid_r, 256, smem, s, p, st->relubits, w32, warps));
       } else {
         RAD_CUDA_TRY(cudaFuncSetAttribute(same_gather_rows_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_budget));
-        launch_kernel(same_gather_rows_kernel<float>, grid_r, 256, smem, s, p, st->relubits, w32, warps);
+        RAD_TRY(launch_kernel(same_gather_rows_kernel<float>, grid_r, 256, smem, s, p, st->relubits, w32, warps));
       }
-      RAD_CUDA_TRY(cudaGetLastError());
       return RAD_OK;
     }
   }
   const int grid = (int)std::min<int64_t>(ceil_div(st->B, 8), 148 * 8);
   if (st->dtype == RAD_BF16)
-    launch_kernel(same_gather_kernel<bf16>, grid, 256, 0, s, p, colscale);
+    RAD_TRY(launch_kernel(same_gather_kernel<bf16>, grid, 256, 0, s, p, colscale));
   else
-    launch_kernel(same_gather_kernel<float>, grid, 256, 0, s, p, colscale);
+    RAD_TRY(launch_kernel(same_gather_kernel<float>, grid, 256, 0, s, p, colscale));
   if (st->relubits != nullptr) {
     const int64_t n = st->B * w32;
     const int g2 = (int)std::min<int64_t>(ceil_div(n, 256), 148 * 16);
     count_launch();
     if (st->dtype == RAD_BF16)
-      launch_kernel(relu_bits_kernel<bf16>, g2, 256, 0, s, static_cast<const bf16*>(A), lda, st->B, st->D, w32, st->relubits);
+      RAD_TRY(launch_kernel(relu_bits_kernel<bf16>, g2, 256, 0, s, static_cast<const bf16*>(A), lda, st->B, st->D, w32, st->relubits));
     else
-      launch_kernel(relu_bits_kernel<float>, g2, 256, 0, s, static_cast<const float*>(A), lda, st->B, st->D, w32, st->relubits);
+      RAD_TRY(launch_kernel(relu_bits_kernel<float>, g2, 256, 0, s, static_cast<const float*>(A), lda, st->B, st->D, w32, st->relubits));
   }
-  RAD_CUDA_TRY(cudaGetLastError());
   return RAD_OK;
 }
 
@@ -1038,7 +1033,8 @@ int static_scratch_address(void** out) {
   if (dev < 0 || dev >= kMaxDevices) return RAD_EUNSUPPORTED;
   if (g_static_scratch_ptr[dev] == nullptr) {
     void* ptr = nullptr;
-    if (cudaGetSymbolAddress(&ptr, g_static_store_scratch) != cudaSuccess || ptr == nullptr) return RAD_ECUDA;
+    RAD_CUDA_TRY(cudaGetSymbolAddress(&ptr, g_static_store_scratch));
+    if (ptr == nullptr) return RAD_ECUDA;
     g_static_scratch_ptr[dev] = ptr;
   }
   *out = g_static_scratch_ptr[dev];

@@ -154,8 +154,8 @@ int launch_offsets_scan(uint32_t* offsets, int64_t ntiles, int64_t* nnz, int64_t
   IndexParams p = {};
   p.ntiles = (int32_t)ntiles; p.offsets = offsets; p.nnz = nnz; p.capacity = capacity; p.dev_status = dev_status;
   count_launch();
-  launch_kernel(offsets_scan_kernel, 1, 1024, 0, s, p, ((uintptr_t)offsets & 15) == 0 ? 1 : 0);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_TRY(launch_kernel(offsets_scan_kernel, 1, 1024, 0, s, p, ((uintptr_t)offsets & 15) == 0 ? 1 : 0));
+  return RAD_OK;
 }
 
 // Index part (keep bits, row offsets, tile offsets, nnz) of a different-sample Bernoulli store.
@@ -174,8 +174,7 @@ int launch_store_index(const rad_store* st, bool check_capacity, int32_t* dev_st
   const int grid = (int)std::min<int64_t>(ceil_div(p.ntiles, kIndexWarps), 148 * 12);
   if (st->law == RAD_LAW_FIXED) return launch_fixed_index(st, check_capacity, dev_status, s);
   count_launch();
-  launch_kernel(store_index_kernel, grid, 32 * kIndexWarps, 0, s, p, ks);
-  if (cudaGetLastError() != cudaSuccess) return RAD_ECUDA;
+  RAD_TRY(launch_kernel(store_index_kernel, grid, 32 * kIndexWarps, 0, s, p, ks));
   return launch_offsets_scan(p.offsets, p.ntiles, p.nnz, p.capacity, dev_status, s);
 }
 

@@ -600,8 +600,7 @@ int launch_typed(const StoreParams& p, const PhiloxKeys& ks, const CUtensorMap& 
   const int64_t nchunks = ceil_div(p.ntiles, kChunk);
   const int grid = (int)std::min<int64_t>(nchunks, grid_cap[dev]);
   count_launch();
-  launch_kernel(kernel, grid, kPipeThreads, smem, s, p, ks, map);
-  RAD_CUDA_TRY(cudaGetLastError());
+  RAD_TRY(launch_kernel(kernel, grid, kPipeThreads, smem, s, p, ks, map));
   return RAD_OK;
 }
 

@@ -393,12 +393,12 @@ int launch_rows_fixed(const RowsParams& p, int dtype, uint64_t seed, int64_t sme
   count_launch();
   if (dtype == RAD_BF16) {
     RAD_CUDA_TRY(cudaFuncSetAttribute(rows_fixed_kernel<bf16, kRowsOut>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmemBudget));
-    launch_kernel(rows_fixed_kernel<bf16, kRowsOut>, grid, 32 * kRowsWarps, (size_t)smem, s, p, ks);
+    RAD_TRY(launch_kernel(rows_fixed_kernel<bf16, kRowsOut>, grid, 32 * kRowsWarps, (size_t)smem, s, p, ks));
   } else {
     RAD_CUDA_TRY(cudaFuncSetAttribute(rows_fixed_kernel<float, kRowsOut>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmemBudget));
-    launch_kernel(rows_fixed_kernel<float, kRowsOut>, grid, 32 * kRowsWarps, (size_t)smem, s, p, ks);
+    RAD_TRY(launch_kernel(rows_fixed_kernel<float, kRowsOut>, grid, 32 * kRowsWarps, (size_t)smem, s, p, ks));
   }
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  return RAD_OK;
 }
 
 }  // namespace
@@ -465,8 +465,7 @@ int launch_replace_index(const rad_store* st, uint32_t* extras, bool check_capac
   const PhiloxKeys ks = philox_expand_key(st->seed);
   count_launch();
   RAD_CUDA_TRY(cudaFuncSetAttribute(replace_index_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmemBudget));
-  launch_kernel(replace_index_kernel, (int)std::min<int64_t>(slabs, 148 * 8), 32 * kRowsWarps, (size_t)smem, s, p, ks, extras, (int32_t)ld);
-  if (cudaGetLastError() != cudaSuccess) return RAD_ECUDA;
+  RAD_TRY(launch_kernel(replace_index_kernel, (int)std::min<int64_t>(slabs, 148 * 8), 32 * kRowsWarps, (size_t)smem, s, p, ks, extras, (int32_t)ld));
   return launch_offsets_scan(st->offsets, slabs * p.ncb, st->nnz, check_capacity ? st->values_capacity : -1, dev_status, s);
 }
 
@@ -480,12 +479,12 @@ int launch_replace_extras(const void* A, int64_t lda, const rad_store* st, const
   const int grid = (int)std::min<int64_t>(ceil_div(st->B, 8), 148 * 64);   // short dependent chains: many warps in flight
   count_launch();
   if (st->dtype == RAD_BF16)
-    launch_kernel(replace_extras_kernel<bf16>, grid, 256, 0, s, static_cast<const bf16*>(A), lda, st->B, ncb, extras, (int32_t)ld, st->keepbits,
-                                                     st->offsets, static_cast<bf16*>(st->values), st->values_capacity, scale);
+    RAD_TRY(launch_kernel(replace_extras_kernel<bf16>, grid, 256, 0, s, static_cast<const bf16*>(A), lda, st->B, ncb, extras, (int32_t)ld, st->keepbits,
+                                                     st->offsets, static_cast<bf16*>(st->values), st->values_capacity, scale));
   else
-    launch_kernel(replace_extras_kernel<float>, grid, 256, 0, s, static_cast<const float*>(A), lda, st->B, ncb, extras, (int32_t)ld, st->keepbits,
-                                                      st->offsets, static_cast<float*>(st->values), st->values_capacity, scale);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+    RAD_TRY(launch_kernel(replace_extras_kernel<float>, grid, 256, 0, s, static_cast<const float*>(A), lda, st->B, ncb, extras, (int32_t)ld, st->keepbits,
+                                                      st->offsets, static_cast<float*>(st->values), st->values_capacity, scale));
+  return RAD_OK;
 }
 
 // Values of the tile-major store `tiles` (index part in place) from the static-shape store `rows` of the same key.
@@ -497,19 +496,19 @@ int rows_to_tiles(const rad_store* rows, const rad_store* tiles, int32_t* dev_st
   const int grid_t = (int)std::min<int64_t>(ceil_div(ntiles, 256), 148 * 8);
   count_launch(2);
   if (rows->dtype == RAD_BF16) {
-    launch_kernel(rows_to_tiles_kernel<bf16>, grid, 256, 0, s, static_cast<const bf16*>(rows->values), reinterpret_cast<const uint16_t*>(rows->keepbits),
+    RAD_TRY(launch_kernel(rows_to_tiles_kernel<bf16>, grid, 256, 0, s, static_cast<const bf16*>(rows->values), reinterpret_cast<const uint16_t*>(rows->keepbits),
                                                     rows->B, k, rows->values_ld, ncb, tiles->keepbits, tiles->offsets,
-                                                    static_cast<bf16*>(tiles->values), tiles->values_capacity, dev_status);
-    launch_kernel(tile_padding_kernel<bf16>, grid_t, 256, 0, s, tiles->keepbits, tiles->offsets, ntiles, static_cast<bf16*>(tiles->values),
-                                                     tiles->values_capacity);
+                                                    static_cast<bf16*>(tiles->values), tiles->values_capacity, dev_status));
+    RAD_TRY(launch_kernel(tile_padding_kernel<bf16>, grid_t, 256, 0, s, tiles->keepbits, tiles->offsets, ntiles, static_cast<bf16*>(tiles->values),
+                                                     tiles->values_capacity));
   } else {
-    launch_kernel(rows_to_tiles_kernel<float>, grid, 256, 0, s, static_cast<const float*>(rows->values), reinterpret_cast<const uint16_t*>(rows->keepbits),
+    RAD_TRY(launch_kernel(rows_to_tiles_kernel<float>, grid, 256, 0, s, static_cast<const float*>(rows->values), reinterpret_cast<const uint16_t*>(rows->keepbits),
                                                      rows->B, k, rows->values_ld, ncb, tiles->keepbits, tiles->offsets,
-                                                     static_cast<float*>(tiles->values), tiles->values_capacity, dev_status);
-    launch_kernel(tile_padding_kernel<float>, grid_t, 256, 0, s, tiles->keepbits, tiles->offsets, ntiles, static_cast<float*>(tiles->values),
-                                                      tiles->values_capacity);
+                                                     static_cast<float*>(tiles->values), tiles->values_capacity, dev_status));
+    RAD_TRY(launch_kernel(tile_padding_kernel<float>, grid_t, 256, 0, s, tiles->keepbits, tiles->offsets, ntiles, static_cast<float*>(tiles->values),
+                                                      tiles->values_capacity));
   }
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  return RAD_OK;
 }
 
 }  // namespace rad

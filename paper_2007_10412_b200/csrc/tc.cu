@@ -1206,7 +1206,7 @@ int launch_pair(const TcParams& p, const CUtensorMap& ta, const CUtensorMap& tb,
   // (SM pairs that can host a cluster; fewer than half the SM count on some parts).
   static int resident_pairs = 0;
   if (resident_pairs == 0) {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return RAD_ECUDA;
+    RAD_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (num_sms() / 2));
     cfg.blockDim = dim3(threads2(kEpiWarps2));
@@ -1225,8 +1225,8 @@ int launch_pair(const TcParams& p, const CUtensorMap& ta, const CUtensorMap& tb,
   }
   const int pairs = (int)std::max<int64_t>(1, std::min<int64_t>(max_units, resident_pairs));
   count_launch();
-  launch_kernel(kernel, 2 * pairs, threads2(kEpiWarps2), smem, s, p, ta, tb);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_TRY(launch_kernel(kernel, 2 * pairs, threads2(kEpiWarps2), smem, s, p, ta, tb));
+  return RAD_OK;
 }
 
 int launch_sparse_pair(const TcParams& p, const CUtensorMap& tb, int64_t max_units, cudaStream_t s) {
@@ -1235,14 +1235,13 @@ int launch_sparse_pair(const TcParams& p, const CUtensorMap& tb, int64_t max_uni
   if (smem > 227 * 1024 || p.num_stages > kSpMaxStages || p.comp_depth > 8) return RAD_EUNSUPPORTED;
   static int resident_pairs = 0;
   if (resident_pairs == 0) {
-    if (cudaFuncSetAttribute(tc_sparse_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
-      return RAD_ECUDA;
+    RAD_CUDA_TRY(cudaFuncSetAttribute(tc_sparse_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     resident_pairs = resident_pairs_of(tc_sparse_pair_kernel, kSpThreads, 227 * 1024);
   }
   const int pairs = (int)std::max<int64_t>(1, std::min<int64_t>(max_units, resident_pairs));
   count_launch();
-  launch_kernel(tc_sparse_pair_kernel, 2 * pairs, kSpThreads, smem, s, p, tb);
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  RAD_TRY(launch_kernel(tc_sparse_pair_kernel, 2 * pairs, kSpThreads, smem, s, p, tb));
+  return RAD_OK;
 }
 
 // Columns of an output tile of the forward pass and the input gradient: the narrowest of 64, 128 and 256 with which
@@ -1363,9 +1362,9 @@ int tc_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, 
     const int64_t work = rows * (H / 4);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(work, 256), 148 * 16));
     count_launch();
-    launch_kernel(dw_reduce_kernel, grid, 256, 0, s, p.partial, d.partial_rows, d.splits, rows, p.N_dev, H, p.row_idx, dW, ldw);
+    RAD_TRY(launch_kernel(dw_reduce_kernel, grid, 256, 0, s, p.partial, d.partial_rows, d.splits, rows, p.N_dev, H, p.row_idx, dW, ldw));
   }
-  return cudaGetLastError() == cudaSuccess ? RAD_OK : RAD_ECUDA;
+  return RAD_OK;
 }
 
 }  // namespace rad

@@ -1,0 +1,71 @@
+// Stand-in for the CUDA runtime, linked with the library's objects for tests of its host side on a machine without a
+// GPU: one sm_100 device, launches that are recorded and do nothing, and one of them that fails when asked to.
+#include <cuda_runtime_api.h>
+
+#include <map>
+#include <string>
+#include <vector>
+
+namespace {
+struct Launch { std::string kernel; unsigned dims[8]; };       // grid, block, shared memory, CTAs of a cluster
+std::vector<Launch> launches;
+std::map<const void*, std::string> names;
+int fail_at = -1;
+cudaError_t last_error = cudaSuccess;
+alignas(256) char device_symbol[256];
+
+cudaError_t set(cudaError_t e) { if (e != cudaSuccess) last_error = e; return e; }
+cudaError_t launch(const void* f, dim3 g, dim3 b, size_t smem, unsigned cluster) {
+  const bool fails = (int)launches.size() == fail_at;
+  launches.push_back({names[f], {g.x, g.y, g.z, b.x, b.y, b.z, (unsigned)smem, cluster}});
+  const bool bad = g.x == 0 || g.x > 0x7fffffffu || g.y == 0 || g.y > 65535 || g.z == 0 || g.z > 65535 || b.x * b.y * b.z > 1024 ||
+                   b.x * b.y * b.z == 0 || smem > 227 * 1024;
+  return set(fails || bad ? cudaErrorInvalidConfiguration : cudaSuccess);
+}
+int encode_tiled(...) { return 0; }
+}  // namespace
+
+extern "C" {
+// ---- for the tests ----
+void fake_reset(int which_fails) { launches.clear(); fail_at = which_fails; last_error = cudaSuccess; }
+int fake_launches() { return (int)launches.size(); }
+int fake_last_error() { return (int)last_error; }
+const char* fake_kernel(int i) { return launches[i].kernel.c_str(); }
+void fake_dims(int i, unsigned* out) { for (int k = 0; k < 8; ++k) out[k] = launches[i].dims[k]; }
+
+// ---- the runtime ----
+void** __cudaRegisterFatBinary(void*) { static void* handle; return &handle; }
+void __cudaRegisterFatBinaryEnd(void**) {}
+void __cudaUnregisterFatBinary(void**) {}
+void __cudaRegisterFunction(void**, const char* host, char*, const char* device, int, uint3*, uint3*, dim3*, dim3*, int*) { names[host] = device; }
+void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
+static thread_local struct { dim3 g, b; size_t s; void* st; } pushed;
+unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t s, struct CUstream_st* st) { pushed = {g, b, s, st}; return 0; }
+cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* s, void* st) {
+  *g = pushed.g; *b = pushed.b; *s = pushed.s; *static_cast<void**>(st) = pushed.st;
+  return cudaSuccess;
+}
+cudaError_t cudaLaunchKernel(const void* f, dim3 g, dim3 b, void**, size_t s, cudaStream_t) { return launch(f, g, b, s, 1); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
+  unsigned cluster = 1;
+  for (unsigned i = 0; i < c->numAttrs; ++i)
+    if (c->attrs[i].id == cudaLaunchAttributeClusterDimension) cluster = c->attrs[i].val.clusterDim.x * c->attrs[i].val.clusterDim.y;
+  return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, cluster);
+}
+cudaError_t cudaGetLastError() { const cudaError_t e = last_error; last_error = cudaSuccess; return e; }
+cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
+  *v = a == cudaDevAttrComputeCapabilityMajor ? 10 : a == cudaDevAttrMultiProcessorCount ? 148 : 0;
+  return cudaSuccess;
+}
+cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaGetDriverEntryPoint(const char*, void** fn, unsigned long long, cudaDriverEntryPointQueryResult* r) {
+  *fn = reinterpret_cast<void*>(encode_tiled);
+  if (r != nullptr) *r = cudaDriverEntryPointSuccess;
+  return cudaSuccess;
+}
+cudaError_t cudaGetSymbolAddress(void** p, const void*) { *p = device_symbol; return cudaSuccess; }
+cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) { *n = 2; return cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t*) { *n = 74; return cudaSuccess; }
+}

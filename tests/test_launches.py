@@ -1,0 +1,149 @@
+"""The library's host side against a stand-in for the CUDA runtime (fake_cudart.cpp): launches are recorded and do
+nothing, and one of them fails when asked to.  No GPU."""
+import ctypes as C
+import os
+import re
+import subprocess
+
+import pytest
+import torch
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    """The binding on the library's objects linked with the stand-in; tensors are host memory that nobody touches."""
+    from paper_2007_10412_b200 import binding, build
+    build.build()
+    path = str(tmp_path_factory.mktemp("fake") / "librad_fake.so")
+    objs = [os.path.join(build.OBJ, s.replace(".cu", ".o")) for s in build.SOURCES]
+    subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-std=c++17", "-I/usr/local/cuda/include", "-Wl,-Bsymbolic", "-o", path,
+                    os.path.join(HERE, "fake_cudart.cpp")] + objs + ["-ldl"], check=True)
+    saved = binding._lib, binding.LIB_PATH, binding._stream
+    binding._lib, binding.LIB_PATH, binding._stream = None, path, lambda: None
+    L = binding.lib()
+    L.fake_kernel.restype = C.c_char_p
+    yield binding
+    binding._lib, binding.LIB_PATH, binding._stream = saved
+
+
+def _aligned(nbytes):
+    t = torch.empty(nbytes + 256, dtype=torch.uint8)
+    return t[(-t.data_ptr()) % 256:][:nbytes]
+
+
+def _launches(b):
+    """(kernel, grid x, y, z, block x, y, z, dynamic shared memory, CTAs of a cluster) of every launch since the reset."""
+    out = []
+    for i in range(b.lib().fake_launches()):
+        d = (C.c_uint * 8)()
+        b.lib().fake_dims(i, d)
+        out.append((b.lib().fake_kernel(i).decode(),) + tuple(d))
+    return out
+
+
+def _mlp(b, dims, B, dtype, act, variant, law="bernoulli"):
+    ctx = b.MLPStep(dims, B, dtype, act, variant, 0.2, device="cpu", law=law)
+    ctx.workspace = _aligned(ctx.workspace.numel())
+    tdt = torch.float32 if dtype == "f32" else torch.bfloat16
+    X, y = torch.empty(B, dims[0], dtype=tdt), torch.empty(B, dtype=torch.int32)
+    Ws = [torch.empty(dims[l], dims[l + 1], dtype=tdt) for l in range(len(dims) - 1)]
+    return lambda: ctx(X, y, Ws, [None] * len(Ws))
+
+
+def _irnn(b, B, T, Hd, variant="different"):
+    ctx = b.IRNNStep(B, T, Hd, 5, variant, 0.2, device="cpu")
+    ctx.workspace = _aligned(ctx.workspace.numel())
+    f = lambda *s: torch.empty(*s)
+    args = [f(B, T), torch.empty(B, dtype=torch.int32), f(Hd), f(Hd), f(Hd, Hd), f(Hd), f(Hd, 5), f(5)]
+    return lambda: ctx(*args)
+
+
+def _cnn(b, B, hw, cin, channels, fc, dtype, variant):
+    ctx = b.CNNStep(B, hw, cin, channels, fc, dtype, variant, 0.2, device="cpu")
+    ctx.workspace = _aligned(ctx.workspace.numel())
+    tdt = torch.float32 if dtype == "f32" else torch.bfloat16
+    cs, fs = [cin] + list(channels), [t.shape[0] for t in ctx.dfc_W] + [fc[-1]]
+    cW = [torch.empty(3, 3, cs[l], cs[l + 1], dtype=tdt) for l in range(len(channels))]
+    fW = [torch.empty(fs[l], fs[l + 1], dtype=tdt) for l in range(len(fc))]
+    X, y = torch.empty(B, hw, hw, cin, dtype=tdt), torch.empty(B, dtype=torch.int32)
+    return lambda: ctx(X, y, cW, [None] * len(cW), fW, [None] * len(fW))
+
+
+def _store(b, variant, dtype, B, D, p=0.2, law="bernoulli", relu_bits=True):
+    st = b.Store(variant, dtype, B, D, p, relu_bits=relu_bits, device="cpu", law=law)
+    st.workspace = _aligned(max(st.workspace.numel(), 256))
+    return st
+
+
+def _store_and_grad(b, variant, dtype, B, D, H, law="bernoulli"):
+    st = _store(b, variant, dtype, B, D, law=law, relu_bits=variant not in ("project", "rows"))
+    tdt = torch.float32 if dtype == "f32" else torch.bfloat16
+    A, dZ, dW = torch.empty(B, D, dtype=tdt), torch.empty(B, H, dtype=tdt), torch.empty(D, H)
+    ws = _aligned(max(256, b.rad_weight_grad_workspace(st, H)))
+
+    def call():
+        b.rad_linear_forward_store(A, st)
+        b.rad_linear_weight_grad(st, dZ, dW, ws)
+    return call
+
+
+def _input_grad(b, B, D, H, dtype, db=True, dx=True):
+    tdt = torch.float32 if dtype == "f32" else torch.bfloat16
+    dZ, W = torch.empty(B, H, dtype=tdt), torch.empty(D, H, dtype=tdt)
+    out, d = torch.empty(B, D, dtype=tdt) if dx else None, torch.empty(H) if db else None
+    ws = _aligned(b.rad_input_grad_workspace(B, H))
+    return lambda: b.rad_linear_input_grad(dZ, W, dZ_prev=out, db=d, workspace=ws)
+
+
+def _xent(b, B, Cn):
+    z, y, loss, dz = torch.empty(B, Cn), torch.empty(B, dtype=torch.int32), torch.empty(1), torch.empty(B, Cn)
+    return lambda: b.rad_softmax_xent(z, y, loss, dz)
+
+
+CALLS = {
+    "mlp f32 different": lambda b: _mlp(b, (40, 33, 20, 7), 50, "f32", "relu", "different"),
+    "mlp f32 same": lambda b: _mlp(b, (40, 33, 20, 7), 50, "f32", "relu", "same"),
+    "mlp f32 projected": lambda b: _mlp(b, (40, 33, 20, 7), 50, "f32", "relu", "project"),
+    "mlp f32 with replacement": lambda b: _mlp(b, (40, 33, 20, 7), 50, "f32", "relu", "different", "replace"),
+    "mlp f32 same with replacement": lambda b: _mlp(b, (40, 33, 20, 7), 50, "f32", "relu", "same", "replace"),
+    "mlp bf16 different": lambda b: _mlp(b, (256, 320, 136, 64), 200, "bf16", "gelu", "different"),
+    "mlp bf16 fixed count": lambda b: _mlp(b, (256, 320, 136, 64), 200, "bf16", "relu", "different", "fixed"),
+    "mlp bf16 with replacement": lambda b: _mlp(b, (256, 320, 136, 64), 200, "bf16", "relu", "different", "replace"),
+    "mlp bf16 redrawn": lambda b: _mlp(b, (256, 320, 136, 64), 200, "bf16", "relu", "redrawn"),
+    "mlp bf16 same": lambda b: _mlp(b, (256, 320, 136, 64), 200, "bf16", "relu", "same"),
+    "irnn": lambda b: _irnn(b, 5, 9, 40),
+    "irnn same": lambda b: _irnn(b, 5, 9, 100, "same"),
+    "cnn f32": lambda b: _cnn(b, 6, 16, 3, (8, 16), (12, 5), "f32", "different"),
+    "cnn f32, five input channels": lambda b: _cnn(b, 6, 16, 5, (8, 16), (12, 5), "f32", "same"),
+    "cnn bf16": lambda b: _cnn(b, 6, 16, 3, (16, 32), (16, 8), "bf16", "different"),
+    "cnn bf16 same": lambda b: _cnn(b, 6, 16, 16, (16, 32), (16, 8), "bf16", "same"),
+    "rows store and gradient": lambda b: _store_and_grad(b, "rows", "bf16", 100, 256, 64, "fixed"),
+    "dense store": lambda b: _store_and_grad(b, "same", "bf16", 3000, 512, 64),
+    "split gradient": lambda b: _store_and_grad(b, "different", "bf16", 8192, 256, 512),
+    "input gradient f32": lambda b: _input_grad(b, 90, 50, 33, "f32"),
+    "input gradient bf16": lambda b: _input_grad(b, 128, 256, 64, "bf16"),
+    "bias gradient in two launches": lambda b: _input_grad(b, 200000, 8, 16, "bf16", dx=False),
+    "loss": lambda b: _xent(b, 100, 10),
+    "loss of many rows": lambda b: _xent(b, 3000, 10),
+}
+
+
+@pytest.mark.parametrize("name", CALLS)
+def test_a_launch_that_fails_is_reported_once_by_the_call_that_made_it(fake, name):
+    """Every launch of a call in turn fails: the call says so, and leaves no error behind for the next check of the runtime's
+    last error (the next call of the library, or the caller's own)."""
+    call = CALLS[name](fake)
+    fake.lib().fake_reset(-1)
+    call()
+    n = fake.lib().fake_launches()
+    assert n > 0 and fake.lib().fake_last_error() == 0
+    for k in range(n):
+        fake.lib().fake_reset(k)
+        with pytest.raises(fake.RadError, match="CUDA call failed"):
+            call()
+        assert fake.lib().fake_last_error() == 0, _launches(fake)[k][0]
+    fake.lib().fake_reset(-1)
+    call()
+    assert fake.lib().fake_launches() == n
