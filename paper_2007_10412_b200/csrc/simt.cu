@@ -873,7 +873,7 @@ int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H
     }
     const int g = (int)std::min<int64_t>(ceil_div(st->D * H, 256), 148 * 16);
     count_launch();
-    launch_kernel(zero_rows_kernel, g, 256, 0, s, dW, ldw, st->D, H);
+    RAD_TRY(launch_kernel(zero_rows_kernel, g, 256, 0, s, dW, ldw, st->D, H));
     return launch_gemm<kEpiScatterRows>(st->dtype, p, std::max<int64_t>(p.M, 1), s);
   }
   const bool low = st->dtype == RAD_BF16;

@@ -147,3 +147,19 @@ def test_a_launch_that_fails_is_reported_once_by_the_call_that_made_it(fake, nam
     fake.lib().fake_reset(-1)
     call()
     assert fake.lib().fake_launches() == n
+
+
+def test_rows_of_dw_that_were_not_kept_are_zeroed_or_the_call_fails(fake):
+    """A same-sample dW of so many tiles that scatter and zeros need a launch each (2^31 - 2 tiles of 64 x 64, which with the CTAs
+    for the zeros beside them are more than a grid can have): the failure of either launch is the call's."""
+    b = fake
+    D, H = 49981 * 64, 42966 * 64
+    st = b.rad_store(b.VARIANTS["same"], b.DTYPES["f32"], 1, D, 0.5, 0, 0, 0, 256, D, D, 256, 256, 256, None, 0)
+    call = lambda: b.lib().rad_linear_weight_grad(C.byref(st), C.c_void_p(256), H, H, C.c_void_p(256), H, None, 0, None, None)
+    b.lib().fake_reset(-1)
+    assert call() == 0
+    names = [l[0] for l in _launches(b)]
+    assert len(names) == 2 and "zero_rows" in names[0]
+    for k in range(2):
+        b.lib().fake_reset(k)
+        assert call() == -3 and b.lib().fake_last_error() == 0
