@@ -514,10 +514,12 @@ extern "C" int rad_irnn_step(const rad_irnn_desc* d, const float* x, const int32
   p.dev_status = dev_status;
   const PhiloxKeys ks = philox_expand_key(d->seed);
   const size_t smem_f = (size_t)d->T * 4;
-  const int64_t w32s = ceil_div(d->Hd, 32);
-  const size_t smem_b = (size_t)((d->T + 3) & ~(int64_t)3) * 4 + (size_t)d->Hd * (size_t)((d->Hd + 3) & ~(int64_t)3) * 4 +
-                        (size_t)d->T * (2 * w32s + 1) * 4;
-  if (smem_f > 200 * 1024 || smem_b > 200 * 1024) return RAD_ELIMIT;
+  // Backward, per row: inputs, the share of dW_hh (rows padded to 16 bytes), keep bits, derivative bits and offsets.  The
+  // longest sequence is the one that fits 200 KB with rows of Hd + 1 floats: the padding takes at most 2 Hd floats more, and
+  // with the 10 KB of static arrays that is still below the 227 KB of a CTA.
+  const size_t row = (size_t)((d->T + 3) & ~(int64_t)3) * 4 + (size_t)d->T * (2 * (size_t)p.w32 + 1) * 4;
+  const size_t smem_b = row + (size_t)d->Hd * (size_t)((d->Hd + 3) & ~(int64_t)3) * 4;
+  if (smem_f > 200 * 1024 || row + (size_t)((d->Hd * (d->Hd + 1) + 3) & ~(int64_t)3) * 4 > 200 * 1024) return RAD_ELIMIT;
   rc = with_parts(p.Hd, [&](auto kp) { return launch_irnn_forward<decltype(kp)::value>(p, ks, smem_f, s); });
   if (rc != RAD_OK) return rc;
 

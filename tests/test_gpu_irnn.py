@@ -55,11 +55,11 @@ def test_irnn_stored_bytes():
 
 
 @pytest.mark.parametrize("B,T,Hd,C", [(1, 1, 1, 2), (3, 4, 8, 3), (2, 5, 33, 4), (151, 9, 63, 3), (2, 17, 81, 10), (3, 8, 97, 2),
-                                      (2, 33, 113, 5), (2, 12, 128, 3)])
+                                      (2, 33, 113, 5), (2, 12, 128, 3), (1, 3544, 125, 3)])
 @pytest.mark.parametrize("p", [0.05, 0.6])
 def test_irnn_step_over_hidden_sizes_and_groups_of_steps(B, T, Hd, C, p):
     """Hidden sizes on either side of every instantiation of the kernels, and numbers of steps that leave whole and partial
-    groups (of eight steps forward, four backward), against the oracle."""
+    groups (of eight steps forward, four backward), the longest sequence of a size among them, against the oracle."""
     import paper_2007_10412_b200 as rad
     args = irnn_inputs(B, T, Hd, C, seed=B + T + Hd, identity=False)
     ref = orc.irnn_step(*args, variant="different", p=p, seed=6, step0=77)

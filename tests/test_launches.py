@@ -163,3 +163,21 @@ def test_rows_of_dw_that_were_not_kept_are_zeroed_or_the_call_fails(fake):
     for k in range(2):
         b.lib().fake_reset(k)
         assert call() == -3 and b.lib().fake_last_error() == 0
+
+
+@pytest.mark.parametrize("Hd", [1, 2, 31, 33, 64, 65, 97, 98, 100, 113, 125, 126, 127, 128])
+def test_longest_sequence_of_the_recurrent_net(fake, Hd):
+    """What a row holds on chip between the passes bounds the number of steps: 200 KB of inputs, keep bits, derivative bits,
+    offsets and a share of dW_hh with rows of Hd + 1 floats.  The launch itself must fit 227 KB with the 10.3 KB that the
+    backward kernel holds in static arrays and the 1 KB every CTA gives up."""
+    w32, share = (Hd + 31) // 32, (Hd * (Hd + 1) + 3) // 4 * 16
+    fits = lambda T: (T + 3) // 4 * 16 + T * (2 * w32 + 1) * 4 + share <= 200 * 1024
+    T = next(t for t in range(13000, 0, -1) if fits(t))
+    fake.lib().fake_reset(-1)
+    _irnn(fake, 1, T, Hd)()
+    for name, *dims in _launches(fake):
+        assert dims[6] + (10624 if "irnn_backward" in name else 16704 if "irnn_forward" in name else 0) + 1024 <= 227 * 1024, name
+    fake.lib().fake_reset(-1)
+    with pytest.raises(fake.RadError, match="larger than the built-in"):
+        _irnn(fake, 1, T + 1, Hd)()
+    assert fake.lib().fake_launches() == 0
