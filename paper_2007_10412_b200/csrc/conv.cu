@@ -570,10 +570,11 @@ int conv_input_grad(int dtype, int64_t B, int H, int W, int Cin, int Cout, const
 int64_t conv_weight_grad_workspace(int64_t B, int Cin, int Cout) { return round_up(B * (9 * Cin + 1) * Cout * 4, 256); }
 
 // Up to four input channels (their sums sit in registers), threads for every (tap, channel pair), an image and a list
-// that leave room for two CTAs on an SM, and values whose place fits the list's 30 bits.
+// that leave room for two CTAs on an SM (so an entry's place fits the list's 30 bits), and an image that the general route
+// takes too (its list holds ten bits per coordinate): a net is refused by its sizes, not by the route.
 bool conv_first_backward_ok(int dtype, int H, int W, int Cin, int Cout, const void* dP) {
   const int es = dtype == RAD_BF16 ? 2 : 4;
-  return Cin <= 4 && Cout % 8 == 0 && 9 * (Cout / 2) <= kFirstThreads && ((uintptr_t)dP & 15) == 0 &&
+  return Cin <= 4 && Cout % 8 == 0 && 9 * (Cout / 2) <= kFirstThreads && H < 1024 && W < 1024 && ((uintptr_t)dP & 15) == 0 &&
          conv_first_smem(H, W, Cout, es, (int64_t)H * W * Cin) <= 110 * 1024;
 }
 

@@ -181,3 +181,17 @@ def test_longest_sequence_of_the_recurrent_net(fake, Hd):
     with pytest.raises(fake.RadError, match="larger than the built-in"):
         _irnn(fake, 1, T + 1, Hd)()
     assert fake.lib().fake_launches() == 0
+
+
+@pytest.mark.parametrize("cin", [1, 5])
+@pytest.mark.parametrize("H,W", [(1024, 2), (2, 1024)])
+def test_images_of_1024_lines_or_columns_stay_refused(fake, H, W, cin):
+    b = fake
+    ch, fc = (C.c_int64 * 1)(8), (C.c_int64 * 1)(5)
+    desc = b.rad_cnn_desc(2, H, W, cin, 1, 1, ch, fc, b.DTYPES["bf16"], b.VARIANTS["different"], 0.2, 0, 0)
+    nbytes, one = C.c_int64(0), b._table([torch.empty(64)])
+    assert b.lib().rad_cnn_workspace(C.byref(desc), C.byref(nbytes), None) == 0
+    some = C.c_void_p(256)
+    b.lib().fake_reset(-1)
+    rc = b.lib().rad_cnn_step(C.byref(desc), some, some, one, one, one, one, one, one, one, one, some, None, some, nbytes.value, None, None)
+    assert rc == -5
