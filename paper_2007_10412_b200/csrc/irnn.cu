@@ -89,7 +89,7 @@ struct UnitDot {
 
 template <int KP>
 __global__ void __launch_bounds__(32 * (KP / 2 + kStoreWarps), 2) irnn_forward_kernel(const RnnParams p, const PhiloxKeys ks, int unit_warps) {
-  begin_after_previous();
+  wait_for_previous();
   extern __shared__ float sm[];
   float* s_x = sm;                                   // T inputs of this row
   constexpr int kGroup = kFwdGroup, kRing = 4 * kGroup;                  // states: two groups of steps and what the store warps still read
@@ -117,6 +117,7 @@ __global__ void __launch_bounds__(32 * (KP / 2 + kStoreWarps), 2) irnn_forward_k
     const int x_step = q == 0 ? kGroup : 0;
     int left = (int)p.T;
     for (int g = 0; left > 0; ++g, left -= kGroup, x += x_step) {
+      if (left <= 4 * kGroup) let_next_start();      // 10 us before the end, about what a launch takes
       float* h = s_h[(g * kGroup) % kRing];          // the group's first state; the next group's first may be the ring's first
       float* h_next = s_h[(g * kGroup + kGroup) % kRing];
 #pragma unroll
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(32 * (KP / 2 + kStoreWarps), 2) irnn_forward_k
 
 template <int KP>
 __global__ void __launch_bounds__(32 * (KP / 2 + kListWarps), 2) irnn_backward_kernel(const RnnParams p, int unit_warps) {
-  begin_after_previous();
+  wait_for_previous();
   extern __shared__ __align__(16) float sm[];
   constexpr int kGroup = kBwdGroup;
   const int Hd = p.Hd;
@@ -329,6 +330,7 @@ __global__ void __launch_bounds__(32 * (KP / 2 + kListWarps), 2) irnn_backward_k
     __syncthreads();
     int left = (int)p.T;
     for (int g = 0; left > 0; ++g, left -= kGroup) {
+      if (left <= 4 * kGroup) let_next_start();      // as in the forward pass
       const int slot0 = (g & 1) * kGroup;
       Update u;
 #pragma unroll

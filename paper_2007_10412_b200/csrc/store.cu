@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(1024) same_mask_kernel(const SameParams p, con
 // values[b, j] = A[b, idx[j]] * scale for j < k', zero up to ld.  One warp per row at a time.
 template <typename T>
 __global__ void __launch_bounds__(256) same_gather_kernel(const SameParams p, const float* colscale) {
-  begin_after_previous();
+  wait_for_previous();
   const int64_t k = min(p.nnz[0], p.ld);
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -383,6 +383,7 @@ __global__ void __launch_bounds__(256) same_gather_kernel(const SameParams p, co
   const T* A = static_cast<const T*>(p.A);
   T* out = static_cast<T*>(p.values);
   for (int64_t b = warp0; b < p.B; b += nwarps) {
+    if (b + nwarps >= p.B) let_next_start();
     const T* rowp = A + b * p.lda;
     T* orow = out + b * p.ld;
     for (int64_t j = lane; j < p.ld; j += 32) {
@@ -404,7 +405,7 @@ __global__ void __launch_bounds__(256) same_gather_kernel(const SameParams p, co
 // columns sit in shared memory as 16-bit numbers (D <= 65536).
 template <typename T>
 __global__ void __launch_bounds__(256) same_gather_rows_kernel(const SameParams p, uint32_t* relubits, int64_t w32, int warps) {
-  begin_after_previous();
+  wait_for_previous();
   extern __shared__ __align__(16) unsigned char s_dyn[];
   constexpr int kPer = 16 / (int)sizeof(T);
   const int64_t k = min(p.nnz[0], p.ld);
@@ -428,6 +429,7 @@ __global__ void __launch_bounds__(256) same_gather_rows_kernel(const SameParams 
   T* out = static_cast<T*>(p.values);
   const int64_t chunks = p.D / kPer;
   for (int64_t b = (int64_t)blockIdx.x * warps + warp; b < p.B; b += (int64_t)gridDim.x * warps) {
+    if (b + (int64_t)gridDim.x * warps >= p.B) let_next_start();
     const T* rowp = A + b * p.lda;
     for (int64_t c = lane; c < chunks; c += 32)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s_row_addr + (uint32_t)(c * 16)), "l"(rowp + c * kPer) : "memory");

@@ -34,12 +34,13 @@ struct IndexParams {
 // the eight turns, gives every row its offset in (row, column) order.
 constexpr int kIndexWarps = 4;
 __global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const IndexParams p, const PhiloxKeys ks) {
-  begin_after_previous();
+  wait_for_previous();
   const int lane = threadIdx.x & 31;
   const uint32_t warp0 = blockIdx.x * kIndexWarps + (threadIdx.x >> 5), nwarps = gridDim.x * kIndexWarps;
   const uint32_t nrows = (uint32_t)p.B, ncols = (uint32_t)p.D, ncb = (uint32_t)p.ncb;
   const int w = lane & 3;
   for (uint32_t tile = warp0; tile < (uint32_t)p.ntiles; tile += nwarps) {
+    if ((uint64_t)tile + nwarps >= (uint32_t)p.ntiles) let_next_start();
     const uint32_t slab = tile / ncb, cb = tile - slab * ncb;
     const uint32_t col0 = cb * kTileCols + 32u * w;
     uint32_t* tw = p.keepbits + (int64_t)tile * kTileWords;

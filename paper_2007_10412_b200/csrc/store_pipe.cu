@@ -182,7 +182,7 @@ __device__ __forceinline__ void copy_scaled(const T* wb, T* out, uint32_t first,
 template <typename T, int S, bool kFill>
 __global__ void __launch_bounds__(kPipeThreads, 2) store_pipelined_kernel(const StoreParams p, const PhiloxKeys ks,
                                                                       const __grid_constant__ CUtensorMap tmA) {
-  begin_after_previous();
+  wait_for_previous();
   // A stage of the ring must always serve the same half of the compute warps: a waiter tells the phases of
   // a barrier apart by one parity bit, which only works if it has itself waited for the phase before.
   static_assert(S % kTilesPerStep == 0, "stages and tiles worked on side by side");
@@ -411,7 +411,10 @@ __global__ void __launch_bounds__(kPipeThreads, 2) store_pipelined_kernel(const 
         }
         bar_arrive(&sm.chunk_ready[slot]);
         ++seq_claim;
-        if (id == kNoChunk) more = false;
+        if (id == kNoChunk) {
+          more = false;
+          let_next_start();                       // what this CTA still has to do are the chunks it has claimed
+        }
         return id;
       };
       uint32_t q[kAhead + 1];                     // claimed, not yet loaded, oldest first

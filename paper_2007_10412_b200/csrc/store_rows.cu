@@ -109,7 +109,7 @@ constexpr int kRowsWarps = 8;
 
 template <typename T, bool kRowsOut>
 __global__ void __launch_bounds__(32 * kRowsWarps) rows_fixed_kernel(const RowsParams p, const PhiloxKeys ks) {
-  begin_after_previous();
+  wait_for_previous();
   extern __shared__ __align__(16) uint32_t s_dyn[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // per warp: bitmap (words), draws (draws_stride), column list (k 16-bit numbers, kRowsOut only)
@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(32 * kRowsWarps) rows_fixed_kernel(const RowsP
 
   if (kRowsOut) {
     for (int64_t row = (int64_t)blockIdx.x * kRowsWarps + warp; row < p.B; row += (int64_t)gridDim.x * kRowsWarps) {
+      if (row + (int64_t)gridDim.x * kRowsWarps >= p.B) let_next_start();
       for (int i = lane; i < p.words; i += 32) bm[i] = 0;
       __syncwarp();
       floyd_row(bm, draws, (uint32_t)row, (uint32_t)p.D, (uint32_t)p.k, p.c2, p.c3, ks, lane);
@@ -166,6 +167,7 @@ __global__ void __launch_bounds__(32 * kRowsWarps) rows_fixed_kernel(const RowsP
   } else {
     // one CTA per slab of 64 rows; warp w takes rows w, w + 8, ...
     for (int64_t slab = blockIdx.x; slab * kTileRows < p.B; slab += gridDim.x) {
+      if ((slab + gridDim.x) * kTileRows >= p.B) let_next_start();
       for (int r = warp; r < kTileRows; r += kRowsWarps) {
         const int64_t row = slab * kTileRows + r;
         for (int i = lane; i < p.words; i += 32) bm[i] = 0;
@@ -260,7 +262,7 @@ __global__ void __launch_bounds__(256) tile_padding_kernel(const uint32_t* keepb
 // extras: `extras_ld` words per row: word 0 = entries that follow, each (column | count << 16), count >= 2.
 __global__ void __launch_bounds__(32 * kRowsWarps) replace_index_kernel(const RowsParams p, const PhiloxKeys ks, uint32_t* extras,
                                                                         int32_t extras_ld) {
-  begin_after_previous();
+  wait_for_previous();
   extern __shared__ __align__(16) uint32_t s_dyn[];
   __shared__ uint32_t s_nrep[kRowsWarps], s_nex[kRowsWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -269,6 +271,7 @@ __global__ void __launch_bounds__(32 * kRowsWarps) replace_index_kernel(const Ro
   uint16_t* rep = reinterpret_cast<uint16_t*>(bm + p.words);
   uint8_t* s_cnt = reinterpret_cast<uint8_t*>(s_dyn + kRowsWarps * per_warp);   // [64 rows][ncb] kept per (row, block)
   for (int64_t slab = blockIdx.x; slab * kTileRows < p.B; slab += gridDim.x) {
+    if ((slab + gridDim.x) * kTileRows >= p.B) let_next_start();
     for (int r = warp; r < kTileRows; r += kRowsWarps) {
       const int64_t row = slab * kTileRows + r;
       for (int i = lane; i < p.words; i += 32) bm[i] = 0;

@@ -573,7 +573,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
   const uint32_t tmem_base = ctl->tmem_base;
   const uint32_t smem_base = smem_u32(smem);
   // so far nothing of another kernel was touched: the above runs under the tail of the kernel before
-  begin_after_previous();
+  wait_for_previous();
   // Same-sample dW (kDwT): the tile is dW^T, M = H, N = kept columns (known on the device only).  The kept
   // columns are cut into the fewest tiles of at most 256 and the tile width bn is what one of them needs,
   // rounded up to the MMA's granule of 16: 105 kept columns cost one tile of 112, not one of 256.
@@ -597,6 +597,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
     bool ok = true;
     for (int64_t u = pair; u < sched.units && ok; u += npairs) {
       const Unit w = sched.unit(u);
+      if (u + npairs >= sched.units) let_next_start();
       const int m_own = (int)w.m0 + 128 * (int)rank, n_own = (int)w.n0 + (bn / 2) * (int)rank;
       for (int kb = w.kb0; kb < w.kb1; ++kb) {
         if (lane == 0) {
@@ -809,7 +810,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
   const uint32_t tmem_base = ctl->tmem_base;
   const uint32_t smem_base = smem_u32(smem);
   // so far nothing of another kernel was touched: the above runs under the tail of the kernel before
-  begin_after_previous();
+  wait_for_previous();
   // this CTA's store tile column (128 columns of the layer input) of a unit, and whether it exists
   auto tile_col_of = [&](const Unit& w) -> int64_t { return (w.m0 + 128 * (int64_t)rank) / kTileCols; };
   // A warp's part of a unit's epilogue: 32-column chunks `first`, first + kSpEpiShare, ... of its lane quarter's rows
@@ -840,6 +841,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
     bool ok = true;
     for (int64_t u = pair; u < sched.units && ok; u += npairs) {
       const Unit w = sched.unit(u);
+      if (u + npairs >= sched.units) let_next_start();
       const int n_own = (int)w.n0 + 128 * (int)rank;       // + 256 for the second half
       for (int kb = w.kb0; kb < w.kb1; ++kb) {
         if (lane == 0) {
