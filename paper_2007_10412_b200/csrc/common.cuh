@@ -356,6 +356,9 @@ __device__ __forceinline__ void st_cluster_f32(float* smem, uint32_t rank, float
 // could have written, or could still read, is touched before; the next launch is let in after the wait, one ahead at
 // most.  A kernel that takes tensor memory lets the next one in only after its allocation: a CTA of the next kernel that
 // allocated first on the same SM would hold what this kernel, whose end it waits for, still has to get.
+// A kernel thus lives while the one before still writes: nothing that could come from there is read through the read-only
+// path (__ldg, ld.global.nc, const __restrict__), which is for memory that nobody writes while the kernel lives, and
+// which the wait does not order.  Ordinary and .cg loads behind the wait are ordered by it, and so are TMA loads.
 // CTAs that wait hold registers and thread slots which a kernel of another stream could use, so the next launch is let in
 // near the end: a kernel whose CTAs each do one piece of work signals as the piece begins (the launch comes when the last
 // CTA has signalled, that is with the last wave), one whose CTAs go on to further pieces as each begins its last one.

@@ -122,7 +122,7 @@ struct CvCtl {
 // 16 bytes of a dense NHWC tensor at pixel (y, x) of the image that starts at T, channel c0 .. c0 + 7, zero outside
 __device__ __forceinline__ uint4 cv_load_pixel(const bf16* T, bool in, int y, int x, int H, int W, int C, int c0) {
   if (!in || y < 0 || y >= H || x < 0 || x >= W) return make_uint4(0u, 0u, 0u, 0u);
-  return __ldg(reinterpret_cast<const uint4*>(T + ((int64_t)y * W + x) * C + c0));
+  return *reinterpret_cast<const uint4*>(T + ((int64_t)y * W + x) * C + c0);
 }
 
 // kCvFwd: forward tile `blockIdx.x` (128 output pixels); kCvDw: filter-gradient unit (m tile, split) = blockIdx;
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kCvThreads, 3) conv_tc_kernel(const ConvTcPara
       for (int j = 0; j < 2; ++j) {
         const int k = (tid >> 3) + 32 * j, c = (tid & 7) * 8;
         const int64_t pix = (kb0 + kb) * kCvK + k;
-        vb[j] = pix < npix && c < Cout ? __ldg(reinterpret_cast<const uint4*>(p.dZ + pix * Cout + c)) : make_uint4(0u, 0u, 0u, 0u);
+        vb[j] = pix < npix && c < Cout ? *reinterpret_cast<const uint4*>(p.dZ + pix * Cout + c) : make_uint4(0u, 0u, 0u, 0u);
       }
     } else {
       const int k0 = kb * kCvK + cc * 8, tap = k0 / C, c0 = k0 - tap * C, ty = tap / 3, tx = tap - 3 * ty;
@@ -230,11 +230,11 @@ __global__ void __launch_bounds__(kCvThreads, 3) conv_tc_kernel(const ConvTcPara
         vb[j] = make_uint4(0u, 0u, 0u, 0u);
         if (kDx) {
           // B: K-major, row n = input channel, k = (tap, co): W[tap, n, co0 .. co0 + 7] is contiguous
-          if (tap < 9 && r < Cin) vb[j] = __ldg(reinterpret_cast<const uint4*>(p.Wt + ((int64_t)tap * Cin + r) * Cout + c0));
+          if (tap < 9 && r < Cin) vb[j] = *reinterpret_cast<const uint4*>(p.Wt + ((int64_t)tap * Cin + r) * Cout + c0);
         } else {
           // B: filter rows k (MN-major: Cout contiguous), 8 chunks of 8 channels per row
           const int kg = kb * kCvK + r;
-          if (kg < ktaps && cc * 8 < Cout) vb[j] = __ldg(reinterpret_cast<const uint4*>(p.Wt + (int64_t)kg * Cout + cc * 8));
+          if (kg < ktaps && cc * 8 < Cout) vb[j] = *reinterpret_cast<const uint4*>(p.Wt + (int64_t)kg * Cout + cc * 8);
         }
       }
     }
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kCvThreads, 3) conv_tc_kernel(const ConvTcPara
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
         const int co = chunk * 32 + j;
-        const float z = __uint_as_float(r[j]) + (p.bias != nullptr && co < Cout ? __ldg(p.bias + co) : 0.0f);
+        const float z = __uint_as_float(r[j]) + (p.bias != nullptr && co < Cout ? p.bias[co] : 0.0f);
         a[j] = __bfloat162float(__float2bfloat16_rn(fmaxf(z, 0.0f)));       // the activation as the device would hold it
       }
       // round 1, partner lane ^ 1: keep channel blocks q & 1 and 2 + (q & 1) of eight

@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(256) same_gather_kernel(const SameParams p, co
     for (int64_t j = lane; j < p.ld; j += 32) {
       float v = 0.0f;
       if (j < k) {
-        const uint32_t col = __ldg(p.idx + j);
+        const uint32_t col = p.idx[j];
         if (col < (uint32_t)p.D) v = __fmul_rn(to_float(rowp[col]), colscale != nullptr ? colscale[j] : p.scale);
         else raise_status(p.dev_status, RAD_DEV_EINTERNAL);
       }
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(256) same_gather_rows_kernel(const SameParams 
   for (int64_t j = tid; j < p.ld; j += blockDim.x) {
     uint32_t col = 0;
     if (j < k) {
-      col = __ldg(p.idx + j);
+      col = p.idx[j];
       if (col >= (uint32_t)p.D) { raise_status(p.dev_status, RAD_DEV_EINTERNAL); col = 0; }
     }
     s_idx[j] = (uint16_t)col;

@@ -177,9 +177,9 @@ struct StoreRow {
   __device__ __forceinline__ void load(const TcParams& p, int64_t m, int64_t n) {
     const int64_t tile = (m >> 6) * p.st_ncb + (n >> 7);
     const uint32_t* tw = p.st_keepbits + tile * kTileWords;
-    bits = __ldg(reinterpret_cast<const uint4*>(tw + (int)(m & 63) * 4));
-    first = __ldg(p.st_offsets + tile);
-    off = __ldg(reinterpret_cast<const unsigned short*>(tw + kBitWords) + (int)(m & 63));
+    bits = *reinterpret_cast<const uint4*>(tw + (int)(m & 63) * 4);
+    first = p.st_offsets[tile];
+    off = reinterpret_cast<const unsigned short*>(tw + kBitWords)[(int)(m & 63)];
   }
 };
 
@@ -197,7 +197,7 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, uint32_t (&r)[
 #pragma unroll
       for (int j = 0; j < 32; j += 4) {
         if (j < nvalid) {
-          const float4 b4 = __ldg(reinterpret_cast<const float4*>(p.bias + n + j));
+          const float4 b4 = *reinterpret_cast<const float4*>(p.bias + n + j);
           v[j] += b4.x; v[j + 1] += b4.y; v[j + 2] += b4.z; v[j + 3] += b4.w;
         }
       }
@@ -270,10 +270,10 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, uint32_t (&r)[
           }
           if (rr == 0 && wq == 0) {
             // zeros between the tile's last value and its padded end
-            const uint4 last = __ldg(reinterpret_cast<const uint4*>(tw + 63 * 4));
-            const uint32_t exact = __ldg(reinterpret_cast<const unsigned short*>(tw + kBitWords) + 63) + __popc(last.x) +
-                                   __popc(last.y) + __popc(last.z) + __popc(last.w);
-            const uint64_t end = min((uint64_t)__ldg(p.st_offsets + tile + 1), cap);
+            const uint4 last = *reinterpret_cast<const uint4*>(tw + 63 * 4);
+            const uint32_t exact = reinterpret_cast<const unsigned short*>(tw + kBitWords)[63] + __popc(last.x) + __popc(last.y) +
+                                   __popc(last.z) + __popc(last.w);
+            const uint64_t end = min((uint64_t)p.st_offsets[tile + 1], cap);
             for (uint64_t q = (uint64_t)first + exact; q < end; ++q) p.st_values[q] = __float2bfloat16_rn(0.0f);
           }
         }
@@ -282,7 +282,13 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, uint32_t (&r)[
   } else {
     if (row_ok) {
       uint32_t bits = 0xffffffffu;
-      if (p.relubits_prev != nullptr) bits = __ldg(p.relubits_prev + m * ((p.N + 31) / 32) + (n >> 5));
+      if (p.relubits_prev != nullptr) bits = p.relubits_prev[m * ((p.N + 31) / 32) + (n >> 5)];
+      uint4 z_prev[4];                            // read before the first store, so that the loads are in flight together
+      if (p.z_prev != nullptr) {
+#pragma unroll
+        for (int j = 0; j < 32; j += 8)
+          if (j < nvalid) z_prev[j >> 3] = *reinterpret_cast<const uint4*>(p.z_prev + m * p.ld_zprev + n + j);
+      }
       uint4* dst = reinterpret_cast<uint4*>(p.out_dx + m * p.ld_dx + n);
 #pragma unroll
       for (int j = 0; j < 32; j += 8) {
@@ -291,7 +297,7 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, uint32_t (&r)[
 #pragma unroll
           for (int e = 0; e < 8; ++e) g[e] = ((bits >> (j + e)) & 1u) ? __uint_as_float(r[j + e]) : 0.0f;
           if (p.z_prev != nullptr) {
-            const uint4 zq = __ldg(reinterpret_cast<const uint4*>(p.z_prev + m * p.ld_zprev + n + j));
+            const uint4 zq = z_prev[j >> 3];
             const uint32_t zw[4] = {zq.x, zq.y, zq.z, zq.w};
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -354,11 +360,17 @@ __device__ __forceinline__ void epilogue_chunk_dwt(const TcParams& p, const uint
       if (jj < nvalid) dst[(int64_t)jj * p.M] = __uint_as_float(r[jj]);
   } else {
 #pragma unroll
-    for (int jj = 0; jj < 32; ++jj) {
-      if (jj < nvalid) {
-        const int64_t row = (int64_t)__ldg(p.row_idx + n + jj);
-        if (row < p.dw_rows) p.out_dw[row * p.ld_dw + h] = __uint_as_float(r[jj]);
-        else raise_status(p.dev_status, RAD_DEV_EINTERNAL);
+    for (int j0 = 0; j0 < 32; j0 += 8) {          // the rows of eight columns are read before the first of their stores
+      uint32_t row[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (j0 + e < nvalid) row[e] = p.row_idx[n + j0 + e];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        if (j0 + e < nvalid) {
+          if (row[e] < p.dw_rows) p.out_dw[row[e] * p.ld_dw + h] = __uint_as_float(r[j0 + e]);
+          else raise_status(p.dev_status, RAD_DEV_EINTERNAL);
+        }
       }
     }
   }
@@ -693,7 +705,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       const int et = tid - 64;                       // 0 .. 32 kEpiWarps2 - 1
       const int64_t h4 = p.M / 4;
       for (int64_t d = blockIdx.x; d < p.dw_rows; d += gridDim.x) {
-        if ((__ldg(p.keep_cols + (d >> 5)) >> (d & 31)) & 1u) continue;
+        if ((p.keep_cols[d >> 5] >> (d & 31)) & 1u) continue;
         float4* rowp = reinterpret_cast<float4*>(p.out_dw + d * p.ld_dw);
         for (int64_t i = et; i < h4; i += 32 * kEpiWarps2) rowp[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
@@ -930,8 +942,8 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
           const int kbl = kb + lane;
           if (kbl < w.kb1) {
             const int64_t t0 = (int64_t)kbl * p.ncb + tile_col;
-            off_lo = __ldg(p.offsets + t0);
-            off_hi = __ldg(p.offsets + t0 + 1);
+            off_lo = p.offsets[t0];
+            off_hi = p.offsets[t0 + 1];
           }
         }
         const int src = (kb - w.kb0) & 31;

@@ -195,3 +195,12 @@ def test_images_of_1024_lines_or_columns_stay_refused(fake, H, W, cin):
     b.lib().fake_reset(-1)
     rc = b.lib().rad_cnn_step(C.byref(desc), some, some, one, one, one, one, one, one, one, one, some, None, some, nbytes.value, None, None)
     assert rc == -5
+
+
+def test_no_kernel_reads_through_the_read_only_path():
+    """A kernel's lifetime overlaps that of the kernel before it, which may write what it reads: loads that are defined only for
+    memory nobody writes meanwhile (ld.global.nc, which __ldg and const __restrict__ parameters give) do not occur."""
+    from paper_2007_10412_b200 import build
+    for name in sorted(os.listdir(build.CSRC)):
+        text = re.sub(r"//[^\n]*|/\*.*?\*/", "", open(os.path.join(build.CSRC, name)).read(), flags=re.S)
+        assert not re.search(r"\b__ldg\b|ld\.global(\.\w+)*\.nc|__restrict", text), name
