@@ -655,6 +655,7 @@ constexpr int kColMaxCluster = 8;          // portable cluster size
 // 186 us (5.8 TB/s) against 216 us with clusters on 128-byte columns and 200 us before; 16384 x 4096 (134 MB), which
 // L2 still helps, 33 against 30 us, so the line lies above it.
 constexpr int64_t kColBigBytes = 256ll << 20;
+constexpr int64_t kColTallRows = 128;      // rows of a thread above which one cluster along the rows is too few CTAs
 template <typename T, int V>
 __device__ __forceinline__ void colsum_load(const T* p, float (&v)[V]) {
   if constexpr (V == 1) {
@@ -746,8 +747,16 @@ int column_sums_of(const T* dZ, int64_t ldz, int64_t B, int64_t H, float* out, f
   // Two launches where a cluster per column block would leave most SMs idle and its threads with a long walk
   // (a convolution's bias gradient: B H W rows of 16 to 64 channels; 4.2 M x 16 bf16 took 75 + 19 us, the second
   // figure one CTA adding 296 partial rows one by one): first one partial row per slab, then the cluster form on those.
-  if (big || (ny == kColMaxCluster && colblocks * ny < 148 && B > 32 * RL * ny && max_slabs > kColMaxCluster)) {
-    const int64_t slabs = std::min<int64_t>(max_slabs, std::max<int64_t>(kColMaxCluster, (big ? 1184 : 592) / colblocks));
+  // `tall`: so many rows that a thread of a cluster would add more than 128 of them one after the other, however many
+  // column blocks there are; CTAs in whole waves of 1184 (eight per SM), at least sixteen slabs.  65536 x 601 float32 86 us
+  // in one launch, 38 in two; bf16 80 and 31; 20000 x 5001 float32 93 and 75; 8192 x 601 (128 rows) 9.2 and 11.5.
+  const bool tall = ny == kColMaxCluster && B > kColTallRows * RL * ny && max_slabs > kColMaxCluster;
+  const bool narrow = ny == kColMaxCluster && colblocks * ny < 148 && B > 32 * RL * ny && max_slabs > kColMaxCluster;
+  if (big || tall || narrow) {
+    int64_t slabs = std::max<int64_t>(kColMaxCluster, (big ? 1184 : 592) / colblocks);
+    if (tall && !big && !narrow)
+      for (int64_t ctas = 1184; (slabs = ctas / colblocks) < 16; ctas += 1184) {}
+    slabs = std::min(max_slabs, slabs);
     const int rc = launch_colsum<T, V>(dZ, ldz, B, H, log_cl, (int)slabs, false, partial, s);
     if (rc != RAD_OK) return rc;
     const bool vec = H % 4 == 0 && ((uintptr_t)partial & 15) == 0;

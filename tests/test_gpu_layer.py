@@ -153,10 +153,11 @@ def test_bias_gradient_alone_on_every_column_sum_route(B, H, dtype):
 
 @pytest.mark.parametrize("B,H,ld,dtype", [(1, 1, 1, "f32"), (33, 8, 8, "bf16"), (1025, 24, 32, "bf16"), (257, 65, 65, "f32"),
                                           (4097, 72, 72, "f32"), (300001, 8, 8, "bf16"), (300001, 7, 7, "f32"),
-                                          (140000, 20, 24, "bf16"), (70000, 132, 132, "f32")])
+                                          (140000, 20, 24, "bf16"), (70000, 132, 132, "f32"), (8192, 601, 601, "f32"),
+                                          (8193, 601, 601, "bf16"), (40001, 603, 605, "f32"), (33000, 1201, 1201, "bf16")])
 def test_bias_gradient_over_clusters_and_slabs(B, H, ld, dtype):
     """Column sums by one CTA, by a cluster of CTAs along the rows and by slabs of rows added in a second launch, with
-    vector and single-element loads (padded rows, odd widths), against float64 sums of the same numbers.  Every chain
+    vector and single-element loads (padded rows, odd widths, tall ones of many column blocks), against float64 sums of the same numbers.  Every chain
     of float32 additions is shorter than 4096 terms of a 2^-24 relative rounding each; the bound allows 33 in a row."""
     import paper_2007_10412_b200 as rad
     tdt = torch.float32 if dtype == "f32" else torch.bfloat16

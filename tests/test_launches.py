@@ -204,3 +204,15 @@ def test_no_kernel_reads_through_the_read_only_path():
     for name in sorted(os.listdir(build.CSRC)):
         text = re.sub(r"//[^\n]*|/\*.*?\*/", "", open(os.path.join(build.CSRC, name)).read(), flags=re.S)
         assert not re.search(r"\b__ldg\b|ld\.global(\.\w+)*\.nc|__restrict", text), name
+
+
+@pytest.mark.parametrize("B,H,dtype", [(65536, 601, "f32"), (65536, 601, "bf16"), (1000000, 601, "f32"), (20000, 5001, "f32"),
+                                       (65536, 2001, "bf16"), (65536, 1200, "bf16"), (9000, 601, "f32")])
+def test_a_tall_matrix_of_any_width_is_summed_by_the_whole_chip(fake, B, H, dtype):
+    """Column sums of more rows than a cluster per column block should walk: a first launch of at least seven CTAs per SM,
+    whatever the width allows for loads, and a second one that adds the slabs."""
+    fake.lib().fake_reset(-1)
+    _input_grad(fake, B, 8, H, dtype, dx=False)()
+    first, second = _launches(fake)
+    assert "colsum_kernel" in first[0] and "colsum_kernel" in second[0]
+    assert first[1] * first[2] >= 7 * 148 and first[8] == 1 and second[2] <= 8
