@@ -322,7 +322,7 @@ inline size_t conv_first_smem(int H, int W, int Cout, int es, int64_t D) {
 
 template <typename T, int kCin>
 __global__ void __launch_bounds__(kFirstThreads) conv_first_backward_kernel(const ConvFirstParams p) {
-  begin_after_previous();
+  wait_for_previous();
   extern __shared__ __align__(16) uint8_t cf_raw[];
   const ConvShape& s = p.s;
   const int Wq = s.W + 2, Cout = s.Cout, image = (s.H + 2) * Wq * Cout;
@@ -344,6 +344,7 @@ __global__ void __launch_bounds__(kFirstThreads) conv_first_backward_kernel(cons
   const T* vals = static_cast<const T*>(p.values);
   for (int64_t b = blockIdx.x; b < s.B; b += gridDim.x) {
     __syncthreads();                                                // the row before has been read
+    if (b + gridDim.x >= s.B) let_next_start();
     if (tid == 0) s_count = 0;
     if (tid < stride)
       for (int i = tid; i < nvec; i += stride) {
