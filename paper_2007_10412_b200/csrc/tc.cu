@@ -468,11 +468,15 @@ __device__ __forceinline__ void expand_word(uint8_t* sA, const uint8_t* sC, int 
 // both CTAs), tmem_empty[b] (even CTA; every epilogue warp of the pair arrives).
 constexpr int kStage2Bytes = 2 * 128 * BK * 2;   // 16 KB of A + 16 KB of B per CTA and stage
 constexpr int kStages2 = 6;
-// Epilogue warps.  Sixteen for a forward pass of up to kWideEpilogueK inputs: its epilogue, which also places the next
-// layer's store, hides its loads and scattered stores behind them (4096 x 1024 x 1024 with ReLU: 25.7 us with eight, 22.2
-// with sixteen).  Eight where the MMAs of a tile outlast the epilogue of the one before anyway (8192 x 4096 x 4096: 224
-// against 234 us) and for the others (input gradient of 4096 x 1024 x 1024: 14.2 against 15.4 us).
-constexpr int64_t kWideEpilogueK = 2048;
+// Epilogue warps, eight or sixteen.  Sixteen for a forward pass of up to kWideEpilogueK inputs that places the next layer's
+// store: more warps hide its loads and scattered stores (us with eight / sixteen, GELU: 4096 x 2048 outputs 50.5 / 40.2
+// from 1024 inputs, 57.0 / 50.1 from 2048, 60.3 / 56.3 from 2560; 8192 x 4096 outputs 171 / 156 from 2048, 180 / 178 from
+// 2560, 195 / 206 from 3072: above, the MMAs of a tile outlast the epilogue of the one before).  Without a store
+// sixteen pay for the arithmetic of a GELU of few inputs (4096 x 512 x 2048 29.3 / 25.5, 16384 x 512 x 2048 78.5 / 62.9),
+// unless it also writes the pre-activations of many tiles (8192 x 1024 x 2048 57.2 / 55.0, but 16384 x 1024 x 2048 94.9 / 101.6
+// and 16384 x 512 x 4096 186 / 196), and cost elsewhere (16384 x 1024 x 4096: ReLU 129 / 148, float32 outputs 156 / 179;
+// input gradient of 4096 x 1024 x 1024 14.2 / 15.4).
+constexpr int64_t kWideEpilogueK = 2048, kWideGeluK = 1024, kWideGeluWaves = 4;
 constexpr int threads2(int epi_warps) { return 32 * (2 + epi_warps); }
 
 struct SmemCtl2 {
@@ -687,7 +691,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       }
     }
   } else {
-    // ===== epilogue: thread = one accumulator row of this CTA, 128 columns per warp =====
+    // ===== epilogue: thread = one accumulator row of this CTA =====
     const int q = warp & 3;
     // the warps of a lane quarter split the tile's 32-column chunks between them
     constexpr int kPerQuarter = kEpiWarps2 / 4;
@@ -714,11 +718,13 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       const Unit w = sched.unit(u);
       const int64_t m = w.m0 + 128 * (int64_t)rank + q * 32 + lane;
       const bool row_ok = m < sched.M;
-      // what the epilogue reads besides the accumulators comes while the MMAs run (a warp's columns lie in one store tile)
+      // what the epilogue reads besides the accumulators comes while the MMAs run (a warp's columns lie in one store tile).
+      // The bias only with sixteen warps: with eight its prefetch costs more than it hides (16384 x 512 x 4096 with GELU 186
+      // us, 165 without)
       StoreRow sr = {};
       if (EPI == kFwd && w.n0 + c_first < n_cols) {
         if (p.st_values != nullptr && row_ok) sr.load(p, m, w.n0 + c_first);
-        if (p.bias != nullptr && lane < own_chunks && w.n0 + c_first + 32 * lane < n_cols)
+        if (kEpiWarps2 > 8 && p.bias != nullptr && lane < own_chunks && w.n0 + c_first + 32 * lane < n_cols)
           asm volatile("prefetch.global.L1 [%0];" ::"l"(p.bias + w.n0 + c_first + 32 * lane));
       }
       if (lane == 0) ok = mbar_wait2(smem_u32(&ctl->tmem_full[0]) + 8u * buf, (buf_phases >> buf) & 1u, wc, 200u);
@@ -1312,7 +1318,10 @@ int tc_forward(int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t 
                                             : (float)kLaneRange / (float)keep_threshold_host(next->p);
   }
   const int64_t units = ceil_div(B, BM) * ceil_div(H, p.bn);
-  return D <= kWideEpilogueK ? launch_pair<kAK, kBMN, kFwd, 16>(p, ta, tb, units, s) : launch_pair<kAK, kBMN, kFwd, 8>(p, ta, tb, units, s);
+  const bool wide = p.st_values != nullptr ? D <= kWideEpilogueK
+                                           : act == RAD_ACT_GELU && D <= kWideGeluK &&
+                                                 (out_zlow == nullptr || units <= kWideGeluWaves * planning_pairs());
+  return wide ? launch_pair<kAK, kBMN, kFwd, 16>(p, ta, tb, units, s) : launch_pair<kAK, kBMN, kFwd, 8>(p, ta, tb, units, s);
 }
 
 int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, const void* W, int64_t ldw,

@@ -216,3 +216,23 @@ def test_a_tall_matrix_of_any_width_is_summed_by_the_whole_chip(fake, B, H, dtyp
     first, second = _launches(fake)
     assert "colsum_kernel" in first[0] and "colsum_kernel" in second[0]
     assert first[1] * first[2] >= 7 * 148 and first[8] == 1 and second[2] <= 8
+
+
+def _pair_kernel(name):
+    """(operand kinds and epilogue, epilogue warps) of a tensor-core kernel's mangled name."""
+    m = re.search(r"tc_gemm_pair_kernelILi(\d)ELi(\d)ELi(\d)ELi(\d+)EE", name)
+    return m and (tuple(int(v) for v in m.groups()[:3]), int(m.group(4)))
+
+
+@pytest.mark.parametrize("B,D,H,act,zlow,warps", [(16384, 1024, 4096, "relu", False, 8), (8192, 2048, 2048, "relu", False, 8),
+                                                  (16384, 1024, 2048, "gelu", True, 8), (8192, 1024, 2048, "gelu", True, 16),
+                                                  (16384, 1024, 2048, "gelu", False, 16), (4096, 1032, 2048, "gelu", False, 8)])
+def test_epilogue_warps_of_a_forward_without_a_store(fake, B, D, H, act, zlow, warps):
+    """Sixteen only for the arithmetic of a GELU of up to 1024 inputs, and then not where it also writes the pre-activations
+    of more than four waves of tiles: elsewhere eight are faster."""
+    bf = torch.bfloat16
+    A, W, out = torch.empty(B, D, dtype=bf), torch.empty(D, H, dtype=bf), torch.empty(B, H, dtype=bf)
+    fake.lib().fake_reset(-1)
+    fake.rad_linear_forward(A, W, None, act, out_act=out, out_zlow=out if zlow else None)
+    (name, *_), = _launches(fake)
+    assert _pair_kernel(name)[1] == warps
