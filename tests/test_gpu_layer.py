@@ -237,14 +237,36 @@ def test_cuda_core_contractions_over_tiles_and_splits(B, D, H, dtype):
         assert ((got.double() - ref).abs() <= bound + 1e-30).all()
 
 
-@pytest.mark.parametrize("B,D,H", [(64, 64, 64), (300, 72, 200), (257, 2048, 136), (1024, 640, 1000), (2500, 2056, 1032),
-                                   (5000, 128, 1096)])
+DENSE_WIDTHS = [
+    # B, D, H, columns of a tile of the forward (H wide) and of the input gradient (D wide), on 66 to 74 SM pairs
+    (64, 64, 64, 64, 64),
+    (300, 72, 200, 64, 64),
+    (257, 2048, 136, 64, 64),
+    (200, 2056, 72, 64, 64),            # above 2048 inputs: eight epilogue warps
+    (1024, 640, 1000, 64, 64),
+    (1280, 520, 1032, 128, 64),
+    (1280, 1032, 520, 64, 128),
+    (1280, 2056, 1032, 128, 256),       # eight epilogue warps
+    (2500, 2056, 1032, 256, 256),
+    (5000, 128, 1096, 256, 64),
+]
+
+
+def dense_tile_width(M, N, pairs):
+    """The narrowest of 64, 128 and 256 columns with which the tiles of 256 rows are one wave of SM pairs, else 256."""
+    return next((w for w in (64, 128) if -(-M // 256) * -(-N // w) <= pairs), 256)
+
+
+@pytest.mark.parametrize("B,D,H,fwd_width,dx_width", DENSE_WIDTHS)
 @pytest.mark.parametrize("act", ["relu", "gelu"])
-def test_dense_tile_widths(B, D, H, act):
+def test_dense_tile_widths(B, D, H, fwd_width, dx_width, act):
     """Forward with the next layer's store and input gradient on the tensor cores at tiles of 64, 128 and 256 columns with
     remainders, and with either number of epilogue warps: the forward's store is the store of its own output bit for
-    bit, values against float64 within one bf16 rounding and the float32 sums' error."""
+    bit, the forward without a store (whose epilogue warps are counted by another rule) gives the same output, values against
+    float64 within one bf16 rounding and the float32 sums' error."""
     import paper_2007_10412_b200 as rad
+    pairs = rad.rad_sm_pairs()
+    assert dense_tile_width(B, H, pairs) == fwd_width and dense_tile_width(B, D, pairs) == dx_width
     bf = torch.bfloat16
     g = torch.Generator(device="cuda").manual_seed(B + D + H)
     rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").to(bf)
@@ -257,12 +279,14 @@ def test_dense_tile_widths(B, D, H, act):
     out, zl = torch.empty(B, H, dtype=bf, device="cuda"), torch.empty(B, H, dtype=bf, device="cuda")
     rad.rad_linear_forward_fill(A, W, b, act, out, fill, out_zlow=zl, relubits=fill.relubits, dev_status=status)
     rad.rad_linear_forward_store(out, own, status)
+    plain = torch.empty_like(out)
+    rad.rad_linear_forward(A, W, b, act, out_act=plain, dev_status=status)
     dX = torch.empty(B, D, dtype=bf, device="cuda")
     rad.rad_linear_input_grad(dZ, W, z_prev=zp if act == "gelu" else None, dZ_prev=dX, dev_status=status)
     torch.cuda.synchronize()
     assert status.item() == 0
     for x, y in ((fill.values, own.values), (fill.keepbits, own.keepbits), (fill.offsets, own.offsets), (fill.nnz, own.nnz),
-                 (fill.relubits, own.relubits)):
+                 (fill.relubits, own.relubits), (plain, out)):
         assert torch.equal(x, y)
     z = A.double() @ W.double() + b.double()
     tol = (max(D, H) ** 0.5 + 16) * 2.0 ** -24
@@ -274,3 +298,27 @@ def test_dense_tile_widths(B, D, H, act):
         d = 0.5 * (1 + torch.erf(x / 2 ** 0.5)) + x * torch.exp(-0.5 * x * x) / (2 * np.pi) ** 0.5
         dx, mx = dx * d, mx * (d.abs() + 1e-3)
     assert ((dX.double() - dx).abs() <= 8 * tol * mx + 2.0 ** -8 * dx.abs()).all()
+
+
+@pytest.mark.parametrize("B", [40, 130, 640])
+def test_different_sample_dw_of_several_units_per_sm_pair(B):
+    """dW of 4000 x 4104 from a different-sample store: 144 tiles of 256 x 512 on at most 74 SM pairs, with one K block per tile
+    (the expanders run several tiles ahead of the epilogue), a few, and more than the ring of stages holds; tiles that
+    reach past either edge.  Against float64; the bound is that of a float32 sum of B products in any order."""
+    import paper_2007_10412_b200 as rad
+    D, H, p = 4000, 4104, 0.3
+    assert -(-D // 256) * -(-H // 512) > rad.rad_sm_pairs()
+    bf = torch.bfloat16
+    g = torch.Generator(device="cuda").manual_seed(B)
+    A, dZ = (torch.randn(B, n, generator=g, device="cuda").to(bf) for n in (D, H))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    st = rad.Store("different", "bf16", B, D, p, seed=3, layer=1, step=2, relu_bits=False)
+    rad.rad_linear_forward_store(A, st, status)
+    dW = torch.full((D, H), float("nan"), device="cuda")
+    rad.rad_linear_weight_grad(st, dZ, dW, dev_status=status)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    keep = torch.from_numpy(orc.keep_mask("different", B, D, p, 3, 1, 2)).cuda()
+    Ah = torch.where(keep, (A.float() * float(orc.scale_factor(p))).to(bf), torch.zeros((), dtype=bf, device="cuda")).double()
+    ref, mag = Ah.T @ dZ.double(), Ah.abs().T @ dZ.double().abs()
+    assert ((dW.double() - ref).abs() <= B * 2.0 ** -24 * mag).all()

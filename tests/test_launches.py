@@ -224,6 +224,31 @@ def _pair_kernel(name):
     return m and (tuple(int(v) for v in m.groups()[:3]), int(m.group(4)))
 
 
+def test_tile_widths_and_epilogue_warps_of_the_dense_kernels(fake):
+    """The widths that the parity tests of the tensor-core layers claim to cover are the ones the library launches, and so
+    are the two counts of epilogue warps: both occur at every width of the forward that one wave of tiles can have."""
+    from test_gpu_layer import DENSE_WIDTHS
+    b, bf = fake, torch.bfloat16
+    pairs, seen = b.rad_sm_pairs(), set()
+    for B, D, H, fwd_width, dx_width in DENSE_WIDTHS:
+        A, W, dZ = torch.empty(B, D, dtype=bf), torch.empty(D, H, dtype=bf), torch.empty(B, H, dtype=bf)
+        nx = _store(b, "different", "bf16", B, H)
+        for forward, width, cols in ((True, fwd_width, H), (False, dx_width, D)):
+            b.lib().fake_reset(-1)
+            if forward:
+                b.rad_linear_forward_fill(A, W, None, "relu", dZ, nx)
+            else:
+                b.rad_linear_input_grad(dZ, W, dZ_prev=A)
+            (name, *dims), = [l for l in _launches(b) if _pair_kernel(l[0])]
+            units = -(-B // 256) * -(-cols // width)
+            assert dims[0] == 2 * min(units, pairs), (B, D, H, name)
+            warps = _pair_kernel(name)[1]
+            assert dims[3] == 32 * (2 + warps)
+            if forward:
+                seen.add((width, warps))
+    assert seen == {(w, n) for w in (64, 128, 256) for n in (8, 16)}
+
+
 @pytest.mark.parametrize("B,D,H,act,zlow,warps", [(16384, 1024, 4096, "relu", False, 8), (8192, 2048, 2048, "relu", False, 8),
                                                   (16384, 1024, 2048, "gelu", True, 8), (8192, 1024, 2048, "gelu", True, 16),
                                                   (16384, 1024, 2048, "gelu", False, 16), (4096, 1032, 2048, "gelu", False, 8)])
