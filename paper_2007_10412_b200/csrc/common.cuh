@@ -327,6 +327,11 @@ __device__ __forceinline__ uint32_t cluster_nctas() {
   asm volatile("mov.u32 %0, %%cluster_nctaid.y;" : "=r"(m));
   return n * m;
 }
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
 // every thread of every CTA of the cluster; shared-memory writes before it are seen by all after it
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -336,13 +341,6 @@ __device__ __forceinline__ float ld_cluster_f32(const float* smem, uint32_t rank
   float v;
   asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %1, %2;\n\tld.shared::cluster.f32 %0, [a];\n\t}"
                : "=f"(v) : "r"((uint32_t)__cvta_generic_to_shared(smem)), "r"(rank) : "memory");
-  return v;
-}
-__device__ __forceinline__ float4 ld_cluster_f32x4(const float* smem, uint32_t rank) {
-  float4 v;
-  asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %4, %5;\n\tld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [a];\n\t}"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"((uint32_t)__cvta_generic_to_shared(smem)), "r"(rank) : "memory");
   return v;
 }
 __device__ __forceinline__ void st_cluster_f32(float* smem, uint32_t rank, float v) {

@@ -47,11 +47,6 @@ struct GemmParams {
 __device__ __forceinline__ void share_barrier() {
   if (cluster_nctas() > 1) cluster_barrier(); else __syncthreads();
 }
-__device__ __forceinline__ uint32_t cluster_rank_1d() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
 __device__ __forceinline__ void copy_async16(float* dst, const float* src, int bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
 }
@@ -129,7 +124,7 @@ struct BlockCopy {
 // 95 / 274 / 554 us at p = 0.1 / 0.5 / 1 on the first shape.
 template <typename T, int TS>
 struct SparseCopy {
-  static constexpr int kN = TS / 4, kWords = TS / 32;
+  static constexpr int kWords = TS / 32;
   const uint32_t* tile; const uint32_t* offset; const T* values;
   int64_t capacity, tile_step; int ncb, w0, r, q;
   uint32_t word[kWords]; int64_t at[kWords];
@@ -211,7 +206,7 @@ __device__ __forceinline__ void gemm_partial(const GemmParams& p, int64_t tile, 
         const int kleft = (int)min((int64_t)BK, k1 - k0 - (int64_t)kb * BK);
         if constexpr (kSparse) {
 #pragma unroll
-          for (int j = 0; j < cs.kN; ++j) {
+          for (int j = 0; j < TS / 4; ++j) {
             const int64_t at = cs.place(j);
             copy_async4(sA + cs.r * kLdA + cs.q + 4 * j, reinterpret_cast<const float*>(cs.values) + (at >= 0 ? at : 0), at >= 0 ? 4 : 0);
           }
@@ -372,7 +367,7 @@ __device__ __forceinline__ void gemm_finish(const GemmParams& p, int64_t tile, i
   const int64_t m0 = (tile / p.gx) * TS, n0 = (tile % p.gx) * TS;
   const bool sums = (EPI == kEpiScatterRows || EPI == kEpiSparse) && p.db != nullptr && m0 == 0;
   const int S = p.splits, rows = TS / S, tid = threadIdx.x;
-  const uint32_t rank0 = cluster_rank_1d() - (uint32_t)split;
+  const uint32_t rank0 = cluster_ctarank() - (uint32_t)split;
   if (sums && split == 0 && tid < TS && n0 + tid < p.N) {
     float s = 0.0f;
     for (int q = 0; q < S; ++q) s += S > 1 ? ld_cluster_f32(smem + 4 * TS * TS + tid, rank0 + q) : smem[4 * TS * TS + tid];
@@ -500,13 +495,15 @@ __device__ __forceinline__ void gemm_walk(const GemmParams& p, int64_t tile, flo
 // (0.60 and 0.46 of the FMA rate), a CTA alone 73 and 26; beginning and end of a CTA (first loads, the groups'
 // sums, epilogue) take 7500 and 3850, the launch 4000, the exchange inside a cluster 800.  Fitted to 32 timings
 // (both tiles, 1 to 8 splits); for 150 x 300 outputs it says 28 / 19 / 19 / 22 thousand clocks for 1 / 2 / 4 / 8 CTAs
-// per 32 x 32 tile at k = 784, measured 26 / 19 / 18 / 23; for 1500 x 777, k = 1001, 102 / 91 / 94 us for 1 / 2 / 4 CTAs
+// per 32 x 32 tile at k = 784, measured 26 / 19 / 18 / 23; for 1500 x 777, k = 1001, 105 / 95 / 101 us for 1 / 2 / 4 CTAs
 // per 64 x 64 tile, measured 112 / 101 / 102.
 // The walking form (no split, no sums at the end) is weighed with figures of its own, and bf16 operands, which both forms
 // widen on the way through registers, with others again (the split form's depend on whether k is contiguous: more
 // address arithmetic and spilled registers then).  So the walking form takes short contractions (4096 x 1001 f32, k =
-// 10: 16 us against 30; the lines cross near k = 200 where the chip is full and near k = 80 where it is not) and bf16
-// shapes that fill the chip (1024 x 1023 x 1021 forward: 92 against 137 us).
+// 10: 17 us against 34; the lines cross near k = 160 where the chip is full and near k = 80 where it is not) and bf16
+// shapes that fill the chip (1024 x 1023 x 1021 forward: 95 against 137 us).  Checked with either form forced: of 120
+// forwards, input gradients and same-sample dW of both types, 16 to 4096 rows, the choice is within 6 % of the better form in
+// 118; the others are bf16 300 x 100 x 700 (forward 10.2 against 9.2 us, dW 16.9 against 13.9).
 struct GemmCost { double pair, alone, ends; };
 inline void plan_gemm(GemmParams& p, int64_t Mgrid, int es, int64_t k_step = 4, bool may_walk = true) {   // splits begin at multiples of k_step
   static const GemmCost split_cost[3][2] = {{{35, 26, 3850}, {106, 73, 7500}},      // f32, at 32 x 32 and 64 x 64

@@ -9,10 +9,11 @@
 // Every kernel here runs on SM pairs: a cluster of two CTAs, one per SM, persistent, with one
 // thread of the even CTA issuing tcgen05.mma.cta_group::2 on operands that both CTAs stage in their
 // own shared memory (TMA, 128-byte swizzle, no multicast) through an mbarrier ring.
-//   dense kernels    256 x 256 tile per pair; each CTA keeps two alternating 128 x 256 float32
+//   dense kernels    256 x 256 tile per pair, or 128 or 64 columns wide where that makes one wave of
+//                    them; each CTA keeps two alternating 128 x 256 float32
 //                    accumulators in tensor memory, so the epilogue of a tile (bias, activation,
 //                    ReLU bits, GELU', stores) runs under the MMAs of the next one.
-//   sparse-A kernel  512 x 256 tile per pair; sixteen "expander" warps per CTA write the A_hat
+//   sparse-A kernel  256 x 512 tile per pair; sixteen "expander" warps per CTA write the A_hat
 //                    tile of each K block into shared memory instead of TMA.
 // Long dW contractions can be split along K; partial tiles are summed in split order by a second
 // kernel, so results are reproducible.
@@ -30,7 +31,6 @@ namespace rad {
 namespace {
 
 constexpr int BM = 256, BN = 256, BK = 64;
-constexpr int kHalfM = 128;
 constexpr int kNumSMsDefault = 148;
 constexpr int kMaxSplits = 16;
 constexpr int kRasterGroup = 16;               // m-tiles per raster group (16 x 4 MB of A panels stay in L2 beside the B panels in flight)
@@ -187,7 +187,7 @@ struct StoreRow {
 // r: the 32 float32 accumulators of row m, columns n .. n+31 (as bit patterns).
 template <int EPI>
 __device__ __forceinline__ void epilogue_chunk(const TcParams& p, uint32_t (&r)[32], int64_t m, int64_t n, bool row_ok,
-                                               int32_t split, const StoreRow& sr) {
+                                               const StoreRow& sr) {
   const int nvalid = (int)min((int64_t)32, p.N - n);      // multiple of 8
   if (EPI == kFwd) {
     float v[32];
@@ -378,7 +378,6 @@ __device__ __forceinline__ void epilogue_chunk_dwt(const TcParams& p, const uint
 
 // ---- shared memory layout -------------------------------------------------------------------------
 constexpr int kIndexBytes = kTileWords * 4;   // keep bits + row offsets of one store tile (1152 B)
-constexpr int kExpanderWarps = 16;            // one thread per keep-bit word of the two halves
 constexpr int kFirstExpanderWarp = 7;        // warp 6 feeds the compressed ring
 // ---- expansion of one keep-bit word into the A_hat tile -------------------------------------------
 // sA: the stage's A tile (four 8 KB blocks of 64 columns, 128-byte rows per K index, 128-byte
@@ -456,7 +455,7 @@ __device__ __forceinline__ void expand_word(uint8_t* sA, const uint8_t* sC, int 
 }
 
 // ---- two-CTA engine (dense operands) -----------------------------------------------------------------
-// A cluster of two CTAs (one SM pair) owns a 256 x 256 output tile.  Each CTA stages 128 rows of
+// A cluster of two CTAs (one SM pair) owns an output tile of 256 rows and 256, 128 or 64 columns.  Each CTA stages 128 rows of
 // the A tile and 128 rows (N) of the B tile per K block and keeps 128 accumulator rows in its own
 // tensor memory; one thread of the even CTA issues tcgen05.mma.cta_group::2, which reads both
 // CTAs' shared memory.  Against the one-CTA tile this halves the operand bytes each SM's shared
@@ -485,18 +484,10 @@ struct SmemCtl2 {
   int abort_flag;
 };
 
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
 __device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank) {   // shared::cluster address
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
   return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // Arrival on a barrier of either CTA of the pair (default semantics, as for a local arrival: what
 // the waiter goes on to touch is ordered by tcgen05 or proxy fences issued before the arrival; a
@@ -584,7 +575,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
-  cluster_sync_all();        // the peer's barriers are initialised before anything arrives on them
+  cluster_barrier();        // the peer's barriers are initialised before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
   const uint32_t smem_base = smem_u32(smem);
@@ -740,7 +731,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
         tmem_ld_wait();
         // a chunk may reach past the tile's width (bn is a multiple of 16) and past the last kept column
         if (EPI == kDwT) epilogue_chunk_dwt(p, r, m, n, (int)min((int64_t)min(32, bn - c0), n_cols - n), row_ok, w.split);
-        else epilogue_chunk<(EPI == kDwT ? kDx : EPI)>(p, r, m, n, row_ok, w.split, sr);
+        else epilogue_chunk<(EPI == kDwT ? kDx : EPI)>(p, r, m, n, row_ok, sr);
       }
       tc_fence_before();
       __syncwarp();
@@ -752,7 +743,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
 
   // ===== teardown: neither CTA leaves (or frees tensor memory) while the other may still use it =====
   tc_fence_before();
-  cluster_sync_all();
+  cluster_barrier();
   if (tid == 0 && ctl->abort_flag != 0) raise_status(p.dev_status, RAD_DEV_ETIMEOUT);
   if (warp == 1) {
     tc_fence_after();
@@ -823,7 +814,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
-  cluster_sync_all();
+  cluster_barrier();
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
   const uint32_t smem_base = smem_u32(smem);
@@ -1018,7 +1009,9 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
         if (++stage == stages) { stage = 0; phase ^= 1u; }
         if (++slot == p.comp_depth) { slot = 0; cphase ^= 1u; }
       }
-      // the next unit's MMAs wait for this unit's accumulators to be read, so the expanders have nothing better to do
+      // The next unit's MMAs wait for this unit's accumulators to be read.  Sharing that is worth more than rebuilding the
+      // next unit's first tiles meanwhile: 1024 x 8192 x 8192 140 us against 147 with the expanders ahead instead (and
+      // sharing the last unit only), 2048 x 4096 x 4096 67 against 68, 8192 x 4096 x 4096 209 against 210.
       if (ok) ok = unit_epilogue(w, 1 + (warp - kFirstExpanderWarp) / 4, unit_phase);
       unit_phase ^= 1u;
     }
@@ -1026,7 +1019,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
 
   // ===== teardown: neither CTA leaves (or frees tensor memory) while the other may still use it =====
   tc_fence_before();
-  cluster_sync_all();
+  cluster_barrier();
   if (tid == 0 && ctl->abort_flag != 0) raise_status(p.dev_status, RAD_DEV_ETIMEOUT);
   if (warp == 1) {
     tc_fence_after();
@@ -1046,11 +1039,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64, 1) wait_probe_pa
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  cluster_sync_all();
+  cluster_barrier();
   const PairWait wc = {&abort_flag, map_to_cta(smem_u32(&abort_flag), rank ^ 1u), limit_ns};
   bool ok = true;
   if (threadIdx.x == 0) ok = mbar_wait2(smem_u32(&bar), 0u, wc, 100u);
-  cluster_sync_all();
+  cluster_barrier();
   if (threadIdx.x == 0 && (!ok || abort_flag != 0)) raise_status(dev_status, RAD_DEV_ETIMEOUT);
 }
 
