@@ -201,12 +201,32 @@ def test_softmax_xent_over_clusters_and_row_lengths(B, C, dtype):
         assert (dz == 0).all()
 
 
-@pytest.mark.parametrize("B,D,H,dtype", [(1, 1, 1, "f32"), (33, 130, 31, "f32"), (65, 1001, 33, "f32"), (150, 784, 300, "f32"),
-                                         (700, 257, 203, "f32"), (2000, 68, 1500, "f32"), (129, 3000, 70, "f32"),
-                                         (90, 100, 30, "bf16"), (700, 515, 333, "bf16")])
+# The forms the CUDA-core GEMM takes, by forward and input gradient: one CTA that walks all of k ("walk", tiles of 32 or 64),
+# or k split over thread groups and up to eight CTAs of a cluster ("split"); from 297 tiles on the walk has several waves.
+CUDA_CORE_FORMS = [
+    # B, D, H, type, forward, input gradient
+    (1, 1, 1, "f32", "walk32", "walk32"),
+    (33, 130, 31, "f32", "split32x8", "walk32"),
+    (65, 1001, 33, "f32", "split32x8", "walk32"),
+    (150, 784, 300, "f32", "split32x2", "split32x1"),
+    (700, 257, 203, "f32", "split32x1", "split32x1"),
+    (2000, 68, 1500, "f32", "walk64", "split64x4"),
+    (129, 3000, 70, "f32", "split32x8", "walk64"),
+    (90, 100, 30, "bf16", "split32x4", "walk32"),
+    (700, 515, 333, "bf16", "split32x1", "walk64"),
+    (4100, 10, 300, "f32", "walk64", "split32x1"),
+    (3000, 20, 10, "f32", "walk32", "walk32"),
+    (130, 33, 9, "bf16", "walk32", "walk32"),
+    (1000, 41, 1001, "bf16", "walk64", "split32x4"),
+    (2100, 203, 601, "bf16", "walk64", "walk64"),
+]
+
+
+@pytest.mark.parametrize("B,D,H,dtype", [c[:4] for c in CUDA_CORE_FORMS])
 def test_cuda_core_contractions_over_tiles_and_splits(B, D, H, dtype):
-    """Forward, input gradient and weight gradients (either mask) on CUDA cores, from one CTA to clusters that share the
-    contraction index, 32 and 64 wide tiles with remainders, aligned and odd leading dimensions, against float64.
+    """Forward, input gradient and weight gradients (either mask) on CUDA cores, in the form that walks the contraction index
+    and in the one that splits it, from one CTA to clusters that share it, 32 and 64 wide tiles with remainders, one wave
+    of tiles and several, aligned and odd leading dimensions, against float64.
     Bound per output: sqrt(K) + 16 roundings of 2^-24 of the sum of magnitudes, plus one bf16 rounding of the result."""
     import paper_2007_10412_b200 as rad
     tdt = torch.float32 if dtype == "f32" else torch.bfloat16

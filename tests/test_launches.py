@@ -261,3 +261,19 @@ def test_epilogue_warps_of_a_forward_without_a_store(fake, B, D, H, act, zlow, w
     fake.rad_linear_forward(A, W, None, act, out_act=out, out_zlow=out if zlow else None)
     (name, *_), = _launches(fake)
     assert _pair_kernel(name)[1] == warps
+
+
+def test_forms_of_the_cuda_core_gemm(fake):
+    """The forms that the parity test of the CUDA-core contractions claims to cover are the ones the library launches."""
+    from test_gpu_layer import CUDA_CORE_FORMS
+    b, tile = fake, {36864: 32, 17408: 64, 55296: 32, 104448: 64}            # by dynamic shared memory
+    for B, D, H, dtype, forward, input_grad in CUDA_CORE_FORMS:
+        tdt = torch.float32 if dtype == "f32" else torch.bfloat16
+        A, W, dZ = torch.empty(B, D, dtype=tdt), torch.empty(D, H, dtype=tdt), torch.empty(B, H, dtype=tdt)
+        for run, form in ((lambda: b.rad_linear_forward(A, W, None, "none", out_act=dZ), forward),
+                          (lambda: b.rad_linear_input_grad(dZ, W, dZ_prev=A), input_grad)):
+            b.lib().fake_reset(-1)
+            run()
+            (name, *dims), = _launches(b)
+            got = f"walk{tile[dims[6]]}" if "gemm_walk_kernel" in name else f"split{tile[dims[6]]}x{dims[7]}"
+            assert got == form, (B, D, H, dtype, name)
