@@ -87,3 +87,26 @@ def test_first_convolution_backward_over_channels_and_rows(B, hw, cin, channels,
     for got, want in zip(ctx.dconv_W + ctx.dconv_b, ref.dW_conv + ref.db_conv):
         fro, mx = rel_err(got.double().cpu().numpy(), want)
         assert fro <= TOL[dtype] and mx <= TOL[dtype] * (1 if dtype == "f32" else 2)
+
+
+@pytest.mark.parametrize("cin", [3, 5])
+def test_padding_is_not_multiplied_with_an_infinite_filter(cin):
+    """A tap outside the image contributes nothing, whatever the filter holds there: with -inf in a corner tap of one output
+    channel and a positive image, the outputs whose tap lies inside are -inf before the ReLU (0 after it) and those on
+    the upper and left border stay what the other taps make of them: the net of a filter with -1e30 in that place."""
+    import paper_2007_10412_b200 as rad
+    B, hw, channels, fc = 3, 4, (8,), (3,)
+    X, y, cW, cb, fW, fb = cnn_inputs(B, hw, cin, channels, fc, "f32", seed=21, bias_zero=False)
+    X = np.abs(X) + np.float32(0.1)
+    cW = [np.abs(cW[0])]                       # so that the border outputs are positive
+    cW[0][0, 0, 0, 2] = -1e30
+    ref = orc.cnn_step(X, y, cW, cb, fW, fb, dtype="f32", variant="different", p=1.0, seed=3, step=2)
+    cW[0][0, 0, 0, 2] = -np.inf
+    ctx = rad.CNNStep(B, hw, cin, channels, fc, "f32", "different", 1.0)
+    ctx(to_dev(X, "f32"), torch.from_numpy(y).cuda(), [to_dev(w, "f32") for w in cW], [to_dev(b, "f32") for b in cb],
+        [to_dev(w, "f32") for w in fW], [to_dev(b, "f32") for b in fb], seed=3, step=2)
+    torch.cuda.synchronize()
+    assert abs(ctx.loss.item() - ref.loss) <= 1e-5 * abs(ref.loss)
+    for got, want in zip(ctx.dconv_W + ctx.dconv_b + ctx.dfc_W + ctx.dfc_b, ref.dW_conv + ref.db_conv + ref.dW_fc + ref.db_fc):
+        fro, mx = rel_err(got.double().cpu().numpy(), want)
+        assert fro <= TOL["f32"] and mx <= TOL["f32"]
