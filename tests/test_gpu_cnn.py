@@ -110,3 +110,58 @@ def test_padding_is_not_multiplied_with_an_infinite_filter(cin):
     for got, want in zip(ctx.dconv_W + ctx.dconv_b + ctx.dfc_W + ctx.dfc_b, ref.dW_conv + ref.db_conv + ref.dW_fc + ref.db_fc):
         fro, mx = rel_err(got.double().cpu().numpy(), want)
         assert fro <= TOL["f32"] and mx <= TOL["f32"]
+
+
+@pytest.mark.parametrize("cin", [1, 3])
+@pytest.mark.parametrize("where", ["gradient", "gradient of a unit that was not active", "input"])
+def test_first_convolution_backward_keeps_infinities_where_they_belong(cin, where):
+    """Backward of the first convolution with one infinity: in the gradient of a pooled output (it reaches the filter entries
+    whose kept inputs its four pixels see, and the bias gradient of its channel), in the gradient of an output none of
+    whose pixels passed the ReLU (it reaches nothing), in a kept input at the corner of the image (it reaches its own
+    channel's taps that lie inside).  Reference: the kept entries one by one, taps outside the image left out."""
+    import paper_2007_10412_b200 as rad
+    from oracle import rad as orad
+    hw, co, p, seed, step, C = 4, 8, (1.0 if where == "input" else 0.3), 6, 2, 2
+    X, _, cW, cb, fW, fb = cnn_inputs(1, hw, cin, (co,), (C,), "f32", seed=5, bias_zero=False)
+    y = np.array([1], np.int32)
+    W = cW[0].copy()
+    if where == "input":
+        X[0, 0, 0, 0] = np.inf
+        W[:, :, 0, :] = -np.abs(W[:, :, 0, :])              # its outputs are -inf before the ReLU, 0 after it
+    X64, W64 = X.astype(np.float64), W.astype(np.float64)
+    Z = np.zeros((hw, hw, co)) + cb[0]
+    taps = [(yy, xx, ky, kx) for yy in range(hw) for xx in range(hw) for ky in range(3) for kx in range(3)
+            if 0 <= yy + ky - 1 < hw and 0 <= xx + kx - 1 < hw]       # output pixel and tap; the input lies inside
+    for yy, xx, ky, kx in taps:
+        Z[yy, xx] += X64[0, yy + ky - 1, xx + kx - 1] @ W64[ky, kx]
+    on = Z > 0
+    active = on.reshape(hw // 2, 2, hw // 2, 2, co).sum(axis=(1, 3)).reshape(-1)              # pixels of a window that passed
+    P = np.where(on, Z, 0.0).reshape(hw // 2, 2, hw // 2, 2, co).mean(axis=(1, 3)).reshape(-1)
+    # logits one of which is far above the other: softmax - onehot is exactly (1, -1), so dP = F[:, 0] - F[:, 1]
+    F = fW[0] * np.float32(1e-3)
+    F[int(np.argmax(P))] = (1e6, -1e6)
+    hot = int(np.argmin(np.where(active > 0, P, np.inf))) if where == "gradient" else int(np.argmin(active))
+    assert (active[hot] > 0) == (where == "gradient") and P[hot] < 0.9
+    if where != "input":
+        F[hot] = (1.8e38, -1.8e38)
+    with np.errstate(all="ignore"):
+        dP = (F[:, 0].astype(np.float32) - F[:, 1].astype(np.float32)).astype(np.float32)
+        assert np.isinf(dP[hot]) == (where != "input")
+        dZ = np.where(on, np.repeat(np.repeat(0.25 * dP.astype(np.float64).reshape(hw // 2, hw // 2, co), 2, 0), 2, 1), 0.0)
+        keep = orad.keep_mask("different", 1, hw * hw * cin, p, seed, 0, step).reshape(hw, hw, cin)
+        A = X64[0] * float(orad.scale_factor(p))
+        want = np.zeros((3, 3, cin, co))
+        for yy, xx, ky, kx in taps:
+            for ci in range(cin):
+                if keep[yy + ky - 1, xx + kx - 1, ci]:
+                    want[ky, kx, ci] += A[yy + ky - 1, xx + kx - 1, ci] * dZ[yy, xx]
+        want_b = dZ.sum(axis=(0, 1))
+    ctx = rad.CNNStep(1, hw, cin, (co,), (C,), "f32", "different", p)
+    ctx(to_dev(X, "f32"), torch.from_numpy(y).cuda(), [to_dev(W, "f32")], [to_dev(cb[0], "f32")], [to_dev(F, "f32")],
+        [torch.zeros(C, device="cuda")], seed=seed, step=step)
+    torch.cuda.synchronize()
+    for got, ref in ((ctx.dconv_W[0], want), (ctx.dconv_b[0], want_b)):
+        got = got.double().cpu().numpy()
+        assert (np.isfinite(got) == np.isfinite(ref)).all()
+        ok = np.isfinite(ref)
+        assert ok.any() and (np.abs(got[ok] - ref[ok]) <= 1e-5 * np.abs(ref[ok]).max()).all()
