@@ -1,8 +1,14 @@
-"""The library beside other work: a second stream of the caller while a long kernel runs and the next one waits for it."""
+"""The library beside other work and inside a CUDA graph: kernels are launched before the kernel ahead of them in the stream
+has ended, which must neither hold up nor mix with what other streams do."""
 import time
 
+import numpy as np
 import pytest
 import torch
+
+from workloads import cnn_inputs, irnn_inputs, mlp_inputs
+
+from gpu_util import to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -35,3 +41,77 @@ def test_a_waiting_kernel_leaves_room_for_another_stream():
         torch.cuda.synchronize()
     assert begin.elapsed_time(done) > 3.0
     assert begin.elapsed_time(beside) < 0.7 * begin.elapsed_time(done)
+
+
+def _step(name, seed):
+    """(step context, its inputs on the device, its results) of a small net."""
+    import paper_2007_10412_b200 as rad
+    kind, dtype, variant = name.split()
+    if kind == "mlp":
+        dims, B = ((70, 52, 33, 10), 90) if dtype == "f32" else ((256, 320, 520, 64), 300)
+        X, y, Ws, bs = mlp_inputs(dims, B, dtype, "normal", seed=seed, bias_zero=False)
+        ctx = rad.MLPStep(dims, B, dtype, "relu", variant, 0.3)
+        args = [to_dev(X, dtype), torch.from_numpy(y).cuda(), [to_dev(W, dtype) for W in Ws], [to_dev(b, "f32") for b in bs]]
+        outs = [ctx.loss, ctx.nnz] + ctx.dW + ctx.db
+    elif kind == "irnn":
+        args = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in irnn_inputs(20, 37, 60, 7, seed=seed, identity=False)]
+        ctx = rad.IRNNStep(20, 37, 60, 7, variant, 0.3)
+        outs = [ctx.loss, ctx.nnz, ctx.dW_hh, ctx.dW_ih, ctx.db, ctx.dW_out, ctx.db_out]
+    else:
+        X, y, cW, cb, fW, fb = cnn_inputs(70, 16, 3, (16, 32), (24, 8), dtype, seed=seed, bias_zero=False)
+        ctx = rad.CNNStep(70, 16, 3, (16, 32), (24, 8), dtype, variant, 0.3)
+        args = [to_dev(X, dtype), torch.from_numpy(y).cuda()] + [[to_dev(w, dtype) for w in cW], [to_dev(b, "f32") for b in cb],
+                                                                 [to_dev(w, dtype) for w in fW], [to_dev(b, "f32") for b in fb]]
+        outs = [ctx.loss, ctx.nnz] + ctx.dconv_W + ctx.dconv_b + ctx.dfc_W + ctx.dfc_b
+    return ctx, args, outs
+
+
+STEPS = ["mlp f32 different", "mlp f32 same", "mlp bf16 different", "mlp bf16 same", "mlp bf16 redrawn", "irnn f32 different",
+         "cnn f32 different", "cnn bf16 different", "cnn bf16 same"]
+
+
+@pytest.mark.parametrize("name", STEPS)
+def test_a_captured_step_replays_bit_for_bit(name):
+    """A training step captured into a CUDA graph gives the results of the plain call, on the inputs of the capture and on
+    others written to the same buffers (sums have a fixed order: equality is exact)."""
+    ctx, args, outs = _step(name, seed=1)
+    _, other, _ = _step(name, seed=2)
+    keep = args[0].clone()
+    want = []
+    for x in (keep, other[0]):
+        args[0].copy_(x)
+        ctx(*args)
+        want.append([o.clone() for o in outs])
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx(*args)
+    for x, ref in zip((keep, other[0], keep), (want[0], want[1], want[0])):
+        args[0].copy_(x)
+        for o in outs:
+            o.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert ctx.dev_status.item() == 0
+        assert all(torch.equal(o, r) for o, r in zip(outs, ref))
+
+
+def test_steps_of_two_streams_at_once():
+    """Different nets stepping on streams of their own at the same time, each with its own workspace: the results are those of
+    the nets stepping alone."""
+    steps = [_step(name, seed=3 + i) for i, name in enumerate(STEPS)]
+    want = []
+    for ctx, args, outs in steps:
+        ctx(*args)
+        want.append([o.clone() for o in outs])
+        for o in outs:
+            o.zero_()
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in steps]
+    for _ in range(5):
+        for stream, (ctx, args, _) in zip(streams, steps):
+            with torch.cuda.stream(stream):
+                ctx(*args)
+    torch.cuda.synchronize()
+    for (ctx, _, outs), ref in zip(steps, want):
+        assert ctx.dev_status.item() == 0
+        assert all(torch.equal(o, r) for o, r in zip(outs, ref))
