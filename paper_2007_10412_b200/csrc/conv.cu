@@ -37,7 +37,7 @@ struct ConvShape {
 // The patch in registers is compiled for three channels, the images of the configured net; the loop that reads its entries
 // tap by tap, four channels at a time, takes the others (whole CNN steps against one thread per output channel: 1 channel,
 // batch 4096 bf16 4010 -> 1107 us; 4 channels 4874 -> 1429; 5 channels, batch 512 float32 1854 -> 1270; 16 channels 2845 -> 2391).
-// Bound by the FMA pipes (first convolution of the CNN, 32 x 32 x 3 -> 16: batch 4096 1405 -> 136 us, with one thread
+// Bound by the FMA pipes (first convolution of the CNN, 32 x 32 x 3 -> 16: batch 4096 1405 -> 148 us, 12 of it for the look at the sums, with one thread
 // per output channel, four shared-memory reads per four multiply-adds and a bounds test per input entry before).
 constexpr int kConvCo = 8;
 template <typename T, int kCin>
@@ -341,7 +341,7 @@ __global__ void conv_weight_grad_kernel(const ConvDwParams p) {
 // which saves tests but holds for finite numbers only.  A CTA whose sums do not come out finite walks its rows again,
 // touching no more than the cells that an entry or a gradient reaches.
 // Bound by instruction issue (about fourteen per kept entry and thread).  CNN, batch 4096: 134 (dZ) + 35 (bias) +
-// 397 + 293 us (filter, row sums) before, 152 + 7 us now; batch 128: 7 + 27 + 100 + 12 us before, 17 + 5 us now.
+// 397 + 293 us (filter, row sums) before, 158 + 7 us now; batch 128: 7 + 27 + 100 + 12 us before, 18 + 5 us now.
 struct ConvFirstParams {
   ConvShape s;
   int32_t variant;
