@@ -379,157 +379,157 @@ __global__ void __launch_bounds__(kFirstThreads) conv_first_backward_kernel(cons
   float db[8] = {};
   const T* vals = static_cast<const T*>(p.values);
   for (bool careful = false;; careful = true) {
-  for (int64_t b = blockIdx.x; b < s.B; b += gridDim.x) {
-    __syncthreads();                                                // the row before has been read
-    if (b + gridDim.x >= s.B) let_next_start();
-    if (tid == 0) s_count = 0;
-    if (tid < stride)
-      for (int i = tid; i < nvec; i += stride) {
-        const int win = i / groups, yp = win / Wp, xp = win - yp * Wp;
-        const int64_t at = (b * Hp * Wp + win) * Cout + g8;
-        const uint32_t bits = p.relubits[at >> 3];
-        T g[8];
-        if constexpr (sizeof(T) == 2) {
-          const uint4 v = *reinterpret_cast<const uint4*>(static_cast<const T*>(p.dP) + at);
-          memcpy(g, &v, 16);
-        } else {
-          const float4 v0 = *reinterpret_cast<const float4*>(static_cast<const T*>(p.dP) + at);
-          const float4 v1 = *reinterpret_cast<const float4*>(static_cast<const T*>(p.dP) + at + 4);
-          memcpy(g, &v0, 16); memcpy(g + 4, &v1, 16);
-        }
-        if (careful) {                                              // none of its four pixels passed the ReLU: it goes nowhere
+    for (int64_t b = blockIdx.x; b < s.B; b += gridDim.x) {
+      __syncthreads();                                                // the row before has been read
+      if (b + gridDim.x >= s.B) let_next_start();
+      if (tid == 0) s_count = 0;
+      if (tid < stride)
+        for (int i = tid; i < nvec; i += stride) {
+          const int win = i / groups, yp = win / Wp, xp = win - yp * Wp;
+          const int64_t at = (b * Hp * Wp + win) * Cout + g8;
+          const uint32_t bits = p.relubits[at >> 3];
+          T g[8];
+          if constexpr (sizeof(T) == 2) {
+            const uint4 v = *reinterpret_cast<const uint4*>(static_cast<const T*>(p.dP) + at);
+            memcpy(g, &v, 16);
+          } else {
+            const float4 v0 = *reinterpret_cast<const float4*>(static_cast<const T*>(p.dP) + at);
+            const float4 v1 = *reinterpret_cast<const float4*>(static_cast<const T*>(p.dP) + at + 4);
+            memcpy(g, &v0, 16); memcpy(g + 4, &v1, 16);
+          }
+          if (careful) {                                              // none of its four pixels passed the ReLU: it goes nowhere
 #pragma unroll
-          for (int c = 0; c < 8; ++c) g[c] = (bits >> (4 * c)) & 0xfu ? g[c] : from_float<T>(0.0f);
-        }
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          g[c] = from_float<T>(0.25f * to_float(g[c]));
-          db[c] += (float)__popc((bits >> (4 * c)) & 0xfu) * to_float(g[c]);
-        }
-#pragma unroll
-        for (int o = 0; o < 4; ++o) {
-          T z[8];
-#pragma unroll
-          for (int c = 0; c < 8; ++c) z[c] = (bits >> (4 * c + o)) & 1u ? g[c] : from_float<T>(0.0f);
-          uint4 v[sizeof(T) / 2];
-          memcpy(v, z, sizeof(z));
-          uint4* dst = reinterpret_cast<uint4*>(s_dz + ((2 * yp + (o >> 1) + 1) * Wq + 2 * xp + (o & 1) + 1) * Cout + g8);
-#pragma unroll
-          for (int q = 0; q < (int)sizeof(T) / 2; ++q) dst[q] = v[q];
-        }
-      }
-    auto put = [&](uint32_t at, int col, float v) {
-      const int pix = col / kCin, ci = col - pix * kCin, y = pix / s.W, x = pix - y * s.W;
-      if (at < (uint32_t)p.list_cap)
-        s_list[at] = make_uint2((uint32_t)(((y + 2) * Wq + x + 2) * Cout) << 2 | (uint32_t)ci, __float_as_uint(v));
-    };
-    __syncthreads();
-    if (p.variant == RAD_SAME_SAMPLE) {
-      const int64_t k = min(p.nnz[0], p.values_ld);
-      for (int64_t j = tid; j < k; j += kFirstThreads) put((uint32_t)j, (int)p.offsets[j], to_float(vals[b * p.values_ld + j]));
-      if (tid == 0) s_count = (uint32_t)min(k, (int64_t)p.list_cap);
-    } else {
-      // row b of the tile-major store: slab b / 64, row r inside it; one keep-bit word per thread and pass
-      const int64_t slab = b / kTileRows;
-      const int r = (int)(b % kTileRows), nwords = p.ncb * 4;
-      for (int w0 = 0; w0 < nwords; w0 += kFirstThreads) {
-        const int wi = w0 + tid;
-        uint32_t word = 0, inrow = 0;
-        int64_t tile = slab * p.ncb;
-        if (wi < nwords) {
-          tile += wi >> 2;
-          const uint32_t* tb = p.keepbits + tile * kTileWords;
-          word = tb[r * 4 + (wi & 3)];
-          for (int q = 0; q < (wi & 3); ++q) inrow += __popc(tb[r * 4 + q]);
-          inrow += (tb[kBitWords + (r >> 1)] >> (16 * (r & 1))) & 0xffffu;          // row offset inside the tile
-        }
-        const uint32_t c = __popc(word);
-        uint32_t incl = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t n = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += n;
-        }
-        if (lane == 31) s_scan[warp] = incl;
-        int64_t vpos = (int64_t)p.offsets[tile] + inrow;
-        __syncthreads();
-        uint32_t at = s_count + incl - c;
-        for (int q = 0; q < warp; ++q) at += s_scan[q];
-        const int col0 = (wi >> 2) * kTileCols + (wi & 3) * 32;
-        while (word != 0) {                                         // four values in flight
-          int bit[4];
-          float v[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            bit[i] = word != 0 ? __ffs(word) - 1 : -1;
-            word &= word - 1;
-            v[i] = bit[i] >= 0 && vpos + i < p.values_capacity ? to_float(vals[vpos + i]) : 0.0f;
+            for (int c = 0; c < 8; ++c) g[c] = (bits >> (4 * c)) & 0xfu ? g[c] : from_float<T>(0.0f);
           }
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (bit[i] >= 0) put(at + i, col0 + bit[i], v[i]);
-          at += 4; vpos += 4;
+          for (int c = 0; c < 8; ++c) {
+            g[c] = from_float<T>(0.25f * to_float(g[c]));
+            db[c] += (float)__popc((bits >> (4 * c)) & 0xfu) * to_float(g[c]);
+          }
+#pragma unroll
+          for (int o = 0; o < 4; ++o) {
+            T z[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) z[c] = (bits >> (4 * c + o)) & 1u ? g[c] : from_float<T>(0.0f);
+            uint4 v[sizeof(T) / 2];
+            memcpy(v, z, sizeof(z));
+            uint4* dst = reinterpret_cast<uint4*>(s_dz + ((2 * yp + (o >> 1) + 1) * Wq + 2 * xp + (o & 1) + 1) * Cout + g8);
+#pragma unroll
+            for (int q = 0; q < (int)sizeof(T) / 2; ++q) dst[q] = v[q];
+          }
         }
-        __syncthreads();
-        if (tid == 0) {
-          uint32_t tot = s_count;
-          for (int q = 0; q < kFirstThreads / 32; ++q) tot += s_scan[q];
-          s_count = min(tot, (uint32_t)p.list_cap);
+      auto put = [&](uint32_t at, int col, float v) {
+        const int pix = col / kCin, ci = col - pix * kCin, y = pix / s.W, x = pix - y * s.W;
+        if (at < (uint32_t)p.list_cap)
+          s_list[at] = make_uint2((uint32_t)(((y + 2) * Wq + x + 2) * Cout) << 2 | (uint32_t)ci, __float_as_uint(v));
+      };
+      __syncthreads();
+      if (p.variant == RAD_SAME_SAMPLE) {
+        const int64_t k = min(p.nnz[0], p.values_ld);
+        for (int64_t j = tid; j < k; j += kFirstThreads) put((uint32_t)j, (int)p.offsets[j], to_float(vals[b * p.values_ld + j]));
+        if (tid == 0) s_count = (uint32_t)min(k, (int64_t)p.list_cap);
+      } else {
+        // row b of the tile-major store: slab b / 64, row r inside it; one keep-bit word per thread and pass
+        const int64_t slab = b / kTileRows;
+        const int r = (int)(b % kTileRows), nwords = p.ncb * 4;
+        for (int w0 = 0; w0 < nwords; w0 += kFirstThreads) {
+          const int wi = w0 + tid;
+          uint32_t word = 0, inrow = 0;
+          int64_t tile = slab * p.ncb;
+          if (wi < nwords) {
+            tile += wi >> 2;
+            const uint32_t* tb = p.keepbits + tile * kTileWords;
+            word = tb[r * 4 + (wi & 3)];
+            for (int q = 0; q < (wi & 3); ++q) inrow += __popc(tb[r * 4 + q]);
+            inrow += (tb[kBitWords + (r >> 1)] >> (16 * (r & 1))) & 0xffffu;          // row offset inside the tile
+          }
+          const uint32_t c = __popc(word);
+          uint32_t incl = c;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t n = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += n;
+          }
+          if (lane == 31) s_scan[warp] = incl;
+          int64_t vpos = (int64_t)p.offsets[tile] + inrow;
+          __syncthreads();
+          uint32_t at = s_count + incl - c;
+          for (int q = 0; q < warp; ++q) at += s_scan[q];
+          const int col0 = (wi >> 2) * kTileCols + (wi & 3) * 32;
+          while (word != 0) {                                         // four values in flight
+            int bit[4];
+            float v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              bit[i] = word != 0 ? __ffs(word) - 1 : -1;
+              word &= word - 1;
+              v[i] = bit[i] >= 0 && vpos + i < p.values_capacity ? to_float(vals[vpos + i]) : 0.0f;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (bit[i] >= 0) put(at + i, col0 + bit[i], v[i]);
+            at += 4; vpos += 4;
+          }
+          __syncthreads();
+          if (tid == 0) {
+            uint32_t tot = s_count;
+            for (int q = 0; q < kFirstThreads / 32; ++q) tot += s_scan[q];
+            s_count = min(tot, (uint32_t)p.list_cap);
+          }
+          if (w0 + kFirstThreads < nwords) __syncthreads();
         }
-        if (w0 + kFirstThreads < nwords) __syncthreads();
       }
-    }
-    __syncthreads();
-    if (worker && careful) {
-      const uint32_t n = s_count;
+      __syncthreads();
+      if (worker && careful) {
+        const uint32_t n = s_count;
 #pragma unroll 1
-      for (uint32_t e = (uint32_t)part; e < n; e += (uint32_t)p.parts) {
-        const uint2 q = s_list[e];
-        const int pix = (int)(q.x >> 2) / Cout, y = pix / Wq - tap / 3, x = pix % Wq - tap % 3;      // in the bordered image
-        if (y < 1 || y > s.H || x < 1 || x > s.W) continue;
-        const T* z = s_dz + (y * Wq + x) * Cout + 2 * cp;
+        for (uint32_t e = (uint32_t)part; e < n; e += (uint32_t)p.parts) {
+          const uint2 q = s_list[e];
+          const int pix = (int)(q.x >> 2) / Cout, y = pix / Wq - tap / 3, x = pix % Wq - tap % 3;      // in the bordered image
+          if (y < 1 || y > s.H || x < 1 || x > s.W) continue;
+          const T* z = s_dz + (y * Wq + x) * Cout + 2 * cp;
 #pragma unroll
-        for (int ci = 0; ci < kCin; ++ci) {
-          const bool mine = (q.x & 3u) == (uint32_t)ci;
-          const float a0 = fmaf(__uint_as_float(q.y), to_float(z[0]), acc[ci][0]), a1 = fmaf(__uint_as_float(q.y), to_float(z[1]), acc[ci][1]);
-          acc[ci][0] = mine ? a0 : acc[ci][0];
-          acc[ci][1] = mine ? a1 : acc[ci][1];
+          for (int ci = 0; ci < kCin; ++ci) {
+            const bool mine = (q.x & 3u) == (uint32_t)ci;
+            const float a0 = fmaf(__uint_as_float(q.y), to_float(z[0]), acc[ci][0]), a1 = fmaf(__uint_as_float(q.y), to_float(z[1]), acc[ci][1]);
+            acc[ci][0] = mine ? a0 : acc[ci][0];
+            acc[ci][1] = mine ? a1 : acc[ci][1];
+          }
         }
-      }
-    } else if (worker) {
-      const uint32_t n = s_count;
+      } else if (worker) {
+        const uint32_t n = s_count;
 #pragma unroll 4
-      for (uint32_t e = (uint32_t)part; e < n; e += (uint32_t)p.parts) {
-        const uint2 q = s_list[e];
-        const T* z = s_dz + ((int)(q.x >> 2) - tap_off);
-        float z0, z1;
-        if constexpr (sizeof(T) == 2) {
-          const uint32_t zz = *reinterpret_cast<const uint32_t*>(z);
-          z0 = __uint_as_float(zz << 16); z1 = __uint_as_float(zz & 0xffff0000u);
-        } else {
-          const float2 zz = *reinterpret_cast<const float2*>(z);
-          z0 = zz.x; z1 = zz.y;
-        }
-        const float v = __uint_as_float(q.y);
+        for (uint32_t e = (uint32_t)part; e < n; e += (uint32_t)p.parts) {
+          const uint2 q = s_list[e];
+          const T* z = s_dz + ((int)(q.x >> 2) - tap_off);
+          float z0, z1;
+          if constexpr (sizeof(T) == 2) {
+            const uint32_t zz = *reinterpret_cast<const uint32_t*>(z);
+            z0 = __uint_as_float(zz << 16); z1 = __uint_as_float(zz & 0xffff0000u);
+          } else {
+            const float2 zz = *reinterpret_cast<const float2*>(z);
+            z0 = zz.x; z1 = zz.y;
+          }
+          const float v = __uint_as_float(q.y);
 #pragma unroll
-        for (int ci = 0; ci < kCin; ++ci) {
-          const float vc = kCin == 1 || (q.x & 3u) == (uint32_t)ci ? v : 0.0f;
-          acc[ci][0] = fmaf(vc, z0, acc[ci][0]);
-          acc[ci][1] = fmaf(vc, z1, acc[ci][1]);
+          for (int ci = 0; ci < kCin; ++ci) {
+            const float vc = kCin == 1 || (q.x & 3u) == (uint32_t)ci ? v : 0.0f;
+            acc[ci][0] = fmaf(vc, z0, acc[ci][0]);
+            acc[ci][1] = fmaf(vc, z1, acc[ci][1]);
+          }
         }
       }
     }
-  }
-  float odd = 0.0f;                                                 // NaN if a sum of this thread is not finite
+    float odd = 0.0f;                                                 // NaN if a sum of this thread is not finite
 #pragma unroll
-  for (int c = 0; c < 8; ++c) odd = fmaf(db[c], 0.0f, odd);
+    for (int c = 0; c < 8; ++c) odd = fmaf(db[c], 0.0f, odd);
 #pragma unroll
-  for (int ci = 0; ci < kCin; ++ci) odd = fmaf(acc[ci][1], 0.0f, fmaf(acc[ci][0], 0.0f, odd));
-  if (!__syncthreads_or(odd != 0.0f ? 1 : 0) || careful) break;
+    for (int ci = 0; ci < kCin; ++ci) odd = fmaf(acc[ci][1], 0.0f, fmaf(acc[ci][0], 0.0f, odd));
+    if (!__syncthreads_or(odd != 0.0f ? 1 : 0) || careful) break;
 #pragma unroll
-  for (int c = 0; c < 8; ++c) db[c] = 0.0f;
+    for (int c = 0; c < 8; ++c) db[c] = 0.0f;
 #pragma unroll
-  for (int ci = 0; ci < kCin; ++ci) acc[ci][0] = acc[ci][1] = 0.0f;
+    for (int ci = 0; ci < kCin; ++ci) acc[ci][0] = acc[ci][1] = 0.0f;
   }
   // the parts' filter sums and the staging threads' bias sums, added in order
   const int ncell = 9 * kCin * Cout;
