@@ -19,7 +19,7 @@
 //                    contiguous in the filter tensor); the epilogue rounds and writes 64 bytes per row and chunk.
 //
 // One CTA (no cluster), eight warps: all of them write operand tiles with the 128-byte swizzle the tensor core
-// expects (16-byte chunk c of row r lands at chunk c ^ (r & 7)), thread 0 issues tcgen05.mma.cta_group::1
+// expects (16-byte chunk c of row r lands at chunk c ^ (r & 7)), one elected thread issues tcgen05.mma.cta_group::1
 // (M128 N64 K16), two shared-memory stages alternate, the 128 x 64 accumulator takes 64 columns of tensor
 // memory.  Every wait is bounded; on expiry the CTA raises RAD_DEV_ETIMEOUT, frees its tensor memory and returns.
 #include <algorithm>
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(kCvThreads, 3) conv_tc_kernel(const ConvTcPara
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (!__syncthreads_and(ok ? 1 : 0)) { ok = false; break; }
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       constexpr uint32_t idesc = cv_idesc(kDw, !kDx);
       const uint32_t a0 = cv_smem(sA), b0 = cv_smem(sB);

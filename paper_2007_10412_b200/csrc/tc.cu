@@ -599,88 +599,81 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
 
   if (warp == 0) {
     // ===== TMA producer: this CTA's 128 rows of A and 128 rows (N) of B, completing on the even CTA's barrier =====
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true;
-    for (int64_t u = pair; u < sched.units && ok; u += npairs) {
-      const Unit w = sched.unit(u);
-      if (u + npairs >= sched.units) let_next_start();
-      const int m_own = (int)w.m0 + 128 * (int)rank, n_own = (int)w.n0 + (bn / 2) * (int)rank;
-      for (int kb = w.kb0; kb < w.kb1; ++kb) {
-        if (lane == 0) {
-          ok = mbar_wait2(smem_u32(&ctl->empty[stage]), phase ^ 1u, wc);
-          if (ok) {
-            const uint32_t sA = smem_base + stage * kStage2Bytes;
-            const uint32_t sB = sA + kStage2Bytes / 2;
-            const uint32_t full = map_to_cta(smem_u32(&ctl->full[stage]), 0u);
-            const int k0 = kb * BK;
-            if (rank == 0) mbar_arrive_expect_tx(smem_u32(&ctl->full[stage]), stage_tx);   // both CTAs' bytes
-            if (AK == kAK) {
-              tma_load_2d_pair(sA, &tmA, k0, m_own, full);                         // 64 (K) x 128 rows
-            } else {
+    if (elect_one()) {
+      const uint32_t full0 = map_to_cta(smem_u32(&ctl->full[0]), 0u);
+      int stage = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      for (int64_t u = pair; u < sched.units && ok; u += npairs) {
+        const Unit w = sched.unit(u);
+        if (u + npairs >= sched.units) let_next_start();
+        const int m_own = (int)w.m0 + 128 * (int)rank, n_own = (int)w.n0 + (bn / 2) * (int)rank;
+        for (int kb = w.kb0; kb < w.kb1; ++kb) {
+          ok = mbar_wait2(smem_u32(&ctl->empty[0]) + 8u * stage, phase ^ 1u, wc);
+          if (!ok) break;
+          const uint32_t sA = smem_base + stage * kStage2Bytes;
+          const uint32_t sB = sA + kStage2Bytes / 2;
+          const uint32_t full = full0 + 8u * stage;
+          const int k0 = kb * BK;
+          if (rank == 0) mbar_arrive_expect_tx(smem_u32(&ctl->full[0]) + 8u * stage, stage_tx);   // both CTAs' bytes
+          if (AK == kAK) {
+            tma_load_2d_pair(sA, &tmA, k0, m_own, full);                         // 64 (K) x 128 rows
+          } else {
 #pragma unroll
-              for (int c = 0; c < 2; ++c) tma_load_2d_pair(sA + c * 8192, &tmA, m_own + c * 64, k0, full);
-            }
-            if (BKIND == kBK_) {
-              tma_load_2d_pair(sB, &tmB, k0, n_own, full);
-            } else {
-#pragma unroll
-              for (int c = 0; c < 2; ++c)
-                if (c < boxes_b) tma_load_2d_pair(sB + c * 8192, &tmB, n_own + c * 64, k0, full);
-            }
+            for (int c = 0; c < 2; ++c) tma_load_2d_pair(sA + c * 8192, &tmA, m_own + c * 64, k0, full);
           }
+          if (BKIND == kBK_) {
+            tma_load_2d_pair(sB, &tmB, k0, n_own, full);
+          } else {
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+              if (c < boxes_b) tma_load_2d_pair(sB + c * 8192, &tmB, n_own + c * 64, k0, full);
+          }
+          if (++stage == kStages2) { stage = 0; phase ^= 1u; }
         }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-        if (!ok) break;
-        if (++stage == kStages2) { stage = 0; phase ^= 1u; }
       }
-    }
-    // tail: every commit aimed at this CTA's stage barriers has landed before the CTA may leave
-    if (lane == 0) {
+      // tail: every commit aimed at this CTA's stage barriers has landed before the CTA may leave
       for (int i = 0; i < kStages2 && ok; ++i) {
-        ok = mbar_wait2(smem_u32(&ctl->empty[stage]), phase ^ 1u, wc);
+        ok = mbar_wait2(smem_u32(&ctl->empty[0]) + 8u * stage, phase ^ 1u, wc);
         if (++stage == kStages2) { stage = 0; phase ^= 1u; }
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
     // ===== MMA issuer: one thread of the even CTA drives both tensor cores =====
-    if (rank == 0) {
+    if (rank == 0 && elect_one()) {
       const uint32_t idesc = make_idesc_pair(AK != kAK, BKIND == kBMN, (uint32_t)bn);
+      // descriptors of stage 0; a step of 16 K rows and a stage are additions to the address field
+      const uint64_t adesc0 = AK == kAK ? make_desc(smem_base, 16, 1024) : make_desc(smem_base, 8192, 1024);
+      const uint64_t bdesc0 = BKIND == kBK_ ? make_desc(smem_base + kStage2Bytes / 2, 16, 1024)
+                                            : make_desc(smem_base + kStage2Bytes / 2, 8192, 1024);
+      constexpr uint32_t a_step = (AK == kAK ? 32 : 2048) >> 4, b_step = (BKIND == kBK_ ? 32 : 2048) >> 4;
       int stage = 0, buf = 0;
       uint32_t phase = 0, buf_phases = 0;          // bit b: phase of accumulator b
       bool ok = true;
       for (int64_t u = pair; u < sched.units && ok; u += npairs) {
         const Unit w = sched.unit(u);
-        if (lane == 0)
-          ok = mbar_wait2(smem_u32(&ctl->tmem_empty[0]) + 8u * buf, ((buf_phases >> buf) & 1u) ^ 1u, wc);
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        ok = mbar_wait2(smem_u32(&ctl->tmem_empty[0]) + 8u * buf, ((buf_phases >> buf) & 1u) ^ 1u, wc);
         if (!ok) break;
         tc_fence_after();
         for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          if (lane == 0) {
-            ok = mbar_wait2(smem_u32(&ctl->full[stage]), phase, wc);
-            if (ok) {
-              tc_fence_after();
-              const uint32_t sA = smem_base + stage * kStage2Bytes;
-              const uint32_t sB = sA + kStage2Bytes / 2;
-#pragma unroll
-              for (int k = 0; k < BK / 16; ++k) {
-                const uint64_t adesc = (AK == kAK) ? make_desc(sA + k * 32, 16, 1024) : make_desc(sA + k * 2048, 8192, 1024);
-                const uint64_t bdesc = (BKIND == kBK_) ? make_desc(sB + k * 32, 16, 1024) : make_desc(sB + k * 2048, 8192, 1024);
-                tc_mma_pair(tmem_base + buf * 256, adesc, bdesc, idesc, (kb > w.kb0 || k > 0) ? 1u : 0u);
-              }
-              tc_commit_pair(smem_u32(&ctl->empty[stage]));          // frees the stage in both CTAs
-              if (kb == w.kb1 - 1) tc_commit_pair(smem_u32(&ctl->tmem_full[0]) + 8u * buf);
-            }
-          }
-          ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+          ok = mbar_wait2(smem_u32(&ctl->full[0]) + 8u * stage, phase, wc);
           if (!ok) break;
+          tc_fence_after();
+          const uint64_t adesc = adesc0 + (uint32_t)(stage * (kStage2Bytes >> 4));
+          const uint64_t bdesc = bdesc0 + (uint32_t)(stage * (kStage2Bytes >> 4));
+#pragma unroll
+          for (int k = 0; k < BK / 16; ++k)
+            tc_mma_pair(tmem_base + buf * 256, adesc + k * a_step, bdesc + k * b_step, idesc, (kb > w.kb0 || k > 0) ? 1u : 0u);
+          tc_commit_pair(smem_u32(&ctl->empty[0]) + 8u * stage);           // frees the stage in both CTAs
           if (++stage == kStages2) { stage = 0; phase ^= 1u; }
         }
+        if (ok) tc_commit_pair(smem_u32(&ctl->tmem_full[0]) + 8u * buf);
         buf_phases ^= 1u << buf;
         buf ^= 1;
       }
     }
+    __syncwarp();
   } else {
     // ===== epilogue: thread = one accumulator row of this CTA =====
     const int q = warp & 3;
@@ -845,75 +838,66 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
 
   if (warp == 0) {
     // ===== dZ producer: this CTA's 128 columns of each 256-column half of the dZ tile =====
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true;
-    for (int64_t u = pair; u < sched.units && ok; u += npairs) {
-      const Unit w = sched.unit(u);
-      if (u + npairs >= sched.units) let_next_start();
-      const int n_own = (int)w.n0 + 128 * (int)rank;       // + 256 for the second half
-      for (int kb = w.kb0; kb < w.kb1; ++kb) {
-        if (lane == 0) {
-          ok = mbar_wait2(smem_u32(&ctl->empty[stage]), phase ^ 1u, wc);
-          if (ok) {
-            const uint32_t sB = smem_base + stage * kSpStageBytes + kSpAStageBytes;
-            if (rank == 0) mbar_arrive_expect_tx(smem_u32(&ctl->full[stage]), 2 * kSpBStageBytes);   // both CTAs' bytes
-            const uint32_t full = map_to_cta(smem_u32(&ctl->full[stage]), 0u);
+    if (elect_one()) {
+      const uint32_t full0 = map_to_cta(smem_u32(&ctl->full[0]), 0u);
+      int stage = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      for (int64_t u = pair; u < sched.units && ok; u += npairs) {
+        const Unit w = sched.unit(u);
+        if (u + npairs >= sched.units) let_next_start();
+        const int n_own = (int)w.n0 + 128 * (int)rank;       // + 256 for the second half
+        for (int kb = w.kb0; kb < w.kb1; ++kb) {
+          ok = mbar_wait2(smem_u32(&ctl->empty[0]) + 8u * stage, phase ^ 1u, wc);
+          if (!ok) break;
+          const uint32_t sB = smem_base + stage * kSpStageBytes + kSpAStageBytes;
+          if (rank == 0) mbar_arrive_expect_tx(smem_u32(&ctl->full[0]) + 8u * stage, 2 * kSpBStageBytes);   // both CTAs' bytes
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-              tma_load_2d_pair(sB + c * 8192, &tmB, n_own + (c >> 1) * 256 + (c & 1) * 64, kb * BK, full);
-          }
+          for (int c = 0; c < 4; ++c)
+            tma_load_2d_pair(sB + c * 8192, &tmB, n_own + (c >> 1) * 256 + (c & 1) * 64, kb * BK, full0 + 8u * stage);
+          if (++stage == stages) { stage = 0; phase ^= 1u; }
         }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-        if (!ok) break;
-        if (++stage == stages) { stage = 0; phase ^= 1u; }
       }
-    }
-    if (lane == 0) {   // every commit aimed at this CTA's stage barriers has landed before the CTA may leave
+      // every commit aimed at this CTA's stage barriers has landed before the CTA may leave
       for (int i = 0; i < stages && ok; ++i) {
-        ok = mbar_wait2(smem_u32(&ctl->empty[stage]), phase ^ 1u, wc);
+        ok = mbar_wait2(smem_u32(&ctl->empty[0]) + 8u * stage, phase ^ 1u, wc);
         if (++stage == stages) { stage = 0; phase ^= 1u; }
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
     // ===== MMA issuer (even CTA) =====
-    if (rank == 0) {
+    if (rank == 0 && elect_one()) {
       constexpr uint32_t idesc = make_idesc_pair(true, true);
+      const uint64_t adesc0 = make_desc(smem_base, 8192, 1024), bdesc0 = make_desc(smem_base + kSpAStageBytes, 8192, 1024);
       int stage = 0;
       uint32_t phase = 0, unit_phase = 0;
       bool ok = true;
       for (int64_t u = pair; u < sched.units && ok; u += npairs) {
         const Unit w = sched.unit(u);
-        if (lane == 0) ok = mbar_wait2(smem_u32(&ctl->tmem_empty), unit_phase ^ 1u, wc);
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        ok = mbar_wait2(smem_u32(&ctl->tmem_empty), unit_phase ^ 1u, wc);
         if (!ok) break;
         tc_fence_after();
         for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          if (lane == 0) {
-            ok = mbar_wait2(smem_u32(&ctl->full[stage]), phase, wc);
-            if (ok) {
-              tc_fence_after();
-              const uint32_t sA = smem_base + stage * kSpStageBytes;
-              const uint32_t sB = sA + kSpAStageBytes;
-#pragma unroll
-              for (int k = 0; k < BK / 16; ++k) {
-                const uint64_t adesc = make_desc(sA + k * 2048, 8192, 1024);
-#pragma unroll
-                for (int j = 0; j < 2; ++j)
-                  tc_mma_pair(tmem_base + j * 256, adesc, make_desc(sB + j * 16384 + k * 2048, 8192, 1024), idesc,
-                              (kb > w.kb0 || k > 0) ? 1u : 0u);
-              }
-              tc_commit_pair(smem_u32(&ctl->empty[stage]));
-              if (kb == w.kb1 - 1) tc_commit_pair(smem_u32(&ctl->tmem_full));
-            }
-          }
-          ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+          ok = mbar_wait2(smem_u32(&ctl->full[0]) + 8u * stage, phase, wc);
           if (!ok) break;
+          tc_fence_after();
+          const uint64_t adesc = adesc0 + (uint32_t)(stage * (kSpStageBytes >> 4));
+          const uint64_t bdesc = bdesc0 + (uint32_t)(stage * (kSpStageBytes >> 4));
+#pragma unroll
+          for (int k = 0; k < BK / 16; ++k)
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+              tc_mma_pair(tmem_base + j * 256, adesc + k * (2048 >> 4), bdesc + (j * 16384 + k * 2048) / 16, idesc,
+                          (kb > w.kb0 || k > 0) ? 1u : 0u);
+          tc_commit_pair(smem_u32(&ctl->empty[0]) + 8u * stage);
           if (++stage == stages) { stage = 0; phase ^= 1u; }
         }
+        if (ok) tc_commit_pair(smem_u32(&ctl->tmem_full));
         unit_phase ^= 1u;
       }
     }
+    __syncwarp();
   } else if (warp < 6) {
     // ===== epilogue: a warp = 32 accumulator rows, every kSpEpiShare-th 32-column chunk (the expanders take the others) =====
     uint32_t unit_phase = 0;
@@ -946,9 +930,10 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
         const int src = (kb - w.kb0) & 31;
         const uint32_t o0 = __shfl_sync(0xffffffffu, off_lo, src);
         const uint32_t o1 = __shfl_sync(0xffffffffu, off_hi, src);
-        if (lane == 0) {
-          ok = mbar_wait2(smem_u32(&ctl->comp_empty[slot]), cphase ^ 1u, wc);
-          if (ok) {
+        bool sent = true;
+        if (elect_one()) {
+          sent = mbar_wait2(smem_u32(&ctl->comp_empty[slot]), cphase ^ 1u, wc);
+          if (sent) {
             const uint32_t cfull = smem_u32(&ctl->comp_full[slot]);
             const uint32_t sC = smem_u32(comp_base) + slot * comp_slot;
             uint32_t vb = have ? (o1 - o0) * 2u : 0u;
@@ -963,7 +948,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
             }
           }
         }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        ok = __all_sync(0xffffffffu, sent);
         if (!ok) break;
         if (++slot == p.comp_depth) { slot = 0; cphase ^= 1u; }
       }
