@@ -137,184 +137,357 @@ struct Unit {
   int32_t split;
 };
 
+// 32-bit arithmetic: a matrix that fits the device has far fewer than 2^31 tiles, and a unit's place costs half a dozen
+// divisions, which nothing overlaps at the start of a launch (64-bit ones: 0.5 us before the first load).
 struct Schedule {
-  int64_t M, m_tiles, n_tiles, ntiles, units;
+  int64_t M;
+  uint32_t m_tiles, n_tiles, ntiles, units;
   int32_t kblocks, splits, bm, bn;
   __device__ Schedule(int64_t M_, int64_t N_, int64_t K_, int32_t splits_, int32_t bm_ = BM, int32_t bn_ = BN) {
     M = M_;
     bm = bm_;
     bn = bn_;
-    m_tiles = (M + bm - 1) / bm;
-    n_tiles = (N_ + bn - 1) / bn;
+    m_tiles = ((uint32_t)M + bm - 1) / bm;
+    n_tiles = ((uint32_t)N_ + bn - 1) / bn;
     ntiles = m_tiles * n_tiles;
-    kblocks = (int32_t)((K_ + BK - 1) / BK);
+    kblocks = (int32_t)(((uint32_t)K_ + BK - 1) / BK);
     splits = splits_;
     units = ntiles * splits;
   }
   // split-major order: CTAs of one wave work on the same K range, so operand panels shared by
   // tiles of a row or column of the grid are read from L2 at about the same time.
-  __device__ Unit unit(int64_t u) const {
+  __device__ Unit unit(uint32_t u) const {
     Unit w;
-    const int64_t s = u / ntiles, t = u % ntiles;
-    const int64_t per_group = kRasterGroup * n_tiles;
-    const int64_t g = t / per_group, r = t % per_group;
-    const int64_t first_m = g * kRasterGroup;
-    const int64_t gm = min((int64_t)kRasterGroup, m_tiles - first_m);
-    w.m0 = (first_m + r % gm) * bm;
-    w.n0 = (r / gm) * bn;
+    const uint32_t s = splits > 1 ? u / ntiles : 0, t = u - s * ntiles;
+    const uint32_t per_group = kRasterGroup * n_tiles;
+    const uint32_t g = t / per_group, r = t - g * per_group;
+    const uint32_t first_m = g * kRasterGroup;
+    const uint32_t gm = min((uint32_t)kRasterGroup, m_tiles - first_m), col = r / gm;
+    w.m0 = (int64_t)(first_m + r - col * gm) * bm;
+    w.n0 = (int64_t)col * bn;
     w.split = (int32_t)s;
-    w.kb0 = (int32_t)(s * kblocks / splits);
-    w.kb1 = (int32_t)((s + 1) * kblocks / splits);
+    w.kb0 = splits > 1 ? (int32_t)(s * (uint32_t)kblocks / (uint32_t)splits) : 0;
+    w.kb1 = splits > 1 ? (int32_t)((s + 1) * (uint32_t)kblocks / (uint32_t)splits) : kblocks;
     return w;
   }
 };
 
+// ---- epilogue of the forward pass and the input gradient ----------------------------------------------
+// A thread holds one accumulator row (32 columns of it at a time).  Storing from there would touch 32 lines of the output
+// per instruction for 16 bytes each, so every warp passes its chunk of 32 rows x 32 columns on through shared memory: a row
+// writes its 64 bytes (bf16) or 128 (float32), 16-byte units swizzled the way the tensor map says so that eight rows take
+// eight bank groups, and one TMA store takes the chunk away.  Rows and columns past the matrix are cut off by the tensor map.
+// What the epilogue reads (the next store's index, ReLU bits, z of the GELU derivative) is on its way before the
+// accumulators are waited for.
+constexpr int kEpiWarps = 8;
+constexpr int kChunkBytes = 32 * 64;             // 32 rows x 32 bf16 columns
+constexpr int kFillBytes = 3584;                 // staged values of the next store, per warp
+constexpr int kBiasBytes = 128 * 4;              // bias of a warp's columns
+constexpr int kEpiBytes = 4 * kChunkBytes + kFillBytes + kBiasBytes;   // of a warp: a ring of four chunks, and those
+constexpr uint32_t kFillValues = kFillBytes / 2;
+
+__device__ __forceinline__ uint32_t chunk16_addr(uint32_t base, int row, int unit) { return base + row * 64 + ((unit ^ ((row >> 1) & 3)) << 4); }
+__device__ __forceinline__ uint32_t chunk32_addr(uint32_t base, int row, int unit) { return base + row * 128 + ((unit ^ (row & 7)) << 4); }
+__device__ __forceinline__ void st_shared16(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+__device__ __forceinline__ uint4 ld_shared16(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int y, uint32_t src) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
+               ::"l"(map), "r"(src), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// all but the newest `N` stores of this thread have read their shared memory
+template <int N> __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void tma_store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&h2);
+}
+__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+
+// Phi(z) (the normal distribution function) and exp(-z^2 / 2) of two numbers at once: upper tail Q(a) = R(a) exp(-a^2 / 2)
+// at a = |z|, R a polynomial in u = a / (a + 4.5) (the form of Hastings' approximations, Abramowitz and Stegun 7.1.26, with
+// coefficients of our own: least squares on [0, 14.5], weights raised where the error is largest until it is level), 4e-9
+// off near 0.  As close to the 64-bit value as 0.5 (1 + erff(z / sqrt 2)) for positive z and closer for negative z (z Phi(z):
+// relative error below 7e-6 down to z = -9, where the erff form is off by 5e-4 at -4 and has nothing left at -6).  erff and
+// __expf, two branches and about 60 instructions an element, held a 128 x 256 tile for 8 us under a GELU derivative.  (The
+// forward pass keeps erff: its results are what the loss is made of, and they stay bit for bit.)
+__device__ __forceinline__ void normal_cdf2(float z0, float z1, f32x2& cdf, f32x2& bell) {
+  const float a0 = fminf(fabsf(z0), 32.0f), a1 = fminf(fabsf(z1), 32.0f);
+  const f32x2 a = pack2(a0, a1);
+  float d0, d1, r0, r1;
+  unpack2(add2(a, pack2(4.5f, 4.5f)), d0, d1);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(d0));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(d1));
+  const f32x2 u = mul2(a, pack2(r0, r1));
+  // -R(u)
+  f32x2 q = pack2(0.10403244942426682f, 0.10403244942426682f);
+  q = fma2_of(q, u, pack2(-0.3818792402744293f, -0.3818792402744293f));
+  q = fma2_of(q, u, pack2(0.33312368392944336f, 0.33312368392944336f));
+  q = fma2_of(q, u, pack2(0.7928810119628906f, 0.7928810119628906f));
+  q = fma2_of(q, u, pack2(-2.6637678146362305f, -2.6637678146362305f));
+  q = fma2_of(q, u, pack2(3.7877349853515625f, 3.7877349853515625f));
+  q = fma2_of(q, u, pack2(-3.2672412395477295f, -3.2672412395477295f));
+  q = fma2_of(q, u, pack2(1.7952399253845215f, 1.7952399253845215f));
+  q = fma2_of(q, u, pack2(-0.5f, -0.5f));
+  float x0, x1, e0, e1, q0, q1;
+  unpack2(mul2(mul2(a, pack2(-0.72134752f, -0.72134752f)), a), x0, x1);       // -a^2 / (2 ln 2)
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(x0));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(x1));
+  bell = pack2(e0, e1);
+  unpack2(mul2(q, bell), q0, q1);
+  // z >= 0: 1 - Q, else Q
+  q0 = __uint_as_float(__float_as_uint(q0) ^ (__float_as_uint(z0) & 0x80000000u));
+  q1 = __uint_as_float(__float_as_uint(q1) ^ (__float_as_uint(z1) & 0x80000000u));
+  cdf = add2(pack2(q0, q1), pack2(__float_as_uint(z0) >> 31 ? 0.0f : 1.0f, __float_as_uint(z1) >> 31 ? 0.0f : 1.0f));
+}
+// GELU'(z) = Phi(z) + z exp(-z^2 / 2) / sqrt(2 pi)
+__device__ __forceinline__ void gelu_grad2(float z0, float z1, float& g0, float& g1) {
+  f32x2 cdf, bell;
+  normal_cdf2(z0, z1, cdf, bell);
+  unpack2(fma2_of(pack2(z0, z1), mul2(bell, pack2(0.39894228f, 0.39894228f)), cdf), g0, g1);
+}
+
 // Where a row's activations go in the next layer's store: the part of its index (in place before the launch) that
-// belongs to one row and one tile of 128 columns.  It needs no accumulator, so it is fetched while the MMAs run.
+// belongs to one row and one tile of 128 columns.
 struct StoreRow {
   uint4 bits;                // the row's four keep-bit words of the tile
-  uint32_t first, off;       // tile offset, row offset
-  __device__ __forceinline__ void load(const TcParams& p, int64_t m, int64_t n) {
-    const int64_t tile = (m >> 6) * p.st_ncb + (n >> 7);
-    const uint32_t* tw = p.st_keepbits + tile * kTileWords;
-    bits = *reinterpret_cast<const uint4*>(tw + (int)(m & 63) * 4);
-    first = p.st_offsets[tile];
-    off = reinterpret_cast<const unsigned short*>(tw + kBitWords)[(int)(m & 63)];
+  uint32_t pos;              // where its first kept entry of the tile goes
+  uint32_t seg, end;         // warp: kept entries of its 32 rows go to seg .. end
+  bool staged;               // warp: they are collected in shared memory and copied out in 16-byte pieces
+  __device__ __forceinline__ void load(const TcParams& p, int64_t m, int64_t n, bool row_ok, bool whole_tile) {
+    bits = make_uint4(0u, 0u, 0u, 0u);
+    pos = end = 0u;
+    if (row_ok) {
+      const int64_t tile = (m >> 6) * p.st_ncb + (n >> 7);
+      const uint32_t* tw = p.st_keepbits + tile * kTileWords;
+      bits = *reinterpret_cast<const uint4*>(tw + (int)(m & 63) * 4);
+      pos = p.st_offsets[tile] + reinterpret_cast<const unsigned short*>(tw + kBitWords)[(int)(m & 63)];
+      end = pos + __popc(bits.x) + __popc(bits.y) + __popc(bits.z) + __popc(bits.w);
+    }
+    // the 32 rows of a warp lie in one tile, one after the other, so their kept entries are neighbours
+    seg = __shfl_sync(0xffffffffu, pos, 0);
+    end = __reduce_max_sync(0xffffffffu, end);
+    staged = whole_tile && ((uintptr_t)p.st_values & 15) == 0 && end > seg && end - (seg & ~7u) <= kFillValues;
   }
 };
 
-// ---- epilogue of one 32-column chunk of one accumulator row ------------------------------------------
-// r: the 32 float32 accumulators of row m, columns n .. n+31 (as bit patterns).
-template <int EPI>
-__device__ __forceinline__ void epilogue_chunk(const TcParams& p, uint32_t (&r)[32], int64_t m, int64_t n, bool row_ok,
-                                               const StoreRow& sr) {
-  const int nvalid = (int)min((int64_t)32, p.N - n);      // multiple of 8
-  if (EPI == kFwd) {
-    float v[32];
+// This row's 32 activations (ab: rounded, two to a word) are keep-bit word `wq` of the next layer's store (Sec. 4.2: the
+// layer input is what is sampled), whose index part (drawn from the key alone) is in place: the kept ones go, scaled and
+// rounded, to consecutive places: into the warp's piece of shared memory at `fill`, or, where that is not used, straight to
+// the store.  `buf`: the chunk buffer that holds the activations.
+__device__ __forceinline__ void place_kept(const TcParams& p, const uint32_t (&ab)[16], const StoreRow& sr, int wq, uint32_t fill,
+                                           uint32_t buf, int lane) {
+  uint32_t word = wq == 0 ? sr.bits.x : wq == 1 ? sr.bits.y : wq == 2 ? sr.bits.z : sr.bits.w;
+  uint32_t pos = sr.pos;
+  if (wq > 0) pos += __popc(sr.bits.x);
+  if (wq > 1) pos += __popc(sr.bits.y);
+  if (wq > 2) pos += __popc(sr.bits.z);
+  if (sr.staged) {
+    // predicated stores, no branches: few lanes keep the same column
+    uint32_t at = fill + 2u * (pos - (sr.seg & ~7u));
 #pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-    if (p.bias != nullptr) {
+    for (int j = 0; j < 32; j += 2) {
+      const uint32_t a = ab[j >> 1], v = pack_bf16(__fmul_rn(bf16_lo(a), p.st_scale), __fmul_rn(bf16_hi(a), p.st_scale));
 #pragma unroll
-      for (int j = 0; j < 32; j += 4) {
-        if (j < nvalid) {
-          const float4 b4 = *reinterpret_cast<const float4*>(p.bias + n + j);
-          v[j] += b4.x; v[j + 1] += b4.y; v[j + 2] += b4.z; v[j + 3] += b4.w;
-        }
-      }
-    }
-    if (row_ok) {
-      if (p.out_z != nullptr) {
-        float4* dst = reinterpret_cast<float4*>(p.out_z + m * p.ld_z + n);
-#pragma unroll
-        for (int j = 0; j < 32; j += 4)
-          if (j < nvalid) dst[j >> 2] = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-      }
-      if (p.out_zlow != nullptr) {
-        uint4* dst = reinterpret_cast<uint4*>(p.out_zlow + m * p.ld_zlow + n);
-#pragma unroll
-        for (int j = 0; j < 32; j += 8) {
-          if (j < nvalid) {
-            __nv_bfloat162 a = __floats2bfloat162_rn(v[j], v[j + 1]), b = __floats2bfloat162_rn(v[j + 2], v[j + 3]);
-            __nv_bfloat162 c = __floats2bfloat162_rn(v[j + 4], v[j + 5]), d = __floats2bfloat162_rn(v[j + 6], v[j + 7]);
-            dst[j >> 3] = make_uint4(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b),
-                                     *reinterpret_cast<uint32_t*>(&c), *reinterpret_cast<uint32_t*>(&d));
-          }
-        }
-      }
-      if (p.out_act != nullptr) {
-        uint32_t bits = 0;
-        uint32_t ab[16];                          // the rounded activations, two to a word
-        uint4* dst = reinterpret_cast<uint4*>(p.out_act + m * p.ld_act + n);
-#pragma unroll
-        for (int j = 0; j < 32; j += 8) {
-#pragma unroll
-          for (int e = 0; e < 8; e += 2) ab[(j + e) >> 1] = 0u;
-          if (j < nvalid) {
-#pragma unroll
-            for (int e = 0; e < 8; e += 2) {
-              float a0 = v[j + e], a1 = v[j + e + 1];
-              if (p.act == RAD_ACT_RELU) { a0 = fmaxf(a0, 0.0f); a1 = fmaxf(a1, 0.0f); }
-              else if (p.act == RAD_ACT_GELU) { a0 = gelu_f(a0); a1 = gelu_f(a1); }
-              const __nv_bfloat162 h2 = __floats2bfloat162_rn(a0, a1);
-              ab[(j + e) >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
-              // the bit is taken from the rounded activation, the tensor the backward sees
-              bits |= (__bfloat162float(h2.x) > 0.0f ? 1u : 0u) << (j + e);
-              bits |= (__bfloat162float(h2.y) > 0.0f ? 1u : 0u) << (j + e + 1);
-            }
-            dst[j >> 3] = make_uint4(ab[j >> 1], ab[(j >> 1) + 1], ab[(j >> 1) + 2], ab[(j >> 1) + 3]);
-          }
-        }
-        if (p.relubits != nullptr) p.relubits[m * p.w32 + (n >> 5)] = bits;
-        if (p.st_values != nullptr) {
-          // This row's 32 activations are one keep-bit word of the next layer's store (Sec. 4.2: the
-          // layer input is what is sampled), whose index part (drawn from the key alone) is in place:
-          // tile offset + row offset + kept entries of the row's earlier words say where they go.
-          const int64_t tile = (m >> 6) * p.st_ncb + (n >> 7);
-          const int rr = (int)(m & 63), wq = (int)((n >> 5) & 3);
-          const uint32_t* tw = p.st_keepbits + tile * kTileWords;
-          const uint4 rowbits = sr.bits;
-          const uint32_t word = wq == 0 ? rowbits.x : wq == 1 ? rowbits.y : wq == 2 ? rowbits.z : rowbits.w;
-          const uint32_t first = sr.first;
-          uint64_t pos = (uint64_t)first + sr.off;
-          if (wq > 0) pos += __popc(rowbits.x);
-          if (wq > 1) pos += __popc(rowbits.y);
-          if (wq > 2) pos += __popc(rowbits.z);
-          const uint64_t cap = (uint64_t)p.st_capacity;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if ((word >> j) & 1u) {
-              const float a = __uint_as_float((j & 1) ? (ab[j >> 1] & 0xffff0000u) : (ab[j >> 1] << 16));
-              if (pos < cap) p.st_values[pos] = __float2bfloat16_rn(__fmul_rn(a, p.st_scale));
-              ++pos;
-            }
-          }
-          if (rr == 0 && wq == 0) {
-            // zeros between the tile's last value and its padded end
-            const uint4 last = *reinterpret_cast<const uint4*>(tw + 63 * 4);
-            const uint32_t exact = reinterpret_cast<const unsigned short*>(tw + kBitWords)[63] + __popc(last.x) + __popc(last.y) +
-                                   __popc(last.z) + __popc(last.w);
-            const uint64_t end = min((uint64_t)p.st_offsets[tile + 1], cap);
-            for (uint64_t q = (uint64_t)first + exact; q < end; ++q) p.st_values[q] = __float2bfloat16_rn(0.0f);
-          }
-        }
-      }
+      for (int e = 0; e < 2; ++e)
+        asm volatile("{\n\t.reg .pred k;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.ne.u32 k, t, 0;\n\t@k st.shared.b16 [%0], %1;\n\t"
+                     "@k add.u32 %0, %0, 2;\n\t}"
+                     : "+r"(at) : "h"((unsigned short)(e ? v >> 16 : v & 0xffffu)), "r"(word), "r"(1u << (j + e)) : "memory");
     }
   } else {
-    if (row_ok) {
-      uint32_t bits = 0xffffffffu;
-      if (p.relubits_prev != nullptr) bits = p.relubits_prev[m * ((p.N + 31) / 32) + (n >> 5)];
-      uint4 z_prev[4];                            // read before the first store, so that the loads are in flight together
-      if (p.z_prev != nullptr) {
+    const uint32_t row = buf + lane * 64;              // 16-byte unit u of the row lies at u ^ ((lane >> 1) & 3)
+    const uint32_t swz = (uint32_t)((lane >> 1) & 3) << 4;
+#pragma unroll 1
+    while (word != 0) {
+      const uint32_t c = (uint32_t)__ffs((int)word) - 1u;
+      word &= word - 1u;
+      unsigned short h;
+      asm volatile("ld.shared.b16 %0, [%1];" : "=h"(h) : "r"(row + ((c << 1) ^ swz)) : "memory");
+      const float v = __fmul_rn(__uint_as_float((uint32_t)h << 16), p.st_scale);
+      if ((int64_t)pos < p.st_capacity) p.st_values[pos] = __float2bfloat16_rn(v);
+      ++pos;
+    }
+  }
+}
+// The warp's staged entries to their places, 16 bytes at a time where all eight are its own.
+__device__ __forceinline__ void copy_kept(const TcParams& p, const StoreRow& sr, uint32_t fill, int lane) {
+  const uint32_t base = sr.seg & ~7u, end = (uint32_t)min((int64_t)sr.end, p.st_capacity);
+  for (uint32_t q = base + 8u * lane; q < end; q += 256u) {
+    const uint4 v = ld_shared16(fill + 2u * (q - base));
+    if (q >= sr.seg && q + 8u <= end) {
+      *reinterpret_cast<uint4*>(p.st_values + q) = v;
+    } else {
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int j = 0; j < 32; j += 8)
-          if (j < nvalid) z_prev[j >> 3] = *reinterpret_cast<const uint4*>(p.z_prev + m * p.ld_zprev + n + j);
-      }
-      uint4* dst = reinterpret_cast<uint4*>(p.out_dx + m * p.ld_dx + n);
+      for (int e = 0; e < 8; ++e)
+        if (q + e >= sr.seg && q + e < end)
+          reinterpret_cast<unsigned short*>(p.st_values)[q + e] = (unsigned short)((e & 1) ? w[e >> 1] >> 16 : w[e >> 1] & 0xffffu);
+    }
+  }
+}
+// zeros between the last value of the tile that starts with this row and its padded end
+__device__ __forceinline__ void pad_store_tile(const TcParams& p, int64_t m, int64_t n) {
+  const int64_t tile = (m >> 6) * p.st_ncb + (n >> 7);
+  const uint32_t* tw = p.st_keepbits + tile * kTileWords;
+  const uint4 last = *reinterpret_cast<const uint4*>(tw + 63 * 4);
+  const uint32_t exact = reinterpret_cast<const unsigned short*>(tw + kBitWords)[63] + __popc(last.x) + __popc(last.y) +
+                         __popc(last.z) + __popc(last.w);
+  const uint32_t end = (uint32_t)min((int64_t)p.st_offsets[tile + 1], p.st_capacity);
+  for (uint32_t q = p.st_offsets[tile] + exact; q < end; ++q) p.st_values[q] = __float2bfloat16_rn(0.0f);
+}
+
+// One chunk of the forward pass: r holds the 32 float32 accumulators of row m, columns n .. n + 31 (as bit patterns);
+// y0 is the warp's first row.  `turn` counts the warp's chunks.  Returns the chunk's ReLU bits.  The activation is a template
+// parameter: what is not used is not there to be jumped over, which cost 4 us a tile of 128 x 256 (instruction fetch).
+template <int ACT>
+__device__ __forceinline__ uint32_t forward_chunk(const TcParams& p, const CUtensorMap* tm_act, const CUtensorMap* tm_zlow,
+                                                  const CUtensorMap* tm_z, const uint32_t (&r)[32], int y0, int n, int lane,
+                                                  uint32_t stage, uint32_t bias, int turn, uint32_t (&ab)[16]) {
+  const int nvalid = min(32, (int)p.N - n);      // multiple of 8
+  float v[32];
+  if (p.bias != nullptr) {
 #pragma unroll
-      for (int j = 0; j < 32; j += 8) {
-        if (j < nvalid) {
-          float g[8];
+    for (int j = 0; j < 32; j += 4) {
+      const uint4 b4 = ld_shared16(bias + 4 * j);
+      v[j] = __uint_as_float(r[j]) + __uint_as_float(b4.x); v[j + 1] = __uint_as_float(r[j + 1]) + __uint_as_float(b4.y);
+      v[j + 2] = __uint_as_float(r[j + 2]) + __uint_as_float(b4.z); v[j + 3] = __uint_as_float(r[j + 3]) + __uint_as_float(b4.w);
+    }
+  } else {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) g[e] = ((bits >> (j + e)) & 1u) ? __uint_as_float(r[j + e]) : 0.0f;
-          if (p.z_prev != nullptr) {
-            const uint4 zq = z_prev[j >> 3];
-            const uint32_t zw[4] = {zq.x, zq.y, zq.z, zq.w};
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+  }
+  const bool z_only = p.out_act == nullptr && p.out_zlow == nullptr;
+  if (p.out_z != nullptr) {
+    // two buffers of 4 KB; where 16-bit results follow they share the ring
+    const uint32_t buf = z_only ? stage + (turn & 1) * 2 * kChunkBytes : stage;
+    if (elect_one()) {
+      if (z_only) tma_store_wait_read<1>();
+      else tma_store_wait_read<0>();
+    }
+    __syncwarp();
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const float z = __uint_as_float((e & 1) ? (zw[e >> 1] & 0xffff0000u) : (zw[e >> 1] << 16));
-              g[e] *= gelu_grad_f(z);
-            }
-          }
-          uint32_t pk[4];
+    for (int j = 0; j < 32; j += 4)
+      st_shared16(chunk32_addr(buf, lane, j >> 2), __float_as_uint(v[j]), __float_as_uint(v[j + 1]), __float_as_uint(v[j + 2]),
+                  __float_as_uint(v[j + 3]));
+    fence_proxy_async();
+    __syncwarp();
+    if (elect_one()) {
+      tma_store_2d(tm_z, n, y0, buf);
+      tma_store_commit();
+    }
+    if (z_only) return 0u;
+  }
+  uint32_t zl[16], bits = 0;
+  if (p.out_zlow != nullptr) {
 #pragma unroll
-          for (int e = 0; e < 8; e += 2) {
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(g[e], g[e + 1]);
-            pk[e >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
-          }
-          dst[j >> 3] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-        }
+    for (int j = 0; j < 32; j += 2) zl[j >> 1] = pack_bf16(v[j], v[j + 1]);
+  }
+  if (p.out_act != nullptr) {
+    if (ACT == RAD_ACT_GELU) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] = gelu_f(v[j]);
+    } else if (ACT == RAD_ACT_RELU) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] = fmaxf(v[j], 0.0f);
+    }
+#pragma unroll
+    for (int j = 0; j < 32; j += 2) ab[j >> 1] = pack_bf16(v[j], v[j + 1]);
+    if (p.relubits != nullptr) {
+      // The bit is taken from the rounded activation, the tensor the backward sees.  A comparison gives a mask for the two
+      // halves of a word; pair i leaves its column 2 i in bit i and 2 i + 1 in bit 16 + i, and the halves are interleaved last.
+      const __nv_bfloat162 zero = __floats2bfloat162_rn(0.0f, 0.0f);
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        bits |= __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&ab[i]), zero) & (0x00010001u << i);
+      uint32_t t = (bits ^ (bits >> 8)) & 0x0000ff00u;
+      bits ^= t ^ (t << 8);
+      t = (bits ^ (bits >> 4)) & 0x00f000f0u;
+      bits ^= t ^ (t << 4);
+      t = (bits ^ (bits >> 2)) & 0x0c0c0c0cu;
+      bits ^= t ^ (t << 2);
+      t = (bits ^ (bits >> 1)) & 0x22222222u;
+      bits ^= t ^ (t << 1);
+    }
+  }
+  // one output takes a buffer of the ring a chunk, two take a pair of them
+  const bool both = p.out_zlow != nullptr && p.out_act != nullptr;
+  if (turn >= 2 || p.out_z != nullptr) {
+    if (elect_one()) {
+      if (p.out_z != nullptr) tma_store_wait_read<0>();
+      else if (both) tma_store_wait_read<1>();
+      else tma_store_wait_read<3>();
+    }
+    __syncwarp();
+  }
+  const uint32_t first = stage + (both ? (turn & 1) * 2 : turn & 3) * kChunkBytes, second = first + kChunkBytes;
+  if (p.out_act != nullptr) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) st_shared16(chunk16_addr(first, lane, u), ab[4 * u], ab[4 * u + 1], ab[4 * u + 2], ab[4 * u + 3]);
+  }
+  if (p.out_zlow != nullptr) {
+    const uint32_t to = both ? second : first;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) st_shared16(chunk16_addr(to, lane, u), zl[4 * u], zl[4 * u + 1], zl[4 * u + 2], zl[4 * u + 3]);
+  }
+  fence_proxy_async();
+  __syncwarp();
+  if (elect_one()) {
+    if (p.out_act != nullptr) tma_store_2d(tm_act, n, y0, first);
+    if (p.out_zlow != nullptr) tma_store_2d(tm_zlow, n, y0, both ? second : first);
+    tma_store_commit();
+  }
+  // columns past the layer's width are not activations
+  return nvalid < 32 ? bits & ((1u << nvalid) - 1u) : bits;
+}
+
+// z of the GELU derivative for a warp's chunk (32 rows from y0, 32 columns from n) into shared memory, four lanes to a row.
+__device__ __forceinline__ void prefetch_z(const TcParams& p, int64_t y0, int64_t n, int lane, uint32_t buf) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int row = 8 * i + (lane >> 2), unit = lane & 3;
+    if (y0 + row < p.M && n + 8 * unit < p.N)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                   ::"r"(chunk16_addr(buf, row, unit)), "l"(p.z_prev + (y0 + row) * p.ld_zprev + n + 8 * unit) : "memory");
+  }
+}
+// One chunk of the input gradient: times the derivative of the activation before (ReLU bits, or GELU' of the z that lies in
+// `buf`), rounded, out through the same buffer.
+template <bool kGelu>
+__device__ __forceinline__ void dx_chunk(const TcParams& p, const CUtensorMap* tm_dx, const uint32_t (&r)[32], int y0, int n, int lane,
+                                         uint32_t bits, uint32_t buf) {
+  float g[32];
+#pragma unroll
+  for (int j = 0; j < 32; ++j) g[j] = ((bits >> j) & 1u) ? __uint_as_float(r[j]) : 0.0f;
+  if (kGelu) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint4 zq = ld_shared16(chunk16_addr(buf, lane, u));
+      const uint32_t zw[4] = {zq.x, zq.y, zq.z, zq.w};
+#pragma unroll
+      for (int e = 0; e < 8; e += 2) {
+        float d0, d1;
+        gelu_grad2(bf16_lo(zw[e >> 1]), bf16_hi(zw[e >> 1]), d0, d1);
+        g[8 * u + e] *= d0;
+        g[8 * u + e + 1] *= d1;
       }
     }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    st_shared16(chunk16_addr(buf, lane, u), pack_bf16(g[8 * u], g[8 * u + 1]), pack_bf16(g[8 * u + 2], g[8 * u + 3]),
+                pack_bf16(g[8 * u + 4], g[8 * u + 5]), pack_bf16(g[8 * u + 6], g[8 * u + 7]));
+  fence_proxy_async();
+  __syncwarp();
+  if (elect_one()) {
+    tma_store_2d(tm_dx, n, y0, buf);
+    tma_store_commit();
   }
 }
 
@@ -466,17 +639,11 @@ __device__ __forceinline__ void expand_word(uint8_t* sA, const uint8_t* sC, int 
 // even CTA's wait on the previous phase, so its bytes never reach an older phase), empty[s] and tmem_full[b] (one per CTA, signalled by the MMA thread's commit to
 // both CTAs), tmem_empty[b] (even CTA; every epilogue warp of the pair arrives).
 constexpr int kStage2Bytes = 2 * 128 * BK * 2;   // 16 KB of A + 16 KB of B per CTA and stage
-constexpr int kStages2 = 6;
-// Epilogue warps, eight or sixteen.  Sixteen for a forward pass of up to kWideEpilogueK inputs that places the next layer's
-// store: more warps hide its loads and scattered stores (us with eight / sixteen, GELU: 4096 x 2048 outputs 50.5 / 40.2
-// from 1024 inputs, 57.0 / 50.1 from 2048, 60.3 / 56.3 from 2560; 8192 x 4096 outputs 171 / 156 from 2048, 180 / 178 from
-// 2560, 195 / 206 from 3072: above, the MMAs of a tile outlast the epilogue of the one before).  Without a store
-// sixteen pay for the arithmetic of a GELU of few inputs (4096 x 512 x 2048 29.3 / 25.5, 16384 x 512 x 2048 78.5 / 62.9),
-// unless it also writes the pre-activations of many tiles (8192 x 1024 x 2048 57.2 / 55.0, but 16384 x 1024 x 2048 94.9 / 101.6
-// and 16384 x 512 x 4096 186 / 196), and cost elsewhere (16384 x 1024 x 4096: ReLU 129 / 148, float32 outputs 156 / 179;
-// input gradient of 4096 x 1024 x 1024 14.2 / 15.4).
-constexpr int64_t kWideEpilogueK = 2048, kWideGeluK = 1024, kWideGeluWaves = 4;
-constexpr int threads2(int epi_warps) { return 32 * (2 + epi_warps); }
+constexpr int kStages2 = 4;
+constexpr int kThreads2 = 32 * (2 + kEpiWarps);
+// A quarter of an SM holds three of the ten warps, and one of a small kernel of another stream has to fit beside them: at most
+// 144 registers a thread (with 168 such a kernel waited for the end of the launch; tests/test_gpu_streams.py).
+constexpr int kRegisterBound2 = 144;
 
 struct SmemCtl2 {
   uint64_t full[kStages2], empty[kStages2], tmem_full[2], tmem_empty[2];
@@ -542,29 +709,36 @@ __host__ __device__ constexpr uint32_t make_idesc_pair(bool a_mn, bool b_mn, uin
          ((n >> 3) << 17) | ((256u >> 4) << 24);
 }
 
-template <int AK, int BKIND, int EPI, int kEpiWarps2>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(kEpiWarps2), 1)
-tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB) {
+// The tensor maps of the outputs: tmO activation or input gradient, tmL pre-activation in bf16, tmZ float32 results.
+// ACT: activation of the forward pass; of the input gradient, RAD_ACT_GELU where it multiplies by GELU'(z_prev).  kFill: the
+// forward pass fills the next layer's store.
+template <int AK, int BKIND, int EPI, int ACT, bool kFill>
+__global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kRegisterBound2)
+tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                    const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmL,
+                    const __grid_constant__ CUtensorMap tmZ) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  SmemCtl2* ctl = reinterpret_cast<SmemCtl2*>(smem + (size_t)kStages2 * kStage2Bytes);
+  uint8_t* epi_smem = smem + (size_t)kStages2 * kStage2Bytes;
+  SmemCtl2* ctl = reinterpret_cast<SmemCtl2*>(epi_smem + kEpiWarps * kEpiBytes);
   volatile int* abort_flag = &ctl->abort_flag;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = cluster_ctarank();         // 0: issues the MMAs; both stage operands and run epilogues
   const uint32_t peer_abort = map_to_cta(smem_u32(&ctl->abort_flag), rank ^ 1u);
   const PairWait wc = {abort_flag, peer_abort, p.wait_limit_ns};
-  const int64_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const uint32_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   if (tid == 0) {
     prefetch_map(&tmA);
     prefetch_map(&tmB);
+    if (EPI != kDwT) prefetch_map(p.out_z != nullptr ? &tmZ : &tmO);
     for (int s = 0; s < kStages2; ++s) {
       mbar_init(smem_u32(&ctl->full[s]), 1);
       mbar_init(smem_u32(&ctl->empty[s]), 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&ctl->tmem_full[b]), 1);
-      mbar_init(smem_u32(&ctl->tmem_empty[b]), 2 * kEpiWarps2);
+      mbar_init(smem_u32(&ctl->tmem_empty[b]), 2 * kEpiWarps);
     }
     ctl->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -579,8 +753,9 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
   const uint32_t smem_base = smem_u32(smem);
-  // so far nothing of another kernel was touched: the above runs under the tail of the kernel before
-  wait_for_previous();
+  // so far nothing of another kernel was touched: the above runs under the tail of the kernel before, and so does the
+  // division of the work, which depends on the parameters only (not for kDwT)
+  if (EPI == kDwT) wait_for_previous();
   // Same-sample dW (kDwT): the tile is dW^T, M = H, N = kept columns (known on the device only).  The kept
   // columns are cut into the fewest tiles of at most 256 and the tile width bn is what one of them needs,
   // rounded up to the MMA's granule of 16: 105 kept columns cost one tile of 112, not one of 256.
@@ -594,6 +769,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
     bn = max(16, (int)(((n_cols + nt - 1) / nt + 15) / 16 * 16));
   }
   const Schedule sched(p.M, n_cols, p.K, p.splits, BM, bn);
+  if (EPI != kDwT) wait_for_previous();
   const int boxes_b = (bn / 2 + 63) / 64;             // 64-column boxes of an MN-major B this CTA stages per K block
   const uint32_t stage_tx = 2u * (uint32_t)(kStage2Bytes / 2 + (BKIND == kBK_ ? bn / 2 * 128 : boxes_b * 8192));
 
@@ -604,7 +780,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int64_t u = pair; u < sched.units && ok; u += npairs) {
+      for (uint32_t u = pair; u < sched.units && ok; u += npairs) {
         const Unit w = sched.unit(u);
         if (u + npairs >= sched.units) let_next_start();
         const int m_own = (int)w.m0 + 128 * (int)rank, n_own = (int)w.n0 + (bn / 2) * (int)rank;
@@ -651,7 +827,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       int stage = 0, buf = 0;
       uint32_t phase = 0, buf_phases = 0;          // bit b: phase of accumulator b
       bool ok = true;
-      for (int64_t u = pair; u < sched.units && ok; u += npairs) {
+      for (uint32_t u = pair; u < sched.units && ok; u += npairs) {
         const Unit w = sched.unit(u);
         ok = mbar_wait2(smem_u32(&ctl->tmem_empty[0]) + 8u * buf, ((buf_phases >> buf) & 1u) ^ 1u, wc);
         if (!ok) break;
@@ -678,59 +854,120 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
     // ===== epilogue: thread = one accumulator row of this CTA =====
     const int q = warp & 3;
     // the warps of a lane quarter split the tile's 32-column chunks between them
-    constexpr int kPerQuarter = kEpiWarps2 / 4;
+    constexpr int kPerQuarter = kEpiWarps / 4;
     const int chunks = (bn + 31) / 32, own_chunks = (chunks + kPerQuarter - 1) / kPerQuarter;
     const int c_first = ((warp - 2) >> 2) * own_chunks * 32;
     const int c_last = min(c_first + own_chunks * 32, chunks * 32);
     const uint32_t empty_bar = map_to_cta(smem_u32(&ctl->tmem_empty[0]), 0u);     // [b] is 8 bytes further
-    int buf = 0;
+    const uint32_t stage = smem_u32(epi_smem) + (warp - 2) * kEpiBytes, fill = stage + 4 * kChunkBytes, bias_row = fill + kFillBytes;
+    int buf = 0, turn = 0;
     uint32_t buf_phases = 0;
     bool ok = true;
     if (EPI == kDwT && p.keep_cols != nullptr) {
       // Rows of dW whose column was not kept are zero (Sec. 4.3: only the sampled part of the weight matrix
       // gets a gradient).  The epilogue warps have nothing to do until the first tile's MMAs retire, so they
       // write those rows now: row d belongs to CTA d mod grid, a thread writes 16 bytes at a time.
-      const int et = tid - 64;                       // 0 .. 32 kEpiWarps2 - 1
+      const int et = tid - 64;                       // 0 .. 32 kEpiWarps - 1
       const int64_t h4 = p.M / 4;
       for (int64_t d = blockIdx.x; d < p.dw_rows; d += gridDim.x) {
         if ((p.keep_cols[d >> 5] >> (d & 31)) & 1u) continue;
         float4* rowp = reinterpret_cast<float4*>(p.out_dw + d * p.ld_dw);
-        for (int64_t i = et; i < h4; i += 32 * kEpiWarps2) rowp[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int64_t i = et; i < h4; i += 32 * kEpiWarps) rowp[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
-    for (int64_t u = pair; u < sched.units && ok; u += npairs) {
+    for (uint32_t u = pair; u < sched.units && ok; u += npairs) {
       const Unit w = sched.unit(u);
-      const int64_t m = w.m0 + 128 * (int64_t)rank + q * 32 + lane;
+      const int64_t m_warp = w.m0 + 128 * (int64_t)rank + q * 32, m = m_warp + lane;
       const bool row_ok = m < sched.M;
-      // what the epilogue reads besides the accumulators comes while the MMAs run (a warp's columns lie in one store tile).
-      // The bias only with sixteen warps: with eight its prefetch costs more than it hides (16384 x 512 x 4096 with GELU 186
-      // us, 165 without)
+      const int64_t n_warp = w.n0 + c_first;
+      // what the epilogue reads besides the accumulators comes while the MMAs run (a warp's columns lie in one store tile)
       StoreRow sr = {};
-      if (EPI == kFwd && w.n0 + c_first < n_cols) {
-        if (p.st_values != nullptr && row_ok) sr.load(p, m, w.n0 + c_first);
-        if (kEpiWarps2 > 8 && p.bias != nullptr && lane < own_chunks && w.n0 + c_first + 32 * lane < n_cols)
-          asm volatile("prefetch.global.L1 [%0];" ::"l"(p.bias + w.n0 + c_first + 32 * lane));
+      uint32_t prev_bits[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu}, act_bits[4] = {};
+      if (EPI == kFwd && kFill && n_warp < n_cols) {
+        sr.load(p, m, n_warp, row_ok, own_chunks == 4);
+        if (row_ok && (m & 63) == 0 && (n_warp & 127) == 0) pad_store_tile(p, m, n_warp);
       }
-      if (lane == 0) ok = mbar_wait2(smem_u32(&ctl->tmem_full[0]) + 8u * buf, (buf_phases >> buf) & 1u, wc, 200u);
+      if (EPI == kFwd && p.bias != nullptr) {
+        // four columns a lane; zero past the layer's width
+        float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (4 * lane < 32 * own_chunks && n_warp + 4 * lane < n_cols) b4 = *reinterpret_cast<const float4*>(p.bias + n_warp + 4 * lane);
+        st_shared16(bias_row + 16 * lane, __float_as_uint(b4.x), __float_as_uint(b4.y), __float_as_uint(b4.z), __float_as_uint(b4.w));
+        __syncwarp();
+      }
+      if (EPI == kDx && n_warp < n_cols) {
+        if (p.relubits_prev != nullptr) {
+          const uint32_t* words = p.relubits_prev + m * ((p.N + 31) / 32) + (n_warp >> 5);
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (row_ok && c < own_chunks && n_warp + 32 * c < n_cols) prev_bits[c] = words[c];
+        }
+        if (elect_one()) tma_store_wait_read<0>();      // the unit before has left the buffers
+        __syncwarp();
+        if (ACT == RAD_ACT_GELU) {
+          for (int c = 0; c < own_chunks; ++c) prefetch_z(p, m_warp, n_warp + 32 * c, lane, stage + c * kChunkBytes);
+          asm volatile("cp.async.commit_group;" ::: "memory");
+        }
+      }
+      if (lane == 0) ok = mbar_wait2(smem_u32(&ctl->tmem_full[0]) + 8u * buf, (buf_phases >> buf) & 1u, wc, 64u);
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       if (!ok) break;
+      if (EPI == kDx && ACT == RAD_ACT_GELU) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+      }
       tc_fence_after();
 #pragma unroll 1
       for (int c0 = c_first; c0 < c_last; c0 += 32) {
         const int64_t n = w.n0 + c0;
-        if (n >= n_cols) break;               // warp-uniform
+        if (n >= n_cols || (EPI != kDwT && m_warp >= sched.M)) break;               // warp-uniform
+        const int c = (c0 - c_first) >> 5;
         uint32_t r[32];
         tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256 + c0), r);
         tmem_ld_wait();
-        // a chunk may reach past the tile's width (bn is a multiple of 16) and past the last kept column
-        if (EPI == kDwT) epilogue_chunk_dwt(p, r, m, n, (int)min((int64_t)min(32, bn - c0), n_cols - n), row_ok, w.split);
-        else epilogue_chunk<(EPI == kDwT ? kDx : EPI)>(p, r, m, n, row_ok, sr);
+        if (EPI == kDwT) {
+          // a chunk may reach past the tile's width (bn is a multiple of 16) and past the last kept column
+          epilogue_chunk_dwt(p, r, m, n, (int)min((int64_t)min(32, bn - c0), n_cols - n), row_ok, w.split);
+        } else if (EPI == kDx) {
+          const uint32_t bits = c == 0 ? prev_bits[0] : c == 1 ? prev_bits[1] : c == 2 ? prev_bits[2] : prev_bits[3];
+          dx_chunk<ACT == RAD_ACT_GELU>(p, &tmO, r, (int)m_warp, (int)n, lane, bits, stage + c * kChunkBytes);
+        } else {
+          uint32_t ab[16];
+          const uint32_t bits = forward_chunk<ACT>(p, &tmO, &tmL, &tmZ, r, (int)m_warp, (int)n, lane, stage, bias_row + 128 * c, turn++, ab);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (i == c) act_bits[i] = bits;
+          if (kFill) {
+            const int at = turn - 1;                   // the chunk's buffer of activations, as forward_chunk took it
+            place_kept(p, ab, sr, (int)(n >> 5) & 3, fill, stage + (p.out_zlow != nullptr ? (at & 1) * 2 : at & 3) * kChunkBytes, lane);
+          }
+        }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_remote(empty_bar + 8u * buf);
+      if (EPI == kFwd) {
+        if (kFill && sr.staged) {
+          __syncwarp();
+          copy_kept(p, sr, fill, lane);
+          __syncwarp();
+        }
+        if (p.relubits != nullptr && row_ok && n_warp < n_cols) {
+          uint32_t* words = p.relubits + m * p.w32 + (n_warp >> 5);
+          if (own_chunks == 4 && p.w32 % 4 == 0 && n_warp + 96 < n_cols && ((uintptr_t)words & 15) == 0) {
+            *reinterpret_cast<uint4*>(words) = make_uint4(act_bits[0], act_bits[1], act_bits[2], act_bits[3]);
+          } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              if (c < own_chunks && n_warp + 32 * c < n_cols) words[c] = act_bits[c];
+          }
+        }
+      }
       buf_phases ^= 1u << buf;
       buf ^= 1;
+    }
+    if (EPI != kDwT) {
+      if (elect_one()) tma_store_wait();               // the results are out, and the buffers no longer read
+      __syncwarp();
     }
   }
 
@@ -785,7 +1022,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
   const uint32_t peer_abort = map_to_cta(smem_u32(&ctl->abort_flag), rank ^ 1u);
   const PairWait wc = {abort_flag, peer_abort, p.wait_limit_ns};
   const Schedule sched(p.M, p.N, p.K, p.splits, kSpBM, kSpBN);
-  const int64_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const uint32_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   if (tid == 0) {
     prefetch_map(&tmB);
     for (int s = 0; s < stages; ++s) {
@@ -843,7 +1080,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int64_t u = pair; u < sched.units && ok; u += npairs) {
+      for (uint32_t u = pair; u < sched.units && ok; u += npairs) {
         const Unit w = sched.unit(u);
         if (u + npairs >= sched.units) let_next_start();
         const int n_own = (int)w.n0 + 128 * (int)rank;       // + 256 for the second half
@@ -873,7 +1110,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
       int stage = 0;
       uint32_t phase = 0, unit_phase = 0;
       bool ok = true;
-      for (int64_t u = pair; u < sched.units && ok; u += npairs) {
+      for (uint32_t u = pair; u < sched.units && ok; u += npairs) {
         const Unit w = sched.unit(u);
         ok = mbar_wait2(smem_u32(&ctl->tmem_empty), unit_phase ^ 1u, wc);
         if (!ok) break;
@@ -902,7 +1139,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
     // ===== epilogue: a warp = 32 accumulator rows, every kSpEpiShare-th 32-column chunk (the expanders take the others) =====
     uint32_t unit_phase = 0;
     bool ok = true;
-    for (int64_t u = pair; u < sched.units && ok; u += npairs) {
+    for (uint32_t u = pair; u < sched.units && ok; u += npairs) {
       ok = unit_epilogue(sched.unit(u), 0, unit_phase);
       unit_phase ^= 1u;
     }
@@ -913,7 +1150,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
     int slot = 0;
     uint32_t cphase = 0;
     bool ok = true;
-    for (int64_t u = pair; u < sched.units && ok; u += npairs) {
+    for (uint32_t u = pair; u < sched.units && ok; u += npairs) {
       const Unit w = sched.unit(u);
       const int64_t tile_col = tile_col_of(w);
       const bool have = tile_col < p.ncb;
@@ -969,7 +1206,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
     int stage = 0, slot = 0;
     uint32_t phase = 0, cphase = 0, turn = 0, unit_phase = 0;
     bool ok = true;
-    for (int64_t u = pair; u < sched.units && ok; u += npairs) {
+    for (uint32_t u = pair; u < sched.units && ok; u += npairs) {
       const Unit w = sched.unit(u);
       const bool have = tile_col_of(w) < p.ncb;
       for (int kb = w.kb0; kb < w.kb1; ++kb, turn ^= 1u) {
@@ -1088,6 +1325,20 @@ int make_map(CUtensorMap* map, const void* ptr, int64_t inner, int64_t outer, in
   return r == CUDA_SUCCESS ? RAD_OK : RAD_ECUDA;
 }
 
+// Output matrix of `cols` x `rows` elements (bf16 or float32), stored in chunks of 32 x 32.
+int make_out_map(CUtensorMap* map, bool f32, void* ptr, int64_t cols, int64_t rows, int64_t ld) {
+  EncodeTiledFn fn = encode_fn();
+  if (fn == nullptr) return RAD_ECUDA;
+  const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)ld * (f32 ? 4 : 2)};
+  const cuuint32_t box[2] = {32, 32};
+  const cuuint32_t estr[2] = {1, 1};
+  const CUresult r = fn(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, f32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                        CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? RAD_OK : RAD_ECUDA;
+}
+
 int num_sms() {
   static int n = 0;
   if (n == 0) {
@@ -1195,35 +1446,23 @@ DwPlan plan_dw(const rad_store* st, int64_t H) {
   }
 }
 
-template <int AK, int BKIND, int EPI, int kEpiWarps2 = 8>
-int launch_pair(const TcParams& p, const CUtensorMap& ta, const CUtensorMap& tb, int64_t max_units, cudaStream_t s) {
-  constexpr size_t smem = (size_t)kStages2 * kStage2Bytes + sizeof(SmemCtl2) + 1024;
+struct OutMaps { CUtensorMap o, l, z; };      // see tc_gemm_pair_kernel; those of absent outputs are not read
+
+template <int AK, int BKIND, int EPI, int ACT = RAD_ACT_NONE, bool kFill = false>
+int launch_pair(const TcParams& p, const CUtensorMap& ta, const CUtensorMap& tb, const OutMaps& out, int64_t max_units, cudaStream_t s) {
+  constexpr size_t smem = (size_t)kStages2 * kStage2Bytes + kEpiWarps * kEpiBytes + sizeof(SmemCtl2) + 1024;
   static_assert(smem <= 227 * 1024, "stage ring too deep");
-  auto kernel = tc_gemm_pair_kernel<AK, BKIND, EPI, kEpiWarps2>;
+  auto kernel = tc_gemm_pair_kernel<AK, BKIND, EPI, ACT, kFill>;
   // The kernel is persistent: the grid must not exceed the clusters that can be resident at once
   // (SM pairs that can host a cluster; fewer than half the SM count on some parts).
   static int resident_pairs = 0;
   if (resident_pairs == 0) {
     RAD_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * (num_sms() / 2));
-    cfg.blockDim = dim3(threads2(kEpiWarps2));
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n <= 0) {
-      (void)cudaGetLastError();
-      n = num_sms() / 2;
-    }
-    resident_pairs = std::min(n, num_sms() / 2);
+    resident_pairs = resident_pairs_of(kernel, kThreads2, smem);
   }
   const int pairs = (int)std::max<int64_t>(1, std::min<int64_t>(max_units, resident_pairs));
   count_launch();
-  RAD_TRY(launch_kernel(kernel, 2 * pairs, threads2(kEpiWarps2), smem, s, p, ta, tb));
+  RAD_TRY(launch_kernel(kernel, 2 * pairs, kThreads2, smem, s, p, ta, tb, out.o, out.l, out.z));
   return RAD_OK;
 }
 
@@ -1296,10 +1535,17 @@ int tc_forward(int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t 
                                             : (float)kLaneRange / (float)keep_threshold_host(next->p);
   }
   const int64_t units = ceil_div(B, BM) * ceil_div(H, p.bn);
-  const bool wide = p.st_values != nullptr ? D <= kWideEpilogueK
-                                           : act == RAD_ACT_GELU && D <= kWideGeluK &&
-                                                 (out_zlow == nullptr || units <= kWideGeluWaves * planning_pairs());
-  return wide ? launch_pair<kAK, kBMN, kFwd, 16>(p, ta, tb, units, s) : launch_pair<kAK, kBMN, kFwd, 8>(p, ta, tb, units, s);
+  OutMaps out = {};
+  if (out_act != nullptr) RAD_TRY(make_out_map(&out.o, false, out_act, H, B, ld_act));
+  if (out_zlow != nullptr) RAD_TRY(make_out_map(&out.l, false, out_zlow, H, B, ld_zlow));
+  if (out_z != nullptr) RAD_TRY(make_out_map(&out.z, true, out_z, H, B, ld_z));
+  if (p.st_values != nullptr)
+    return act == RAD_ACT_GELU   ? launch_pair<kAK, kBMN, kFwd, RAD_ACT_GELU, true>(p, ta, tb, out, units, s)
+           : act == RAD_ACT_RELU ? launch_pair<kAK, kBMN, kFwd, RAD_ACT_RELU, true>(p, ta, tb, out, units, s)
+                                 : launch_pair<kAK, kBMN, kFwd, RAD_ACT_NONE, true>(p, ta, tb, out, units, s);
+  return act == RAD_ACT_GELU   ? launch_pair<kAK, kBMN, kFwd, RAD_ACT_GELU>(p, ta, tb, out, units, s)
+         : act == RAD_ACT_RELU ? launch_pair<kAK, kBMN, kFwd, RAD_ACT_RELU>(p, ta, tb, out, units, s)
+                               : launch_pair<kAK, kBMN, kFwd>(p, ta, tb, out, units, s);
 }
 
 int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, const void* W, int64_t ldw,
@@ -1317,7 +1563,11 @@ int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, 
   p.out_dx = static_cast<bf16*>(dZ_prev); p.ld_dx = ldp;
   p.dev_status = dev_status;
   p.wait_limit_ns = wait_limit_ns();
-  return launch_pair<kAK, kBK_, kDx>(p, ta, tb, ceil_div(B, BM) * ceil_div(D, bn), s);
+  OutMaps out = {};
+  RAD_TRY(make_out_map(&out.o, false, dZ_prev, D, B, ldp));
+  const int64_t units = ceil_div(B, BM) * ceil_div(D, bn);
+  return z_prev != nullptr ? launch_pair<kAK, kBK_, kDx, RAD_ACT_GELU>(p, ta, tb, out, units, s)
+                           : launch_pair<kAK, kBK_, kDx>(p, ta, tb, out, units, s);
 }
 
 int sm_pairs() { return planning_pairs(); }
@@ -1349,7 +1599,7 @@ int tc_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, 
     if (rc != RAD_OK) return rc;
     p.M = H; p.N = nmax; p.N_dev = st->nnz; p.row_idx = st->offsets; p.keep_cols = st->keepbits;
     const int64_t n_expect = std::max<int64_t>(1, (int64_t)std::llround((double)st->D * store_keep_fraction(st)));
-    rc = launch_pair<kAMN, kBMN, kDwT>(p, ta, tb, ceil_div(H, BM) * ceil_div(std::min(n_expect, nmax), BN) * d.splits, s);
+    rc = launch_pair<kAMN, kBMN, kDwT>(p, ta, tb, OutMaps{}, ceil_div(H, BM) * ceil_div(std::min(n_expect, nmax), BN) * d.splits, s);
   } else {
     ta = tb;                                           // unused by the sparse-A kernel
     p.M = st->D;

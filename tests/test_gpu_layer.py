@@ -342,3 +342,37 @@ def test_different_sample_dw_of_several_units_per_sm_pair(B):
     Ah = torch.where(keep, (A.float() * float(orc.scale_factor(p))).to(bf), torch.zeros((), dtype=bf, device="cuda")).double()
     ref, mag = Ah.T @ dZ.double(), Ah.abs().T @ dZ.double().abs()
     assert ((dW.double() - ref).abs() <= B * 2.0 ** -24 * mag).all()
+
+
+@pytest.mark.parametrize("B,D,H", [(64, 64, 64), (300, 72, 136), (2500, 64, 1032)])
+@pytest.mark.parametrize("p,shift", [(0.05, 0), (0.05, 1), (0.9, 0)])
+def test_outputs_in_chunks_and_the_store_beside_them(B, D, H, p, shift):
+    """Outputs with rows longer than the layer's width keep what lies past it; every combination of outputs gives the same
+    bits; the next store is the same whether a warp stages its entries (16-byte aligned values, few of them) or not."""
+    import paper_2007_10412_b200 as rad
+    bf = torch.bfloat16
+    g = torch.Generator(device="cuda").manual_seed(B + H)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    A, W, b = rnd(B, D).to(bf), rnd(D, H).to(bf), rnd(H)
+    new = lambda dt, ld: torch.full((B, ld), -7.0, dtype=dt, device="cuda")
+    act, zl, z = new(bf, H + 24), new(bf, H + 8), new(torch.float32, H + 4)
+    rad.rad_linear_forward(A, W, b, "gelu", out_act=act[:, :H], out_zlow=zl[:, :H], out_z=z[:, :H])
+    a2, z2 = new(bf, H), new(torch.float32, H)
+    rad.rad_linear_forward(A, W, b, "gelu", out_act=a2)
+    rad.rad_linear_forward(A, W, b, "none", out_z=z2)
+    st = rad.Store("different", "bf16", B, H, p, seed=3, layer=1, step=2, relu_bits=False)
+    own = rad.Store("different", "bf16", B, H, p, seed=3, layer=1, step=2, relu_bits=False)
+    room = torch.zeros(st.values.numel() + 8, dtype=bf, device="cuda")
+    st.c.values = room[shift:].data_ptr()
+    own.values.zero_()
+    a3 = new(bf, H)
+    rad.rad_linear_forward_fill(A, W, b, "gelu", a3, st)
+    rad.rad_linear_forward_store(a3, own)
+    torch.cuda.synchronize()
+    for full, width in ((act, H), (zl, H), (z, H)):
+        assert (full[:, width:] == -7.0).all()
+    assert torch.equal(act[:, :H], a2) and torch.equal(z[:, :H], z2) and torch.equal(zl[:, :H], z2.to(bf)) and torch.equal(a3, a2)
+    assert torch.equal(room[shift:shift + own.values.numel()], own.values)
+    want = A.double() @ W.double() + b.double()
+    mag = A.double().abs() @ W.double().abs() + b.double().abs()
+    assert ((z2.double() - want).abs() <= (D ** 0.5 + 16) * 2.0 ** -24 * mag).all()      # float32 sums in any order
