@@ -221,6 +221,8 @@ bool input_grad_on_tc(int32_t dtype, int64_t B, int64_t D, int64_t H, const void
          (z_prev == nullptr || (((uintptr_t)z_prev & 15) == 0 && ld_zprev % 8 == 0));
 }
 
+}  // namespace
+
 // rad_linear_weight_grad for a bitmask or column-list store (index held or drawn again); where the contraction
 // runs on the CUDA cores and passes over dZ anyway, it also leaves the bias gradient in `db` (*db_written says
 // whether it did).
@@ -228,7 +230,7 @@ bool input_grad_on_tc(int32_t dtype, int64_t B, int64_t D, int64_t H, const void
 // launch and *ig_done is set, otherwise the caller runs rad_linear_input_grad as usual.
 int weight_grad_and_bias(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, float* dW, int64_t ldw, void* workspace,
                          int64_t workspace_bytes, int32_t* dev_status, void* stream, float* db, bool* db_written,
-                         const SimtInputGrad* ig = nullptr, bool* ig_done = nullptr) {
+                         const SimtInputGrad* ig, bool* ig_done) {
   if (db_written != nullptr) *db_written = false;
   if (ig_done != nullptr) *ig_done = false;
   if (st != nullptr && st->variant == RAD_REDRAWN_SAMPLE) {
@@ -261,7 +263,6 @@ int weight_grad_and_bias(const rad_store* st, const void* dZ, int64_t ldz, int64
     return simt_weight_grad(st, dZ, ldz, H, dW, ldw, dev_status, s, db, db_written, ig, ig_done);
   return simt_weight_grad(st, dZ, ldz, H, dW, ldw, dev_status, s, db, db_written);
 }
-}  // namespace
 }  // namespace rad
 
 extern "C" int rad_weight_grad_workspace(const rad_store* st, int64_t H, int64_t* bytes) {
@@ -346,7 +347,6 @@ extern "C" int rad_linear_forward(int32_t dtype, int32_t act, int64_t B, int64_t
 }
 
 namespace rad {
-namespace {
 // Whether the forward GEMM can fill `next` from its epilogue: tensor-core shapes, a different-sample store under a
 // law whose index can be made from the key alone.
 bool fill_can_fuse(int dtype, int64_t B, int64_t D, int64_t H, const void* A, int64_t lda, const void* W, int64_t ldw,
@@ -360,14 +360,12 @@ bool fill_can_fuse(int dtype, int64_t B, int64_t D, int64_t H, const void* A, in
          (double)B * (double)H < 4294967296.0 * 0.75;
 }
 
-}  // namespace
-}  // namespace rad
-
-extern "C" int rad_linear_forward_fill(int32_t dtype, int32_t act, int64_t B, int64_t D, int64_t H, const void* A,
-                                       int64_t lda, const void* W, int64_t ldw, const float* bias, void* out_act,
-                                       int64_t ld_act, void* out_zlow, int64_t ld_zlow, uint32_t* relubits,
-                                       const rad_store* next, int32_t index_ready, void* workspace,
-                                       int64_t workspace_bytes, int32_t* dev_status, void* stream) {
+// rad_linear_forward_fill.  ahead: the index part of `next` is in place and, where the forward does not fill it from its
+// epilogue, its values wait in this queue (index_ready alone draws the store again in that case).
+int forward_fill(int32_t dtype, int32_t act, int64_t B, int64_t D, int64_t H, const void* A, int64_t lda, const void* W, int64_t ldw,
+                 const float* bias, void* out_act, int64_t ld_act, void* out_zlow, int64_t ld_zlow, uint32_t* relubits,
+                 const rad_store* next, int32_t index_ready, StoreQueue* ahead, void* workspace, int64_t workspace_bytes,
+                 int32_t* dev_status, void* stream) {
   if (!valid_dtype(dtype) || B <= 0 || D <= 0 || H <= 0 || A == nullptr || W == nullptr || out_act == nullptr)
     return RAD_EINVAL;
   if (act != RAD_ACT_NONE && act != RAD_ACT_RELU && act != RAD_ACT_GELU) return RAD_EINVAL;
@@ -382,14 +380,14 @@ extern "C" int rad_linear_forward_fill(int32_t dtype, int32_t act, int64_t B, in
     rad_store full = *next;
     full.variant = RAD_DIFFERENT_SAMPLE;
     full.keepbits = static_cast<uint32_t*>(workspace);
-    return rad_linear_forward_fill(dtype, act, B, D, H, A, lda, W, ldw, bias, out_act, ld_act, out_zlow, ld_zlow, relubits,
-                                   &full, 0, static_cast<char*>(workspace) + head, workspace_bytes - head, dev_status, stream);
+    return forward_fill(dtype, act, B, D, H, A, lda, W, ldw, bias, out_act, ld_act, out_zlow, ld_zlow, relubits, &full, 0, nullptr,
+                        static_cast<char*>(workspace) + head, workspace_bytes - head, dev_status, stream);
   }
   int rc = check_device();
   if (rc != RAD_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   bool fused = fill_can_fuse(dtype, B, D, H, A, lda, W, ldw, bias, out_act, ld_act, out_zlow, ld_zlow, next);
-  if (fused && !index_ready) {
+  if (fused && !index_ready && ahead == nullptr) {
     rc = launch_store_index(next, true, dev_status, s);
     if (rc == RAD_EUNSUPPORTED) fused = false;        // rows too long for the fixed-count index: the separate calls below
     else if (rc != RAD_OK) return rc;
@@ -406,7 +404,18 @@ extern "C" int rad_linear_forward_fill(int32_t dtype, int32_t act, int64_t B, in
   if (rc != RAD_OK) return rc;
   rad_store tmp = *next;
   tmp.relubits = bits_from_store ? relubits : nullptr;
+  if (ahead != nullptr) return ahead->add({out_act, ld_act, tmp});
   return rad_linear_forward_store(out_act, ld_act, &tmp, workspace, workspace_bytes, dev_status, stream);
+}
+}  // namespace rad
+
+extern "C" int rad_linear_forward_fill(int32_t dtype, int32_t act, int64_t B, int64_t D, int64_t H, const void* A,
+                                       int64_t lda, const void* W, int64_t ldw, const float* bias, void* out_act,
+                                       int64_t ld_act, void* out_zlow, int64_t ld_zlow, uint32_t* relubits,
+                                       const rad_store* next, int32_t index_ready, void* workspace,
+                                       int64_t workspace_bytes, int32_t* dev_status, void* stream) {
+  return forward_fill(dtype, act, B, D, H, A, lda, W, ldw, bias, out_act, ld_act, out_zlow, ld_zlow, relubits, next, index_ready,
+                      nullptr, workspace, workspace_bytes, dev_status, stream);
 }
 
 extern "C" int rad_input_grad_workspace(int64_t B, int64_t H, int64_t* bytes) {
@@ -497,12 +506,35 @@ extern "C" int rad_mlp_step(const rad_mlp_desc* net, const void* X, const int32_
     // the ReLU bits of a hidden layer's input are written by the epilogue of the layer that produces it
     s.relubits = nullptr;
   }
-  // the network input is stored by the stand-alone kernel; every hidden layer's input is stored from the
-  // epilogue of the GEMM that produces it (or by the same stand-alone call where that kernel does not apply)
   TraceRange step_range("rad_mlp_step");
+  const auto out_of = [&](int l) { return static_cast<void*>(ws + plan.act[l & 1]); };                      // activation of layer l
+  const auto z_of = [&](int l) { return plan.layer[l].preact >= 0 ? static_cast<void*>(ws + plan.layer[l].preact) : nullptr; };   // its z
+  // Index parts depend on the key alone: those of all layers that can use them are drawn in one go.  Every hidden layer's
+  // input is then stored from the epilogue of the GEMM that produces it, or by one launch that puts values in place.
+  bool ahead[64] = {};
+  if (net->variant == RAD_DIFFERENT_SAMPLE && net->law == RAD_LAW_BERNOULLI) {
+    TraceRange r("store indices");
+    rad_store list[64];
+    int n = 0;
+    for (int l = 0; l < L; ++l) {
+      const int64_t D = l > 0 ? net->dims[l - 1] : 0, H = net->dims[l];
+      ahead[l] = store_indices_ok(&st[l]) ||
+                 (l > 0 && fill_can_fuse(net->dtype, B, D, H, l > 1 ? out_of(l - 2) : X, D, W[l - 1], H, b != nullptr ? b[l - 1] : nullptr,
+                                         out_of(l - 1), H, z_of(l), H, &st[l]));
+      if (ahead[l]) list[n++] = st[l];
+    }
+    if (n > 0) {
+      rc = launch_store_indices(list, n, true, dev_status, static_cast<cudaStream_t>(stream));
+      if (rc != RAD_OK) return rc;
+    }
+  }
+  StoreQueue queue;
+  queue.dev_status = dev_status;
+  queue.s = static_cast<cudaStream_t>(stream);
   {
     TraceRange r("store input");
-    rc = rad_linear_forward_store(X, net->dims[0], &st[0], ws + plan.scratch, plan.scratch_bytes, dev_status, stream);
+    rc = ahead[0] ? queue.add({X, net->dims[0], st[0]})
+                  : rad_linear_forward_store(X, net->dims[0], &st[0], ws + plan.scratch, plan.scratch_bytes, dev_status, stream);
   }
   if (rc != RAD_OK) return rc;
   const void* a_in = X;
@@ -518,17 +550,20 @@ extern "C" int rad_mlp_step(const rad_mlp_desc* net, const void* X, const int32_
       if (rc != RAD_OK) return rc;
       break;
     }
-    void* a_out = ws + plan.act[l & 1];
-    // a GELU net keeps the pre-activation of layer l for the backward of layer l + 1's input
-    void* zlow = net->act == RAD_ACT_GELU ? ws + plan.layer[l + 1].preact : nullptr;
+    void* a_out = out_of(l);
+    void* zlow = z_of(l + 1);          // a GELU net keeps the pre-activation of layer l for the backward of layer l + 1's input
     uint32_t* rbits = plan.layer[l + 1].relubits >= 0 ? reinterpret_cast<uint32_t*>(ws + plan.layer[l + 1].relubits) : nullptr;
-    rc = rad_linear_forward_fill(net->dtype, net->act, B, D, H, a_in, ld_in, W[l], H, b != nullptr ? b[l] : nullptr,
-                                 a_out, H, zlow, H, rbits, &st[l + 1], 0, ws + plan.scratch,
-                                 plan.scratch_bytes, dev_status, stream);
+    rc = forward_fill(net->dtype, net->act, B, D, H, a_in, ld_in, W[l], H, b != nullptr ? b[l] : nullptr, a_out, H, zlow, H, rbits,
+                      &st[l + 1], 0, ahead[l + 1] ? &queue : nullptr, ws + plan.scratch, plan.scratch_bytes, dev_status, stream);
+    if (rc != RAD_OK) return rc;
+    // still alone: the input of layer l, whose buffer the next layer writes, or the last input there is
+    if (queue.n == 1 && (queue.in[0].A == a_in || l == L - 2)) rc = queue.flush();
     if (rc != RAD_OK) return rc;
     a_in = a_out;
     ld_in = H;
   }
+  rc = queue.flush();
+  if (rc != RAD_OK) return rc;
   for (int l = 1; l < L; ++l)
     st[l].relubits = plan.layer[l].relubits >= 0 ? reinterpret_cast<uint32_t*>(ws + plan.layer[l].relubits) : nullptr;
   const int64_t C = net->dims[L];

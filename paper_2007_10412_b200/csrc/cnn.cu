@@ -147,12 +147,42 @@ extern "C" int rad_cnn_step(const rad_cnn_desc* d, const void* X, const int32_t*
     q.nnz = nnz_out != nullptr ? nnz_out + 2 * idx : reinterpret_cast<int64_t*>(ws + pl.nnz[idx]);
     q.relubits = nullptr;
   };
+  for (int idx = 0; idx < nl; ++idx)
+    make_store(idx, idx < pl.nc ? (int64_t)pl.H[idx] * pl.W[idx] * pl.Cin[idx] : pl.fdim[idx - pl.nc]);
+  for (int l = 0; l < pl.nc; ++l)
+    if (conv_W[l] == nullptr || dconv_W[l] == nullptr || dconv_b[l] == nullptr) return RAD_EINVAL;
+  for (int l = 0; l < pl.nf; ++l)
+    if (fc_W[l] == nullptr || dfc_W[l] == nullptr || dfc_b[l] == nullptr) return RAD_EINVAL;
+  // index parts depend on the key alone: those of all layers that can use them in one go
+  bool ahead[2 * kMaxLayers] = {};
+  rad_store list[2 * kMaxLayers];
+  int n_ahead = 0;
+  for (int idx = 0; idx < nl; ++idx) {
+    const int l = idx - pl.nc;
+    ahead[idx] = store_indices_ok(&st[idx]) ||
+                 (l > 0 && fill_can_fuse(d->dtype, B, pl.fdim[l - 1], pl.fdim[l], ws + pl.act[(idx - 1) & 1], pl.fdim[l - 1], fc_W[l - 1],
+                                         pl.fdim[l], fc_b != nullptr ? fc_b[l - 1] : nullptr, ws + pl.act[(idx - 1) & 1], pl.fdim[l],
+                                         nullptr, 0, &st[idx]));
+    if (ahead[idx]) list[n_ahead++] = st[idx];
+  }
+  if (n_ahead > 0) {
+    rc = launch_store_indices(list, n_ahead, true, dev_status, s);
+    if (rc != RAD_OK) return rc;
+  }
+  StoreQueue queue;
+  queue.dev_status = dev_status;
+  queue.s = s;
+  // Stores the input of a layer, or queues it; one that is queued already is the input of the layer before, whose buffer is
+  // written next.
+  auto store_input = [&](const void* a, int idx) {
+    if (ahead[idx]) return queue.add({a, st[idx].D, st[idx]});
+    const int rq = queue.flush();
+    return rq != RAD_OK ? rq : rad_linear_forward_store(a, st[idx].D, &st[idx], ws + pl.scratch, pl.scratch_bytes, dev_status, stream);
+  };
   // ---- forward ----
   const void* a_in = X;
   for (int l = 0; l < pl.nc; ++l) {
-    if (conv_W[l] == nullptr || dconv_W[l] == nullptr || dconv_b[l] == nullptr) return RAD_EINVAL;
-    make_store(l, (int64_t)pl.H[l] * pl.W[l] * pl.Cin[l]);
-    rc = rad_linear_forward_store(a_in, st[l].D, &st[l], ws + pl.scratch, pl.scratch_bytes, dev_status, stream);
+    rc = store_input(a_in, l);
     if (rc != RAD_OK) return rc;
     void* a_out = ws + pl.act[l & 1];
     // tensor cores where the shape allows (Cin 16 / 32 / 64: the later convolutions), CUDA cores otherwise
@@ -166,22 +196,27 @@ extern "C" int rad_cnn_step(const rad_cnn_desc* d, const void* X, const int32_t*
     if (rc != RAD_OK) return rc;
     a_in = a_out;
   }
+  rc = store_input(a_in, pl.nc);
+  if (rc != RAD_OK) return rc;
   for (int l = 0; l < pl.nf; ++l) {
     const int idx = pl.nc + l;
-    if (fc_W[l] == nullptr || dfc_W[l] == nullptr || dfc_b[l] == nullptr) return RAD_EINVAL;
     const int64_t D = pl.fdim[l], H = pl.fdim[l + 1];
-    make_store(idx, D);
-    rc = rad_linear_forward_store(a_in, D, &st[idx], ws + pl.scratch, pl.scratch_bytes, dev_status, stream);
+    const float* bias = fc_b != nullptr ? fc_b[l] : nullptr;
+    if (l == pl.nf - 1) {
+      rc = rad_linear_forward(d->dtype, RAD_ACT_NONE, B, D, H, a_in, D, fc_W[l], H, bias, nullptr, H,
+                              reinterpret_cast<float*>(ws + pl.logits), H, nullptr, 0, nullptr, dev_status, stream);
+    } else {
+      void* a_out = ws + pl.act[idx & 1];
+      rc = forward_fill(d->dtype, RAD_ACT_RELU, B, D, H, a_in, D, fc_W[l], H, bias, a_out, H, nullptr, 0,
+                        reinterpret_cast<uint32_t*>(ws + pl.relubits[idx + 1]), &st[idx + 1], 0, ahead[idx + 1] ? &queue : nullptr, ws + pl.scratch,
+                        pl.scratch_bytes, dev_status, stream);
+      if (rc == RAD_OK && queue.n == 1 && queue.in[0].A == a_in) rc = queue.flush();      // its buffer is written next
+      a_in = a_out;
+    }
     if (rc != RAD_OK) return rc;
-    const bool last = l == pl.nf - 1;
-    void* a_out = last ? nullptr : ws + pl.act[idx & 1];
-    rc = rad_linear_forward(d->dtype, last ? RAD_ACT_NONE : RAD_ACT_RELU, B, D, H, a_in, D, fc_W[l], H,
-                            fc_b != nullptr ? fc_b[l] : nullptr, a_out, H,
-                            last ? reinterpret_cast<float*>(ws + pl.logits) : nullptr, H, nullptr, 0,
-                            last ? nullptr : reinterpret_cast<uint32_t*>(ws + pl.relubits[idx + 1]), dev_status, stream);
-    if (rc != RAD_OK) return rc;
-    a_in = a_out;
   }
+  rc = queue.flush();
+  if (rc != RAD_OK) return rc;
   // ---- loss ----
   const int64_t C = pl.fdim[pl.nf];
   void* g = ws + pl.grad[(nl - 1) & 1];
@@ -192,14 +227,19 @@ extern "C" int rad_cnn_step(const rad_cnn_desc* d, const void* X, const int32_t*
   for (int l = pl.nf - 1; l >= 0; --l) {
     const int idx = pl.nc + l;
     const int64_t D = pl.fdim[l], H = pl.fdim[l + 1];
-    rc = rad_linear_weight_grad(&st[idx], g, H, H, dfc_W[l], H, ws + pl.scratch, pl.scratch_bytes, dev_status, stream);
-    if (rc != RAD_OK) return rc;
     void* g_prev = ws + pl.grad[(idx - 1) & 1];
     // the first linear layer reads the pooled map, which is not a ReLU output: no mask there
-    rc = rad_linear_input_grad(d->dtype, B, D, H, g, H, fc_W[l], H,
-                               l > 0 ? reinterpret_cast<const uint32_t*>(ws + pl.relubits[idx]) : nullptr, nullptr, 0,
-                               g_prev, D, dfc_b[l], ws + pl.scratch, pl.scratch_bytes, dev_status, stream);
+    const uint32_t* mask = l > 0 ? reinterpret_cast<const uint32_t*>(ws + pl.relubits[idx]) : nullptr;
+    const SimtInputGrad ig = {fc_W[l], H, mask, nullptr, 0, g_prev, D};
+    bool db_done = false, dx_done = false;
+    rc = weight_grad_and_bias(&st[idx], g, H, H, dfc_W[l], H, ws + pl.scratch, pl.scratch_bytes, dev_status, stream, dfc_b[l], &db_done,
+                              &ig, &dx_done);
     if (rc != RAD_OK) return rc;
+    if (!db_done || !dx_done) {
+      rc = rad_linear_input_grad(d->dtype, B, D, H, g, H, fc_W[l], H, mask, nullptr, 0, dx_done ? nullptr : g_prev, D,
+                                 db_done ? nullptr : dfc_b[l], ws + pl.scratch, pl.scratch_bytes, dev_status, stream);
+      if (rc != RAD_OK) return rc;
+    }
     g = g_prev;
   }
   // ---- backward: conv blocks (g = gradient of the pooled output of block l) ----

@@ -251,6 +251,39 @@ int column_sums(int dtype, int64_t B, int64_t H, const void* dZ, int64_t ldz, fl
                 void* workspace, int64_t workspace_bytes, cudaStream_t s);
 int64_t column_sums_workspace(int64_t B, int64_t H);
 
+// store.cu: values and ReLU bits of a different-sample Bernoulli store whose index part is in place
+bool store_indices_ok(const rad_store* st);
+struct StoreInput { const void* A; int64_t lda; rad_store st; };
+int launch_store_values(const StoreInput* in, int n, int32_t* dev_status, cudaStream_t s);     // one or two stores of one type
+// The layer inputs of a net whose values are still to be put in place.  They are needed in the backward pass only, so a
+// launch takes two; an activation has to be stored before the forward pass comes round to its buffer again.
+struct StoreQueue {
+  StoreInput in[2];
+  int n = 0;
+  int32_t* dev_status;
+  cudaStream_t s;
+  int add(const StoreInput& x) {
+    in[n++] = x;
+    return n == 2 ? flush() : RAD_OK;
+  }
+  int flush() {
+    const int k = n;
+    n = 0;
+    return k > 0 ? launch_store_values(in, k, dev_status, s) : RAD_OK;
+  }
+};
+
+// api.cu: the routes behind rad_linear_forward_fill and rad_linear_weight_grad, for the whole-net steps
+bool fill_can_fuse(int dtype, int64_t B, int64_t D, int64_t H, const void* A, int64_t lda, const void* W, int64_t ldw, const float* bias,
+                   const void* out_act, int64_t ld_act, const void* out_zlow, int64_t ld_zlow, const rad_store* next);
+int forward_fill(int32_t dtype, int32_t act, int64_t B, int64_t D, int64_t H, const void* A, int64_t lda, const void* W, int64_t ldw,
+                 const float* bias, void* out_act, int64_t ld_act, void* out_zlow, int64_t ld_zlow, uint32_t* relubits,
+                 const rad_store* next, int32_t index_ready, StoreQueue* ahead, void* workspace, int64_t workspace_bytes,
+                 int32_t* dev_status, void* stream);
+int weight_grad_and_bias(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, float* dW, int64_t ldw, void* workspace,
+                         int64_t workspace_bytes, int32_t* dev_status, void* stream, float* db, bool* db_written,
+                         const SimtInputGrad* ig = nullptr, bool* ig_done = nullptr);
+
 // 3x3 convolution layers (conv.cu)
 int conv_forward_pool(int dtype, int64_t B, int H, int W, int Cin, int Cout, const void* X, const void* Wt,
                       const float* bias, void* P, uint32_t* relubits, cudaStream_t st);
@@ -287,6 +320,8 @@ int tc_forward(int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t 
 // store_index.cu: keep bits, row offsets, tile offsets and nnz of a different-sample Bernoulli store from the
 // key alone (no layer input is read)
 int launch_store_index(const rad_store* st, bool check_capacity, int32_t* dev_status, cudaStream_t s);
+// of all (Bernoulli) stores of a net, which share seed, step and keep probability
+int launch_store_indices(const rad_store* st, int n, bool check_capacity, int32_t* dev_status, cudaStream_t s);
 int launch_offsets_scan(uint32_t* offsets, int64_t ntiles, int64_t* nnz, int64_t capacity, int32_t* dev_status, cudaStream_t s);
 // store_rows.cu: fixed-count law (exactly k columns per row): static-shape store, key-only index, re-tiling
 bool rows_store_ok(const rad_store* st);
@@ -372,6 +407,10 @@ __device__ __forceinline__ float ld_cluster_f32(const float* smem, uint32_t rank
 __device__ __forceinline__ void st_cluster_f32(float* smem, uint32_t rank, float v) {
   asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, %1;\n\tst.shared::cluster.f32 [a], %2;\n\t}"
                ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "r"(rank), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster_u32(uint32_t* smem, uint32_t rank, uint32_t v) {
+  asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, %1;\n\tst.shared::cluster.u32 [a], %2;\n\t}"
+               ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "r"(rank), "r"(v) : "memory");
 }
 // ---- launches ------------------------------------------------------------------------------------
 // Every kernel may be launched while the one before it in the stream still runs (programmatic stream serialization): its

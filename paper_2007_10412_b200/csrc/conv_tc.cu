@@ -371,8 +371,9 @@ __global__ void __launch_bounds__(kCvThreads, 3) conv_tc_kernel(const ConvTcPara
   }
 }
 
-// A_hat (B x D, zero where dropped) from a compact store: the buffer is cleared first, then the kept values
-// are dropped in place.  different-sample: a thread per keep-bit word; same-sample: a thread per kept entry.
+// A_hat (B x D, zero where dropped) from a compact store.  different-sample: a thread per keep-bit word writes its 32
+// columns, zeros first, so that the buffer needs no clearing of its own (a clear between two kernels costs both of them their
+// overlap: 3 us).  same-sample: the buffer is cleared, then a thread per kept entry.
 __global__ void __launch_bounds__(256) densify_different_kernel(const bf16* values, const uint32_t* keepbits, const uint32_t* offsets,
                                                                 int64_t B, int64_t D, int32_t ncb, int64_t capacity, bf16* out) {
   begin_after_previous();
@@ -380,16 +381,19 @@ __global__ void __launch_bounds__(256) densify_different_kernel(const bf16* valu
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nwords; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t tile = i / kBitWords;
     const int t = (int)(i - tile * kBitWords), r = t >> 2, w = t & 3;
+    const int64_t row = (tile / ncb) * kTileRows + r, col0 = (tile % ncb) * kTileCols + 32 * w;
+    if (row >= B || col0 >= D) continue;
+    bf16* dst = out + row * D + col0;               // D is a multiple of 64: whole words, 16-byte aligned
+#pragma unroll
+    for (int j = 0; j < 4; ++j) reinterpret_cast<uint4*>(dst)[j] = make_uint4(0u, 0u, 0u, 0u);
     const uint32_t* tw = keepbits + tile * kTileWords;
     uint32_t word = tw[t];
-    if (word == 0) continue;
     int64_t pos = (int64_t)offsets[tile] + ((tw[kBitWords + (r >> 1)] >> (16 * (r & 1))) & 0xffffu);
     for (int q = 0; q < w; ++q) pos += __popc(tw[r * 4 + q]);
-    const int64_t row = (tile / ncb) * kTileRows + r, col0 = (tile % ncb) * kTileCols + 32 * w;
     while (word != 0) {
       const int b = __ffs(word) - 1;
       word &= word - 1;
-      if (row < B && col0 + b < D && pos < capacity) out[row * D + col0 + b] = values[pos];
+      if (pos < capacity) dst[b] = values[pos];
       ++pos;
     }
   }
@@ -474,9 +478,9 @@ int conv_tc_weight_grad(const rad_store* store, int H, int W, int Cin, int Cout,
   if (workspace == nullptr || workspace_bytes < conv_tc_weight_grad_workspace(B, H, W, Cin, Cout)) return RAD_EWORKSPACE;
   bf16* dense = static_cast<bf16*>(workspace);
   float* partial = reinterpret_cast<float*>(static_cast<char*>(workspace) + round_up(B * D * 2, 256));
-  RAD_CUDA_TRY(cudaMemsetAsync(dense, 0, (size_t)(B * D * 2), st));
   count_launch();
   if (store->variant == RAD_SAME_SAMPLE) {
+    RAD_CUDA_TRY(cudaMemsetAsync(dense, 0, (size_t)(B * D * 2), st));
     RAD_TRY(launch_kernel(densify_same_kernel, (unsigned)std::min<int64_t>(ceil_div(B * store->values_ld, 256), 148 * 16), 256, 0, st, static_cast<const bf16*>(store->values), store->offsets, store->nnz, B, D, store->values_ld, dense));
   } else {
     const int32_t ncb = (int32_t)ceil_div(D, kTileCols);

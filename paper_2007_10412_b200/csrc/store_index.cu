@@ -5,9 +5,13 @@
 // then drops the kept values into place from its epilogue (tc.cu), and a caller learns the exact size of a
 // store before it allocates `values`.
 //
-//   store_index_kernel   one tile (64 x 128 entries) per warp and turn: draw and write the keep-bit words,
-//                        in-tile row offsets from warp scans, exact kept count of the tile into offsets[tile]
-//   offsets_scan_kernel  one CTA turns the counts into padded exclusive prefixes in place and writes nnz
+// The index parts of all layers of a net are drawn in one go (a net's layers share seed, step and keep probability).
+//
+//   store_index_small_kernel  layers of few tiles: one launch, a cluster of eight CTAs per layer, which hand their kept
+//                             counts on through distributed shared memory
+//   store_index_kernel        one tile (64 x 128 entries) per warp and turn: draw and write the keep-bit words,
+//                             in-tile row offsets from warp scans, exact kept count of the tile into offsets[tile]
+//   offsets_scan_kernel       one CTA per layer turns the counts into padded exclusive prefixes in place and writes nnz
 //
 // Layout and bits are those of the one-pass store kernels.
 #include <algorithm>
@@ -17,56 +21,122 @@
 namespace rad {
 namespace {
 
-struct IndexParams {
-  int64_t B, D;
-  int32_t ncb, ntiles;
-  KeepThreshold T;
-  uint32_t c2, c3;
+struct IndexLayer {
+  uint32_t rows, cols, ncb, ntiles;
+  uint32_t tile0;       // tiles of the layers before it
+  uint32_t c2;
   uint32_t* keepbits;
   uint32_t* offsets;
   int64_t* nnz;
   int64_t capacity;     // elements of `values` the caller holds; < 0: not checked
+};
+constexpr int kIndexLayers = 16;   // layers of one launch
+struct IndexParams {
+  IndexLayer layer[kIndexLayers];
+  int32_t nlayers;
+  uint32_t ntiles;      // of all of them
+  KeepThreshold T;
+  uint32_t c3;
   int32_t* dev_status;
 };
 
-// One warp per tile and turn, no CTA-wide step: lane l draws words l, l + 32, ... of the tile (word t = row
-// t / 4, columns 32 (t % 4) ..), so a warp's stores are contiguous and a warp scan per turn, carried over
-// the eight turns, gives every row its offset in (row, column) order.
-constexpr int kIndexWarps = 4;
-__global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const IndexParams p, const PhiloxKeys ks) {
+// One tile by one warp, no CTA-wide step: lane l draws words l, l + 32, ... of the tile (word t = row t / 4, columns
+// 32 (t % 4) ..), so a warp's stores are contiguous and a warp scan per turn, carried over the eight turns, gives every
+// row its offset in (row, column) order.  Returns the tile's kept count.
+__device__ __forceinline__ uint32_t index_tile(const IndexLayer& L, uint32_t tile, const KeepThreshold& T, uint32_t c3, const PhiloxKeys& ks,
+                                               int lane) {
+  const uint32_t slab = tile / L.ncb, cb = tile - slab * L.ncb;
+  const int w = lane & 3;
+  const uint32_t col0 = cb * kTileCols + 32u * w;
+  uint32_t* tw = L.keepbits + (int64_t)tile * kTileWords;
+  uint32_t base = 0;
+#pragma unroll 2
+  for (int i = 0; i < kBitWords / 32; ++i) {
+    const int r = i * 8 + (lane >> 2);
+    const uint32_t row = slab * kTileRows + r;
+    uint32_t m = 0;
+    if (row < L.rows && col0 < L.cols) {
+      m = philox_keep32(col0 >> 5, row, L.c2, c3, ks, T);
+      const uint32_t nv = L.cols - col0;
+      if (nv < 32) m &= (1u << nv) - 1u;
+    }
+    tw[i * 32 + lane] = m;
+    const uint32_t c = __popc(m);
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t n = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += n;
+    }
+    if (w == 0) reinterpret_cast<uint16_t*>(tw + kBitWords)[r] = (uint16_t)(base + incl - c);
+    base += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  return base;
+}
+__device__ __forceinline__ uint32_t padded_count(uint32_t c) { return (c + kValueAlign - 1) / kValueAlign * kValueAlign; }
+__device__ __forceinline__ void write_totals(const IndexLayer& L, uint32_t padded, uint32_t exact, int32_t* dev_status) {
+  L.offsets[L.ntiles] = padded;
+  L.nnz[0] = (int64_t)exact;
+  L.nnz[1] = (int64_t)padded;
+  if (L.capacity >= 0 && (int64_t)padded > L.capacity) raise_status(dev_status, RAD_DEV_ECAPACITY);
+}
+
+constexpr int kIndexWarps = 16;
+constexpr int kIndexSmemOne = 120 * 1024, kIndexSmemTwo = 100 * 1024;     // asked for so that one or two CTAs fit an SM
+__global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const __grid_constant__ IndexParams p, const PhiloxKeys ks) {
   wait_for_previous();
   const int lane = threadIdx.x & 31;
   const uint32_t warp0 = blockIdx.x * kIndexWarps + (threadIdx.x >> 5), nwarps = gridDim.x * kIndexWarps;
-  const uint32_t nrows = (uint32_t)p.B, ncols = (uint32_t)p.D, ncb = (uint32_t)p.ncb;
-  const int w = lane & 3;
-  for (uint32_t tile = warp0; tile < (uint32_t)p.ntiles; tile += nwarps) {
-    if ((uint64_t)tile + nwarps >= (uint32_t)p.ntiles) let_next_start();
-    const uint32_t slab = tile / ncb, cb = tile - slab * ncb;
-    const uint32_t col0 = cb * kTileCols + 32u * w;
-    uint32_t* tw = p.keepbits + (int64_t)tile * kTileWords;
-    uint32_t base = 0;
-#pragma unroll 2
-    for (int i = 0; i < kBitWords / 32; ++i) {
-      const int r = i * 8 + (lane >> 2);
-      const uint32_t row = slab * kTileRows + r;
-      uint32_t m = 0;
-      if (row < nrows && col0 < ncols) {
-        m = philox_keep32(col0 >> 5, row, p.c2, p.c3, ks, p.T);
-        const uint32_t nv = ncols - col0;
-        if (nv < 32) m &= (1u << nv) - 1u;
-      }
-      tw[i * 32 + lane] = m;
-      const uint32_t c = __popc(m);
-      uint32_t incl = c;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t n = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += n;
-      }
-      if (w == 0) reinterpret_cast<uint16_t*>(tw + kBitWords)[r] = (uint16_t)(base + incl - c);
-      base += __shfl_sync(0xffffffffu, incl, 31);
+  int l = 0;
+  for (uint32_t t = warp0; t < p.ntiles; t += nwarps) {
+    if ((uint64_t)t + nwarps >= p.ntiles) let_next_start();
+    while (l + 1 < p.nlayers && t >= p.layer[l + 1].tile0) ++l;
+    const uint32_t tile = t - p.layer[l].tile0;
+    const uint32_t count = index_tile(p.layer[l], tile, p.T, p.c3, ks, lane);
+    if (lane == 0) p.layer[l].offsets[tile] = count;
+  }
+}
+
+// Layers of at most kSmallIndexTiles tiles: cluster l (eight CTAs) makes layer l, CTA r of it a run of its tiles.  What
+// bounds a small index is launches, not the draw: drawn and scanned in two launches per layer, the layers of a
+// 640-520-392-200 net at batch 328 took 20 us of its step, in one launch for all of them 6.  An SM draws a tile in 0.26 us (three generator calls per word, 3 G calls/s), so with
+// more than twelve tiles a CTA the two launches of the general form, on all SMs, are faster.
+constexpr int kSmallIndexCtas = 8, kSmallIndexTiles = 12 * kSmallIndexCtas;
+__global__ void __launch_bounds__(32 * kIndexWarps) store_index_small_kernel(const __grid_constant__ IndexParams p, const PhiloxKeys ks) {
+  begin_after_previous();
+  __shared__ uint32_t s_count[kSmallIndexTiles / kSmallIndexCtas];
+  __shared__ uint32_t s_padded[kSmallIndexCtas], s_exact[kSmallIndexCtas];      // of every CTA of the cluster
+  const IndexLayer& L = p.layer[blockIdx.x / kSmallIndexCtas];
+  const uint32_t rank = cluster_ctarank(), per = (L.ntiles + kSmallIndexCtas - 1) / kSmallIndexCtas;
+  const uint32_t t0 = min(rank * per, L.ntiles), n = min(per, L.ntiles - t0);
+  const int tid = threadIdx.x, lane = tid & 31;
+  for (uint32_t i = tid >> 5; i < n; i += kIndexWarps) {
+    const uint32_t count = index_tile(L, t0 + i, p.T, p.c3, ks, lane);
+    if (lane == 0) s_count[i] = count;
+  }
+  __syncthreads();
+  if (tid < kSmallIndexCtas) {
+    uint32_t padded = 0, exact = 0;
+    for (uint32_t i = 0; i < n; ++i) {
+      padded += padded_count(s_count[i]);
+      exact += s_count[i];
     }
-    if (lane == 0) p.offsets[tile] = base;
+    st_cluster_u32(&s_padded[rank], (uint32_t)tid, padded);
+    st_cluster_u32(&s_exact[rank], (uint32_t)tid, exact);
+  }
+  cluster_barrier();
+  if (tid == 0) {
+    uint32_t at = 0, exact = 0, all = 0;
+    for (uint32_t r = 0; r < kSmallIndexCtas; ++r) {
+      if (r < rank) at += s_padded[r];
+      all += s_padded[r];
+      exact += s_exact[r];
+    }
+    for (uint32_t i = 0; i < n; ++i) {
+      L.offsets[t0 + i] = at;
+      at += padded_count(s_count[i]);
+    }
+    if (rank == 0) write_totals(L, all, exact, p.dev_status);
   }
 }
 
@@ -75,27 +145,30 @@ __global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const Ind
 // tiles per round; a thread takes 16 consecutive tiles (four 16-byte loads and stores where `offsets` is
 // 16-byte aligned), adds them up locally, and one warp scan plus one pass over the warp sums places them.
 constexpr int kScanPer = 16;
-__global__ void __launch_bounds__(1024) offsets_scan_kernel(const IndexParams p, int vec) {
+__global__ void __launch_bounds__(1024) offsets_scan_kernel(const __grid_constant__ IndexParams p) {
   begin_after_previous();
+  const IndexLayer& L = p.layer[blockIdx.x];
+  uint32_t* offsets = L.offsets;
+  const bool vec = ((uintptr_t)offsets & 15) == 0;
   __shared__ uint64_t s_warp[32];                   // padded sum in the high half, exact sum in the low half
   __shared__ uint64_t s_carry;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) s_carry = 0;
   __syncthreads();
-  const int64_t ntiles = p.ntiles;
+  const int64_t ntiles = L.ntiles;
   for (int64_t r0 = 0; r0 < ntiles; r0 += 1024 * kScanPer) {
     const int64_t t0 = r0 + (int64_t)tid * kScanPer;
-    const bool whole = vec != 0 && t0 + kScanPer <= ntiles;
+    const bool whole = vec && t0 + kScanPer <= ntiles;
     uint32_t c[kScanPer];
     if (whole) {
 #pragma unroll
       for (int i = 0; i < kScanPer; i += 4) {
-        const uint4 q = *reinterpret_cast<const uint4*>(p.offsets + t0 + i);
+        const uint4 q = *reinterpret_cast<const uint4*>(offsets + t0 + i);
         c[i] = q.x; c[i + 1] = q.y; c[i + 2] = q.z; c[i + 3] = q.w;
       }
     } else {
 #pragma unroll
-      for (int i = 0; i < kScanPer; ++i) c[i] = t0 + i < ntiles ? p.offsets[t0 + i] : 0u;
+      for (int i = 0; i < kScanPer; ++i) c[i] = t0 + i < ntiles ? offsets[t0 + i] : 0u;
     }
     // a round holds at most 16384 * 8192 entries: 32 bits each for the padded and the exact sum
     uint64_t mine = 0;
@@ -128,11 +201,11 @@ __global__ void __launch_bounds__(1024) offsets_scan_kernel(const IndexParams p,
     if (whole) {
 #pragma unroll
       for (int i = 0; i < kScanPer; i += 4)
-        *reinterpret_cast<uint4*>(p.offsets + t0 + i) = make_uint4(o[i], o[i + 1], o[i + 2], o[i + 3]);
+        *reinterpret_cast<uint4*>(offsets + t0 + i) = make_uint4(o[i], o[i + 1], o[i + 2], o[i + 3]);
     } else {
 #pragma unroll
       for (int i = 0; i < kScanPer; ++i)
-        if (t0 + i < ntiles) p.offsets[t0 + i] = o[i];
+        if (t0 + i < ntiles) offsets[t0 + i] = o[i];
     }
     __syncthreads();                                // everyone has read the carry and the warp sums
     if (tid == 0) s_carry = carry + round_total;
@@ -140,10 +213,7 @@ __global__ void __launch_bounds__(1024) offsets_scan_kernel(const IndexParams p,
   }
   if (tid == 0) {
     const uint64_t total = s_carry;
-    p.offsets[ntiles] = (uint32_t)(total >> 32);
-    p.nnz[0] = (int64_t)(total & 0xffffffffu);
-    p.nnz[1] = (int64_t)(total >> 32);
-    if (p.capacity >= 0 && (int64_t)(total >> 32) > p.capacity) raise_status(p.dev_status, RAD_DEV_ECAPACITY);
+    write_totals(L, (uint32_t)(total >> 32), (uint32_t)(total & 0xffffffffu), p.dev_status);
   }
 }
 
@@ -153,30 +223,61 @@ __global__ void __launch_bounds__(1024) offsets_scan_kernel(const IndexParams p,
 int launch_offsets_scan(uint32_t* offsets, int64_t ntiles, int64_t* nnz, int64_t capacity, int32_t* dev_status,
                         cudaStream_t s) {
   IndexParams p = {};
-  p.ntiles = (int32_t)ntiles; p.offsets = offsets; p.nnz = nnz; p.capacity = capacity; p.dev_status = dev_status;
+  p.nlayers = 1; p.dev_status = dev_status;
+  p.layer[0].ntiles = (uint32_t)ntiles; p.layer[0].offsets = offsets; p.layer[0].nnz = nnz; p.layer[0].capacity = capacity;
   count_launch();
-  RAD_TRY(launch_kernel(offsets_scan_kernel, 1, 1024, 0, s, p, ((uintptr_t)offsets & 15) == 0 ? 1 : 0));
+  RAD_TRY(launch_kernel(offsets_scan_kernel, 1, 1024, 0, s, p));
   return RAD_OK;
 }
 
-// Index part (keep bits, row offsets, tile offsets, nnz) of a different-sample Bernoulli store.
+// Index parts (keep bits, row offsets, tile offsets, nnz) of the different-sample Bernoulli stores of one net: one seed,
+// step and keep probability.
+int launch_store_indices(const rad_store* st, int n, bool check_capacity, int32_t* dev_status, cudaStream_t s) {
+  const PhiloxKeys ks = philox_expand_key(st[0].seed);
+  for (int first = 0; first < n; first += kIndexLayers) {
+    IndexParams p = {};
+    p.nlayers = std::min(n - first, kIndexLayers);
+    p.T = make_keep_threshold(keep_threshold_host(st[0].p));
+    p.c3 = st[0].step;
+    p.dev_status = dev_status;
+    bool small = true;
+    for (int l = 0; l < p.nlayers; ++l) {
+      const rad_store& q = st[first + l];
+      IndexLayer& L = p.layer[l];
+      L.rows = (uint32_t)q.B; L.cols = (uint32_t)q.D;
+      L.ncb = (uint32_t)ceil_div(q.D, kTileCols);
+      L.ntiles = (uint32_t)ceil_div(q.B, kTileRows) * L.ncb;
+      L.tile0 = p.ntiles;
+      L.c2 = counter_word2(q.layer, RAD_DIFFERENT_SAMPLE);
+      L.keepbits = q.keepbits; L.offsets = q.offsets; L.nnz = q.nnz;
+      L.capacity = check_capacity ? q.values_capacity : -1;
+      p.ntiles += L.ntiles;
+      small = small && L.ntiles <= (uint32_t)kSmallIndexTiles;
+    }
+    count_launch();
+    if (small) {
+      RAD_TRY(launch_with_cluster(store_index_small_kernel, p.nlayers * kSmallIndexCtas, 32 * kIndexWarps, 0, dim3(kSmallIndexCtas, 1, 1),
+                                  s, p, ks));
+      continue;
+    }
+    // One CTA of sixteen warps on every SM, two where there are tiles for them, and the shared memory says so: started early
+    // beside a tensor-core kernel that leaves a few SMs idle, CTAs without that share those few (1024 tiles behind an
+    // input gradient on 128 of 148 SMs: 12.5 us, 6 otherwise).
+    static std::atomic<uint64_t> ready{0};
+    const int64_t ctas = ceil_div(p.ntiles, kIndexWarps);
+    if (!allow_smem(store_index_kernel, kIndexSmemOne, ready)) return RAD_ECUDA;
+    RAD_TRY(launch_kernel(store_index_kernel, (unsigned)std::min<int64_t>(ctas, 2 * 148), 32 * kIndexWarps,
+                          ctas <= 148 ? kIndexSmemOne : kIndexSmemTwo, s, p, ks));
+    count_launch();
+    RAD_TRY(launch_kernel(offsets_scan_kernel, p.nlayers, 1024, 0, s, p));
+  }
+  return RAD_OK;
+}
+
+// Index part of one different-sample store.
 int launch_store_index(const rad_store* st, bool check_capacity, int32_t* dev_status, cudaStream_t s) {
-  const uint32_t T = keep_threshold_host(st->p);
-  IndexParams p;
-  p.B = st->B; p.D = st->D;
-  p.ncb = (int32_t)ceil_div(st->D, kTileCols);
-  p.ntiles = (int32_t)(ceil_div(st->B, kTileRows) * p.ncb);
-  p.T = make_keep_threshold(T);
-  p.c2 = counter_word2(st->layer, RAD_DIFFERENT_SAMPLE); p.c3 = st->step;
-  p.keepbits = st->keepbits; p.offsets = st->offsets; p.nnz = st->nnz;
-  p.capacity = check_capacity ? st->values_capacity : -1;
-  p.dev_status = dev_status;
-  const PhiloxKeys ks = philox_expand_key(st->seed);
-  const int grid = (int)std::min<int64_t>(ceil_div(p.ntiles, kIndexWarps), 148 * 12);
   if (st->law == RAD_LAW_FIXED) return launch_fixed_index(st, check_capacity, dev_status, s);
-  count_launch();
-  RAD_TRY(launch_kernel(store_index_kernel, grid, 32 * kIndexWarps, 0, s, p, ks));
-  return launch_offsets_scan(p.offsets, p.ntiles, p.nnz, p.capacity, dev_status, s);
+  return launch_store_indices(st, 1, check_capacity, dev_status, s);
 }
 
 }  // namespace rad

@@ -24,6 +24,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -37,7 +38,11 @@ constexpr int kRasterGroup = 16;               // m-tiles per raster group (16 x
 
 enum AKind { kAK = 0, kAMN = 1, kASparse = 2 };
 enum BKind { kBK_ = 0, kBMN = 1 };
-enum EpiKind { kFwd = 0, kDx = 1, kDwT = 2 };
+// Epilogues: forward pass by activation (RAD_ACT_*), without and with the filling of the next layer's store; input gradient,
+// plain or masked by ReLU bits, and times GELU'(z); same-sample dW, transposed.
+enum EpiKind { kFwd = 0, kFwdFill = 3, kDx = 6, kDxGelu = 7, kDwT = 8 };
+constexpr bool is_forward(int epi) { return epi < kDx; }
+constexpr bool is_dx(int epi) { return epi == kDx || epi == kDxGelu; }
 
 struct TcParams {
   int64_t M, N, K;
@@ -179,11 +184,12 @@ struct Schedule {
 // eight bank groups, and one TMA store takes the chunk away.  Rows and columns past the matrix are cut off by the tensor map.
 // What the epilogue reads (the next store's index, ReLU bits, z of the GELU derivative) is on its way before the
 // accumulators are waited for.
-constexpr int kEpiWarps = 8;
 constexpr int kChunkBytes = 32 * 64;             // 32 rows x 32 bf16 columns
-constexpr int kFillBytes = 3584;                 // staged values of the next store, per warp
-constexpr int kBiasBytes = 128 * 4;              // bias of a warp's columns
-constexpr int kEpiBytes = 4 * kChunkBytes + kFillBytes + kBiasBytes;   // of a warp: a ring of four chunks, and those
+constexpr int kRingBytes = 32 * kChunkBytes;     // chunk buffers of all epilogue warps: four each of eight, two each of sixteen
+constexpr int kFillBytes = 3584;                 // kept values of 32 rows and 128 columns on their way to the next store
+constexpr int kFillBuffers = 8;                  // four lane quarters, two tiles of 128 columns
+constexpr int kBiasBytes = 8 * 128 * 4;          // every warp's columns of the bias
+constexpr int kEpiBytes = kRingBytes + kFillBuffers * kFillBytes + kBiasBytes;
 constexpr uint32_t kFillValues = kFillBytes / 2;
 
 __device__ __forceinline__ uint32_t chunk16_addr(uint32_t base, int row, int unit) { return base + row * 64 + ((unit ^ ((row >> 1) & 3)) << 4); }
@@ -260,7 +266,7 @@ struct StoreRow {
   uint4 bits;                // the row's four keep-bit words of the tile
   uint32_t pos;              // where its first kept entry of the tile goes
   uint32_t seg, end;         // warp: kept entries of its 32 rows go to seg .. end
-  bool staged;               // warp: they are collected in shared memory and copied out in 16-byte pieces
+  bool staged;               // warp: they are collected in shared memory and copied out in 16-byte pieces, by the warps of the tile
   __device__ __forceinline__ void load(const TcParams& p, int64_t m, int64_t n, bool row_ok, bool whole_tile) {
     bits = make_uint4(0u, 0u, 0u, 0u);
     pos = end = 0u;
@@ -316,10 +322,10 @@ __device__ __forceinline__ void place_kept(const TcParams& p, const uint32_t (&a
     }
   }
 }
-// The warp's staged entries to their places, 16 bytes at a time where all eight are its own.
-__device__ __forceinline__ void copy_kept(const TcParams& p, const StoreRow& sr, uint32_t fill, int lane) {
+// The staged entries to their places, 16 bytes at a time where all eight belong to the rows, by `threads` threads.
+__device__ __forceinline__ void copy_kept(const TcParams& p, const StoreRow& sr, uint32_t fill, int thread, int threads) {
   const uint32_t base = sr.seg & ~7u, end = (uint32_t)min((int64_t)sr.end, p.st_capacity);
-  for (uint32_t q = base + 8u * lane; q < end; q += 256u) {
+  for (uint32_t q = base + 8u * thread; q < end; q += 8u * threads) {
     const uint4 v = ld_shared16(fill + 2u * (q - base));
     if (q >= sr.seg && q + 8u <= end) {
       *reinterpret_cast<uint4*>(p.st_values + q) = v;
@@ -343,10 +349,14 @@ __device__ __forceinline__ void pad_store_tile(const TcParams& p, int64_t m, int
   for (uint32_t q = p.st_offsets[tile] + exact; q < end; ++q) p.st_values[q] = __float2bfloat16_rn(0.0f);
 }
 
+// the ring's slot of a chunk: one, or the first of two
+template <int kSlots>
+__device__ __forceinline__ int chunk_slot(int turn, bool both) { return both ? turn % (kSlots / 2) * 2 : turn % kSlots; }
+
 // One chunk of the forward pass: r holds the 32 float32 accumulators of row m, columns n .. n + 31 (as bit patterns);
-// y0 is the warp's first row.  `turn` counts the warp's chunks.  Returns the chunk's ReLU bits.  The activation is a template
+// y0 is the warp's first row.  `turn` counts the warp's chunks, `stage` is its ring of kSlots chunk buffers.  Returns the chunk's ReLU bits.  The activation is a template
 // parameter: what is not used is not there to be jumped over, which cost 4 us a tile of 128 x 256 (instruction fetch).
-template <int ACT>
+template <int ACT, int kSlots>
 __device__ __forceinline__ uint32_t forward_chunk(const TcParams& p, const CUtensorMap* tm_act, const CUtensorMap* tm_zlow,
                                                   const CUtensorMap* tm_z, const uint32_t (&r)[32], int y0, int n, int lane,
                                                   uint32_t stage, uint32_t bias, int turn, uint32_t (&ab)[16]) {
@@ -365,10 +375,10 @@ __device__ __forceinline__ uint32_t forward_chunk(const TcParams& p, const CUten
   }
   const bool z_only = p.out_act == nullptr && p.out_zlow == nullptr;
   if (p.out_z != nullptr) {
-    // two buffers of 4 KB; where 16-bit results follow they share the ring
-    const uint32_t buf = z_only ? stage + (turn & 1) * 2 * kChunkBytes : stage;
+    // buffers of 4 KB; where 16-bit results follow they share the ring
+    const uint32_t buf = z_only ? stage + turn % (kSlots / 2) * 2 * kChunkBytes : stage;
     if (elect_one()) {
-      if (z_only) tma_store_wait_read<1>();
+      if (z_only) tma_store_wait_read<kSlots / 2 - 1>();
       else tma_store_wait_read<0>();
     }
     __syncwarp();
@@ -418,15 +428,15 @@ __device__ __forceinline__ uint32_t forward_chunk(const TcParams& p, const CUten
   }
   // one output takes a buffer of the ring a chunk, two take a pair of them
   const bool both = p.out_zlow != nullptr && p.out_act != nullptr;
-  if (turn >= 2 || p.out_z != nullptr) {
+  if (turn >= kSlots / 2 || p.out_z != nullptr) {
     if (elect_one()) {
       if (p.out_z != nullptr) tma_store_wait_read<0>();
-      else if (both) tma_store_wait_read<1>();
-      else tma_store_wait_read<3>();
+      else if (both) tma_store_wait_read<kSlots / 2 - 1>();
+      else tma_store_wait_read<kSlots - 1>();
     }
     __syncwarp();
   }
-  const uint32_t first = stage + (both ? (turn & 1) * 2 : turn & 3) * kChunkBytes, second = first + kChunkBytes;
+  const uint32_t first = stage + chunk_slot<kSlots>(turn, both) * kChunkBytes, second = first + kChunkBytes;
   if (p.out_act != nullptr) {
 #pragma unroll
     for (int u = 0; u < 4; ++u) st_shared16(chunk16_addr(first, lane, u), ab[4 * u], ab[4 * u + 1], ab[4 * u + 2], ab[4 * u + 3]);
@@ -640,13 +650,15 @@ __device__ __forceinline__ void expand_word(uint8_t* sA, const uint8_t* sC, int 
 // both CTAs), tmem_empty[b] (even CTA; every epilogue warp of the pair arrives).
 constexpr int kStage2Bytes = 2 * 128 * BK * 2;   // 16 KB of A + 16 KB of B per CTA and stage
 constexpr int kStages2 = 4;
-constexpr int kThreads2 = 32 * (2 + kEpiWarps);
-// A quarter of an SM holds three of the ten warps, and one of a small kernel of another stream has to fit beside them: at most
-// 144 registers a thread (with 168 such a kernel waited for the end of the launch; tests/test_gpu_streams.py).
-constexpr int kRegisterBound2 = 144;
+constexpr int64_t kWideEpilogueK = 2048, kWideGeluK = 1024, kWideGeluWaves = 4;
+constexpr int threads2(int epi_warps) { return 32 * (2 + epi_warps); }
+// A quarter of an SM holds three of ten warps, or five of eighteen, and one of a small kernel of another stream has to fit
+// beside them (with 168 registers a thread, of ten warps, such a kernel waited for the end of the launch;
+// tests/test_gpu_streams.py).
+constexpr int register_bound2(int epi_warps) { return epi_warps == 8 ? 144 : 96; }
 
 struct SmemCtl2 {
-  uint64_t full[kStages2], empty[kStages2], tmem_full[2], tmem_empty[2];
+  uint64_t full[kStages2], empty[kStages2], tmem_full[2], tmem_empty[2], group[kFillBuffers];
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -710,17 +722,15 @@ __host__ __device__ constexpr uint32_t make_idesc_pair(bool a_mn, bool b_mn, uin
 }
 
 // The tensor maps of the outputs: tmO activation or input gradient, tmL pre-activation in bf16, tmZ float32 results.
-// ACT: activation of the forward pass; of the input gradient, RAD_ACT_GELU where it multiplies by GELU'(z_prev).  kFill: the
-// forward pass fills the next layer's store.
-template <int AK, int BKIND, int EPI, int ACT, bool kFill>
-__global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kRegisterBound2)
+template <int AK, int BKIND, int EPI, int kEpiWarps>
+__global__ void __cluster_dims__(2, 1, 1) __maxnreg__(register_bound2(kEpiWarps))
 tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmL,
                     const __grid_constant__ CUtensorMap tmZ) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* epi_smem = smem + (size_t)kStages2 * kStage2Bytes;
-  SmemCtl2* ctl = reinterpret_cast<SmemCtl2*>(epi_smem + kEpiWarps * kEpiBytes);
+  SmemCtl2* ctl = reinterpret_cast<SmemCtl2*>(epi_smem + kEpiBytes);
   volatile int* abort_flag = &ctl->abort_flag;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -740,6 +750,8 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       mbar_init(smem_u32(&ctl->tmem_full[b]), 1);
       mbar_init(smem_u32(&ctl->tmem_empty[b]), 2 * kEpiWarps);
     }
+    if (is_forward(EPI))             // the warps that fill one store tile together: four in a tile of 32 columns each
+      for (int g = 0; g < kFillBuffers; ++g) mbar_init(smem_u32(&ctl->group[g]), p.bn == 256 ? kEpiWarps / 8 : kEpiWarps / 4);
     ctl->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -859,7 +871,27 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
     const int c_first = ((warp - 2) >> 2) * own_chunks * 32;
     const int c_last = min(c_first + own_chunks * 32, chunks * 32);
     const uint32_t empty_bar = map_to_cta(smem_u32(&ctl->tmem_empty[0]), 0u);     // [b] is 8 bytes further
-    const uint32_t stage = smem_u32(epi_smem) + (warp - 2) * kEpiBytes, fill = stage + 4 * kChunkBytes, bias_row = fill + kFillBytes;
+    constexpr int kSlots = 32 / kEpiWarps;
+    const uint32_t stage = smem_u32(epi_smem) + (warp - 2) * kSlots * kChunkBytes;
+    const uint32_t bias_row = smem_u32(epi_smem) + kRingBytes + kFillBuffers * kFillBytes + (warp - 2) * (kBiasBytes / kEpiWarps);
+    // the warps of a lane quarter whose columns make up one store tile fill one buffer and copy it out together
+    const bool whole_tile = bn >= 128;
+    const int group = whole_tile ? 4 / own_chunks : 1, first_tile = ((warp - 2) >> 2) / group;
+    const uint32_t fill = smem_u32(epi_smem) + kRingBytes + (q + 4 * (first_tile & 1)) * kFillBytes;
+    const int group_thread = lane + 32 * (((warp - 2) >> 2) % group);
+    const uint32_t group_bar = smem_u32(&ctl->group[q + 4 * (first_tile & 1)]);
+    uint32_t group_phase = 0;
+    const auto group_sync = [&]() -> bool {             // a bounded wait like the others
+      __syncwarp();
+      if (group == 1) return true;
+      bool met = true;
+      if (lane == 0) {
+        mbar_arrive(group_bar);
+        met = mbar_wait2(group_bar, group_phase, wc);
+      }
+      group_phase ^= 1u;
+      return __shfl_sync(0xffffffffu, met ? 1 : 0, 0) != 0;
+    };
     int buf = 0, turn = 0;
     uint32_t buf_phases = 0;
     bool ok = true;
@@ -879,22 +911,23 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       const Unit w = sched.unit(u);
       const int64_t m_warp = w.m0 + 128 * (int64_t)rank + q * 32, m = m_warp + lane;
       const bool row_ok = m < sched.M;
-      const int64_t n_warp = w.n0 + c_first;
+      // (sixteen warps are more than a tile of 64 columns has chunks: the last ones have nothing to do)
+      const int64_t n_warp = c_first < c_last ? w.n0 + c_first : n_cols, n_tile = n_warp & ~(int64_t)127;
       // what the epilogue reads besides the accumulators comes while the MMAs run (a warp's columns lie in one store tile)
       StoreRow sr = {};
       uint32_t prev_bits[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu}, act_bits[4] = {};
-      if (EPI == kFwd && kFill && n_warp < n_cols) {
-        sr.load(p, m, n_warp, row_ok, own_chunks == 4);
+      if (EPI >= kFwdFill && EPI < kDx && c_first < c_last && n_tile < n_cols) {
+        sr.load(p, m, n_tile, row_ok, whole_tile);
         if (row_ok && (m & 63) == 0 && (n_warp & 127) == 0) pad_store_tile(p, m, n_warp);
       }
-      if (EPI == kFwd && p.bias != nullptr) {
+      if (is_forward(EPI) && p.bias != nullptr) {
         // four columns a lane; zero past the layer's width
         float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
         if (4 * lane < 32 * own_chunks && n_warp + 4 * lane < n_cols) b4 = *reinterpret_cast<const float4*>(p.bias + n_warp + 4 * lane);
-        st_shared16(bias_row + 16 * lane, __float_as_uint(b4.x), __float_as_uint(b4.y), __float_as_uint(b4.z), __float_as_uint(b4.w));
+        if (4 * lane < 32 * own_chunks) st_shared16(bias_row + 16 * lane, __float_as_uint(b4.x), __float_as_uint(b4.y), __float_as_uint(b4.z), __float_as_uint(b4.w));
         __syncwarp();
       }
-      if (EPI == kDx && n_warp < n_cols) {
+      if (is_dx(EPI) && n_warp < n_cols) {
         if (p.relubits_prev != nullptr) {
           const uint32_t* words = p.relubits_prev + m * ((p.N + 31) / 32) + (n_warp >> 5);
 #pragma unroll
@@ -903,7 +936,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
         }
         if (elect_one()) tma_store_wait_read<0>();      // the unit before has left the buffers
         __syncwarp();
-        if (ACT == RAD_ACT_GELU) {
+        if (EPI == kDxGelu) {
           for (int c = 0; c < own_chunks; ++c) prefetch_z(p, m_warp, n_warp + 32 * c, lane, stage + c * kChunkBytes);
           asm volatile("cp.async.commit_group;" ::: "memory");
         }
@@ -911,7 +944,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       if (lane == 0) ok = mbar_wait2(smem_u32(&ctl->tmem_full[0]) + 8u * buf, (buf_phases >> buf) & 1u, wc, 64u);
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       if (!ok) break;
-      if (EPI == kDx && ACT == RAD_ACT_GELU) {
+      if (EPI == kDxGelu) {
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
       }
@@ -927,29 +960,29 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
         if (EPI == kDwT) {
           // a chunk may reach past the tile's width (bn is a multiple of 16) and past the last kept column
           epilogue_chunk_dwt(p, r, m, n, (int)min((int64_t)min(32, bn - c0), n_cols - n), row_ok, w.split);
-        } else if (EPI == kDx) {
+        } else if (is_dx(EPI)) {
           const uint32_t bits = c == 0 ? prev_bits[0] : c == 1 ? prev_bits[1] : c == 2 ? prev_bits[2] : prev_bits[3];
-          dx_chunk<ACT == RAD_ACT_GELU>(p, &tmO, r, (int)m_warp, (int)n, lane, bits, stage + c * kChunkBytes);
+          dx_chunk<EPI == kDxGelu>(p, &tmO, r, (int)m_warp, (int)n, lane, bits, stage + c * kChunkBytes);
         } else {
           uint32_t ab[16];
-          const uint32_t bits = forward_chunk<ACT>(p, &tmO, &tmL, &tmZ, r, (int)m_warp, (int)n, lane, stage, bias_row + 128 * c, turn++, ab);
+          const uint32_t bits = forward_chunk<EPI % 3, kSlots>(p, &tmO, &tmL, &tmZ, r, (int)m_warp, (int)n, lane, stage, bias_row + 128 * c, turn++, ab);
 #pragma unroll
           for (int i = 0; i < 4; ++i)
             if (i == c) act_bits[i] = bits;
-          if (kFill) {
-            const int at = turn - 1;                   // the chunk's buffer of activations, as forward_chunk took it
-            place_kept(p, ab, sr, (int)(n >> 5) & 3, fill, stage + (p.out_zlow != nullptr ? (at & 1) * 2 : at & 3) * kChunkBytes, lane);
-          }
+          if (EPI >= kFwdFill)                         // from the chunk's buffer of activations, as forward_chunk took it
+            place_kept(p, ab, sr, (int)(n >> 5) & 3, fill, stage + chunk_slot<kSlots>(turn - 1, p.out_zlow != nullptr) * kChunkBytes, lane);
         }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_remote(empty_bar + 8u * buf);
-      if (EPI == kFwd) {
-        if (kFill && sr.staged) {
-          __syncwarp();
-          copy_kept(p, sr, fill, lane);
-          __syncwarp();
+      if (is_forward(EPI)) {
+        if (EPI >= kFwdFill && sr.staged) {              // all warps of the tile or none
+          ok = group_sync();
+          if (!ok) break;
+          copy_kept(p, sr, fill, group_thread, 32 * group);
+          ok = group_sync();
+          if (!ok) break;
         }
         if (p.relubits != nullptr && row_ok && n_warp < n_cols) {
           uint32_t* words = p.relubits + m * p.w32 + (n_warp >> 5);
@@ -1448,21 +1481,21 @@ DwPlan plan_dw(const rad_store* st, int64_t H) {
 
 struct OutMaps { CUtensorMap o, l, z; };      // see tc_gemm_pair_kernel; those of absent outputs are not read
 
-template <int AK, int BKIND, int EPI, int ACT = RAD_ACT_NONE, bool kFill = false>
+template <int AK, int BKIND, int EPI, int kEpiWarps = 8>
 int launch_pair(const TcParams& p, const CUtensorMap& ta, const CUtensorMap& tb, const OutMaps& out, int64_t max_units, cudaStream_t s) {
-  constexpr size_t smem = (size_t)kStages2 * kStage2Bytes + kEpiWarps * kEpiBytes + sizeof(SmemCtl2) + 1024;
+  constexpr size_t smem = (size_t)kStages2 * kStage2Bytes + kEpiBytes + sizeof(SmemCtl2) + 1024;
   static_assert(smem <= 227 * 1024, "stage ring too deep");
-  auto kernel = tc_gemm_pair_kernel<AK, BKIND, EPI, ACT, kFill>;
+  auto kernel = tc_gemm_pair_kernel<AK, BKIND, EPI, kEpiWarps>;
   // The kernel is persistent: the grid must not exceed the clusters that can be resident at once
   // (SM pairs that can host a cluster; fewer than half the SM count on some parts).
   static int resident_pairs = 0;
   if (resident_pairs == 0) {
     RAD_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    resident_pairs = resident_pairs_of(kernel, kThreads2, smem);
+    resident_pairs = resident_pairs_of(kernel, threads2(kEpiWarps), smem);
   }
   const int pairs = (int)std::max<int64_t>(1, std::min<int64_t>(max_units, resident_pairs));
   count_launch();
-  RAD_TRY(launch_kernel(kernel, 2 * pairs, kThreads2, smem, s, p, ta, tb, out.o, out.l, out.z));
+  RAD_TRY(launch_kernel(kernel, 2 * pairs, threads2(kEpiWarps), smem, s, p, ta, tb, out.o, out.l, out.z));
   return RAD_OK;
 }
 
@@ -1539,13 +1572,24 @@ int tc_forward(int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t 
   if (out_act != nullptr) RAD_TRY(make_out_map(&out.o, false, out_act, H, B, ld_act));
   if (out_zlow != nullptr) RAD_TRY(make_out_map(&out.l, false, out_zlow, H, B, ld_zlow));
   if (out_z != nullptr) RAD_TRY(make_out_map(&out.z, true, out_z, H, B, ld_z));
-  if (p.st_values != nullptr)
-    return act == RAD_ACT_GELU   ? launch_pair<kAK, kBMN, kFwd, RAD_ACT_GELU, true>(p, ta, tb, out, units, s)
-           : act == RAD_ACT_RELU ? launch_pair<kAK, kBMN, kFwd, RAD_ACT_RELU, true>(p, ta, tb, out, units, s)
-                                 : launch_pair<kAK, kBMN, kFwd, RAD_ACT_NONE, true>(p, ta, tb, out, units, s);
-  return act == RAD_ACT_GELU   ? launch_pair<kAK, kBMN, kFwd, RAD_ACT_GELU>(p, ta, tb, out, units, s)
-         : act == RAD_ACT_RELU ? launch_pair<kAK, kBMN, kFwd, RAD_ACT_RELU>(p, ta, tb, out, units, s)
-                               : launch_pair<kAK, kBMN, kFwd>(p, ta, tb, out, units, s);
+  const bool fill = p.st_values != nullptr;
+  const bool wide = fill ? D <= kWideEpilogueK
+                         : act == RAD_ACT_GELU && D <= kWideGeluK && (out_zlow == nullptr || units <= kWideGeluWaves * planning_pairs());
+  const auto launch = [&](auto epi) {
+    constexpr int E = decltype(epi)::value;
+    // without a store only a GELU has a form with sixteen warps
+    if constexpr (E >= kFwdFill || E == kFwd + RAD_ACT_GELU)
+      if (wide) return launch_pair<kAK, kBMN, E, 16>(p, ta, tb, out, units, s);
+    return launch_pair<kAK, kBMN, E>(p, ta, tb, out, units, s);
+  };
+  switch (act + (fill ? kFwdFill : kFwd)) {
+    case kFwd + RAD_ACT_RELU: return launch(std::integral_constant<int, kFwd + RAD_ACT_RELU>());
+    case kFwd + RAD_ACT_GELU: return launch(std::integral_constant<int, kFwd + RAD_ACT_GELU>());
+    case kFwdFill + RAD_ACT_NONE: return launch(std::integral_constant<int, kFwdFill + RAD_ACT_NONE>());
+    case kFwdFill + RAD_ACT_RELU: return launch(std::integral_constant<int, kFwdFill + RAD_ACT_RELU>());
+    case kFwdFill + RAD_ACT_GELU: return launch(std::integral_constant<int, kFwdFill + RAD_ACT_GELU>());
+    default: return launch(std::integral_constant<int, kFwd>());
+  }
 }
 
 int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, const void* W, int64_t ldw,
@@ -1566,7 +1610,7 @@ int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, 
   OutMaps out = {};
   RAD_TRY(make_out_map(&out.o, false, dZ_prev, D, B, ldp));
   const int64_t units = ceil_div(B, BM) * ceil_div(D, bn);
-  return z_prev != nullptr ? launch_pair<kAK, kBK_, kDx, RAD_ACT_GELU>(p, ta, tb, out, units, s)
+  return z_prev != nullptr ? launch_pair<kAK, kBK_, kDxGelu>(p, ta, tb, out, units, s)
                            : launch_pair<kAK, kBK_, kDx>(p, ta, tb, out, units, s);
 }
 

@@ -186,3 +186,23 @@ def test_small_net_step_equals_the_layer_calls_and_counts_its_launches(name, var
         assert fro <= 1e-5 and mx <= 1e-5, (l, fro, mx)
         dz = dzp
     assert torch.equal(loss, ctx.loss)
+
+
+@pytest.mark.parametrize("dims,B,dtype", [((32,) * 18 + (8,), 40, "f32"), ((1024, 1152, 8), 768, "f32"), ((1152, 1024, 64), 768, "bf16"),
+                                          ((384, 200, 16), 4100, "f32"), ((96, 72, 64, 64), 65, "bf16")])
+def test_indices_of_all_layers_in_one_go(dims, B, dtype):
+    """More layers than one launch takes, layers of 96 tiles (the most that one cluster makes) and more, tiles with remainders:
+    kept counts of every layer are the oracle's, and so is the gradient that is formed from the stores."""
+    import paper_2007_10412_b200 as rad
+    X, y, Ws, bs = mlp_inputs(dims, B, dtype, "normal", seed=len(dims) + B, bias_zero=False)
+    ctx = rad.MLPStep(dims, B, dtype, "relu", "different", 0.2)
+    ctx(to_dev(X, dtype), torch.from_numpy(y).cuda(), [to_dev(W, dtype) for W in Ws], [to_dev(b, "f32") for b in bs], seed=11, step=3)
+    torch.cuda.synchronize()
+    assert ctx.dev_status.item() == 0
+    ref = orc.mlp_step(X, y, Ws, bs, dtype=dtype, variant="different", p=0.2, seed=11, step=3)
+    nnz = ctx.nnz.cpu().numpy().reshape(-1, 2)
+    for l, d in enumerate(dims[:-1]):
+        assert nnz[l, 0] == orc.keep_mask("different", B, d, 0.2, 11, l, 3).sum()
+    # the last layer's gradient: no ReLU sign that a rounding could turn stands between it and the loss
+    g = ctx.dW[-1].double().cpu().numpy()
+    assert np.linalg.norm(g - ref.dW[-1]) <= (1e-5 if dtype == "f32" else 2e-2) * np.linalg.norm(ref.dW[-1])
