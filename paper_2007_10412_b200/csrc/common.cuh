@@ -333,7 +333,7 @@ int launch_replace_index(const rad_store* st, uint32_t* extras, bool check_capac
 int launch_replace_extras(const void* A, int64_t lda, const rad_store* st, const uint32_t* extras, cudaStream_t s);
 int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, const void* W,
                   int64_t ldw, const uint32_t* relubits_prev, const void* z_prev, int64_t ld_zprev,
-                  void* dZ_prev, int64_t ldp, int32_t* dev_status, cudaStream_t s);
+                  void* dZ_prev, int64_t ldp, float* db, int32_t* dev_status, cudaStream_t s);
 int tc_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, float* dW,
                    int64_t ldw, void* workspace, int64_t workspace_bytes, int32_t* dev_status,
                    cudaStream_t s);

@@ -63,6 +63,7 @@ struct TcParams {
   bf16* st_values; const uint32_t* st_keepbits; const uint32_t* st_offsets; int64_t st_capacity; int32_t st_ncb; float st_scale;
   // input-grad epilogue
   const uint32_t* relubits_prev; const bf16* z_prev; int64_t ld_zprev; bf16* out_dx; int64_t ld_dx;
+  const bf16* dz; int64_t ld_dz; float* db;    // db (optional): also the column sums of dZ
   // dW epilogue
   float* out_dw; int64_t ld_dw; int64_t dw_rows; const uint32_t* row_idx; float* partial; int64_t partial_rows;
   int32_t* dev_status;
@@ -559,6 +560,75 @@ __device__ __forceinline__ void epilogue_chunk_dwt(const TcParams& p, const uint
   }
 }
 
+// ---- bias gradient beside the input gradient ------------------------------------------------------------
+// The epilogue warps have nothing to do while the MMAs of a tile run, so they add up the columns of dZ meanwhile, a share
+// of the work per tile: a CTA takes groups of 16 columns (8 where that gives every CTA a group: 32 bytes of a row are a
+// sector), a thread 16 bytes of every (256 >> shift)-th row, eight loads in flight.  As a launch of its own this took 4 to 9
+// us behind every input gradient of a net of ordinary size, and 0.2 ms at 65536 x 8192.
+// Sums of eight rows as a tree, then one after the other, then over lanes and warps.
+struct ColumnSums {
+  float acc[8];
+  uint32_t group, step, turn;
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
+  }
+};
+constexpr int kSumThreads = 256, kSumLoads = 8;
+__device__ __forceinline__ void add_bf16x8(const uint4& q, float (&v)[8]) {
+  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    v[2 * i] += bf16_lo(w[i]);
+    v[2 * i + 1] += bf16_hi(w[i]);
+  }
+}
+// One step: kSumLoads rows a thread.
+__device__ __forceinline__ void column_sums_step(const TcParams& p, ColumnSums& cs, int shift, int thread) {
+  const int64_t col = ((int64_t)cs.group << shift) * 8 + 8 * (thread & ((1 << shift) - 1));
+  const uint32_t lanes = kSumThreads >> shift;
+  const int64_t row0 = (int64_t)cs.step * lanes * kSumLoads + (thread >> shift);
+  uint4 q[kSumLoads];
+#pragma unroll
+  for (int j = 0; j < kSumLoads; ++j) {
+    const int64_t row = row0 + (int64_t)j * lanes;
+    q[j] = make_uint4(0u, 0u, 0u, 0u);
+    if (row < p.M && col < p.K) q[j] = *reinterpret_cast<const uint4*>(p.dz + row * p.ld_dz + col);
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float v[8];
+    const uint32_t w[4] = {q[4 * h].x, q[4 * h].y, q[4 * h].z, q[4 * h].w};
+    float u[8];
+    const uint32_t x[4] = {q[4 * h + 2].x, q[4 * h + 2].y, q[4 * h + 2].z, q[4 * h + 2].w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      v[2 * i] = bf16_lo(w[i]);
+      v[2 * i + 1] = bf16_hi(w[i]);
+      u[2 * i] = bf16_lo(x[i]);
+      u[2 * i + 1] = bf16_hi(x[i]);
+    }
+    add_bf16x8(q[4 * h + 1], v);
+    add_bf16x8(q[4 * h + 3], u);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) cs.acc[i] += v[i] + u[i];
+  }
+}
+// A warp's sums of the group it has gone through, into `red` (16 columns).
+__device__ __forceinline__ void column_sums_warp(ColumnSums& cs, int shift, int lane, float* red) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    if (o < (1 << shift)) continue;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) cs.acc[i] += __shfl_xor_sync(0xffffffffu, cs.acc[i], o);
+  }
+  if (lane < (1 << shift)) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) red[8 * lane + i] = cs.acc[i];
+  }
+  cs.clear();
+}
+
 // ---- shared memory layout -------------------------------------------------------------------------
 constexpr int kIndexBytes = kTileWords * 4;   // keep bits + row offsets of one store tile (1152 B)
 constexpr int kFirstExpanderWarp = 7;        // warp 6 feeds the compressed ring
@@ -750,6 +820,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       mbar_init(smem_u32(&ctl->tmem_full[b]), 1);
       mbar_init(smem_u32(&ctl->tmem_empty[b]), 2 * kEpiWarps);
     }
+    if (is_dx(EPI)) mbar_init(smem_u32(&ctl->group[0]), kEpiWarps);       // all of them, for the bias gradient
     if (is_forward(EPI))             // the warps that fill one store tile together: four in a tile of 32 columns each
       for (int g = 0; g < kFillBuffers; ++g) mbar_init(smem_u32(&ctl->group[g]), p.bn == 256 ? kEpiWarps / 8 : kEpiWarps / 4);
     ctl->abort_flag = 0;
@@ -895,11 +966,25 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
     int buf = 0, turn = 0;
     uint32_t buf_phases = 0;
     bool ok = true;
+    // bias gradient: this CTA's column groups are blockIdx.x, blockIdx.x + gridDim.x, ...; `quota` steps per tile
+    ColumnSums cs;
+    cs.clear();
+    cs.group = blockIdx.x; cs.step = 0; cs.turn = 0;
+    const int et = tid - 64;                           // 0 .. 32 kEpiWarps - 1
+    const int sum_shift = p.K > 8 * (int64_t)gridDim.x ? 1 : 0;
+    uint32_t sum_groups = 0, sum_steps = 0, quota = 0;
+    if (is_dx(EPI) && p.db != nullptr) {
+      const uint32_t rows = (kSumThreads >> sum_shift) * kSumLoads, cols = 8u << sum_shift;
+      sum_groups = ((uint32_t)p.K + cols - 1) / cols;
+      sum_steps = ((uint32_t)p.M + rows - 1) / rows;
+      const uint32_t own_groups = cs.group < sum_groups ? (sum_groups - cs.group + gridDim.x - 1) / gridDim.x : 0;
+      const uint32_t own_units = (sched.units - pair + npairs - 1) / npairs;
+      quota = (own_groups * sum_steps + own_units - 1) / own_units;
+    }
     if (EPI == kDwT && p.keep_cols != nullptr) {
       // Rows of dW whose column was not kept are zero (Sec. 4.3: only the sampled part of the weight matrix
       // gets a gradient).  The epilogue warps have nothing to do until the first tile's MMAs retire, so they
       // write those rows now: row d belongs to CTA d mod grid, a thread writes 16 bytes at a time.
-      const int et = tid - 64;                       // 0 .. 32 kEpiWarps - 1
       const int64_t h4 = p.M / 4;
       for (int64_t d = blockIdx.x; d < p.dw_rows; d += gridDim.x) {
         if ((p.keep_cols[d >> 5] >> (d & 31)) & 1u) continue;
@@ -940,6 +1025,32 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
           for (int c = 0; c < own_chunks; ++c) prefetch_z(p, m_warp, n_warp + 32 * c, lane, stage + c * kChunkBytes);
           asm volatile("cp.async.commit_group;" ::: "memory");
         }
+      }
+      if (is_dx(EPI) && p.db != nullptr) {
+        for (uint32_t k = 0; k < quota && cs.group < sum_groups && ok; ++k) {
+          column_sums_step(p, cs, sum_shift, et);
+          if (++cs.step < sum_steps) continue;
+          // the group is through: two buffers, so that one meeting of the warps per group is enough
+          float* red = reinterpret_cast<float*>(epi_smem + kRingBytes) + (cs.turn & 1) * kEpiWarps * 16;
+          column_sums_warp(cs, sum_shift, lane, red + (warp - 2) * 16);
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive(smem_u32(&ctl->group[0]));
+            ok = mbar_wait2(smem_u32(&ctl->group[0]), cs.turn & 1, wc);
+          }
+          ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+          const int64_t col = ((int64_t)cs.group << sum_shift) * 8 + et;
+          if (ok && et < (8 << sum_shift) && col < p.K) {
+            float t = 0.0f;
+#pragma unroll
+            for (int i = 0; i < kEpiWarps; ++i) t += red[i * 16 + et];
+            p.db[col] = t;
+          }
+          cs.group += gridDim.x;
+          cs.step = 0;
+          ++cs.turn;
+        }
+        if (!ok) break;
       }
       if (lane == 0) ok = mbar_wait2(smem_u32(&ctl->tmem_full[0]) + 8u * buf, (buf_phases >> buf) & 1u, wc, 64u);
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
@@ -1594,7 +1705,7 @@ int tc_forward(int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t 
 
 int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, const void* W, int64_t ldw,
                   const uint32_t* relubits_prev, const void* z_prev, int64_t ld_zprev, void* dZ_prev, int64_t ldp,
-                  int32_t* dev_status, cudaStream_t s) {
+                  float* db, int32_t* dev_status, cudaStream_t s) {
   CUtensorMap ta, tb;
   int rc = make_map(&ta, dZ, H, B, ldz, 128);         // K-major A (K = H)
   if (rc != RAD_OK) return rc;
@@ -1605,6 +1716,7 @@ int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, 
   p.M = B; p.N = D; p.K = H; p.splits = 1; p.num_stages = 3; p.bn = bn;
   p.relubits_prev = relubits_prev; p.z_prev = static_cast<const bf16*>(z_prev); p.ld_zprev = ld_zprev;
   p.out_dx = static_cast<bf16*>(dZ_prev); p.ld_dx = ldp;
+  p.dz = static_cast<const bf16*>(dZ); p.ld_dz = ldz; p.db = db;
   p.dev_status = dev_status;
   p.wait_limit_ns = wait_limit_ns();
   OutMaps out = {};

@@ -376,3 +376,28 @@ def test_outputs_in_chunks_and_the_store_beside_them(B, D, H, p, shift):
     want = A.double() @ W.double() + b.double()
     mag = A.double().abs() @ W.double().abs() + b.double().abs()
     assert ((z2.double() - want).abs() <= (D ** 0.5 + 16) * 2.0 ** -24 * mag).all()      # float32 sums in any order
+
+
+@pytest.mark.parametrize("B,D,H,ld", [(64, 64, 64, 64), (130, 72, 200, 208), (2049, 128, 1184, 1184), (2100, 64, 1192, 1192),
+                                      (20000, 1096, 264, 264), (1024, 64, 4744, 4744)])
+@pytest.mark.parametrize("act", ["relu", "gelu"])
+def test_bias_gradient_beside_the_input_gradient(B, D, H, ld, act):
+    """Column sums made by the input gradient's launch: one group of 8 or 16 columns per CTA and several, rows that end inside a
+    step, several tiles per SM pair; the input gradient is the same with and without them.  Bound: eight rows as a tree, then
+    at most B / 1024 + 1 steps, lanes and warps, each a float32 rounding of the sum of magnitudes."""
+    import paper_2007_10412_b200 as rad
+    bf = torch.bfloat16
+    g = torch.Generator(device="cuda").manual_seed(B + H)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").to(bf)
+    dZ, W = rnd(B, ld)[:, :H], rnd(D, H)
+    z = rnd(B, D) if act == "gelu" else None
+    bits = torch.randint(-2 ** 31, 2 ** 31, (B * ((D + 31) // 32),), generator=g, device="cuda", dtype=torch.int64).to(torch.int32)
+    kw = dict(z_prev=z, relubits_prev=None if act == "gelu" else bits)
+    db, dX, dX2 = torch.full((H,), float("nan"), device="cuda"), torch.empty(B, D, dtype=bf, device="cuda"), torch.empty(B, D, dtype=bf, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rad.rad_linear_input_grad(dZ, W, dZ_prev=dX, db=db, dev_status=status, **kw)
+    rad.rad_linear_input_grad(dZ, W, dZ_prev=dX2, **kw)
+    torch.cuda.synchronize()
+    assert status.item() == 0 and torch.equal(dX, dX2)
+    x = dZ.double()
+    assert ((db.double() - x.sum(0)).abs() <= (3 + 2 * (B / 1024 + 1) + 5 + 8) * 2.0 ** -24 * x.abs().sum(0)).all()
