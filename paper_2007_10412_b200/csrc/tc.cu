@@ -13,7 +13,7 @@
 //                    them; each CTA keeps two alternating 128 x 256 float32
 //                    accumulators in tensor memory, so the epilogue of a tile (bias, activation,
 //                    ReLU bits, GELU', stores) runs under the MMAs of the next one.
-//   sparse-A kernel  256 x 512 tile per pair; sixteen "expander" warps per CTA write the A_hat
+//   sparse-A kernel  256 x 512 tile per pair (256 or 128 columns where 512 would leave SMs idle); sixteen "expander" warps per CTA write the A_hat
 //                    tile of each K block into shared memory instead of TMA.
 // Long dW contractions can be split along K; partial tiles are summed in split order by a second
 // kernel, so results are reproducible.
@@ -1135,11 +1135,10 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
 // Roles per CTA: 0 dZ producer, 1 MMA issuer (even CTA) and tensor-memory owner, 2-5 epilogue,
 // 6 producer of the compressed ring, 7-22 expanders (two groups on alternate K blocks).  full[s] lives in the even CTA: one arrival
 // with the dZ bytes of both CTAs plus one per expander warp of either CTA.
-constexpr int kSpBM = 256, kSpBN = 512;
+constexpr int kSpBM = 256, kSpBN = 512;      // widest tile: see plan_dw
 constexpr int kSpAStageBytes = 128 * BK * 2;           // 16 KB: this CTA's 128 columns of A_hat
-constexpr int kSpBStageBytes = 256 * BK * 2;           // 32 KB: this CTA's 2 x 128 columns of dZ
-constexpr int kSpStageBytes = kSpAStageBytes + kSpBStageBytes;
-constexpr int kSpMaxStages = 4;
+constexpr int sparse_stage_bytes(int bn) { return kSpAStageBytes + bn / 2 * BK * 2; }    // and this CTA's bn / 2 columns of dZ
+constexpr int kSpMaxStages = 6;
 constexpr int kSpExpanderWarps = 8;                    // per K block: one thread per keep-bit word of the store tile
 constexpr int kSpExpanderGroups = 2;                   // groups of eight warps take alternate K blocks
 constexpr int kSpEpiShare = 1 + kSpExpanderWarps * kSpExpanderGroups / 4;   // warps of a lane quarter that share the epilogue
@@ -1155,9 +1154,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSpThreads, 1)
 tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  const int stages = p.num_stages;
+  const int stages = p.num_stages, bn = p.bn;       // tile of 512 columns (two MMAs per 16 rows of K), 256 or 128
+  const int stage_bytes = kSpAStageBytes + bn / 2 * BK * 2;
   const int comp_slot = kIndexBytes + p.comp_cap;               // index data + values of this CTA's store tile of one K block
-  uint8_t* comp_base = smem + (size_t)stages * kSpStageBytes;
+  uint8_t* comp_base = smem + (size_t)stages * stage_bytes;
   SmemCtlSp* ctl = reinterpret_cast<SmemCtlSp*>(comp_base + (size_t)p.comp_depth * comp_slot);
   volatile int* abort_flag = &ctl->abort_flag;
 
@@ -1165,7 +1165,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
   const uint32_t rank = cluster_ctarank();
   const uint32_t peer_abort = map_to_cta(smem_u32(&ctl->abort_flag), rank ^ 1u);
   const PairWait wc = {abort_flag, peer_abort, p.wait_limit_ns};
-  const Schedule sched(p.M, p.N, p.K, p.splits, kSpBM, kSpBN);
+  const Schedule sched(p.M, p.N, p.K, p.splits, kSpBM, bn);
   const uint32_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   if (tid == 0) {
     prefetch_map(&tmB);
@@ -1206,7 +1206,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
     tc_fence_after();
     const int64_t m0 = w.m0 + 128 * (int64_t)rank + q * 32;
 #pragma unroll 1
-    for (int c0 = first * 32; c0 < kSpBN; c0 += kSpEpiShare * 32) {
+    for (int c0 = first * 32; c0 < bn; c0 += kSpEpiShare * 32) {
       const int64_t n = w.n0 + c0;
       if (n >= p.N) break;                  // warp-uniform
       epilogue_dw(p, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, m0, n, w.split, lane);
@@ -1227,15 +1227,15 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
       for (uint32_t u = pair; u < sched.units && ok; u += npairs) {
         const Unit w = sched.unit(u);
         if (u + npairs >= sched.units) let_next_start();
-        const int n_own = (int)w.n0 + 128 * (int)rank;       // + 256 for the second half
+        const int n_own = (int)w.n0 + min(bn, 256) / 2 * (int)rank;       // + 256 for the second half
         for (int kb = w.kb0; kb < w.kb1; ++kb) {
           ok = mbar_wait2(smem_u32(&ctl->empty[0]) + 8u * stage, phase ^ 1u, wc);
           if (!ok) break;
-          const uint32_t sB = smem_base + stage * kSpStageBytes + kSpAStageBytes;
-          if (rank == 0) mbar_arrive_expect_tx(smem_u32(&ctl->full[0]) + 8u * stage, 2 * kSpBStageBytes);   // both CTAs' bytes
+          const uint32_t sB = smem_base + stage * stage_bytes + kSpAStageBytes;
+          if (rank == 0) mbar_arrive_expect_tx(smem_u32(&ctl->full[0]) + 8u * stage, (uint32_t)bn * BK * 2);   // both CTAs' bytes
 #pragma unroll
           for (int c = 0; c < 4; ++c)
-            tma_load_2d_pair(sB + c * 8192, &tmB, n_own + (c >> 1) * 256 + (c & 1) * 64, kb * BK, full0 + 8u * stage);
+            if (c * 128 < bn) tma_load_2d_pair(sB + c * 8192, &tmB, n_own + (c >> 1) * 256 + (c & 1) * 64, kb * BK, full0 + 8u * stage);
           if (++stage == stages) { stage = 0; phase ^= 1u; }
         }
       }
@@ -1249,7 +1249,8 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
   } else if (warp == 1) {
     // ===== MMA issuer (even CTA) =====
     if (rank == 0 && elect_one()) {
-      constexpr uint32_t idesc = make_idesc_pair(true, true);
+      const uint32_t idesc = make_idesc_pair(true, true, (uint32_t)min(bn, 256));
+      const bool halves = bn > 256;
       const uint64_t adesc0 = make_desc(smem_base, 8192, 1024), bdesc0 = make_desc(smem_base + kSpAStageBytes, 8192, 1024);
       int stage = 0;
       uint32_t phase = 0, unit_phase = 0;
@@ -1263,14 +1264,15 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
           ok = mbar_wait2(smem_u32(&ctl->full[0]) + 8u * stage, phase, wc);
           if (!ok) break;
           tc_fence_after();
-          const uint64_t adesc = adesc0 + (uint32_t)(stage * (kSpStageBytes >> 4));
-          const uint64_t bdesc = bdesc0 + (uint32_t)(stage * (kSpStageBytes >> 4));
+          const uint64_t adesc = adesc0 + (uint32_t)(stage * (stage_bytes >> 4));
+          const uint64_t bdesc = bdesc0 + (uint32_t)(stage * (stage_bytes >> 4));
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
 #pragma unroll
             for (int j = 0; j < 2; ++j)
-              tc_mma_pair(tmem_base + j * 256, adesc + k * (2048 >> 4), bdesc + (j * 16384 + k * 2048) / 16, idesc,
-                          (kb > w.kb0 || k > 0) ? 1u : 0u);
+              if (j == 0 || halves)
+                tc_mma_pair(tmem_base + j * 256, adesc + k * (2048 >> 4), bdesc + (j * 16384 + k * 2048) / 16, idesc,
+                            (kb > w.kb0 || k > 0) ? 1u : 0u);
           tc_commit_pair(smem_u32(&ctl->empty[0]) + 8u * stage);
           if (++stage == stages) { stage = 0; phase ^= 1u; }
         }
@@ -1361,7 +1363,7 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
           if (!ok) break;
           // columns past the layer's width keep whatever the buffer held: their accumulator rows are never written
           if (have) {
-            uint8_t* sA = smem + (size_t)stage * kSpStageBytes;
+            uint8_t* sA = smem + (size_t)stage * stage_bytes;
             const uint8_t* sC = comp_base + (size_t)slot * comp_slot;
             expand_word(sA, sC, 0, r, wq, (uint32_t)p.comp_cap >> 1);
             fence_proxy_async();
@@ -1494,7 +1496,7 @@ int num_sms() {
   return n;
 }
 
-// K splits for a dW contraction.  Cost model in units of one CTA working through one K block
+// K splits of a same-sample dW.  Cost model in units of one CTA working through one K block
 // (about 1024 tensor-pipe clocks): waves x K blocks per unit, plus what writing and re-reading the
 // float32 partial tiles costs at HBM speed.  Pure function of the shapes, so the workspace query
 // and the launch agree.
@@ -1513,7 +1515,31 @@ int choose_splits(int64_t m_tiles, int64_t n_tiles, int64_t kblocks, int64_t bm 
   return best;
 }
 
-struct DwPlan { int splits; int64_t partial_rows; int64_t bytes; int comp_cap; int stages; int comp_depth; };
+// Tile width and K splits of a different-sample dW of D x H from B rows.  What bounds it: a K block costs its expansion, 0.58 us
+// whatever the width (0.84 at half the entries), up to 512 columns, whose MMAs and loads take 0.6; the epilogue 1.2 us per 128
+// columns (a SM stores 50 bytes per ns); a launch its start and end; partial tiles a second launch and their bytes.  So a
+// wide tile where the units fill the chip, a narrow one where they do not (us, wide / chosen: 328 x 640 x 520 13.5 / 9.4,
+// 1024 x 512 x 512 14.0 / 11.0, 1024 x 2048 x 2048 20.1 / 17.9, 2048 x 1024 x 4096 29.9 / 27.3; kept at 512: 4096 x 2048 x 2048
+// 40.6 against 46.0 at 256).  A pure function of the shapes, so that the workspace query and the launch agree.
+struct SparseTile { int bn, splits; };
+SparseTile choose_sparse_tile(int64_t B, int64_t D, int64_t H, double keep, int64_t pairs) {
+  const int64_t kblocks = ceil_div(B, BK), m_tiles = ceil_div(D, kSpBM);
+  const double out_us = (double)(m_tiles * kSpBM) * (double)H * 4.0 / 7.5e6;
+  SparseTile best = {kSpBN, 1};
+  double best_cost = 1e300;
+  for (int bn = kSpBN; bn >= 128; bn /= 2) {
+    const double kblock_us = (bn == kSpBN ? 0.62 : 0.58) + 0.65 * std::max(0.0, keep - 0.1), epilogue_us = bn / 128 * 1.25;
+    for (int s = 1; s <= kMaxSplits && s <= kblocks; ++s) {
+      const double waves = (double)ceil_div(m_tiles * ceil_div(H, bn) * s, pairs);
+      const double beyond_l2 = out_us * s > 14.0 ? 2.0 : 1.0;         // 100 MB: partial tiles go through memory
+      const double cost = waves * ((double)ceil_div(kblocks, s) * kblock_us + epilogue_us) + (s > 1 ? 2.5 + out_us * (s + 1) * beyond_l2 : 0.0);
+      if (cost < best_cost - 1e-9) { best_cost = cost; best = {bn, s}; }
+    }
+  }
+  return best;
+}
+
+struct DwPlan { int bn; int splits; int64_t partial_rows; int64_t bytes; int comp_cap; int stages; int comp_depth; };
 
 // Clusters of two CTAs of `kernel` that can be resident at once.
 template <typename K>
@@ -1579,12 +1605,15 @@ DwPlan plan_dw(const rad_store* st, int64_t H) {
     int64_t cap = (int64_t)(n * pe + 8.0 * std::sqrt(n * pe * (1.0 - pe)) + 16.0);
     cap = std::min<int64_t>(round_up(cap, 8), (int64_t)n) * 2;
     d.comp_cap = (int)round_up(cap, 128);
-    // shared memory: 48 KB per A/B stage plus a ring of compressed slots
+    const SparseTile tile = choose_sparse_tile(st->B, st->D, H, pe, planning_pairs());
+    d.bn = tile.bn;
+    d.splits = tile.splits;
+    // shared memory: the A/B stages (48 KB for a tile of 512 columns) plus a ring of compressed slots
     const int64_t budget = 227 * 1024 - 2048 - (int64_t)sizeof(SmemCtlSp);
-    const int64_t slot = kIndexBytes + d.comp_cap;
-    d.stages = (4 * kSpStageBytes + 3 * slot <= budget) ? 4 : (3 * kSpStageBytes + 2 * slot <= budget) ? 3 : 2;
-    d.comp_depth = (int)std::max<int64_t>(2, std::min<int64_t>(8, (budget - d.stages * kSpStageBytes) / slot));
-    d.splits = choose_splits(ceil_div(m_expect, kSpBM), ceil_div(H, kSpBN), kblocks, kSpBM, planning_pairs(), kSpBN);
+    const int64_t slot = kIndexBytes + d.comp_cap, stage = sparse_stage_bytes(d.bn);
+    d.stages = kSpMaxStages;
+    while (d.stages > 2 && d.stages * stage + (d.stages > 3 ? 3 : 2) * slot > budget) --d.stages;
+    d.comp_depth = (int)std::max<int64_t>(2, std::min<int64_t>(8, (budget - d.stages * stage) / slot));
     d.bytes = d.splits > 1 ? (int64_t)d.splits * d.partial_rows * H * 4 : 0;
     return d;
   }
@@ -1611,7 +1640,7 @@ int launch_pair(const TcParams& p, const CUtensorMap& ta, const CUtensorMap& tb,
 }
 
 int launch_sparse_pair(const TcParams& p, const CUtensorMap& tb, int64_t max_units, cudaStream_t s) {
-  const size_t smem = (size_t)p.num_stages * kSpStageBytes + (size_t)p.comp_depth * (kIndexBytes + p.comp_cap) +
+  const size_t smem = (size_t)p.num_stages * sparse_stage_bytes(p.bn) + (size_t)p.comp_depth * (kIndexBytes + p.comp_cap) +
                       sizeof(SmemCtlSp) + 1024;
   if (smem > 227 * 1024 || p.num_stages > kSpMaxStages || p.comp_depth > 8) return RAD_EUNSUPPORTED;
   static int resident_pairs = 0;
@@ -1742,7 +1771,7 @@ int tc_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, 
   int rc = make_map(&tb, dZ, H, st->B, ldz, 64);      // MN-major B: box 64 (N = h) x 64 K rows (b)
   if (rc != RAD_OK) return rc;
   TcParams p = {};
-  p.N = H; p.K = st->B; p.splits = d.splits; p.num_stages = d.stages; p.comp_depth = d.comp_depth;
+  p.N = H; p.K = st->B; p.splits = d.splits; p.bn = d.bn; p.num_stages = d.stages; p.comp_depth = d.comp_depth;
   p.out_dw = dW; p.ld_dw = ldw; p.dw_rows = st->D; p.partial = static_cast<float*>(workspace); p.partial_rows = d.partial_rows;
   p.dev_status = dev_status;
   p.wait_limit_ns = wait_limit_ns();
@@ -1761,7 +1790,7 @@ int tc_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, 
     p.M = st->D;
     p.values = static_cast<const bf16*>(st->values); p.keepbits = st->keepbits; p.offsets = st->offsets;
     p.values_capacity = st->values_capacity; p.ncb = (int32_t)ceil_div(st->D, kTileCols); p.comp_cap = d.comp_cap;
-    rc = launch_sparse_pair(p, tb, ceil_div(st->D, kSpBM) * ceil_div(H, kSpBN) * d.splits, s);
+    rc = launch_sparse_pair(p, tb, ceil_div(st->D, kSpBM) * ceil_div(H, d.bn) * d.splits, s);
   }
   if (rc != RAD_OK) return rc;
   if (d.splits > 1) {

@@ -401,3 +401,25 @@ def test_bias_gradient_beside_the_input_gradient(B, D, H, ld, act):
     assert status.item() == 0 and torch.equal(dX, dX2)
     x = dZ.double()
     assert ((db.double() - x.sum(0)).abs() <= (3 + 2 * (B / 1024 + 1) + 5 + 8) * 2.0 ** -24 * x.abs().sum(0)).all()
+
+
+@pytest.mark.parametrize("B,D,H", [(64, 64, 64), (328, 264, 136), (1000, 520, 264), (4160, 256, 264), (1024, 2048, 2040), (70, 1032, 520)])
+@pytest.mark.parametrize("p", [0.1, 0.7])
+def test_different_sample_dw_over_tile_widths(B, D, H, p):
+    """dW from a different-sample store in tiles of 128, 256 and 512 columns, with and without K splits, with rows and columns
+    that end inside a tile.  Against float64: the sum of B products in any order."""
+    import paper_2007_10412_b200 as rad
+    bf = torch.bfloat16
+    g = torch.Generator(device="cuda").manual_seed(B + D + H)
+    A, dZ = (torch.randn(B, n, generator=g, device="cuda").to(bf) for n in (D, H))
+    st = rad.Store("different", "bf16", B, D, p, seed=5, layer=1, step=2, relu_bits=False)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rad.rad_linear_forward_store(A, st, status)
+    dW = torch.full((D, H), float("nan"), device="cuda")
+    rad.rad_linear_weight_grad(st, dZ, dW, dev_status=status)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    keep = torch.from_numpy(orc.keep_mask("different", B, D, p, 5, 1, 2)).cuda()
+    kept = torch.where(keep, (A.float() * rad.rad_scale(p)).to(bf), torch.zeros((), dtype=bf, device="cuda")).double()
+    mag = kept.abs().T @ dZ.double().abs()
+    assert ((dW.double() - kept.T @ dZ.double()).abs() <= (B ** 0.5 + 16) * 2.0 ** -24 * mag).all()
