@@ -31,6 +31,7 @@ namespace {
 
 constexpr int kCvM = 128, kCvN = 64, kCvK = 64;
 constexpr int kCvThreads = 256;
+constexpr int kCvPerSm = 4;                      // CTAs that fit an SM: shared memory, 64 registers a thread, 256 tensor-memory columns
 constexpr int kCvABytes = kCvM * kCvK * 2;       // 16 KB either way round
 constexpr int kCvBBytes = kCvK * kCvN * 2;       // 8 KB
 constexpr int kCvStageBytes = kCvABytes + kCvBBytes;
@@ -135,7 +136,7 @@ __device__ __forceinline__ uint4 cv_load_pixel(const bf16* T, bool in, int y, in
 // 210 -> 58, input gradient 339 -> 175 / 165 -> 78.
 enum { kCvFwd = 0, kCvDw = 1, kCvDx = 2 };
 template <int kMode>
-__global__ void __launch_bounds__(kCvThreads, 3) conv_tc_kernel(const ConvTcParams p) {
+__global__ void __launch_bounds__(kCvThreads, kCvPerSm) conv_tc_kernel(const ConvTcParams p) {
   wait_for_previous();
   constexpr bool kDw = kMode == kCvDw, kDx = kMode == kCvDx;
   extern __shared__ uint8_t cv_raw[];
@@ -456,10 +457,10 @@ int conv_tc_input_grad(int64_t B, int H, int W, int Cin, int Cout, const void* d
   return RAD_OK;
 }
 
-// K blocks of 64 pixels per CTA of the filter-gradient kernel, and the splits that follow from it: enough for three
+// K blocks of 64 pixels per CTA of the filter-gradient kernel, and the splits that follow from it: enough for four
 // CTAs on every SM (a K block is a chain of latencies, so CTAs side by side are what hides them), at least four each.
 static int conv_tc_splits(int64_t npix, int Cin, int* kblocks_per_split) {
-  const int64_t kblocks = ceil_div(npix, kCvK), want = std::max<int64_t>(1, 3 * 148 / ceil_div(9 * Cin, kCvM));
+  const int64_t kblocks = ceil_div(npix, kCvK), want = std::max<int64_t>(1, kCvPerSm * 148 / ceil_div(9 * Cin, kCvM));
   const int64_t per = std::max<int64_t>(4, ceil_div(kblocks, want));
   *kblocks_per_split = (int)per;
   return (int)ceil_div(kblocks, per);
