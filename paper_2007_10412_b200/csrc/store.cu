@@ -466,20 +466,33 @@ __global__ void __launch_bounds__(256) same_gather_rows_kernel(const SameParams 
   }
 }
 
-// relubits[b, w] = bits of (A[b, 32w .. 32w+31] > 0).  One thread per output word.
+// relubits[b, w] = bits of (A[b, 32w .. 32w+31] > 0).  A warp makes eight words at a time, a lane one column of each: the
+// loads of a word are one line and all eight are in flight together.  (With a thread per word its 32 loads followed one
+// another through 32 lines per warp: 5.0 us for 150 x 300 float32.)
 template <typename T>
 __global__ void __launch_bounds__(256) relu_bits_kernel(const T* A, int64_t lda, int64_t B, int64_t D,
                                                         int64_t w32, uint32_t* out) {
   begin_after_previous();
+  constexpr int kWords = 8;
   const int64_t n = B * w32;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = i / w32, w = i % w32;
-    const T* rowp = A + b * lda + w * 32;
-    const int nv = (int)min((int64_t)32, D - w * 32);
-    uint32_t m = 0;
-    for (int c = 0; c < nv; ++c) m |= (to_float(rowp[c]) > 0.0f ? 1u : 0u) << c;
-    out[i] = m;
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t i0 = warp * kWords; i0 < n; i0 += warps * kWords) {
+    int64_t b = i0 / w32, w = i0 - b * w32;
+    bool pos[kWords];
+#pragma unroll
+    for (int j = 0; j < kWords; ++j) {
+      const int64_t c = w * 32 + lane;
+      pos[j] = b < B && c < D && to_float(A[b * lda + c]) > 0.0f;
+      if (++w == w32) { w = 0; ++b; }
+    }
+    uint32_t mine = 0;
+#pragma unroll
+    for (int j = 0; j < kWords; ++j) {
+      const uint32_t m = __ballot_sync(0xffffffffu, pos[j]);
+      if (lane == j) mine = m;
+    }
+    if (lane < kWords && i0 + lane < n) out[i0 + lane] = mine;
   }
 }
 
@@ -729,7 +742,7 @@ int launch_wait_probe_lookback(uint64_t limit_ns, int32_t* dev_status, cudaStrea
 }
 int launch_relu_bits(int dtype, const void* A, int64_t lda, int64_t B, int64_t D, uint32_t* relubits, cudaStream_t s) {
   const int64_t w32 = ceil_div(D, 32), n = B * w32;
-  const int g2 = (int)std::min<int64_t>(ceil_div(n, 256), 148 * 16);
+  const int g2 = (int)std::min<int64_t>(ceil_div(n, 64), 148 * 8);        // eight warps of eight words
   count_launch();
   if (dtype == RAD_BF16)
     RAD_TRY(launch_kernel(relu_bits_kernel<bf16>, g2, 256, 0, s, static_cast<const bf16*>(A), lda, B, D, w32, relubits));
@@ -1053,7 +1066,7 @@ extern "C" int rad_linear_forward_store(const void* A, int64_t lda, const rad_st
     RAD_TRY(launch_kernel(same_gather_kernel<float>, grid, 256, 0, s, p, colscale));
   if (st->relubits != nullptr) {
     const int64_t n = st->B * w32;
-    const int g2 = (int)std::min<int64_t>(ceil_div(n, 256), 148 * 16);
+    const int g2 = (int)std::min<int64_t>(ceil_div(n, 64), 148 * 8);        // eight warps of eight words
     count_launch();
     if (st->dtype == RAD_BF16)
       RAD_TRY(launch_kernel(relu_bits_kernel<bf16>, g2, 256, 0, s, static_cast<const bf16*>(A), lda, st->B, st->D, w32, st->relubits));
