@@ -12,7 +12,8 @@
 //   dense kernels    256 x 256 tile per pair, or 128 or 64 columns wide where that makes one wave of
 //                    them; each CTA keeps two alternating 128 x 256 float32
 //                    accumulators in tensor memory, so the epilogue of a tile (bias, activation,
-//                    ReLU bits, GELU', stores) runs under the MMAs of the next one.
+//                    ReLU bits, GELU', TMA stores) runs under the MMAs of the next one.  The input
+//                    gradient's epilogue warps make the bias gradient while they wait.
 //   sparse-A kernel  256 x 512 tile per pair (256 or 128 columns where 512 would leave SMs idle); sixteen "expander" warps per CTA write the A_hat
 //                    tile of each K block into shared memory instead of TMA.
 // Long dW contractions can be split along K; partial tiles are summed in split order by a second
@@ -720,6 +721,11 @@ __device__ __forceinline__ void expand_word(uint8_t* sA, const uint8_t* sC, int 
 // both CTAs), tmem_empty[b] (even CTA; every epilogue warp of the pair arrives).
 constexpr int kStage2Bytes = 2 * 128 * BK * 2;   // 16 KB of A + 16 KB of B per CTA and stage
 constexpr int kStages2 = 4;
+// Epilogue warps, eight or sixteen.  Sixteen for a forward pass of up to kWideEpilogueK inputs that places the next layer's store
+// and for a GELU of up to kWideGeluK inputs: more warps hide the latencies of erff and of the stores (a tile of 256 x 256 in us,
+// eight / sixteen: GELU 7.3 / 6.3, with pre-activations and store 10.3 / 9.9, ReLU with store 5.7 / 5.7); with more inputs the
+// MMAs of a tile outlast the epilogue of the one before, and where a GELU without a store also writes the pre-activations of
+// many tiles eight were faster (16384 x 512 x 4096 186 / 196).
 constexpr int64_t kWideEpilogueK = 2048, kWideGeluK = 1024, kWideGeluWaves = 4;
 constexpr int threads2(int epi_warps) { return 32 * (2 + epi_warps); }
 // A quarter of an SM holds three of ten warps, or five of eighteen, and one of a small kernel of another stream has to fit
@@ -1655,10 +1661,11 @@ int launch_sparse_pair(const TcParams& p, const CUtensorMap& tb, int64_t max_uni
 }
 
 // Columns of an output tile of the forward pass and the input gradient: the narrowest of 64, 128 and 256 with which
-// the tiles are still one wave of SM pairs, else 256.  An MMA takes the same time at every width, so within a wave a
-// narrower tile only spreads loads and epilogues over more SMs (2048 x 1024 x 1024 forward with store: 21.8 / 16.9 /
-// 22.0 us at 256 / 128 / 64, which are 32 / 64 / 128 tiles on 74 pairs; 328 x 640 x 520: 18.1 / 16.3 / 12.8), and a
-// second wave costs the whole contraction again (4096 x 1024 x 1024: 22.2 / 25.0 / 36.1).
+// the tiles are still one wave of SM pairs, else 256.  Per K block an MMA of 256 columns takes 0.27 us, one of 64 or 128 with
+// its loads 0.17 to 0.2: within a wave a narrower tile is no slower there and spreads loads and epilogues over more SMs
+// (2048 x 1024 x 1024 forward with store: 21.8 / 16.9 / 22.0 us at 256 / 128 / 64 columns, which are 32 / 64 / 128 tiles on
+// 74 pairs), a second wave costs most of the contraction again (4096 x 1024 x 1024: 22.2 / 25.0 / 36.1; both before the
+// single-thread roles were elected).
 int dense_tile_width(int64_t M, int64_t N) {
   for (int bn = 64; bn < BN; bn *= 2)
     if (ceil_div(M, BM) * ceil_div(N, bn) <= planning_pairs()) return bn;
