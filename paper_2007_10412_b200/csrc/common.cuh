@@ -354,22 +354,6 @@ __device__ __forceinline__ void fma2(f32x2& acc, f32x2 a, f32x2 b) {
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
 
-__device__ __forceinline__ f32x2 fma2_of(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 v;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
-  return v;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 v;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
-  return v;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 v;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
-  return v;
-}
-
 // ---- clusters of CTAs ----------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t cluster_nctas() {
   uint32_t n;

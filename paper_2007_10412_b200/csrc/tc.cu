@@ -219,49 +219,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
-// Phi(z) (the normal distribution function) and exp(-z^2 / 2) of two numbers at once: upper tail Q(a) = R(a) exp(-a^2 / 2)
-// at a = |z|, R a polynomial in u = a / (a + 4.5) (the form of Hastings' approximations, Abramowitz and Stegun 7.1.26, with
-// coefficients of our own: least squares on [0, 14.5], weights raised where the error is largest until it is level), 4e-9
-// off near 0.  As close to the 64-bit value as 0.5 (1 + erff(z / sqrt 2)) for positive z and closer for negative z (z Phi(z):
-// relative error below 7e-6 down to z = -9, where the erff form is off by 5e-4 at -4 and has nothing left at -6).  erff and
-// __expf, two branches and about 60 instructions an element, held a 128 x 256 tile for 8 us under a GELU derivative.  (The
-// forward pass keeps erff: its results are what the loss is made of, and they stay bit for bit.)
-__device__ __forceinline__ void normal_cdf2(float z0, float z1, f32x2& cdf, f32x2& bell) {
-  const float a0 = fminf(fabsf(z0), 32.0f), a1 = fminf(fabsf(z1), 32.0f);
-  const f32x2 a = pack2(a0, a1);
-  float d0, d1, r0, r1;
-  unpack2(add2(a, pack2(4.5f, 4.5f)), d0, d1);
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(d0));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(d1));
-  const f32x2 u = mul2(a, pack2(r0, r1));
-  // -R(u)
-  f32x2 q = pack2(0.10403244942426682f, 0.10403244942426682f);
-  q = fma2_of(q, u, pack2(-0.3818792402744293f, -0.3818792402744293f));
-  q = fma2_of(q, u, pack2(0.33312368392944336f, 0.33312368392944336f));
-  q = fma2_of(q, u, pack2(0.7928810119628906f, 0.7928810119628906f));
-  q = fma2_of(q, u, pack2(-2.6637678146362305f, -2.6637678146362305f));
-  q = fma2_of(q, u, pack2(3.7877349853515625f, 3.7877349853515625f));
-  q = fma2_of(q, u, pack2(-3.2672412395477295f, -3.2672412395477295f));
-  q = fma2_of(q, u, pack2(1.7952399253845215f, 1.7952399253845215f));
-  q = fma2_of(q, u, pack2(-0.5f, -0.5f));
-  float x0, x1, e0, e1, q0, q1;
-  unpack2(mul2(mul2(a, pack2(-0.72134752f, -0.72134752f)), a), x0, x1);       // -a^2 / (2 ln 2)
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(x0));
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(x1));
-  bell = pack2(e0, e1);
-  unpack2(mul2(q, bell), q0, q1);
-  // z >= 0: 1 - Q, else Q
-  q0 = __uint_as_float(__float_as_uint(q0) ^ (__float_as_uint(z0) & 0x80000000u));
-  q1 = __uint_as_float(__float_as_uint(q1) ^ (__float_as_uint(z1) & 0x80000000u));
-  cdf = add2(pack2(q0, q1), pack2(__float_as_uint(z0) >> 31 ? 0.0f : 1.0f, __float_as_uint(z1) >> 31 ? 0.0f : 1.0f));
-}
-// GELU'(z) = Phi(z) + z exp(-z^2 / 2) / sqrt(2 pi)
-__device__ __forceinline__ void gelu_grad2(float z0, float z1, float& g0, float& g1) {
-  f32x2 cdf, bell;
-  normal_cdf2(z0, z1, cdf, bell);
-  unpack2(fma2_of(pack2(z0, z1), mul2(bell, pack2(0.39894228f, 0.39894228f)), cdf), g0, g1);
-}
-
 // Where a row's activations go in the next layer's store: the part of its index (in place before the launch) that
 // belongs to one row and one tile of 128 columns.
 struct StoreRow {
@@ -470,7 +427,9 @@ __device__ __forceinline__ void prefetch_z(const TcParams& p, int64_t y0, int64_
   }
 }
 // One chunk of the input gradient: times the derivative of the activation before (ReLU bits, or GELU' of the z that lies in
-// `buf`), rounded, out through the same buffer.
+// `buf`), rounded, out through the same buffer.  GELU' is the function of the CUDA-core route, so that a net's gradients do not
+// depend on the route a shape takes.  Its erff and exponential are what bounds a GELU net's input gradient of few inputs (us,
+// with / without: 16384 x 1024 x 1024 67 / 37, 8192 x 2048 x 512 62 / 25; 16384 x 4096 x 4096 385 / 351, under the MMAs).
 template <bool kGelu>
 __device__ __forceinline__ void dx_chunk(const TcParams& p, const CUtensorMap* tm_dx, const uint32_t (&r)[32], int y0, int n, int lane,
                                          uint32_t bits, uint32_t buf) {
@@ -484,10 +443,8 @@ __device__ __forceinline__ void dx_chunk(const TcParams& p, const CUtensorMap* t
       const uint32_t zw[4] = {zq.x, zq.y, zq.z, zq.w};
 #pragma unroll
       for (int e = 0; e < 8; e += 2) {
-        float d0, d1;
-        gelu_grad2(bf16_lo(zw[e >> 1]), bf16_hi(zw[e >> 1]), d0, d1);
-        g[8 * u + e] *= d0;
-        g[8 * u + e + 1] *= d1;
+        g[8 * u + e] *= gelu_grad_f(bf16_lo(zw[e >> 1]));
+        g[8 * u + e + 1] *= gelu_grad_f(bf16_hi(zw[e >> 1]));
       }
     }
   }

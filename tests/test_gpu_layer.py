@@ -403,6 +403,31 @@ def test_bias_gradient_beside_the_input_gradient(B, D, H, ld, act):
     assert ((db.double() - x.sum(0)).abs() <= (3 + 2 * (B / 1024 + 1) + 5 + 8) * 2.0 ** -24 * x.abs().sum(0)).all()
 
 
+@pytest.mark.parametrize("D,ldp", [(64, 72), (256, 264)])
+def test_gelu_derivative_is_the_same_function_on_both_routes(D, ldp):
+    """The input gradient of a GELU net at every bf16 pre-activation there is, infinities and NaN among them.  dZ has one 1 in a
+    row, so the float32 sum is an entry of W on the tensor cores and on the CUDA cores (taken where the output's row stride
+    is odd), and what is left is the product with GELU': the two routes give the same bits."""
+    import paper_2007_10412_b200 as rad
+    bf = torch.bfloat16
+    B, H = 65536 // D, 64
+    g = torch.Generator(device="cuda").manual_seed(D)
+    z = torch.arange(-32768, 32768, device="cuda").to(torch.int16)[torch.randperm(65536, generator=g, device="cuda")].view(bf).view(B, D)
+    W = torch.randn(D, H, generator=g, device="cuda").to(bf)
+    dZ = torch.zeros(B, H, dtype=bf, device="cuda")
+    dZ[torch.arange(B, device="cuda"), torch.arange(B, device="cuda") % H] = 1
+    outs = [torch.zeros(B, ld, dtype=bf, device="cuda")[:, :D] for ld in (ldp, ldp + 1)]
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for out in outs:
+        rad.rad_linear_input_grad(dZ, W, z_prev=z, dZ_prev=out, dev_status=status)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    tensor, cuda = (out.contiguous() for out in outs)
+    nan = torch.isnan(cuda)
+    assert torch.equal(torch.isnan(tensor), nan)
+    assert torch.equal(tensor[~nan].view(torch.int16), cuda[~nan].view(torch.int16))
+
+
 @pytest.mark.parametrize("B,D,H", [(64, 64, 64), (328, 264, 136), (1000, 520, 264), (4160, 256, 264), (1024, 2048, 2040), (70, 1032, 520)])
 @pytest.mark.parametrize("p", [0.1, 0.7])
 def test_different_sample_dw_over_tile_widths(B, D, H, p):
