@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const __g
 // more than twelve tiles a CTA the two launches of the general form, on all SMs, are faster.
 constexpr int kSmallIndexCtas = 8, kSmallIndexTiles = 12 * kSmallIndexCtas;
 __global__ void __launch_bounds__(32 * kIndexWarps) store_index_small_kernel(const __grid_constant__ IndexParams p, const PhiloxKeys ks) {
+  cluster_started_arrive();                             // waited for behind the draw
   begin_after_previous();
   __shared__ uint32_t s_count[kSmallIndexTiles / kSmallIndexCtas];
   __shared__ uint32_t s_padded[kSmallIndexCtas], s_exact[kSmallIndexCtas];      // of every CTA of the cluster
@@ -115,6 +116,7 @@ __global__ void __launch_bounds__(32 * kIndexWarps) store_index_small_kernel(con
     if (lane == 0) s_count[i] = count;
   }
   __syncthreads();
+  cluster_started_wait();                               // before the first write to a peer: a CTA without tiles is here at once
   if (tid < kSmallIndexCtas) {
     uint32_t padded = 0, exact = 0;
     for (uint32_t i = 0; i < n; ++i) {
