@@ -733,6 +733,20 @@ __device__ __forceinline__ bool mbar_wait2(uint32_t bar, uint32_t parity, const 
     }
   }
 }
+// Several warps meet on a barrier that one lane of each arrives at and waits for (a bounded wait like the others): what any of
+// their threads wrote to shared memory before is seen by all of them after it.  The waiting lane has seen the others' writes,
+// and a warp barrier, which a shuffle is not, hands that on to its warp.
+__device__ __forceinline__ bool warps_meet(uint32_t bar, uint32_t parity, const PairWait& wc, int lane) {
+  __syncwarp();
+  bool met = true;
+  if (lane == 0) {
+    mbar_arrive(bar);
+    met = mbar_wait2(bar, parity, wc);
+  }
+  met = __shfl_sync(0xffffffffu, met ? 1 : 0, 0) != 0;
+  __syncwarp();
+  return met;
+}
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t cbar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
@@ -915,16 +929,11 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
     const int group_thread = lane + 32 * (((warp - 2) >> 2) % group);
     const uint32_t group_bar = smem_u32(&ctl->group[q + 4 * (first_tile & 1)]);
     uint32_t group_phase = 0;
-    const auto group_sync = [&]() -> bool {             // a bounded wait like the others
-      __syncwarp();
-      if (group == 1) return true;
-      bool met = true;
-      if (lane == 0) {
-        mbar_arrive(group_bar);
-        met = mbar_wait2(group_bar, group_phase, wc);
-      }
+    const auto group_sync = [&]() -> bool {
+      if (group == 1) { __syncwarp(); return true; }
+      const bool met = warps_meet(group_bar, group_phase, wc, lane);
       group_phase ^= 1u;
-      return __shfl_sync(0xffffffffu, met ? 1 : 0, 0) != 0;
+      return met;
     };
     int buf = 0, turn = 0;
     uint32_t buf_phases = 0;
@@ -996,12 +1005,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
           // the group is through: two buffers, so that one meeting of the warps per group is enough
           float* red = reinterpret_cast<float*>(epi_smem + kRingBytes) + (cs.turn & 1) * kEpiWarps * 16;
           column_sums_warp(cs, sum_shift, lane, red + (warp - 2) * 16);
-          __syncwarp();
-          if (lane == 0) {
-            mbar_arrive(smem_u32(&ctl->group[0]));
-            ok = mbar_wait2(smem_u32(&ctl->group[0]), cs.turn & 1, wc);
-          }
-          ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+          ok = warps_meet(smem_u32(&ctl->group[0]), cs.turn & 1, wc, lane);
           const int64_t col = ((int64_t)cs.group << sum_shift) * 8 + et;
           if (ok && et < (8 << sum_shift) && col < p.K) {
             float t = 0.0f;

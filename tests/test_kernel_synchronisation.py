@@ -1,5 +1,6 @@
-"""A CTA may touch another CTA's shared memory only once that one is known to have started.  Read off the sources: a kernel
-that breaks this goes wrong on rare runs only, if at all."""
+"""Rules of memory between threads, read off the sources: a kernel that breaks one goes wrong on rare runs only, if at all.
+A CTA may touch another CTA's shared memory only once that one is known to have started.  Where one lane waits for its warp, the
+others read what the wait was for only behind a warp barrier: a shuffle orders no memory."""
 import glob
 import os
 import re
@@ -38,3 +39,24 @@ def test_peers_have_started_before_the_first_write_to_them(file, kernel, body):
     # ... and nobody leaves while a peer may still write to it
     last = [m.start() for m in re.finditer(REMOTE, body)][-1]
     assert "cluster_barrier()" in body[last:], (file, kernel)
+
+
+def _after_lane_waits():
+    """(file and line, what follows) of every place where a warp learns from its first lane how that lane's wait ended."""
+    out = []
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        text = open(path).read()
+        for m in re.finditer(r"__shfl_sync\(0xffffffffu, \w+ \? 1 : 0, 0\)[^;]*;", text):
+            out.append((f"{os.path.basename(path)}:{text[:m.start()].count(chr(10)) + 1}", text[m.end():m.end() + 240]))
+    return out
+
+
+LANE_WAITS = _after_lane_waits()
+
+
+@pytest.mark.parametrize("place,rest", LANE_WAITS, ids=[w[0] for w in LANE_WAITS])
+def test_a_wait_by_one_lane_is_handed_on_to_its_warp(place, rest):
+    """A warp barrier comes next, or a fence of tensor memory where it is accumulators that are read."""
+    leave = r"(if \(!\w+\) (break|return false);\s*)?"
+    copies = r"(if \(EPI == kDxGelu\) \{[^}]*\}\s*)?"
+    assert re.match(r"\s*" + leave + copies + r"(__syncwarp\(\)|tc_fence_after\(\));", rest), place
