@@ -1,4 +1,5 @@
-// Shared by the two different-sample store kernels: launch parameters and the look-back status word.
+// Shared by the two different-sample store kernels: launch parameters and the look-back status word; and what the dense
+// epilogue stages of a store.
 #pragma once
 
 #include "common.cuh"
@@ -46,6 +47,18 @@ __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// ---- kept entries staged in shared memory (tc.cu) -----------------------------------------------
+// The kept entries of 32 rows and 128 columns on their way to the next store: elements `first & ~7` .. of `values`, where `first`
+// is the place of the first row's first entry.
+constexpr int kFillBytes = 3584;
+constexpr uint32_t kFillValues = kFillBytes / 2;
+// Do the entries of one row, pos .. end, lie behind the first row's and inside the buffer?  An index that was drawn for the store
+// says yes to the first of these always; memory that holds something else may not, and then nothing is staged.
+__host__ __device__ constexpr bool row_in_order(uint32_t first, uint32_t pos, uint32_t end) { return pos >= first && end >= pos; }
+__host__ __device__ constexpr bool row_fits_stage(uint32_t first, uint32_t pos, uint32_t end) {
+  return row_in_order(first, pos, end) && end - (first & ~7u) <= kFillValues;
 }
 
 // Bits of (a > 0) for 32 consecutive entries in shared memory; zero of either sign gives 0.

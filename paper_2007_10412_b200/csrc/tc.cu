@@ -27,7 +27,7 @@
 #include <cmath>
 #include <type_traits>
 
-#include "common.cuh"
+#include "store.cuh"
 
 namespace rad {
 namespace {
@@ -188,11 +188,9 @@ struct Schedule {
 // accumulators are waited for.
 constexpr int kChunkBytes = 32 * 64;             // 32 rows x 32 bf16 columns
 constexpr int kRingBytes = 32 * kChunkBytes;     // chunk buffers of all epilogue warps: four each of eight, two each of sixteen
-constexpr int kFillBytes = 3584;                 // kept values of 32 rows and 128 columns on their way to the next store
 constexpr int kFillBuffers = 8;                  // four lane quarters, two tiles of 128 columns
 constexpr int kBiasBytes = 8 * 128 * 4;          // every warp's columns of the bias
 constexpr int kEpiBytes = kRingBytes + kFillBuffers * kFillBytes + kBiasBytes;
-constexpr uint32_t kFillValues = kFillBytes / 2;
 
 __device__ __forceinline__ uint32_t chunk16_addr(uint32_t base, int row, int unit) { return base + row * 64 + ((unit ^ ((row >> 1) & 3)) << 4); }
 __device__ __forceinline__ uint32_t chunk32_addr(uint32_t base, int row, int unit) { return base + row * 128 + ((unit ^ (row & 7)) << 4); }
@@ -238,8 +236,11 @@ struct StoreRow {
     }
     // the 32 rows of a warp lie in one tile, one after the other, so their kept entries are neighbours
     seg = __shfl_sync(0xffffffffu, pos, 0);
+    const bool in_order = __all_sync(0xffffffffu, !row_ok || row_in_order(seg, pos, end));
+    const bool fits = __all_sync(0xffffffffu, !row_ok || row_fits_stage(seg, pos, end));
+    if (!in_order) raise_status(p.dev_status, RAD_DEV_EINTERNAL);      // not this store's index: entry by entry, inside `values`
     end = __reduce_max_sync(0xffffffffu, end);
-    staged = whole_tile && ((uintptr_t)p.st_values & 15) == 0 && end > seg && end - (seg & ~7u) <= kFillValues;
+    staged = whole_tile && ((uintptr_t)p.st_values & 15) == 0 && end > seg && fits;
   }
 };
 
@@ -304,8 +305,9 @@ __device__ __forceinline__ void pad_store_tile(const TcParams& p, int64_t m, int
   const uint4 last = *reinterpret_cast<const uint4*>(tw + 63 * 4);
   const uint32_t exact = reinterpret_cast<const unsigned short*>(tw + kBitWords)[63] + __popc(last.x) + __popc(last.y) +
                          __popc(last.z) + __popc(last.w);
-  const uint32_t end = (uint32_t)min((int64_t)p.st_offsets[tile + 1], p.st_capacity);
-  for (uint32_t q = p.st_offsets[tile] + exact; q < end; ++q) p.st_values[q] = __float2bfloat16_rn(0.0f);
+  // 64 bits: places past 2^32 are no places of the buffer's beginning
+  const uint64_t end = min((uint64_t)p.st_offsets[tile + 1], (uint64_t)p.st_capacity);
+  for (uint64_t q = (uint64_t)p.st_offsets[tile] + exact; q < end; ++q) p.st_values[q] = __float2bfloat16_rn(0.0f);
 }
 
 // the ring's slot of a chunk: one, or the first of two
