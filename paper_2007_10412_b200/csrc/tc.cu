@@ -1079,6 +1079,8 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       buf ^= 1;
     }
     if (EPI != kDwT) {
+      // a unit that was given up may have left z on its way
+      if (EPI == kDxGelu) asm volatile("cp.async.wait_all;" ::: "memory");
       if (elect_one()) tma_store_wait();               // the results are out, and the buffers no longer read
       __syncwarp();
     }

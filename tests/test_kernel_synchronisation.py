@@ -60,3 +60,13 @@ def test_a_wait_by_one_lane_is_handed_on_to_its_warp(place, rest):
     leave = r"(if \(!\w+\) (break|return false);\s*)?"
     copies = r"(if \(EPI == kDxGelu\) \{[^}]*\}\s*)?"
     assert re.match(r"\s*" + leave + copies + r"(__syncwarp\(\)|tc_fence_after\(\));", rest), place
+
+
+def test_a_dense_kernel_that_gives_up_waits_for_its_own_copies():
+    """A wait that runs out leaves the loop over the units between a copy's start and the wait for it: behind the loop, and
+    before the CTA leaves, both kinds of copies of the epilogue warps are waited for."""
+    body, = [k[2] for k in _kernels() if k[1] == "tc_gemm_pair_kernel"]
+    assert "prefetch_z(" in body and body.index("prefetch_z(") < body.rindex("if (!ok) break;")
+    tail = body[body.rindex("buf ^= 1;"):]
+    assert re.search(r"if \(EPI == kDxGelu\) asm volatile\(\"cp\.async\.wait_all;\"", tail) and "tma_store_wait();" in tail
+    assert tail.index("cp.async.wait_all") < tail.index("cluster_barrier()") > tail.index("tma_store_wait();")
