@@ -1590,7 +1590,7 @@ DwPlan plan_dw(const rad_store* st, int64_t H) {
   }
 }
 
-struct OutMaps { CUtensorMap o, l, z; };      // see tc_gemm_pair_kernel; those of absent outputs are not read
+struct OutMaps { CUtensorMap o, l, z; };      // see tc_gemm_pair_kernel; those of absent outputs are not written through
 
 template <int AK, int BKIND, int EPI, int kEpiWarps = 8>
 int launch_pair(const TcParams& p, const CUtensorMap& ta, const CUtensorMap& tb, const OutMaps& out, int64_t max_units, cudaStream_t s) {
@@ -1684,6 +1684,10 @@ int tc_forward(int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t 
   if (out_act != nullptr) RAD_TRY(make_out_map(&out.o, false, out_act, H, B, ld_act));
   if (out_zlow != nullptr) RAD_TRY(make_out_map(&out.l, false, out_zlow, H, B, ld_zlow));
   if (out_z != nullptr) RAD_TRY(make_out_map(&out.z, true, out_z, H, B, ld_z));
+  // the kernel fetches a map ahead of time: each is one that was encoded
+  if (out_act == nullptr) out.o = out_zlow != nullptr ? out.l : out.z;
+  if (out_zlow == nullptr) out.l = out.o;
+  if (out_z == nullptr) out.z = out.o;
   const bool fill = p.st_values != nullptr;
   const bool wide = fill ? D <= kWideEpilogueK
                          : act == RAD_ACT_GELU && D <= kWideGeluK && (out_zlow == nullptr || units <= kWideGeluWaves * planning_pairs());
@@ -1722,6 +1726,7 @@ int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, 
   p.wait_limit_ns = wait_limit_ns();
   OutMaps out = {};
   RAD_TRY(make_out_map(&out.o, false, dZ_prev, D, B, ldp));
+  out.l = out.z = out.o;
   const int64_t units = ceil_div(B, BM) * ceil_div(D, bn);
   return z_prev != nullptr ? launch_pair<kAK, kBK_, kDxGelu>(p, ta, tb, out, units, s)
                            : launch_pair<kAK, kBK_, kDx>(p, ta, tb, out, units, s);
@@ -1756,7 +1761,7 @@ int tc_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, 
     if (rc != RAD_OK) return rc;
     p.M = H; p.N = nmax; p.N_dev = st->nnz; p.row_idx = st->offsets; p.keep_cols = st->keepbits;
     const int64_t n_expect = std::max<int64_t>(1, (int64_t)std::llround((double)st->D * store_keep_fraction(st)));
-    rc = launch_pair<kAMN, kBMN, kDwT>(p, ta, tb, OutMaps{}, ceil_div(H, BM) * ceil_div(std::min(n_expect, nmax), BN) * d.splits, s);
+    rc = launch_pair<kAMN, kBMN, kDwT>(p, ta, tb, OutMaps{tb, tb, tb}, ceil_div(H, BM) * ceil_div(std::min(n_expect, nmax), BN) * d.splits, s);
   } else {
     ta = tb;                                           // unused by the sparse-A kernel
     p.M = st->D;

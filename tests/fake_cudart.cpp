@@ -2,12 +2,13 @@
 // GPU: one sm_100 device, launches that are recorded and do nothing, and one of them that fails when asked to.
 #include <cuda_runtime_api.h>
 
+#include <cstdint>
 #include <map>
 #include <string>
 #include <vector>
 
 namespace {
-struct Launch { std::string kernel; unsigned dims[8]; };       // grid, block, shared memory, CTAs of a cluster
+struct Launch { std::string kernel; unsigned dims[8]; int maps; };   // grid, block, shared memory, CTAs of a cluster; see fake_maps
 std::vector<Launch> launches;
 std::map<const void*, std::string> names;
 int fail_at = -1;
@@ -15,14 +16,18 @@ cudaError_t last_error = cudaSuccess;
 alignas(256) char device_symbol[256];
 
 cudaError_t set(cudaError_t e) { if (e != cudaSuccess) last_error = e; return e; }
-cudaError_t launch(const void* f, dim3 g, dim3 b, size_t smem, unsigned cluster) {
+constexpr uint64_t kEncoded = 0x6d617021;         // what encode_tiled leaves in a tensor map
+cudaError_t launch(const void* f, dim3 g, dim3 b, size_t smem, unsigned cluster, void** args) {
   const bool fails = (int)launches.size() == fail_at;
-  launches.push_back({names[f], {g.x, g.y, g.z, b.x, b.y, b.z, (unsigned)smem, cluster}});
+  int maps = 0;
+  if (names[f].find("tc_gemm_pair_kernel") != std::string::npos)         // parameters, then five tensor maps
+    for (int i = 0; i < 5; ++i) maps |= (*static_cast<const uint64_t*>(args[1 + i]) == kEncoded ? 1 : 0) << i;
+  launches.push_back({names[f], {g.x, g.y, g.z, b.x, b.y, b.z, (unsigned)smem, cluster}, maps});
   const bool bad = g.x == 0 || g.x > 0x7fffffffu || g.y == 0 || g.y > 65535 || g.z == 0 || g.z > 65535 || b.x * b.y * b.z > 1024 ||
                    b.x * b.y * b.z == 0 || smem > 227 * 1024;
   return set(fails || bad ? cudaErrorInvalidConfiguration : cudaSuccess);
 }
-int encode_tiled(...) { return 0; }
+int encode_tiled(uint64_t* map, ...) { *map = kEncoded; return 0; }
 }  // namespace
 
 extern "C" {
@@ -31,6 +36,7 @@ void fake_reset(int which_fails) { launches.clear(); fail_at = which_fails; last
 int fake_launches() { return (int)launches.size(); }
 int fake_last_error() { return (int)last_error; }
 const char* fake_kernel(int i) { return launches[i].kernel.c_str(); }
+int fake_maps(int i) { return launches[i].maps; }        // bit k: tensor map k of a dense tensor-core kernel was encoded
 void fake_dims(int i, unsigned* out) { for (int k = 0; k < 8; ++k) out[k] = launches[i].dims[k]; }
 
 // ---- the runtime ----
@@ -45,12 +51,12 @@ cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* s, void* st) {
   *g = pushed.g; *b = pushed.b; *s = pushed.s; *static_cast<void**>(st) = pushed.st;
   return cudaSuccess;
 }
-cudaError_t cudaLaunchKernel(const void* f, dim3 g, dim3 b, void**, size_t s, cudaStream_t) { return launch(f, g, b, s, 1); }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
+cudaError_t cudaLaunchKernel(const void* f, dim3 g, dim3 b, void** args, size_t s, cudaStream_t) { return launch(f, g, b, s, 1, args); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
   unsigned cluster = 1;
   for (unsigned i = 0; i < c->numAttrs; ++i)
     if (c->attrs[i].id == cudaLaunchAttributeClusterDimension) cluster = c->attrs[i].val.clusterDim.x * c->attrs[i].val.clusterDim.y;
-  return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, cluster);
+  return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, cluster, args);
 }
 cudaError_t cudaGetLastError() { const cudaError_t e = last_error; last_error = cudaSuccess; return e; }
 cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }

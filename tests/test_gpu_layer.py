@@ -378,6 +378,23 @@ def test_outputs_in_chunks_and_the_store_beside_them(B, D, H, p, shift):
     assert ((z2.double() - want).abs() <= (D ** 0.5 + 16) * 2.0 ** -24 * mag).all()      # float32 sums in any order
 
 
+@pytest.mark.parametrize("act", ["none", "relu", "gelu"])
+@pytest.mark.parametrize("B,D,H", [(64, 64, 64), (300, 72, 136), (2500, 64, 1032)])
+def test_pre_activations_as_the_only_output(B, D, H, act):
+    """The forward pass on the tensor cores with its bf16 pre-activations as the only output: the same bits as beside others."""
+    import paper_2007_10412_b200 as rad
+    bf = torch.bfloat16
+    g = torch.Generator(device="cuda").manual_seed(B + H)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    A, W, b = rnd(B, D).to(bf), rnd(D, H).to(bf), rnd(H)
+    alone, beside, out = (torch.full((B, H), -7.0, dtype=bf, device="cuda") for _ in range(3))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rad.rad_linear_forward(A, W, b, act, out_zlow=alone, dev_status=status)
+    rad.rad_linear_forward(A, W, b, act, out_act=out, out_zlow=beside, dev_status=status)
+    torch.cuda.synchronize()
+    assert status.item() == 0 and torch.equal(alone, beside)
+
+
 @pytest.mark.parametrize("B,D,H,ld", [(64, 64, 64, 64), (130, 72, 200, 208), (2049, 128, 1184, 1184), (2100, 64, 1192, 1192),
                                       (20000, 1096, 264, 264), (1024, 64, 4744, 4744)])
 @pytest.mark.parametrize("act", ["relu", "gelu"])

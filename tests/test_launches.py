@@ -277,3 +277,25 @@ def test_forms_of_the_cuda_core_gemm(fake):
             (name, *dims), = _launches(b)
             got = f"walk{tile[dims[6]]}" if "gemm_walk_kernel" in name else f"split{tile[dims[6]]}x{dims[7]}"
             assert got == form, (B, D, H, dtype, name)
+
+
+@pytest.mark.parametrize("act", ["relu", "gelu", "none"])
+@pytest.mark.parametrize("outputs", ["act", "z", "zlow", "act z", "act zlow", "z zlow", "act z zlow", "fill", "input gradient", "same"])
+def test_every_tensor_map_of_a_dense_kernel_is_an_encoded_one(fake, act, outputs):
+    """Also those of outputs that are not asked for: the kernel fetches a map before it knows what is stored through it."""
+    b, bf, (B, D, H) = fake, torch.bfloat16, (300, 256, 136)
+    A, W, o, z, zl = (torch.empty(*s, dtype=t) for s, t in (((B, D), bf), ((D, H), bf), ((B, H), bf), ((B, H), torch.float32), ((B, H), bf)))
+    same = _store(b, "same", "bf16", B, D)
+    b.lib().fake_reset(-1)
+    if outputs == "fill":
+        b.rad_linear_forward_fill(A, W, None, act, o, _store(b, "different", "bf16", B, H))
+    elif outputs == "input gradient":
+        b.rad_linear_input_grad(o, W, z_prev=A if act == "gelu" else None, dZ_prev=torch.empty(B, D, dtype=bf))
+    elif outputs == "same":
+        b.rad_linear_weight_grad(same, o, torch.empty(D, H))
+    else:
+        want = outputs.split()
+        b.rad_linear_forward(A, W, None, act, out_act=o if "act" in want else None, out_z=z if "z" in want else None,
+                             out_zlow=zl if "zlow" in want else None)
+    dense = [i for i in range(b.lib().fake_launches()) if _pair_kernel(b.lib().fake_kernel(i).decode())]
+    assert len(dense) == 1 and b.lib().fake_maps(dense[0]) == 31
