@@ -438,15 +438,16 @@ extern "C" int rad_linear_input_grad(int32_t dtype, int64_t B, int64_t D, int64_
   if (rc != RAD_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const bool on_tc = dZ_prev != nullptr && input_grad_on_tc(dtype, B, D, H, dZ, ldz, W, ldw, z_prev, ld_zprev, dZ_prev, ldp);
+  const bool beside = on_tc && db != nullptr && tc_sums_beside(B, D, H);
   if (db != nullptr) {
-    // on the tensor cores the sums are made beside the contraction (in no workspace, which is asked for all the same)
-    if (on_tc && (workspace == nullptr || workspace_bytes < column_sums_workspace(B, H))) return RAD_EWORKSPACE;
-    if (!on_tc) rc = column_sums(dtype, B, H, dZ, ldz, db, workspace, workspace_bytes, s);
+    // sums that are made beside the contraction use no workspace, which is asked for all the same
+    if (beside && (workspace == nullptr || workspace_bytes < column_sums_workspace(B, H))) return RAD_EWORKSPACE;
+    if (!beside) rc = column_sums(dtype, B, H, dZ, ldz, db, workspace, workspace_bytes, s);
     if (rc != RAD_OK) return rc;
   }
   if (dZ_prev == nullptr) return RAD_OK;
   if (on_tc)
-    return tc_input_grad(B, D, H, dZ, ldz, W, ldw, relubits_prev, z_prev, ld_zprev, dZ_prev, ldp, db, dev_status, s);
+    return tc_input_grad(B, D, H, dZ, ldz, W, ldw, relubits_prev, z_prev, ld_zprev, dZ_prev, ldp, beside ? db : nullptr, dev_status, s);
   return simt_input_grad(dtype, B, D, H, dZ, ldz, W, ldw, relubits_prev, z_prev, ld_zprev, dZ_prev, ldp, s);
 }
 

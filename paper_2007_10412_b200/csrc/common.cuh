@@ -334,6 +334,7 @@ int launch_replace_extras(const void* A, int64_t lda, const rad_store* st, const
 int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, const void* W,
                   int64_t ldw, const uint32_t* relubits_prev, const void* z_prev, int64_t ld_zprev,
                   void* dZ_prev, int64_t ldp, float* db, int32_t* dev_status, cudaStream_t s);
+bool tc_sums_beside(int64_t B, int64_t D, int64_t H);      // does tc_input_grad also make db, or is that another launch?
 int tc_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, float* dW,
                    int64_t ldw, void* workspace, int64_t workspace_bytes, int32_t* dev_status,
                    cudaStream_t s);

@@ -535,6 +535,7 @@ struct ColumnSums {
   }
 };
 constexpr int kSumThreads = 256, kSumLoads = 8;
+__host__ __device__ constexpr int sum_shift(int64_t columns, int64_t ctas) { return columns > 8 * ctas ? 1 : 0; }   // 16-byte loads a row: 1 or 2
 __device__ __forceinline__ void add_bf16x8(const uint4& q, float (&v)[8]) {
   const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
@@ -945,10 +946,10 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
     cs.clear();
     cs.group = blockIdx.x; cs.step = 0; cs.turn = 0;
     const int et = tid - 64;                           // 0 .. 32 kEpiWarps - 1
-    const int sum_shift = p.K > 8 * (int64_t)gridDim.x ? 1 : 0;
+    const int shift = sum_shift(p.K, (int64_t)gridDim.x);
     uint32_t sum_groups = 0, sum_steps = 0, quota = 0;
     if (is_dx(EPI) && p.db != nullptr) {
-      const uint32_t rows = (kSumThreads >> sum_shift) * kSumLoads, cols = 8u << sum_shift;
+      const uint32_t rows = (kSumThreads >> shift) * kSumLoads, cols = 8u << shift;
       sum_groups = ((uint32_t)p.K + cols - 1) / cols;
       sum_steps = ((uint32_t)p.M + rows - 1) / rows;
       const uint32_t own_groups = cs.group < sum_groups ? (sum_groups - cs.group + gridDim.x - 1) / gridDim.x : 0;
@@ -1002,14 +1003,14 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       }
       if (is_dx(EPI) && p.db != nullptr) {
         for (uint32_t k = 0; k < quota && cs.group < sum_groups && ok; ++k) {
-          column_sums_step(p, cs, sum_shift, et);
+          column_sums_step(p, cs, shift, et);
           if (++cs.step < sum_steps) continue;
           // the group is through: two buffers, so that one meeting of the warps per group is enough
           float* red = reinterpret_cast<float*>(epi_smem + kRingBytes) + (cs.turn & 1) * kEpiWarps * 16;
-          column_sums_warp(cs, sum_shift, lane, red + (warp - 2) * 16);
+          column_sums_warp(cs, shift, lane, red + (warp - 2) * 16);
           ok = warps_meet(smem_u32(&ctl->group[0]), cs.turn & 1, wc, lane);
-          const int64_t col = ((int64_t)cs.group << sum_shift) * 8 + et;
-          if (ok && et < (8 << sum_shift) && col < p.K) {
+          const int64_t col = ((int64_t)cs.group << shift) * 8 + et;
+          if (ok && et < (8 << shift) && col < p.K) {
             float t = 0.0f;
 #pragma unroll
             for (int i = 0; i < kEpiWarps; ++i) t += red[i * 16 + et];
@@ -1706,6 +1707,21 @@ int tc_forward(int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t 
     case kFwdFill + RAD_ACT_GELU: return launch(std::integral_constant<int, kFwdFill + RAD_ACT_GELU>());
     default: return launch(std::integral_constant<int, kFwd>());
   }
+}
+
+// Whether the bias gradient goes beside the input gradient or into a launch of its own.  Beside it costs the CTAs of the
+// contraction, however few, about 1.1 us per group of columns and 1.7 us per further step down the rows, of which each K block of
+// their tiles hides 0.15 us; the launch costs 2.5 us and its reading.  Us, beside / separate: 4096 rows, dZ 1024 wide and inputs
+// 1024 wide 11.0 / 17.5, 1024 x 8192 to 1024 28.0 / 35.5, but 256 x 4096 to 64 148 / 16, 16384 x 4096 to 256 101 / 70.  Over
+// 238 shapes (64 to 16384 rows, 64 to 8192 columns) the choice is the faster one, or within 3 % of it but for five where it is
+// within 8 %.
+bool tc_sums_beside(int64_t B, int64_t D, int64_t H) {
+  const int64_t bn = dense_tile_width(B, D), units = ceil_div(B, BM) * ceil_div(D, bn);
+  const int64_t pairs = std::min<int64_t>(units, planning_pairs());
+  const int shift = sum_shift(H, 2 * pairs);
+  const int64_t groups = ceil_div(ceil_div(H, 8ll << shift), 2 * pairs), steps = ceil_div(B, (int64_t)(kSumThreads >> shift) * kSumLoads);
+  const double sums = (double)groups * (1.1 + 1.7 * (double)(steps - 1)), hidden = 0.15 * (double)(ceil_div(units, pairs) * ceil_div(H, BK));
+  return sums <= hidden + 2.5 + (double)B * (double)H * 2.0 / 6e6;
 }
 
 int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, const void* W, int64_t ldw,

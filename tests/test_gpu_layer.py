@@ -395,12 +395,27 @@ def test_pre_activations_as_the_only_output(B, D, H, act):
     assert status.item() == 0 and torch.equal(alone, beside)
 
 
-@pytest.mark.parametrize("B,D,H,ld", [(64, 64, 64, 64), (130, 72, 200, 208), (2049, 128, 1184, 1184), (2100, 64, 1192, 1192),
-                                      (20000, 1096, 264, 264), (1024, 64, 4744, 4744)])
+BIAS_ROUTES = [
+    # B, D, H, row stride of dZ, are the column sums made by the input gradient's launch?
+    (64, 64, 64, 64, True),
+    (130, 72, 200, 208, False),
+    (300, 1032, 200, 208, True),
+    (2049, 128, 1184, 1184, False),
+    (2100, 64, 1192, 1192, False),
+    (20000, 1096, 264, 264, False),
+    (1024, 64, 4744, 4744, False),
+    (256, 64, 4096, 4096, False),
+    (200, 4096, 8192, 8192, True),          # four groups of columns per CTA
+    (1100, 2048, 4104, 4104, True),         # ... of two steps down the rows each
+    (9000, 2048, 1032, 1032, True),         # five steps, four tiles per SM pair
+]
+
+
+@pytest.mark.parametrize("B,D,H,ld", [r[:4] for r in BIAS_ROUTES])
 @pytest.mark.parametrize("act", ["relu", "gelu"])
 def test_bias_gradient_beside_the_input_gradient(B, D, H, ld, act):
-    """Column sums made by the input gradient's launch: one group of 8 or 16 columns per CTA and several, rows that end inside a
-    step, several tiles per SM pair; the input gradient is the same with and without them.  Bound: eight rows as a tree, then
+    """Column sums asked for with the input gradient, made by its launch (one group of 8 or 16 columns per CTA and several, rows
+    that end inside a step, several tiles per SM pair) or by one of their own; the input gradient is the same with and without them.  Bound: eight rows as a tree, then
     at most B / 1024 + 1 steps, lanes and warps, each a float32 rounding of the sum of magnitudes."""
     import paper_2007_10412_b200 as rad
     bf = torch.bfloat16

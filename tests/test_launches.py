@@ -299,3 +299,21 @@ def test_every_tensor_map_of_a_dense_kernel_is_an_encoded_one(fake, act, outputs
                              out_zlow=zl if "zlow" in want else None)
     dense = [i for i in range(b.lib().fake_launches()) if _pair_kernel(b.lib().fake_kernel(i).decode())]
     assert len(dense) == 1 and b.lib().fake_maps(dense[0]) == 31
+
+
+def test_where_the_bias_gradient_is_made(fake):
+    """The routes that the parity test of the bias gradient claims to cover are the ones the library takes: beside the input
+    gradient where its K blocks hide the sums or nearly so, in a launch of its own where few CTAs would be held up by them.  A
+    workspace that is too small is refused on either route."""
+    from test_gpu_layer import BIAS_ROUTES
+    b, bf = fake, torch.bfloat16
+    for B, D, H, ld, beside in BIAS_ROUTES:
+        dZ, W, out, db = torch.empty(B, ld, dtype=bf)[:, :H], torch.empty(D, H, dtype=bf), torch.empty(B, D, dtype=bf), torch.empty(H)
+        ws = _aligned(b.rad_input_grad_workspace(B, H))
+        b.lib().fake_reset(-1)
+        b.rad_linear_input_grad(dZ, W, dZ_prev=out, db=db, workspace=ws)
+        names = [l[0] for l in _launches(b)]
+        assert [bool(_pair_kernel(n)) for n in names][-1] and (len(names) == 1) == beside, (B, D, H, names)
+        assert beside or all("colsum_kernel" in n for n in names[:-1])
+        with pytest.raises(b.RadError, match="workspace too small"):
+            b.rad_linear_input_grad(dZ, W, dZ_prev=out, db=db, workspace=ws[:-1])
