@@ -61,6 +61,14 @@ __host__ __device__ constexpr bool row_fits_stage(uint32_t first, uint32_t pos, 
   return row_in_order(first, pos, end) && end - (first & ~7u) <= kFillValues;
 }
 
+// ---- the values of one tile as a bulk copy (tc.cu) -----------------------------------------------
+// Tile offsets of a store are multiples of 8 elements and ascend; others would make a copy that is misaligned or runs away.
+__host__ __device__ constexpr bool tile_in_order(uint32_t begin, uint32_t end) { return ((begin | end) & 7u) == 0u && begin <= end; }
+// Elements begin .. end of a buffer of `capacity`, in at most `room` bytes of shared memory.
+__host__ __device__ constexpr bool tile_fits(uint32_t begin, uint32_t end, int64_t capacity, uint32_t room) {
+  return (int64_t)end <= capacity && (uint64_t)(end - begin) * 2u <= room;
+}
+
 // Bits of (a > 0) for 32 consecutive entries in shared memory; zero of either sign gives 0.
 __device__ __forceinline__ uint32_t positive32(const float* src) {
   uint32_t m = 0;

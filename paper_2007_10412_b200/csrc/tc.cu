@@ -1291,10 +1291,11 @@ tc_sparse_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmB)
           if (sent) {
             const uint32_t cfull = smem_u32(&ctl->comp_full[slot]);
             const uint32_t sC = smem_u32(comp_base) + slot * comp_slot;
-            uint32_t vb = have ? (o1 - o0) * 2u : 0u;
-            if (vb > (uint32_t)p.comp_cap || (int64_t)o1 > p.values_capacity) {
-              vb = 0;
-              raise_status(p.dev_status, RAD_DEV_ECAPACITY);
+            uint32_t vb = 0;
+            if (have) {
+              if (!tile_in_order(o0, o1)) raise_status(p.dev_status, RAD_DEV_EINTERNAL);          // no store's offsets
+              else if (!tile_fits(o0, o1, p.values_capacity, (uint32_t)p.comp_cap)) raise_status(p.dev_status, RAD_DEV_ECAPACITY);
+              else vb = (o1 - o0) * 2u;
             }
             mbar_arrive_expect_tx(cfull, (have ? (uint32_t)kIndexBytes : 0u) + vb);
             if (have) {

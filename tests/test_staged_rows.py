@@ -1,4 +1,5 @@
-"""Which rows of a store the dense epilogue stages in shared memory: the rule of csrc/store.cuh, run on the host."""
+"""Which rows of a store the dense epilogue stages in shared memory, and which tiles the different-sample weight gradient copies
+there: the rules of csrc/store.cuh, run on the host."""
 import os
 import subprocess
 
@@ -44,13 +45,33 @@ int main() {
     }
     if (all != (last - (first & ~7u) <= kFillValues)) ++refused;
   }
+  // a tile that is let in is a copy of whole 16-byte pieces from inside the buffer, no longer than its room
+  long long bad = 0, copied = 0;
+  for (int i = 0; i < 2000000; ++i) {
+    const uint32_t near = rng() >> (rng() % 32), begin = (rng() & 1) ? near & ~7u : near;
+    const uint32_t end = (rng() & 3) ? begin + (rng() % 1025) * ((rng() & 3) ? 8u : 1u) : (uint32_t)rng();
+    const int64_t capacity = (rng() & 1) ? (int64_t)end + (int64_t)(rng() % 33) - 16 : (int64_t)rng();
+    const uint32_t room = 128u * (1u + rng() % 128u);
+    if (!tile_in_order(begin, end) || !tile_fits(begin, end, capacity, room)) continue;
+    ++copied;
+    const uint64_t bytes = ((uint64_t)end - begin) * 2u;
+    if (begin % 8 != 0 || bytes % 16 != 0 || end < begin || (int64_t)end > capacity || bytes > room) ++bad;
+  }
+  for (uint32_t begin : at)
+    for (uint32_t end : at)
+      if (tile_in_order(begin, end) && tile_fits(begin, end, 0xffffffffll, 16384u) && (end < begin || end - begin > 8192u)) ++bad;
+  // every tile of a store that its buffer holds is copied
+  for (uint32_t kept = 0; kept <= 8192; kept += 8)
+    if (!tile_in_order(1u << 30, (1u << 30) + kept) || !tile_fits(1u << 30, (1u << 30) + kept, (1ll << 30) + kept, 16384u)) ++bad;
+  outside += bad;
+  taken = taken > 100000 && copied > 100000 ? taken : 0;
   printf("%lld %lld %d\n", outside, refused, taken > 100000 ? 1 : 0);
   return 0;
 }
 """
 
 
-def test_a_staged_row_lies_in_the_buffer_whatever_the_index_holds(tmp_path):
+def test_staged_rows_and_tiles_lie_in_their_buffers_whatever_the_index_holds(tmp_path):
     src, exe = tmp_path / "rows.cu", tmp_path / "rows"
     src.write_text(PROGRAM)
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
