@@ -117,6 +117,10 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+}
 // 16 lanes x 32 columns: register 4 i + e holds lane (thread / 4) + 8 (e / 2), column 8 i + 2 (thread % 4) + e % 2.
 __device__ __forceinline__ void tmem_ld16x32(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
@@ -430,30 +434,44 @@ __device__ __forceinline__ void prefetch_z(const TcParams& p, int64_t y0, int64_
 }
 // One chunk of the input gradient: times the derivative of the activation before (ReLU bits, or GELU' of the z that lies in
 // `buf`), rounded, out through the same buffer.  GELU' is the function of the CUDA-core route, so that a net's gradients do not
-// depend on the route a shape takes.  Its erff and exponential are what bounds a GELU net's input gradient of few inputs (us,
-// with / without: 16384 x 1024 x 1024 67 / 37, 8192 x 2048 x 512 62 / 25; 16384 x 4096 x 4096 385 / 351, under the MMAs).
+// depend on the route a shape takes.  Its erff and exponential are what bounds a GELU net's input gradient of few inputs.  They
+// are made for eight columns a turn: with the code of 32 in one piece, which every warp fetches anew for every chunk, 16384 x
+// 2048 x 1024 took 95 us instead of 79, 16384 x 4096 x 64 166 instead of 128 (sixteen warps: 123 for the latter, but more where
+// the MMAs bound: 4096 x 2048 x 2048 32.7 against 30.9).
 template <bool kGelu>
-__device__ __forceinline__ void dx_chunk(const TcParams& p, const CUtensorMap* tm_dx, const uint32_t (&r)[32], int y0, int n, int lane,
-                                         uint32_t bits, uint32_t buf) {
-  float g[32];
-#pragma unroll
-  for (int j = 0; j < 32; ++j) g[j] = ((bits >> j) & 1u) ? __uint_as_float(r[j]) : 0.0f;
+__device__ __forceinline__ void dx_chunk(const CUtensorMap* tm_dx, uint32_t taddr, int y0, int n, int lane, uint32_t bits, uint32_t buf) {
   if (kGelu) {
-#pragma unroll
+#pragma unroll 1
     for (int u = 0; u < 4; ++u) {
-      const uint4 zq = ld_shared16(chunk16_addr(buf, lane, u));
+      uint32_t r[8];
+      tmem_ld8(taddr + 8 * u, r);
+      const uint32_t at = chunk16_addr(buf, lane, u);
+      const uint4 zq = ld_shared16(at);
       const uint32_t zw[4] = {zq.x, zq.y, zq.z, zq.w};
+      float g[8];
 #pragma unroll
       for (int e = 0; e < 8; e += 2) {
-        g[8 * u + e] *= gelu_grad_f(bf16_lo(zw[e >> 1]));
-        g[8 * u + e + 1] *= gelu_grad_f(bf16_hi(zw[e >> 1]));
+        g[e] = gelu_grad_f(bf16_lo(zw[e >> 1]));
+        g[e + 1] = gelu_grad_f(bf16_hi(zw[e >> 1]));
       }
-    }
-  }
+      tmem_ld_wait();
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
-    st_shared16(chunk16_addr(buf, lane, u), pack_bf16(g[8 * u], g[8 * u + 1]), pack_bf16(g[8 * u + 2], g[8 * u + 3]),
-                pack_bf16(g[8 * u + 4], g[8 * u + 5]), pack_bf16(g[8 * u + 6], g[8 * u + 7]));
+      for (int e = 0; e < 8; ++e) g[e] *= ((bits >> e) & 1u) ? __uint_as_float(r[e]) : 0.0f;
+      st_shared16(at, pack_bf16(g[0], g[1]), pack_bf16(g[2], g[3]), pack_bf16(g[4], g[5]), pack_bf16(g[6], g[7]));
+      bits >>= 8;
+    }
+  } else {
+    uint32_t r[32];
+    tmem_ld32(taddr, r);
+    tmem_ld_wait();
+    float g[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) g[j] = ((bits >> j) & 1u) ? __uint_as_float(r[j]) : 0.0f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      st_shared16(chunk16_addr(buf, lane, u), pack_bf16(g[8 * u], g[8 * u + 1]), pack_bf16(g[8 * u + 2], g[8 * u + 3]),
+                  pack_bf16(g[8 * u + 4], g[8 * u + 5]), pack_bf16(g[8 * u + 6], g[8 * u + 7]));
+  }
   fence_proxy_async();
   __syncwarp();
   if (elect_one()) {
@@ -1035,15 +1053,18 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
         const int64_t n = w.n0 + c0;
         if (n >= n_cols || (EPI != kDwT && m_warp >= sched.M)) break;               // warp-uniform
         const int c = (c0 - c_first) >> 5;
+        const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256 + c0);
         uint32_t r[32];
-        tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256 + c0), r);
-        tmem_ld_wait();
+        if (!is_dx(EPI)) {
+          tmem_ld32(taddr, r);
+          tmem_ld_wait();
+        }
         if (EPI == kDwT) {
           // a chunk may reach past the tile's width (bn is a multiple of 16) and past the last kept column
           epilogue_chunk_dwt(p, r, m, n, (int)min((int64_t)min(32, bn - c0), n_cols - n), row_ok, w.split);
         } else if (is_dx(EPI)) {
           const uint32_t bits = c == 0 ? prev_bits[0] : c == 1 ? prev_bits[1] : c == 2 ? prev_bits[2] : prev_bits[3];
-          dx_chunk<EPI == kDxGelu>(p, &tmO, r, (int)m_warp, (int)n, lane, bits, stage + c * kChunkBytes);
+          dx_chunk<EPI == kDxGelu>(&tmO, taddr, (int)m_warp, (int)n, lane, bits, stage + c * kChunkBytes);
         } else {
           uint32_t ab[16];
           const uint32_t bits = forward_chunk<EPI % 3, kSlots>(p, &tmO, &tmL, &tmZ, r, (int)m_warp, (int)n, lane, stage, bias_row + 128 * c, turn++, ab);
