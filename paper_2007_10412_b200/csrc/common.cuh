@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 #include <utility>
 
@@ -421,6 +422,14 @@ __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.
 __device__ __forceinline__ void begin_after_previous() {
   wait_for_previous();
   let_next_start();
+}
+// Shared memory that a launch of `ctas` CTAs asks for so that no SM takes more of them than its share: CTAs that come up
+// early find a few SMs idle beside the kernel before, and without that they share those few.
+constexpr int kNumSms = 148, kSpreadSmemMax = 120 * 1024;
+inline size_t spread_smem(int64_t ctas, size_t needed) {
+  const int64_t per_sm = ceil_div(ctas, kNumSms);
+  const size_t share = per_sm == 1 ? kSpreadSmemMax : per_sm == 2 ? 100 * 1024 : 0;       // one CTA, two CTAs fit
+  return std::max(needed, share);
 }
 // Every caller passes the code on.
 template <typename... P, typename... Args>

@@ -317,3 +317,21 @@ def test_where_the_bias_gradient_is_made(fake):
         assert beside or all("colsum_kernel" in n for n in names[:-1])
         with pytest.raises(b.RadError, match="workspace too small"):
             b.rad_linear_input_grad(dZ, W, dZ_prev=out, db=db, workspace=ws[:-1])
+
+
+@pytest.mark.parametrize("B", [6, 64, 128, 150, 300])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_convolutions_of_few_ctas_spread_over_the_chip(fake, B, dtype):
+    """A CUDA-core convolution of at most one CTA per SM asks for more than half of an SM's shared memory, one of two for more
+    than a third: launched early behind a kernel that leaves SMs idle, its CTAs would otherwise share those."""
+    fake.lib().rad_set_conv_kernel(1)
+    try:
+        fake.lib().fake_reset(-1)
+        _cnn(fake, B, 32, 3, (16, 32, 64), (128, 10), dtype, "different")()
+    finally:
+        fake.lib().rad_set_conv_kernel(0)
+    forward = [l for l in _launches(fake) if "conv_forward_pool_kernel" in l[0]]
+    assert len(forward) == 3
+    for name, gx, gy, gz, bx, by, bz, smem, cluster in forward:
+        per_sm = -(-gx // 148)
+        assert smem <= 227 * 1024 and (per_sm > 2 or (per_sm + 1) * (smem + 1024) > 228 * 1024), (name, gx, smem)
