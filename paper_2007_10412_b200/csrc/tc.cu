@@ -194,7 +194,10 @@ constexpr int kChunkBytes = 32 * 64;             // 32 rows x 32 bf16 columns
 constexpr int kRingBytes = 32 * kChunkBytes;     // chunk buffers of all epilogue warps: four each of eight, two each of sixteen
 constexpr int kFillBuffers = 8;                  // four lane quarters, two tiles of 128 columns
 constexpr int kBiasBytes = 8 * 128 * 4;          // every warp's columns of the bias
-constexpr int kEpiBytes = kRingBytes + kFillBuffers * kFillBytes + kBiasBytes;
+constexpr int kSumBytes = 2 * 8 * 16 * 4;        // every warp's sums of a group of columns (bias gradient), twice
+// What an epilogue takes of the shared memory; the ring of operand stages gets the rest.
+constexpr int fill_bytes(int epi) { return epi >= kFwdFill && epi < kDx ? kFillBuffers * kFillBytes : 0; }
+constexpr int epi_bytes(int epi) { return epi == kDwT ? 0 : kRingBytes + (is_dx(epi) ? kSumBytes : fill_bytes(epi) + kBiasBytes); }
 
 __device__ __forceinline__ uint32_t chunk16_addr(uint32_t base, int row, int unit) { return base + row * 64 + ((unit ^ ((row >> 1) & 3)) << 4); }
 __device__ __forceinline__ uint32_t chunk32_addr(uint32_t base, int row, int unit) { return base + row * 128 + ((unit ^ (row & 7)) << 4); }
@@ -697,8 +700,13 @@ __device__ __forceinline__ void expand_word(uint8_t* sA, const uint8_t* sC, int 
 // both CTAs' TMA complete on it: the odd CTA reloads a stage only after the commit that follows the
 // even CTA's wait on the previous phase, so its bytes never reach an older phase), empty[s] and tmem_full[b] (one per CTA, signalled by the MMA thread's commit to
 // both CTAs), tmem_empty[b] (even CTA; every epilogue warp of the pair arrives).
-constexpr int kStage2Bytes = 2 * 128 * BK * 2;   // 16 KB of A + 16 KB of B per CTA and stage
-constexpr int kStages2 = 4;
+// A stage is 16 KB of A and as much of B as the tile is wide (MN-major: in boxes of 64 columns), and as many stages as there is
+// room for are in flight: narrow tiles of long contractions wait for memory and not for the tensor core.  Us with four stages
+// of 32 KB / so: 32768 x 4096 to 64 columns, input gradient 61.6 / 53.9, same-sample dW, which has no epilogue buffers and
+// whose width only the device knows, 51.6 / 46.9 (16384 x 4096 x 1024: 39.5 / 33.6); forward: see dense_tile_width.
+constexpr int kStage2ABytes = 128 * BK * 2;
+constexpr int kStages2 = 6;
+constexpr int stage2_bytes(int bkind, int bn) { return kStage2ABytes + (bkind == kBK_ ? bn / 2 * BK * 2 : (bn / 2 + 63) / 64 * 8192); }
 // Epilogue warps, eight or sixteen.  Sixteen for a forward pass of up to kWideEpilogueK inputs that places the next layer's store
 // and for a GELU of up to kWideGeluK inputs: more warps hide the latencies of erff and of the stores (a tile of 256 x 256 in us,
 // eight / sixteen: GELU 7.3 / 6.3, with pre-activations and store 10.3 / 9.9, ReLU with store 5.7 / 5.7); with more inputs the
@@ -797,8 +805,9 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
                     const __grid_constant__ CUtensorMap tmZ) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint8_t* epi_smem = smem + (size_t)kStages2 * kStage2Bytes;
-  SmemCtl2* ctl = reinterpret_cast<SmemCtl2*>(epi_smem + kEpiBytes);
+  const int stages = p.num_stages, stage_bytes = stage2_bytes(BKIND, EPI == kDwT ? BN : p.bn);
+  uint8_t* epi_smem = smem + (size_t)stages * stage_bytes;
+  SmemCtl2* ctl = reinterpret_cast<SmemCtl2*>(epi_smem + epi_bytes(EPI));
   volatile int* abort_flag = &ctl->abort_flag;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -810,7 +819,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
     prefetch_map(&tmA);
     prefetch_map(&tmB);
     if (EPI != kDwT) prefetch_map(p.out_z != nullptr ? &tmZ : &tmO);
-    for (int s = 0; s < kStages2; ++s) {
+    for (int s = 0; s < stages; ++s) {
       mbar_init(smem_u32(&ctl->full[s]), 1);
       mbar_init(smem_u32(&ctl->empty[s]), 1);
     }
@@ -852,7 +861,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
   const Schedule sched(p.M, n_cols, p.K, p.splits, BM, bn);
   if (EPI != kDwT) wait_for_previous();
   const int boxes_b = (bn / 2 + 63) / 64;             // 64-column boxes of an MN-major B this CTA stages per K block
-  const uint32_t stage_tx = 2u * (uint32_t)(kStage2Bytes / 2 + (BKIND == kBK_ ? bn / 2 * 128 : boxes_b * 8192));
+  const uint32_t stage_tx = 2u * (uint32_t)(kStage2ABytes + (BKIND == kBK_ ? bn / 2 * 128 : boxes_b * 8192));
 
   if (warp == 0) {
     // ===== TMA producer: this CTA's 128 rows of A and 128 rows (N) of B, completing on the even CTA's barrier =====
@@ -868,8 +877,8 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
         for (int kb = w.kb0; kb < w.kb1; ++kb) {
           ok = mbar_wait2(smem_u32(&ctl->empty[0]) + 8u * stage, phase ^ 1u, wc);
           if (!ok) break;
-          const uint32_t sA = smem_base + stage * kStage2Bytes;
-          const uint32_t sB = sA + kStage2Bytes / 2;
+          const uint32_t sA = smem_base + stage * stage_bytes;
+          const uint32_t sB = sA + kStage2ABytes;
           const uint32_t full = full0 + 8u * stage;
           const int k0 = kb * BK;
           if (rank == 0) mbar_arrive_expect_tx(smem_u32(&ctl->full[0]) + 8u * stage, stage_tx);   // both CTAs' bytes
@@ -886,13 +895,13 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
             for (int c = 0; c < 2; ++c)
               if (c < boxes_b) tma_load_2d_pair(sB + c * 8192, &tmB, n_own + c * 64, k0, full);
           }
-          if (++stage == kStages2) { stage = 0; phase ^= 1u; }
+          if (++stage == stages) { stage = 0; phase ^= 1u; }
         }
       }
       // tail: every commit aimed at this CTA's stage barriers has landed before the CTA may leave
-      for (int i = 0; i < kStages2 && ok; ++i) {
+      for (int i = 0; i < stages && ok; ++i) {
         ok = mbar_wait2(smem_u32(&ctl->empty[0]) + 8u * stage, phase ^ 1u, wc);
-        if (++stage == kStages2) { stage = 0; phase ^= 1u; }
+        if (++stage == stages) { stage = 0; phase ^= 1u; }
       }
     }
     __syncwarp();
@@ -902,8 +911,8 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
       const uint32_t idesc = make_idesc_pair(AK != kAK, BKIND == kBMN, (uint32_t)bn);
       // descriptors of stage 0; a step of 16 K rows and a stage are additions to the address field
       const uint64_t adesc0 = AK == kAK ? make_desc(smem_base, 16, 1024) : make_desc(smem_base, 8192, 1024);
-      const uint64_t bdesc0 = BKIND == kBK_ ? make_desc(smem_base + kStage2Bytes / 2, 16, 1024)
-                                            : make_desc(smem_base + kStage2Bytes / 2, 8192, 1024);
+      const uint64_t bdesc0 = BKIND == kBK_ ? make_desc(smem_base + kStage2ABytes, 16, 1024)
+                                            : make_desc(smem_base + kStage2ABytes, 8192, 1024);
       constexpr uint32_t a_step = (AK == kAK ? 32 : 2048) >> 4, b_step = (BKIND == kBK_ ? 32 : 2048) >> 4;
       int stage = 0, buf = 0;
       uint32_t phase = 0, buf_phases = 0;          // bit b: phase of accumulator b
@@ -917,13 +926,13 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
           ok = mbar_wait2(smem_u32(&ctl->full[0]) + 8u * stage, phase, wc);
           if (!ok) break;
           tc_fence_after();
-          const uint64_t adesc = adesc0 + (uint32_t)(stage * (kStage2Bytes >> 4));
-          const uint64_t bdesc = bdesc0 + (uint32_t)(stage * (kStage2Bytes >> 4));
+          const uint64_t adesc = adesc0 + (uint32_t)(stage * (stage_bytes >> 4));
+          const uint64_t bdesc = bdesc0 + (uint32_t)(stage * (stage_bytes >> 4));
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)
             tc_mma_pair(tmem_base + buf * 256, adesc + k * a_step, bdesc + k * b_step, idesc, (kb > w.kb0 || k > 0) ? 1u : 0u);
           tc_commit_pair(smem_u32(&ctl->empty[0]) + 8u * stage);           // frees the stage in both CTAs
-          if (++stage == kStages2) { stage = 0; phase ^= 1u; }
+          if (++stage == stages) { stage = 0; phase ^= 1u; }
         }
         if (ok) tc_commit_pair(smem_u32(&ctl->tmem_full[0]) + 8u * buf);
         buf_phases ^= 1u << buf;
@@ -942,7 +951,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
     const uint32_t empty_bar = map_to_cta(smem_u32(&ctl->tmem_empty[0]), 0u);     // [b] is 8 bytes further
     constexpr int kSlots = 32 / kEpiWarps;
     const uint32_t stage = smem_u32(epi_smem) + (warp - 2) * kSlots * kChunkBytes;
-    const uint32_t bias_row = smem_u32(epi_smem) + kRingBytes + kFillBuffers * kFillBytes + (warp - 2) * (kBiasBytes / kEpiWarps);
+    const uint32_t bias_row = smem_u32(epi_smem) + kRingBytes + fill_bytes(EPI) + (warp - 2) * (kBiasBytes / kEpiWarps);
     // the warps of a lane quarter whose columns make up one store tile fill one buffer and copy it out together
     const bool whole_tile = bn >= 128;
     const int group = whole_tile ? 4 / own_chunks : 1, first_tile = ((warp - 2) >> 2) / group;
@@ -1576,7 +1585,7 @@ int planning_pairs() {
 }
 
 DwPlan plan_dw(const rad_store* st, int64_t H) {
-  DwPlan d;
+  DwPlan d = {};
   const int64_t kblocks = ceil_div(st->B, BK);
   int64_t m_expect;
   if (st->variant == RAD_SAME_SAMPLE) {
@@ -1616,16 +1625,18 @@ DwPlan plan_dw(const rad_store* st, int64_t H) {
 struct OutMaps { CUtensorMap o, l, z; };      // see tc_gemm_pair_kernel; those of absent outputs are not written through
 
 template <int AK, int BKIND, int EPI, int kEpiWarps = 8>
-int launch_pair(const TcParams& p, const CUtensorMap& ta, const CUtensorMap& tb, const OutMaps& out, int64_t max_units, cudaStream_t s) {
-  constexpr size_t smem = (size_t)kStages2 * kStage2Bytes + kEpiBytes + sizeof(SmemCtl2) + 1024;
-  static_assert(smem <= 227 * 1024, "stage ring too deep");
+int launch_pair(const TcParams& params, const CUtensorMap& ta, const CUtensorMap& tb, const OutMaps& out, int64_t max_units, cudaStream_t s) {
+  TcParams p = params;
+  const int stage = stage2_bytes(BKIND, EPI == kDwT ? BN : p.bn), rest = epi_bytes(EPI) + (int)sizeof(SmemCtl2) + 1024;
+  p.num_stages = std::min(kStages2, (227 * 1024 - rest) / stage);
+  const size_t smem = (size_t)p.num_stages * stage + rest;
   auto kernel = tc_gemm_pair_kernel<AK, BKIND, EPI, kEpiWarps>;
   // The kernel is persistent: the grid must not exceed the clusters that can be resident at once
   // (SM pairs that can host a cluster; fewer than half the SM count on some parts).
   static int resident_pairs = 0;
   if (resident_pairs == 0) {
-    RAD_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    resident_pairs = resident_pairs_of(kernel, threads2(kEpiWarps), smem);
+    RAD_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    resident_pairs = resident_pairs_of(kernel, threads2(kEpiWarps), 227 * 1024);
   }
   const int pairs = (int)std::max<int64_t>(1, std::min<int64_t>(max_units, resident_pairs));
   count_launch();
@@ -1653,10 +1664,12 @@ int launch_sparse_pair(const TcParams& p, const CUtensorMap& tb, int64_t max_uni
 // its loads 0.17 to 0.2: within a wave a narrower tile is no slower there and spreads loads and epilogues over more SMs
 // (2048 x 1024 x 1024 forward with store: 21.8 / 16.9 / 22.0 us at 256 / 128 / 64 columns, which are 32 / 64 / 128 tiles on
 // 74 pairs), a second wave costs most of the contraction again (4096 x 1024 x 1024: 22.2 / 25.0 / 36.1; both before the
-// single-thread roles were elected).
-int dense_tile_width(int64_t M, int64_t N) {
+// single-thread roles were elected).  A tile is no wider than the matrix needs either, or its stages are few and half empty (forward
+// of 32768 x 4096 to 64 columns: 64.5 us in tiles of 256 columns and four stages, 49.2 now), but at least 128 where a store is filled, whose
+// entries are staged by tiles of that width.
+int dense_tile_width(int64_t M, int64_t N, int least = 64) {
   for (int bn = 64; bn < BN; bn *= 2)
-    if (ceil_div(M, BM) * ceil_div(N, bn) <= planning_pairs()) return bn;
+    if (ceil_div(M, BM) * ceil_div(N, bn) <= planning_pairs() || (N <= bn && bn >= least)) return bn;
   return BN;
 }
 
@@ -1687,7 +1700,7 @@ int tc_forward(int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t 
   rc = make_map(&tb, W, H, D, ldw, 64);               // MN-major B: box 64 (N) x 64 K rows
   if (rc != RAD_OK) return rc;
   TcParams p = {};
-  p.M = B; p.N = H; p.K = D; p.splits = 1; p.num_stages = 3; p.bn = dense_tile_width(B, H);
+  p.M = B; p.N = H; p.K = D; p.splits = 1; p.bn = dense_tile_width(B, H, next != nullptr ? 128 : 64);
   p.bias = bias; p.act = act;
   p.out_act = static_cast<bf16*>(out_act); p.ld_act = ld_act; p.out_z = out_z; p.ld_z = ld_z;
   p.out_zlow = static_cast<bf16*>(out_zlow); p.ld_zlow = ld_zlow; p.relubits = relubits; p.w32 = ceil_div(H, 32);
@@ -1756,7 +1769,7 @@ int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, 
   rc = make_map(&tb, W, H, D, ldw, bn / 2);           // K-major B: rows d (N), K = H contiguous
   if (rc != RAD_OK) return rc;
   TcParams p = {};
-  p.M = B; p.N = D; p.K = H; p.splits = 1; p.num_stages = 3; p.bn = bn;
+  p.M = B; p.N = D; p.K = H; p.splits = 1; p.bn = bn;
   p.relubits_prev = relubits_prev; p.z_prev = static_cast<const bf16*>(z_prev); p.ld_zprev = ld_zprev;
   p.out_dx = static_cast<bf16*>(dZ_prev); p.ld_dx = ldp;
   p.dz = static_cast<const bf16*>(dZ); p.ld_dz = ldz; p.db = db;

@@ -287,6 +287,21 @@ def test_dense_tile_widths(B, D, H, fwd_width, dx_width, act):
     import paper_2007_10412_b200 as rad
     pairs = rad.rad_sm_pairs()
     assert dense_tile_width(B, H, pairs) == fwd_width and dense_tile_width(B, D, pairs) == dx_width
+    _check_dense(B, D, H, act)
+
+
+@pytest.mark.parametrize("B,D,H", [(20000, 200, 64), (19500, 128, 72), (20001, 72, 128), (38000, 64, 64)])
+@pytest.mark.parametrize("act", ["relu", "gelu"])
+def test_narrow_outputs_of_many_rows(B, D, H, act):
+    """More tiles than SM pairs in one column of tiles, of 64 or 128 columns as the matrix needs and of 128 where a store is
+    filled: the same checks as for the other tile widths."""
+    import paper_2007_10412_b200 as rad
+    assert -(-B // 256) > rad.rad_sm_pairs()
+    _check_dense(B, D, H, act)
+
+
+def _check_dense(B, D, H, act):
+    import paper_2007_10412_b200 as rad
     bf = torch.bfloat16
     g = torch.Generator(device="cuda").manual_seed(B + D + H)
     rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").to(bf)

@@ -335,3 +335,32 @@ def test_convolutions_of_few_ctas_spread_over_the_chip(fake, B, dtype):
     for name, gx, gy, gz, bx, by, bz, smem, cluster in forward:
         per_sm = -(-gx // 148)
         assert smem <= 227 * 1024 and (per_sm > 2 or (per_sm + 1) * (smem + 1024) > 228 * 1024), (name, gx, smem)
+
+
+def test_stages_of_the_dense_kernels(fake):
+    """The ring of operand stages takes what the epilogue leaves of the shared memory, up to six stages, and a stage is no wider
+    than the tile: (stages, bytes of one, bytes of the epilogue's buffers)."""
+    b, bf, MB, ring = fake, torch.bfloat16, 32768, 32 * 2048
+    T = lambda *s: torch.empty(*s, dtype=bf)
+
+    def smem(call):
+        b.lib().fake_reset(-1)
+        call()
+        (l,) = [l for l in _launches(b) if _pair_kernel(l[0])]
+        return l[7]
+    bias, fill = 4096, 8 * 3584
+    for D, H, with_store, stages, stage, epilogue in ((4096, 64, False, 6, 24576, ring + bias), (4096, 128, False, 6, 24576, ring + bias),
+                                                      (4096, 512, False, 4, 32768, ring + bias), (4096, 64, True, 5, 24576, ring + bias + fill),
+                                                      (4096, 512, True, 4, 32768, ring + bias + fill)):
+        if with_store:
+            got = smem(lambda: b.rad_linear_forward_fill(T(MB, D), T(D, H), None, "relu", T(MB, H), _store(b, "different", "bf16", MB, H)))
+        else:
+            got = smem(lambda: b.rad_linear_forward(T(MB, D), T(D, H), None, "relu", out_act=T(MB, H)))
+        assert 1024 < got - stages * stage - epilogue < 2048 and got <= 227 * 1024, (D, H, with_store, got)
+    for D, stages, stage in ((64, 6, 20480), (128, 6, 24576), (512, 5, 32768)):
+        got = smem(lambda: b.rad_linear_input_grad(T(MB, 4096), T(D, 4096), dZ_prev=T(MB, D)))
+        assert 1024 < got - stages * stage - ring - 1024 < 2048 and got <= 227 * 1024, (D, got)
+    same = _store(b, "same", "bf16", 4096, 512, relu_bits=False)
+    ws = _aligned(max(256, b.rad_weight_grad_workspace(same, 256)))
+    got = smem(lambda: b.rad_linear_weight_grad(same, T(4096, 256), torch.empty(512, 256), ws))
+    assert 1024 < got - 6 * 32768 < 2048
