@@ -31,8 +31,9 @@ struct IndexLayer {
   int64_t capacity;     // elements of `values` the caller holds; < 0: not checked
 };
 constexpr int kIndexLayers = 16;   // layers of one launch
+template <int kLayers>
 struct IndexParams {
-  IndexLayer layer[kIndexLayers];
+  IndexLayer layer[kLayers];
   int32_t nlayers;
   uint32_t ntiles;      // of all of them
   KeepThreshold T;
@@ -82,18 +83,21 @@ __device__ __forceinline__ void write_totals(const IndexLayer& L, uint32_t padde
 }
 
 constexpr int kIndexWarps = 16;
-constexpr int kIndexSmemOne = 120 * 1024, kIndexSmemTwo = 100 * 1024;     // asked for so that one or two CTAs fit an SM
-__global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const __grid_constant__ IndexParams p, const PhiloxKeys ks) {
+// (One layer has a form of its own: fewer registers, 65536 tiles 160 us instead of 163.)
+template <int kLayers>
+__global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const __grid_constant__ IndexParams<kLayers> p, const PhiloxKeys ks) {
   wait_for_previous();
   const int lane = threadIdx.x & 31;
-  const uint32_t warp0 = blockIdx.x * kIndexWarps + (threadIdx.x >> 5), nwarps = gridDim.x * kIndexWarps;
+  const uint32_t warps = blockDim.x >> 5, warp0 = blockIdx.x * warps + (threadIdx.x >> 5), nwarps = gridDim.x * warps;
   int l = 0;
+  IndexLayer layer = p.layer[0];                    // in registers: out of the parameters by a variable index, every use would be a load
   for (uint32_t t = warp0; t < p.ntiles; t += nwarps) {
     if ((uint64_t)t + nwarps >= p.ntiles) let_next_start();
-    while (l + 1 < p.nlayers && t >= p.layer[l + 1].tile0) ++l;
-    const uint32_t tile = t - p.layer[l].tile0;
-    const uint32_t count = index_tile(p.layer[l], tile, p.T, p.c3, ks, lane);
-    if (lane == 0) p.layer[l].offsets[tile] = count;
+    if (kLayers > 1)
+      while (l + 1 < p.nlayers && t >= p.layer[l + 1].tile0) layer = p.layer[++l];
+    const uint32_t tile = t - layer.tile0;
+    const uint32_t count = index_tile(layer, tile, p.T, p.c3, ks, lane);
+    if (lane == 0) layer.offsets[tile] = count;
   }
 }
 
@@ -102,7 +106,7 @@ __global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const __g
 // 640-520-392-200 net at batch 328 took 20 us of its step, in one launch for all of them 6.  An SM draws a tile in 0.26 us (three generator calls per word, 3 G calls/s), so with
 // more than twelve tiles a CTA the two launches of the general form, on all SMs, are faster.
 constexpr int kSmallIndexCtas = 8, kSmallIndexTiles = 12 * kSmallIndexCtas;
-__global__ void __launch_bounds__(32 * kIndexWarps) store_index_small_kernel(const __grid_constant__ IndexParams p, const PhiloxKeys ks) {
+__global__ void __launch_bounds__(32 * kIndexWarps) store_index_small_kernel(const __grid_constant__ IndexParams<kIndexLayers> p, const PhiloxKeys ks) {
   cluster_started_arrive();                             // waited for behind the draw
   begin_after_previous();
   __shared__ uint32_t s_count[kSmallIndexTiles / kSmallIndexCtas];
@@ -147,9 +151,10 @@ __global__ void __launch_bounds__(32 * kIndexWarps) store_index_small_kernel(con
 // tiles per round; a thread takes 16 consecutive tiles (four 16-byte loads and stores where `offsets` is
 // 16-byte aligned), adds them up locally, and one warp scan plus one pass over the warp sums places them.
 constexpr int kScanPer = 16;
-__global__ void __launch_bounds__(1024) offsets_scan_kernel(const __grid_constant__ IndexParams p) {
+template <int kLayers>
+__global__ void __launch_bounds__(1024) offsets_scan_kernel(const __grid_constant__ IndexParams<kLayers> p) {
   begin_after_previous();
-  const IndexLayer& L = p.layer[blockIdx.x];
+  const IndexLayer L = p.layer[kLayers > 1 ? blockIdx.x : 0];
   uint32_t* offsets = L.offsets;
   const bool vec = ((uintptr_t)offsets & 15) == 0;
   __shared__ uint64_t s_warp[32];                   // padded sum in the high half, exact sum in the low half
@@ -224,20 +229,40 @@ __global__ void __launch_bounds__(1024) offsets_scan_kernel(const __grid_constan
 // Exact kept counts per tile in offsets[0 .. ntiles) -> padded exclusive prefixes, offsets[ntiles] and nnz.
 int launch_offsets_scan(uint32_t* offsets, int64_t ntiles, int64_t* nnz, int64_t capacity, int32_t* dev_status,
                         cudaStream_t s) {
-  IndexParams p = {};
+  IndexParams<1> p = {};
   p.nlayers = 1; p.dev_status = dev_status;
   p.layer[0].ntiles = (uint32_t)ntiles; p.layer[0].offsets = offsets; p.layer[0].nnz = nnz; p.layer[0].capacity = capacity;
   count_launch();
-  RAD_TRY(launch_kernel(offsets_scan_kernel, 1, 1024, 0, s, p));
-  return RAD_OK;
+  return launch_kernel(offsets_scan_kernel<1>, 1, 1024, 0, s, p);
 }
+
+namespace {
+// Up to kLayers layers of one seed, step and keep probability: the general form.
+template <int kLayers>
+int launch_index_tiles(const IndexParams<kLayers>& p, const PhiloxKeys& ks, cudaStream_t s) {
+  // Tiles spread over all SMs: an SM draws one in 0.26 us, so 256 tiles are for 64 SMs and not for sixteen (7.7 us with the scan
+  // instead of 10.6).  Up to sixteen tiles an SM one CTA of as many warps as that takes, at least four, and the shared memory
+  // says so: started early beside a tensor-core kernel that leaves a few SMs idle, CTAs without that share those few (1024
+  // tiles behind an input gradient on 128 of 148 SMs: 12.5 us, 6 otherwise).  More tiles: CTAs of four warps (8192 tiles 23.4 us,
+  // 25.4 with five of eight an SM), and of eight where every warp has several (16384 tiles 41.1 us, 43.3 with four).
+  static std::atomic<uint64_t> ready{0};
+  if (!allow_smem(store_index_kernel<kLayers>, kSpreadSmemMax, ready)) return RAD_ECUDA;
+  const int64_t per_sm = ceil_div(p.ntiles, kNumSms);
+  const int warps = per_sm <= 4 ? 4 : per_sm <= 8 ? 8 : per_sm <= kIndexWarps ? kIndexWarps : per_sm <= 64 ? 4 : 8;
+  const int64_t most = (per_sm <= kIndexWarps ? 1 : per_sm <= 64 ? 12 : 5) * kNumSms, ctas = std::min(ceil_div(p.ntiles, warps), most);
+  count_launch();
+  RAD_TRY(launch_kernel(store_index_kernel<kLayers>, (unsigned)ctas, 32 * warps, spread_smem(ctas, 0), s, p, ks));
+  count_launch();
+  return launch_kernel(offsets_scan_kernel<kLayers>, p.nlayers, 1024, 0, s, p);
+}
+}  // namespace
 
 // Index parts (keep bits, row offsets, tile offsets, nnz) of the different-sample Bernoulli stores of one net: one seed,
 // step and keep probability.
 int launch_store_indices(const rad_store* st, int n, bool check_capacity, int32_t* dev_status, cudaStream_t s) {
   const PhiloxKeys ks = philox_expand_key(st[0].seed);
   for (int first = 0; first < n; first += kIndexLayers) {
-    IndexParams p = {};
+    IndexParams<kIndexLayers> p = {};
     p.nlayers = std::min(n - first, kIndexLayers);
     p.T = make_keep_threshold(keep_threshold_host(st[0].p));
     p.c3 = st[0].step;
@@ -256,22 +281,15 @@ int launch_store_indices(const rad_store* st, int n, bool check_capacity, int32_
       p.ntiles += L.ntiles;
       small = small && L.ntiles <= (uint32_t)kSmallIndexTiles;
     }
-    count_launch();
     if (small) {
+      count_launch();
       RAD_TRY(launch_with_cluster(store_index_small_kernel, p.nlayers * kSmallIndexCtas, 32 * kIndexWarps, 0, dim3(kSmallIndexCtas, 1, 1),
                                   s, p, ks));
-      continue;
+    } else if (p.nlayers == 1) {
+      RAD_TRY(launch_index_tiles(IndexParams<1>{{p.layer[0]}, 1, p.ntiles, p.T, p.c3, p.dev_status}, ks, s));
+    } else {
+      RAD_TRY(launch_index_tiles(p, ks, s));
     }
-    // One CTA of sixteen warps on every SM, two where there are tiles for them, and the shared memory says so: started early
-    // beside a tensor-core kernel that leaves a few SMs idle, CTAs without that share those few (1024 tiles behind an
-    // input gradient on 128 of 148 SMs: 12.5 us, 6 otherwise).
-    static std::atomic<uint64_t> ready{0};
-    const int64_t ctas = ceil_div(p.ntiles, kIndexWarps);
-    if (!allow_smem(store_index_kernel, kIndexSmemOne, ready)) return RAD_ECUDA;
-    RAD_TRY(launch_kernel(store_index_kernel, (unsigned)std::min<int64_t>(ctas, 2 * 148), 32 * kIndexWarps,
-                          ctas <= 148 ? kIndexSmemOne : kIndexSmemTwo, s, p, ks));
-    count_launch();
-    RAD_TRY(launch_kernel(offsets_scan_kernel, p.nlayers, 1024, 0, s, p));
   }
   return RAD_OK;
 }

@@ -35,6 +35,27 @@ def test_index_from_the_key_alone_is_bit_exact(B, D, p):
     assert nnz[0] == ref.nnz and nnz[1] == offs[-1]
 
 
+@pytest.mark.parametrize("B,D", [(449, 128), (64, 1100), (700, 200), (5640, 120), (768, 1024), (6200, 120), (2500, 2060)])
+def test_index_of_as_many_tiles_as_a_cluster_makes_and_of_one_more(B, D):
+    """One cluster of eight CTAs with 8, 9, 22, 89 and 96 tiles (ranks without tiles, with a part of their share, with the most they
+    hold), and the general form with 97 and 680: everything an index has is the oracle's, bit for bit."""
+    import paper_2007_10412_b200 as rad
+    seed, layer, step, p = (5 << 32) + 3, 2, 11, 0.2
+    ref = orc.forward_store(np.ones((B, D), np.float32), "f32", "different", p, seed, layer, step, with_relu_bits=False)
+    st = rad.Store("different", "f32", B, D, p, seed=seed, layer=layer, step=step, relu_bits=False)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for _ in range(3):
+        st.keepbits.fill_(-1)
+        st.offsets.fill_(-1)
+        rad.rad_store_index(st, status)
+        torch.cuda.synchronize()
+        assert status.item() == 0
+        kb, _, offs = tile_major(ref)
+        assert np.array_equal(u32(st.keepbits), kb) and np.array_equal(u32(st.offsets), offs)
+        nnz = st.nnz.cpu().numpy()
+        assert nnz[0] == ref.nnz and nnz[1] == offs[-1]
+
+
 def test_index_reports_a_short_values_buffer_and_rejects_other_variants():
     import paper_2007_10412_b200 as rad
     st = rad.Store("different", "bf16", 300, 512, 0.5, capacity=1024)

@@ -189,9 +189,11 @@ def test_small_net_step_equals_the_layer_calls_and_counts_its_launches(name, var
 
 
 @pytest.mark.parametrize("dims,B,dtype", [((32,) * 18 + (8,), 40, "f32"), ((1024, 1152, 8), 768, "f32"), ((1152, 1024, 64), 768, "bf16"),
-                                          ((384, 200, 16), 4100, "f32"), ((96, 72, 64, 64), 65, "bf16")])
+                                          ((384, 200, 16), 4100, "f32"), ((96, 72, 64, 64), 65, "bf16"),
+                                          ((1024, 1000, 8), 768, "f32"), ((120, 128, 8), 5640, "f32"), ((520, 264, 1024, 64), 768, "bf16")])
 def test_indices_of_all_layers_in_one_go(dims, B, dtype):
-    """More layers than one launch takes, layers of 96 tiles (the most that one cluster makes) and more, tiles with remainders:
+    """More layers than one launch takes; nets whose largest layer has 96 tiles (the most that one cluster makes, so that all
+    layers take that form), 89, and more (then none does); tiles with remainders:
     kept counts of every layer are the oracle's, and so is the gradient that is formed from the stores."""
     import paper_2007_10412_b200 as rad
     X, y, Ws, bs = mlp_inputs(dims, B, dtype, "normal", seed=len(dims) + B, bias_zero=False)

@@ -364,3 +364,23 @@ def test_stages_of_the_dense_kernels(fake):
     ws = _aligned(max(256, b.rad_weight_grad_workspace(same, 256)))
     got = smem(lambda: b.rad_linear_weight_grad(same, T(4096, 256), torch.empty(512, 256), ws))
     assert 1024 < got - 6 * 32768 < 2048
+
+
+@pytest.mark.parametrize("B,D,tiles", [(64, 128, 1), (768, 1024, 96), (6200, 120, 97), (2048, 1024, 256), (8192, 1024, 1024), (4096, 4096, 2048),
+                                       (8192, 8192, 8192), (16384, 8192, 16384)])
+def test_tiles_of_an_index_are_spread_over_the_chip(fake, B, D, tiles):
+    """Up to 96 tiles one cluster; then as many CTAs as leave no SM with more tiles than its share (rounded up to four, eight or
+    sixteen), each with more than half of an SM's shared memory where there are at most as many as SMs."""
+    b = fake
+    st = _store(b, "different", "bf16", B, D, relu_bits=False)
+    b.lib().fake_reset(-1)
+    b.rad_store_index(st)
+    first, *rest = _launches(b)
+    if tiles <= 96:
+        assert "store_index_small_kernel" in first[0] and first[1] == first[8] == 8 and not rest
+        return
+    assert "store_index_kernel" in first[0] and len(rest) == 1 and "offsets_scan_kernel" in rest[0][0]
+    ctas, warps, share = first[1], first[4] // 32, -(-tiles // 148)
+    assert warps == next((w for w in (4, 8, 16) if share <= w), 4 if share <= 64 else 8)
+    assert ctas == (-(-tiles // warps) if share <= 16 else min(-(-tiles // warps), 148 * (12 if share <= 64 else 5)))
+    assert share > 16 or 2 * first[7] > 228 * 1024
