@@ -167,3 +167,26 @@ def test_pipelined_kernel_reports_a_short_values_buffer():
         rad.rad_set_store_kernel(prev)
     assert status.item() == 1                     # RAD_DEV_ECAPACITY
     assert st.nnz.cpu().numpy()[0] == ref.nnz
+
+
+@pytest.mark.parametrize("B,D,dtype", [(40000, 31, "bf16"), (13001, 72, "bf16"), (14001, 72, "bf16"), (3400, 384, "bf16"), (3400, 385, "bf16"),
+                                       (65536, 1, "f32"), (32001, 33, "f32"), (33001, 33, "f32"), (17000, 128, "f32"), (13200, 129, "f32"), (7, 40, "f32")])
+def test_relu_bits_of_narrow_rows(B, D, dtype):
+    """The bits beside a same-sample store, by a thread per word (many narrow rows) and by a lane per column (the others), on
+    either side of the lines between them, with words that end inside a row, NaN, infinities and zeros of both signs."""
+    import paper_2007_10412_b200 as rad
+    g = torch.Generator(device="cuda").manual_seed(B + D)
+    A = torch.randn(B, D, generator=g, device="cuda")
+    A.view(-1)[::7] = 0.0
+    for i, v in enumerate((-0.0, float("nan"), float("inf"), -float("inf"))):
+        A.view(-1)[3 + i::29] = v
+    A = A.to(torch.float32 if dtype == "f32" else torch.bfloat16)
+    st = rad.Store("same", dtype, B, D, 0.5, relu_bits=True)
+    st.relubits.fill_(-1)
+    rad.rad_linear_forward_store(A, st)
+    torch.cuda.synchronize()
+    w32 = (D + 31) // 32
+    bits = torch.zeros(B, w32 * 32, dtype=torch.int64, device="cuda")
+    bits[:, :D] = A > 0
+    want = (bits.view(B, w32, 32) << torch.arange(32, device="cuda")).sum(2)
+    assert torch.equal(st.relubits.view(B, w32).long() & 0xffffffff, want)

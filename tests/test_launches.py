@@ -384,3 +384,16 @@ def test_tiles_of_an_index_are_spread_over_the_chip(fake, B, D, tiles):
     assert warps == next((w for w in (4, 8, 16) if share <= w), 4 if share <= 64 else 8)
     assert ctas == (-(-tiles // warps) if share <= 16 else min(-(-tiles // warps), 148 * (12 if share <= 64 else 5)))
     assert share > 16 or 2 * first[7] > 228 * 1024
+
+
+@pytest.mark.parametrize("B,D,dtype,thread", [(40000, 31, "bf16", True), (13001, 72, "bf16", False), (14001, 72, "bf16", True), (3400, 384, "bf16", None),
+                                              (3400, 383, "bf16", True), (3400, 385, "bf16", False), (65536, 1, "f32", True), (32001, 33, "f32", False),
+                                              (33001, 33, "f32", True), (17000, 127, "f32", True), (13200, 129, "f32", False), (7, 40, "f32", False)])
+def test_form_of_the_relu_bits(fake, B, D, dtype, thread):
+    """A thread per word for many narrow rows, a lane per column for the others; rows that the store's own kernel stages take
+    neither."""
+    st = _store(fake, "same", dtype, B, D)
+    fake.lib().fake_reset(-1)
+    fake.rad_linear_forward_store(torch.empty(B, D, dtype=torch.float32 if dtype == "f32" else torch.bfloat16), st)
+    names = [l[0] for l in _launches(fake) if "relu_bits" in l[0]]
+    assert [("thread" in n) for n in names] == ([] if thread is None else [thread])
