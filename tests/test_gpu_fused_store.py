@@ -159,3 +159,27 @@ def test_fused_store_reports_a_short_values_buffer():
     assert status.item() == rad.RAD_DEV_ECAPACITY
     assert (guard == 7.0).all()
     assert st.nnz.cpu().numpy()[0] == orc.keep_mask("different", B, H, p, 0, 0, 0).sum()
+
+
+@pytest.mark.parametrize("capacity", [8, 4096, 4101, 9003])
+@pytest.mark.parametrize("D", [256, 2304])                       # sixteen epilogue warps, eight
+def test_staged_entries_stop_at_the_capacity(capacity, D):
+    """A store sparse enough for its entries to go through shared memory (p = 0.1), into a buffer that is too short, at places
+    that end inside a 16-byte piece as well: what fits is the full store's, what lies behind the buffer stays as it was."""
+    import paper_2007_10412_b200 as rad
+    B, H, p = 328, 512, 0.1
+    X, _, Ws, bs = mlp_inputs((D, H), B, dtype="bf16", x_dist="normal", seed=3)
+    args = to_dev(X, "bf16"), to_dev(Ws[0], "bf16"), to_dev(bs[0], "f32"), "relu"
+    out_act = torch.empty(B, H, dtype=torch.bfloat16, device="cuda")
+    full = rad.Store("different", "bf16", B, H, p, relu_bits=False)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rad.rad_linear_forward_fill(*args, out_act, full, dev_status=status)
+    torch.cuda.synchronize()
+    assert status.item() == 0 and int(full.nnz[1]) > 2 * capacity - 8192
+    short = rad.Store("different", "bf16", B, H, p, relu_bits=False)
+    room = torch.full((capacity + 4096,), 7.0, dtype=torch.bfloat16, device="cuda")
+    short.c.values, short.c.values_capacity = room.data_ptr(), capacity
+    rad.rad_linear_forward_fill(*args, out_act, short, dev_status=status)
+    torch.cuda.synchronize()
+    assert status.item() == rad.RAD_DEV_ECAPACITY
+    assert torch.equal(room[:capacity], full.values[:capacity]) and (room[capacity:] == 7.0).all()

@@ -337,7 +337,7 @@ def _check_dense(B, D, H, act):
 
 @pytest.mark.parametrize("B", [40, 130, 640])
 def test_different_sample_dw_of_several_units_per_sm_pair(B):
-    """dW of 4000 x 4104 from a different-sample store: 144 tiles of 256 x 512 on at most 74 SM pairs, with one K block per tile
+    """dW of 4000 x 4104 from a different-sample store: 144 tiles of 256 x 512 or 272 half as wide on at most 74 SM pairs, with one K block per tile
     (the expanders run several tiles ahead of the epilogue), a few, and more than the ring of stages holds; tiles that
     reach past either edge.  Against float64; the bound is that of a float32 sum of B products in any order."""
     import paper_2007_10412_b200 as rad
@@ -478,8 +478,30 @@ def test_gelu_derivative_is_the_same_function_on_both_routes(D, ldp):
 @pytest.mark.parametrize("B,D,H", [(64, 64, 64), (328, 264, 136), (1000, 520, 264), (4160, 256, 264), (1024, 2048, 2040), (70, 1032, 520)])
 @pytest.mark.parametrize("p", [0.1, 0.7])
 def test_different_sample_dw_over_tile_widths(B, D, H, p):
-    """dW from a different-sample store in tiles of 128, 256 and 512 columns, with and without K splits, with rows and columns
-    that end inside a tile.  Against float64: the sum of B products in any order."""
+    """dW from a different-sample store of few and of many tiles, sparse and dense, with rows and columns that end inside a tile."""
+    _check_dw(B, D, H, p)
+
+
+DW_TILES = [
+    # B, D, H, p, columns of a tile, K splits
+    (328, 264, 136, 0.1, 128, 6),
+    (200, 520, 136, 0.1, 128, 1),
+    (200, 2056, 1032, 0.1, 256, 1),
+    (700, 264, 1544, 0.7, 256, 4),
+    (200, 2056, 2056, 0.1, 512, 1),
+    (4096, 2040, 2040, 0.1, 512, 2),
+    (1500, 520, 2056, 0.7, 512, 4),
+]
+
+
+@pytest.mark.parametrize("B,D,H,p", [c[:4] for c in DW_TILES])
+def test_different_sample_dw_at_every_tile_width_and_split(B, D, H, p):
+    """Tiles of 128, 256 and 512 columns, each with and without a split of the rows, none a whole number of tiles."""
+    _check_dw(B, D, H, p)
+
+
+def _check_dw(B, D, H, p):
+    """Against float64: the sum of B products in any order."""
     import paper_2007_10412_b200 as rad
     bf = torch.bfloat16
     g = torch.Generator(device="cuda").manual_seed(B + D + H)

@@ -397,3 +397,22 @@ def test_form_of_the_relu_bits(fake, B, D, dtype, thread):
     fake.rad_linear_forward_store(torch.empty(B, D, dtype=torch.float32 if dtype == "f32" else torch.bfloat16), st)
     names = [l[0] for l in _launches(fake) if "relu_bits" in l[0]]
     assert [("thread" in n) for n in names] == ([] if thread is None else [thread])
+
+
+def test_tiles_of_the_different_sample_weight_gradient(fake):
+    """The tile widths and splits that the parity test claims to cover are those of the launches: pairs of CTAs, partial tiles
+    in the workspace, and a second launch where there are any."""
+    from test_gpu_layer import DW_TILES
+    b, bf = fake, torch.bfloat16
+    for B, D, H, p, cols, splits in DW_TILES:
+        st = _store(b, "different", "bf16", B, D, p=p, relu_bits=False)
+        need = b.rad_weight_grad_workspace(st, H)
+        rows = -(-D // 256) * 256
+        assert need == (-(-splits * rows * H * 4 // 256) * 256 if splits > 1 else 0), (B, D, H, need)
+        b.lib().fake_reset(-1)
+        b.rad_linear_weight_grad(st, torch.empty(B, H, dtype=bf), torch.empty(D, H), _aligned(max(need, 256)))
+        launches = _launches(b)
+        units = {w: -(-D // 256) * -(-H // w) * splits for w in (128, 256, 512)}
+        assert "tc_sparse_pair_kernel" in launches[0][0] and len(launches) == (2 if splits > 1 else 1)
+        assert units[cols] <= 74 and [w for w in units if 2 * min(units[w], 74) == launches[0][1]] == [cols]
+    assert {(c[4], c[5] > 1) for c in DW_TILES} == {(w, s) for w in (128, 256, 512) for s in (False, True)}
