@@ -10,12 +10,14 @@
 // thread of the even CTA issuing tcgen05.mma.cta_group::2 on operands that both CTAs stage in their
 // own shared memory (TMA, 128-byte swizzle, no multicast) through an mbarrier ring.
 //   dense kernels    256 x 256 tile per pair, or 128 or 64 columns wide where that makes one wave of
-//                    them; each CTA keeps two alternating 128 x 256 float32
+//                    them or the matrix has no more; each CTA keeps two alternating 128 x 256 float32
 //                    accumulators in tensor memory, so the epilogue of a tile (bias, activation,
 //                    ReLU bits, GELU', TMA stores) runs under the MMAs of the next one.  The input
-//                    gradient's epilogue warps make the bias gradient while they wait.
-//   sparse-A kernel  256 x 512 tile per pair (256 or 128 columns where 512 would leave SMs idle); sixteen "expander" warps per CTA write the A_hat
-//                    tile of each K block into shared memory instead of TMA.
+//                    gradient's epilogue warps make the bias gradient while they wait, where the
+//                    K blocks of the tiles hide it.
+//   sparse-A kernel  256 x 512 tile per pair (256 or 128 columns where 512 would leave SMs idle);
+//                    sixteen "expander" warps per CTA write the A_hat tile of each K block into
+//                    shared memory instead of TMA.
 // Long dW contractions can be split along K; partial tiles are summed in split order by a second
 // kernel, so results are reproducible.
 // Every mbarrier wait is bounded: on expiry both CTAs of the pair raise their abort flags, all
@@ -49,21 +51,21 @@ struct TcParams {
   int64_t M, N, K;
   const int64_t* N_dev;      // same-sample dW: N = number of kept columns, read on the device
   const uint32_t* keep_cols; // same-sample dW: bit d set = column d of the layer input was kept
-  int32_t bn;                // dense forward and input gradient: columns of an output tile (64, 128 or 256)
+  int32_t bn;                // columns of an output tile (forward, input gradient: 64, 128 or 256; sparse A: 128, 256 or 512)
   int32_t splits;            // K splits (1: epilogue writes final results)
-  int32_t num_stages;
+  int32_t num_stages;        // of the ring of operand stages
   int32_t comp_depth;        // sparse A: depth of the ring of compressed (index + values) buffers
   // sparse A (different-sample store)
   const bf16* values; const uint32_t* keepbits; const uint32_t* offsets;
   int64_t values_capacity; int32_t ncb; int32_t comp_cap;   // comp_cap: value bytes per half-stage
   // forward epilogue
-  const float* bias; int32_t act;
-  bf16* out_act; int64_t ld_act; float* out_z; int64_t ld_z; bf16* out_zlow; int64_t ld_zlow;
+  const float* bias;
+  const bf16* out_act; const float* out_z; const bf16* out_zlow;    // null: not asked for (written through their tensor maps)
   uint32_t* relubits; int64_t w32;
   // forward epilogue that also fills the next layer's store (index part already in place)
   bf16* st_values; const uint32_t* st_keepbits; const uint32_t* st_offsets; int64_t st_capacity; int32_t st_ncb; float st_scale;
   // input-grad epilogue
-  const uint32_t* relubits_prev; const bf16* z_prev; int64_t ld_zprev; bf16* out_dx; int64_t ld_dx;
+  const uint32_t* relubits_prev; const bf16* z_prev; int64_t ld_zprev;
   const bf16* dz; int64_t ld_dz; float* db;    // db (optional): also the column sums of dZ
   // dW epilogue
   float* out_dw; int64_t ld_dw; int64_t dw_rows; const uint32_t* row_idx; float* partial; int64_t partial_rows;
@@ -1128,7 +1130,7 @@ tc_gemm_pair_kernel(const TcParams p, const __grid_constant__ CUtensorMap tmA, c
 }
 
 // ---- two-CTA engine, sparse A (different-sample dW) --------------------------------------------------
-// The pair owns a 256 x 512 tile of dW.  Each CTA rebuilds 128 columns of A_hat (one store tile per
+// The pair owns a 256 x 512 tile of dW (narrower tiles take the first of the two halves, or half of that).  Each CTA rebuilds 128 columns of A_hat (one store tile per
 // K block) in shared memory and loads its half of the dZ tile (two blocks of 128 columns); per 16
 // rows of K two MMAs (M256 N256), one per 256-column half of the tile; the two 128 x 256
 // accumulators of a CTA fill its tensor memory.  A store tile is expanded once per 512 output
@@ -1592,9 +1594,6 @@ DwPlan plan_dw(const rad_store* st, int64_t H) {
     // transposed tile: M = H, N = kept columns in tiles of at most 256 (the kernel fits the width to the count)
     m_expect = std::max<int64_t>(1, (int64_t)std::llround((double)st->D * store_keep_fraction(st)));
     d.partial_rows = round_up(std::min(st->values_ld, round_up(st->D, 8)), 16);
-    d.comp_cap = 0;
-    d.stages = 3;
-    d.comp_depth = 0;
     const int64_t n_tiles = ceil_div(m_expect, BN);
     const int64_t bn = round_up(ceil_div(m_expect, n_tiles), 16);
     d.splits = choose_splits(ceil_div(H, BM), n_tiles, kblocks, BM, planning_pairs(), bn, (double)bn / BN);
@@ -1701,9 +1700,9 @@ int tc_forward(int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t 
   if (rc != RAD_OK) return rc;
   TcParams p = {};
   p.M = B; p.N = H; p.K = D; p.splits = 1; p.bn = dense_tile_width(B, H, next != nullptr ? 128 : 64);
-  p.bias = bias; p.act = act;
-  p.out_act = static_cast<bf16*>(out_act); p.ld_act = ld_act; p.out_z = out_z; p.ld_z = ld_z;
-  p.out_zlow = static_cast<bf16*>(out_zlow); p.ld_zlow = ld_zlow; p.relubits = relubits; p.w32 = ceil_div(H, 32);
+  p.bias = bias;
+  p.out_act = static_cast<const bf16*>(out_act); p.out_z = out_z; p.out_zlow = static_cast<const bf16*>(out_zlow);
+  p.relubits = relubits; p.w32 = ceil_div(H, 32);
   p.dev_status = dev_status;
   p.wait_limit_ns = wait_limit_ns();
   if (next != nullptr) {
@@ -1771,7 +1770,6 @@ int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, 
   TcParams p = {};
   p.M = B; p.N = D; p.K = H; p.splits = 1; p.bn = bn;
   p.relubits_prev = relubits_prev; p.z_prev = static_cast<const bf16*>(z_prev); p.ld_zprev = ld_zprev;
-  p.out_dx = static_cast<bf16*>(dZ_prev); p.ld_dx = ldp;
   p.dz = static_cast<const bf16*>(dZ); p.ld_dz = ldz; p.db = db;
   p.dev_status = dev_status;
   p.wait_limit_ns = wait_limit_ns();
