@@ -133,6 +133,11 @@ __device__ __forceinline__ void tmem_ld16x32(uint32_t taddr, uint32_t (&r)[16]) 
       : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// the same where other work lies between the load and the wait: naming the registers keeps their uses behind it
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])::"memory");
+}
 
 // Shared-memory matrix descriptor, 128-byte swizzle.  K-major: rows of 64 elements (128 B), eight
 // rows form a 1024 B swizzle atom, SBO = 1024 B between atoms along M/N.  MN-major: rows of 64
@@ -459,7 +464,7 @@ __device__ __forceinline__ void dx_chunk(const CUtensorMap* tm_dx, uint32_t tadd
         g[e] = gelu_grad_f(bf16_lo(zw[e >> 1]));
         g[e + 1] = gelu_grad_f(bf16_hi(zw[e >> 1]));
       }
-      tmem_ld_wait();
+      tmem_ld_wait(r);
 #pragma unroll
       for (int e = 0; e < 8; ++e) g[e] *= ((bits >> e) & 1u) ? __uint_as_float(r[e]) : 0.0f;
       st_shared16(at, pack_bf16(g[0], g[1]), pack_bf16(g[2], g[3]), pack_bf16(g[4], g[5]), pack_bf16(g[6], g[7]));

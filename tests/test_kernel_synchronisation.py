@@ -70,3 +70,16 @@ def test_a_dense_kernel_that_gives_up_waits_for_its_own_copies():
     tail = body[body.rindex("buf ^= 1;"):]
     assert re.search(r"if \(EPI == kDxGelu\) asm volatile\(\"cp\.async\.wait_all;\"", tail) and "tma_store_wait();" in tail
     assert tail.index("cp.async.wait_all") < tail.index("cluster_barrier()") > tail.index("tma_store_wait();")
+
+
+def test_accumulators_are_used_behind_the_wait_for_them():
+    """A load from tensor memory fills its registers at the wait, not at the load: the wait comes next, or names the registers, or
+    the compiler could move their uses in front of it."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "tc.cu")).read())
+    loads = list(re.finditer(r"\btmem_ld(?:8|16x32|32)\(([^;{]*), (\w+)(?:\[\d\])?\);", text))
+    assert len(loads) == 5
+    for m in loads:
+        rest = text[m.end():]
+        wait = re.search(r"\btmem_ld_wait\((\w*)\);", rest)
+        next_to_it = re.fullmatch(r"\s*(tmem_ld\w*\([^;]*;\s*)*", rest[:wait.start()])
+        assert next_to_it or wait.group(1) == m.group(2), text[m.start():m.end() + 200]
