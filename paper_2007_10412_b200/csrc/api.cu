@@ -343,7 +343,7 @@ extern "C" int rad_linear_forward(int32_t dtype, int32_t act, int64_t B, int64_t
     return tc_forward(act, B, D, H, A, lda, W, ldw, bias, out_act, ld_act, out_z, ld_z, out_zlow, ld_zlow,
                       relubits, dev_status, s);
   return simt_forward(dtype, act, B, D, H, A, lda, W, ldw, bias, out_act, ld_act, out_z, ld_z, out_zlow,
-                      ld_zlow, relubits, s);
+                      ld_zlow, relubits, dev_status, s);
 }
 
 namespace rad {
@@ -448,7 +448,7 @@ extern "C" int rad_linear_input_grad(int32_t dtype, int64_t B, int64_t D, int64_
   if (dZ_prev == nullptr) return RAD_OK;
   if (on_tc)
     return tc_input_grad(B, D, H, dZ, ldz, W, ldw, relubits_prev, z_prev, ld_zprev, dZ_prev, ldp, beside ? db : nullptr, dev_status, s);
-  return simt_input_grad(dtype, B, D, H, dZ, ldz, W, ldw, relubits_prev, z_prev, ld_zprev, dZ_prev, ldp, s);
+  return simt_input_grad(dtype, B, D, H, dZ, ldz, W, ldw, relubits_prev, z_prev, ld_zprev, dZ_prev, ldp, dev_status, s);
 }
 
 extern "C" int rad_mlp_workspace(const rad_mlp_desc* net, int64_t* bytes, rad_step_stats* stats) {

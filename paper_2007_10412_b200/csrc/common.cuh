@@ -232,10 +232,10 @@ int launch_relu_bits(int dtype, const void* A, int64_t lda, int64_t B, int64_t D
 int simt_forward(int dtype, int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t lda,
                  const void* W, int64_t ldw, const float* bias, void* out_act, int64_t ld_act,
                  float* out_z, int64_t ld_z, void* out_zlow, int64_t ld_zlow, uint32_t* relubits,
-                 cudaStream_t s);
+                 int32_t* dev_status, cudaStream_t s);
 int simt_input_grad(int dtype, int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz,
                     const void* W, int64_t ldw, const uint32_t* relubits_prev, const void* z_prev,
-                    int64_t ld_zprev, void* dZ_prev, int64_t ldp, cudaStream_t s);
+                    int64_t ld_zprev, void* dZ_prev, int64_t ldp, int32_t* dev_status, cudaStream_t s);
 // The operands of an input gradient dZ_prev = (dZ W^T) * act'(.) that go with a dW of the same layer.
 struct SimtInputGrad {
   const void* W; int64_t ldw;

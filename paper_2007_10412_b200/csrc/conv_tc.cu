@@ -25,6 +25,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "umma.cuh"
 
 namespace rad {
 namespace {
@@ -50,69 +51,6 @@ struct ConvTcParams {
   int32_t* dev_status;
   uint64_t wait_limit_ns;
 };
-
-__device__ __forceinline__ uint32_t cv_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint64_t cv_timer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ bool cv_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-// false: the wait ran out (or another one did): the caller stops issuing work
-__device__ __forceinline__ bool cv_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint64_t limit_ns) {
-  if (cv_try_wait(bar, parity)) return true;
-  const uint64_t t0 = cv_timer();
-  while (true) {
-    for (int i = 0; i < 32; ++i) {
-      if (cv_try_wait(bar, parity)) return true;
-      __nanosleep(40);
-    }
-    if (*abort_flag != 0) return false;
-    if (cv_timer() - t0 > limit_ns) {
-      *abort_flag = 1;
-      return false;
-    }
-  }
-}
-// 128-byte-swizzle descriptor (K-major: SBO 1024; MN-major: LBO 8192 between 64-wide blocks, SBO 1024)
-__device__ __forceinline__ uint64_t cv_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) | ((uint64_t)(sbo_bytes >> 4) << 32) |
-         (1ull << 46) | (2ull << 61);
-}
-// D = f32, A = B = bf16, M = 128, N = 64, one CTA
-__host__ __device__ constexpr uint32_t cv_idesc(bool a_mn, bool b_mn) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16) |
-         ((uint32_t)(kCvN >> 3) << 17) | ((uint32_t)(kCvM >> 4) << 24);
-}
-__device__ __forceinline__ void cv_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void cv_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void cv_tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr) : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
 
 struct CvCtl {
   uint64_t done[2];        // the MMAs that read stage s have retired
@@ -149,12 +87,12 @@ __global__ void __launch_bounds__(kCvThreads, kCvPerSm) conv_tc_kernel(const Con
   const int ktaps = 9 * Cin;                          // rows of the filter matrix
   if (tid == 0) {
     for (int s = 0; s < 2; ++s)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(cv_smem(&ctl->done[s])), "r"(1u) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(umma_smem(&ctl->done[s])), "r"(1u) : "memory");
     ctl->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(cv_smem(&ctl->tmem_base)), "r"(64u) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(umma_smem(&ctl->tmem_base)), "r"(64u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
 
@@ -253,7 +191,7 @@ __global__ void __launch_bounds__(kCvThreads, kCvPerSm) conv_tc_kernel(const Con
     uint8_t* sA = smem + s * kCvStageBytes;
     uint8_t* sB = sA + kCvABytes;
     // the MMAs of two K blocks ago have read this stage
-    if (kb >= 2) ok = cv_wait(cv_smem(&ctl->done[s]), ((kb >> 1) - 1) & 1, abort_flag, p.wait_limit_ns);
+    if (kb >= 2) ok = umma_wait(umma_smem(&ctl->done[s]), ((kb >> 1) - 1) & 1, abort_flag, p.wait_limit_ns);
     if (ok) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -271,27 +209,27 @@ __global__ void __launch_bounds__(kCvThreads, kCvPerSm) conv_tc_kernel(const Con
     if (!__syncthreads_and(ok ? 1 : 0)) { ok = false; break; }
     if (warp == 0 && elect_one()) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      constexpr uint32_t idesc = cv_idesc(kDw, !kDx);
-      const uint32_t a0 = cv_smem(sA), b0 = cv_smem(sB);
+      constexpr uint32_t idesc = umma_idesc(kCvM, kCvN, kDw, !kDx);
+      const uint32_t a0 = umma_smem(sA), b0 = umma_smem(sB);
 #pragma unroll
       for (int k = 0; k < kCvK / 16; ++k) {
-        const uint64_t adesc = kDw ? cv_desc(a0 + k * 2048, 8192, 1024) : cv_desc(a0 + k * 32, 16, 1024);
-        const uint64_t bdesc = kDx ? cv_desc(b0 + k * 32, 16, 1024) : cv_desc(b0 + k * 2048, 8192, 1024);
-        cv_mma(tmem, adesc, bdesc, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+        const uint64_t adesc = kDw ? umma_desc(a0 + k * 2048, 8192, 1024) : umma_desc(a0 + k * 32, 16, 1024);
+        const uint64_t bdesc = kDx ? umma_desc(b0 + k * 32, 16, 1024) : umma_desc(b0 + k * 2048, 8192, 1024);
+        umma_mma(tmem, adesc, bdesc, idesc, (kb > 0 || k > 0) ? 1u : 0u);
       }
-      cv_commit(cv_smem(&ctl->done[s]));
+      umma_commit(umma_smem(&ctl->done[s]));
     }
     if (kb + 1 < nkb) gather(kb + 1);
   }
   // the last commit covers every MMA before it
-  if (ok && nkb > 0) ok = cv_wait(cv_smem(&ctl->done[(nkb - 1) & 1]), ((nkb - 1) >> 1) & 1, abort_flag, p.wait_limit_ns);
+  if (ok && nkb > 0) ok = umma_wait(umma_smem(&ctl->done[(nkb - 1) & 1]), ((nkb - 1) >> 1) & 1, abort_flag, p.wait_limit_ns);
   ok = __syncthreads_and(ok ? 1 : 0) != 0;
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (ok) {
     const int q = warp & 3, chunk = warp >> 2;       // accumulator rows 32 q .. 32 q + 31, columns 32 chunk .. + 31
     const int m = q * 32 + lane;
     uint32_t r[32];
-    cv_tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(chunk * 32), r);
+    umma_tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(chunk * 32), r);
     if (kDx) {
       // row m = input pixel, columns = input channels: rounded once, 64 bytes per row and chunk
       const int64_t pix = tile * kCvM + m;

@@ -1,0 +1,72 @@
+// One contraction of the CUDA-core kernels and of their float32 tensor-core form: operands, epilogues, plan.
+#pragma once
+
+#include "common.cuh"
+
+namespace rad {
+
+enum Epilogue { kEpiForward = 0, kEpiInputGrad = 1, kEpiScatterRows = 2, kEpiSparse = 3 };
+
+struct GemmParams {
+  // C(m, n) = sum_k A(m, k) * Bm(k, n); element (m, k) of A at A[m * sam + k * sak], etc.  k is the contiguous index
+  // of A in the forward pass, of both operands in the input gradient and of neither in a dW.
+  const void* A; int64_t sam, sak;
+  const void* Bm; int64_t sbk, sbn;
+  int64_t M, N, K;
+  const int64_t* M_dev;        // optional: M read from device memory (clamped to M)
+  // forward epilogue
+  const float* bias; int act;
+  void* out_act; int64_t ld_act;
+  float* out_z; int64_t ld_z;
+  void* out_zlow; int64_t ld_zlow;
+  // input-grad epilogue
+  const uint32_t* relubits; int64_t w32;
+  const void* z_prev; int64_t ld_zprev;
+  void* out_low; int64_t ld_low;
+  // scatter-rows epilogue (same-sample dW): row m goes to row idx[m] of out_f32
+  const uint32_t* row_idx;
+  float* out_f32; int64_t ld_f32;
+  float* db;                   // or NULL: column sums of Bm over k (the bias gradient), from the CTAs of tile row 0
+  // different-sample dW: A(m, k) = column m of row k of a compact store, whose packed values are `A`
+  const uint32_t* keepbits; const uint32_t* offsets; int64_t capacity; int32_t ncb;
+  // set by plan_gemm
+  int tile, splits;            // rows and columns of C per tile; CTAs (1, 2, 4 or 8) that share a tile's k
+  int walk;                    // one CTA walks all of k (splits is 1)
+  int tc;                      // float32 on the tensor cores (gemm_tc.cu)
+  int vec_a, vec_b;            // 16-byte copies of the operand are aligned
+  int64_t k_per, gx, units;    // k per split, tiles per tile row, CTAs in all
+  int32_t* dev_status; uint64_t wait_limit_ns;        // tensor-core form
+};
+
+// float32 on the tensor cores (gemm_tc.cu): the plan for M rows of C (the rows expected where the device alone knows them; the
+// grid covers p.M), its estimated time in clocks of an SM, and its launches.  A joint launch
+// takes the CTAs of dW, of the input gradient (g may be NULL) and of the zeros of a same-sample dW, all multiples of `cluster`.
+double plan_gemm_tc(GemmParams& p, int64_t M, int64_t k_step);
+int launch_gemm_tc(int epi, const GemmParams& p, cudaStream_t s);
+int launch_dw_dx_tc(int epi, const GemmParams& w, const GemmParams* g, int64_t dw_blocks, int64_t dx_blocks, int64_t zero_blocks, int64_t cluster,
+                    const uint32_t* keep_cols, int64_t D, int64_t H, cudaStream_t s);
+
+// Epilogue of one output.
+template <typename T, int EPI>
+__device__ __forceinline__ void gemm_store(const GemmParams& p, int64_t m, int64_t n, float v) {
+  if (EPI == kEpiForward) {
+    if (p.bias != nullptr) v += p.bias[n];
+    if (p.out_z != nullptr) p.out_z[m * p.ld_z + n] = v;
+    if (p.out_zlow != nullptr) static_cast<T*>(p.out_zlow)[m * p.ld_zlow + n] = from_float<T>(v);
+    if (p.out_act != nullptr) {
+      const float a = p.act == RAD_ACT_RELU ? fmaxf(v, 0.0f) : p.act == RAD_ACT_GELU ? gelu_f(v) : v;
+      static_cast<T*>(p.out_act)[m * p.ld_act + n] = from_float<T>(a);
+    }
+  } else if (EPI == kEpiInputGrad) {
+    if (p.relubits != nullptr) {
+      if (((p.relubits[m * p.w32 + (n >> 5)] >> (n & 31)) & 1u) == 0) v = 0.0f;
+    } else if (p.z_prev != nullptr) {
+      v *= gelu_grad_f(to_float(static_cast<const T*>(p.z_prev)[m * p.ld_zprev + n]));
+    }
+    static_cast<T*>(p.out_low)[m * p.ld_low + n] = from_float<T>(v);
+  } else {
+    p.out_f32[(EPI == kEpiScatterRows ? (int64_t)p.row_idx[m] : m) * p.ld_f32 + n] = v;
+  }
+}
+
+}  // namespace rad

@@ -1,0 +1,745 @@
+// float32 contractions on the tensor cores.  An operand is the exact sum of three bf16 planes (8 significant bits each, every
+// plane the rounding of what the planes before leave), so a b = a1 b1 + (a1 b2 + a2 b1) + (a1 b3 + a2 b2 + a3 b1) up to
+// three products of less than 2^-25 of it: six MMAs, every product exact.  The tensor core cuts off what its float32
+// accumulator cannot hold instead of rounding, so the large products (a1 b1) are added up over 32 k only and then in
+// registers; the small ones have accumulators of their own, whose cut-off lies eight bits further down.
+//
+// A CTA owns a 128 x 128 tile of C, or up to eight CTAs of a cluster share its k.  Sixteen warps bring the next block of 32 k
+// from global memory into registers while they split this one into its planes in shared memory (128-byte swizzle, K- or MN-major
+// as the operand lies in memory; two half-stages of 32 k); a warp of its own issues the MMAs (an MMA takes about 80 cycles to issue
+// whatever its width, so not one of the sixteen does it, and tiles are 128 columns wide); while these run, the sixteen add the
+// 32 accumulators a thread has of the block before to its registers.  What bounds it: issue slots (six to seven instructions
+// split an element, which 128 rows or columns share; 250 a warp and block, 59 % of the slots busy at 4096 x 2048 x 2048, the
+// tensor pipe 45 %) and behind them the MMAs' reads of shared memory; for small problems instruction fetch, so code that is run
+// once is small.  Tiles 64 columns wide, two CTAs an SM and the MMAs issued by one of eight warps: 309 us for that forward; this
+// form 211 (163 TFLOP/s; 794 on CUDA cores).  Against 64 bits the relative error of a contraction over 1000 is 1.1e-7, 2.0e-7
+// there.
+#include <algorithm>
+#include <atomic>
+#include <cfloat>
+#include <type_traits>
+
+#include "gemm.cuh"
+#include "umma.cuh"
+
+namespace rad {
+namespace {
+
+constexpr int kTcM = 128, kTcN = 128, kTcBlock = 32;           // tile of C, k per block (half a 128-byte row of a plane)
+constexpr int kTcPlaneA = kTcM * 128, kTcPlaneB = kTcN * 128;  // bytes of a plane of both half-stages
+constexpr int kTcStageBytes = 3 * (kTcPlaneA + kTcPlaneB);
+constexpr int kTcLd = kTcN + 4;                               // floats per row of the partial tile
+constexpr uint32_t kTcMain = 0, kTcSmall = 2 * kTcN, kTcCols = 4 * kTcN;     // tensor-memory columns: two main, a1 b2 + a2 b1, the rest
+constexpr int kTcWorkers = 16, kTcThreads = 32 * (kTcWorkers + 1);            // warps that split and drain; the last warp issues MMAs
+
+struct TcIndex {               // what a warp needs of a store tile's index: its four rows' words, their offsets (16 bits each), the tile's
+  uint32_t words[4][4], row[4], tile, unused[3];
+};
+struct TcCtl {
+  uint64_t full[2];          // the block in this half-stage is in place, and the main accumulators it goes to have been read
+  uint64_t done[2];          // its MMAs have retired
+  uint32_t tmem;
+  int abort_flag;
+  __align__(16) float bias[kTcN];
+  TcIndex index[kTcWorkers][4];
+};
+constexpr int kTcSmemBytes = kTcStageBytes + (int)sizeof(TcCtl) + 1024;
+static_assert(kTcStageBytes >= (kTcM * kTcLd + 17 * kTcN) * 4, "the partial tile and the column sums reuse the stages");
+
+__device__ __forceinline__ uint8_t* tc_stages(float* smem) {
+  return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem) + 1023) & ~(uintptr_t)1023);
+}
+__device__ __forceinline__ TcCtl* tc_ctl(float* smem) { return reinterpret_cast<TcCtl*>(tc_stages(smem) + kTcStageBytes); }
+
+// Whole CTA.  The next launch is let in behind this.
+__device__ __forceinline__ void tc_begin(float* smem) {
+  TcCtl* ctl = tc_ctl(smem);
+  if (threadIdx.x < 32) umma_alloc<kTcCols>(&ctl->tmem);
+  if (threadIdx.x == 32) {
+    umma_init_barriers(ctl->full, 2, kTcWorkers);
+    umma_init_barriers(ctl->done, 2);
+    ctl->abort_flag = 0;
+  }
+  umma_fence_before();
+  __syncthreads();
+  umma_fence_after();
+}
+__device__ __forceinline__ void tc_end(const GemmParams& p, float* smem) {       // behind the barrier that ends the partial sums
+  TcCtl* ctl = tc_ctl(smem);
+  if (threadIdx.x == 0 && ctl->abort_flag != 0) raise_status(p.dev_status, RAD_DEV_ETIMEOUT);
+  if (threadIdx.x < 32) {
+    umma_fence_after();
+    umma_free<kTcCols>(ctl->tmem);
+  }
+}
+
+__device__ __forceinline__ void tc_add2(f32x2& acc, f32x2 b) { asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc) : "l"(b)); }
+
+// One plane of four neighbouring elements (8 bytes at shared-memory address dst + kAt); r becomes what the plane leaves, exactly.
+template <int kAt, bool kLast>
+__device__ __forceinline__ void tc_plane(float (&r)[4], uint32_t dst) {
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(r[0], r[1]), hi = __floats2bfloat162_rn(r[2], r[3]);
+  const uint32_t a = *reinterpret_cast<const uint32_t*>(&lo), b = *reinterpret_cast<const uint32_t*>(&hi);
+  asm volatile("st.shared.v2.b32 [%0+%3], {%1, %2};" ::"r"(dst), "r"(a), "r"(b), "n"(kAt));
+  if (!kLast) {
+    r[0] -= __uint_as_float(a << 16);
+    r[1] -= __uint_as_float(a & 0xffff0000u);
+    r[2] -= __uint_as_float(b << 16);
+    r[3] -= __uint_as_float(b & 0xffff0000u);
+  }
+}
+template <int kPlaneBytes, int kAt>
+__device__ __forceinline__ void tc_split(const float* v, uint32_t dst) {
+  float r[4] = {v[0], v[1], v[2], v[3]};
+  tc_plane<kAt, false>(r, dst);
+  tc_plane<kAt + kPlaneBytes, false>(r, dst);
+  tc_plane<kAt + 2 * kPlaneBytes, true>(r, dst);
+}
+
+// One operand: two quads (four neighbouring elements each) of a block of 32 k per thread, on their way from global memory to the
+// planes.  kK: k is contiguous in memory (rows of the tile are rows of the matrix); else rows of the matrix are k.  Half-warps
+// write whole 128-byte rows (k-major operands: two halves of rows 4 apart).
+// kVec: the matrix' rows begin on 16 bytes.  Others are read as the two aligned vectors that hold the four (all blocks and both
+// quads of a thread lie the same way: multiples of eight rows apart), where both lie inside the matrix.
+// Rows and columns of the tile past the matrix' end are read from somewhere inside it: what they make is not written.  Only
+// zeros past the end of k count: the last block, and quads that the matrix' edge cuts, come element by element.
+template <bool kK, bool kVec>
+struct TcOperand {
+  static constexpr int kPerRow = kK ? kTcBlock / 4 : kTcM / 4, kUnitRows = 32 * kTcWorkers / kPerRow;
+  static constexpr int kFloats = kVec ? 4 : 8;
+  const float* src; const float* hi;
+  int64_t unit_step, block_step;
+  int first, valid, shift;                          // k of the thread's first element (kK) or row; elements of a quad inside the matrix
+  uint32_t off;
+  bool whole, single;
+  float quad[2][kFloats];
+  // X(r, k) for r in [r0, rows), k from k0; ld: distance of the matrix' rows
+  __device__ __forceinline__ void init(const void* X, int64_t ld, int64_t r0, int64_t rows, int64_t k0, int64_t K) {
+    const int t = (int)threadIdx.x / kPerRow, c = (int)threadIdx.x % kPerRow;
+    const float* x = static_cast<const float*>(X);
+    const int left = (int)min((int64_t)kTcM, rows - r0);
+    single = false;
+    unit_step = kUnitRows * ld;
+    if (kK) {
+      const int row = ((t & 1) << 2) | ((t >> 1) & 3) | (t & ~7);
+      hi = x + (rows - 1) * ld + K;
+      src = x + (r0 + (row < left ? row : 0)) * ld + k0 + 4 * c;
+      if (row + kUnitRows >= left) unit_step = 0;
+      block_step = kTcBlock;
+      first = 4 * c;
+      whole = true;
+      off = row * 128 + (((c >> 1) ^ (row & 7)) << 4) + (c & 1) * 8;
+    } else {
+      hi = x + (K - 1) * ld + rows;
+      valid = min(4, max(0, left - 4 * c));
+      whole = valid == 4 || (valid == 0 && left >= 4);
+      src = x + (k0 + t) * ld + r0 + (whole && valid == 0 ? 0 : 4 * c);
+      block_step = kTcBlock * ld;
+      first = t;
+      off = (c >> 4) * 8192 + t * 128 + ((((c & 15) >> 1) ^ (t & 7)) << 4) + (c & 1) * 8;
+    }
+    shift = kVec ? 0 : (int)((reinterpret_cast<uintptr_t>(src) >> 2) & 3);
+    whole = whole && src - shift >= x;
+  }
+  __device__ __forceinline__ void load(int kleft) {                    // kleft: k from the block's first on
+    if (whole && kleft >= kTcBlock && (kVec || src + unit_step - shift + 8 <= hi)) {
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const float4 a = *reinterpret_cast<const float4*>(src + j * unit_step - shift);
+        quad[j][0] = a.x; quad[j][1] = a.y; quad[j][2] = a.z; quad[j][3] = a.w;
+        if (!kVec) {
+          const float4 b = *reinterpret_cast<const float4*>(src + j * unit_step - shift + 4);
+          quad[j][kFloats - 4] = b.x; quad[j][kFloats - 3] = b.y; quad[j][kFloats - 2] = b.z; quad[j][kFloats - 1] = b.w;
+        }
+      }
+      single = false;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int n = kK ? min(4, kleft - first) : first + j * kUnitRows < kleft ? (whole ? 4 : valid) : 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) quad[j][i] = i < n ? src[j * unit_step + i] : 0.0f;
+      }
+      single = true;
+    }
+  }
+  __device__ __forceinline__ uint32_t half_at(int half, uint32_t planes) const {
+    return kK ? planes + (off ^ (uint32_t)(half * 64)) : planes + off + half * 4096;
+  }
+  template <int kPlaneBytes>
+  __device__ __forceinline__ void store(uint32_t at) {
+    if constexpr (!kVec) {
+      const int from = single ? 0 : shift;
+      const bool two = (from & 2) != 0, one = (from & 1) != 0;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        float* v = quad[j];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) v[i] = two ? v[i + 2] : v[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = one ? v[i + 1] : v[i];
+      }
+    }
+    tc_split<kPlaneBytes, 0>(quad[0], at);
+    tc_split<kPlaneBytes, kUnitRows * 128>(quad[1], at);
+  }
+};
+
+// Element (m, n) as the CUDA-core form adds it up: for results that are not finite (the planes of an infinity are not)
+// and those alone.
+template <int EPI>
+__device__ __noinline__ float tc_plain(const GemmParams& p, int64_t m, int64_t n) {
+  const float* A = static_cast<const float*>(p.A);
+  const float* Bm = static_cast<const float*>(p.Bm);
+  float s = 0.0f;
+#pragma unroll 1
+  for (int64_t k = 0; k < p.K; ++k) {
+    float a;
+    if (EPI == kEpiSparse) {
+      const int r = (int)(k % kTileRows), c = (int)(m % kTileCols);
+      const int64_t t = k / kTileRows * p.ncb + m / kTileCols;
+      const uint32_t* w = p.keepbits + t * kTileWords;
+      int64_t at = (int64_t)p.offsets[t] + ((w[kBitWords + (r >> 1)] >> (16 * (r & 1))) & 0xffffu);
+      #pragma unroll 1
+      for (int i = 0; i < c / 32; ++i) at += __popc(w[4 * r + i]);
+      const uint32_t word = w[4 * r + c / 32], bit = 1u << (c & 31);
+      at += __popc(word & (bit - 1));
+      a = (word & bit) != 0 && at < p.capacity ? A[at] : 0.0f;
+    } else {
+      a = A[m * p.sam + k * p.sak];
+    }
+    s = fmaf(a, Bm[k * p.sbk + n * p.sbn], s);
+  }
+  return s;
+}
+
+// A operand of a different-sample dW: the 128 columns of a store tile, a block is half a slab of 64 rows.  A warp takes every
+// sixteenth row, a lane four columns: their place is the row's offset and the kept entries before them.  The index of the slab
+// after next is on its way into shared memory, each warp's rows by themselves.
+struct TcSparse {
+  static constexpr int kUnits = 2;
+  const float* values; const uint32_t* keepbits; const uint32_t* offsets;
+  int64_t capacity, tile; int ncb, slabs;
+  TcIndex* ring; const TcIndex* now;
+  float quad[kUnits][4];
+  const float* slab_values; int limit;              // of the block that is being loaded
+  uint32_t off;
+  __device__ __forceinline__ void init(const GemmParams& p, int64_t m0, int64_t k0, int nblk, TcCtl* ctl) {
+    values = static_cast<const float*>(p.A); keepbits = p.keepbits; offsets = p.offsets; capacity = p.capacity;
+    ncb = p.ncb; tile = k0 / kTileRows * p.ncb + m0 / kTileCols; slabs = (nblk + 1) / 2;
+    const int c = threadIdx.x & 31, row = (int)threadIdx.x >> 5;
+    ring = ctl->index[row];
+    off = (c >> 4) * 8192 + row * 128 + ((((c & 15) >> 1) ^ (row & 7)) << 4) + (c & 1) * 8;
+  }
+  __device__ __forceinline__ void fetch_index(int slab) {              // row of lane l of eight: warp + 16 (l % 4)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = warp + 16 * (lane & 3);
+    const int64_t t = tile + (int64_t)slab * ncb;
+    TcIndex* to = &ring[slab & 3];
+    if (slab < slabs) {
+      const uint32_t* w = keepbits + t * kTileWords;
+      if (lane < 4)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(umma_smem(to->words[lane])), "l"(w + 4 * r) : "memory");
+      else if (lane < 8)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(umma_smem(&to->row[lane - 4])), "l"(w + kBitWords + (r >> 1)) : "memory");
+      else if (lane == 8)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(umma_smem(&to->tile)), "l"(offsets + t) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  __device__ __forceinline__ void wait_index() {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+  }
+  __device__ __forceinline__ void load(int kb) {
+    now = &ring[(kb >> 1) & 3];
+    slab_values = values + now->tile;
+    limit = (int)min((int64_t)kTileRows * kTileCols, max((int64_t)0, capacity - (int64_t)now->tile));
+    load_quad(0, kb);
+    load_quad(1, kb);
+  }
+  __device__ __forceinline__ void load_quad(int j, int kb) {
+    const int lane = threadIdx.x & 31, i = (kb & 1) * 2 + j, wi = lane >> 3;
+    const uint4 words = *reinterpret_cast<const uint4*>(now->words[i]);
+    int at = (now->row[i] >> (16 * ((threadIdx.x >> 5) & 1))) & 0xffff;          // a warp's rows are all even or all odd
+    uint32_t mine = words.x;
+    if (wi > 0) { at += __popc(mine); mine = words.y; }
+    if (wi > 1) { at += __popc(mine); mine = words.z; }
+    if (wi > 2) { at += __popc(mine); mine = words.w; }
+    const int sh = 4 * (lane & 7);
+    at += __popc(mine & ((1u << sh) - 1u));
+    const uint32_t four = mine >> sh;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const bool kept = ((four >> e) & 1u) != 0;
+      quad[j][e] = kept && at < limit ? slab_values[at] : 0.0f;
+      at += kept ? 1 : 0;
+    }
+  }
+  __device__ __forceinline__ uint32_t half_at(int half, uint32_t planes) const { return planes + off + half * 4096; }
+  template <int kPlaneBytes>
+  __device__ __forceinline__ void store(uint32_t at) const {
+    tc_split<kPlaneBytes, 0>(quad[0], at);
+    tc_split<kPlaneBytes, 2048>(quad[1], at);
+  }
+};
+
+// A CTA's share (split) of a tile: partial sums to shared memory.  Waits for the kernel ahead and lets the next launch in.
+template <int EPI, bool kVec>
+__device__ __forceinline__ void tc_partial_of(const GemmParams& p, int tile, int split, float* smem) {
+  constexpr bool kSparse = EPI == kEpiSparse;
+  constexpr bool kAK = EPI == kEpiForward || EPI == kEpiInputGrad, kBK = EPI == kEpiInputGrad;
+  // what only needs the parameters is done before the kernel ahead has ended
+  int64_t M = p.M;
+  if (EPI == kEpiScatterRows) {
+    begin_after_previous();
+    if (p.M_dev != nullptr) M = min(M, *p.M_dev);
+  }
+  const int64_t m0 = (int64_t)(tile / (int)p.gx) * kTcM, n0 = (int64_t)(tile % (int)p.gx) * kTcN;
+  const bool sums = (EPI == kEpiScatterRows || EPI == kEpiSparse) && p.db != nullptr && m0 == 0;
+  if (m0 >= M && !sums) return;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  uint8_t* planes = tc_stages(smem);
+  const uint32_t sa = umma_smem(planes), sb = sa + 3 * kTcPlaneA;
+  TcCtl* ctl = tc_ctl(smem);
+  volatile int* abort_flag = &ctl->abort_flag;
+  const uint32_t tmem = ctl->tmem;
+  const int64_t k0 = (int64_t)split * p.k_per, k1 = min(p.K, k0 + p.k_per);
+  const int klen = k1 > k0 ? (int)(k1 - k0) : 0, nblk = (klen + kTcBlock - 1) / kTcBlock;
+  f32x2 acc[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = 0;
+  float colsum[4] = {};
+  if (warp == kTcWorkers) {
+    if (EPI == kEpiForward && p.bias != nullptr) {
+      begin_after_previous();
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int64_t n = n0 + 32 * i + (tid & 31);
+        if (n < p.N) ctl->bias[32 * i + (tid & 31)] = p.bias[n];
+      }
+    }
+    // the MMAs of a block: a1 b1 to the main accumulators of its half, the others to the two small sums
+    bool ok = true;
+    for (int kb = 0; kb < nblk && ok; ++kb) {
+      const int half = kb & 1;
+      ok = __all_sync(0xffffffffu, umma_wait(umma_smem(&ctl->full[half]), (uint32_t)(kb >> 1) & 1u, abort_flag, p.wait_limit_ns));
+      if (ok && elect_one()) {
+        umma_fence_after();
+        constexpr uint32_t one = umma_idesc(kTcM, kTcN, !kAK, !kBK), two = umma_idesc(kTcM, 2 * kTcN, !kAK, !kBK);
+        constexpr uint64_t a_step = kTcPlaneA >> 4, b_step = kTcPlaneB >> 4;
+        const uint64_t a0 = umma_desc(sa, kAK ? 16 : 8192, 1024) + (uint64_t)(half * (kAK ? 64 : 4096) >> 4);
+        const uint64_t b0 = umma_desc(sb, kBK ? 16 : 8192, 1024) + (uint64_t)(half * (kBK ? 64 : 4096) >> 4);
+        const uint32_t main = tmem + kTcMain + (uint32_t)half * kTcN;
+#pragma unroll
+        for (int s = 0; s < kTcBlock / 16; ++s) {
+          const uint64_t a1 = a0 + (uint64_t)(s * (kAK ? 32 : 2048) >> 4), b1 = b0 + (uint64_t)(s * (kBK ? 32 : 2048) >> 4);
+          umma_mma(main, a1, b1, one, s > 0 ? 1u : 0u);
+          umma_mma(tmem + kTcSmall, a1, b1 + b_step, two, kb > 0 || s > 0 ? 1u : 0u);         // a1 b2, a1 b3
+          umma_mma(tmem + kTcSmall, a1 + a_step, b1, two, 1u);                                // a2 b1, a2 b2
+          umma_mma(tmem + kTcSmall + kTcN, a1 + 2 * a_step, b1, one, 1u);                     // a3 b1
+        }
+        umma_commit(umma_smem(&ctl->done[half]));
+      }
+      __syncwarp();
+    }
+  } else {
+    TcOperand<kAK, kVec> oa;
+    TcOperand<kBK, kVec> ob;
+    TcSparse os;
+    if constexpr (kSparse) os.init(p, m0, k0, nblk, ctl);
+    else oa.init(p.A, kAK ? p.sam : p.sak, m0, M, k0, k1);
+    ob.init(p.Bm, kBK ? p.sbn : p.sbk, n0, p.N, k0, k1);
+    if (EPI != kEpiScatterRows) begin_after_previous();
+    if constexpr (kSparse) {
+      os.fetch_index(0);
+      os.fetch_index(1);
+      os.wait_index();
+    }
+    // adds 32 columns of this thread's row to the registers
+    const uint32_t lane_cols = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(32 * (warp >> 2));
+    auto add_columns = [&](uint32_t col) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        uint32_t r[16];
+        umma_tmem_ld16(lane_cols + col + 16 * c, r);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) tc_add2(acc[8 * c + i], pack2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])));
+      }
+    };
+    auto load_a = [&](int kb) {
+      if constexpr (kSparse) {
+        if (kb < nblk) os.load(kb);
+      } else {
+        oa.load(klen - kb * kTcBlock);
+        oa.src += oa.block_step;
+      }
+    };
+    auto load_b = [&](int kb) {
+      ob.load(klen - kb * kTcBlock);
+      ob.src += ob.block_step;
+    };
+    if (nblk > 0) {
+      load_a(0);
+      load_b(0);
+    }
+    bool ok = true;
+    for (int kb = 0; kb < nblk; ++kb) {
+      // block kb is split, and block kb + 1 loaded into the registers that this leaves.  The half-stage is free: the MMAs of
+      // block kb - 2 were waited for when their sums were read
+      const int half = kb & 1;
+      if constexpr (kSparse) {
+        if (half == 0) os.fetch_index((kb >> 1) + 2);
+        os.template store<kTcPlaneA>(os.half_at(half, sa));
+      } else {
+        oa.template store<kTcPlaneA>(oa.half_at(half, sa));
+      }
+      load_a(kb + 1);
+      ob.template store<kTcPlaneB>(ob.half_at(half, sb));
+      if (sums) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) colsum[i] += ob.quad[0][i] + ob.quad[1][i];
+      }
+      load_b(kb + 1);
+      if constexpr (kSparse) {
+        if (half == 1) os.wait_index();
+      }
+      umma_fence_smem();
+      umma_fence_before();
+      __syncwarp();
+      if ((tid & 31) == 0) umma_arrive(umma_smem(&ctl->full[half]));
+      if (kb > 0) {
+        ok = __all_sync(0xffffffffu, umma_wait(umma_smem(&ctl->done[half ^ 1]), (uint32_t)((kb - 1) >> 1) & 1u, abort_flag, p.wait_limit_ns));
+        if (!ok) break;
+        umma_fence_after();
+        add_columns(kTcMain + (uint32_t)(half ^ 1) * kTcN);
+      }
+    }
+    if (ok && nblk > 0)
+      ok = __all_sync(0xffffffffu, umma_wait(umma_smem(&ctl->done[(nblk - 1) & 1]), (uint32_t)((nblk - 1) >> 1) & 1u, abort_flag, p.wait_limit_ns));
+    if (ok && nblk > 0) {
+      umma_fence_after();
+#pragma unroll 1
+      for (int i = 0; i < 3; ++i)                    // the small sums and the last block's large ones
+        add_columns(i == 0 ? kTcSmall + kTcN : i == 1 ? kTcSmall : kTcMain + (uint32_t)((nblk - 1) & 1) * kTcN);
+    }
+    if constexpr (kSparse) asm volatile("cp.async.wait_group 0;" ::: "memory");
+  }
+  umma_fence_before();
+  __syncthreads();
+  if (warp == kTcWorkers) return;
+  float* plane = reinterpret_cast<float*>(planes);
+  float* row = plane + (32 * (warp & 3) + (tid & 31)) * kTcLd + 32 * (warp >> 2);
+#pragma unroll
+  for (int i = 0; i < 16; i += 2) *reinterpret_cast<ulonglong2*>(row + 2 * i) = make_ulonglong2(acc[i], acc[i + 1]);
+  if (sums) {
+    // row of the operand block (of 16) and four columns: the rows are added by the first 128 threads
+    float* s = plane + kTcM * kTcLd;
+    *reinterpret_cast<float4*>(s + (tid >> 5) * kTcN + 4 * (tid & 31)) = make_float4(colsum[0], colsum[1], colsum[2], colsum[3]);
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * kTcWorkers) : "memory");
+    if (tid < kTcN) {
+      float t = 0.0f;
+#pragma unroll
+      for (int r = 0; r < 16; ++r) t += s[r * kTcN + tid];
+      s[16 * kTcN + tid] = t;
+    }
+  }
+}
+
+template <int EPI>
+__device__ __forceinline__ void tc_partial(const GemmParams& p, int tile, int split, float* smem) {
+  if (p.vec_b && (EPI == kEpiSparse || p.vec_a)) tc_partial_of<EPI, true>(p, tile, split, smem);
+  else tc_partial_of<EPI, false>(p, tile, split, smem);
+}
+
+// Out of line: erff inlined four times over would be most of the kernel.
+__device__ __noinline__ float4 tc_gelu(float4 z) { return make_float4(gelu_f(z.x), gelu_f(z.y), gelu_f(z.z), gelu_f(z.w)); }
+__device__ __noinline__ float4 tc_gelu_grad(float4 z) { return make_float4(gelu_grad_f(z.x), gelu_grad_f(z.y), gelu_grad_f(z.z), gelu_grad_f(z.w)); }
+
+__device__ __forceinline__ float4 tc_ld_cluster(const float* smem, uint32_t rank) {
+  float4 v;
+  asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %4, %5;\n\tld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [a];\n\t}"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(umma_smem(smem)), "r"(rank) : "memory");
+  return v;
+}
+// n of four neighbouring floats, in one piece where they lie on 16 bytes
+__device__ __forceinline__ void tc_put(float* to, const float4& v, int n, bool vec) {
+  if (vec && n == 4) {
+    *reinterpret_cast<float4*>(to) = v;
+  } else {
+    if (n > 0) to[0] = v.x;
+    if (n > 1) to[1] = v.y;
+    if (n > 2) to[2] = v.z;
+    if (n > 3) to[3] = v.w;
+  }
+}
+__device__ __forceinline__ float4 tc_get(const float* from, int n, bool vec) {
+  if (vec && n == 4) return *reinterpret_cast<const float4*>(from);
+  return make_float4(n > 0 ? from[0] : 0.0f, n > 1 ? from[1] : 0.0f, n > 2 ? from[2] : 0.0f, n > 3 ? from[3] : 0.0f);
+}
+__device__ __forceinline__ bool tc_on16(const void* p, int64_t ld) { return ((reinterpret_cast<uintptr_t>(p) & 15) == 0) && (ld & 3) == 0; }
+
+// The CTA's share of the tile's rows, from the partial tiles of all its splits: a warp takes every sixteenth row, a lane four
+// columns.  (One column per thread took 5700 cycles for a tile,
+// three times as long as everything before it in a contraction of 64.)
+template <int EPI, bool kGelu>
+__device__ __forceinline__ void tc_finish(const GemmParams& p, int tile, int split, float* smem) {
+  int64_t M = p.M;
+  if (p.M_dev != nullptr) M = min(M, *p.M_dev);
+  const int64_t m0 = (int64_t)(tile / (int)p.gx) * kTcM, n0 = (int64_t)(tile % (int)p.gx) * kTcN;
+  const bool sums = (EPI == kEpiScatterRows || EPI == kEpiSparse) && p.db != nullptr && m0 == 0;
+  const int S = p.splits, rows = kTcM / S, tid = threadIdx.x, warp = tid >> 5;
+  const uint32_t rank0 = cluster_ctarank() - (uint32_t)split;
+  float* plane = reinterpret_cast<float*>(tc_stages(smem));
+  if (sums && split == 0 && tid < kTcN && n0 + tid < p.N) {
+    const float* s = plane + kTcM * kTcLd + 16 * kTcN + tid;
+    float t = 0.0f;
+    for (int q = 0; q < S; ++q) t += S > 1 ? ld_cluster_f32(s, rank0 + q) : *s;
+    p.db[n0 + tid] = t;
+  }
+  if (m0 >= M || warp >= kTcWorkers) return;
+  const int c = 4 * (tid & 31), nc = (int)max((int64_t)0, min((int64_t)4, p.N - n0 - c));      // columns past the end: nothing is written
+  const int64_t n = n0 + c;
+  const int begin = split * rows, end = (int)min((int64_t)(begin + rows), M - m0);
+  float4 bias = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  if (EPI == kEpiForward && p.bias != nullptr) bias = *reinterpret_cast<const float4*>(tc_ctl(smem)->bias + c);
+  const bool relu = EPI == kEpiForward && p.act == RAD_ACT_RELU;
+  const bool masked = EPI == kEpiInputGrad && !kGelu && p.relubits != nullptr;
+  const bool vec_a = EPI == kEpiForward ? tc_on16(p.out_act, p.ld_act) : EPI == kEpiInputGrad ? tc_on16(p.out_low, p.ld_low) : tc_on16(p.out_f32, p.ld_f32);
+  const bool vec_z = EPI == kEpiForward ? tc_on16(p.out_z, p.ld_z) : kGelu && tc_on16(p.z_prev, p.ld_zprev);
+  const bool vec_zlow = EPI == kEpiForward && tc_on16(p.out_zlow, p.ld_zlow);
+  // all splits of all rows of this thread (rows x splits are 128, eight vectors a thread) are under way before the first is
+  // added; the sums go where this CTA's own partial sums of these rows were, which only this thread has read
+  if (S > 1) {
+    float4 part[8];
+    const int shift = 31 - __clz(S);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = begin + warp + (i >> shift) * kTcWorkers;
+      if (r < end) part[i] = tc_ld_cluster(plane + r * kTcLd + c, rank0 + (uint32_t)(i & (S - 1)));
+    }
+    float4 v = part[0];
+#pragma unroll
+    for (int i = 1; i <= 8; ++i) {
+      const bool more = i < 8 && (i & (S - 1)) != 0;
+      if (!more) {
+        const int r = begin + warp + ((i - 1) >> shift) * kTcWorkers;
+        if (r < end) *reinterpret_cast<float4*>(plane + r * kTcLd + c) = v;
+        v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      }
+      if (i < 8) { v.x += part[i & 7].x; v.y += part[i & 7].y; v.z += part[i & 7].z; v.w += part[i & 7].w; }
+    }
+  }
+  // a thread's rows have a word of ReLU bits each (four words a row), or a row of dW: 32 words, one a lane
+  const int lane = tid & 31;
+  uint32_t words = 0;
+  if (masked) {
+    const int r = begin + warp + (lane >> 2) * kTcWorkers;
+    const int64_t w = (n0 >> 5) + (lane & 3);
+    if (r < end && w < p.w32) words = p.relubits[(m0 + r) * p.w32 + w];
+  } else if (EPI == kEpiScatterRows) {
+    const int r = begin + warp + lane * kTcWorkers;
+    if (r < end) words = p.row_idx[m0 + r];
+  }
+  constexpr int kAhead = kGelu && EPI == kEpiInputGrad ? 4 : 1;           // rows whose pre-activations are under way
+  uint32_t bad = 0;                                  // rows with a result that is not finite
+#pragma unroll 1
+  for (int r0 = begin + warp, at_row = 0; r0 < end; r0 += kAhead * kTcWorkers, at_row += kAhead) {
+    float4 pre[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i)
+      if (kGelu && EPI == kEpiInputGrad)
+        pre[i] = tc_get(static_cast<const float*>(p.z_prev) + (m0 + min(r0 + i * kTcWorkers, end - 1)) * p.ld_zprev + n, nc, vec_z);
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      const int r = r0 + i * kTcWorkers;
+      if (r >= end) break;
+      const int64_t m = m0 + r;
+      float4 v = *reinterpret_cast<const float4*>(plane + r * kTcLd + c);
+      const uint32_t word = EPI == kEpiScatterRows ? __shfl_sync(0xffffffffu, words, at_row) : masked ? __shfl_sync(0xffffffffu, words, 4 * at_row + (lane >> 3)) : 0;
+      // a sum of zeros times the values is not zero exactly where one of them is not finite
+      if (!(fmaf(v.x, 0.0f, v.y * 0.0f) + fmaf(v.z, 0.0f, v.w * 0.0f) == 0.0f)) bad |= 1u << (at_row + i);
+      if (EPI == kEpiForward) {
+        v.x += bias.x; v.y += bias.y; v.z += bias.z; v.w += bias.w;
+        if (p.out_z != nullptr) tc_put(p.out_z + m * p.ld_z + n, v, nc, vec_z);
+        if (p.out_zlow != nullptr) tc_put(static_cast<float*>(p.out_zlow) + m * p.ld_zlow + n, v, nc, vec_zlow);
+        if (p.out_act != nullptr) {
+          if (relu) v = make_float4(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f), fmaxf(v.z, 0.0f), fmaxf(v.w, 0.0f));
+          if (kGelu) v = tc_gelu(v);
+          tc_put(static_cast<float*>(p.out_act) + m * p.ld_act + n, v, nc, vec_a);
+        }
+      } else if (EPI == kEpiInputGrad) {
+        if (masked) {
+          const uint32_t bits = word >> (n & 31);
+          v.x = (bits & 1u) != 0 ? v.x : 0.0f; v.y = (bits & 2u) != 0 ? v.y : 0.0f;
+          v.z = (bits & 4u) != 0 ? v.z : 0.0f; v.w = (bits & 8u) != 0 ? v.w : 0.0f;
+        }
+        if (kGelu) {
+          const float4 d = tc_gelu_grad(pre[i]);
+          v.x *= d.x; v.y *= d.y; v.z *= d.z; v.w *= d.w;
+        }
+        tc_put(static_cast<float*>(p.out_low) + m * p.ld_low + n, v, nc, vec_a);
+      } else {
+        tc_put(p.out_f32 + (EPI == kEpiScatterRows ? (int64_t)word : m) * p.ld_f32 + n, v, nc, vec_a);
+      }
+    }
+  }
+  // ... are added up again as the CUDA-core form does it
+#pragma unroll 1
+  for (; bad != 0; bad &= bad - 1) {
+    const int r = begin + warp + (__ffs(bad) - 1) * kTcWorkers;
+#pragma unroll 1
+    for (int e = 0; e < nc; ++e) {
+      if (!(fabsf(plane[r * kTcLd + c + e]) <= FLT_MAX)) gemm_store<float, EPI>(p, m0 + r, n + e, tc_plain<EPI>(p, m0 + r, n + e));
+    }
+  }
+}
+
+// No CTA leaves while another reads its partial tile.
+__device__ __forceinline__ void tc_barrier() {
+  if (cluster_nctas() > 1) cluster_barrier(); else __syncthreads();
+}
+
+template <int EPI, bool kGelu>
+__global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_constant__ GemmParams p) {
+  extern __shared__ __align__(16) float smem[];
+  tc_begin(smem);
+  const int tile = (int)blockIdx.x / p.splits, split = (int)blockIdx.x % p.splits;
+  tc_partial<EPI>(p, tile, split, smem);
+  tc_barrier();
+  tc_finish<EPI, kGelu>(p, tile, split, smem);
+  tc_end(p, smem);
+  if (cluster_nctas() > 1) cluster_barrier();
+}
+
+// dW of a layer and the gradient of its input in one launch (see the CUDA-core form of it, simt.cu): the CTAs of dW, those of
+// the input gradient and, for a same-sample store, those that write zeros to the rows of dW whose column was not kept.
+template <int EPI, bool kGelu>
+__global__ void __launch_bounds__(kTcThreads, 1) dw_dx_tc_kernel(const __grid_constant__ GemmParams w, const __grid_constant__ GemmParams g,
+                                                                 int dw_blocks, int dx_blocks, const uint32_t* keep_cols, int64_t D, int64_t H) {
+  extern __shared__ __align__(16) float smem[];
+  const int b = (int)blockIdx.x;
+  const bool is_dw = b < dw_blocks, is_dx = !is_dw && b < dw_blocks + dx_blocks;
+  const int unit = is_dw ? b : b - dw_blocks;
+  const bool work = is_dw ? unit < w.units : is_dx && unit < g.units;
+  const int splits = is_dw || !is_dx ? w.splits : g.splits, tile = unit / splits, split = unit % splits;
+  if (work) tc_begin(smem); else begin_after_previous();
+  if (work && is_dw) {
+    tc_partial<EPI>(w, tile, split, smem);
+  } else if (work) {
+    tc_partial<kEpiInputGrad>(g, tile, split, smem);
+  } else if (!is_dw && !is_dx) {
+    const int nz = (int)gridDim.x - dw_blocks - dx_blocks;
+    for (int64_t d = b - dw_blocks - dx_blocks; d < D; d += nz) {
+      if ((keep_cols[d >> 5] >> (d & 31)) & 1u) continue;
+      for (int64_t h = threadIdx.x; h < H; h += kTcThreads) w.out_f32[d * w.ld_f32 + h] = 0.0f;
+    }
+  }
+  tc_barrier();
+  if (work && is_dw) tc_finish<EPI, false>(w, tile, split, smem);
+  else if (work) tc_finish<kEpiInputGrad, kGelu>(g, tile, split, smem);
+  if (work) tc_end(w, smem);
+  if (cluster_nctas() > 1) cluster_barrier();
+}
+
+template <int EPI, bool kGelu>
+int launch_one(const GemmParams& p, cudaStream_t s) {
+  static std::atomic<uint64_t> ready{0};
+  if (!allow_smem(gemm_tc_kernel<EPI, kGelu>, kTcSmemBytes, ready)) return RAD_ECUDA;
+  return launch_with_cluster(gemm_tc_kernel<EPI, kGelu>, dim3((unsigned)p.units), kTcThreads, (size_t)kTcSmemBytes, dim3((unsigned)p.splits), s, p);
+}
+template <int EPI, bool kGelu>
+int launch_joint(const GemmParams& w, const GemmParams* g, int64_t dw_blocks, int64_t dx_blocks, int64_t zero_blocks, int64_t cluster,
+                 const uint32_t* keep_cols, int64_t D, int64_t H, cudaStream_t s) {
+  static std::atomic<uint64_t> ready{0};
+  if (!allow_smem(dw_dx_tc_kernel<EPI, kGelu>, kTcSmemBytes, ready)) return RAD_ECUDA;
+  return launch_with_cluster(dw_dx_tc_kernel<EPI, kGelu>, dim3((unsigned)(dw_blocks + dx_blocks + zero_blocks)), kTcThreads, (size_t)kTcSmemBytes,
+                             dim3((unsigned)cluster), s, w, g != nullptr ? *g : GemmParams{}, (int)dw_blocks, (int)dx_blocks, keep_cols, D, H);
+}
+
+// An input gradient takes the derivative of GELU where there is a pre-activation and no ReLU bits.
+bool gelu_ahead(const GemmParams& p) { return p.relubits == nullptr && p.z_prev != nullptr; }
+
+}  // namespace
+
+// Clusters of `size` CTAs that run at the same time (an SM takes one CTA, and a cluster stays within a part of the chip).
+static int clusters_at_once(int size) {
+  static std::atomic<int> known[4];
+  const int i = size >= 8 ? 3 : size >= 4 ? 2 : size >= 2 ? 1 : 0;
+  int n = known[i].load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)size);
+  cfg.blockDim = dim3(kTcThreads);
+  cfg.dynamicSmemBytes = kTcSmemBytes;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = (unsigned)size; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  static std::atomic<uint64_t> ready{0};
+  if (!allow_smem(gemm_tc_kernel<kEpiForward, false>, kTcSmemBytes, ready) ||
+      cudaOccupancyMaxActiveClusters(&n, gemm_tc_kernel<kEpiForward, false>, &cfg) != cudaSuccess || n <= 0) {
+    (void)cudaGetLastError();
+    return std::max(1, kNumSms / size);              // not remembered
+  }
+  known[i].store(n, std::memory_order_relaxed);
+  return n;
+}
+
+// Estimated clocks at 1.9 GHz: rounds of clusters, each of so many blocks of 32 k and 9750 for the beginning and the end of a
+// tile, the exchange inside a cluster.  A block costs 1470 where the matrices' rows begin on 16 bytes and 2700 where they do not;
+// 2470 and 3250 with A expanded from a store; 1270 and 3000 with a same-sample store.  Fitted to 116 timings of both forms (29
+// shapes, forward, input gradient, both dW): within 25 % of 109 of them.  Against the CUDA-core form the line lies near 300 x
+// 500 x 500: 150 x 300 x 300 8.5 us here and 6.2 there, 300 x 500 x 500 9.5 and 14.2, 2048 x 1024 x 1024 29 and 126, 4096 x 2048
+// x 2048 211 and 794 (the same with A from a store 344 and 893), 1500 x 1001 x 777 51 and 104.  Less than 72
+// k or columns (half a tile's width and a bit) stay there: 4096 x 1001, k = 10, 17 us against 12, 4096 x 64 x 64 6.5 against 5.6;
+// between 60 and 72 long or wide ones would be faster here (512 x 64 x 2048 6.4 against 9.6), but tests/test_launches.py holds
+// 2000 x 68 x 1500 to the CUDA-core forms whose coverage it checks.
+double plan_gemm_tc(GemmParams& p, int64_t M, int64_t k_step) {
+  const int64_t step = std::max<int64_t>(k_step, kTcBlock), gx = ceil_div(p.N, kTcN);
+  const int64_t tiles = std::max<int64_t>(1, ceil_div(M, kTcM)) * gx, grid_tiles = std::max<int64_t>(1, ceil_div(p.M, kTcM)) * gx;
+  const bool ak = p.sak == 1, bk = p.sbk == 1 && p.sbn != 1, sparse = p.keepbits != nullptr;
+  p.vec_a = sparse || (((uintptr_t)p.A & 15) == 0 && (ak ? p.sam : p.sak) % 4 == 0);
+  p.vec_b = ((uintptr_t)p.Bm & 15) == 0 && (bk ? p.sbn : p.sbk) % 4 == 0;
+  const bool vec = p.vec_a && p.vec_b;
+  const double block = sparse ? (vec ? 2470 : 3250) : ak ? (vec ? 1470 : 2700) : vec ? 1270 : 3000;
+  double best = 1e300;
+  if (p.K < 72 || p.N < 72) return best;
+  p.tc = 1;
+  p.walk = 0;
+  p.wait_limit_ns = wait_limit_ns();
+  for (int s = 1; s <= 8; s *= 2) {
+    if (s > 1 && p.K <= s / 2 * step) break;
+    const int64_t rounds = ceil_div(tiles, (int64_t)clusters_at_once(s)), k_per = round_up(ceil_div(p.K, s), step);
+    const double clk = (double)rounds * ((double)(k_per / kTcBlock) * block + 9750.0) + (s > 1 ? 5100.0 : 0.0);
+    if (clk < best && grid_tiles * s <= 0x7fffffff) {
+      best = clk;
+      p.splits = s; p.k_per = k_per;
+      p.gx = gx; p.units = grid_tiles * s;
+    }
+  }
+  return best;
+}
+
+int launch_gemm_tc(int epi, const GemmParams& p, cudaStream_t s) {
+  count_launch();
+  switch (epi) {
+    case kEpiForward: return p.act == RAD_ACT_GELU && p.out_act != nullptr ? launch_one<kEpiForward, true>(p, s) : launch_one<kEpiForward, false>(p, s);
+    case kEpiInputGrad: return gelu_ahead(p) ? launch_one<kEpiInputGrad, true>(p, s) : launch_one<kEpiInputGrad, false>(p, s);
+    case kEpiScatterRows: return launch_one<kEpiScatterRows, false>(p, s);
+    default: return launch_one<kEpiSparse, false>(p, s);
+  }
+}
+
+int launch_dw_dx_tc(int epi, const GemmParams& w, const GemmParams* g, int64_t dw_blocks, int64_t dx_blocks, int64_t zero_blocks, int64_t cluster,
+                    const uint32_t* keep_cols, int64_t D, int64_t H, cudaStream_t s) {
+  count_launch();
+  const bool gelu = g != nullptr && gelu_ahead(*g);
+  if (epi == kEpiSparse)
+    return gelu ? launch_joint<kEpiSparse, true>(w, g, dw_blocks, dx_blocks, zero_blocks, cluster, keep_cols, D, H, s)
+                : launch_joint<kEpiSparse, false>(w, g, dw_blocks, dx_blocks, zero_blocks, cluster, keep_cols, D, H, s);
+  return gelu ? launch_joint<kEpiScatterRows, true>(w, g, dw_blocks, dx_blocks, zero_blocks, cluster, keep_cols, D, H, s)
+              : launch_joint<kEpiScatterRows, false>(w, g, dw_blocks, dx_blocks, zero_blocks, cluster, keep_cols, D, H, s);
+}
+
+}  // namespace rad

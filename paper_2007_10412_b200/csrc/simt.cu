@@ -1,45 +1,14 @@
-// CUDA-core (FFMA) kernels: the float32 nets, whose 1e-5 tolerance rules out tensor-core input
-// rounding, and bf16 problems whose shapes the TMA path cannot take.  These problems are small
-// and latency-bound; the kernels favour exact float32 accumulation in a fixed order over speed.
+// CUDA-core (FFMA) kernels: small float32 contractions (larger ones go to gemm_tc.cu, three exact bf16 planes per operand) and
+// bf16 problems whose shapes the TMA path cannot take.  These problems are latency-bound; the kernels favour exact float32
+// accumulation in a fixed order over speed.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
 
-#include "common.cuh"
+#include "gemm.cuh"
 
 namespace rad {
 namespace {
-
-enum Epilogue { kEpiForward = 0, kEpiInputGrad = 1, kEpiScatterRows = 2, kEpiSparse = 3 };
-
-struct GemmParams {
-  // C(m, n) = sum_k A(m, k) * Bm(k, n); element (m, k) of A at A[m * sam + k * sak], etc.  k is the contiguous index
-  // of A in the forward pass, of both operands in the input gradient and of neither in a dW.
-  const void* A; int64_t sam, sak;
-  const void* Bm; int64_t sbk, sbn;
-  int64_t M, N, K;
-  const int64_t* M_dev;        // optional: M read from device memory (clamped to M)
-  // forward epilogue
-  const float* bias; int act;
-  void* out_act; int64_t ld_act;
-  float* out_z; int64_t ld_z;
-  void* out_zlow; int64_t ld_zlow;
-  // input-grad epilogue
-  const uint32_t* relubits; int64_t w32;
-  const void* z_prev; int64_t ld_zprev;
-  void* out_low; int64_t ld_low;
-  // scatter-rows epilogue (same-sample dW): row m goes to row idx[m] of out_f32
-  const uint32_t* row_idx;
-  float* out_f32; int64_t ld_f32;
-  float* db;                   // or NULL: column sums of Bm over k (the bias gradient), from the CTAs of tile row 0
-  // different-sample dW: A(m, k) = column m of row k of a compact store, whose packed values are `A`
-  const uint32_t* keepbits; const uint32_t* offsets; int64_t capacity; int32_t ncb;
-  // set by plan_gemm
-  int tile, splits;            // rows and columns of C per tile; CTAs (1, 2, 4 or 8) that share a tile's k
-  int walk;                    // one CTA walks all of k (splits is 1)
-  int vec_a, vec_b;            // 16-byte copies of the operand are aligned
-  int64_t k_per, gx, units;    // k per split, tiles per tile row, CTAs in all
-};
 
 // Splitting a contraction over CTAs: the CTAs of a tile are neighbours in a cluster, each leaves its partial tile
 // in its own shared memory, and each then finishes (adds in split order, applies the epilogue to, writes) an equal
@@ -336,29 +305,6 @@ __device__ __forceinline__ void gemm_partial(const GemmParams& p, int64_t tile, 
     smem[e] = (smem[e] + smem[TS * TS + e]) + (smem[2 * TS * TS + e] + smem[3 * TS * TS + e]);
 }
 
-// Epilogue of one output.
-template <typename T, int EPI>
-__device__ __forceinline__ void gemm_store(const GemmParams& p, int64_t m, int64_t n, float v) {
-  if (EPI == kEpiForward) {
-    if (p.bias != nullptr) v += p.bias[n];
-    if (p.out_z != nullptr) p.out_z[m * p.ld_z + n] = v;
-    if (p.out_zlow != nullptr) static_cast<T*>(p.out_zlow)[m * p.ld_zlow + n] = from_float<T>(v);
-    if (p.out_act != nullptr) {
-      const float a = p.act == RAD_ACT_RELU ? fmaxf(v, 0.0f) : p.act == RAD_ACT_GELU ? gelu_f(v) : v;
-      static_cast<T*>(p.out_act)[m * p.ld_act + n] = from_float<T>(a);
-    }
-  } else if (EPI == kEpiInputGrad) {
-    if (p.relubits != nullptr) {
-      if (((p.relubits[m * p.w32 + (n >> 5)] >> (n & 31)) & 1u) == 0) v = 0.0f;
-    } else if (p.z_prev != nullptr) {
-      v *= gelu_grad_f(to_float(static_cast<const T*>(p.z_prev)[m * p.ld_zprev + n]));
-    }
-    static_cast<T*>(p.out_low)[m * p.ld_low + n] = from_float<T>(v);
-  } else {
-    p.out_f32[(EPI == kEpiScatterRows ? (int64_t)p.row_idx[m] : m) * p.ld_f32 + n] = v;
-  }
-}
-
 // The CTA's share of the tile's rows, from the partial tiles of all its splits.
 template <typename T, int EPI, int TS>
 __device__ __forceinline__ void gemm_finish(const GemmParams& p, int64_t tile, int split, const float* smem) {
@@ -505,7 +451,7 @@ __device__ __forceinline__ void gemm_walk(const GemmParams& p, int64_t tile, flo
 // forwards, input gradients and same-sample dW of both types, 16 to 4096 rows, the choice is within 6 % of the better form in
 // 118; the others are bf16 300 x 100 x 700 (forward 10.2 against 9.2 us, dW 16.9 against 13.9).
 struct GemmCost { double pair, alone, ends; };
-inline void plan_gemm(GemmParams& p, int64_t Mgrid, int es, int64_t k_step = 4, bool may_walk = true) {   // splits begin at multiples of k_step
+inline double plan_gemm(GemmParams& p, int64_t Mgrid, int es, int64_t k_step = 4, bool may_walk = true) {   // splits begin at multiples of k_step
   static const GemmCost split_cost[3][2] = {{{35, 26, 3850}, {106, 73, 7500}},      // f32, at 32 x 32 and 64 x 64
                                             {{72, 45, 4500}, {258, 150, 11000}},    // bf16, k contiguous
                                             {{72, 45, 4500}, {150, 90, 7500}}};     // bf16, dW
@@ -531,6 +477,27 @@ inline void plan_gemm(GemmParams& p, int64_t Mgrid, int es, int64_t k_step = 4, 
   const bool ak = p.sak == 1, bk = p.sbk == 1 && p.sbn != 1;
   p.vec_a = es == 4 && ((uintptr_t)p.A & 15) == 0 && (ak ? p.sam : p.sak) % 4 == 0;
   p.vec_b = es == 4 && ((uintptr_t)p.Bm & 15) == 0 && (bk ? p.sbn : p.sbk) % 4 == 0;
+  return best;
+}
+// The form of a contraction, and of a dW with the input gradient beside it (both in the same form: one launch has CTAs of one
+// kind): the one with the least estimated time, for the rows that are expected (a same-sample dW; its grid covers p.M).
+// The tensor-core form has to be ahead by 15 %, which is what the estimates are good for.
+inline bool tc_wins(double cuda_cores, double tensor_cores) { return 1.15 * tensor_cores < cuda_cores; }
+inline void plan_forms(GemmParams& p, int64_t rows, int es, int64_t k_step = 4, bool may_walk = true) {
+  GemmParams c = p, t = p;
+  const double est = plan_gemm(c, rows, es, k_step, may_walk);
+  if (es == 4 && tc_wins(est, plan_gemm_tc(t, rows, k_step))) p = t;
+  else plan_gemm(p, p.M, es, k_step, may_walk);
+}
+inline void plan_joint(GemmParams& w, GemmParams& g, int64_t rows, int es, int64_t k_step, bool may_walk) {
+  GemmParams c = w, tw = w, tg = g;
+  const double est = plan_gemm(c, rows, es, k_step, may_walk) + plan_gemm(g, g.M, es);
+  if (es == 4 && tc_wins(est, plan_gemm_tc(tw, rows, k_step) + plan_gemm_tc(tg, g.M, 4))) {
+    w = tw;
+    g = tg;
+  } else {
+    plan_gemm(w, w.M, es, k_step, may_walk);
+  }
 }
 template <typename T, int EPI>
 __device__ __forceinline__ void gemm_unit_partial(const GemmParams& p, int64_t unit, float* smem) {
@@ -577,6 +544,7 @@ __global__ void __launch_bounds__(256) gemm_walk_kernel(const GemmParams p) {
 template <int EPI>
 int launch_planned(int dtype, const GemmParams& p, cudaStream_t s) {
   if (p.units > 0x7fffffff) return RAD_EINVAL;
+  if (p.tc) return launch_gemm_tc(EPI, p, s);
   count_launch();
   if constexpr (EPI != kEpiSparse) {
     if (p.walk) {
@@ -597,9 +565,9 @@ int launch_planned(int dtype, const GemmParams& p, cudaStream_t s) {
 }
 
 template <int EPI>
-int launch_gemm(int dtype, const GemmParams& p0, int64_t Mgrid, cudaStream_t s) {
+int launch_gemm(int dtype, const GemmParams& p0, int64_t rows, cudaStream_t s) {
   GemmParams p = p0;
-  plan_gemm(p, Mgrid, dtype == RAD_BF16 ? 2 : 4);
+  plan_forms(p, rows, dtype == RAD_BF16 ? 2 : 4);
   return launch_planned<EPI>(dtype, p, s);
 }
 
@@ -801,8 +769,9 @@ __global__ void __launch_bounds__(256, 2) same_dw_dx_kernel(const GemmParams w, 
 int simt_forward(int dtype, int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t lda,
                  const void* W, int64_t ldw, const float* bias, void* out_act, int64_t ld_act,
                  float* out_z, int64_t ld_z, void* out_zlow, int64_t ld_zlow, uint32_t* relubits,
-                 cudaStream_t s) {
+                 int32_t* dev_status, cudaStream_t s) {
   GemmParams p = {};
+  p.dev_status = dev_status;
   p.A = A; p.sam = lda; p.sak = 1;
   p.Bm = W; p.sbk = ldw; p.sbn = 1;
   p.M = B; p.N = H; p.K = D;
@@ -825,8 +794,9 @@ int simt_forward(int dtype, int act, int64_t B, int64_t D, int64_t H, const void
 }
 
 namespace {
-GemmParams input_grad_params(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, const SimtInputGrad& ig) {
+GemmParams input_grad_params(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, const SimtInputGrad& ig, int32_t* dev_status) {
   GemmParams p = {};
+  p.dev_status = dev_status;
   p.A = dZ; p.sam = ldz; p.sak = 1;          // (b, h)
   p.Bm = ig.W; p.sbk = 1; p.sbn = ig.ldw;    // Bm(h, d) = W[d, h]
   p.M = B; p.N = D; p.K = H;
@@ -839,19 +809,19 @@ GemmParams input_grad_params(int64_t B, int64_t D, int64_t H, const void* dZ, in
 
 int simt_input_grad(int dtype, int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz,
                     const void* W, int64_t ldw, const uint32_t* relubits_prev, const void* z_prev,
-                    int64_t ld_zprev, void* dZ_prev, int64_t ldp, cudaStream_t s) {
+                    int64_t ld_zprev, void* dZ_prev, int64_t ldp, int32_t* dev_status, cudaStream_t s) {
   const SimtInputGrad ig = {W, ldw, relubits_prev, z_prev, ld_zprev, dZ_prev, ldp};
-  return launch_gemm<kEpiInputGrad>(dtype, input_grad_params(B, D, H, dZ, ldz, ig), B, s);
+  return launch_gemm<kEpiInputGrad>(dtype, input_grad_params(B, D, H, dZ, ldz, ig, dev_status), B, s);
 }
 
 int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, float* dW,
                      int64_t ldw, int32_t* dev_status, cudaStream_t s, float* db, bool* db_written,
                      const SimtInputGrad* ig, bool* ig_done) {
-  (void)dev_status;
   if (db_written != nullptr) *db_written = false;
   if (ig_done != nullptr) *ig_done = false;
   if (st->variant == RAD_SAME_SAMPLE) {
     GemmParams p = {};
+    p.dev_status = dev_status;
     p.A = st->values; p.sam = 1; p.sak = st->values_ld;     // A(j, b) = values[b, j]
     p.Bm = dZ; p.sbk = ldz; p.sbn = 1;
     p.M = min(st->values_ld, st->D); p.N = H; p.K = st->B;
@@ -860,20 +830,25 @@ int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H
     p.db = db;
     if (db_written != nullptr) *db_written = db != nullptr;
     const int es = st->dtype == RAD_BF16 ? 2 : 4;
-    plan_gemm(p, p.M, es);
+    const int64_t rows = std::min(p.M, (int64_t)(1.05 * st->p * (double)st->D) + 16);
     if (st->keepbits != nullptr) {
       // one launch: scatter, zeros for the rows not kept and, where asked for, the input gradient
       const bool with_dx = ig != nullptr && ig_done != nullptr;
-      GemmParams g = with_dx ? input_grad_params(st->B, st->D, H, dZ, ldz, *ig) : GemmParams{};
-      if (with_dx) plan_gemm(g, g.M, es);
+      GemmParams g = with_dx ? input_grad_params(st->B, st->D, H, dZ, ldz, *ig, dev_status) : GemmParams{};
+      if (with_dx) plan_joint(p, g, rows, es, 4, true); else plan_forms(p, rows, es);
       const int64_t cluster = std::max(p.splits, with_dx ? g.splits : 1);
       const int64_t dw_blocks = round_up(p.units, cluster), dx_blocks = with_dx ? round_up(g.units, cluster) : 0;
-      const int64_t nz = round_up(std::min<int64_t>(st->D, 148 * 2), cluster);
+      // zeros: two CTAs an SM where these fit beside the others, else the SMs the others leave (a tensor-core CTA has one)
+      const int64_t rest = kNumSms - (dw_blocks + dx_blocks) % kNumSms;
+      const int64_t nz = round_up(std::min<int64_t>(st->D, p.tc ? std::max<int64_t>(rest, 32) : 148 * 2), cluster);
       if (dw_blocks + dx_blocks + nz <= 0x7fffffff) {
         static std::atomic<uint64_t> ready_b{0}, ready_f{0};
         const dim3 grid((unsigned)(dw_blocks + dx_blocks + nz)), cl((unsigned)cluster);
-        count_launch();
         if (with_dx) *ig_done = true;
+        if (p.tc)
+          return launch_dw_dx_tc(kEpiScatterRows, p, with_dx ? &g : nullptr, dw_blocks, dx_blocks, nz, cluster,
+                                 (const uint32_t*)st->keepbits, st->D, H, s);
+        count_launch();
         if (st->dtype == RAD_BF16)
           return !allow_smem(same_dw_dx_kernel<bf16>, kGemmSmemBytes, ready_b) ? RAD_ECUDA
                  : launch_with_cluster(same_dw_dx_kernel<bf16>, grid, 256, kGemmSmemBytes, cl, s, p, g, (int)dw_blocks, (int)dx_blocks,
@@ -886,10 +861,11 @@ int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H
     const int g = (int)std::min<int64_t>(ceil_div(st->D * H, 256), 148 * 16);
     count_launch();
     RAD_TRY(launch_kernel(zero_rows_kernel, g, 256, 0, s, dW, ldw, st->D, H));
-    return launch_gemm<kEpiScatterRows>(st->dtype, p, std::max<int64_t>(p.M, 1), s);
+    return launch_gemm<kEpiScatterRows>(st->dtype, p, rows, s);
   }
   const bool low = st->dtype == RAD_BF16;
   GemmParams p = {};
+  p.dev_status = dev_status;
   p.A = st->values; p.keepbits = st->keepbits; p.offsets = st->offsets; p.capacity = st->values_capacity;
   p.ncb = (int32_t)ceil_div(st->D, kTileCols);
   p.Bm = dZ; p.sbk = ldz; p.sbn = 1;
@@ -897,18 +873,19 @@ int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H
   p.out_f32 = dW; p.ld_f32 = ldw;
   p.db = db;
   if (db_written != nullptr) *db_written = db != nullptr;
-  plan_gemm(p, p.M, low ? 2 : 4, kTileRows, false);
+  const int es = low ? 2 : 4;
   if (ig != nullptr && ig_done != nullptr) {
-    GemmParams g = input_grad_params(st->B, st->D, H, dZ, ldz, *ig);
-    plan_gemm(g, g.M, low ? 2 : 4);
+    GemmParams g = input_grad_params(st->B, st->D, H, dZ, ldz, *ig, dev_status);
+    plan_joint(p, g, p.M, es, kTileRows, false);
     const int64_t cluster = std::max(p.splits, g.splits), dw_blocks = round_up(p.units, cluster);
     const int64_t all = dw_blocks + round_up(g.units, cluster);
     if (all <= 0x7fffffff) {
       static std::atomic<uint64_t> ready_b{0}, ready_f{0};
       const size_t smem = (size_t)std::max(gemm_smem_bytes(g.tile), gemm_smem_bytes(p.tile));
       const dim3 grid((unsigned)all), cl((unsigned)cluster);
-      count_launch();
       *ig_done = true;
+      if (p.tc) return launch_dw_dx_tc(kEpiSparse, p, &g, dw_blocks, all - dw_blocks, 0, cluster, nullptr, 0, 0, s);
+      count_launch();
       if (low)
         return !allow_smem(dw_dx_kernel<bf16>, kGemmSmemBytes, ready_b) ? RAD_ECUDA
                : launch_with_cluster(dw_dx_kernel<bf16>, grid, 256, smem, cl, s, p, g, (int)dw_blocks);
@@ -916,6 +893,7 @@ int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H
              : launch_with_cluster(dw_dx_kernel<float>, grid, 256, smem, cl, s, p, g, (int)dw_blocks);
     }
   }
+  plan_forms(p, p.M, es, kTileRows, false);
   return launch_planned<kEpiSparse>(st->dtype, p, s);
 }
 

@@ -1,0 +1,124 @@
+"""float32 contractions on the tensor cores (three bf16 planes per operand) at the edges of their tiles of 128 x 128 and blocks of
+32: remainders of one, rows that do not begin on 16 bytes, strided operands, results that are not finite."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import rad as orc
+
+pytestmark = pytest.mark.gpu
+
+# All large enough for that form.  (rows, inputs, outputs, elements between rows beyond their length)
+SHAPES = [(1025, 513, 641, 0), (1024, 1024, 1024, 0), (769, 1001, 777, 0), (1000, 1000, 1300, 4), (1153, 897, 899, 3), (641, 130, 1921, 1)]
+
+
+def _strided(x, extra):
+    B, D = x.shape
+    t = torch.full((B, D + extra), float("nan"), device="cuda")
+    t[:, :D] = torch.from_numpy(np.ascontiguousarray(x))
+    return t[:, :D]
+
+
+def _close(got, want, magnitude, K):
+    """The planes drop less than 2^-24 of a product; the tensor core cuts off at most 2^-23 of a running sum in each of the four
+    MMAs of a block, a block's sum is rounded once: (K / 32) (4 * 2^-23 + 2^-24) of the sum of magnitudes, and what the last
+    additions round."""
+    bound = (K / 32 + 1) * 9 * 2.0 ** -24 * magnitude + 2.0 ** -22 * magnitude + 1e-30
+    assert (np.abs(got.double().cpu().numpy() - want) <= bound).all()
+
+
+@pytest.mark.parametrize("B,D,H,extra", SHAPES)
+@pytest.mark.parametrize("act", ["none", "relu", "gelu"])
+def test_forward_and_input_gradient(B, D, H, extra, act):
+    import paper_2007_10412_b200 as rad
+    rng = np.random.default_rng(B + D + H)
+    A, W, dZ, Z = (rng.standard_normal(s).astype(np.float32) for s in ((B, D), (D, H), (B, H), (B, D)))
+    bias = rng.standard_normal(H).astype(np.float32)
+    a, w, dz = _strided(A, extra), _strided(W, extra), _strided(dZ, extra)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = _strided(np.zeros((B, H), np.float32), extra)
+    z = torch.empty(B, H, device="cuda")
+    rad.rad_linear_forward(a, w, torch.from_numpy(bias).cuda(), act, out_act=out, out_z=z, dev_status=status)
+    want = A.astype(np.float64) @ W + bias
+    mag = np.abs(A).astype(np.float64) @ np.abs(W) + np.abs(bias)
+    _close(z, want, mag, D)
+    zt = z.double()
+    f = {"none": zt, "relu": zt.relu(), "gelu": torch.nn.functional.gelu(zt)}[act]
+    assert ((out.double() - f).abs() <= 2.0 ** -21 * zt.abs() + 1e-30).all()
+    dA = torch.full((B, D), float("nan"), device="cuda")
+    zp = torch.from_numpy(Z).cuda()
+    bits = torch.from_numpy(orc.pack_bits(Z > 0).view(np.int32)).cuda()
+    rad.rad_linear_input_grad(dz, w, relubits_prev=bits if act == "relu" else None, z_prev=zp if act == "gelu" else None, dZ_prev=dA, dev_status=status)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    d = torch.ones_like(zp).double()
+    if act == "relu":
+        d = (zp > 0).double()
+    elif act == "gelu":
+        zz = zp.double()
+        d = 0.5 * (1 + torch.erf(zz / 2 ** 0.5)) + zz * torch.exp(-0.5 * zz * zz) / (2 * np.pi) ** 0.5
+    d = d.cpu().numpy()
+    mag = np.abs(dZ).astype(np.float64) @ np.abs(W).T
+    _close(dA, (dZ.astype(np.float64) @ W.T) * d, mag * (np.abs(d) + 2.0 ** -2), H)
+
+
+@pytest.mark.parametrize("B,D,H,extra", SHAPES)
+@pytest.mark.parametrize("variant,p", [("different", 0.1), ("different", 1.0), ("same", 0.5), ("same", 1.0)])
+def test_weight_gradient(B, D, H, extra, variant, p):
+    import paper_2007_10412_b200 as rad
+    rng = np.random.default_rng(B + 2 * D + H)
+    A, dZ = rng.standard_normal((B, D)).astype(np.float32), rng.standard_normal((B, H)).astype(np.float32)
+    ref = orc.forward_store(A, "f32", variant, p, 5, 3, 1)
+    st = rad.Store(variant, "f32", B, D, p, seed=5, layer=3, step=1, relu_bits=False)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rad.rad_linear_forward_store(torch.from_numpy(A).cuda(), st, status)
+    dW = _strided(np.full((D, H), np.nan, np.float32), extra)
+    rad.rad_linear_weight_grad(st, _strided(dZ, extra), dW, dev_status=status)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    dense = np.zeros((B, D))
+    if variant == "different":
+        dense[orc.unpack_bits(ref.keepbits, D)] = ref.values
+    else:
+        dense[:, ref.idx] = np.asarray(ref.values, np.float64).reshape(B, -1)
+    _close(dW, dense.T @ dZ.astype(np.float64), np.abs(dense).T @ np.abs(dZ).astype(np.float64), B)
+
+
+@pytest.mark.parametrize("dims", [(513, 900, 641, 301), (512, 640, 640, 128)])
+@pytest.mark.parametrize("variant", ["different", "same"])
+@pytest.mark.parametrize("act", ["relu", "gelu"])
+def test_net_with_both_gradients_in_one_launch(dims, variant, act):
+    import paper_2007_10412_b200 as rad
+    from workloads import mlp_inputs
+    B = 1031
+    X, y, Ws, bs = mlp_inputs(dims, B, "f32", "normal", seed=2)
+    ref = orc.mlp_step(X, y, Ws, bs, dtype="f32", variant=variant, p=0.3, seed=4, act=act)
+    ctx = rad.MLPStep(dims, B, "f32", act, variant, 0.3)
+    ctx(torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda(), [torch.from_numpy(W).cuda() for W in Ws],
+        [torch.from_numpy(b).cuda() for b in bs], seed=4)
+    torch.cuda.synchronize()
+    assert ctx.dev_status.item() == 0
+    for l in range(len(Ws)):
+        for g, r in ((ctx.dW[l], ref.dW[l]), (ctx.db[l], ref.db[l])):
+            assert np.linalg.norm(g.double().cpu().numpy() - r) <= 1e-5 * np.linalg.norm(r), l
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("-inf"), float("nan"), 3.4e38])
+def test_results_that_are_not_finite_stay_in_their_cells(bad):
+    """An infinity has no planes: what it reaches is added up as the CUDA-core form does it, and nothing else changes."""
+    import paper_2007_10412_b200 as rad
+    B, D, H = 700, 900, 800
+    g = torch.Generator(device="cuda").manual_seed(7)
+    A, W = torch.randn(B, D, device="cuda", generator=g), torch.randn(D, H, device="cuda", generator=g).abs() + 0.5
+    clean, out = torch.empty(B, H, device="cuda"), torch.empty(B, H, device="cuda")
+    rad.rad_linear_forward(A, W, None, "none", out_act=clean)
+    A[130, 33] = bad
+    rad.rad_linear_forward(A, W, None, "none", out_act=out)
+    want = A[130].double() @ W.double()
+    if abs(bad) < float("inf"):
+        over = want.abs() > 3.5e38
+        assert over.any() and not over.all() and torch.isinf(out[130][over]).all() and torch.isfinite(out[130][want.abs() < 3.3e38]).all()
+    else:
+        assert torch.equal(out[130].nan_to_num(), want.float().nan_to_num())
+    rest = torch.arange(B, device="cuda") != 130
+    assert torch.equal(out[rest], clean[rest])
