@@ -185,8 +185,11 @@ extern "C" int rad_cnn_step(const rad_cnn_desc* d, const void* X, const int32_t*
     rc = store_input(a_in, l);
     if (rc != RAD_OK) return rc;
     void* a_out = ws + pl.act[l & 1];
-    // tensor cores where the shape allows (Cin 16 / 32 / 64: the later convolutions), CUDA cores otherwise
-    if (conv_tc_ok(d->dtype, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], a_in, conv_W[l]))
+    // tensor cores where the shape allows (bf16, up to eight or 16 / 32 / 64 channels), CUDA cores otherwise
+    if (conv_stage_forward_ok(d->dtype, B, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], a_in, conv_W[l], a_out))
+      rc = conv_stage_forward_pool(B, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], a_in, conv_W[l], conv_b != nullptr ? conv_b[l] : nullptr, a_out,
+                                   reinterpret_cast<uint32_t*>(ws + pl.relubits[l]), dev_status, s);
+    else if (conv_tc_ok(d->dtype, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], a_in, conv_W[l]))
       rc = conv_tc_forward_pool(B, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], a_in, conv_W[l],
                                 conv_b != nullptr ? conv_b[l] : nullptr, a_out, reinterpret_cast<uint32_t*>(ws + pl.relubits[l]),
                                 dev_status, s);
@@ -262,7 +265,9 @@ extern "C" int rad_cnn_step(const rad_cnn_desc* d, const void* X, const int32_t*
     if (rc != RAD_OK) return rc;
     if (l > 0) {
       void* g_prev = ws + pl.grad[(l - 1) & 1];
-      if (conv_tc_dx_ok(d->dtype, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], dz, conv_W[l], g_prev))
+      if (conv_stage_dx_ok(d->dtype, B, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], dz, conv_W[l], g_prev))
+        rc = conv_stage_input_grad(B, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], dz, conv_W[l], g_prev, dev_status, s);
+      else if (conv_tc_dx_ok(d->dtype, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], dz, conv_W[l], g_prev))
         rc = conv_tc_input_grad(B, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], dz, conv_W[l], g_prev, dev_status, s);
       else
         rc = conv_input_grad(d->dtype, B, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], dz, conv_W[l], g_prev, s);

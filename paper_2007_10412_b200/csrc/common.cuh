@@ -311,6 +311,15 @@ bool conv_tc_dx_ok(int dtype, int H, int W, int Cin, int Cout, const void* dZ, c
 int conv_tc_input_grad(int64_t B, int H, int W, int Cin, int Cout, const void* dZ, const void* Wt, void* dX, int32_t* dev_status,
                        cudaStream_t st);
 
+// the same from staged images (conv_stage.cu): forward and input gradient of images that fit a CTA's shared memory
+bool conv_tensor_allowed();       // rad_set_conv_kernel
+bool conv_stage_forward_ok(int dtype, int64_t B, int H, int W, int Cin, int Cout, const void* X, const void* Wt, const void* P);
+int conv_stage_forward_pool(int64_t B, int H, int W, int Cin, int Cout, const void* X, const void* Wt, const float* bias, void* P,
+                            uint32_t* relubits, int32_t* dev_status, cudaStream_t st);
+bool conv_stage_dx_ok(int dtype, int64_t B, int H, int W, int Cin, int Cout, const void* dZ, const void* Wt, const void* dX);
+int conv_stage_input_grad(int64_t B, int H, int W, int Cin, int Cout, const void* dZ, const void* Wt, void* dX, int32_t* dev_status,
+                          cudaStream_t st);
+
 // tcgen05 kernels (bf16, aligned)
 bool tc_shape_ok(int64_t B, int64_t D, int64_t H, const void* p0, int64_t ld0, const void* p1,
                  int64_t ld1);

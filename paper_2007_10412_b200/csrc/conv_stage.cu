@@ -1,0 +1,401 @@
+// 3x3 convolutions on the tensor cores from staged images: forward with pooling, and input gradient (bf16, NHWC, zero padding
+// 1).  The patch-gathering kernels of conv_tc.cu read every pixel nine times, once per tap, through registers; here a CTA brings
+// whole images into shared memory once, in planes of 16 bytes (eight channels) per pixel, pixel after pixel.  Eight such
+// pixels are a core matrix of a K-major operand without swizzle, and a descriptor may begin at any pixel, so the A operand of
+// a tap is the same plane at another start address: no patch matrix exists anywhere.
+//
+//   forward         the padded image lies in four planes by the parity of row and column.  A row of the MMA is a pooling window,
+//                   its four pixels are four accumulators side by side in tensor memory (the pixels of the windows at one place in
+//                   them read one plane per tap, shifted by whole windows), so a thread holds the whole window: bias, ReLU, four
+//                   derivative bits and the average need no exchange.
+//   input gradient  dX[pixel] = sum over taps of dZ[pixel - tap] W[tap]: one plane of the padded dZ; a row of the MMA is a pixel.
+// Rows that are no window or pixel (the padding between image rows and images) compute something that is not written.
+// Up to eight input channels (a first convolution) fill one plane of sixteen bytes; K = 16 then takes two taps, whose
+// distance is the descriptor's: (ty, 0) and (ty, 2), (0, 1) and (2, 1), and (1, 1) with a plane of zeros.
+// A CTA keeps the filters and goes from one group of images to the next; two or three CTAs on an SM hide each other's copies,
+// MMAs and epilogues.  What bounds it: instruction issue of the forward epilogue (about ten per conv output), then the copies.
+#include <algorithm>
+#include <cfloat>
+
+#include "common.cuh"
+#include "umma.cuh"
+
+namespace rad {
+namespace {
+
+constexpr int kCsThreads = 256;
+constexpr int kCsStageMax = 56 * 1024;           // staged images of a CTA, unless one image needs more
+
+struct ConvStageParams {
+  int64_t B;
+  int32_t H, W, Cin, Cout;
+  const bf16* A;            // forward: conv input; input gradient: dZ
+  const bf16* Wt;           // 3 x 3 x Cin x Cout
+  const float* bias;
+  bf16* out;                // forward: pooled output; input gradient: dX
+  uint32_t* relubits;
+  int32_t G, tiles, chunks, npad, cols, chunk_stride, b_bytes;       // images of a group, its tiles of 128 rows, 16-byte planes, ...
+  int32_t raw_bytes;        // up to eight channels: a group's images as they are in memory, or 0: read entry by entry
+  int64_t groups;
+  int32_t* dev_status;
+  uint64_t wait_limit_ns;
+};
+struct CsCtl {
+  uint64_t done;
+  uint32_t tmem;
+  int abort_flag;
+  float bias[64];
+};
+
+// Descriptor without swizzle, K-major: 8 rows of 16 bytes are 128 contiguous bytes, the next eight rows follow; `lbo` bytes to
+// the second eight of K.
+__device__ __forceinline__ uint64_t cs_desc(uint32_t saddr, uint32_t lbo) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) | (1ull << 46);
+}
+__device__ __forceinline__ void cs_tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+}
+// the wait names the registers: nothing that uses them moves in front of it
+__device__ __forceinline__ void cs_tmem_wait8(uint32_t (&r)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]) :: "memory");
+}
+
+// A conv output whose sum is not finite, added up over the taps inside the image alone (the padding's zeros times an infinite
+// filter are no numbers).
+__device__ __noinline__ float cs_plain(const ConvStageParams& p, int64_t img, int y, int x, int co) {
+  float z = 0.0f;
+  for (int t = 0; t < 9; ++t) {
+    const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
+    if (yy < 0 || yy >= p.H || xx < 0 || xx >= p.W) continue;
+    const bf16* a = p.A + ((img * p.H + yy) * p.W + xx) * p.Cin;
+    for (int c = 0; c < p.Cin; ++c) z = fmaf(__bfloat162float(a[c]), __bfloat162float(p.Wt[((int64_t)t * p.Cin + c) * p.Cout + co]), z);
+  }
+  return z;
+}
+
+// The outputs of a window that are not finite, out of line.
+__device__ __noinline__ void cs_repair(const ConvStageParams& p, int64_t img, int y, int x, int c0, uint32_t (&r)[4][8]) {
+  for (int q = 0; q < 4; ++q)
+    for (int c = 0; c < 8; ++c)
+      if (!(fabsf(__uint_as_float(r[q][c])) <= FLT_MAX)) r[q][c] = __float_as_uint(cs_plain(p, img, y + (q >> 1), x + (q & 1), c0 + c));
+}
+
+template <bool kDx>
+__global__ void __launch_bounds__(kCsThreads, 3) conv_stage_kernel(const __grid_constant__ ConvStageParams p) {
+  extern __shared__ uint8_t cs_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(cs_raw) + 127) & ~(uintptr_t)127);
+  constexpr int kPlanes = kDx ? 1 : 4;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int H = p.H, W = p.W, C = kDx ? p.Cout : p.Cin, N = kDx ? p.Cin : p.Cout;
+  const int Pw = kDx ? W + 2 : (W >> 1) + 1, Ph = kDx ? H + 2 : (H >> 1) + 1, NP = Ph * Pw;        // places of a plane per image
+  const int plane = p.chunks * p.chunk_stride;
+  uint8_t* sB = smem + kPlanes * plane + (p.chunks == 1 ? 128 * 16 : 0);       // behind the planes: zeros for the tap without a partner
+  CsCtl* ctl = reinterpret_cast<CsCtl*>(sB + p.b_bytes);
+  volatile int* abort_flag = &ctl->abort_flag;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(umma_smem(&ctl->tmem)), "r"((uint32_t)p.cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 32) {
+    umma_init_barriers(&ctl->done, 1);
+    ctl->abort_flag = 0;
+  }
+  // zeros around the images (and where a tap without a partner reads): copies of images leave them as they are
+  for (int i = tid * 16; i < kPlanes * plane + (p.chunks == 1 ? 128 * 16 : 0); i += kCsThreads * 16) *reinterpret_cast<uint4*>(smem + i) = make_uint4(0u, 0u, 0u, 0u);
+  wait_for_previous();
+  __syncthreads();
+  // ---- images: a warp per line, 16 bytes (eight channels of a pixel) a lane; those of few channels come as they are first ----
+  uint8_t* raw = reinterpret_cast<uint8_t*>(ctl) + ((sizeof(CsCtl) + 15) & ~15);
+  const int log_c = 31 - __clz(p.chunks), per_line = W << log_c;
+  auto for_pixels = [&](int nimg, auto f) {           // f(destination, first entry of the eight in the group's images)
+    for (int line = warp; line < nimg * H; line += kCsThreads / 32) {
+      const int g = line / H, y = line - g * H + 1;
+      uint8_t* dst = smem + (kDx ? (g * NP + y * Pw) * 16 : 2 * (y & 1) * plane + (g * NP + (y >> 1) * Pw) * 16);
+      for (int i = lane; i < per_line; i += 32) {
+        const int c8 = i & (p.chunks - 1), x = (i >> log_c) + 1;
+        f(dst + c8 * p.chunk_stride + (kDx ? x * 16 : (x & 1) * plane + (x >> 1) * 16), (int64_t)line * W * C + (x - 1) * C + 8 * c8);
+      }
+    }
+  };
+  auto fetch = [&](int64_t group) {                   // asynchronous
+    const int nimg = (int)min((int64_t)p.G, p.B - group * p.G);
+    const bf16* images = p.A + group * p.G * H * W * C;
+    if (p.chunks > 1) {
+      for_pixels(nimg, [&](uint8_t* to, int64_t at) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(umma_smem(to)), "l"(images + at) : "memory");
+      });
+    } else if (p.raw_bytes > 0) {
+      const int bytes = nimg * H * W * C * 2;
+      for (int i = tid * 16; i < bytes; i += kCsThreads * 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(umma_smem(raw + i)), "l"(reinterpret_cast<const uint8_t*>(images) + i) : "memory");
+    }
+  };
+  fetch(blockIdx.x);
+  // ---- filters: (tap, eight of K, output column) of 16 bytes; columns and channels that there are not are zeros ----
+  {
+    const int kc = p.chunks, cols8 = p.npad >> 3, items = (9 * kc + (kc == 1 ? 1 : 0)) * cols8;
+    for (int i = tid; i < items; i += kCsThreads) {
+      const int row = i / cols8, o = i - row * cols8, t = row / kc, c8 = row - t * kc;
+      uint4 in[8], out[8];
+      if (kDx) {
+        // a column is an input channel: its eight output channels are neighbours in the filter
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          out[c] = 8 * o + c < N ? *reinterpret_cast<const uint4*>(p.Wt + ((int64_t)t * p.Cin + 8 * o + c) * p.Cout + 8 * c8) : make_uint4(0u, 0u, 0u, 0u);
+      } else {
+        // eight channels (rows of the filter) by eight columns, turned
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          in[c] = t < 9 && 8 * c8 + c < C && 8 * o < N ? *reinterpret_cast<const uint4*>(p.Wt + ((int64_t)t * C + 8 * c8 + c) * N + 8 * o) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+          uint32_t w[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            w[e] = __byte_perm(reinterpret_cast<const uint32_t*>(&in[2 * e])[n >> 1], reinterpret_cast<const uint32_t*>(&in[2 * e + 1])[n >> 1], (n & 1) ? 0x7632 : 0x5410);
+          out[n] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+      }
+#pragma unroll
+      for (int n = 0; n < 8; ++n) *reinterpret_cast<uint4*>(sB + (row * p.npad + 8 * o + n) * 16) = out[n];
+    }
+    if (!kDx && tid < 64) ctl->bias[tid] = p.bias != nullptr && tid < N ? p.bias[tid] : 0.0f;
+  }
+  umma_fence_before();
+  __syncthreads();
+  umma_fence_after();
+  const uint32_t tmem = ctl->tmem;
+  uint32_t phase = 0;
+  bool ok = true;
+  for (int64_t group = blockIdx.x; group < p.groups && ok; group += gridDim.x) {
+    if (group + gridDim.x >= p.groups) let_next_start();
+    const int64_t img0 = group * p.G;
+    const int nimg = (int)min((int64_t)p.G, p.B - img0);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (p.chunks == 1) {
+      if (p.raw_bytes > 0) __syncthreads();
+      const uint16_t* from = p.raw_bytes > 0 ? reinterpret_cast<const uint16_t*>(raw) : reinterpret_cast<const uint16_t*>(p.A + img0 * H * W * C);
+      for_pixels(nimg, [&](uint8_t* to, int64_t at) {
+        uint32_t e[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) e[c] = c < C ? (uint32_t)from[at + c] : 0u;
+        *reinterpret_cast<uint4*>(to) = make_uint4(e[0] | e[1] << 16, e[2] | e[3] << 16, e[4] | e[5] << 16, e[6] | e[7] << 16);
+      });
+    }
+    umma_fence_smem();
+    __syncthreads();
+    const int64_t next = group + gridDim.x;
+    if (p.chunks == 1 && next < p.groups) fetch(next);          // its images go where these have been read
+
+    for (int tile = 0; tile < p.tiles && ok; ++tile) {
+      if (warp == 0 && elect_one()) {
+        umma_fence_after();
+        const uint32_t a0 = umma_smem(smem) + (uint32_t)(tile * 128 * 16), b0 = umma_smem(sB);
+        const uint32_t idesc = umma_idesc(128, p.npad, false, false);
+        const uint32_t nb = (uint32_t)p.npad * 16u, cs = (uint32_t)p.chunk_stride;
+        if (p.chunks > 1) {
+          for (int cls = 0; cls < kPlanes; ++cls) {
+            for (int t = 0; t < 9; ++t) {
+              const int ty = t / 3, tx = t - 3 * ty;
+              // forward: pixel (py, px) of the window reads padded row 2 wy + py + ty; input gradient: padded row y + 2 - ty
+              const int ry = kDx ? 2 - ty : (cls >> 1) + ty, rx = kDx ? 2 - tx : (cls & 1) + tx;
+              const uint32_t at = a0 + (kDx ? (uint32_t)(ry * Pw + rx) * 16u
+                                            : (uint32_t)((2 * (ry & 1) + (rx & 1)) * plane) + (uint32_t)((ry >> 1) * Pw + (rx >> 1)) * 16u);
+              for (int c = 0; c < p.chunks; c += 2)
+                umma_mma(tmem + (uint32_t)(cls * p.npad), cs_desc(at + (uint32_t)c * cs, cs), cs_desc(b0 + (uint32_t)(t * p.chunks + c) * nb, nb), idesc,
+                         t > 0 || c > 0 ? 1u : 0u);
+            }
+          }
+        } else {
+          for (int cls = 0; cls < kPlanes; ++cls) {
+            auto place = [&](int ty, int tx) {
+              const int ry = (cls >> 1) + ty, rx = (cls & 1) + tx;
+              return (uint32_t)((2 * (ry & 1) + (rx & 1)) * plane) + (uint32_t)((ry >> 1) * Pw + (rx >> 1)) * 16u;
+            };
+            const uint32_t d = tmem + (uint32_t)(cls * p.npad);
+            for (int ty = 0; ty < 3; ++ty)               // (ty, 0) and (ty, 2): neighbours in one plane
+              umma_mma(d, cs_desc(a0 + place(ty, 0), 16u), cs_desc(b0 + (uint32_t)(3 * ty) * nb, 2u * nb), idesc, ty > 0 ? 1u : 0u);
+            umma_mma(d, cs_desc(a0 + place(0, 1), (uint32_t)Pw * 16u), cs_desc(b0 + nb, 6u * nb), idesc, 1u);       // (0, 1) and (2, 1)
+            const uint32_t mid = a0 + place(1, 1);
+            umma_mma(d, cs_desc(mid, umma_smem(smem) + (uint32_t)(kPlanes * plane) - mid), cs_desc(b0 + 4u * nb, 5u * nb), idesc, 1u);
+          }
+        }
+        umma_commit(umma_smem(&ctl->done));
+      }
+      __syncwarp();
+      ok = __all_sync(0xffffffffu, umma_wait(umma_smem(&ctl->done), phase, abort_flag, p.wait_limit_ns));
+      phase ^= 1u;
+      umma_fence_after();
+      if (p.chunks > 1 && ok && tile + 1 == p.tiles && next < p.groups) fetch(next);       // the last MMAs have read the planes
+      if (ok) {
+        const int m = tile * 128 + 32 * (warp & 3) + lane, g = m / NP, rem = m - g * NP, wy = rem / Pw, wx = rem - wy * Pw;
+        const bool in = g < nimg && wy < (kDx ? H : H >> 1) && wx < (kDx ? W : W >> 1);
+        const int64_t pix = ((img0 + g) * (kDx ? H : H >> 1) + wy) * (kDx ? W : W >> 1) + wx;
+        const uint32_t row = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+        for (int c0 = 8 * (warp >> 2); c0 < N; c0 += 16) {
+          if (kDx) {
+            uint32_t r[8];
+            cs_tmem_ld8(row + (uint32_t)c0, r);
+            cs_tmem_wait8(r);
+            if (in) {
+              uint32_t w[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1]));
+                w[e] = *reinterpret_cast<const uint32_t*>(&h2);
+              }
+              *reinterpret_cast<uint4*>(p.out + pix * N + c0) = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+          } else {
+            uint32_t r[4][8];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) cs_tmem_ld8(row + (uint32_t)(q * p.npad + c0), r[q]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) cs_tmem_wait8(r[q]);
+            if (in) {
+              // a sum of zeros times the values is not zero where one of them is not finite
+              float odd = 0.0f;
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int c = 0; c < 8; ++c) odd = fmaf(__uint_as_float(r[q][c]), 0.0f, odd);
+              if (odd != 0.0f) {
+                uint32_t whole[4][8];                  // what is passed by address lies in memory
+#pragma unroll
+                for (int i = 0; i < 32; ++i) whole[i >> 3][i & 7] = r[i >> 3][i & 7];
+                cs_repair(p, img0 + g, 2 * wy, 2 * wx, c0, whole);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) r[i >> 3][i & 7] = whole[i >> 3][i & 7];
+              }
+              uint32_t word = 0, packed[4];
+#pragma unroll
+              for (int c = 0; c < 8; c += 2) {
+                const float2 b2 = *reinterpret_cast<const float2*>(&ctl->bias[c0 + c]);
+                float lo[4], hi[4];
+                uint32_t bits = 0;                       // derivative bits of the two channels from bits 0 and 16 on
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                  // the activations as the device would hold them: two bf16, which are above zero where any bit is set
+                  const __nv_bfloat162 a2 = __floats2bfloat162_rn(fmaxf(__uint_as_float(r[q][c]) + b2.x, 0.0f), fmaxf(__uint_as_float(r[q][c + 1]) + b2.y, 0.0f));
+                  const uint32_t a = *reinterpret_cast<const uint32_t*>(&a2);
+                  bits |= ((a + 0x7fff7fffu) & 0x80008000u) >> (15 - q);
+                  lo[q] = __uint_as_float(a << 16);
+                  hi[q] = __uint_as_float(a & 0xffff0000u);
+                }
+                word |= ((bits & 15u) | (bits >> 12)) << (4 * c);
+                const __nv_bfloat162 h2 = __floats2bfloat162_rn(0.25f * (((lo[0] + lo[1]) + lo[2]) + lo[3]), 0.25f * (((hi[0] + hi[1]) + hi[2]) + hi[3]));
+                packed[c >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
+              }
+              *reinterpret_cast<uint4*>(p.out + pix * N + c0) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+              p.relubits[(pix * N + c0) >> 3] = word;
+            }
+          }
+        }
+      }
+      umma_fence_before();
+      ok = __syncthreads_and(ok ? 1 : 0) != 0;           // everyone has read the accumulators
+    }
+  }
+  if (tid == 0 && ctl->abort_flag != 0) raise_status(p.dev_status, RAD_DEV_ETIMEOUT);
+  if (warp == 0) {
+    umma_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)p.cols) : "memory");
+  }
+}
+
+// Images of a group and what follows from it: the fewest rounds of tiles over the chip (three CTAs an SM), a group's copies
+// counted as a tile and a half.  False: one image does not fit.
+template <bool kDx>
+bool plan_stage(ConvStageParams& p, size_t* smem) {
+  const int C = kDx ? p.Cout : p.Cin, N = kDx ? p.Cin : p.Cout, planes = kDx ? 1 : 4;
+  const int Pw = kDx ? p.W + 2 : p.W / 2 + 1, NP = Pw * (kDx ? p.H + 2 : p.H / 2 + 1), reach = kDx ? 2 * Pw + 2 : Pw + 1;
+  p.chunks = C <= 8 ? 1 : C / 8;
+  p.npad = (int)round_up(N, 16);
+  p.cols = 32;
+  while (p.cols < (kDx ? 1 : 4) * p.npad) p.cols *= 2;
+  p.b_bytes = (9 * p.chunks + (p.chunks == 1 ? 1 : 0)) * p.npad * 16;
+  double best = 1e300;
+  for (int G = 1; G <= 12; ++G) {
+    // rows up to the last window or pixel of the last image; behind them the reach of the taps
+    const int last = (G - 1) * NP + (kDx ? (p.H - 1) * Pw + p.W : (p.H / 2 - 1) * Pw + p.W / 2), tiles = (int)ceil_div(last, 128);
+    const int places = std::max(G * NP, tiles * 128 + reach), stride = (int)round_up(places, 8) * 16;
+    const size_t stage = (size_t)planes * p.chunks * stride;
+    // images of few channels come through shared memory as they are, where a group of them is whole vectors
+    const int64_t image = (int64_t)p.H * p.W * C * 2;
+    const int raw = p.chunks == 1 && image % 16 == 0 && ((uintptr_t)p.A & 15) == 0 ? (int)(G * image) : 0;
+    const size_t all = stage + (p.chunks == 1 ? 128 * 16 : 0) + (size_t)p.b_bytes + ((sizeof(CsCtl) + 15) & ~(size_t)15) + (size_t)raw + 128;
+    if (all > 220 * 1024 || (G > 1 && stage > kCsStageMax)) break;
+    const double cost = (double)ceil_div(ceil_div(p.B, G), 3 * kNumSms) * (tiles + 1.5);
+    if (cost < best) {
+      best = cost;
+      p.G = G; p.tiles = tiles; p.chunk_stride = stride; p.raw_bytes = raw;
+      p.groups = ceil_div(p.B, G);
+      *smem = all;
+    }
+  }
+  return best < 1e300;
+}
+
+template <bool kDx>
+int launch_stage(const ConvStageParams& p, size_t smem, cudaStream_t st) {
+  RAD_CUDA_TRY(cudaFuncSetAttribute(conv_stage_kernel<kDx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>({3, 512 / p.cols, (int64_t)(227 * 1024 / (smem + 1024))}));
+  count_launch();
+  return launch_kernel(conv_stage_kernel<kDx>, (unsigned)std::min(p.groups, per_sm * kNumSms), kCsThreads, smem, st, p);
+}
+
+ConvStageParams stage_shape(int64_t B, int H, int W, int Cin, int Cout) {
+  ConvStageParams p = {};
+  p.B = B; p.H = H; p.W = W; p.Cin = Cin; p.Cout = Cout;
+  p.wait_limit_ns = wait_limit_ns();
+  return p;
+}
+
+}  // namespace
+
+// Where images are many: a CTA's way in (filters, first images, first MMAs) takes 9 us whatever the batch.  Images of 32 x 32 x 3
+// to 16 channels: 12.5 us against 13.3 on CUDA cores at 256 (65536 windows), 11.1 against 7.2 at 64, 79 against 148 at 4096; 16 x 16 x
+// 16 to 32: 11.8 against 14.2 from gathered patches at 256, 10.6 against 9.8 at 128 (8192 windows), 61 against 148 at 4096; 8 x 8 x
+// 32 to 64: 24.5 against 18.5 at 1024 (16384 windows), 38 against 54 at 4096.  Input gradients: 8 x 8 x 64 to 32 9.7 against 13.8
+// at 128, 44 against 76 at 4096; 16 x 16 x 32 to 16 9.8 against 11.1 at 128, 9.5 against 8.9 at 64 (16384 pixels), 63 against 164.
+static bool many_windows(int64_t B, int H, int W, int Cin) {
+  return B * (H / 2) * (W / 2) >= (Cin <= 8 ? 57344 : Cin == 16 ? 12288 : 28672);
+}
+static bool many_pixels(int64_t B, int H, int W, int Cout) { return B * H * W >= (Cout == 64 ? 4096 : 24576); }
+
+bool conv_stage_forward_ok(int dtype, int64_t B, int H, int W, int Cin, int Cout, const void* X, const void* Wt, const void* P) {
+  if (dtype != RAD_BF16 || !many_windows(B, H, W, Cin) || ((uintptr_t)Wt & 15) != 0 || !conv_tensor_allowed() || H % 2 != 0 || W % 2 != 0 || Cout % 8 != 0 || Cout < 8 || Cout > 64 || ((uintptr_t)P & 15) != 0) return false;
+  if (Cin > 8 && ((Cin != 16 && Cin != 32 && Cin != 64) || ((uintptr_t)X & 15) != 0)) return false;
+  ConvStageParams p = stage_shape(B, H, W, Cin, Cout);
+  size_t smem = 0;
+  return plan_stage<false>(p, &smem);
+}
+int conv_stage_forward_pool(int64_t B, int H, int W, int Cin, int Cout, const void* X, const void* Wt, const float* bias, void* P,
+                            uint32_t* relubits, int32_t* dev_status, cudaStream_t st) {
+  ConvStageParams p = stage_shape(B, H, W, Cin, Cout);
+  size_t smem = 0;
+  p.A = static_cast<const bf16*>(X);
+  if (!plan_stage<false>(p, &smem)) return RAD_EINVAL;
+  p.Wt = static_cast<const bf16*>(Wt); p.bias = bias; p.out = static_cast<bf16*>(P);
+  p.relubits = relubits; p.dev_status = dev_status;
+  return launch_stage<false>(p, smem, st);
+}
+
+bool conv_stage_dx_ok(int dtype, int64_t B, int H, int W, int Cin, int Cout, const void* dZ, const void* Wt, const void* dX) {
+  if (!conv_tc_dx_ok(dtype, H, W, Cin, Cout, dZ, Wt, dX) || !many_pixels(B, H, W, Cout)) return false;
+  ConvStageParams p = stage_shape(B, H, W, Cin, Cout);
+  size_t smem = 0;
+  return plan_stage<true>(p, &smem);
+}
+int conv_stage_input_grad(int64_t B, int H, int W, int Cin, int Cout, const void* dZ, const void* Wt, void* dX, int32_t* dev_status,
+                          cudaStream_t st) {
+  ConvStageParams p = stage_shape(B, H, W, Cin, Cout);
+  size_t smem = 0;
+  if (!plan_stage<true>(p, &smem)) return RAD_EINVAL;
+  p.A = static_cast<const bf16*>(dZ); p.Wt = static_cast<const bf16*>(Wt); p.out = static_cast<bf16*>(dX); p.dev_status = dev_status;
+  return launch_stage<true>(p, smem, st);
+}
+
+}  // namespace rad

@@ -353,6 +353,8 @@ int g_conv_kernel = RAD_CONV_KERNEL_AUTO;
 
 }  // namespace
 
+bool conv_tensor_allowed() { return g_conv_kernel != RAD_CONV_KERNEL_SIMT; }
+
 // Shapes the tensor-core kernels take: bf16, Cin 16, 32 or 64 (a 64-deep K block is a whole number of taps),
 // Cout a multiple of 8 up to 64, even H and W.
 bool conv_tc_ok(int dtype, int H, int W, int Cin, int Cout, const void* X, const void* Wt) {

@@ -1,0 +1,81 @@
+"""Convolutions from staged images (forward with pooling, input gradient): batches that leave a group of images incomplete, image sizes
+whose places are no multiple of a tile, channel counts that are padded, against the CUDA-core kernels and the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import cnn as orc
+from workloads import cnn_inputs
+
+from gpu_util import TOL, rel_err, to_dev
+
+pytestmark = pytest.mark.gpu
+
+# batches large enough for the staged form in (convolution, input gradient) of every case
+CASES = [
+    # B, hw, cin, channels, fc
+    (259, 32, 3, (16, 32), (5,)),
+    (1031, 16, 5, (16, 24, 8), (5,)),        # input gradient from 24 channels: gathered
+    (3701, 8, 8, (32, 64), (3,)),
+    (14339, 4, 1, (8, 16), (3,)),            # images of 4 x 4, then 2 x 2
+    (901, 16, 16, (64, 16), (4,)),
+]
+
+
+def _step(rad, case, kernel, data):
+    B, hw, cin, channels, fc = case
+    X, y, cW, cb, fW, fb = data
+    prev = rad.rad_set_conv_kernel(kernel)
+    try:
+        ctx = rad.CNNStep(B, hw, cin, channels, fc, "bf16", "different", 0.3)
+        ctx(to_dev(X, "bf16"), torch.from_numpy(y).cuda(), [to_dev(w, "bf16") for w in cW], [to_dev(b, "f32") for b in cb],
+            [to_dev(w, "bf16") for w in fW], [to_dev(b, "f32") for b in fb], seed=3, step=2)
+        torch.cuda.synchronize()
+    finally:
+        rad.rad_set_conv_kernel(prev)
+    assert ctx.dev_status.item() == 0
+    return ctx
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_staged_convolutions_against_the_cuda_cores(case):
+    """Whole steps with either set of kernels: products and sums are float32 in both, so activations differ by bf16 roundings."""
+    import paper_2007_10412_b200 as rad
+    B, hw, cin, channels, fc = case
+    data = cnn_inputs(B, hw, cin, channels, fc, "bf16", seed=B, bias_zero=False)
+    a, b = _step(rad, case, "simt", data), _step(rad, case, "tensor", data)
+    assert abs(a.loss.item() - b.loss.item()) <= 2e-3 * abs(a.loss.item())
+    assert torch.equal(a.nnz, b.nnz)
+    for x, y in zip(a.dconv_W + a.dconv_b + a.dfc_W + a.dfc_b, b.dconv_W + b.dconv_b + b.dfc_W + b.dfc_b):
+        fro, mx = rel_err(y.double().cpu().numpy(), x.double().cpu().numpy())
+        assert fro <= TOL["bf16"] and mx <= 2 * TOL["bf16"], (fro, mx)
+
+
+def test_staged_convolutions_against_the_oracle():
+    import paper_2007_10412_b200 as rad
+    case = (257, 32, 3, (16, 32), (5,))
+    B, hw, cin, channels, fc = case
+    data = cnn_inputs(B, hw, cin, channels, fc, "bf16", seed=5, bias_zero=False)
+    X, y, cW, cb, fW, fb = data
+    ref = orc.cnn_step(X, y, cW, cb, fW, fb, dtype="bf16", variant="different", p=0.3, seed=3, step=2)
+    ctx = _step(rad, case, "tensor", data)
+    for got, want in zip(ctx.dconv_W + ctx.dconv_b + ctx.dfc_W + ctx.dfc_b, ref.dW_conv + ref.db_conv + ref.dW_fc + ref.db_fc):
+        fro, mx = rel_err(got.double().cpu().numpy(), want)
+        assert fro <= TOL["bf16"] and mx <= 2 * TOL["bf16"], (fro, mx)
+
+
+def test_an_infinite_filter_is_not_multiplied_with_padding():
+    """A corner tap of -inf on a positive image: outputs it reaches are 0 behind the ReLU, those on the border it does not reach
+    (the padding's zeros times an infinity are no numbers) are what the other taps make of them."""
+    import paper_2007_10412_b200 as rad
+    case = (260, 32, 3, (16,), (3,))
+    B, hw, cin, channels, fc = case
+    X, y, cW, cb, fW, fb = cnn_inputs(B, hw, cin, channels, fc, "bf16", seed=8, bias_zero=False)
+    X, cW = np.abs(X) + np.float32(0.125), [np.abs(cW[0])]
+    cW[0][0, 0, 0, 2] = -1e30
+    want = _step(rad, case, "tensor", (X, y, cW, cb, fW, fb))
+    cW[0][0, 0, 0, 2] = -np.inf
+    got = _step(rad, case, "tensor", (X, y, cW, cb, fW, fb))
+    assert torch.isfinite(got.loss).all() and torch.equal(got.loss, want.loss)
+    for g, w in zip(got.dconv_b + got.dfc_W + got.dfc_b, want.dconv_b + want.dfc_W + want.dfc_b):
+        assert torch.equal(g, w)
