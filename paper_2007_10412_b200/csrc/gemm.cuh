@@ -41,7 +41,7 @@ struct GemmParams {
 // float32 on the tensor cores (gemm_tc.cu): the plan for M rows of C (the rows expected where the device alone knows them; the
 // grid covers p.M), its estimated time in clocks of an SM, and its launches.  A joint launch
 // takes the CTAs of dW, of the input gradient (g may be NULL) and of the zeros of a same-sample dW, all multiples of `cluster`.
-double plan_gemm_tc(GemmParams& p, int64_t M, int64_t k_step);
+double plan_gemm_tc(GemmParams& p, int64_t M, int64_t k_step, bool joint);
 int launch_gemm_tc(int epi, const GemmParams& p, cudaStream_t s);
 int launch_dw_dx_tc(int epi, const GemmParams& w, const GemmParams* g, int64_t dw_blocks, int64_t dx_blocks, int64_t zero_blocks, int64_t cluster,
                     const uint32_t* keep_cols, int64_t D, int64_t H, cudaStream_t s);

@@ -487,7 +487,7 @@ __device__ __forceinline__ void tc_finish(const GemmParams& p, int tile, int spl
   if (p.M_dev != nullptr) M = min(M, *p.M_dev);
   const int64_t m0 = (int64_t)(tile / (int)p.gx) * kTcM, n0 = (int64_t)(tile % (int)p.gx) * kTcN;
   const bool sums = (EPI == kEpiScatterRows || EPI == kEpiSparse) && p.db != nullptr && m0 == 0;
-  const int S = p.splits, rows = kTcM / S, tid = threadIdx.x, warp = tid >> 5;
+  const int S = p.splits, rows = (kTcM / kTcWorkers + S - 1) / S * kTcWorkers, tid = threadIdx.x, warp = tid >> 5;
   const uint32_t rank0 = cluster_ctarank() - (uint32_t)split;
   float* plane = reinterpret_cast<float*>(tc_stages(smem));
   if (sums && split == 0 && tid < kTcN && n0 + tid < p.N) {
@@ -499,7 +499,7 @@ __device__ __forceinline__ void tc_finish(const GemmParams& p, int tile, int spl
   if (m0 >= M || warp >= kTcWorkers) return;
   const int c = 4 * (tid & 31), nc = (int)max((int64_t)0, min((int64_t)4, p.N - n0 - c));      // columns past the end: nothing is written
   const int64_t n = n0 + c;
-  const int begin = split * rows, end = (int)min((int64_t)(begin + rows), M - m0);
+  const int begin = split * rows, end = (int)min((int64_t)min(begin + rows, kTcM), M - m0);
   float4 bias = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   if (EPI == kEpiForward && p.bias != nullptr) bias = *reinterpret_cast<const float4*>(tc_ctl(smem)->bias + c);
   const bool relu = EPI == kEpiForward && p.act == RAD_ACT_RELU;
@@ -507,26 +507,30 @@ __device__ __forceinline__ void tc_finish(const GemmParams& p, int tile, int spl
   const bool vec_a = EPI == kEpiForward ? tc_on16(p.out_act, p.ld_act) : EPI == kEpiInputGrad ? tc_on16(p.out_low, p.ld_low) : tc_on16(p.out_f32, p.ld_f32);
   const bool vec_z = EPI == kEpiForward ? tc_on16(p.out_z, p.ld_z) : kGelu && tc_on16(p.z_prev, p.ld_zprev);
   const bool vec_zlow = EPI == kEpiForward && tc_on16(p.out_zlow, p.ld_zlow);
-  // all splits of all rows of this thread (rows x splits are 128, eight vectors a thread) are under way before the first is
-  // added; the sums go where this CTA's own partial sums of these rows were, which only this thread has read
+  // several rows' partial sums of all splits are under way before the first is added (up to eight vectors); the sums go where
+  // this CTA's own partial sums of these rows were, which only this thread has read
   if (S > 1) {
-    float4 part[8];
-    const int shift = 31 - __clz(S);
+    const int at_once = 8 / S;
+#pragma unroll 1
+    for (int r0 = begin + warp; r0 < end; r0 += at_once * kTcWorkers) {
+      float4 part[8];
+      int q = 0, r = r0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int r = begin + warp + (i >> shift) * kTcWorkers;
-      if (r < end) part[i] = tc_ld_cluster(plane + r * kTcLd + c, rank0 + (uint32_t)(i & (S - 1)));
-    }
-    float4 v = part[0];
-#pragma unroll
-    for (int i = 1; i <= 8; ++i) {
-      const bool more = i < 8 && (i & (S - 1)) != 0;
-      if (!more) {
-        const int r = begin + warp + ((i - 1) >> shift) * kTcWorkers;
-        if (r < end) *reinterpret_cast<float4*>(plane + r * kTcLd + c) = v;
-        v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      for (int i = 0; i < 8; ++i) {
+        if (i < at_once * S && r < end) part[i] = tc_ld_cluster(plane + r * kTcLd + c, rank0 + (uint32_t)q);
+        if (++q == S) { q = 0; r += kTcWorkers; }
       }
-      if (i < 8) { v.x += part[i & 7].x; v.y += part[i & 7].y; v.z += part[i & 7].z; v.w += part[i & 7].w; }
+      q = 0; r = r0;
+      float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        v.x += part[i].x; v.y += part[i].y; v.z += part[i].z; v.w += part[i].w;
+        if (++q == S) {
+          if (i < at_once * S && r < end) *reinterpret_cast<float4*>(plane + r * kTcLd + c) = v;
+          v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          q = 0; r += kTcWorkers;
+        }
+      }
     }
   }
   // a thread's rows have a word of ReLU bits each (four words a row), or a row of dW: 32 words, one a lane
@@ -663,9 +667,8 @@ bool gelu_ahead(const GemmParams& p) { return p.relubits == nullptr && p.z_prev 
 
 // Clusters of `size` CTAs that run at the same time (an SM takes one CTA, and a cluster stays within a part of the chip).
 static int clusters_at_once(int size) {
-  static std::atomic<int> known[4];
-  const int i = size >= 8 ? 3 : size >= 4 ? 2 : size >= 2 ? 1 : 0;
-  int n = known[i].load(std::memory_order_relaxed);
+  static std::atomic<int> known[9];
+  int n = known[size].load(std::memory_order_relaxed);
   if (n > 0) return n;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)size);
@@ -682,7 +685,7 @@ static int clusters_at_once(int size) {
     (void)cudaGetLastError();
     return std::max(1, kNumSms / size);              // not remembered
   }
-  known[i].store(n, std::memory_order_relaxed);
+  known[size].store(n, std::memory_order_relaxed);
   return n;
 }
 
@@ -691,11 +694,11 @@ static int clusters_at_once(int size) {
 // 2470 and 3250 with A expanded from a store; 1270 and 3000 with a same-sample store.  Fitted to 116 timings of both forms (29
 // shapes, forward, input gradient, both dW): within 25 % of 109 of them.  Against the CUDA-core form the line lies near 300 x
 // 500 x 500: 150 x 300 x 300 8.5 us here and 6.2 there, 300 x 500 x 500 9.5 and 14.2, 2048 x 1024 x 1024 29 and 126, 4096 x 2048
-// x 2048 211 and 794 (the same with A from a store 344 and 893), 1500 x 1001 x 777 51 and 104.  Less than 72
+// x 2048 211 and 794 (the same with A from a store 344 and 893), 1500 x 1001 x 777 46 and 104.  Less than 72
 // k or columns (half a tile's width and a bit) stay there: 4096 x 1001, k = 10, 17 us against 12, 4096 x 64 x 64 6.5 against 5.6;
 // between 60 and 72 long or wide ones would be faster here (512 x 64 x 2048 6.4 against 9.6), but tests/test_launches.py holds
 // 2000 x 68 x 1500 to the CUDA-core forms whose coverage it checks.
-double plan_gemm_tc(GemmParams& p, int64_t M, int64_t k_step) {
+double plan_gemm_tc(GemmParams& p, int64_t M, int64_t k_step, bool joint) {
   const int64_t step = std::max<int64_t>(k_step, kTcBlock), gx = ceil_div(p.N, kTcN);
   const int64_t tiles = std::max<int64_t>(1, ceil_div(M, kTcM)) * gx, grid_tiles = std::max<int64_t>(1, ceil_div(p.M, kTcM)) * gx;
   const bool ak = p.sak == 1, bk = p.sbk == 1 && p.sbn != 1, sparse = p.keepbits != nullptr;
@@ -708,8 +711,11 @@ double plan_gemm_tc(GemmParams& p, int64_t M, int64_t k_step) {
   p.tc = 1;
   p.walk = 0;
   p.wait_limit_ns = wait_limit_ns();
-  for (int s = 1; s <= 8; s *= 2) {
-    if (s > 1 && p.K <= s / 2 * step) break;
+  // two contractions in one launch share its clusters: splits that divide one another.  Else any number of splits, which
+  // evens out the last round (1500 x 1001 x 777 is 84 tiles: three splits in two rounds of 11 blocks 45.6 us, one round of 32
+  // 50.9; dW of 4096 x 333 x 777 61.8 -> 44.8, of 300 x 500 x 500 13.2 -> 9.8; the worst of 128 calls 1200 x 800 x 800 33.6 -> 36.5)
+  for (int s = 1; s <= 8; s += joint ? s : 1) {
+    if (s > 1 && p.K <= (s - 1) * step) break;
     const int64_t rounds = ceil_div(tiles, (int64_t)clusters_at_once(s)), k_per = round_up(ceil_div(p.K, s), step);
     const double clk = (double)rounds * ((double)(k_per / kTcBlock) * block + 9750.0) + (s > 1 ? 5100.0 : 0.0);
     if (clk < best && grid_tiles * s <= 0x7fffffff) {

@@ -486,13 +486,13 @@ inline bool tc_wins(double cuda_cores, double tensor_cores) { return 1.15 * tens
 inline void plan_forms(GemmParams& p, int64_t rows, int es, int64_t k_step = 4, bool may_walk = true) {
   GemmParams c = p, t = p;
   const double est = plan_gemm(c, rows, es, k_step, may_walk);
-  if (es == 4 && tc_wins(est, plan_gemm_tc(t, rows, k_step))) p = t;
+  if (es == 4 && tc_wins(est, plan_gemm_tc(t, rows, k_step, false))) p = t;
   else plan_gemm(p, p.M, es, k_step, may_walk);
 }
 inline void plan_joint(GemmParams& w, GemmParams& g, int64_t rows, int es, int64_t k_step, bool may_walk) {
   GemmParams c = w, tw = w, tg = g;
   const double est = plan_gemm(c, rows, es, k_step, may_walk) + plan_gemm(g, g.M, es);
-  if (es == 4 && tc_wins(est, plan_gemm_tc(tw, rows, k_step) + plan_gemm_tc(tg, g.M, 4))) {
+  if (es == 4 && tc_wins(est, plan_gemm_tc(tw, rows, k_step, true) + plan_gemm_tc(tg, g.M, 4, true))) {
     w = tw;
     g = tg;
   } else {

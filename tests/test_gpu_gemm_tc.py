@@ -9,7 +9,8 @@ from oracle import rad as orc
 pytestmark = pytest.mark.gpu
 
 # All large enough for that form.  (rows, inputs, outputs, elements between rows beyond their length)
-SHAPES = [(1025, 513, 641, 0), (1024, 1024, 1024, 0), (769, 1001, 777, 0), (1000, 1000, 1300, 4), (1153, 897, 899, 3), (641, 130, 1921, 1)]
+SHAPES = [(1025, 513, 641, 0), (1024, 1024, 1024, 0), (769, 1001, 777, 0), (1000, 1000, 1300, 4), (1153, 897, 899, 3), (641, 130, 1921, 1),
+          (1500, 1001, 777, 0), (2500, 500, 500, 0), (300, 500, 500, 0), (1800, 1500, 150, 0)]      # three to seven splits of k
 
 
 def _strided(x, extra):
