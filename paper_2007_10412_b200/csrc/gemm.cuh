@@ -46,11 +46,28 @@ int launch_gemm_tc(int epi, const GemmParams& p, cudaStream_t s);
 int launch_dw_dx_tc(int epi, const GemmParams& w, const GemmParams* g, int64_t dw_blocks, int64_t dx_blocks, int64_t zero_blocks, int64_t cluster,
                     const uint32_t* keep_cols, int64_t D, int64_t H, cudaStream_t s);
 
+// What an output needs besides its sum: its bias, its word of ReLU bits or its row of dW, its pre-activation.
+struct GemmSide { float bias, z; uint32_t word; };
+template <typename T, int EPI>
+__device__ __forceinline__ void gemm_prefetch(const GemmParams& p, int64_t m, int64_t n, uint32_t& word, float& z) {
+  word = 0;
+  z = 0.0f;
+  if (EPI == kEpiScatterRows) word = p.row_idx[m];
+  if (EPI == kEpiInputGrad && p.relubits != nullptr) word = p.relubits[m * p.w32 + (n >> 5)];
+  else if (EPI == kEpiInputGrad && p.z_prev != nullptr) z = to_float(static_cast<const T*>(p.z_prev)[m * p.ld_zprev + n]);
+}
+template <typename T, int EPI>
+__device__ __forceinline__ GemmSide gemm_side(const GemmParams& p, int64_t m, int64_t n) {
+  GemmSide s;
+  s.bias = EPI == kEpiForward && p.bias != nullptr ? p.bias[n] : 0.0f;
+  gemm_prefetch<T, EPI>(p, m, n, s.word, s.z);
+  return s;
+}
 // Epilogue of one output.
 template <typename T, int EPI>
-__device__ __forceinline__ void gemm_store(const GemmParams& p, int64_t m, int64_t n, float v) {
+__device__ __forceinline__ void gemm_store(const GemmParams& p, int64_t m, int64_t n, float v, const GemmSide& side) {
   if (EPI == kEpiForward) {
-    if (p.bias != nullptr) v += p.bias[n];
+    v += side.bias;
     if (p.out_z != nullptr) p.out_z[m * p.ld_z + n] = v;
     if (p.out_zlow != nullptr) static_cast<T*>(p.out_zlow)[m * p.ld_zlow + n] = from_float<T>(v);
     if (p.out_act != nullptr) {
@@ -59,13 +76,13 @@ __device__ __forceinline__ void gemm_store(const GemmParams& p, int64_t m, int64
     }
   } else if (EPI == kEpiInputGrad) {
     if (p.relubits != nullptr) {
-      if (((p.relubits[m * p.w32 + (n >> 5)] >> (n & 31)) & 1u) == 0) v = 0.0f;
+      if (((side.word >> (n & 31)) & 1u) == 0) v = 0.0f;
     } else if (p.z_prev != nullptr) {
-      v *= gelu_grad_f(to_float(static_cast<const T*>(p.z_prev)[m * p.ld_zprev + n]));
+      v *= gelu_grad_f(side.z);
     }
     static_cast<T*>(p.out_low)[m * p.ld_low + n] = from_float<T>(v);
   } else {
-    p.out_f32[(EPI == kEpiScatterRows ? (int64_t)p.row_idx[m] : m) * p.ld_f32 + n] = v;
+    p.out_f32[(EPI == kEpiScatterRows ? (int64_t)side.word : m) * p.ld_f32 + n] = v;
   }
 }
 

@@ -593,7 +593,7 @@ __device__ __forceinline__ void tc_finish(const GemmParams& p, int tile, int spl
     const int r = begin + warp + (__ffs(bad) - 1) * kTcWorkers;
 #pragma unroll 1
     for (int e = 0; e < nc; ++e) {
-      if (!(fabsf(plane[r * kTcLd + c + e]) <= FLT_MAX)) gemm_store<float, EPI>(p, m0 + r, n + e, tc_plain<EPI>(p, m0 + r, n + e));
+      if (!(fabsf(plane[r * kTcLd + c + e]) <= FLT_MAX)) gemm_store<float, EPI>(p, m0 + r, n + e, tc_plain<EPI>(p, m0 + r, n + e), gemm_side<float, EPI>(p, m0 + r, n + e));
     }
   }
 }
