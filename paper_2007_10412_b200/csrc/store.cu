@@ -383,14 +383,67 @@ __global__ void __launch_bounds__(1024) same_mask_kernel(const SameParams p, con
   }
 }
 
-// values[b, j] = A[b, idx[j]] * scale for j < k', zero up to ld.  One warp per row at a time.
-template <typename T>
-__global__ void __launch_bounds__(256) same_gather_kernel(const SameParams p, const float* colscale) {
+// The same by every CTA of a gather for itself (256 threads, a keep-bit word each: D <= kDrawColumns): the column list goes to
+// shared memory, the first CTA writes keep bits, list and counts as well.  Three generator outputs a thread and one scan, before
+// the kernel ahead has ended: a launch less per store (MNIST-shaped step of fifteen launches 68.8 -> 62 us).
+constexpr int64_t kDrawColumns = 256 * 32;
+struct SameDraw { uint32_t word, place; int64_t kept; };               // the thread's keep bits, their first place; columns kept
+__device__ __forceinline__ SameDraw draw_columns(const SameParams& p, const PhiloxKeys& ks, uint16_t* s_idx) {
+  __shared__ uint32_t s_warp[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  SameDraw d;
+  d.word = 0;
+  if (tid * 32 < p.D) d.word = philox_keep32((uint32_t)tid, 0u, p.c2, p.c3, ks, p.T) & (0xffffffffu >> (32 - min(32, (int)p.D - 32 * tid)));
+  const uint32_t c = __popc(d.word);
+  uint32_t incl = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t n = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += n;
+  }
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  uint32_t before = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    const uint32_t n = s_warp[w];
+    before += w < warp ? n : 0u;
+    all += n;
+  }
+  d.place = before + incl - c;
+  d.kept = all;
+  uint32_t at = d.place;
+  for (uint32_t m = d.word; m != 0; m &= m - 1, ++at)
+    if (at < p.ld) s_idx[at] = (uint16_t)(32 * tid + __ffs(m) - 1);
+  __syncthreads();
+  return d;
+}
+__device__ __forceinline__ void write_columns(const SameParams& p, const SameDraw& d) {       // the first CTA, behind the wait
+  const int tid = threadIdx.x;
+  if (tid * 32 < p.D) p.keepbits[tid] = d.word;
+  uint32_t at = d.place;
+  for (uint32_t m = d.word; m != 0; m &= m - 1, ++at) p.idx[at] = (uint32_t)(32 * tid + __ffs(m) - 1);
+  if (tid == 0) {
+    p.nnz[0] = d.kept;
+    p.nnz[1] = d.kept * p.B;
+    if (d.kept > p.ld) raise_status(p.dev_status, RAD_DEV_ECAPACITY);
+  }
+}
+
+// values[b, j] = A[b, idx[j]] * scale for j < k', zero up to ld.  One warp per row at a time, `ctas` CTAs of which this is number
+// `cta`.  kDraw: the columns are drawn here.
+template <typename T, bool kDraw>
+__device__ __forceinline__ void same_gather(const SameParams& p, const PhiloxKeys& ks, const float* colscale, int cta, int ctas) {
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  uint16_t* s_idx = reinterpret_cast<uint16_t*>(s_dyn);
+  SameDraw draw = {};
+  if (kDraw) draw = draw_columns(p, ks, s_idx);
   wait_for_previous();
-  const int64_t k = min(p.nnz[0], p.ld);
+  if (kDraw && cta == 0) write_columns(p, draw);
+  const int64_t k = min(kDraw ? draw.kept : p.nnz[0], p.ld);
   const int lane = threadIdx.x & 31;
-  const int64_t warp0 = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int64_t nwarps = (int64_t)gridDim.x * 8;
+  const int64_t warp0 = (int64_t)cta * 8 + (threadIdx.x >> 5);
+  const int64_t nwarps = (int64_t)ctas * 8;
   const T* A = static_cast<const T*>(p.A);
   T* out = static_cast<T*>(p.values);
   for (int64_t b = warp0; b < p.B; b += nwarps) {
@@ -400,7 +453,7 @@ __global__ void __launch_bounds__(256) same_gather_kernel(const SameParams p, co
     for (int64_t j = lane; j < p.ld; j += 32) {
       float v = 0.0f;
       if (j < k) {
-        const uint32_t col = p.idx[j];
+        const uint32_t col = kDraw ? s_idx[j] : p.idx[j];
         if (col < (uint32_t)p.D) v = __fmul_rn(to_float(rowp[col]), colscale != nullptr ? colscale[j] : p.scale);
         else raise_status(p.dev_status, RAD_DEV_EINTERNAL);
       }
@@ -408,22 +461,29 @@ __global__ void __launch_bounds__(256) same_gather_kernel(const SameParams p, co
     }
   }
 }
+template <typename T, bool kDraw>
+__global__ void __launch_bounds__(256) same_gather_kernel(const SameParams p, const PhiloxKeys ks, const float* colscale) {
+  same_gather<T, kDraw>(p, ks, colscale, (int)blockIdx.x, (int)gridDim.x);
+}
 
 // The same gather with every access 16 bytes wide, for masks dense enough that most of a row is needed
 // anyway (or when the 1-bit ReLU derivatives of the row are wanted, which need all of it): a warp brings a
 // whole row of A into its own shared-memory buffer with asynchronous 16-byte copies, takes the ReLU bits
 // from there, and writes the gathered row eight (bf16) or four (f32) outputs per lane and store.  The kept
 // columns sit in shared memory as 16-bit numbers (D <= 65536).
-template <typename T>
-__global__ void __launch_bounds__(256) same_gather_rows_kernel(const SameParams p, uint32_t* relubits, int64_t w32, int warps) {
-  wait_for_previous();
+template <typename T, bool kDraw>
+__global__ void __launch_bounds__(256) same_gather_rows_kernel(const SameParams p, const PhiloxKeys ks, uint32_t* relubits, int64_t w32, int warps) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   constexpr int kPer = 16 / (int)sizeof(T);
-  const int64_t k = min(p.nnz[0], p.ld);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint16_t* s_idx = reinterpret_cast<uint16_t*>(s_dyn);
+  SameDraw draw = {};
+  if (kDraw) draw = draw_columns(p, ks, s_idx);
+  wait_for_previous();
+  if (kDraw && blockIdx.x == 0) write_columns(p, draw);
+  const int64_t k = min(kDraw ? draw.kept : p.nnz[0], p.ld);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t idx_bytes = (p.ld * 2 + 15) / 16 * 16;
-  for (int64_t j = tid; j < p.ld; j += blockDim.x) {
+  for (int64_t j = tid; !kDraw && j < p.ld; j += blockDim.x) {
     uint32_t col = 0;
     if (j < k) {
       col = p.idx[j];
@@ -470,13 +530,11 @@ __global__ void __launch_bounds__(256) same_gather_rows_kernel(const SameParams 
 // loads of a word are one line and all eight are in flight together.  (With a thread per word its 32 loads followed one
 // another through 32 lines per warp: 5.0 us for 150 x 300 float32.)
 template <typename T>
-__global__ void __launch_bounds__(256) relu_bits_kernel(const T* A, int64_t lda, int64_t B, int64_t D,
-                                                        int64_t w32, uint32_t* out) {
-  begin_after_previous();
+__device__ __forceinline__ void relu_bits_by_lane(const T* A, int64_t lda, int64_t B, int64_t D, int64_t w32, uint32_t* out, int cta, int ctas) {
   constexpr int kWords = 8;
   const int64_t n = B * w32;
   const int lane = threadIdx.x & 31;
-  const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const int64_t warp = (int64_t)cta * (blockDim.x >> 5) + (threadIdx.x >> 5), warps = (int64_t)ctas * (blockDim.x >> 5);
   for (int64_t i0 = warp * kWords; i0 < n; i0 += warps * kWords) {
     const int64_t b = n <= 0xffffffffll ? (int64_t)((uint32_t)i0 / (uint32_t)w32) : i0 / w32;
     int64_t c = (i0 - b * w32) * 32 + lane;         // column of the row at `row`
@@ -496,6 +554,22 @@ __global__ void __launch_bounds__(256) relu_bits_kernel(const T* A, int64_t lda,
       if (lane == j) mine = m;
     }
     if (lane < kWords && i0 + lane < n) out[i0 + lane] = mine;
+  }
+}
+template <typename T>
+__global__ void __launch_bounds__(256) relu_bits_kernel(const T* A, int64_t lda, int64_t B, int64_t D, int64_t w32, uint32_t* out) {
+  begin_after_previous();
+  relu_bits_by_lane(A, lda, B, D, w32, out, (int)blockIdx.x, (int)gridDim.x);
+}
+// A same-sample store of few columns and the ReLU bits of its rows in one launch: neither reads what the other writes.
+template <typename T>
+__global__ void __launch_bounds__(256) same_gather_relu_bits_kernel(const SameParams p, const PhiloxKeys ks, int gathers, int64_t w32, uint32_t* relubits) {
+  const int cta = (int)blockIdx.x;
+  if (cta < gathers) {
+    same_gather<T, true>(p, ks, nullptr, cta, gathers);
+  } else {
+    begin_after_previous();
+    relu_bits_by_lane(static_cast<const T*>(p.A), p.lda, p.B, p.D, w32, relubits, cta - gathers, (int)gridDim.x - gathers);
   }
 }
 // The same, one thread per word (see launch_relu_bits).
@@ -761,10 +835,14 @@ int launch_wait_probe_lookback(uint64_t limit_ns, int32_t* dev_status, cudaStrea
 // word idle and issues as many loads for it as for a full one.  Us of the store around it, thread / lane: bf16 65536 x 72
 // 18.2 / 22.4, 65536 x 300 37.4 / 42.7, but 65536 x 500 62.8 / 62.5, 20000 x 784 34.0 / 32.0, 4096 x 136 8.2 / 7.4; float32, whose
 // lines a thread walks half as far, 65536 x 72 21.3 / 23.0, 65536 x 8 13.8 / 16.5, but 65536 x 200 39.9 / 35.5, 16384 x 72 10.0 / 9.8.
+static bool relu_bits_by_thread(int dtype, int64_t w32, int64_t n) { return dtype == RAD_BF16 ? w32 <= 12 && n >= 40000 : w32 <= 4 && n >= 65536; }
+static unsigned relu_bits_grid(bool by_thread, int64_t n) {
+  return (unsigned)(by_thread ? std::min<int64_t>(ceil_div(n, 256), 148 * 16) : std::min<int64_t>(ceil_div(n, 64), 148 * 32));
+}
 int launch_relu_bits(int dtype, const void* A, int64_t lda, int64_t B, int64_t D, uint32_t* relubits, cudaStream_t s) {
   const int64_t w32 = ceil_div(D, 32), n = B * w32;
-  const bool by_thread = dtype == RAD_BF16 ? w32 <= 12 && n >= 40000 : w32 <= 4 && n >= 65536;
-  const unsigned grid = (unsigned)(by_thread ? std::min<int64_t>(ceil_div(n, 256), 148 * 16) : std::min<int64_t>(ceil_div(n, 64), 148 * 32));
+  const bool by_thread = relu_bits_by_thread(dtype, w32, n);
+  const unsigned grid = relu_bits_grid(by_thread, n);
   count_launch();
   if (dtype == RAD_BF16)
     return launch_kernel(by_thread ? relu_bits_thread_kernel<bf16> : relu_bits_kernel<bf16>, grid, 256, 0, s, static_cast<const bf16*>(A), lda, B, D, w32, relubits);
@@ -1037,7 +1115,8 @@ extern "C" int rad_linear_forward_store(const void* A, int64_t lda, const rad_st
   p.values = st->values; p.ld = st->values_ld; p.keepbits = st->keepbits; p.idx = st->offsets;
   p.nnz = st->nnz; p.dev_status = dev_status;
   const float* colscale = nullptr;
-  count_launch(2);
+  const bool draw = !replace && st->D <= kDrawColumns;                    // the columns are drawn by the gather's CTAs
+  count_launch(draw ? 1 : 2);
   if (replace) {
     SameReplaceParams r;
     r.D = st->D; r.k = k;
@@ -1048,7 +1127,7 @@ extern "C" int rad_linear_forward_store(const void* A, int64_t lda, const rad_st
     r.colscale = reinterpret_cast<float*>(static_cast<char*>(workspace) + 256 + 4 * st->D);
     colscale = r.colscale;
     RAD_TRY(launch_kernel(same_replace_mask_kernel, 1, 1024, 0, s, p, r, ks));
-  } else {
+  } else if (!draw) {
     RAD_TRY(launch_kernel(same_mask_kernel, 1, 1024, 0, s, p, ks));
   }
   // Dense masks (most 32-byte sectors of a row hold a kept column) and calls that also want the ReLU bits take
@@ -1069,21 +1148,25 @@ extern "C" int rad_linear_forward_store(const void* A, int64_t lda, const rad_st
           sms = 148;
       }
       const int grid_r = (int)std::min<int64_t>(ceil_div(st->B, warps), sms);
-      if (st->dtype == RAD_BF16) {
-        RAD_CUDA_TRY(cudaFuncSetAttribute(same_gather_rows_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_budget));
-        RAD_TRY(launch_kernel(same_gather_rows_kernel<bf16>, grid_r, 256, smem, s, p, st->relubits, w32, warps));
-      } else {
-        RAD_CUDA_TRY(cudaFuncSetAttribute(same_gather_rows_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_budget));
-        RAD_TRY(launch_kernel(same_gather_rows_kernel<float>, grid_r, 256, smem, s, p, st->relubits, w32, warps));
-      }
-      return RAD_OK;
+      const auto rows = [&](auto kernel) {
+        RAD_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_budget));
+        return launch_kernel(kernel, grid_r, 256, smem, s, p, ks, st->relubits, w32, warps);
+      };
+      if (st->dtype == RAD_BF16) return draw ? rows(same_gather_rows_kernel<bf16, true>) : rows(same_gather_rows_kernel<bf16, false>);
+      return draw ? rows(same_gather_rows_kernel<float, true>) : rows(same_gather_rows_kernel<float, false>);
     }
   }
   const int grid = (int)std::min<int64_t>(ceil_div(st->B, 8), 148 * 8);
-  if (st->dtype == RAD_BF16)
-    RAD_TRY(launch_kernel(same_gather_kernel<bf16>, grid, 256, 0, s, p, colscale));
-  else
-    RAD_TRY(launch_kernel(same_gather_kernel<float>, grid, 256, 0, s, p, colscale));
+  const size_t list = draw ? (size_t)round_up(std::min(st->values_ld, kDrawColumns) * 2, 16) : 0;
+  if (draw && st->relubits != nullptr && !relu_bits_by_thread(st->dtype, w32, st->B * w32)) {
+    const auto both = [&](auto kernel) {
+      return launch_kernel(kernel, (unsigned)grid + relu_bits_grid(false, st->B * w32), 256, list, s, p, ks, grid, w32, st->relubits);
+    };
+    return st->dtype == RAD_BF16 ? both(same_gather_relu_bits_kernel<bf16>) : both(same_gather_relu_bits_kernel<float>);
+  }
+  const auto gather = [&](auto kernel) { return launch_kernel(kernel, grid, 256, list, s, p, ks, colscale); };
+  if (st->dtype == RAD_BF16) RAD_TRY(draw ? gather(same_gather_kernel<bf16, true>) : gather(same_gather_kernel<bf16, false>));
+  else RAD_TRY(draw ? gather(same_gather_kernel<float, true>) : gather(same_gather_kernel<float, false>));
   if (st->relubits != nullptr) return launch_relu_bits(st->dtype, A, lda, st->B, st->D, st->relubits, s);
   return RAD_OK;
 }
