@@ -43,13 +43,12 @@ struct IndexParams {
 
 // One tile by one warp, no CTA-wide step: lane l draws words l, l + 32, ... of the tile (word t = row t / 4, columns
 // 32 (t % 4) ..), so a warp's stores are contiguous and a warp scan per turn, carried over the eight turns, gives every
-// row its offset in (row, column) order.  Returns the tile's kept count.
+// row its offset in (row, column) order.  `tw`: the tile's words, in `keepbits` or in shared memory.  Returns the tile's kept count.
 __device__ __forceinline__ uint32_t index_tile(const IndexLayer& L, uint32_t tile, const KeepThreshold& T, uint32_t c3, const PhiloxKeys& ks,
-                                               int lane) {
+                                               int lane, uint32_t* tw) {
   const uint32_t slab = tile / L.ncb, cb = tile - slab * L.ncb;
   const int w = lane & 3;
   const uint32_t col0 = cb * kTileCols + 32u * w;
-  uint32_t* tw = L.keepbits + (int64_t)tile * kTileWords;
   uint32_t base = 0;
 #pragma unroll 2
   for (int i = 0; i < kBitWords / 32; ++i) {
@@ -74,6 +73,17 @@ __device__ __forceinline__ uint32_t index_tile(const IndexLayer& L, uint32_t til
   }
   return base;
 }
+__device__ __forceinline__ uint32_t* tile_words(const IndexLayer& L, uint32_t tile) { return L.keepbits + (int64_t)tile * kTileWords; }
+// A tile that was drawn into shared memory to its place, by its warp.
+__device__ __forceinline__ void place_tile(const IndexLayer& L, uint32_t tile, const uint32_t* words, int lane) {
+  uint32_t* tw = tile_words(L, tile);
+  __syncwarp();
+  if (((uintptr_t)tw & 15) == 0) {
+    for (int i = lane; i < kTileWords / 4; i += 32) reinterpret_cast<uint4*>(tw)[i] = reinterpret_cast<const uint4*>(words)[i];
+  } else {
+    for (int i = lane; i < kTileWords; i += 32) tw[i] = words[i];
+  }
+}
 __device__ __forceinline__ uint32_t padded_count(uint32_t c) { return (c + kValueAlign - 1) / kValueAlign * kValueAlign; }
 __device__ __forceinline__ void write_totals(const IndexLayer& L, uint32_t padded, uint32_t exact, int32_t* dev_status) {
   L.offsets[L.ntiles] = padded;
@@ -84,10 +94,29 @@ __device__ __forceinline__ void write_totals(const IndexLayer& L, uint32_t padde
 
 constexpr int kIndexWarps = 16;
 // (One layer has a form of its own: fewer registers, 65536 tiles 160 us instead of 163.)
+// ahead: a tile per warp at most, drawn into the shared memory that spreads the CTAs before the kernel ahead has ended: the key is
+// all it takes.
 template <int kLayers>
-__global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const __grid_constant__ IndexParams<kLayers> p, const PhiloxKeys ks) {
-  wait_for_previous();
+__global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const __grid_constant__ IndexParams<kLayers> p, const PhiloxKeys ks, int ahead) {
   const int lane = threadIdx.x & 31;
+  if (ahead) {
+    extern __shared__ __align__(16) uint32_t s_tiles[];
+    const uint32_t t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    uint32_t* words = s_tiles + (threadIdx.x >> 5) * kTileWords;
+    int l = 0;
+    if (kLayers > 1)
+      while (l + 1 < p.nlayers && t >= p.layer[l + 1].tile0) ++l;
+    const IndexLayer layer = p.layer[l];
+    uint32_t count = 0;
+    if (t < p.ntiles) count = index_tile(layer, t - layer.tile0, p.T, p.c3, ks, lane, words);
+    begin_after_previous();
+    if (t < p.ntiles) {
+      place_tile(layer, t - layer.tile0, words, lane);
+      if (lane == 0) layer.offsets[t - layer.tile0] = count;
+    }
+    return;
+  }
+  wait_for_previous();
   const uint32_t warps = blockDim.x >> 5, warp0 = blockIdx.x * warps + (threadIdx.x >> 5), nwarps = gridDim.x * warps;
   int l = 0;
   IndexLayer layer = p.layer[0];                    // in registers: out of the parameters by a variable index, every use would be a load
@@ -96,7 +125,7 @@ __global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const __g
     if (kLayers > 1)
       while (l + 1 < p.nlayers && t >= p.layer[l + 1].tile0) layer = p.layer[++l];
     const uint32_t tile = t - layer.tile0;
-    const uint32_t count = index_tile(layer, tile, p.T, p.c3, ks, lane);
+    const uint32_t count = index_tile(layer, tile, p.T, p.c3, ks, lane, tile_words(layer, tile));
     if (lane == 0) layer.offsets[tile] = count;
   }
 }
@@ -106,18 +135,21 @@ __global__ void __launch_bounds__(32 * kIndexWarps) store_index_kernel(const __g
 // 640-520-392-200 net at batch 328 took 20 us of its step, in one launch for all of them 6.  An SM draws a tile in 0.26 us (three generator calls per word, 3 G calls/s), so with
 // more than twelve tiles a CTA the two launches of the general form, on all SMs, are faster.
 constexpr int kSmallIndexCtas = 8, kSmallIndexTiles = 12 * kSmallIndexCtas;
+// Everything but the writes is done before the kernel ahead has ended: the key is all it takes.
 __global__ void __launch_bounds__(32 * kIndexWarps) store_index_small_kernel(const __grid_constant__ IndexParams<kIndexLayers> p, const PhiloxKeys ks) {
   cluster_started_arrive();                             // waited for behind the draw
-  begin_after_previous();
-  __shared__ uint32_t s_count[kSmallIndexTiles / kSmallIndexCtas];
+  constexpr int kTiles = kSmallIndexTiles / kSmallIndexCtas;
+  static_assert(kTiles <= kIndexWarps, "a tile per warp");
+  __shared__ __align__(16) uint32_t s_words[kTiles][kTileWords];
+  __shared__ uint32_t s_count[kTiles];
   __shared__ uint32_t s_padded[kSmallIndexCtas], s_exact[kSmallIndexCtas];      // of every CTA of the cluster
   const IndexLayer& L = p.layer[blockIdx.x / kSmallIndexCtas];
   const uint32_t rank = cluster_ctarank(), per = (L.ntiles + kSmallIndexCtas - 1) / kSmallIndexCtas;
   const uint32_t t0 = min(rank * per, L.ntiles), n = min(per, L.ntiles - t0);
-  const int tid = threadIdx.x, lane = tid & 31;
-  for (uint32_t i = tid >> 5; i < n; i += kIndexWarps) {
-    const uint32_t count = index_tile(L, t0 + i, p.T, p.c3, ks, lane);
-    if (lane == 0) s_count[i] = count;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (warp < n) {
+    const uint32_t count = index_tile(L, t0 + warp, p.T, p.c3, ks, lane, s_words[warp]);
+    if (lane == 0) s_count[warp] = count;
   }
   __syncthreads();
   cluster_started_wait();                               // before the first write to a peer: a CTA without tiles is here at once
@@ -131,6 +163,8 @@ __global__ void __launch_bounds__(32 * kIndexWarps) store_index_small_kernel(con
     st_cluster_u32(&s_exact[rank], (uint32_t)tid, exact);
   }
   cluster_barrier();
+  begin_after_previous();
+  if (warp < n) place_tile(L, t0 + warp, s_words[warp], lane);
   if (tid == 0) {
     uint32_t at = 0, exact = 0, all = 0;
     for (uint32_t r = 0; r < kSmallIndexCtas; ++r) {
@@ -251,7 +285,9 @@ int launch_index_tiles(const IndexParams<kLayers>& p, const PhiloxKeys& ks, cuda
   const int warps = per_sm <= 4 ? 4 : per_sm <= 8 ? 8 : per_sm <= kIndexWarps ? kIndexWarps : per_sm <= 64 ? 4 : 8;
   const int64_t most = (per_sm <= kIndexWarps ? 1 : per_sm <= 64 ? 12 : 5) * kNumSms, ctas = std::min(ceil_div(p.ntiles, warps), most);
   count_launch();
-  RAD_TRY(launch_kernel(store_index_kernel<kLayers>, (unsigned)ctas, 32 * warps, spread_smem(ctas, 0), s, p, ks));
+  const size_t smem = spread_smem(ctas, 0);
+  const int ahead = ctas * warps >= p.ntiles && smem >= (size_t)warps * kTileWords * 4 ? 1 : 0;
+  RAD_TRY(launch_kernel(store_index_kernel<kLayers>, (unsigned)ctas, 32 * warps, smem, s, p, ks, ahead));
   count_launch();
   return launch_kernel(offsets_scan_kernel<kLayers>, p.nlayers, 1024, 0, s, p);
 }
