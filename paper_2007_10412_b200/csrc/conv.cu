@@ -160,16 +160,16 @@ __global__ void __launch_bounds__(256) conv_forward_pool_kernel(const ConvShape 
 // pixels of 16-byte writes.  Bound by memory: 4096 x 16 x 16 x 32 bf16 16 us, 69 with one channel per thread.
 template <typename T>
 __global__ void __launch_bounds__(256) conv_dz_kernel(const ConvShape s, const T* dP, const uint32_t* relubits, T* dZ) {
-  begin_after_previous();
   const int Hp = s.H / 2, Wp = s.W / 2, groups = s.Cout / 8;
   const int64_t total = s.B * Hp * Wp * groups;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total) return;
   const int64_t win = i / groups;
   const int co = (int)(i - win * groups) * 8;
   const int64_t line = win / Wp;
   const int xp = (int)(win - line * Wp), yp = (int)(line % Hp);
   const int64_t b = line / Hp;
+  begin_after_previous();
+  if (i >= total) return;
   const uint32_t bits = relubits[i];
   constexpr int kV = (int)sizeof(T) / 2;             // 16-byte words of eight entries
   T g[8];

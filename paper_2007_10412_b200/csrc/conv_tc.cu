@@ -75,7 +75,6 @@ __device__ __forceinline__ uint4 cv_load_pixel(const bf16* T, bool in, int y, in
 enum { kCvFwd = 0, kCvDw = 1, kCvDx = 2 };
 template <int kMode>
 __global__ void __launch_bounds__(kCvThreads, kCvPerSm) conv_tc_kernel(const ConvTcParams p) {
-  wait_for_previous();
   constexpr bool kDw = kMode == kCvDw, kDx = kMode == kCvDx;
   extern __shared__ uint8_t cv_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(cv_raw) + 1023) & ~(uintptr_t)1023);
@@ -178,6 +177,7 @@ __global__ void __launch_bounds__(kCvThreads, kCvPerSm) conv_tc_kernel(const Con
       }
     }
   };
+  wait_for_previous();                                // behind the tensor memory and all that only needs the parameters
   if (nkb > 0) gather(0);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();

@@ -749,7 +749,9 @@ int column_sums_of(const T* dZ, int64_t ldz, int64_t B, int64_t H, float* out, f
   // column blocks there are; CTAs in whole waves of 1184 (eight per SM), at least sixteen slabs.  65536 x 601 float32 86 us
   // in one launch, 38 in two; bf16 80 and 31; 20000 x 5001 float32 93 and 75; 8192 x 601 (128 rows) 9.2 and 11.5.
   const bool tall = ny == kColMaxCluster && B > kColTallRows * RL * ny && max_slabs > kColMaxCluster;
-  const bool narrow = ny == kColMaxCluster && colblocks * ny < 148 && B > 32 * RL * ny && max_slabs > kColMaxCluster;
+  // (bf16 from twelve rows a thread on: 8192 x 64 5.5 us in one launch, 3.9 in two, 8192 x 256 5.7 and 4.2, 4096 x 256 4.0 and 3.6, 2100 x
+  // 256 3.2 and 3.5; float32 8192 x 512 4.4 and 5.1)
+  const bool narrow = ny == kColMaxCluster && colblocks * ny < 148 && B > (V == 8 ? 12 : 32) * RL * ny && max_slabs > kColMaxCluster;
   if (big || tall || narrow) {
     int64_t slabs = std::max<int64_t>(kColMaxCluster, (big ? 1184 : 592) / colblocks);
     if (tall && !big && !narrow)
