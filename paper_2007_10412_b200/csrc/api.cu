@@ -365,7 +365,7 @@ bool fill_can_fuse(int dtype, int64_t B, int64_t D, int64_t H, const void* A, in
 int forward_fill(int32_t dtype, int32_t act, int64_t B, int64_t D, int64_t H, const void* A, int64_t lda, const void* W, int64_t ldw,
                  const float* bias, void* out_act, int64_t ld_act, void* out_zlow, int64_t ld_zlow, uint32_t* relubits,
                  const rad_store* next, int32_t index_ready, StoreQueue* ahead, void* workspace, int64_t workspace_bytes,
-                 int32_t* dev_status, void* stream) {
+                 int32_t* dev_status, void* stream, bool beside) {
   if (!valid_dtype(dtype) || B <= 0 || D <= 0 || H <= 0 || A == nullptr || W == nullptr || out_act == nullptr)
     return RAD_EINVAL;
   if (act != RAD_ACT_NONE && act != RAD_ACT_RELU && act != RAD_ACT_GELU) return RAD_EINVAL;
@@ -394,7 +394,7 @@ int forward_fill(int32_t dtype, int32_t act, int64_t B, int64_t D, int64_t H, co
   }
   if (fused)
     return tc_forward(act, B, D, H, A, lda, W, ldw, bias, out_act, ld_act, nullptr, 0, out_zlow, ld_zlow, relubits,
-                      dev_status, s, next);
+                      dev_status, s, next, beside && ahead != nullptr);
   // shapes the fused epilogue does not take: the same results from the two separate calls
   // Where the forward runs on the CUDA cores its ReLU bits would be one more launch: there they come from the
   // store kernels, which look at every entry anyway (not from the projection store, which does not).
@@ -424,11 +424,11 @@ extern "C" int rad_input_grad_workspace(int64_t B, int64_t H, int64_t* bytes) {
   return RAD_OK;
 }
 
-extern "C" int rad_linear_input_grad(int32_t dtype, int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz,
-                                     const void* W, int64_t ldw, const uint32_t* relubits_prev,
-                                     const void* z_prev, int64_t ld_zprev, void* dZ_prev, int64_t ldp,
-                                     float* db, void* workspace, int64_t workspace_bytes,
-                                     int32_t* dev_status, void* stream) {
+// rad_linear_input_grad.  `beside_ahead`: the contraction may run beside the launch ahead of it (this call's or the caller's), which
+// neither writes what the contraction reads nor reads what it writes.
+static int input_grad(int32_t dtype, int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, const void* W, int64_t ldw,
+                      const uint32_t* relubits_prev, const void* z_prev, int64_t ld_zprev, void* dZ_prev, int64_t ldp, float* db,
+                      void* workspace, int64_t workspace_bytes, int32_t* dev_status, void* stream, bool beside_ahead) {
   if (!valid_dtype(dtype) || B <= 0 || D <= 0 || H <= 0 || dZ == nullptr || W == nullptr) return RAD_EINVAL;
   if (ldz < H || ldw < H) return RAD_EINVAL;
   if (dZ_prev == nullptr && db == nullptr) return RAD_EINVAL;
@@ -447,8 +447,18 @@ extern "C" int rad_linear_input_grad(int32_t dtype, int64_t B, int64_t D, int64_
   }
   if (dZ_prev == nullptr) return RAD_OK;
   if (on_tc)
-    return tc_input_grad(B, D, H, dZ, ldz, W, ldw, relubits_prev, z_prev, ld_zprev, dZ_prev, ldp, beside ? db : nullptr, dev_status, s);
+    return tc_input_grad(B, D, H, dZ, ldz, W, ldw, relubits_prev, z_prev, ld_zprev, dZ_prev, ldp, beside ? db : nullptr, dev_status, s,
+                         beside_ahead);
   return simt_input_grad(dtype, B, D, H, dZ, ldz, W, ldw, relubits_prev, z_prev, ld_zprev, dZ_prev, ldp, dev_status, s);
+}
+
+extern "C" int rad_linear_input_grad(int32_t dtype, int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz,
+                                     const void* W, int64_t ldw, const uint32_t* relubits_prev,
+                                     const void* z_prev, int64_t ld_zprev, void* dZ_prev, int64_t ldp,
+                                     float* db, void* workspace, int64_t workspace_bytes,
+                                     int32_t* dev_status, void* stream) {
+  return input_grad(dtype, B, D, H, dZ, ldz, W, ldw, relubits_prev, z_prev, ld_zprev, dZ_prev, ldp, db, workspace, workspace_bytes,
+                    dev_status, stream, false);
 }
 
 extern "C" int rad_mlp_workspace(const rad_mlp_desc* net, int64_t* bytes, rad_step_stats* stats) {
@@ -543,6 +553,7 @@ extern "C" int rad_mlp_step(const rad_mlp_desc* net, const void* X, const int32_
   if (rc != RAD_OK) return rc;
   const void* a_in = X;
   int64_t ld_in = net->dims[0];
+  bool beside = false;
   for (int l = 0; l < L; ++l) {
     TraceRange r("forward layer");
     const int64_t D = net->dims[l], H = net->dims[l + 1];
@@ -558,8 +569,10 @@ extern "C" int rad_mlp_step(const rad_mlp_desc* net, const void* X, const int32_
     void* zlow = z_of(l + 1);          // a GELU net keeps the pre-activation of layer l for the backward of layer l + 1's input
     uint32_t* rbits = plan.layer[l + 1].relubits >= 0 ? reinterpret_cast<uint32_t*>(ws + plan.layer[l + 1].relubits) : nullptr;
     rc = forward_fill(net->dtype, net->act, B, D, H, a_in, ld_in, W[l], H, b != nullptr ? b[l] : nullptr, a_out, H, zlow, H, rbits,
-                      &st[l + 1], 0, ahead[l + 1] ? &queue : nullptr, ws + plan.scratch, plan.scratch_bytes, dev_status, stream);
+                      &st[l + 1], 0, ahead[l + 1] ? &queue : nullptr, ws + plan.scratch, plan.scratch_bytes, dev_status, stream, beside);
     if (rc != RAD_OK) return rc;
+    // the network input's values are put in place beside the second layer, which reads and writes other buffers
+    beside = l == 0 && queue.n == 1 && queue.in[0].A == X;
     // still alone: the input of layer l, whose buffer the next layer writes, or the last input there is
     if (queue.n == 1 && (queue.in[0].A == a_in || l == L - 2)) rc = queue.flush();
     if (rc != RAD_OK) return rc;
@@ -589,9 +602,9 @@ extern "C" int rad_mlp_step(const rad_mlp_desc* net, const void* X, const int32_
       rc = rad_linear_weight_grad(&st[l], dz, H, H, dW[l], H, ws + plan.scratch, plan.scratch_bytes, dev_status, stream);
     if (rc != RAD_OK) return rc;
     if ((dz_prev != nullptr && !dx_done) || !db_done) {
-      rc = rad_linear_input_grad(net->dtype, B, D, H, dz, H, W[l], H, st[l].relubits, z_prev, D,
-                                 dx_done ? nullptr : dz_prev, D, db_done ? nullptr : db[l], ws + plan.scratch,
-                                 plan.scratch_bytes, dev_status, stream);
+      // the sum of dW's parts, or dW itself, or the column sums stand ahead: they share dZ with the input gradient, as readers
+      rc = input_grad(net->dtype, B, D, H, dz, H, W[l], H, st[l].relubits, z_prev, D, dx_done ? nullptr : dz_prev, D,
+                      db_done ? nullptr : db[l], ws + plan.scratch, plan.scratch_bytes, dev_status, stream, true);
       if (rc != RAD_OK) return rc;
     }
     dz = dz_prev;

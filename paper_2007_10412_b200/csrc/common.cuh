@@ -280,7 +280,7 @@ bool fill_can_fuse(int dtype, int64_t B, int64_t D, int64_t H, const void* A, in
 int forward_fill(int32_t dtype, int32_t act, int64_t B, int64_t D, int64_t H, const void* A, int64_t lda, const void* W, int64_t ldw,
                  const float* bias, void* out_act, int64_t ld_act, void* out_zlow, int64_t ld_zlow, uint32_t* relubits,
                  const rad_store* next, int32_t index_ready, StoreQueue* ahead, void* workspace, int64_t workspace_bytes,
-                 int32_t* dev_status, void* stream);
+                 int32_t* dev_status, void* stream, bool beside = false);
 int weight_grad_and_bias(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, float* dW, int64_t ldw, void* workspace,
                          int64_t workspace_bytes, int32_t* dev_status, void* stream, float* db, bool* db_written,
                          const SimtInputGrad* ig = nullptr, bool* ig_done = nullptr);
@@ -326,7 +326,7 @@ bool tc_shape_ok(int64_t B, int64_t D, int64_t H, const void* p0, int64_t ld0, c
 int tc_forward(int act, int64_t B, int64_t D, int64_t H, const void* A, int64_t lda, const void* W,
                int64_t ldw, const float* bias, void* out_act, int64_t ld_act, float* out_z,
                int64_t ld_z, void* out_zlow, int64_t ld_zlow, uint32_t* relubits,
-               int32_t* dev_status, cudaStream_t s, const rad_store* next = nullptr);
+               int32_t* dev_status, cudaStream_t s, const rad_store* next = nullptr, bool beside = false);
 // store_index.cu: keep bits, row offsets, tile offsets and nnz of a different-sample Bernoulli store from the
 // key alone (no layer input is read)
 int launch_store_index(const rad_store* st, bool check_capacity, int32_t* dev_status, cudaStream_t s);
@@ -343,7 +343,7 @@ int launch_replace_index(const rad_store* st, uint32_t* extras, bool check_capac
 int launch_replace_extras(const void* A, int64_t lda, const rad_store* st, const uint32_t* extras, cudaStream_t s);
 int tc_input_grad(int64_t B, int64_t D, int64_t H, const void* dZ, int64_t ldz, const void* W,
                   int64_t ldw, const uint32_t* relubits_prev, const void* z_prev, int64_t ld_zprev,
-                  void* dZ_prev, int64_t ldp, float* db, int32_t* dev_status, cudaStream_t s);
+                  void* dZ_prev, int64_t ldp, float* db, int32_t* dev_status, cudaStream_t s, bool beside = false);
 bool tc_sums_beside(int64_t B, int64_t D, int64_t H);      // does tc_input_grad also make db, or is that another launch?
 int tc_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H, float* dW,
                    int64_t ldw, void* workspace, int64_t workspace_bytes, int32_t* dev_status,
@@ -426,6 +426,9 @@ __device__ __forceinline__ void st_cluster_u32(uint32_t* smem, uint32_t rank, ui
 // CTA has signalled, that is with the last wave), one whose CTAs go on to further pieces as each begins its last one.
 // With the signal at the start of the pair kernels a small kernel of another stream waited 4.1 ms of a 65536 x 8192 x
 // 8192 forward for room; with this rule it runs in 20 us beside it.
+// A tensor-core kernel with `beside` set has nothing to do with the kernel ahead: neither reads or overwrites what the other
+// writes.  It begins at once (the kernel ahead let it in behind its own wait, so all before that one has ended) and waits at its
+// own end instead, so that for the kernels behind it one end still means all ends.  Never two of these in a row.
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void begin_after_previous() {

@@ -208,3 +208,52 @@ def test_indices_of_all_layers_in_one_go(dims, B, dtype):
     # the last layer's gradient: no ReLU sign that a rounding could turn stands between it and the loss
     g = ctx.dW[-1].double().cpu().numpy()
     assert np.linalg.norm(g - ref.dW[-1]) <= (1e-5 if dtype == "f32" else 2e-2) * np.linalg.norm(ref.dW[-1])
+
+
+@pytest.mark.parametrize("dims,B,variant,act", [((640, 520, 392, 200), 328, "different", "relu"), ((640, 520, 392, 200), 328, "same", "relu"),
+                                                ((72, 264, 64, 64, 72), 65, "different", "gelu"), ((1024, 1024, 520, 64), 4096, "different", "relu"),
+                                                ((512, 136, 512, 64), 2500, "redrawn", "relu"), ((256, 2048, 64, 128), 640, "same", "gelu")])
+def test_contractions_beside_the_kernel_ahead_leave_the_step_as_it_is(dims, B, variant, act):
+    """In a bf16 step an input gradient runs beside the sum of dW's parts (or dW, or the column sums), and the second layer's forward
+    beside the values of the network input, where their tiles leave room; the larger of these nets have layers on either side
+    of that line.  Several steps in a row, whose buffers are the same, and the last of them equals the layer calls bit for bit."""
+    import paper_2007_10412_b200 as rad
+    L = len(dims) - 1
+    X, y, Ws, bs = mlp_inputs(dims, B, "bf16", "normal", 7, bias_zero=False)
+    dX, dy = to_dev(X, "bf16"), torch.from_numpy(y).cuda()
+    dWs, dbs = [to_dev(W, "bf16") for W in Ws], [to_dev(b, "f32") for b in bs]
+    ctx = rad.MLPStep(dims, B, "bf16", act, variant, 0.1)
+    for t in ctx.dW:
+        t.fill_(float("nan"))
+    for step in range(12):
+        ctx(dX, dy, dWs, dbs, seed=21, step=step)
+    torch.cuda.synchronize()
+    assert ctx.dev_status.item() == 0
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    stores = [rad.Store("same" if variant == "same" else "different", "bf16", B, dims[l], 0.1, seed=21, layer=l, step=11, relu_bits=False)
+              for l in range(L)]
+    rbits = [None] + [torch.empty(B * ((dims[l] + 31) // 32), dtype=torch.int32, device="cuda") if act == "relu" else None for l in range(1, L)]
+    pre = [None] + [torch.empty(B, dims[l], dtype=torch.bfloat16, device="cuda") if act == "gelu" else None for l in range(1, L)]
+    a = dX
+    rad.rad_linear_forward_store(a, stores[0], status)
+    for l in range(L - 1):
+        out = torch.empty(B, dims[l + 1], dtype=torch.bfloat16, device="cuda")
+        rad.rad_linear_forward(a, dWs[l], dbs[l], act, out_act=out, out_zlow=pre[l + 1], relubits=rbits[l + 1], dev_status=status)
+        rad.rad_linear_forward_store(out, stores[l + 1], status)
+        a = out
+    logits = torch.empty(B, dims[L], dtype=torch.float32, device="cuda")
+    rad.rad_linear_forward(a, dWs[L - 1], dbs[L - 1], "none", out_z=logits, dev_status=status)
+    loss = torch.zeros(1, dtype=torch.float32, device="cuda")
+    dz = torch.empty(B, dims[L], dtype=torch.bfloat16, device="cuda")
+    rad.rad_softmax_xent(logits, dy, loss, dz)
+    for l in range(L - 1, -1, -1):
+        dW = torch.full((dims[l], dims[l + 1]), float("nan"), dtype=torch.float32, device="cuda")
+        db = torch.empty(dims[l + 1], dtype=torch.float32, device="cuda")
+        rad.rad_linear_weight_grad(stores[l], dz, dW, dev_status=status)
+        dzp = torch.empty(B, dims[l], dtype=torch.bfloat16, device="cuda") if l > 0 else None
+        rad.rad_linear_input_grad(dz, dWs[l], relubits_prev=rbits[l], z_prev=pre[l], dZ_prev=dzp, db=db, dev_status=status)
+        torch.cuda.synchronize()
+        assert status.item() == 0
+        assert torch.equal(dW, ctx.dW[l]) and torch.equal(db, ctx.db[l]), l
+        dz = dzp
+    assert torch.equal(loss, ctx.loss)

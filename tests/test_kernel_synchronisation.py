@@ -83,3 +83,17 @@ def test_accumulators_are_used_behind_the_wait_for_them():
         wait = re.search(r"\btmem_ld_wait\((\w*)\);", rest)
         next_to_it = re.fullmatch(r"\s*(tmem_ld\w*\([^;]*;\s*)*", rest[:wait.start()])
         assert next_to_it or wait.group(1) == m.group(2), text[m.start():m.end() + 200]
+
+
+def test_a_kernel_beside_the_one_ahead_ends_after_it():
+    """A launch that does not wait for the kernel ahead at its beginning waits at its end: whoever waits for it waits for both."""
+    found = 0
+    for file, kernel, body in _kernels():
+        skips = re.findall(r"if \(([^;]*!p\.beside[^;]*)\) wait_for_previous\(\);", body)
+        if not skips:
+            continue
+        found += 1
+        assert len(skips) == 1 and body.count("p.beside") == 2, (file, kernel)
+        assert re.search(r"p\.beside && tid == 0\) wait_for_previous\(\);\s*$", body.rstrip().rstrip("}").rstrip()), (file, kernel)
+        assert "return;" not in body, (file, kernel)                       # no thread leaves before
+    assert found == 1
