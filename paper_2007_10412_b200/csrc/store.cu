@@ -470,7 +470,9 @@ __global__ void __launch_bounds__(256) same_gather_kernel(const SameParams p, co
 // anyway (or when the 1-bit ReLU derivatives of the row are wanted, which need all of it): a warp brings a
 // whole row of A into its own shared-memory buffer with asynchronous 16-byte copies, takes the ReLU bits
 // from there, and writes the gathered row eight (bf16) or four (f32) outputs per lane and store.  The kept
-// columns sit in shared memory as 16-bit numbers (D <= 65536).
+// columns sit in shared memory as 16-bit numbers (D <= 65536).  What bounds it beside DRAM is the shared-memory pipe: a
+// lane's columns come in one access (bf16 65536 x 8192, p = 0.5 335 -> 267 us), and the lanes begin the ReLU words of their 128-byte
+// pieces a bank group apart (with bits 470 -> 356, float32 889 -> 577).
 template <typename T, bool kDraw>
 __global__ void __launch_bounds__(256) same_gather_rows_kernel(const SameParams p, const PhiloxKeys ks, uint32_t* relubits, int64_t w32, int warps) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
@@ -491,6 +493,7 @@ __global__ void __launch_bounds__(256) same_gather_rows_kernel(const SameParams 
     }
     s_idx[j] = (uint16_t)col;
   }
+  for (int64_t j = draw.kept + tid; kDraw && j < p.ld; j += blockDim.x) s_idx[j] = 0;
   __syncthreads();
   if (warp >= warps) return;
   const int64_t row_bytes = p.D * (int64_t)sizeof(T);
@@ -508,17 +511,25 @@ __global__ void __launch_bounds__(256) same_gather_rows_kernel(const SameParams 
     __syncwarp();
     if (relubits != nullptr) {
       for (int64_t w = lane; w < w32; w += 32) {
-        uint32_t m = positive32(s_row + w * 32);    // D is a multiple of 32 on this path
+        uint32_t m = positive32(s_row + w * 32, sizeof(T) == 4 ? lane : lane >> 1);    // D is a multiple of 32 on this path
         relubits[b * w32 + w] = m;
       }
     }
     T* orow = out + b * p.ld;
     for (int64_t j0 = (int64_t)lane * kPer; j0 < p.ld; j0 += 32 * kPer) {
+      uint32_t cols[kPer / 2];                       // two columns a word, all of a store's in one access
+      if constexpr (kPer == 8) {
+        const uint4 q = *reinterpret_cast<const uint4*>(s_idx + j0);
+        cols[0] = q.x; cols[1] = q.y; cols[2] = q.z; cols[3] = q.w;
+      } else {
+        const uint2 q = *reinterpret_cast<const uint2*>(s_idx + j0);
+        cols[0] = q.x; cols[1] = q.y;
+      }
       __align__(16) T v[kPer];
 #pragma unroll
       for (int e = 0; e < kPer; ++e) {
-        const float a = j0 + e < k ? to_float(s_row[s_idx[j0 + e]]) : 0.0f;
-        v[e] = from_float<T>(__fmul_rn(a, p.scale));
+        const float a = to_float(s_row[e & 1 ? cols[e >> 1] >> 16 : cols[e >> 1] & 0xffffu]);
+        v[e] = from_float<T>(j0 + e < k ? __fmul_rn(a, p.scale) : 0.0f);
       }
       *reinterpret_cast<uint4*>(orow + j0) = *reinterpret_cast<const uint4*>(v);
     }
@@ -1115,7 +1126,11 @@ extern "C" int rad_linear_forward_store(const void* A, int64_t lda, const rad_st
   p.values = st->values; p.ld = st->values_ld; p.keepbits = st->keepbits; p.idx = st->offsets;
   p.nnz = st->nnz; p.dev_status = dev_status;
   const float* colscale = nullptr;
-  const bool draw = !replace && st->D <= kDrawColumns;                    // the columns are drawn by the gather's CTAs
+  // The columns are drawn by the gather's CTAs, but for the largest float32 stores without ReLU bits: those run at the rate of the
+  // DRAM, and CTAs that all start at once, in step, take longer than ones that read the list first (65536 x 8192, p = 0.3 / 0.5 / 1
+  // 452 / 540 / 691 us against 424 / 509 / 734; 65536 x 4096 220 / 285 / 371 against 212 / 284 / 346; 16384 x 8192 113 / 140 / 180 against 112 / 137 / 209).
+  const bool in_step = st->dtype == RAD_F32 && st->relubits == nullptr && st->B * st->D >= ((int64_t)192 << 20);
+  const bool draw = !replace && st->D <= kDrawColumns && !in_step;
   count_launch(draw ? 1 : 2);
   if (replace) {
     SameReplaceParams r;

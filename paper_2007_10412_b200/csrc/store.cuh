@@ -69,29 +69,33 @@ __host__ __device__ constexpr bool tile_fits(uint32_t begin, uint32_t end, int64
   return (int64_t)end <= capacity && (uint64_t)(end - begin) * 2u <= room;
 }
 
-// Bits of (a > 0) for 32 consecutive entries in shared memory; zero of either sign gives 0.
-__device__ __forceinline__ uint32_t positive32(const float* src) {
+// Bits of (a > 0) for 32 consecutive entries in shared memory; zero of either sign gives 0.  The sixteen-byte pieces are taken
+// from piece `first` on: lanes whose entries lie a multiple of 128 bytes apart meet no bank conflict if they begin apart.
+__device__ __forceinline__ uint32_t positive32(const float* src, int first = 0) {
   uint32_t m = 0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int k = 0; k < 8; ++k) {
+    const int i = (k + first) & 7;
     const float4 v = reinterpret_cast<const float4*>(src)[i];
-    m |= (v.x > 0.0f ? 1u : 0u) << (4 * i) | (v.y > 0.0f ? 1u : 0u) << (4 * i + 1) |
-         (v.z > 0.0f ? 1u : 0u) << (4 * i + 2) | (v.w > 0.0f ? 1u : 0u) << (4 * i + 3);
+    m |= ((v.x > 0.0f ? 1u : 0u) | (v.y > 0.0f ? 2u : 0u) | (v.z > 0.0f ? 4u : 0u) | (v.w > 0.0f ? 8u : 0u)) << (4 * i);
   }
   return m;
 }
-__device__ __forceinline__ uint32_t positive32(const bf16* src) {
+__device__ __forceinline__ uint32_t positive32(const bf16* src, int first = 0) {
   uint32_t m = 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int k = 0; k < 4; ++k) {
+    const int i = (k + first) & 3;
     const uint4 q = reinterpret_cast<const uint4*>(src)[i];
     const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+    uint32_t bits = 0;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       // positive: sign clear and some other bit set (the add carries into the sign position)
       const uint32_t nz = ((w[j] & 0x7fff7fffu) + 0x7fff7fffu) & ~w[j] & 0x80008000u;
-      m |= ((nz >> 15) & 1u) << (8 * i + 2 * j) | (nz >> 31) << (8 * i + 2 * j + 1);
+      bits |= ((nz >> 15) & 1u) << (2 * j) | (nz >> 31) << (2 * j + 1);
     }
+    m |= bits << (8 * i);
   }
   return m;
 }

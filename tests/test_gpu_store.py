@@ -190,3 +190,30 @@ def test_relu_bits_of_narrow_rows(B, D, dtype):
     bits[:, :D] = A > 0
     want = (bits.view(B, w32, 32) << torch.arange(32, device="cuda")).sum(2)
     assert torch.equal(st.relubits.view(B, w32).long() & 0xffffffff, want)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("B,D,p,relu", [(3, 31, 0.5, True), (3, 32, 0.5, True), (9, 33, 0.5, True), (300, 96, 1.0, True), (5, 8160, 0.9, False), (5, 8191, 0.1, True),
+                                        (9, 8192, 0.5, True), (3, 8192, 0.1, False), (3, 8193, 0.1, True), (9, 8224, 0.5, True), (70000, 1, 0.5, True)])
+def test_same_sample_columns_drawn_by_the_gather(B, D, p, relu, dtype):
+    """Rows up to the longest whose columns every CTA of the gather draws for itself and beyond (a list made by a kernel of its
+    own), with and without ReLU bits, more CTAs than one, words with remainders: list, counts, values and bits are the oracle's."""
+    import paper_2007_10412_b200 as rad
+    A, _ = layer_inputs(B, D, 1, dtype=dtype, seed=B + D + 2, relu_like=True)
+    seed, layer, step = (1 << 33) + 5, 2, 9
+    ref = orc.forward_store(A, dtype, "same", p, seed, layer, step)
+    st = rad.Store("same", dtype, B, D, p, seed=seed, layer=layer, step=step, capacity="worst", relu_bits=relu)
+    st.values.fill_(7.0)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rad.rad_linear_forward_store(to_dev(A, dtype), st, status)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    k, ld = ref.idx.size, st.c.values_ld
+    assert st.nnz.cpu().tolist()[:2] == [k, k * B]
+    assert np.array_equal(u32(st.offsets)[:k], ref.idx.astype(np.uint32))
+    assert np.array_equal(u32(st.keepbits), ref.keepbits.reshape(-1))
+    got = bits_host(st.values[:B * ld]).reshape(B, ld)
+    assert np.array_equal(got[:, :k], bits_of(ref.values, dtype).reshape(B, k))
+    assert (got[:, k:] == 0).all()
+    if relu:
+        assert np.array_equal(u32(st.relubits).reshape(B, -1), ref.relubits)
