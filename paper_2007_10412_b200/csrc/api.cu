@@ -442,7 +442,7 @@ static int input_grad(int32_t dtype, int64_t B, int64_t D, int64_t H, const void
   if (db != nullptr) {
     // sums that are made beside the contraction use no workspace, which is asked for all the same
     if (beside && (workspace == nullptr || workspace_bytes < column_sums_workspace(B, H))) return RAD_EWORKSPACE;
-    if (!beside) rc = column_sums(dtype, B, H, dZ, ldz, db, workspace, workspace_bytes, s);
+    if (!beside) rc = column_sums(dtype, B, H, dZ, ldz, db, workspace, workspace_bytes, s, beside_ahead && dZ_prev == nullptr);
     if (rc != RAD_OK) return rc;
   }
   if (dZ_prev == nullptr) return RAD_OK;

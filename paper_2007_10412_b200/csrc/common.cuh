@@ -249,7 +249,7 @@ int simt_weight_grad(const rad_store* st, const void* dZ, int64_t ldz, int64_t H
                      float* db = nullptr, bool* db_written = nullptr,
                      const SimtInputGrad* ig = nullptr, bool* ig_done = nullptr);
 int column_sums(int dtype, int64_t B, int64_t H, const void* dZ, int64_t ldz, float* db,
-                void* workspace, int64_t workspace_bytes, cudaStream_t s);
+                void* workspace, int64_t workspace_bytes, cudaStream_t s, bool beside = false);
 int64_t column_sums_workspace(int64_t B, int64_t H);
 
 // store.cu: values and ReLU bits of a different-sample Bernoulli store whose index part is in place
@@ -426,9 +426,9 @@ __device__ __forceinline__ void st_cluster_u32(uint32_t* smem, uint32_t rank, ui
 // CTA has signalled, that is with the last wave), one whose CTAs go on to further pieces as each begins its last one.
 // With the signal at the start of the pair kernels a small kernel of another stream waited 4.1 ms of a 65536 x 8192 x
 // 8192 forward for room; with this rule it runs in 20 us beside it.
-// A tensor-core kernel with `beside` set has nothing to do with the kernel ahead: neither reads or overwrites what the other
-// writes.  It begins at once (the kernel ahead let it in behind its own wait, so all before that one has ended) and waits at its
-// own end instead, so that for the kernels behind it one end still means all ends.  Never two of these in a row.
+// A kernel with `beside` set has nothing to do with the kernel ahead: neither reads or overwrites what the other writes.  It
+// begins at once (the kernel ahead let it in behind its own wait, so all before that one has ended) and waits at its own end
+// instead, so that for the kernels behind it one end still means all ends.  Never two of these in a row.
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void begin_after_previous() {

@@ -675,8 +675,9 @@ __device__ __forceinline__ void colsum_load(const T* p, float (&v)[V]) {
 // the number of partial rows (cluster of one) where a second launch adds them
 template <typename T, int V>
 __global__ void __launch_bounds__(256) colsum_kernel(const T* dZ, int64_t ldz, int64_t B, int64_t H, int log_cl,
-                                                     int64_t rows_per_cta, float* out) {
-  begin_after_previous();
+                                                     int64_t rows_per_cta, float* out, bool beside) {
+  if (!beside) wait_for_previous();
+  let_next_start();
   __shared__ float s_warp[8][32 * V];
   __shared__ float s_cta[32 * V];
   const int CL = 1 << log_cl, RL = 256 >> log_cl, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -712,28 +713,30 @@ __global__ void __launch_bounds__(256) colsum_kernel(const T* dZ, int64_t ldz, i
     if (clustered) s_cta[tid] = t;
     else if (hc < H) out[(int64_t)blockIdx.y * H + hc] = t;
   }
-  if (!clustered) return;
-  cluster_barrier();
-  if (blockIdx.y == 0 && tid < CL * V && hc < H) {
-    float t = 0.0f;
-    for (int q = 0; q < (int)gridDim.y; ++q) t += ld_cluster_f32(&s_cta[tid], (uint32_t)q);
-    out[hc] = t;
+  if (clustered) {
+    cluster_barrier();
+    if (blockIdx.y == 0 && tid < CL * V && hc < H) {
+      float t = 0.0f;
+      for (int q = 0; q < (int)gridDim.y; ++q) t += ld_cluster_f32(&s_cta[tid], (uint32_t)q);
+      out[hc] = t;
+    }
+    cluster_barrier();                     // no CTA leaves while another reads its sums
   }
-  cluster_barrier();                       // no CTA leaves while another reads its sums
+  if (beside && tid == 0) wait_for_previous();
 }
 
 template <typename T, int V>
-int launch_colsum(const T* dZ, int64_t ldz, int64_t B, int64_t H, int log_cl, int ny, bool clustered, float* out, cudaStream_t s) {
+int launch_colsum(const T* dZ, int64_t ldz, int64_t B, int64_t H, int log_cl, int ny, bool clustered, float* out, cudaStream_t s, bool beside = false) {
   const int64_t colblocks = ceil_div(H, (int64_t)V << log_cl);
   count_launch();
   return launch_with_cluster(colsum_kernel<T, V>, dim3((unsigned)colblocks, (unsigned)ny), 256, 0, clustered ? dim3(1, (unsigned)ny) : dim3(1),
-                             s, dZ, ldz, B, H, log_cl, ceil_div(B, (int64_t)ny), out);
+                             s, dZ, ldz, B, H, log_cl, ceil_div(B, (int64_t)ny), out, beside);
 }
 
 // Column lanes of a CTA: eight 16-byte vectors make a 128-byte line; a narrow matrix gets the power of two that
 // holds its columns, so that the other threads are row lanes.
 template <typename T, int V>
-int column_sums_of(const T* dZ, int64_t ldz, int64_t B, int64_t H, float* out, float* partial, int64_t max_slabs, cudaStream_t s) {
+int column_sums_of(const T* dZ, int64_t ldz, int64_t B, int64_t H, float* out, float* partial, int64_t max_slabs, cudaStream_t s, bool beside = false) {
   int log_cl = 0;
   const int64_t vecs = ceil_div(H, (int64_t)V);
   const bool big = V > 1 && vecs >= 32 && B * H * (int64_t)sizeof(T) >= kColBigBytes && max_slabs > kColMaxCluster;
@@ -763,7 +766,7 @@ int column_sums_of(const T* dZ, int64_t ldz, int64_t B, int64_t H, float* out, f
     return vec ? column_sums_of<float, 4>(partial, H, slabs, H, out, nullptr, 0, s)
                : column_sums_of<float, 1>(partial, H, slabs, H, out, nullptr, 0, s);
   }
-  return launch_colsum<T, V>(dZ, ldz, B, H, log_cl, ny, true, out, s);
+  return launch_colsum<T, V>(dZ, ldz, B, H, log_cl, ny, true, out, s, beside);
 }
 
 }  // namespace
@@ -932,19 +935,19 @@ int64_t column_sums_workspace(int64_t B, int64_t H) {
 }
 
 int column_sums(int dtype, int64_t B, int64_t H, const void* dZ, int64_t ldz, float* db, void* workspace,
-                int64_t workspace_bytes, cudaStream_t s) {
+                int64_t workspace_bytes, cudaStream_t s, bool beside) {
   if (workspace == nullptr || workspace_bytes < column_sums_workspace(B, H)) return RAD_EWORKSPACE;
   float* partial = static_cast<float*>(workspace);
   const int64_t slabs = ceil_div(B, kColChunkRows);          // partial rows the workspace holds
   const bool aligned = ((uintptr_t)dZ & 15) == 0;
   if (dtype == RAD_BF16) {
     const bf16* z = static_cast<const bf16*>(dZ);
-    return aligned && H % 8 == 0 && ldz % 8 == 0 ? column_sums_of<bf16, 8>(z, ldz, B, H, db, partial, slabs, s)
-                                                 : column_sums_of<bf16, 1>(z, ldz, B, H, db, partial, slabs, s);
+    return aligned && H % 8 == 0 && ldz % 8 == 0 ? column_sums_of<bf16, 8>(z, ldz, B, H, db, partial, slabs, s, beside)
+                                                 : column_sums_of<bf16, 1>(z, ldz, B, H, db, partial, slabs, s, beside);
   }
   const float* z = static_cast<const float*>(dZ);
-  return aligned && H % 4 == 0 && ldz % 4 == 0 ? column_sums_of<float, 4>(z, ldz, B, H, db, partial, slabs, s)
-                                               : column_sums_of<float, 1>(z, ldz, B, H, db, partial, slabs, s);
+  return aligned && H % 4 == 0 && ldz % 4 == 0 ? column_sums_of<float, 4>(z, ldz, B, H, db, partial, slabs, s, beside)
+                                               : column_sums_of<float, 1>(z, ldz, B, H, db, partial, slabs, s, beside);
 }
 
 }  // namespace rad
