@@ -266,7 +266,8 @@ extern "C" int rad_cnn_step(const rad_cnn_desc* d, const void* X, const int32_t*
     if (l > 0) {
       void* g_prev = ws + pl.grad[(l - 1) & 1];
       if (conv_stage_dx_ok(d->dtype, B, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], dz, conv_W[l], g_prev))
-        rc = conv_stage_input_grad(B, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], dz, conv_W[l], g_prev, dev_status, s);
+        // beside the column sums, which read dZ as well and write db and the scratch
+        rc = conv_stage_input_grad(B, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], dz, conv_W[l], g_prev, dev_status, s, true);
       else if (conv_tc_dx_ok(d->dtype, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], dz, conv_W[l], g_prev))
         rc = conv_tc_input_grad(B, pl.H[l], pl.W[l], pl.Cin[l], pl.Cout[l], dz, conv_W[l], g_prev, dev_status, s);
       else

@@ -318,7 +318,7 @@ int conv_stage_forward_pool(int64_t B, int H, int W, int Cin, int Cout, const vo
                             uint32_t* relubits, int32_t* dev_status, cudaStream_t st);
 bool conv_stage_dx_ok(int dtype, int64_t B, int H, int W, int Cin, int Cout, const void* dZ, const void* Wt, const void* dX);
 int conv_stage_input_grad(int64_t B, int H, int W, int Cin, int Cout, const void* dZ, const void* Wt, void* dX, int32_t* dev_status,
-                          cudaStream_t st);
+                          cudaStream_t st, bool beside);
 
 // tcgen05 kernels (bf16, aligned)
 bool tc_shape_ok(int64_t B, int64_t D, int64_t H, const void* p0, int64_t ld0, const void* p1,

@@ -39,6 +39,7 @@ struct ConvStageParams {
   int64_t groups;
   int32_t* dev_status;
   uint64_t wait_limit_ns;
+  bool beside;              // runs beside the kernel ahead, and waits for its end at its own end
 };
 struct CsCtl {
   uint64_t done;
@@ -104,7 +105,7 @@ __global__ void __launch_bounds__(kCsThreads, 3) conv_stage_kernel(const __grid_
   }
   // zeros around the images (and where a tap without a partner reads): copies of images leave them as they are
   for (int i = tid * 16; i < kPlanes * plane + (p.chunks == 1 ? 128 * 16 : 0); i += kCsThreads * 16) *reinterpret_cast<uint4*>(smem + i) = make_uint4(0u, 0u, 0u, 0u);
-  wait_for_previous();
+  if (!p.beside) wait_for_previous();
   __syncthreads();
   // ---- images: a warp per line, 16 bytes (eight channels of a pixel) a lane; those of few channels come as they are first ----
   uint8_t* raw = reinterpret_cast<uint8_t*>(ctl) + ((sizeof(CsCtl) + 15) & ~15);
@@ -303,6 +304,7 @@ __global__ void __launch_bounds__(kCsThreads, 3) conv_stage_kernel(const __grid_
     umma_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)p.cols) : "memory");
   }
+  if (p.beside && tid == 0) wait_for_previous();
 }
 
 // Images of a group and what follows from it: the fewest rounds of tiles over the chip (three CTAs an SM), a group's copies
@@ -390,11 +392,12 @@ bool conv_stage_dx_ok(int dtype, int64_t B, int H, int W, int Cin, int Cout, con
   return plan_stage<true>(p, &smem);
 }
 int conv_stage_input_grad(int64_t B, int H, int W, int Cin, int Cout, const void* dZ, const void* Wt, void* dX, int32_t* dev_status,
-                          cudaStream_t st) {
+                          cudaStream_t st, bool beside) {
   ConvStageParams p = stage_shape(B, H, W, Cin, Cout);
   size_t smem = 0;
   if (!plan_stage<true>(p, &smem)) return RAD_EINVAL;
   p.A = static_cast<const bf16*>(dZ); p.Wt = static_cast<const bf16*>(Wt); p.out = static_cast<bf16*>(dX); p.dev_status = dev_status;
+  p.beside = beside;
   return launch_stage<true>(p, smem, st);
 }
 

@@ -96,4 +96,4 @@ def test_a_kernel_beside_the_one_ahead_ends_after_it():
         assert len(skips) == 1 and len(re.findall(r"\bbeside\b", body)) == 2, (file, kernel)
         assert re.search(r"\bbeside && tid == 0\) wait_for_previous\(\);\s*$", body.rstrip().rstrip("}").rstrip()), (file, kernel)
         assert "return;" not in body, (file, kernel)                       # no thread leaves before
-    assert found == 2
+    assert found == 3
